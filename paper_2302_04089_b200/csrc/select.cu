@@ -13,121 +13,310 @@
 // (ties: lowest s), stores the argmin per (module, b) in global scratch and walks it back from
 // b = n_buckets.  All comparisons are on float64 sums formed in module order, which is what makes
 // the chosen levels reproducible bit for bit.
+//
+// What bounds it: instruction issue (one addition and one comparison per option and bucket), so the
+// programme evaluates only what can matter, without changing any value it returns:
+//   * Buckets.  Row m is needed from lo[m] = n_buckets - (largest units of modules m, m + 1, ...)
+//     on, because no walk back reaches below, and is constant from hi[m] = (largest units of
+//     modules 0 .. m - 1) on, where every option fits; only lo .. hi is computed and reads beyond
+//     hi are clamped to it.  With a budget of half the dense run time that is half of the buckets.
+//   * Options.  f_m does not increase with b (a larger budget keeps every choice), so over a block
+//     of buckets [b0, b1] option s costs at least f_m[b1 - u_s] + c_s, and the best option of any
+//     bucket costs at most min_s f_m[b0 - u_s] + c_s.  Options whose lower bound lies above that
+//     are skipped (rounding is monotone, so the bounds hold for the rounded sums too).  A warp takes
+//     64 buckets: its lanes test one option each, then all lanes evaluate the 3 to 6 of (on the
+//     paper's grid) 13 or 44 options that are left.  32 buckets leave fewer options but pay the
+//     test twice as often, 128 leave twice as many.
 #include <math.h>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ziplm {
 namespace {
 
 constexpr int SEL_THREADS = 1024;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int SEL_BLK = 64;               // buckets a warp works on at a time
 constexpr int SEL_MAX_OPT = 255;          // options per module (argmin stored in a byte)
 constexpr int SEL_MAX_BUCKETS = 12000;    // two float64 rows of n_buckets + 1 fit shared memory
 constexpr int SEL_MAX_MOD = 512;          // modules per search (coefficient vectors in shared memory)
+constexpr int SEL_MAX_CLUSTER = 16;       // CTAs (steps at a time) of one search
+constexpr int SEL_SMEM_MOD = 1024;        // up to here the per-module bounds are in shared memory
+constexpr size_t SEL_SMEM_MAX = 227 * 1024 - 8192;      // dynamic shared memory a kernel here may use
 
-// The dynamic programme and its walk back for one coefficient vector `coef` [n_mod] (global or
-// shared memory), run by the whole CTA.  f0 / f1 are the two value rows in shared memory, `ch`
-// this CTA's [n_mod][n_buckets + 1] argmin scratch.  On return thread 0 holds the result in
-// *total / *tsum (total = inf: nothing fits) and has written sel[0 .. n_mod); *nonfinite is a
-// shared flag that is raised when a cost or a time is NaN.  Ends with a barrier.
-__device__ void dp_solve(const float* __restrict__ loss, const float* __restrict__ base_loss,
-                         const float* __restrict__ time, const int* __restrict__ n_opt, int n_mod,
-                         int max_opt, const float* coef, double per_unit, int n_buckets, double* f0,
-                         double* f1, double* s_cost, int* s_units, int* nonfinite, unsigned char* ch,
-                         int* sel, double* total, double* tsum) {
-    const int tid = threadIdx.x;
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    for (int b = tid; b <= n_buckets; b += SEL_THREADS) f0[b] = 0.0;
-    for (int m = 0; m < n_mod; ++m) {
-        const int no = min(max(n_opt[m], 0), max_opt);
-        __syncthreads();
-        for (int s = tid; s < no; s += SEL_THREADS) {
-            const double p = (double)loss[(size_t)m * max_opt + s] / (double)base_loss[m];
-            s_cost[s] = (double)coef[m] * p;
-            const double u = ceil((double)time[(size_t)m * max_opt + s] * per_unit);
-            // an option that cannot fit (or has a negative time) is never taken
-            s_units[s] = (u >= 0.0 && u <= (double)n_buckets) ? (int)u : n_buckets + 1;
-            if (s_cost[s] != s_cost[s] || u != u) *nonfinite = 1;
+// What one CTA works with.  The rows are in shared memory; so are the tables (priors p and units u of
+// every option) when they fit, otherwise they are formed module by module in the same place.
+struct DpCta {
+    const float* loss; const float* base_loss; const float* time; const int* n_opt;
+    int n_mod, max_opt, n_buckets;
+    double per_unit;
+    double* f0; double* f1;          // value rows
+    double* p; int* u;               // [n_mod or 1][max_opt]
+    int* lo; int* hi;                // [n_mod + 1] each: row m is computed on lo[m] .. hi[m]
+    unsigned char* ch;               // [n_mod][n_buckets + 1] argmins (global)
+    bool resident;                   // all modules' tables at once
+};
+
+// Where the dynamic shared memory of a CTA goes; the same arithmetic on host and device.
+struct DpLayout {
+    size_t bounds, p, u, total;
+    bool resident, bounds_in_smem;
+    __host__ __device__ DpLayout(int n_mod, int max_opt, int n_buckets) {
+        const size_t rows = 2 * (size_t)(n_buckets + 1) * sizeof(double);
+        bounds_in_smem = n_mod <= SEL_SMEM_MOD;
+        p = rows;
+        const size_t b = bounds_in_smem ? (2 * (size_t)n_mod + 2) * sizeof(int) : 0;
+        const size_t all = (size_t)n_mod * max_opt;
+        resident = rows + b + all * (sizeof(double) + sizeof(int)) <= SEL_SMEM_MAX;
+        const size_t n = resident ? all : (size_t)max_opt;
+        u = p + n * sizeof(double);
+        bounds = u + n * sizeof(int);
+        total = bounds + b;
+    }
+};
+
+// Prior and units of one option; raises *nonfinite for a NaN (a coefficient is checked when used).
+__device__ __forceinline__ void dp_option(const DpCta& w, int m, int s, double* p, int* u, int* nonfinite) {
+    const size_t at = (size_t)m * w.max_opt + s;
+    *p = (double)w.loss[at] / (double)w.base_loss[m];
+    const double t = ceil((double)w.time[at] * w.per_unit);
+    // an option that cannot fit (or has a negative time) is never taken
+    *u = (t >= 0.0 && t <= (double)w.n_buckets) ? (int)t : w.n_buckets + 1;
+    if (t != t) *nonfinite = 1;
+}
+
+__device__ __forceinline__ int dp_units(const DpCta& w, int m, int s) {
+    return w.resident ? w.u[(size_t)m * w.max_opt + s]
+                      : (int)ceil((double)w.time[(size_t)m * w.max_opt + s] * w.per_unit);
+}
+
+__device__ __forceinline__ int dp_count(const DpCta& w, int m) { return min(max(w.n_opt[m], 0), w.max_opt); }
+
+// Tables (when resident) and bounds of a CTA; ends with a barrier.
+__device__ void dp_setup(DpCta& w, int* nonfinite) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int m = tid >> 5; m < w.n_mod; m += SEL_WARPS) {
+        const int no = dp_count(w, m);
+        int most = 0;
+        for (int s = lane; s < no; s += 32) {
+            double p;
+            int u;
+            dp_option(w, m, s, &p, &u, nonfinite);
+            if (w.resident) { w.p[(size_t)m * w.max_opt + s] = p; w.u[(size_t)m * w.max_opt + s] = u; }
+            if (u <= w.n_buckets) most = max(most, u);
         }
-        __syncthreads();
-        // four buckets per thread and pass, so that an option's units and cost are fetched once
-        // for four evaluations
-        for (int b0 = tid; b0 <= n_buckets; b0 += 4 * SEL_THREADS) {
-            double best[4] = {inf, inf, inf, inf};
-            int arg[4] = {0, 0, 0, 0};
-            for (int s = 0; s < no; ++s) {
-                const int u = s_units[s];
-                const double c = s_cost[s];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int b = b0 + j * SEL_THREADS;
-                    if (b <= n_buckets && u <= b) {
-                        const double v = f0[b - u] + c;
-                        if (v < best[j]) { best[j] = v; arg[j] = s; }
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int b = b0 + j * SEL_THREADS;
-                if (b <= n_buckets) {
-                    f1[b] = best[j];
-                    ch[(size_t)m * (n_buckets + 1) + b] = (unsigned char)arg[j];
-                }
-            }
-        }
-        double* t = f0; f0 = f1; f1 = t;
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (lane == 0) w.hi[m + 1] = most;
     }
     __syncthreads();
     if (tid == 0) {
-        *total = f0[n_buckets];
-        *tsum = 0.0;
-        if (*total < inf) {
-            int b = n_buckets;
-            double acc = 0.0;
-            for (int m = n_mod - 1; m >= 0; --m) {
-                const int s = ch[(size_t)m * (n_buckets + 1) + b];
-                sel[m] = s;
-                const double tm = (double)time[(size_t)m * max_opt + s];
-                acc += tm;
-                b -= (int)ceil(tm * per_unit);
-            }
-            *tsum = acc;
-        }
+        int lo = w.n_buckets, hi = 0;
+        w.lo[w.n_mod] = lo;
+        for (int m = w.n_mod - 1; m >= 0; --m) w.lo[m] = lo = max(0, lo - w.hi[m + 1]);
+        w.hi[0] = 0;
+        for (int m = 1; m <= w.n_mod; ++m) w.hi[m] = hi = min(w.n_buckets, hi + w.hi[m]);
     }
     __syncthreads();
 }
 
+// Floats as signed integers in the same order.
+__device__ __forceinline__ int float_order(float v) {
+    const int i = __float_as_int(v);
+    return i ^ ((i >> 31) & 0x7fffffff);
+}
+
+// One row of the programme, buckets [lo, hi], by the whole CTA.  R: options per lane.
+template <int R>
+__device__ __forceinline__ void dp_row(const double* f0, double* f1, const double* p, const int* u, int no,
+                                       double coef, int lo, int hi, int hi_prev, unsigned char* ch,
+                                       int* nonfinite) {
+    const int lane = threadIdx.x & 31;
+    const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    double c[R];
+    int us[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int s = r * 32 + lane;
+        us[r] = s < no ? u[s] : 0x40000000;
+        c[r] = s < no ? coef * p[s] : inf;
+        if (c[r] != c[r]) *nonfinite = 1;
+    }
+    for (int b0 = lo + (threadIdx.x >> 5) * SEL_BLK; b0 <= hi; b0 += SEL_WARPS * SEL_BLK) {
+        const int b1 = min(b0 + SEL_BLK - 1, hi);
+        float low[R];
+        int bound = 0x7f800000;                                   // +inf
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (r > 0 && r * 32 >= no) { low[r] = __int_as_float(0x7f800000); continue; }
+            const int i0 = min(b0 - us[r], hi_prev), i1 = min(b1 - us[r], hi_prev);
+            const double v0 = i0 >= 0 ? f0[i0] + c[r] : inf;
+            low[r] = __double2float_rd(i1 >= 0 ? f0[i1] + c[r] : inf);
+            const float up = __double2float_ru(v0);
+            if (up == up) bound = min(bound, float_order(up));
+        }
+        bound = __reduce_min_sync(0xffffffffu, bound);
+        double best0 = inf, best1 = inf;
+        int arg0 = 0, arg1 = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (r > 0 && r * 32 >= no) break;
+            unsigned left = __ballot_sync(0xffffffffu, us[r] <= b1 && float_order(low[r]) <= bound);
+            while (left) {
+                const int src = __ffs(left) - 1;
+                left &= left - 1;
+                const int uu = __shfl_sync(0xffffffffu, us[r], src);
+                const double cc = __shfl_sync(0xffffffffu, c[r], src);
+                const int i = b0 + lane - uu;
+                if (i >= 0) {
+                    const double v = f0[min(i, hi_prev)] + cc;
+                    if (v < best0) { best0 = v; arg0 = r * 32 + src; }
+                }
+                if (i + 32 >= 0) {
+                    const double v = f0[min(i + 32, hi_prev)] + cc;
+                    if (v < best1) { best1 = v; arg1 = r * 32 + src; }
+                }
+            }
+        }
+        const int b = b0 + lane;
+        if (b <= hi) { f1[b] = best0; ch[b] = (unsigned char)arg0; }
+        if (b + 32 <= hi) { f1[b + 32] = best1; ch[b + 32] = (unsigned char)arg1; }
+    }
+}
+
+// The dynamic programme and its walk back for one coefficient vector (global or shared memory), run
+// by the whole CTA.  Returns the minimal cost (inf: nothing fits) in every thread; then sel[0 ..
+// n_mod) (global) holds the chosen options.  *nonfinite is a shared flag that is raised when a cost
+// is NaN.  Ends with a barrier.
+template <int R>
+__device__ double dp_solve(DpCta& w, const float* coef, int* nonfinite, int* sel) {
+    const int tid = threadIdx.x, lane = tid & 31, B = w.n_buckets;
+    const size_t pitch = (size_t)(B + 1);
+    const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    double* f0 = w.f0;
+    double* f1 = w.f1;
+    if (tid == 0) f0[0] = 0.0;                   // row 0 is 0 everywhere: hi[0] = 0
+    __syncthreads();
+    int hi = 0;
+    for (int m = 0; m < w.n_mod; ++m) {
+        const int no = dp_count(w, m), next = w.hi[m + 1];
+        const double* p = w.p;
+        const int* u = w.u;
+        if (w.resident) {
+            p += (size_t)m * w.max_opt;
+            u += (size_t)m * w.max_opt;
+        } else {
+            for (int s = tid; s < no; s += SEL_THREADS) dp_option(w, m, s, w.p + s, w.u + s, nonfinite);
+            __syncthreads();
+        }
+        dp_row<R>(f0, f1, p, u, no, (double)coef[m], min(w.lo[m + 1], next), next, hi, w.ch + m * pitch,
+                  nonfinite);
+        __syncthreads();
+        double* t = f0; f0 = f1; f1 = t;
+        hi = next;
+    }
+    const double total = f0[hi];
+    if (total < inf && tid < 32) {
+        // walk back, two modules a round: the argmins of module m - 1 for every option of module m
+        // are fetched together with module m's own, so a round waits for memory once
+        int b = B;
+        for (int m = w.n_mod - 1; m >= 0; m -= 2) {
+            const int no = dp_count(w, m), prev = w.hi[m], first = min(w.lo[m], prev);
+            const int s = w.ch[m * pitch + min(b, w.hi[m + 1])];
+            int um = 0, s1 = 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int o = r * 32 + lane;
+                int u = 0, c = 0;
+                if (o < no) {
+                    u = dp_units(w, m, o);
+                    const int i = min(b - u, prev);
+                    if (m > 0 && i >= first) c = w.ch[(m - 1) * pitch + i];
+                }
+                u = __shfl_sync(0xffffffffu, u, s & 31);
+                c = __shfl_sync(0xffffffffu, c, s & 31);
+                if ((s >> 5) == r) { um = u; s1 = c; }
+            }
+            b -= um;
+            if (lane == 0) sel[m] = s;
+            if (m > 0) {
+                if (lane == 0) sel[m - 1] = s1;
+                b -= dp_units(w, m - 1, s1);
+            }
+        }
+    }
+    __syncthreads();
+    return total;
+}
+
+// Sum of row[m][sel[m]] over the modules, float64, in the order first, first + step, ...; warp 0 (the
+// warp that wrote sel) calls it and every lane has the sum.
+__device__ double dp_sum(const DpCta& w, const float* row, const int* sel, bool descending) {
+    const int lane = threadIdx.x & 31;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < w.n_mod; k0 += 32) {
+        const int k = k0 + lane, m = descending ? w.n_mod - 1 - k : k;
+        const double v = k < w.n_mod ? (double)row[(size_t)m * w.max_opt + sel[m]] : 0.0;
+        const int n = min(32, w.n_mod - k0);
+        for (int j = 0; j < n; ++j) acc += __shfl_sync(0xffffffffu, v, j);
+    }
+    return acc;
+}
+
+__device__ __forceinline__ void dp_bind(DpCta& w, const float* loss, const float* base_loss, const float* time,
+                                        const int* n_opt, int n_mod, int max_opt, int n_buckets,
+                                        double per_unit, unsigned char* ch, int* bounds) {
+    extern __shared__ double sel_smem[];
+    const DpLayout at(n_mod, max_opt, n_buckets);
+    char* base = reinterpret_cast<char*>(sel_smem);
+    w.loss = loss; w.base_loss = base_loss; w.time = time; w.n_opt = n_opt;
+    w.n_mod = n_mod; w.max_opt = max_opt; w.n_buckets = n_buckets; w.per_unit = per_unit;
+    w.f0 = sel_smem;
+    w.f1 = sel_smem + (n_buckets + 1);
+    w.p = reinterpret_cast<double*>(base + at.p);
+    w.u = reinterpret_cast<int*>(base + at.u);
+    w.lo = at.bounds_in_smem ? reinterpret_cast<int*>(base + at.bounds) : bounds;
+    w.hi = w.lo + n_mod + 1;
+    w.ch = ch;
+    w.resident = at.resident;
+}
+
+// One CTA per SM takes candidates blockIdx.x, blockIdx.x + gridDim.x, ...: the tables are formed once
+// and the argmins of a CTA's candidates share one piece of scratch, which then stays in L2.
+template <int R>
 __global__ void __launch_bounds__(SEL_THREADS)
 k_select_levels(const float* __restrict__ loss, const float* __restrict__ base_loss,
                 const float* __restrict__ time, const int* __restrict__ n_opt, int n_mod, int max_opt,
-                const float* __restrict__ coef, double budget, int n_buckets,
-                unsigned char* __restrict__ choice, int* __restrict__ selected,
-                double* __restrict__ cost_out, double* __restrict__ time_out, int* __restrict__ status) {
-    extern __shared__ double sel_smem[];
-    __shared__ double s_cost[SEL_MAX_OPT];
-    __shared__ int s_units[SEL_MAX_OPT];
-    __shared__ int s_nonfinite;
-    __shared__ double s_total, s_tsum;
-    const int k = blockIdx.x, tid = threadIdx.x;
+                const float* __restrict__ coef, int K, double budget, int n_buckets, unsigned char* choice,
+                int* bounds, int* selected, double* __restrict__ cost_out, double* __restrict__ time_out,
+                int* __restrict__ status) {
+    __shared__ int s_table_bad, s_nonfinite;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    if (tid == 0) s_nonfinite = 0;
+    DpCta w;
+    dp_bind(w, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budget,
+            choice + blockIdx.x * ((size_t)n_mod * (n_buckets + 1)), bounds + blockIdx.x * (2 * (size_t)n_mod + 2));
+    if (threadIdx.x == 0) s_table_bad = 0;
     __syncthreads();
-    dp_solve(loss, base_loss, time, n_opt, n_mod, max_opt, coef + (size_t)k * n_mod,
-             (double)n_buckets / budget, n_buckets, sel_smem, sel_smem + (n_buckets + 1), s_cost, s_units,
-             &s_nonfinite, choice + (size_t)k * n_mod * (size_t)(n_buckets + 1),
-             selected + (size_t)k * n_mod, &s_total, &s_tsum);
-    if (tid == 0) {
-        if (s_nonfinite || !(s_total < inf)) {      // a NaN came in, or nothing fits the budget
-            status[k] = s_nonfinite ? (int)ZIPLM_ERR_NONFINITE : (int)ZIPLM_ERR_INVALID_ARG;
-            cost_out[k] = inf;
-            time_out[k] = 0.0;
-            for (int m = 0; m < n_mod; ++m) selected[(size_t)k * n_mod + m] = -1;
-        } else {
-            status[k] = (int)ZIPLM_OK;
-            cost_out[k] = s_total;
-            time_out[k] = s_tsum;
+    dp_setup(w, &s_table_bad);
+    for (int k = blockIdx.x; k < K; k += gridDim.x) {
+        if (threadIdx.x == 0) s_nonfinite = s_table_bad;
+        int* sel = selected + (size_t)k * n_mod;
+        const double total = dp_solve<R>(w, coef + (size_t)k * n_mod, &s_nonfinite, sel);
+        if (threadIdx.x < 32) {
+            const bool ok = !s_nonfinite && total < inf;      // no NaN came in, and the budget can be met
+            const double tsum = ok ? dp_sum(w, time, sel, true) : 0.0;
+            if (!ok)
+                for (int m = threadIdx.x; m < n_mod; m += 32) sel[m] = -1;
+            if (threadIdx.x == 0) {
+                status[k] = ok ? (int)ZIPLM_OK : s_nonfinite ? (int)ZIPLM_ERR_NONFINITE : (int)ZIPLM_ERR_INVALID_ARG;
+                cost_out[k] = ok ? total : inf;
+                time_out[k] = tsum;
+            }
         }
+        __syncthreads();
     }
 }
 
@@ -136,73 +325,113 @@ k_select_levels(const float* __restrict__ loss, const float* __restrict__ base_l
 // probability 0.1 per coefficient gives the paper's "10 % in expectation"), solves the dynamic
 // programme, scores the selection and keeps the mutated vector when the score is strictly lower.
 // The score of a selection is sum_m objective[m][s_m]: a separable stand-in for the calibration
-// loss of the stitched model, which only the caller's model can give.  One CTA runs one whole
-// search (its own budget), so many speedup targets are searched at once.
+// loss of the stitched model, which only the caller's model can give.
+//
+// A step needs the vector that the steps before it left, but few steps are accepted (16 of 1000 on
+// the paper's grid).  So a cluster of CTAs runs one search, every CTA the whole programme of another
+// step, all from the current best vector: the first accepted step in step order counts, the ones
+// behind it are evaluated again from the new vector, and the outcome is that of one step at a time.
+template <int R>
 __global__ void __launch_bounds__(SEL_THREADS)
 k_search_levels(const float* __restrict__ loss, const float* __restrict__ base_loss,
                 const float* __restrict__ time, const int* __restrict__ n_opt, int n_mod, int max_opt,
                 const float* __restrict__ objective, const float* __restrict__ coef0,
                 const double* __restrict__ budgets, int n_buckets, const unsigned char* __restrict__ mask,
-                const float* __restrict__ values, int n_steps, unsigned char* __restrict__ choice,
-                int* __restrict__ trial_sel, int* __restrict__ best_sel, float* __restrict__ best_coef,
+                const float* __restrict__ values, int n_steps, unsigned char* choice, int* trial_sel,
+                int* bounds, int* __restrict__ best_sel, float* __restrict__ best_coef,
                 double* __restrict__ best_obj, int* __restrict__ n_accepted, int* __restrict__ status) {
-    extern __shared__ double sel_smem[];
-    __shared__ double s_cost[SEL_MAX_OPT];
-    __shared__ int s_units[SEL_MAX_OPT];
     __shared__ float c_best[SEL_MAX_MOD], c_try[SEL_MAX_MOD];
-    __shared__ int s_nonfinite, s_accept;
-    __shared__ double s_total, s_tsum, s_best;
-    const int k = blockIdx.x, tid = threadIdx.x;
+    __shared__ int s_nonfinite;
+    __shared__ double s_score[2][SEL_MAX_CLUSTER];       // scores of even and odd rounds (inf: nothing fits)
+    __shared__ int s_bad[2][SEL_MAX_CLUSTER];            // whether a NaN came in
+    cg::cluster_group cluster = cg::this_cluster();
+    const int P = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int k = blockIdx.x / P, tid = threadIdx.x;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    const double per_unit = (double)n_buckets / budgets[k];
-    int* trial = trial_sel + (size_t)k * n_mod;
-    int* best = best_sel + (size_t)k * n_mod;
-    unsigned char* ch = choice + (size_t)k * n_mod * (size_t)(n_buckets + 1);
-    if (tid == 0) { s_nonfinite = 0; s_best = inf; }
+    DpCta w;
+    dp_bind(w, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budgets[k],
+            choice + blockIdx.x * ((size_t)n_mod * (n_buckets + 1)), bounds + blockIdx.x * (2 * (size_t)n_mod + 2));
+    int* trial = trial_sel + (size_t)blockIdx.x * n_mod;
+    const unsigned char* mk = mask + (size_t)k * n_steps * n_mod;
+    const float* val = values + (size_t)k * n_steps * n_mod;
+    if (tid == 0) s_nonfinite = 0;
     for (int m = tid; m < n_mod; m += SEL_THREADS) c_best[m] = coef0[(size_t)k * n_mod + m];
-    int accepted = 0;
-    for (int step = 0; step <= n_steps; ++step) {          // step 0 scores coef0 itself
-        __syncthreads();
-        for (int m = tid; m < n_mod; m += SEL_THREADS) {
-            float c = c_best[m];
-            if (step > 0 && mask[((size_t)k * n_steps + (step - 1)) * n_mod + m])
-                c = values[((size_t)k * n_steps + (step - 1)) * n_mod + m];
-            c_try[m] = c;
-        }
-        __syncthreads();
-        dp_solve(loss, base_loss, time, n_opt, n_mod, max_opt, c_try, per_unit, n_buckets, sel_smem,
-                 sel_smem + (n_buckets + 1), s_cost, s_units, &s_nonfinite, ch, trial, &s_total, &s_tsum);
-        if (tid == 0) {
-            s_accept = 0;
-            if (s_total < inf && !s_nonfinite) {
-                double score = 0.0;
-                for (int m = 0; m < n_mod; ++m) score += (double)objective[(size_t)m * max_opt + trial[m]];
-                if (score < s_best) { s_best = score; s_accept = 1; }
+    __syncthreads();
+    dp_setup(w, &s_nonfinite);
+    const int table_bad = s_nonfinite;
+    double best = inf;
+    bool bad = false;
+    int accepted = 0, round = 0;
+    for (int step = 0; step <= n_steps; ++round) {         // step 0 scores coef0 itself
+        const int mine = step + rank;
+        if (mine <= n_steps) {
+            for (int m = tid; m < n_mod; m += SEL_THREADS) {
+                float c = c_best[m];
+                if (mine > 0 && mk[(size_t)(mine - 1) * n_mod + m]) c = val[(size_t)(mine - 1) * n_mod + m];
+                c_try[m] = c;
+            }
+            if (tid == 0) s_nonfinite = table_bad;
+            const double total = dp_solve<R>(w, c_try, &s_nonfinite, trial);     // opens with a barrier
+            if (tid < 32) {
+                const double score = total < inf ? dp_sum(w, objective, trial, false) : inf;
+                if (tid < P) {
+                    cluster.map_shared_rank(&s_score[round & 1][0], tid)[rank] = score;
+                    cluster.map_shared_rank(&s_bad[round & 1][0], tid)[rank] = s_nonfinite;
+                }
             }
         }
+        cluster.sync();
+        // every CTA reads the same scores and comes to the same end of the round
+        const int n = min(P, n_steps - step + 1);
+        int winner = -1;
+        for (int q = 0; q < n && winner < 0; ++q) {
+            const double score = s_score[round & 1][q];
+            if (s_bad[round & 1][q]) bad = true;
+            if (!bad && score < best) { best = score; winner = q; }
+        }
+        if (winner >= 0) {
+            const int at = step + winner;
+            if (at > 0) {
+                ++accepted;
+                for (int m = tid; m < n_mod; m += SEL_THREADS)
+                    if (mk[(size_t)(at - 1) * n_mod + m]) c_best[m] = val[(size_t)(at - 1) * n_mod + m];
+            }
+            if (rank == winner)
+                for (int m = tid; m < n_mod; m += SEL_THREADS) best_sel[(size_t)k * n_mod + m] = trial[m];
+            step = at + 1;
+        } else {
+            step += n;
+        }
         __syncthreads();
-        if (s_accept) {
-            for (int m = tid; m < n_mod; m += SEL_THREADS) { c_best[m] = c_try[m]; best[m] = trial[m]; }
-            if (step > 0) ++accepted;
+        if (bad) break;                                    // nothing is accepted any more
+    }
+    cluster.sync();                                        // no CTA leaves while others may write to it
+    const bool ok = best < inf;
+    if (rank == 0) {
+        for (int m = tid; m < n_mod; m += SEL_THREADS) {
+            best_coef[(size_t)k * n_mod + m] = c_best[m];
+            if (!ok) best_sel[(size_t)k * n_mod + m] = -1;
+        }
+        if (tid == 0) {
+            best_obj[k] = best;
+            n_accepted[k] = accepted;
+            status[k] = bad ? (int)ZIPLM_ERR_NONFINITE : ok ? (int)ZIPLM_OK : (int)ZIPLM_ERR_INVALID_ARG;
         }
     }
-    __syncthreads();
-    const bool ok = s_best < inf;
-    for (int m = tid; m < n_mod; m += SEL_THREADS) {
-        best_coef[(size_t)k * n_mod + m] = c_best[m];
-        if (!ok) best[m] = -1;
-    }
-    if (tid == 0) {
-        best_obj[k] = s_best;
-        n_accepted[k] = accepted;
-        status[k] = s_nonfinite ? (int)ZIPLM_ERR_NONFINITE : ok ? (int)ZIPLM_OK : (int)ZIPLM_ERR_INVALID_ARG;
-    }
 }
+// Pieces of scratch of a search call: a search runs on 16 CTAs at most, and on several only while
+// there are SMs for all searches.
+int search_slices(int S) { return S > 16 * SEL_MAX_CLUSTER ? S : S * SEL_MAX_CLUSTER < 256 ? S * SEL_MAX_CLUSTER : 256; }
+
+// The kernels are instantiated for the options a lane holds: 32, 64 or 255 options per module.
+template <typename F>
+F by_options(int max_opt, F r1, F r2, F r8) { return max_opt <= 32 ? r1 : max_opt <= 64 ? r2 : r8; }
 
 }  // namespace
 
 size_t select_workspace_bytes(int K, int n_mod, int n_buckets) {
-    return align_up((size_t)K * n_mod * (size_t)(n_buckets + 1));
+    return align_up((size_t)K * n_mod * (size_t)(n_buckets + 1)) +
+           align_up((size_t)K * (2 * (size_t)n_mod + 2) * sizeof(int));
 }
 
 ziplm_status run_select_levels(const float* loss, const float* base_loss, const float* time,
@@ -211,18 +440,26 @@ ziplm_status run_select_levels(const float* loss, const float* base_loss, const 
                                int* status, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (max_opt > SEL_MAX_OPT || n_buckets > SEL_MAX_BUCKETS) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < select_workspace_bytes(K, n_mod, n_buckets)) return ZIPLM_ERR_WORKSPACE;
-    const size_t smem = 2 * (size_t)(n_buckets + 1) * sizeof(double);
-    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_select_levels, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-    k_select_levels<<<K, SEL_THREADS, smem, st>>>(loss, base_loss, time, n_opt, n_mod, max_opt, coef, budget,
-                                                  n_buckets, static_cast<unsigned char*>(ws), selected,
-                                                  cost, time_sum, status);
+    Carver c(ws);
+    unsigned char* choice = c.take<unsigned char>((size_t)K * n_mod * (size_t)(n_buckets + 1));
+    int* bounds = c.take<int>((size_t)K * (2 * (size_t)n_mod + 2));
+    int dev = 0, sms = 0;
+    ZIPLM_CHECK_CUDA(cudaGetDevice(&dev));
+    ZIPLM_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const size_t smem = DpLayout(n_mod, max_opt, n_buckets).total;
+    auto kernel = by_options(max_opt, k_select_levels<1>, k_select_levels<2>, k_select_levels<8>);
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<K < sms ? K : sms, SEL_THREADS, smem, st>>>(loss, base_loss, time, n_opt, n_mod, max_opt, coef, K,
+                                                         budget, n_buckets, choice, bounds, selected, cost,
+                                                         time_sum, status);
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }
 
 size_t search_workspace_bytes(int S, int n_mod, int n_buckets) {
-    return align_up((size_t)S * n_mod * (size_t)(n_buckets + 1)) + align_up((size_t)S * n_mod * sizeof(int));
+    const size_t n = (size_t)search_slices(S);
+    return align_up(n * n_mod * (size_t)(n_buckets + 1)) + align_up(n * n_mod * sizeof(int)) +
+           align_up(n * (2 * (size_t)n_mod + 2) * sizeof(int));
 }
 
 ziplm_status run_search_levels(const float* loss, const float* base_loss, const float* time,
@@ -233,15 +470,39 @@ ziplm_status run_search_levels(const float* loss, const float* base_loss, const 
                                size_t ws_bytes, cudaStream_t st) {
     if (max_opt > SEL_MAX_OPT || n_buckets > SEL_MAX_BUCKETS || n_mod > SEL_MAX_MOD) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < search_workspace_bytes(S, n_mod, n_buckets)) return ZIPLM_ERR_WORKSPACE;
+    const int slices = search_slices(S);
     Carver c(ws);
-    unsigned char* choice = c.take<unsigned char>((size_t)S * n_mod * (size_t)(n_buckets + 1));
-    int* trial = c.take<int>((size_t)S * n_mod);
-    const size_t smem = 2 * (size_t)(n_buckets + 1) * sizeof(double);
-    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_search_levels, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-    k_search_levels<<<S, SEL_THREADS, smem, st>>>(loss, base_loss, time, n_opt, n_mod, max_opt, objective,
-                                                  coef0, budgets, n_buckets, mask, values, n_steps, choice,
-                                                  trial, best_sel, best_coef, best_obj, n_accepted, status);
+    unsigned char* choice = c.take<unsigned char>((size_t)slices * n_mod * (size_t)(n_buckets + 1));
+    int* trial = c.take<int>((size_t)slices * n_mod);
+    int* bounds = c.take<int>((size_t)slices * (2 * (size_t)n_mod + 2));
+    const size_t smem = DpLayout(n_mod, max_opt, n_buckets).total;
+    auto kernel = by_options(max_opt, k_search_levels<1>, k_search_levels<2>, k_search_levels<8>);
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(SEL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    // the largest cluster with which all searches still run at once
+    int P = SEL_MAX_CLUSTER;
+    for (; P > 1; P /= 2) {
+        if ((long long)S * P > slices || P > n_steps + 1) continue;
+        int most = 0;
+        attr[0].val.clusterDim.x = P;
+        cfg.gridDim = dim3(S * P);
+        if (cudaOccupancyMaxActiveClusters(&most, kernel, &cfg) == cudaSuccess && most >= S) break;
+        (void)cudaGetLastError();
+    }
+    attr[0].val.clusterDim.x = P;
+    cfg.gridDim = dim3(S * P);
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, loss, base_loss, time, n_opt, n_mod, max_opt, objective,
+                                        coef0, budgets, n_buckets, mask, values, n_steps, choice, trial, bounds,
+                                        best_sel, best_coef, best_obj, n_accepted, status));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }

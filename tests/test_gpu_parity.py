@@ -710,3 +710,50 @@ def test_mutation_search_matches_oracle_bit_for_bit(n_mod, max_opt, n_buckets, s
                           float(budgets[1]), n_buckets)
     assert out0["selected"][1].tolist() == ref["selected"][0].tolist()
     assert out0["n_accepted"].tolist() == [0, 0, 0]
+
+
+@pytest.mark.parametrize("n_mod,max_opt,n_buckets,K,frac", [
+    (20, 255, 12000, 1, 0.4),       # tables of all modules do not fit shared memory; eight options per lane
+    (1100, 3, 60, 2, 0.9),          # per-module bounds in global memory; far fewer buckets than modules
+    (4, 33, 64, 200, 0.5),          # more candidates than SMs; rows of one block and one bucket
+    (3, 32, 6500, 5, 3.0),          # budget above the dense run time: rows end before the last bucket
+])
+def test_level_selection_bounds_and_table_layouts(n_mod, max_opt, n_buckets, K, frac):
+    z = zb()
+    loss, base, time, n_opt = synthetic_database(300 + n_mod, n_mod, max_opt)
+    coef = torch.rand(K, n_mod, generator=torch.Generator().manual_seed(5)) * 3 + 0.05
+    budget = frac * float(sum(time[m, 0] for m in range(n_mod)))
+    out = z.select_levels(loss.cuda(), base.cuda(), time.cuda(), n_opt.cuda(), coef.cuda(), budget, n_buckets)
+    torch.cuda.synchronize()
+    for k in range(0, K, 9):
+        sel, cost, t_sum = zo.select_levels(loss.numpy(), base.numpy(), time.numpy(), n_opt.numpy(),
+                                            coef[k].numpy(), budget, n_buckets)
+        if sel is None:
+            assert int(out["status"][k]) == int(z.Status.ERR_INVALID_ARG)
+            continue
+        assert int(out["status"][k]) == 0 and out["selected"][k].tolist() == sel
+        assert float(out["cost"][k]) == cost and abs(float(out["time_sum"][k]) - t_sum) <= 1e-12 * t_sum
+
+
+@pytest.mark.parametrize("S,steps", [(1, 100), (11, 37), (40, 9), (150, 5)])
+def test_mutation_search_cluster_sizes(S, steps):
+    """One search on a cluster of 16, 8, 2 and 1 thread blocks, each block a step of its own."""
+    z = zb()
+    n_mod, max_opt, n_buckets = 6, 20, 300
+    loss, base, time, n_opt = synthetic_database(77, n_mod, max_opt)
+    g = torch.Generator().manual_seed(S)
+    mask = (torch.rand(S, steps, n_mod, generator=g) < 0.3).to(torch.uint8)
+    values = torch.rand(S, steps, n_mod, generator=g) * 3 + 0.05
+    objective = torch.nan_to_num(loss / base[:, None] * (torch.rand(n_mod, 1, generator=g) + 0.5), nan=0.0)
+    coef0 = torch.ones(S, n_mod)
+    budgets = (0.2 + 0.7 * torch.rand(S, generator=g)).double() * float(time[:, 0].sum())
+    out = z.search_levels(loss.cuda(), base.cuda(), time.cuda(), n_opt.cuda(), objective.cuda(), coef0.cuda(),
+                          budgets.cuda(), n_buckets, mask.cuda(), values.cuda())
+    torch.cuda.synchronize()
+    for k in range(0, S, 7):
+        sel, c, score, acc = zo.search_levels(loss.numpy(), base.numpy(), time.numpy(), n_opt.numpy(),
+                                              objective.numpy(), coef0[k].numpy(), float(budgets[k]),
+                                              n_buckets, mask[k].numpy(), values[k].numpy())
+        assert int(out["status"][k]) == 0 and out["selected"][k].tolist() == sel
+        assert int(out["n_accepted"][k]) == acc and float(out["objective"][k]) == score
+        assert np.array_equal(out["coef"][k].cpu().numpy(), c)
