@@ -46,37 +46,53 @@ constexpr int SEL_MAX_BUCKETS = 12000;    // two float64 rows of n_buckets + 1 f
 constexpr int SEL_MAX_MOD = 512;          // modules per search (coefficient vectors in shared memory)
 constexpr int SEL_MAX_CLUSTER = 16;       // CTAs (steps at a time) of one search
 constexpr int SEL_SMEM_MOD = 1024;        // up to here the per-module bounds are in shared memory
-constexpr size_t SEL_SMEM_MAX = 227 * 1024 - 8192;      // dynamic shared memory a kernel here may use
+constexpr int SEL_SMEM_MAX = 227 * 1024 - 8192;      // dynamic shared memory a kernel here may use
 
-// What one CTA works with.  The rows are in shared memory; so are the tables (priors p and units u of
-// every option) when they fit, otherwise they are formed module by module in the same place.
+// Everything a CTA keeps in shared memory is addressed as elements of this array, never through stored
+// pointers: the compiler then knows the address space, and a load is one shared-memory instruction.
+//   two value rows, each behind a guard entry of +inf (the value of a negative bucket);
+//   the priors and units of every option, or of one module at a time where not all fit;
+//   per-module bounds; argmins of the last modules in what is left.
+extern __shared__ double sel_smem[];
+
+__device__ __forceinline__ int* sel_ints() { return reinterpret_cast<int*>(sel_smem); }
+__device__ __forceinline__ unsigned char* sel_bytes() { return reinterpret_cast<unsigned char*>(sel_smem); }
+
+__host__ __device__ __forceinline__ int sel_pitch(int n_buckets) { return (n_buckets + 16) & ~15; }
+
+// Where the parts are (bytes); the same arithmetic on host and device.
+struct DpLayout {
+    int rows, p, u, row_cost, bounds, argmin, total;
+    bool resident, bounds_in_smem;
+    __host__ __device__ DpLayout(int n_mod, int max_opt, int n_buckets) {
+        rows = 2 * (n_buckets + 2) * (int)sizeof(double);
+        rows = (rows + 15) & ~15;
+        bounds_in_smem = n_mod <= SEL_SMEM_MOD;
+        const int b = bounds_in_smem ? (3 * n_mod + 2) * (int)sizeof(int) : 0;
+        const int costs = 2 * ((max_opt + 1) & ~1) * (int)sizeof(double2);
+        const long long all = (long long)n_mod * max_opt;
+        resident = rows + costs + b + all * (int)(sizeof(double) + sizeof(int)) <= SEL_SMEM_MAX;
+        const int n = resident ? (int)all : 0;
+        row_cost = rows;
+        p = row_cost + costs;
+        u = p + n * (int)sizeof(double);
+        bounds = u + n * (int)sizeof(int);
+        argmin = (bounds + b + 15) & ~15;
+        total = SEL_SMEM_MAX;
+    }
+};
+
+// What one CTA works with.
 struct DpCta {
     const float* loss; const float* base_loss; const float* time; const int* n_opt;
     int n_mod, max_opt, n_buckets;
     double per_unit;
-    double* f0; double* f1;          // value rows
-    double* p; int* u;               // [n_mod or 1][max_opt]
+    int p, u, cost;                  // elements of sel_smem as double, int, double2
     int* lo; int* hi;                // [n_mod + 1] each: row m is computed on lo[m] .. hi[m]
-    unsigned char* ch;               // [n_mod][n_buckets + 1] argmins (global)
+    int* at;                         // [n_mod]: where bucket 0 of module m's argmins is in sel_bytes()
+    int direct, fetched;             // modules >= direct keep them there, those >= fetched are copied there
+    unsigned char* ch;               // [n_mod][sel_pitch] argmins (global)
     bool resident;                   // all modules' tables at once
-};
-
-// Where the dynamic shared memory of a CTA goes; the same arithmetic on host and device.
-struct DpLayout {
-    size_t bounds, p, u, total;
-    bool resident, bounds_in_smem;
-    __host__ __device__ DpLayout(int n_mod, int max_opt, int n_buckets) {
-        const size_t rows = 2 * (size_t)(n_buckets + 1) * sizeof(double);
-        bounds_in_smem = n_mod <= SEL_SMEM_MOD;
-        p = rows;
-        const size_t b = bounds_in_smem ? (2 * (size_t)n_mod + 2) * sizeof(int) : 0;
-        const size_t all = (size_t)n_mod * max_opt;
-        resident = rows + b + all * (sizeof(double) + sizeof(int)) <= SEL_SMEM_MAX;
-        const size_t n = resident ? all : (size_t)max_opt;
-        u = p + n * sizeof(double);
-        bounds = u + n * sizeof(int);
-        total = bounds + b;
-    }
 };
 
 // Prior and units of one option; raises *nonfinite for a NaN (a coefficient is checked when used).
@@ -90,14 +106,14 @@ __device__ __forceinline__ void dp_option(const DpCta& w, int m, int s, double* 
 }
 
 __device__ __forceinline__ int dp_units(const DpCta& w, int m, int s) {
-    return w.resident ? w.u[(size_t)m * w.max_opt + s]
+    return w.resident ? sel_ints()[w.u + m * w.max_opt + s]
                       : (int)ceil((double)w.time[(size_t)m * w.max_opt + s] * w.per_unit);
 }
 
 __device__ __forceinline__ int dp_count(const DpCta& w, int m) { return min(max(w.n_opt[m], 0), w.max_opt); }
 
-// Tables (when resident) and bounds of a CTA; ends with a barrier.
-__device__ void dp_setup(DpCta& w, int* nonfinite) {
+// Tables (when resident), bounds and places of a CTA; ends with a barrier.
+__device__ void dp_setup(DpCta& w, const DpLayout& lay, int* nonfinite) {
     const int tid = threadIdx.x, lane = tid & 31;
     for (int m = tid >> 5; m < w.n_mod; m += SEL_WARPS) {
         const int no = dp_count(w, m);
@@ -106,57 +122,75 @@ __device__ void dp_setup(DpCta& w, int* nonfinite) {
             double p;
             int u;
             dp_option(w, m, s, &p, &u, nonfinite);
-            if (w.resident) { w.p[(size_t)m * w.max_opt + s] = p; w.u[(size_t)m * w.max_opt + s] = u; }
+            if (w.resident) { sel_smem[w.p + m * w.max_opt + s] = p; sel_ints()[w.u + m * w.max_opt + s] = u; }
             if (u <= w.n_buckets) most = max(most, u);
         }
         most = __reduce_max_sync(0xffffffffu, most);
         if (lane == 0) w.hi[m + 1] = most;
     }
     __syncthreads();
+    __shared__ int s_direct, s_fetched;
     if (tid == 0) {
         int lo = w.n_buckets, hi = 0;
         w.lo[w.n_mod] = lo;
         for (int m = w.n_mod - 1; m >= 0; --m) w.lo[m] = lo = max(0, lo - w.hi[m + 1]);
         w.hi[0] = 0;
         for (int m = 1; m <= w.n_mod; ++m) w.hi[m] = hi = min(w.n_buckets, hi + w.hi[m]);
+        int m = w.n_mod - 1, used = lay.argmin;
+        for (; m >= 0; --m) {
+            const int first = min(w.lo[m + 1], w.hi[m + 1]), n = w.hi[m + 1] - first + 1;
+            if (used + n > lay.total) break;
+            w.at[m] = used - first;
+            used += n;
+        }
+        s_direct = m + 1;
+        for (used = 0; m >= 0; --m) {            // over the value rows, when these are done with
+            const int first = min(w.lo[m + 1], w.hi[m + 1]) & ~15, n = (w.hi[m + 1] + 16 - first) & ~15;
+            if (used + n > lay.rows) break;
+            w.at[m] = used - first;
+            used += n;
+        }
+        s_fetched = m + 1;
     }
     __syncthreads();
+    w.direct = s_direct;
+    w.fetched = s_fetched;
 }
 
-// Floats as signed integers in the same order.
-__device__ __forceinline__ int float_order(float v) {
-    const int i = __float_as_int(v);
+// The upper word of a float64 as an integer that does not decrease with the value.
+__device__ __forceinline__ int value_order(double v) {
+    const int i = __double2hiint(v);
     return i ^ ((i >> 31) & 0x7fffffff);
 }
 
-// One row of the programme, buckets [lo, hi], by the whole CTA.  R: options per lane.
+// One row of the programme, buckets [lo, hi], by the whole CTA; f0 and f1 are the rows' places in
+// sel_smem, cost that of the module's (cost, units) pairs.  R: options a lane tests.
 template <int R>
-__device__ __forceinline__ void dp_row(const double* f0, double* f1, const double* p, const int* u, int no,
-                                       double coef, int lo, int hi, int hi_prev, unsigned char* ch,
-                                       int* nonfinite) {
+__device__ __forceinline__ void dp_row(int f0, int f1, int cost, int no, int lo, int hi, int hi_prev,
+                                       unsigned char* ch, int at) {
     const int lane = threadIdx.x & 31;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    const double2* table = reinterpret_cast<const double2*>(sel_smem) + cost;
     double c[R];
     int us[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int s = r * 32 + lane;
-        us[r] = s < no ? u[s] : 0x40000000;
-        c[r] = s < no ? coef * p[s] : inf;
-        if (c[r] != c[r]) *nonfinite = 1;
+        // a lane without an option holds a NaN, which sorts behind every bound
+        const double2 t = s < no ? table[s] : make_double2(__longlong_as_double(0x7ff8000000000000LL), 0.0);
+        c[r] = t.x;
+        us[r] = __double2loint(t.y);
     }
     for (int b0 = lo + (threadIdx.x >> 5) * SEL_BLK; b0 <= hi; b0 += SEL_WARPS * SEL_BLK) {
         const int b1 = min(b0 + SEL_BLK - 1, hi);
-        float low[R];
-        int bound = 0x7f800000;                                   // +inf
+        int low[R];
+        int bound = 0x7ff00000;                                   // +inf
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            if (r > 0 && r * 32 >= no) { low[r] = __int_as_float(0x7f800000); continue; }
-            const int i0 = min(b0 - us[r], hi_prev), i1 = min(b1 - us[r], hi_prev);
-            const double v0 = i0 >= 0 ? f0[i0] + c[r] : inf;
-            low[r] = __double2float_rd(i1 >= 0 ? f0[i1] + c[r] : inf);
-            const float up = __double2float_ru(v0);
-            if (up == up) bound = min(bound, float_order(up));
+            if (r > 0 && r * 32 >= no) break;
+            const double up = sel_smem[f0 + max(min(b0 - us[r], hi_prev), -1)] + c[r];
+            low[r] = value_order(sel_smem[f0 + max(min(b1 - us[r], hi_prev), -1)] + c[r]);
+            if (up == up) bound = min(bound, value_order(up));
         }
         bound = __reduce_min_sync(0xffffffffu, bound);
         double best0 = inf, best1 = inf;
@@ -164,26 +198,48 @@ __device__ __forceinline__ void dp_row(const double* f0, double* f1, const doubl
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (r > 0 && r * 32 >= no) break;
-            unsigned left = __ballot_sync(0xffffffffu, us[r] <= b1 && float_order(low[r]) <= bound);
+            unsigned left = __ballot_sync(0xffffffffu, low[r] <= bound);
             while (left) {
-                const int src = __ffs(left) - 1;
+                const int s = r * 32 + __ffs(left) - 1;
                 left &= left - 1;
-                const int uu = __shfl_sync(0xffffffffu, us[r], src);
-                const double cc = __shfl_sync(0xffffffffu, c[r], src);
-                const int i = b0 + lane - uu;
-                if (i >= 0) {
-                    const double v = f0[min(i, hi_prev)] + cc;
-                    if (v < best0) { best0 = v; arg0 = r * 32 + src; }
-                }
-                if (i + 32 >= 0) {
-                    const double v = f0[min(i + 32, hi_prev)] + cc;
-                    if (v < best1) { best1 = v; arg1 = r * 32 + src; }
-                }
+                const double2 t = table[s];
+                const int i = b0 + lane - __double2loint(t.y);
+                const double v0 = sel_smem[f0 + max(min(i, hi_prev), -1)] + t.x;
+                const double v1 = sel_smem[f0 + max(min(i + 32, hi_prev), -1)] + t.x;
+                if (v0 < best0) { best0 = v0; arg0 = s; }
+                if (v1 < best1) { best1 = v1; arg1 = s; }
             }
         }
         const int b = b0 + lane;
-        if (b <= hi) { f1[b] = best0; ch[b] = (unsigned char)arg0; }
-        if (b + 32 <= hi) { f1[b + 32] = best1; ch[b + 32] = (unsigned char)arg1; }
+        if (b <= hi) sel_smem[f1 + b] = best0;
+        if (b + 32 <= hi) sel_smem[f1 + b + 32] = best1;
+        if (ch) {
+            if (b <= hi) ch[b] = (unsigned char)arg0;
+            if (b + 32 <= hi) ch[b + 32] = (unsigned char)arg1;
+        } else {
+            if (b <= hi) sel_bytes()[at + b] = (unsigned char)arg0;
+            if (b + 32 <= hi) sel_bytes()[at + b + 32] = (unsigned char)arg1;
+        }
+    }
+}
+
+// (cost, units) pairs of module m into half m & 1 of the cost table, by the whole CTA.
+__device__ __forceinline__ void dp_costs(const DpCta& w, int m, const float* coef, int* nonfinite) {
+    const int no = dp_count(w, m);
+    double2* table = reinterpret_cast<double2*>(sel_smem) + w.cost + (m & 1) * ((w.max_opt + 1) & ~1);
+    // the last threads: where warps have unequal numbers of blocks, theirs have fewer
+    for (int s = SEL_THREADS - 1 - (int)threadIdx.x; s < no; s += SEL_THREADS) {
+        double p;
+        int u;
+        if (w.resident) {
+            p = sel_smem[w.p + m * w.max_opt + s];
+            u = sel_ints()[w.u + m * w.max_opt + s];
+        } else {
+            dp_option(w, m, s, &p, &u, nonfinite);
+        }
+        const double c = (double)coef[m] * p;
+        if (c != c) *nonfinite = 1;
+        table[s] = make_double2(c, __hiloint2double(0, u));
     }
 }
 
@@ -192,59 +248,47 @@ __device__ __forceinline__ void dp_row(const double* f0, double* f1, const doubl
 // n_mod) (global) holds the chosen options.  *nonfinite is a shared flag that is raised when a cost
 // is NaN.  Ends with a barrier.
 template <int R>
-__device__ double dp_solve(DpCta& w, const float* coef, int* nonfinite, int* sel) {
-    const int tid = threadIdx.x, lane = tid & 31, B = w.n_buckets;
-    const size_t pitch = (size_t)(B + 1);
+__device__ double dp_solve(const DpCta& w, const float* coef, int* nonfinite, int* sel) {
+    const int tid = threadIdx.x, lane = tid & 31, B = w.n_buckets, pitch = sel_pitch(B);
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    double* f0 = w.f0;
-    double* f1 = w.f1;
-    if (tid == 0) f0[0] = 0.0;                   // row 0 is 0 everywhere: hi[0] = 0
+    int f0 = 1, f1 = B + 3;
+    if (tid == 0) {
+        sel_smem[f0 - 1] = sel_smem[f1 - 1] = inf;
+        sel_smem[f0] = 0.0;                      // row 0 is 0 everywhere: hi[0] = 0
+    }
+    dp_costs(w, 0, coef, nonfinite);
     __syncthreads();
     int hi = 0;
     for (int m = 0; m < w.n_mod; ++m) {
-        const int no = dp_count(w, m), next = w.hi[m + 1];
-        const double* p = w.p;
-        const int* u = w.u;
-        if (w.resident) {
-            p += (size_t)m * w.max_opt;
-            u += (size_t)m * w.max_opt;
-        } else {
-            for (int s = tid; s < no; s += SEL_THREADS) dp_option(w, m, s, w.p + s, w.u + s, nonfinite);
-            __syncthreads();
-        }
-        dp_row<R>(f0, f1, p, u, no, (double)coef[m], min(w.lo[m + 1], next), next, hi, w.ch + m * pitch,
-                  nonfinite);
+        const int next = w.hi[m + 1];
+        if (m + 1 < w.n_mod) dp_costs(w, m + 1, coef, nonfinite);
+        const bool direct = m >= w.direct;
+        dp_row<R>(f0, f1, w.cost + (m & 1) * ((w.max_opt + 1) & ~1), dp_count(w, m), min(w.lo[m + 1], next), next,
+                  hi, direct ? nullptr : w.ch + (size_t)m * pitch, direct ? w.at[m] : 0);
         __syncthreads();
-        double* t = f0; f0 = f1; f1 = t;
+        const int t = f0; f0 = f1; f1 = t;
         hi = next;
     }
-    const double total = f0[hi];
-    if (total < inf && tid < 32) {
-        // walk back, two modules a round: the argmins of module m - 1 for every option of module m
-        // are fetched together with module m's own, so a round waits for memory once
-        int b = B;
-        for (int m = w.n_mod - 1; m >= 0; m -= 2) {
-            const int no = dp_count(w, m), prev = w.hi[m], first = min(w.lo[m], prev);
-            const int s = w.ch[m * pitch + min(b, w.hi[m + 1])];
-            int um = 0, s1 = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int o = r * 32 + lane;
-                int u = 0, c = 0;
-                if (o < no) {
-                    u = dp_units(w, m, o);
-                    const int i = min(b - u, prev);
-                    if (m > 0 && i >= first) c = w.ch[(m - 1) * pitch + i];
-                }
-                u = __shfl_sync(0xffffffffu, u, s & 31);
-                c = __shfl_sync(0xffffffffu, c, s & 31);
-                if ((s >> 5) == r) { um = u; s1 = c; }
-            }
-            b -= um;
-            if (lane == 0) sel[m] = s;
-            if (m > 0) {
-                if (lane == 0) sel[m - 1] = s1;
-                b -= dp_units(w, m - 1, s1);
+    const double total = sel_smem[f0 + hi];
+    __syncthreads();
+    if (total < inf) {
+        // the walk is a chain of one look-up per module: bring the argmins that are in global memory
+        // over the value rows first, two warps a module
+        for (int m = w.direct - 1 - (tid >> 6); m >= w.fetched; m -= SEL_THREADS / 64) {
+            const int first = min(w.lo[m + 1], w.hi[m + 1]) & ~15, n = (w.hi[m + 1] + 16 - first) / 16;
+            const uint4* src = reinterpret_cast<const uint4*>(w.ch + (size_t)m * pitch + first);
+            uint4* dst = reinterpret_cast<uint4*>(sel_bytes() + w.at[m] + first);
+#pragma unroll 4
+            for (int e = tid & 63; e < n; e += 64) dst[e] = src[e];
+        }
+        __syncthreads();
+        if (tid < 32) {
+            int b = B;
+            for (int m = w.n_mod - 1; m >= 0; --m) {
+                const int i = min(b, w.hi[m + 1]);
+                const int s = m >= w.fetched ? sel_bytes()[w.at[m] + i] : w.ch[(size_t)m * pitch + i];
+                if (lane == 0) sel[m] = s;
+                b -= dp_units(w, m, s);
             }
         }
     }
@@ -266,22 +310,20 @@ __device__ double dp_sum(const DpCta& w, const float* row, const int* sel, bool 
     return acc;
 }
 
-__device__ __forceinline__ void dp_bind(DpCta& w, const float* loss, const float* base_loss, const float* time,
-                                        const int* n_opt, int n_mod, int max_opt, int n_buckets,
-                                        double per_unit, unsigned char* ch, int* bounds) {
-    extern __shared__ double sel_smem[];
-    const DpLayout at(n_mod, max_opt, n_buckets);
-    char* base = reinterpret_cast<char*>(sel_smem);
+__device__ __forceinline__ void dp_bind(DpCta& w, const DpLayout& lay, const float* loss, const float* base_loss,
+                                        const float* time, const int* n_opt, int n_mod, int max_opt,
+                                        int n_buckets, double per_unit, unsigned char* choice, int* bounds) {
     w.loss = loss; w.base_loss = base_loss; w.time = time; w.n_opt = n_opt;
     w.n_mod = n_mod; w.max_opt = max_opt; w.n_buckets = n_buckets; w.per_unit = per_unit;
-    w.f0 = sel_smem;
-    w.f1 = sel_smem + (n_buckets + 1);
-    w.p = reinterpret_cast<double*>(base + at.p);
-    w.u = reinterpret_cast<int*>(base + at.u);
-    w.lo = at.bounds_in_smem ? reinterpret_cast<int*>(base + at.bounds) : bounds;
+    w.p = lay.p / (int)sizeof(double);
+    w.u = lay.u / (int)sizeof(int);
+    w.cost = lay.row_cost / (int)sizeof(double2);
+    w.lo = lay.bounds_in_smem ? sel_ints() + lay.bounds / (int)sizeof(int)
+                              : bounds + blockIdx.x * (3 * (size_t)n_mod + 2);
     w.hi = w.lo + n_mod + 1;
-    w.ch = ch;
-    w.resident = at.resident;
+    w.at = w.hi + n_mod + 1;
+    w.ch = choice + blockIdx.x * ((size_t)n_mod * sel_pitch(n_buckets));
+    w.resident = lay.resident;
 }
 
 // One CTA per SM takes candidates blockIdx.x, blockIdx.x + gridDim.x, ...: the tables are formed once
@@ -295,14 +337,16 @@ k_select_levels(const float* __restrict__ loss, const float* __restrict__ base_l
                 int* __restrict__ status) {
     __shared__ int s_table_bad, s_nonfinite;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    const DpLayout lay(n_mod, max_opt, n_buckets);
     DpCta w;
-    dp_bind(w, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budget,
-            choice + blockIdx.x * ((size_t)n_mod * (n_buckets + 1)), bounds + blockIdx.x * (2 * (size_t)n_mod + 2));
+    dp_bind(w, lay, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budget, choice,
+            bounds);
     if (threadIdx.x == 0) s_table_bad = 0;
     __syncthreads();
-    dp_setup(w, &s_table_bad);
+    dp_setup(w, lay, &s_table_bad);
     for (int k = blockIdx.x; k < K; k += gridDim.x) {
         if (threadIdx.x == 0) s_nonfinite = s_table_bad;
+        __syncthreads();
         int* sel = selected + (size_t)k * n_mod;
         const double total = dp_solve<R>(w, coef + (size_t)k * n_mod, &s_nonfinite, sel);
         if (threadIdx.x < 32) {
@@ -348,16 +392,17 @@ k_search_levels(const float* __restrict__ loss, const float* __restrict__ base_l
     const int P = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int k = blockIdx.x / P, tid = threadIdx.x;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    const DpLayout lay(n_mod, max_opt, n_buckets);
     DpCta w;
-    dp_bind(w, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budgets[k],
-            choice + blockIdx.x * ((size_t)n_mod * (n_buckets + 1)), bounds + blockIdx.x * (2 * (size_t)n_mod + 2));
+    dp_bind(w, lay, loss, base_loss, time, n_opt, n_mod, max_opt, n_buckets, (double)n_buckets / budgets[k], choice,
+            bounds);
     int* trial = trial_sel + (size_t)blockIdx.x * n_mod;
     const unsigned char* mk = mask + (size_t)k * n_steps * n_mod;
     const float* val = values + (size_t)k * n_steps * n_mod;
     if (tid == 0) s_nonfinite = 0;
     for (int m = tid; m < n_mod; m += SEL_THREADS) c_best[m] = coef0[(size_t)k * n_mod + m];
     __syncthreads();
-    dp_setup(w, &s_nonfinite);
+    dp_setup(w, lay, &s_nonfinite);
     const int table_bad = s_nonfinite;
     double best = inf;
     bool bad = false;
@@ -371,7 +416,8 @@ k_search_levels(const float* __restrict__ loss, const float* __restrict__ base_l
                 c_try[m] = c;
             }
             if (tid == 0) s_nonfinite = table_bad;
-            const double total = dp_solve<R>(w, c_try, &s_nonfinite, trial);     // opens with a barrier
+            __syncthreads();
+            const double total = dp_solve<R>(w, c_try, &s_nonfinite, trial);
             if (tid < 32) {
                 const double score = total < inf ? dp_sum(w, objective, trial, false) : inf;
                 if (tid < P) {
@@ -430,8 +476,8 @@ F by_options(int max_opt, F r1, F r2, F r8) { return max_opt <= 32 ? r1 : max_op
 }  // namespace
 
 size_t select_workspace_bytes(int K, int n_mod, int n_buckets) {
-    return align_up((size_t)K * n_mod * (size_t)(n_buckets + 1)) +
-           align_up((size_t)K * (2 * (size_t)n_mod + 2) * sizeof(int));
+    return align_up((size_t)K * n_mod * (size_t)sel_pitch(n_buckets)) +
+           align_up((size_t)K * (3 * (size_t)n_mod + 2) * sizeof(int));
 }
 
 ziplm_status run_select_levels(const float* loss, const float* base_loss, const float* time,
@@ -441,8 +487,8 @@ ziplm_status run_select_levels(const float* loss, const float* base_loss, const 
     if (max_opt > SEL_MAX_OPT || n_buckets > SEL_MAX_BUCKETS) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < select_workspace_bytes(K, n_mod, n_buckets)) return ZIPLM_ERR_WORKSPACE;
     Carver c(ws);
-    unsigned char* choice = c.take<unsigned char>((size_t)K * n_mod * (size_t)(n_buckets + 1));
-    int* bounds = c.take<int>((size_t)K * (2 * (size_t)n_mod + 2));
+    unsigned char* choice = c.take<unsigned char>((size_t)K * n_mod * (size_t)sel_pitch(n_buckets));
+    int* bounds = c.take<int>((size_t)K * (3 * (size_t)n_mod + 2));
     int dev = 0, sms = 0;
     ZIPLM_CHECK_CUDA(cudaGetDevice(&dev));
     ZIPLM_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -458,8 +504,8 @@ ziplm_status run_select_levels(const float* loss, const float* base_loss, const 
 
 size_t search_workspace_bytes(int S, int n_mod, int n_buckets) {
     const size_t n = (size_t)search_slices(S);
-    return align_up(n * n_mod * (size_t)(n_buckets + 1)) + align_up(n * n_mod * sizeof(int)) +
-           align_up(n * (2 * (size_t)n_mod + 2) * sizeof(int));
+    return align_up(n * n_mod * (size_t)sel_pitch(n_buckets)) + align_up(n * n_mod * sizeof(int)) +
+           align_up(n * (3 * (size_t)n_mod + 2) * sizeof(int));
 }
 
 ziplm_status run_search_levels(const float* loss, const float* base_loss, const float* time,
@@ -472,9 +518,9 @@ ziplm_status run_search_levels(const float* loss, const float* base_loss, const 
     if (ws_bytes < search_workspace_bytes(S, n_mod, n_buckets)) return ZIPLM_ERR_WORKSPACE;
     const int slices = search_slices(S);
     Carver c(ws);
-    unsigned char* choice = c.take<unsigned char>((size_t)slices * n_mod * (size_t)(n_buckets + 1));
+    unsigned char* choice = c.take<unsigned char>((size_t)slices * n_mod * (size_t)sel_pitch(n_buckets));
     int* trial = c.take<int>((size_t)slices * n_mod);
-    int* bounds = c.take<int>((size_t)slices * (2 * (size_t)n_mod + 2));
+    int* bounds = c.take<int>((size_t)slices * (3 * (size_t)n_mod + 2));
     const size_t smem = DpLayout(n_mod, max_opt, n_buckets).total;
     auto kernel = by_options(max_opt, k_search_levels<1>, k_search_levels<2>, k_search_levels<8>);
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
