@@ -100,7 +100,7 @@ ziplm_status ziplm_damped_inverse(const float* H, int L, int d, float damp_frac,
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(layer_status, 0, sizeof(int) * L, st));
     PhaseScope ps(PH_INVERSE, st);
-    return run_damped_inverse(H, L, d, damp_frac, Hinv, nullptr, 0, nullptr, nullptr, layer_status,
+    return run_damped_inverse(H, L, d, damp_frac, Hinv, nullptr, 0, 0, nullptr, nullptr, layer_status,
                               workspace, workspace_bytes, st);
 }
 

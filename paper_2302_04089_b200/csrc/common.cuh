@@ -75,9 +75,9 @@ size_t inverse_workspace_bytes(int L, int d);
 
 // (H + lambda I)^-1 in float64.  out64 (may be null) receives the full symmetric [L, d, d]
 // matrix; tri32/diag64 (may be null) receive the strictly lower triangle in fp32 with row pitch
-// `pitch32` and the diagonal in float64; lam_out (may be null) receives lambda per layer.
+// `pitch32`, rows32 rows per layer, and the diagonal in float64 (rows32 entries per layer); lam_out (may be null) receives lambda per layer.
 ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, double* out64,
-                                float* tri32, int pitch32, double* diag64, double* lam_out,
+                                float* tri32, int pitch32, int rows32, double* diag64, double* lam_out,
                                 int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st);
 
 size_t neuron_workspace_bytes(int L, int r, int d, int n_levels);

@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_factor_small(double* A, do
 // triangles) + fp64 diag.
 // One CTA per 128 x 64 macro tile that reaches the lower triangle.
 __global__ void __launch_bounds__(GT, 2) k_lauum(const double* M, int dp, int T, int d, double* out64,
-                                                 float* tri32, int pitch32, double* diag64) {
+                                                 float* tri32, int pitch32, int rows32, double* diag64) {
     extern __shared__ __align__(16) double smem[];
     const int l = blockIdx.y;
     int I, J;
@@ -694,11 +694,11 @@ __global__ void __launch_bounds__(GT, 2) k_lauum(const double* M, int dp, int T,
                     o[(size_t)col * d + row] = v;
                 }
                 if (tri32 && row > col) {       // both triangles: a column can then be read as a row
-                    float* t = tri32 + (size_t)l * d * pitch32;
+                    float* t = tri32 + (size_t)l * rows32 * pitch32;
                     t[(size_t)row * pitch32 + col] = (float)v;
                     t[(size_t)col * pitch32 + row] = (float)v;
                 }
-                if (diag64 && row == col) diag64[(size_t)l * d + row] = v;
+                if (diag64 && row == col) diag64[(size_t)l * rows32 + row] = v;
             }
 }
 
@@ -804,7 +804,7 @@ size_t inverse_workspace_bytes(int L, int d) {
 }
 
 ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, double* out64,
-                                float* tri32, int pitch32, double* diag64, double* lam_out,
+                                float* tri32, int pitch32, int rows32, double* diag64, double* lam_out,
                                 int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (ws_bytes < inverse_workspace_bytes(L, d)) return ZIPLM_ERR_WORKSPACE;
     const int dp = round_up_int(d, kTile), T = dp / kTile;
@@ -828,7 +828,7 @@ ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, d
             k_lauum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProductSmemBytes);
         if (attr != cudaSuccess) return ZIPLM_ERR_CUDA;
         k_lauum<<<dim3(lower_macro_count(T), L), GT, kProductSmemBytes, st>>>(ctx.M, dp, T, d, out64, tri32,
-                                                                            pitch32, diag64);
+                                                                            pitch32, rows32, diag64);
         ZIPLM_CHECK_LAUNCH();
     }
     if (lam_out) {
@@ -873,6 +873,6 @@ extern "C" ziplm_status ziplm_damped_inverse_noalloc(const float* H, int L, int 
     // Every part of the scratch that a kernel reads is written earlier in the same call (the
     // damped copy, the factor, the lower tiles of its inverse, lambda), so nothing left behind
     // by the previous call needs clearing.
-    return run_damped_inverse(H, L, d, damp_frac, Hinv, nullptr, 0, nullptr, nullptr, layer_status,
+    return run_damped_inverse(H, L, d, damp_frac, Hinv, nullptr, 0, 0, nullptr, nullptr, layer_status,
                               scratch, kBuiltinScratchBytes, st);
 }

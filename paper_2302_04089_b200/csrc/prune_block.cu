@@ -448,7 +448,7 @@ ziplm_status run_prune_blocks(const float* W, const float* H, int L, int r, int 
     ziplm_status s;
     {
         PhaseScope ps(PH_INVERSE, st);
-        s = run_damped_inverse(H, L, d, damp_frac, w.A, nullptr, 0, nullptr, w.lam, layer_status,
+        s = run_damped_inverse(H, L, d, damp_frac, w.A, nullptr, 0, 0, nullptr, w.lam, layer_status,
                                w.inv_ws, w.inv_bytes, st);
     }
     if (s != ZIPLM_OK) return s;

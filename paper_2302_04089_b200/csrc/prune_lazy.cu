@@ -62,8 +62,10 @@ struct LazyState {
     int pad;
 };
 
-// Wt = W^T (zero padded to rp), float64 column norms, identity index, state reset.
-__global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, int r, int d, int rp,
+// Wt = W^T (zero padded to rp), float64 column norms, identity index, state reset.  Positions d .. ld - 1
+// (ld: d rounded up to 4, the pitch of the matrices) get index -1 and zero weights: they are removed from
+// the start.
+__global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, int r, int d, int ld, int rp,
                                                    float* __restrict__ Wt, double* __restrict__ dQ,
                                                    int* __restrict__ idx,
                                                    LazyState* __restrict__ state) {
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
     const int c0 = blockIdx.x * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const float* Wl = W + (size_t)l * r * d;
-    float* Wtl = Wt + (size_t)l * d * rp;
+    float* Wtl = Wt + (size_t)l * ld * rp;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int i0 = 0; i0 < rp; i0 += 32) {
 #pragma unroll
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
             const int cc = ty + 8 * m;
             const int c = c0 + cc, i = i0 + tx;
             const float v = tile[tx][cc];
-            if (c < d && i < rp) Wtl[(size_t)c * rp + i] = v;
+            if (c < ld && i < rp) Wtl[(size_t)c * rp + i] = v;
             acc[m] += (double)v * (double)v;
         }
         __syncthreads();
@@ -98,13 +100,13 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const int c = c0 + ty + 8 * m;
-        if (tx == 0 && c < d) {
-            dQ[(size_t)l * d + c] = s;
-            idx[(size_t)l * d + c] = c;
+        if (tx == 0 && c < ld) {
+            dQ[(size_t)l * ld + c] = s;
+            idx[(size_t)l * ld + c] = c < d ? c : -1;
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        state[l].sumrho = 0.0; state[l].dw2 = 0.0; state[l].n_new = d; state[l].pad = 0;
+        state[l].sumrho = 0.0; state[l].dw2 = 0.0; state[l].n_new = ld; state[l].pad = 0;
     }
 }
 
@@ -718,7 +720,7 @@ __global__ void __launch_bounds__(256, 3) k_lazy_update_w(int n_new, int m, int 
 constexpr int kRefresh = 64;
 __device__ void lazy_refresh_gram(int n, int d, int r, int rp, const float* __restrict__ Wl,
                                   float* __restrict__ Ql, double* __restrict__ dQl, float* sW);
-__global__ void __launch_bounds__(256) k_lazy_refresh(int n, int d, int r, int rp,
+__global__ void __launch_bounds__(256) k_lazy_refresh(int n, int d_in, int d, int r, int rp,
                                                       const float* __restrict__ H,
                                                       const double* __restrict__ lam,
                                                       const int* __restrict__ idx,
@@ -736,14 +738,14 @@ __global__ void __launch_bounds__(256) k_lazy_refresh(int n, int d, int r, int r
                           dQ + (size_t)l * d, reinterpret_cast<float*>(dyn_refresh));
         return;
     }
-    const float* Hl = H + (size_t)l * d * d;
+    const float* Hl = H + (size_t)l * d_in * d_in;       // the caller's H has the width d_in itself as its pitch
     float* Al = A + (size_t)l * d * d;
     if (tid == 0) flag = 0;
     if (tid < n) sidx[tid] = idx[(size_t)l * d + tid];
     __syncthreads();
     for (int e = tid; e < n * n; e += 256) {
         const int i = e / n, j = e % n;
-        sB[i][j] = (double)Hl[(size_t)sidx[i] * d + sidx[j]] + (i == j ? lam[l] : 0.0);
+        sB[i][j] = (double)Hl[(size_t)sidx[i] * d_in + sidx[j]] + (i == j ? lam[l] : 0.0);
     }
     __syncthreads();
     // Cholesky B = C C^T, column by column
@@ -840,7 +842,7 @@ __global__ void __launch_bounds__(256) k_lazy_pos_of(int n, int d, const int* __
 
 // W_snap = current weights in original column order, removed columns exactly zero; accumulates
 // ||W - W_snap||_F^2 for the loss identity.
-__global__ void __launch_bounds__(256) k_lazy_snapshot(int r, int d, int rp,
+__global__ void __launch_bounds__(256) k_lazy_snapshot(int r, int d, int ld, int rp,
                                                        const float* __restrict__ W,
                                                        const float* __restrict__ Wt,
                                                        const int* __restrict__ pos_of,
@@ -851,11 +853,11 @@ __global__ void __launch_bounds__(256) k_lazy_snapshot(int r, int d, int rp,
     const int l = blockIdx.z;
     const int c0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const float* Wtl = Wt + (size_t)l * d * rp;
+    const float* Wtl = Wt + (size_t)l * ld * rp;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         const int cc = ty + 8 * m, c = c0 + cc, i = i0 + tx;
-        const int pos = (c < d) ? pos_of[(size_t)l * d + c] : -1;
+        const int pos = (c < d) ? pos_of[(size_t)l * ld + c] : -1;
         tile[cc][tx] = (pos >= 0 && i < r) ? Wtl[(size_t)pos * rp + i] : 0.f;
     }
     __syncthreads();
@@ -893,19 +895,28 @@ __global__ void k_lazy_loss(int L, int n_levels, int slot, const double* __restr
 }
 
 // base_loss = ||W X||_F^2 = 1/2 tr(W H W^T) = 1/2 <W^T W, H>: one elementwise pass over the Gram
-// matrix (full symmetric right after the product kernel) and the undamped Hessian.
-__global__ void __launch_bounds__(256) k_lazy_base_loss(int d, const float* __restrict__ Q,
+// matrix (pitch ld, full symmetric right after the product kernel) and the undamped Hessian (pitch d).
+__global__ void __launch_bounds__(256) k_lazy_base_loss(int d, int ld, const float* __restrict__ Q,
                                                         const float* __restrict__ H,
                                                         double* __restrict__ acc64) {
     __shared__ double red[8];
     const int l = blockIdx.y;
-    const size_t count = (size_t)d * d / 4;
-    const float4* q4 = reinterpret_cast<const float4*>(Q + (size_t)l * d * d);
-    const float4* h4 = reinterpret_cast<const float4*>(H + (size_t)l * d * d);
+    const float* Ql = Q + (size_t)l * ld * ld;
+    const float* Hl = H + (size_t)l * d * d;
     double acc = 0.0;
-    for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < count; e += (size_t)gridDim.x * 256) {
-        const float4 a = __ldg(q4 + e), b = __ldg(h4 + e);
-        acc += (double)a.x * b.x + (double)a.y * b.y + (double)a.z * b.z + (double)a.w * b.w;
+    if (d == ld) {
+        const size_t count = (size_t)d * d / 4;
+        const float4* q4 = reinterpret_cast<const float4*>(Ql);
+        const float4* h4 = reinterpret_cast<const float4*>(Hl);
+        for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < count; e += (size_t)gridDim.x * 256) {
+            const float4 a = __ldg(q4 + e), b = __ldg(h4 + e);
+            acc += (double)a.x * b.x + (double)a.y * b.y + (double)a.z * b.z + (double)a.w * b.w;
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < d; i += gridDim.x * 8)
+            for (int j = lane; j < d; j += 32)
+                acc += (double)Ql[(size_t)i * ld + j] * Hl[(size_t)i * d + j];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -931,31 +942,33 @@ struct LazyWs {
     float* P; int* sched;              // packed operands and work counter of the tensor-core update
     LazyState* state; double* lam; double* base_acc;
     void* aux; size_t aux_bytes;       // shared by the inverse and by the Gram-matrix product
-    int rp; size_t total;
+    int rp, ld; size_t total;
 };
 
 LazyWs carve_lazy(void* ws, int L, int r, int d) {
     LazyWs w;
     w.rp = round_up_int(r, 4);
+    w.ld = round_up_int(d, 4);
+    const int ld = w.ld;
     Carver c(ws);
-    for (int b = 0; b < 2; ++b) w.A[b] = c.take<float>((size_t)L * d * d);
-    for (int b = 0; b < 2; ++b) w.Q[b] = c.take<float>((size_t)L * d * d);
-    for (int b = 0; b < 2; ++b) w.Wt[b] = c.take<float>((size_t)L * d * w.rp);
-    for (int b = 0; b < 2; ++b) w.dA[b] = c.take<double>((size_t)L * d);
-    for (int b = 0; b < 2; ++b) w.dQ[b] = c.take<double>((size_t)L * d);
-    for (int b = 0; b < 2; ++b) w.idx[b] = c.take<int>((size_t)L * d);
-    w.src = c.take<int>((size_t)L * d);
-    w.pos_of = c.take<int>((size_t)L * d);
-    w.U = c.take<float>((size_t)L * BMAX * d);
-    w.Z = c.take<float>((size_t)L * BMAX * d);
+    for (int b = 0; b < 2; ++b) w.A[b] = c.take<float>((size_t)L * ld * ld);
+    for (int b = 0; b < 2; ++b) w.Q[b] = c.take<float>((size_t)L * ld * ld);
+    for (int b = 0; b < 2; ++b) w.Wt[b] = c.take<float>((size_t)L * ld * w.rp);
+    for (int b = 0; b < 2; ++b) w.dA[b] = c.take<double>((size_t)L * ld);
+    for (int b = 0; b < 2; ++b) w.dQ[b] = c.take<double>((size_t)L * ld);
+    for (int b = 0; b < 2; ++b) w.idx[b] = c.take<int>((size_t)L * ld);
+    w.src = c.take<int>((size_t)L * ld);
+    w.pos_of = c.take<int>((size_t)L * ld);
+    w.U = c.take<float>((size_t)L * BMAX * ld);
+    w.Z = c.take<float>((size_t)L * BMAX * ld);
     w.C = c.take<float>((size_t)L * BMAX * w.rp);
-    w.P = c.take<float>(lazy_tc_pack_floats(L, d, w.rp));
+    w.P = c.take<float>(lazy_tc_pack_floats(L, ld, w.rp));
     w.sched = c.take<int>(2);
     w.state = c.take<LazyState>((size_t)L);
     w.lam = c.take<double>((size_t)L);
     w.base_acc = c.take<double>((size_t)L);
     const size_t inv = inverse_workspace_bytes(L, d);
-    const size_t gram = hessian_tc_workspace_bytes(L, d, w.rp, ZIPLM_F32, false);
+    const size_t gram = hessian_tc_workspace_bytes(L, ld, w.rp, ZIPLM_F32, false);
     w.aux_bytes = inv > gram ? inv : gram;
     w.aux = c.take<char>(w.aux_bytes);
     w.total = c.off;
@@ -964,7 +977,7 @@ LazyWs carve_lazy(void* ws, int L, int r, int d) {
 
 }  // namespace
 
-bool lazy_path_supported(int d) { return d % 4 == 0 && d <= CLUSTER_MAX * SLICE_MAX && d >= 4; }
+bool lazy_path_supported(int d) { return d >= 1 && d <= CLUSTER_MAX * SLICE_MAX; }
 
 size_t lazy_workspace_bytes(int L, int r, int d, int n_levels) {
     (void)n_levels;
@@ -978,11 +991,13 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     if (!lazy_path_supported(d)) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < lazy_workspace_bytes(L, r, d, n_levels)) return ZIPLM_ERR_WORKSPACE;
     LazyWs w = carve_lazy(ws, L, r, d);
-    const int G = d, rp = w.rp;
+    // The matrices have the pitch ld = d rounded up to 4, so that every row starts on 16 bytes (128-bit
+    // loads, TMA); the up to three positions behind d are treated as removed ones.
+    const int G = d, rp = w.rp, ld = w.ld;
     ziplm_status s;
     {
         PhaseScope ps(PH_INVERSE, st);
-        s = run_damped_inverse(H, L, d, damp_frac, nullptr, w.A[0], d, w.dA[0], w.lam, layer_status,
+        s = run_damped_inverse(H, L, d, damp_frac, nullptr, w.A[0], ld, ld, w.dA[0], w.lam, layer_status,
                                w.aux, w.aux_bytes, st);
     }
     if (s != ZIPLM_OK) return s;
@@ -991,16 +1006,16 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         ZIPLM_CHECK_CUDA(cudaMemsetAsync(order, 0xFF, sizeof(int) * (size_t)L * G, st));
         if (saliency)
             ZIPLM_CHECK_CUDA(cudaMemsetAsync(saliency, 0, sizeof(float) * (size_t)L * G, st));
-        k_lazy_init<<<dim3((d + 31) / 32, L), 256, 0, st>>>(W, r, d, rp, w.Wt[0], w.dQ[0], w.idx[0],
+        k_lazy_init<<<dim3((ld + 31) / 32, L), 256, 0, st>>>(W, r, d, ld, rp, w.Wt[0], w.dQ[0], w.idx[0],
                                                            w.state);
         ZIPLM_CHECK_LAUNCH();
         // Q = W^T W: the symmetric product kernel of the Hessian with X = W^T (K = d_row)
-        ziplm_status g = run_hessian_tc(w.Q[0], w.Wt[0], ZIPLM_F32, false, L, d, rp, rp, 1.0f, 0.0f, w.aux,
+        ziplm_status g = run_hessian_tc(w.Q[0], w.Wt[0], ZIPLM_F32, false, L, ld, rp, rp, 1.0f, 0.0f, w.aux,
                                         w.aux_bytes, st);
         if (g != ZIPLM_OK) return g;
         if (base_loss) {
             ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.base_acc, 0, sizeof(double) * L, st));
-            k_lazy_base_loss<<<dim3(148, L), 256, 0, st>>>(d, w.Q[0], H, w.base_acc);
+            k_lazy_base_loss<<<dim3(148, L), 256, 0, st>>>(d, ld, w.Q[0], H, w.base_acc);
             ZIPLM_CHECK_LAUNCH();
             k_lazy_base_finish<<<(L + 63) / 64, 64, 0, st>>>(L, w.base_acc, base_loss);
             ZIPLM_CHECK_LAUNCH();
@@ -1015,35 +1030,36 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     int cur = 0;
     auto snapshot = [&](int n, int slot) -> ziplm_status {
         PhaseScope ps(PH_SNAPSHOT, st);
-        k_lazy_pos_of<<<L, 256, 0, st>>>(n, d, w.idx[cur], w.pos_of);
+        k_lazy_pos_of<<<L, 256, 0, st>>>(n, ld, w.idx[cur], w.pos_of);
         ZIPLM_CHECK_LAUNCH();
         k_lazy_snapshot<<<dim3((d + 31) / 32, (r + 31) / 32, L), 256, 0, st>>>(
-            r, d, rp, W, w.Wt[cur], w.pos_of, W_snap, n_levels, slot, w.state);
+            r, d, ld, rp, W, w.Wt[cur], w.pos_of, W_snap, n_levels, slot, w.state);
         ZIPLM_CHECK_LAUNCH();
         k_lazy_loss<<<(L + 63) / 64, 64, 0, st>>>(L, n_levels, slot, w.lam, w.state, loss);
         ZIPLM_CHECK_LAUNCH();
         return ZIPLM_OK;
     };
 
-    int n = G, slot = 0, t = 0;
+    int slot = 0, t = 0;
+    int n = G;
     int prio_least = 0, prio_greatest = 0;
     ZIPLM_CHECK_CUDA(cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest));
     const int steps_priority = prio_greatest;
     if (slot < n_levels && levels[slot] == n) {
-        s = snapshot(n, slot++);
+        s = snapshot(ld, slot++);
         if (s != ZIPLM_OK) return s;
     }
     const int n_min = n_levels > 0 ? levels[n_levels - 1] : G;
     // n = live structures, npos = positions of the arrays (live ones and those removed since the
     // last block that squeezed the removed positions out)
-    int npos = G;
+    int npos = ld;
     const bool every_block = option_value(ZIPLM_OPT_COMPACT_EVERY_BLOCK) == 1;
     CUtensorMap map_p, map_a[2], map_q[2], map_w[2];
-    if (!lazy_tc_make_map(&map_p, w.P, L, d, rp)) return ZIPLM_ERR_CUDA;
+    if (!lazy_tc_make_map(&map_p, w.P, L, ld, rp)) return ZIPLM_ERR_CUDA;
     for (int b = 0; b < 2; ++b)
-        if (!lazy_tc_make_matrix_map(&map_a[b], w.A[b], L, d, d) ||
-            !lazy_tc_make_matrix_map(&map_q[b], w.Q[b], L, d, d) ||
-            !lazy_tc_make_matrix_map(&map_w[b], w.Wt[b], L, d, rp))
+        if (!lazy_tc_make_matrix_map(&map_a[b], w.A[b], L, ld, ld) ||
+            !lazy_tc_make_matrix_map(&map_q[b], w.Q[b], L, ld, ld) ||
+            !lazy_tc_make_matrix_map(&map_w[b], w.Wt[b], L, ld, rp))
             return ZIPLM_ERR_CUDA;
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.sched, 0, sizeof(int) * 2, st));
     constexpr size_t kRefreshSmem = sizeof(double) * 2 * kRefresh * (kRefresh + 1);
@@ -1085,7 +1101,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(
-                &cfg, k_lazy_steps, npos, S, t, nsteps, compact, d, G, r, rp, (const float*)w.A[cur],
+                &cfg, k_lazy_steps, npos, S, t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
                 (const float*)w.Q[cur], (const float*)w.Wt[cur], (const double*)w.dA[cur],
                 (const double*)w.dQ[cur], (const int*)w.idx[cur], w.dA[nxt], w.dQ[nxt], w.idx[nxt],
                 w.src, w.U, w.Z, w.C, w.state, order, saliency, layer_status));
@@ -1098,13 +1114,13 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         if (n_new > 0 && (compact || n_new <= 1)) {     // a dense block updates W^T in the tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_W, st);
             k_lazy_update_w<<<dim3((n_new + 63) / 64, (rp + 255) / 256, L), 256, 0, st>>>(
-                n_new, nsteps, d, rp, w.Wt[cur], w.Wt[nxt], w.src, w.U, w.C);
+                n_new, nsteps, ld, rp, w.Wt[cur], w.Wt[nxt], w.src, w.U, w.C);
             ZIPLM_CHECK_LAUNCH();
         }
         if (n_new > 1 && !compact) {
             // every position stays in place: dense tiles, tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);
-            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, n_new, nsteps, d, rp,
+            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, n_new, nsteps, ld, rp,
                                       w.A[nxt], w.Q[nxt], w.Wt[nxt], w.U, w.Z, w.C, w.P, w.sched,
                                       layer_status, 0u, st);
             if (s != ZIPLM_OK) return s;
@@ -1112,7 +1128,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);
             const int T = (n_new + 63) / 64;
             k_lazy_update_aq<<<dim3(T * (T + 1) / 2, L), 128, 0, st>>>(
-                n_new, nsteps, d, w.A[cur], w.Q[cur], w.A[nxt], w.Q[nxt], w.src, w.U, w.Z);
+                n_new, nsteps, ld, w.A[cur], w.Q[cur], w.A[nxt], w.Q[nxt], w.src, w.U, w.Z);
             ZIPLM_CHECK_LAUNCH();
         }
         cur = nxt;
@@ -1121,7 +1137,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         t += nsteps;
         if (refresh) {
             PhaseScope ps(PH_LAZY_REFRESH, st);
-            k_lazy_refresh<<<dim3(L, 2), 256, kRefreshSmem, st>>>(npos, d, r, rp, H, w.lam, w.idx[cur],
+            k_lazy_refresh<<<dim3(L, 2), 256, kRefreshSmem, st>>>(npos, d, ld, r, rp, H, w.lam, w.idx[cur],
                                                                   w.Wt[cur], w.A[cur], w.Q[cur], w.dA[cur],
                                                                   w.dQ[cur], layer_status);
             ZIPLM_CHECK_LAUNCH();

@@ -539,7 +539,7 @@ ziplm_status run_prune_neurons(const float* W, const float* H, int L, int r, int
     ziplm_status s;
     {
         PhaseScope ps(PH_INVERSE, st);
-        s = run_damped_inverse(H, L, d, damp_frac, nullptr, w.A, w.pitch, w.diag, w.lam, layer_status,
+        s = run_damped_inverse(H, L, d, damp_frac, nullptr, w.A, w.pitch, d, w.diag, w.lam, layer_status,
                                w.inv_ws, w.inv_bytes, st);
     }
     if (s != ZIPLM_OK) return s;

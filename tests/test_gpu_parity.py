@@ -757,3 +757,13 @@ def test_mutation_search_cluster_sizes(S, steps):
         assert int(out["status"][k]) == 0 and out["selected"][k].tolist() == sel
         assert int(out["n_accepted"][k]) == acc and float(out["objective"][k]) == score
         assert np.array_equal(out["coef"][k].cpu().numpy(), c)
+
+
+@pytest.mark.parametrize("d,r,levels", [(1, 3, [0]), (3, 5, [2, 0]), (66, 9, [65, 64, 63, 0]),
+                                        (769, 20, [600, 64, 0]), (1535, 12, [1500, 700, 1])])
+def test_delayed_path_widths_that_are_no_multiple_of_four(d, r, levels):
+    """The positions behind the width (pitch rounded up to 4) count as removed: below and above a
+    slice of the steps kernel, through dense and compaction blocks and the exact rebuild."""
+    sh = wl.scaled(wl.CONFIGS["c3_bert_base_fc2"][0], d_col=d, d_row=r, d_latent=max(4, d // 4),
+                   n_tokens=2 * d + 8, n_layers=2, levels=tuple(levels))
+    run_case(sh)
