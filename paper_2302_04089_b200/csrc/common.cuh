@@ -100,6 +100,14 @@ ziplm_status run_prune_blocks(const float* W, const float* H, int L, int r, int 
                               float* loss, float* base_loss, int* order, float* saliency,
                               int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st);
 
+// Widths of attention heads (multiples of 16 from 32 to 128; prune_heads.cu); chosen by run_prune_blocks.
+bool heads_path_supported(int g);
+size_t heads_workspace_bytes(int L, int r, int d, int g, int n_levels);
+ziplm_status run_prune_heads(const float* W, const float* H, int L, int r, int d, int g, float damp_frac,
+                             const int* levels, int n_levels, float* W_snap, float* loss, float* base_loss,
+                             int* order, float* saliency, int* layer_status, void* ws, size_t ws_bytes,
+                             cudaStream_t st);
+
 // base_loss[l] = 1/2 tr(W[l] H[l] W[l]^T) = ||W X||_F^2; acc64 is an [L] float64 scratch.
 ziplm_status run_base_loss(const float* W, const float* H, int L, int r, int d, double* acc64,
                            float* base_loss, cudaStream_t st);

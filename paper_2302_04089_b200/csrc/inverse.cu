@@ -332,9 +332,8 @@ struct SmallSmem {
     double ta[kTile * PS];       // operand tiles, as stored (row-major)
     double tb[kTile * PS];
     double td[kTile * PS];       // inverse of the current diagonal factor tile
-    double s[kTile][kTile + 1];  // leaf work array: the factor (lower part)
-    double col[2][kTile];        // current column of the leaf factorisation (double-buffered)
-    double dinv[kTile];          // reciprocal diagonal of the factor
+    double row[2][kTile + 1];    // leaf: current row and the diagonal entry behind it (double-buffered)
+    double piv[kTile];           // leaf: pivots
     int flag;                    // first error seen by this CTA
 };
 
@@ -400,176 +399,94 @@ __device__ __forceinline__ void small_epilogue(const SmallAcc& acc, Fn f) {
             f(r0 + 8 * i, c0 + 8 * j, make_double2(acc.d[i][j][0], acc.d[i][j][1]));
 }
 
-// One warp: acc(16 x 16) += A(16 x K) B(K x 16), operands anywhere in shared memory
-// (A[m * lda + k], B[k * ldb + n]); K a multiple of 4.
-__device__ __forceinline__ void warp_mma16(double (&acc)[2][2][2], const double* A, int lda,
-                                           const double* B, int ldb, int K) {
-    const int lane = threadIdx.x & 31;
-    for (int k0 = 0; k0 < K; k0 += 4) {
-        double a[2], b[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            a[i] = A[(8 * i + (lane >> 2)) * lda + k0 + (lane & 3)];
-            b[i] = B[(k0 + (lane & 3)) * ldb + 8 * i + (lane >> 2)];
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) dmma884(acc[i][j], a[i], b[j]);
-    }
-}
-
-// One warp: C(16 x 16) = sign * acc, C[m * ldc + n].
-__device__ __forceinline__ void warp_store16(const double (&acc)[2][2][2], double* C, int ldc, double sign) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                C[(8 * i + (lane >> 2)) * ldc + 8 * j + 2 * (lane & 3) + e] = sign * acc[i][j][e];
-}
-
-// Leaf: Cholesky factor of the 64 x 64 tile at Ag -> Fg (lower, upper part zeroed), the inverse of
-// that factor -> Mg and sm.td (lower, upper part zeroed).  Starts and ends with a barrier.
-//   Factor: threads 0..255 hold the tile in registers, cyclically (rows ty + 16 a, columns
-//   tx + 16 b, tx constant over half a warp), so a column step is one barrier, eight
-//   shared-memory reads and 16 FMAs per thread; only the warp that owns the column publishes it.
-//   Inverse: the four 16 x 16 diagonal blocks by forward substitution (one thread per column),
-//   then the off-diagonal blocks of the 32- and 64-wide levels as products
-//   M21 = -M22 (L21 M11) on the tensor core.
-__device__ __forceinline__ void leaf_factor(const double* Ag, double* Fg, double* Mg, int dp,
-                                            SmallSmem& sm) {
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const bool worker = tid < 256;
-    const int ty = tid & 15, tx = (tid >> 4) & 15;
+// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg and sm.td (lower, upper part
+// zeroed).  The factor itself is not needed.  Starts and ends with a barrier.
+// Elimination of [A | I] in place: at column k the rows i > k become
+//     r_ij -= (r_ik / r_kk) r_kj   for all j != k,      r_ik = -r_ik / r_kk,
+// which leaves the Schur complement in the columns j > k and row i of L^-1 (A = L D L^T) in the columns
+// j < i; M = D^-1/2 L^-1.  Threads 0 .. 255 hold the tile in registers, cyclically (rows ty + 16 a,
+// columns tx + 16 b).  The Schur complement is kept in both triangles, so row k is also column k, and a
+// step is one barrier: the half-warp that owns row k publishes it, and every thread forms the next pivot
+// and its reciprocal by itself from the published row and diagonal entry, beside its 16 updates, so that
+// the updates do not wait for a reciprocal.  (The earlier leaf, a Cholesky factor column by column and
+// then its inverse from 16 x 16 blocks, took 37 us; a chain of 64 x (barrier, load, two FMAs, store).)
+__device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp, SmallSmem& sm) {
+    const int tid = threadIdx.x;
+    const int tx = tid & 15, ty = (tid >> 4) & 15;
     __syncthreads();                          // earlier readers of the shared arrays are done
-    tile_async(sm.tb, Ag, dp);
-    cp_async_commit();
-    for (int e = tid; e < kTile * PS; e += kSmallThreads) sm.ta[e] = 0.0;   // the inverse is built in ta
-    cp_async_wait<0>();
-    __syncthreads();
-    double r[4][4];
-    if (worker) {
+    if (tid < 256) {
+        double r[4][4];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) r[a][b] = sm.tb[(ty + 16 * a) * PS + tx + 16 * b];
-    }
-    for (int c = 0; c < kTile; ++c) {
-        const int cb = c >> 4, ct = c & 15;
-        double* col = sm.col[c & 1];
-        if (worker && tx == ct) {
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                double v = r[a][0];
-#pragma unroll
-                for (int b = 1; b < 4; ++b) v = (b == cb) ? r[a][b] : v;
-                col[ty + 16 * a] = v;
+            for (int b = 0; b < 4; ++b) {
+                // the lower triangle is the valid one
+                const int i = ty + 16 * a, j = tx + 16 * b;
+                r[a][b] = Ag[i >= j ? (size_t)i * dp + j : (size_t)j * dp + i];
             }
-        }
-        __syncthreads();
-        if (worker) {
-            double p = col[c];
+        int flag = 0;
+        auto pivot = [&](double p) {
             if (!(p > 0.0) || !isfinite(p)) {   // not positive definite (or NaN): flag, keep going
-                if (tid == 0 && !sm.flag) sm.flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
+                if (!flag) flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
                 p = 1.0;
             }
-            const double rinv = rsqrt(p);
-            if (tid == 0) sm.dinv[c] = rinv;    // 1 / L_cc
-            double li[4], lj[4];
+            return p;
+        };
+        auto barrier = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+        if (tid == 0) sm.row[1][kTile] = r[0][0];
+        barrier();
+        double p = pivot(sm.row[1][kTile]), rp = __drcp_rn(p);
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                li[a] = col[ty + 16 * a] * rinv;
-                lj[a] = col[tx + 16 * a] * rinv;
-            }
-            // Columns <= c are final.  Rows <= c of the later columns lie above the diagonal:
-            // they are never used, so they are updated along with the rest.
+        for (int kb = 0; kb < 4; ++kb) {
+#pragma unroll 1
+            for (int kt = 0; kt < 16; ++kt) {
+                const int k = 16 * kb + kt;
+                double* v = sm.row[k & 1];
+                if (ty == kt) {
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (tx + 16 * b > c) {
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) r[a][b] = fma(-li[a], lj[b], r[a][b]);
+                    for (int b = 0; b < 4; ++b) v[tx + 16 * b] = r[kb][b];
                 }
-            if (tx == ct) {
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const int i = ty + 16 * a;
-                    const double v = i > c ? li[a] : p * rinv;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-                        if (b == cb && i >= c) r[a][b] = v;
+                if (kt < 15) {
+                    if (tx == kt + 1 && ty == kt + 1) v[kTile] = r[kb][kb];
+                } else if (tid == 0) {
+                    v[kTile] = kb < 3 ? r[kb < 3 ? kb + 1 : 3][kb < 3 ? kb + 1 : 3] : 1.0;
                 }
+                if (tid == 0) sm.piv[k] = p;
+                barrier();
+                double vi[4], vj[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) { vi[a] = v[ty + 16 * a]; vj[a] = v[tx + 16 * a]; }
+                const double vn = k + 1 < kTile ? v[k + 1] : 0.0;
+                const double p_next = pivot(fma(-(vn * rp), vn, v[kTile]));
+                const double rp_next = __drcp_rn(p_next);
+#pragma unroll
+                for (int a = kb; a < 4; ++a) {                   // the rows behind k
+                    if (a == kb && ty <= kt) continue;
+                    const double f = vi[a] * rp;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const double x = fma(-f, vj[b], r[a][b]);
+                        r[a][b] = (b == kb && tx == kt) ? -f : x;
+                    }
+                }
+                p = p_next;
+                rp = rp_next;
             }
         }
-    }
-    if (worker) {
+        if (tid == 0 && flag && !sm.flag) sm.flag = flag;
+        barrier();
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < 4; ++a) {
+            const int i = ty + 16 * a;
+            const double sc = rsqrt(sm.piv[i]);
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (tx + 16 * b <= ty + 16 * a) sm.s[ty + 16 * a][tx + 16 * b] = r[a][b];
-    }
-    __syncthreads();
-    // ---- inverse of the factor, built in sm.ta (pitch PS, zero above the diagonal) ----
-    if (tid < kTile) {
-        // column cc of diagonal block q: x_i = (delta_i,cc - sum_{cc <= k < i} L_ik x_k) / L_ii
-        const int q0 = tid & ~15, cc = tid & 15;
-        double x[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            double acc = (i == cc) ? 1.0 : 0.0;
-#pragma unroll
-            for (int k = 0; k < i; ++k) acc = fma(-sm.s[q0 + i][q0 + k], x[k], acc);
-            x[i] = (i >= cc) ? acc * sm.dinv[q0 + i] : 0.0;
-            sm.ta[(q0 + i) * PS + q0 + cc] = x[i];
+            for (int b = 0; b < 4; ++b) {
+                const int j = tx + 16 * b;
+                const double x = j < i ? r[a][b] * sc : j == i ? sc : 0.0;
+                Mg[(size_t)i * dp + j] = x;
+                sm.td[i * PS + j] = x;
+            }
         }
-    }
-    __syncthreads();
-    double acc[2][2][2];
-    auto zero = [&]() {
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
-    };
-    // 32-wide level: blocks (1,0) and (3,2) of 16 x 16; warp q does pair q.  tb holds L21 M11.
-    if (warp < 2) {
-        const int o = 32 * warp;
-        zero();
-        warp_mma16(acc, &sm.s[o + 16][o], kTile + 1, sm.ta + o * PS + o, PS, 16);
-        warp_store16(acc, sm.tb + (o + 16) * PS + o, PS, 1.0);
-    }
-    __syncthreads();
-    if (warp < 2) {
-        const int o = 32 * warp;
-        zero();
-        warp_mma16(acc, sm.ta + (o + 16) * PS + o + 16, PS, sm.tb + (o + 16) * PS + o, PS, 16);
-        warp_store16(acc, sm.ta + (o + 16) * PS + o, PS, -1.0);
-    }
-    __syncthreads();
-    // 64-wide level: block (rows 32.., cols 0..31); warp w < 4 does the 16 x 16 part (w / 2, w % 2).
-    if (warp < 4) {
-        const int rb = 32 + 16 * (warp >> 1), cb = 16 * (warp & 1);
-        zero();
-        warp_mma16(acc, &sm.s[rb][0], kTile + 1, sm.ta + cb, PS, 32);
-        warp_store16(acc, sm.tb + rb * PS + cb, PS, 1.0);
-    }
-    __syncthreads();
-    if (warp < 4) {
-        const int rb = 32 + 16 * (warp >> 1), cb = 16 * (warp & 1);
-        zero();
-        warp_mma16(acc, sm.ta + rb * PS + 32, PS, sm.tb + 32 * PS + cb, PS, 32);
-        warp_store16(acc, sm.ta + rb * PS + cb, PS, -1.0);
-    }
-    __syncthreads();
-    for (int e = tid; e < kTile * kTile; e += kSmallThreads) {
-        const int i = e >> 6, jj = e & 63;
-        const double m = sm.ta[i * PS + jj];
-        Fg[(size_t)i * dp + jj] = (jj <= i) ? sm.s[i][jj] : 0.0;
-        Mg[(size_t)i * dp + jj] = m;
-        sm.td[i * PS + jj] = m;
     }
     __syncthreads();
 }
@@ -590,7 +507,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_factor_small(double* A, do
     if (threadIdx.x == 0) sm.flag = 0;
     SmallAcc acc;
     for (int j = 0; j < nt; ++j) {
-        leaf_factor(tile(A, j, j), tile(F, j, j), tile(M, j, j), dp, sm);
+        leaf_factor(tile(A, j, j), tile(M, j, j), dp, sm);
         // F_ij = A_ij D_j^T
         for (int i = j + 1; i < nt; ++i) {
             tile_async(sm.ta, tile(A, i, j), dp);

@@ -433,7 +433,7 @@ BlockWs carve_block(void* ws, int L, int r, int d, int g) {
 }  // namespace
 
 size_t block_workspace_bytes(int L, int r, int d, int g, int n_levels) {
-    (void)n_levels;
+    if (heads_path_supported(g)) return heads_workspace_bytes(L, r, d, g, n_levels);
     return carve_block(nullptr, L, r, d, g).total;
 }
 
@@ -443,6 +443,9 @@ ziplm_status run_prune_blocks(const float* W, const float* H, int L, int r, int 
                               int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (g > GMAX) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < block_workspace_bytes(L, r, d, g, n_levels)) return ZIPLM_ERR_WORKSPACE;
+    if (heads_path_supported(g))
+        return run_prune_heads(W, H, L, r, d, g, damp_frac, levels, n_levels, W_snap, loss, base_loss, order,
+                               saliency, layer_status, ws, ws_bytes, st);
     BlockWs w = carve_block(ws, L, r, d, g);
     const int G = d / g;
     ziplm_status s;

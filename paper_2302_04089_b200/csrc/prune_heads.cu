@@ -1,0 +1,585 @@
+// Greedy structured OBS for attention heads: structures of g consecutive columns, g a multiple of 16
+// from 32 to 128 (prune_block.cu serves the other widths).
+//
+// With S the columns of the selected head and B = (H^-1)[S,S], everything a step needs follows from
+//     T  = B^-1 (H^-1)[S,:]                                  (g x d)
+//     H^-1 <- H^-1 - (H^-1)[:,S] T                           (Eq. 4)
+//     W    <- W    - W[:,S] T                                (Eq. 3)
+// and the saliency rho_S = tr(W[:,S] B^-1 W[:,S]^T) = <B^-1, Q[S,S]> (Eq. 2) from the Gram matrix
+// Q = W^T W, which is carried along instead of being formed again from W for every head and step:
+//     Q <- Q - V^T T - T^T V,   V = Q[S,:] - 1/2 Q[S,S] T.
+// The whole state (H^-1, Q, W) is float64.  Removed heads stay in place and are skipped.
+//
+// A layer has 8 to 16 heads, so the loop is short and used to be bound by latency: a Cholesky
+// factorisation with three barriers per column, a forward substitution and a Gram product over all
+// rows of W for every head and step (232 us a step for 12 layers of 12 heads of 64), then another
+// 250 us for the update on the float64 FMA pipe.  Here every product is a g x g x g tile product on
+// the float64 tensor-core instruction, the inverse of a head's block is one pass of symmetric sweeps
+// in registers (one barrier per column), and a step is two launches: `solve` (which also selects) and
+// `update` (whose diagonal tiles go on to score their head for the next step, and whose tiles of W
+// write the snapshot).
+#include <math.h>
+
+#include "common.cuh"
+
+namespace ziplm {
+namespace {
+
+constexpr int HT = 256;          // threads per CTA
+constexpr int KCH = 32;          // k-chunk of a tile product
+constexpr int P_MK = KCH + 4;    // pitch of a chunk stored [m][k]; like g + 4 it is 4 mod 16, so that the
+                                 // 16 lanes of a half-warp's fragment load hit 16 different 8-byte banks
+
+// Shape of the tile products of heads of 8 * G8 columns.  A warp owns UN units of one row of 8 x 8
+// fragments by half of the columns; all its units lie in the same half and share its fragments.
+template <int G8>
+struct HeadShape {
+    static constexpr int g = 8 * G8, CF = G8 / 2, UN = (2 * G8 + 7) / 8, P_KM = g + 4;
+    static constexpr int kOperand = KCH * P_KM > g * P_MK ? KCH * P_KM : g * P_MK;     // doubles
+    static constexpr size_t kSmem = sizeof(double) * 4 * kOperand;                     // two stages
+};
+
+template <int G8>
+struct HeadAcc {
+    using S = HeadShape<G8>;
+    double d[S::UN][S::CF][2];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int u = 0; u < S::UN; ++u)
+#pragma unroll
+            for (int j = 0; j < S::CF; ++j) d[u][j][0] = d[u][j][1] = 0.0;
+    }
+    // f(row, col, pair) with col even, for every pair this thread holds
+    template <typename F>
+    __device__ __forceinline__ void visit(F f) const {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int u = 0; u < S::UN; ++u) {
+            const int rf = (warp + 8 * u) >> 1;
+            if (rf >= G8) continue;
+#pragma unroll
+            for (int j = 0; j < S::CF; ++j)
+                f(8 * rf + (lane >> 2), 8 * ((warp & 1) * S::CF + j) + 2 * (lane & 3),
+                  make_double2(d[u][j][0], d[u][j][1]));
+        }
+    }
+};
+
+__device__ __forceinline__ void h_dmma(double (&d)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
+__device__ __forceinline__ void h_cp16(double* dst, const double* src, bool ok) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(src), "r"(ok ? 16u : 0u) : "memory");
+}
+
+// Start the copy of one chunk of an operand: KM: P[k * ld + m], m < g, kept [k][m], rows k >= k_valid
+// zero; otherwise P[m * ld + k], kept [m][k], rows m >= m_valid and columns k >= k_valid zero.
+template <int G8, bool KM>
+__device__ __forceinline__ void h_chunk(double* s, const double* P, size_t ld, int k0, int k_valid, int m_valid) {
+    using S = HeadShape<G8>;
+    for (int e = threadIdx.x; e < S::g * KCH / 2; e += HT) {
+        if (KM) {
+            const int k = e / (S::g / 2), m = 2 * (e % (S::g / 2));
+            const bool ok = k0 + k < k_valid;
+            h_cp16(s + k * S::P_KM + m, P + (ok ? (size_t)(k0 + k) * ld + m : 0), ok);
+        } else {
+            const int m = e / (KCH / 2), k = 2 * (e % (KCH / 2));
+            const bool ok = m < m_valid && k0 + k < k_valid;
+            h_cp16(s + m * P_MK + k, P + (ok ? (size_t)m * ld + k0 + k : 0), ok);
+        }
+    }
+}
+
+template <int G8, bool KM>
+__device__ __forceinline__ double h_frag(const double* s, int m0, int kk, int lane) {
+    return KM ? s[(kk * 4 + (lane & 3)) * HeadShape<G8>::P_KM + m0 + (lane >> 2)]
+              : s[(m0 + (lane >> 2)) * P_MK + kk * 4 + (lane & 3)];
+}
+
+// acc(g x g) += X (g x K) Y (K x g).  XKM: X(m,k) = X[k * ldx + m], else X[m * ldx + k] with rows from
+// x_rows on zero; YKM: Y(k,n) = Y[k * ldy + n], else Y[n * ldy + k].  K is a multiple of 16 unless both
+// are stored by k.  Starts with every thread past its use of smem and ends with a barrier.
+template <int G8, bool XKM, bool YKM>
+__device__ __forceinline__ void h_product(HeadAcc<G8>& acc, const double* X, size_t ldx, int x_rows,
+                                          const double* Y, size_t ldy, int K, double* smem) {
+    using S = HeadShape<G8>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nch = (K + KCH - 1) / KCH;
+    auto start = [&](int c) {
+        double* s = smem + (c & 1) * 2 * S::kOperand;
+        h_chunk<G8, XKM>(s, X, ldx, c * KCH, K, x_rows);
+        h_chunk<G8, YKM>(s + S::kOperand, Y, ldy, c * KCH, K, S::g);
+    };
+    start(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int c = 0; c < nch; ++c) {
+        if (c + 1 < nch) start(c + 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const double* sx = smem + (c & 1) * 2 * S::kOperand;
+        const double* sy = sx + S::kOperand;
+        const int steps = (min(KCH, K - c * KCH) + 3) / 4;        // (a row past K is zero)
+#pragma unroll 2
+        for (int kk = 0; kk < steps; ++kk) {
+            double b[S::CF];
+#pragma unroll
+            for (int j = 0; j < S::CF; ++j) b[j] = h_frag<G8, YKM>(sy, 8 * ((warp & 1) * S::CF + j), kk, lane);
+#pragma unroll
+            for (int u = 0; u < S::UN; ++u) {
+                const int rf = (warp + 8 * u) >> 1;
+                if (rf >= G8) continue;
+                const double a = h_frag<G8, XKM>(sx, 8 * rf, kk, lane);
+#pragma unroll
+                for (int j = 0; j < S::CF; ++j) h_dmma(acc.d[u][j], a, b[j]);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Everything the kernels of a call work on.
+struct Heads {
+    int L, G, r, d;
+    const float* W; const float* H;
+    double* A; double* Q; double* W64;      // [d][d] (Q and, after the first step, A: lower blocks), [r][d]
+    double* P; double* T; double* V;        // [g][d]: (H^-1)[S,:], T, V of the step
+    double* Bneg;                           // [G][g][g]: -(head's block of H^-1)^-1
+    double* rho;                            // [G]: saliencies of the live heads
+    double* rho_sel;                        // [G]: of the removed ones, by step
+    double* dw2;                            // [n_levels + 1]: ||W - W_snap||^2 by level, then 2 * base loss
+    int* alive;                             // [2][G], by step parity
+    int* chosen;                            // [1]
+    int* steps_of;                          // [n_levels], shared by the layers: removals of a level
+    float* W_snap; int n_levels;
+    int* order; float* saliency; int* layer_status;
+};
+
+// Row block i >= j of a lower-triangular pair index.
+__device__ __forceinline__ void pair_index(int x, int& i, int& j) {
+    i = (int)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
+    while (i * (i + 1) / 2 > x) --i;
+    while ((i + 1) * (i + 2) / 2 <= x) ++i;
+    j = x - i * (i + 1) / 2;
+}
+
+// Sum over the CTA, in thread 0.
+__device__ __forceinline__ double h_sum(double v, double* red) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < HT / 32; ++w) t += red[w];
+    return t;
+}
+
+// rho of head s of layer l and -(H^-1)[S,S]^-1, from the diagonal blocks of H^-1 and Q: symmetric
+// sweeps a_ij -= a_ik a_kj / a_kk over all k, the block in registers, cyclically over the 16 x 16
+// threads.  A column is one barrier: the half-warp that owns row k publishes it, and every thread forms
+// the next pivot and its reciprocal by itself from the published row and diagonal entry, beside its
+// updates, so that neither waits for the other.  The pivots are those of the Cholesky factorisation.
+template <int G8>
+__device__ void h_score(const Heads& w, int l, int s, double* red, double (*v)[HeadShape<G8>::g + 1]) {
+    using S = HeadShape<G8>;
+    constexpr int NB = S::g / 16;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const size_t at = (size_t)l * w.d * w.d + (size_t)s * S::g * w.d + (size_t)s * S::g;
+    double a[NB][NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) a[i][j] = w.A[at + (size_t)(ty + 16 * i) * w.d + tx + 16 * j];
+    int flag = 0;
+    auto reciprocal = [&](double p) {
+        if (!(p > 0.0) || !isfinite(p)) {          // not positive definite (or NaN): flag, keep going
+            if (!flag) flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
+            p = 1.0;
+        }
+        return __drcp_rn(p);
+    };
+    if (tid == 0) v[1][S::g] = a[0][0];
+    __syncthreads();
+    double rp = reciprocal(v[1][S::g]);
+#pragma unroll
+    for (int kb = 0; kb < NB; ++kb) {
+#pragma unroll 1
+        for (int kt = 0; kt < 16; ++kt) {
+            const int k = 16 * kb + kt;
+            double* vk = v[k & 1];
+            if (ty == kt) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j) vk[tx + 16 * j] = a[kb][j];
+            }
+            // the diagonal entry behind the pivot
+            if (kt < 15) {
+                if (tx == kt + 1 && ty == kt + 1) vk[S::g] = a[kb][kb];
+            } else if (tid == 0) {
+                vk[S::g] = kb + 1 < NB ? a[kb + 1 < NB ? kb + 1 : kb][kb + 1 < NB ? kb + 1 : kb] : 1.0;
+            }
+            __syncthreads();
+            double vi[NB], vj[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i) { vi[i] = vk[ty + 16 * i]; vj[i] = vk[tx + 16 * i]; }
+            const double vn = k + 1 < S::g ? vk[k + 1] : 0.0;
+            const double rp_next = reciprocal(fma(-(vn * rp), vn, vk[S::g]));
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                const double f = vi[i] * rp;
+                const bool row = i == kb && ty == kt;
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const bool col = j == kb && tx == kt;
+                    const double upd = fma(-f, vj[j], a[i][j]);
+                    a[i][j] = row ? (col ? -rp : vj[j] * rp) : (col ? f : upd);
+                }
+            }
+            rp = rp_next;
+        }
+    }
+    double part = 0.0;
+    double* B = w.Bneg + ((size_t)l * w.G + s) * S::g * S::g;
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            B[(ty + 16 * i) * S::g + tx + 16 * j] = a[i][j];
+            part = fma(-a[i][j], w.Q[at + (size_t)(ty + 16 * i) * w.d + tx + 16 * j], part);
+        }
+    const double rho = h_sum(part, red);
+    if (tid == 0) {
+        w.rho[(size_t)l * w.G + s] = rho;
+        if (flag) set_layer_status(w.layer_status, l, flag);
+    }
+}
+
+__global__ void __launch_bounds__(HT) k_heads_init(Heads w) {
+    const size_t count = (size_t)w.L * w.r * w.d;
+    for (size_t i = (size_t)blockIdx.x * HT + threadIdx.x; i < count; i += (size_t)gridDim.x * HT)
+        w.W64[i] = (double)w.W[i];
+    for (int i = blockIdx.x * HT + threadIdx.x; i < w.L * w.G; i += gridDim.x * HT)
+        w.alive[(size_t)(i / w.G) * 2 * w.G + i % w.G] = 1;
+}
+
+// Block (i, j), i >= j, of Q = W^T W, and its share of <Q, H> = 2 ||W X||^2.
+template <int G8>
+__global__ void __launch_bounds__(HT) k_heads_gram(Heads w) {
+    using S = HeadShape<G8>;
+    extern __shared__ __align__(16) double smem[];
+    __shared__ double red[HT / 32];
+    const int l = blockIdx.y;
+    int i, j;
+    pair_index(blockIdx.x, i, j);
+    const double* Wl = w.W64 + (size_t)l * w.r * w.d;
+    HeadAcc<G8> acc;
+    acc.zero();
+    h_product<G8, true, true>(acc, Wl + i * S::g, w.d, S::g, Wl + j * S::g, w.d, w.r, smem);
+    const size_t at = (size_t)l * w.d * w.d + (size_t)i * S::g * w.d + (size_t)j * S::g;
+    double part = 0.0;
+    acc.visit([&](int row, int col, double2 x) {
+        const size_t o = at + (size_t)row * w.d + col;
+        *reinterpret_cast<double2*>(w.Q + o) = x;
+        part += x.x * (double)w.H[o] + x.y * (double)w.H[o + 1];
+    });
+    const double t = h_sum(part, red);
+    if (threadIdx.x == 0) atomicAdd(w.dw2 + (size_t)l * (w.n_levels + 1) + w.n_levels, i == j ? t : 2.0 * t);
+}
+
+template <int G8>
+__global__ void __launch_bounds__(HT) k_heads_score(Heads w) {
+    __shared__ double red[HT / 32], v[2][HeadShape<G8>::g + 1];
+    h_score<G8>(w, blockIdx.y, blockIdx.x, red, v);
+}
+
+// Selection (argmin of rho over the live heads, ties to the lowest index; every CTA makes it for
+// itself) and, for the columns of head blockIdx.x, P = (H^-1)[S,:], T = B^-1 P, V = Q[S,:] - Q[S,S] T / 2.
+template <int G8>
+__global__ void __launch_bounds__(HT) k_heads_solve(Heads w, int t) {
+    using S = HeadShape<G8>;
+    extern __shared__ __align__(16) double smem[];
+    __shared__ int s_pick;
+    const int l = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
+    const int* alive = w.alive + ((size_t)l * 2 + (t & 1)) * w.G;
+    if (tid < 32) {
+        double best = INFINITY;
+        int at = 0x7fffffff;
+        for (int s = tid; s < w.G; s += 32) {
+            if (!alive[s]) continue;
+            double x = w.rho[(size_t)l * w.G + s];
+            if (!(x == x)) x = INFINITY;
+            if (x < best || (x == best && s < at)) { best = x; at = s; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double x = __shfl_xor_sync(0xffffffffu, best, o);
+            const int s = __shfl_xor_sync(0xffffffffu, at, o);
+            if (x < best || (x == best && s < at)) { best = x; at = s; }
+        }
+        if (tid == 0) s_pick = at;
+        if (j == 0) {
+            for (int s = tid; s < w.G; s += 32)
+                w.alive[((size_t)l * 2 + ((t + 1) & 1)) * w.G + s] = s == at ? 0 : alive[s];
+            if (tid == 0) {
+                if (!isfinite(best)) set_layer_status(w.layer_status, l, ZIPLM_ERR_NONFINITE);
+                w.chosen[l] = at;
+                w.rho_sel[(size_t)l * w.G + t] = isfinite(best) ? best : 0.0;
+                w.order[(size_t)l * w.G + t] = at;
+                if (w.saliency) w.saliency[(size_t)l * w.G + t] = (float)best;
+            }
+        }
+    }
+    __syncthreads();
+    const int s = s_pick;
+    if (!alive[j] || j == s) return;
+    const size_t lay = (size_t)l * w.d * w.d, out = (size_t)l * S::g * w.d + (size_t)j * S::g;
+    const bool below = j > s;       // the block is stored as (j, s): transposed
+    const size_t blk = lay + (below ? (size_t)j * S::g * w.d + (size_t)s * S::g
+                                    : (size_t)s * S::g * w.d + (size_t)j * S::g);
+    const double* Bn = w.Bneg + ((size_t)l * w.G + s) * S::g * S::g;
+    HeadAcc<G8> acc;
+    acc.zero();
+    // B^-1 is symmetric: stored by k as well as by m
+    if (below) h_product<G8, true, false>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
+    else h_product<G8, true, true>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
+    acc.visit([&](int k, int n, double2 x) {
+        *reinterpret_cast<double2*>(w.T + out + (size_t)k * w.d + n) = make_double2(-x.x, -x.y);
+        const size_t o = below ? blk + (size_t)n * w.d + k : blk + (size_t)k * w.d + n;
+        *reinterpret_cast<double2*>(w.P + out + (size_t)k * w.d + n) =
+            below ? make_double2(w.A[o], w.A[o + w.d]) : *reinterpret_cast<const double2*>(w.A + o);
+    });
+    __syncthreads();                // T is read back below, by the whole CTA
+    const size_t ss = lay + (size_t)s * S::g * w.d + (size_t)s * S::g;
+    acc.zero();
+    h_product<G8, true, true>(acc, w.Q + ss, w.d, S::g, w.T + out, w.d, S::g, smem);
+    acc.visit([&](int k, int n, double2 x) {
+        const size_t o = below ? blk + (size_t)n * w.d + k : blk + (size_t)k * w.d + n;
+        const double2 q = below ? make_double2(w.Q[o], w.Q[o + w.d]) : *reinterpret_cast<const double2*>(w.Q + o);
+        *reinterpret_cast<double2*>(w.V + out + (size_t)k * w.d + n) =
+            make_double2(fma(-0.5, x.x, q.x), fma(-0.5, x.y, q.y));
+    });
+}
+
+// CTAs 0 .. G - 1: diagonal blocks of H^-1 and Q, then the head's next score (the longest CTAs first);
+// the next G (G - 1) / 2: blocks below the diagonal; the rest: blocks of g rows of W and, when `slot` is a
+// level, of the snapshot.
+template <int G8>
+__global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, int rescore) {
+    using S = HeadShape<G8>;
+    extern __shared__ __align__(16) double smem[];
+    __shared__ double red[HT / 32], v[2][S::g + 1];
+    const int l = blockIdx.y, x = blockIdx.x, n_pairs = w.G * (w.G + 1) / 2;
+    if (slot >= 0 && x == 0 && l == 0 && threadIdx.x == 0) w.steps_of[slot] = t + 1;
+    const int* alive = w.alive + ((size_t)l * 2 + ((t + 1) & 1)) * w.G;
+    const size_t ops = (size_t)l * S::g * w.d;
+    HeadAcc<G8> acc;
+    if (x < n_pairs) {
+        int i = x, j = x;
+        if (x >= w.G) { pair_index(x - w.G, i, j); ++i; }
+        if (!alive[i] || !alive[j]) return;
+        const size_t at = (size_t)l * w.d * w.d + (size_t)i * S::g * w.d + (size_t)j * S::g;
+        auto subtract = [&](double* M) {
+            acc.visit([&](int row, int col, double2 d) {
+                double2* o = reinterpret_cast<double2*>(M + at + (size_t)row * w.d + col);
+                double2 cur = *o;
+                cur.x -= d.x; cur.y -= d.y;
+                *o = cur;
+            });
+        };
+        const double *Ti = w.T + ops + i * S::g, *Tj = w.T + ops + j * S::g;
+        acc.zero();
+        h_product<G8, true, true>(acc, w.P + ops + i * S::g, w.d, S::g, Tj, w.d, S::g, smem);
+        subtract(w.A);
+        acc.zero();
+        h_product<G8, true, true>(acc, w.V + ops + i * S::g, w.d, S::g, Tj, w.d, S::g, smem);
+        h_product<G8, true, true>(acc, Ti, w.d, S::g, w.V + ops + j * S::g, w.d, S::g, smem);
+        subtract(w.Q);
+        if (i == j && rescore) {
+            __syncthreads();
+            h_score<G8>(w, l, i, red, v);
+        }
+        return;
+    }
+    const int j = (x - n_pairs) % w.G, b = (x - n_pairs) / w.G, row0 = b * S::g;
+    const int rows = min(S::g, w.r - row0);
+    const float* W0 = w.W + ((size_t)l * w.r + row0) * w.d + (size_t)j * S::g;
+    float* snap = slot < 0 ? nullptr
+                           : w.W_snap + (((size_t)l * w.n_levels + slot) * w.r + row0) * w.d + (size_t)j * S::g;
+    double part = 0.0;
+    if (!alive[j]) {
+        if (!snap) return;
+        for (int e = threadIdx.x; e < rows * (S::g / 4); e += HT) {
+            const size_t o = (size_t)(e / (S::g / 4)) * w.d + 4 * (e % (S::g / 4));
+            for (int c = 0; c < 4; ++c) {
+                part += (double)W0[o + c] * (double)W0[o + c];
+                snap[o + c] = 0.f;
+            }
+        }
+    } else {
+        double* Wl = w.W64 + ((size_t)l * w.r + row0) * w.d;
+        acc.zero();
+        h_product<G8, false, true>(acc, Wl + (size_t)w.chosen[l] * S::g, w.d, rows, w.T + ops + j * S::g, w.d, S::g,
+                                   smem);
+        acc.visit([&](int row, int col, double2 d) {
+            if (row >= rows) return;
+            const size_t o = (size_t)row * w.d + col;
+            double2* p = reinterpret_cast<double2*>(Wl + (size_t)j * S::g + o);
+            double2 cur = *p;
+            cur.x -= d.x; cur.y -= d.y;
+            *p = cur;
+            if (snap) {
+                const float f0 = (float)cur.x, f1 = (float)cur.y, e0 = W0[o] - f0, e1 = W0[o + 1] - f1;
+                snap[o] = f0;
+                snap[o + 1] = f1;
+                part += (double)e0 * e0 + (double)e1 * e1;
+            }
+        });
+    }
+    if (!snap) return;
+    const double sum = h_sum(part, red);
+    if (threadIdx.x == 0 && sum != 0.0) atomicAdd(w.dw2 + (size_t)l * (w.n_levels + 1) + slot, sum);
+}
+
+// Losses of all levels (half the sum of the saliencies removed so far, less the damping's share: every
+// rho is twice the increase of the damped objective) and the base loss.  One warp per layer.
+__global__ void __launch_bounds__(32) k_heads_loss(Heads w, const double* __restrict__ lam, float* __restrict__ loss,
+                                                   float* __restrict__ base_loss) {
+    const int l = blockIdx.x;
+    const double* dw2 = w.dw2 + (size_t)l * (w.n_levels + 1);
+    for (int q = threadIdx.x; q < w.n_levels; q += 32) {
+        double sum = 0.0;
+        for (int t = 0; t < w.steps_of[q]; ++t) sum += w.rho_sel[(size_t)l * w.G + t];
+        const double x = 0.5 * sum - 0.5 * lam[l] * dw2[q];
+        loss[(size_t)l * w.n_levels + q] = (float)(x > 0.0 ? x : 0.0);
+    }
+    if (threadIdx.x == 0 && base_loss) base_loss[l] = (float)(0.5 * dw2[w.n_levels]);
+}
+
+struct HeadsWs {
+    Heads h;
+    double* lam; void* inv_ws; size_t inv_bytes, zero_bytes; void* zero; size_t total;
+};
+
+HeadsWs carve_heads(void* ws, int L, int r, int d, int g, int n_levels) {
+    HeadsWs w = {};
+    const int G = d / g;
+    w.h.L = L; w.h.G = G; w.h.r = r; w.h.d = d; w.h.n_levels = n_levels;
+    Carver c(ws);
+    w.h.A = c.take<double>((size_t)L * d * d);
+    w.h.Q = c.take<double>((size_t)L * d * d);
+    w.h.W64 = c.take<double>((size_t)L * r * d);
+    w.h.P = c.take<double>((size_t)L * g * d);
+    w.h.T = c.take<double>((size_t)L * g * d);
+    w.h.V = c.take<double>((size_t)L * g * d);
+    w.h.Bneg = c.take<double>((size_t)L * G * g * g);
+    w.h.rho = c.take<double>((size_t)L * G);
+    w.h.rho_sel = c.take<double>((size_t)L * G);
+    w.h.alive = c.take<int>((size_t)L * 2 * G);
+    w.h.chosen = c.take<int>((size_t)L);
+    const size_t z0 = c.off;                               // zeroed together
+    w.h.dw2 = c.take<double>((size_t)L * (n_levels + 1));
+    w.h.steps_of = c.take<int>((size_t)n_levels);
+    w.zero = w.h.dw2;
+    w.zero_bytes = c.off - z0;
+    w.lam = c.take<double>((size_t)L);
+    w.inv_bytes = inverse_workspace_bytes(L, d);
+    w.inv_ws = c.take<char>(w.inv_bytes);
+    w.total = c.off;
+    return w;
+}
+
+template <int G8>
+ziplm_status run_heads(HeadsWs& ws, float damp_frac, const int* levels, float* loss, float* base_loss,
+                       cudaStream_t st) {
+    Heads& w = ws.h;
+    const int L = w.L, G = w.G, g = 8 * G8, n_levels = w.n_levels;
+    constexpr int smem = (int)HeadShape<G8>::kSmem;
+    ziplm_status s;
+    {
+        PhaseScope ps(PH_INVERSE, st);
+        s = run_damped_inverse(w.H, L, w.d, damp_frac, w.A, nullptr, 0, 0, nullptr, ws.lam, w.layer_status,
+                               ws.inv_ws, ws.inv_bytes, st);
+    }
+    if (s != ZIPLM_OK) return s;
+    const int n_steps = n_levels > 0 ? G - levels[n_levels - 1] : 0;
+    int slot = 0;
+    {
+        PhaseScope ps(PH_INIT, st);
+        ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.order, 0xFF, sizeof(int) * (size_t)L * G, st));
+        if (w.saliency) ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.saliency, 0, sizeof(float) * (size_t)L * G, st));
+        ZIPLM_CHECK_CUDA(cudaMemsetAsync(ws.zero, 0, ws.zero_bytes, st));
+        k_heads_init<<<592, HT, 0, st>>>(w);
+        ZIPLM_CHECK_LAUNCH();
+        if (n_steps > 0 || base_loss) {
+            ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_gram<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            k_heads_gram<G8><<<dim3(G * (G + 1) / 2, L), HT, smem, st>>>(w);
+            ZIPLM_CHECK_LAUNCH();
+        }
+        if (n_levels > 0 && levels[0] == G) {              // the unpruned level: loss 0
+            const size_t n = (size_t)w.r * w.d;
+            for (int l = 0; l < L; ++l)
+                ZIPLM_CHECK_CUDA(cudaMemcpyAsync(w.W_snap + (size_t)l * n_levels * n, w.W + l * n, n * sizeof(float),
+                                                 cudaMemcpyDeviceToDevice, st));
+            ++slot;
+        }
+    }
+    if (n_steps > 0) {
+        PhaseScope ps(PH_BLOCK_SCORE, st);
+        k_heads_score<G8><<<dim3(G, L), HT, 0, st>>>(w);
+        ZIPLM_CHECK_LAUNCH();
+    }
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_solve<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_update<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int ctas = G * (G + 1) / 2 + G * ((w.r + g - 1) / g);
+    for (int t = 0; t < n_steps; ++t) {
+        {
+            PhaseScope ps(PH_BLOCK_SCORE, st);
+            k_heads_solve<G8><<<dim3(G, L), HT, smem, st>>>(w, t);
+            ZIPLM_CHECK_LAUNCH();
+        }
+        const bool level = levels[slot] == G - t - 1;
+        if (G - t > 1 || level) {
+            PhaseScope ps(PH_BLOCK_UPDATE, st);
+            k_heads_update<G8><<<dim3(ctas, L), HT, smem, st>>>(w, t, level ? slot : -1, t + 1 < n_steps);
+            ZIPLM_CHECK_LAUNCH();
+        }
+        if (level) ++slot;
+    }
+    k_heads_loss<<<L, 32, 0, st>>>(w, ws.lam, loss, base_loss);
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
+}  // namespace
+
+bool heads_path_supported(int g) { return g >= 32 && g <= 128 && g % 16 == 0; }
+
+size_t heads_workspace_bytes(int L, int r, int d, int g, int n_levels) {
+    return carve_heads(nullptr, L, r, d, g, n_levels).total;
+}
+
+ziplm_status run_prune_heads(const float* W, const float* H, int L, int r, int d, int g, float damp_frac,
+                             const int* levels, int n_levels, float* W_snap, float* loss, float* base_loss,
+                             int* order, float* saliency, int* layer_status, void* ws, size_t ws_bytes,
+                             cudaStream_t st) {
+    if (!heads_path_supported(g)) return ZIPLM_ERR_UNSUPPORTED;
+    HeadsWs w = carve_heads(ws, L, r, d, g, n_levels);
+    if (ws_bytes < w.total) return ZIPLM_ERR_WORKSPACE;
+    w.h.W = W; w.h.H = H; w.h.W_snap = W_snap; w.h.order = order; w.h.saliency = saliency;
+    w.h.layer_status = layer_status;
+    switch (g / 8) {
+        case 4: return run_heads<4>(w, damp_frac, levels, loss, base_loss, st);
+        case 6: return run_heads<6>(w, damp_frac, levels, loss, base_loss, st);
+        case 8: return run_heads<8>(w, damp_frac, levels, loss, base_loss, st);
+        case 10: return run_heads<10>(w, damp_frac, levels, loss, base_loss, st);
+        case 12: return run_heads<12>(w, damp_frac, levels, loss, base_loss, st);
+        case 14: return run_heads<14>(w, damp_frac, levels, loss, base_loss, st);
+        default: return run_heads<16>(w, damp_frac, levels, loss, base_loss, st);
+    }
+}
+
+}  // namespace ziplm
