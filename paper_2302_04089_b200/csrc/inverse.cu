@@ -10,6 +10,7 @@
 // loop that follows needs the diagonal of H^-1 to roughly 1e-7 relative, which an fp32
 // factorisation of a matrix with condition number 1e3 .. 1e5 does not give.  The matrix is
 // padded to a multiple of 64 with an identity block, whose inverse is again the identity.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <mutex>
@@ -324,14 +325,13 @@ __global__ void __launch_bounds__(GT, 2) k_dgemm_pair(GemmTask t1, int n1, GemmT
     else dgemm_task<false, false>(t2, dp, blockIdx.x - n1, blockIdx.y, smem);
 }
 
-// ---- base case of the recursion: a range of up to kSmallMax tiles, one CTA per layer ----------
+// ---- base case of the recursion: a range of up to kSmallMax tiles, one cluster per layer -------
 constexpr int kSmallMax = 4;
 constexpr int PS = kTile + 4;    // pitch of a 64 x 64 operand tile in shared memory (4 mod 16)
 
 struct SmallSmem {
     double ta[kTile * PS];       // operand tiles, as stored (row-major)
     double tb[kTile * PS];
-    double td[kTile * PS];       // inverse of the current diagonal factor tile
     double row[2][kTile + 1];    // leaf: current row and the diagonal entry behind it (double-buffered)
     double piv[kTile];           // leaf: pivots
     int flag;                    // first error seen by this CTA
@@ -399,8 +399,7 @@ __device__ __forceinline__ void small_epilogue(const SmallAcc& acc, Fn f) {
             f(r0 + 8 * i, c0 + 8 * j, make_double2(acc.d[i][j][0], acc.d[i][j][1]));
 }
 
-// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg and sm.td (lower, upper part
-// zeroed).  The factor itself is not needed.  Starts and ends with a barrier.
+// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg (lower, upper part zeroed).  The factor itself is not needed.  Starts and ends with a barrier.
 // Elimination of [A | I] in place: at column k the rows i > k become
 //     r_ij -= (r_ik / r_kk) r_kj   for all j != k,      r_ik = -r_ik / r_kk,
 // which leaves the Schur complement in the columns j > k and row i of L^-1 (A = L D L^T) in the columns
@@ -484,92 +483,94 @@ __device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp
                 const int j = tx + 16 * b;
                 const double x = j < i ? r[a][b] * sc : j == i ? sc : 0.0;
                 Mg[(size_t)i * dp + j] = x;
-                sm.td[i * PS + j] = x;
             }
         }
     }
     __syncthreads();
 }
 
-// Factor the tile range [lo, lo + nt), nt <= kSmallMax, of every layer with one CTA per layer:
-// right-looking tile Cholesky (A -> F) followed by the block forward substitution for M = F^-1.
-// Every product is a 64 x 64 x 64 tile product of the whole CTA on the float64 tensor core, with
-// its operands fetched from global memory (the L2) into shared memory.
+// Factor the tile range [lo, lo + nt), nt <= kSmallMax, of every layer with one cluster of four CTAs per
+// layer: right-looking elimination of [A | I] by tiles.  Stage j: rank 0 turns the diagonal tile into
+// M_jj; then F_ij = A_ij M_jj^T below it and M_jk = M_jj X_jk left of it; then A_ik -= F_ij F_kj^T and
+// X_ik -= F_ij M_jk (X_ik, kept in M's tile, is what M_ik is before its own row's stage).  The tiles of a
+// phase are independent and dealt out to the ranks; rank 0 updates the next diagonal tile first and goes
+// on to its leaf without waiting for the others, so the chain is leaf, one product, leaf, ...: two cluster
+// barriers a stage.  Every product is a 64 x 64 x 64 tile product of a whole CTA on the float64 tensor
+// core, its operands fetched from global memory (the L2) into shared memory; on one CTA alone the 32
+// products of four tiles took 150 us of 184.
+constexpr int kSmallCluster = 4;
 __global__ void __launch_bounds__(kSmallThreads, 1) k_factor_small(double* A, double* F, double* M, int dp, int lo,
                                                         int nt, int* layer_status) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
-    const int l = blockIdx.x;
+    const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int l = blockIdx.x / CS;
     const size_t lay = (size_t)l * dp * dp;
     auto tile = [&](double* base, int i, int j) {
         return base + lay + (size_t)(lo + i) * kTile * dp + (size_t)(lo + j) * kTile;
     };
     if (threadIdx.x == 0) sm.flag = 0;
-    SmallAcc acc;
+    // operands into shared memory: ta = x, tb = y
+    auto fetch = [&](const double* x, const double* y) {
+        __syncthreads();                                   // the previous product's readers are done
+        tile_async(sm.ta, x, dp);
+        tile_async(sm.tb, y, dp);
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+    };
+    // out = sign * product (+ out)
+    auto store = [&](const SmallAcc& acc, double* out, double sign, bool add) {
+        small_epilogue(acc, [&](int r, int c, double2 v) {
+            double2* o = reinterpret_cast<double2*>(out + (size_t)r * dp + c);
+            double2 x = make_double2(sign * v.x, sign * v.y);
+            if (add) { const double2 cur = *o; x.x += cur.x; x.y += cur.y; }
+            *o = x;
+        });
+    };
     for (int j = 0; j < nt; ++j) {
-        leaf_factor(tile(A, j, j), tile(M, j, j), dp, sm);
-        // F_ij = A_ij D_j^T
-        for (int i = j + 1; i < nt; ++i) {
-            tile_async(sm.ta, tile(A, i, j), dp);
-            cp_async_commit();
-            cp_async_wait<0>();
-            __syncthreads();
+        if (rank == 0) leaf_factor(tile(A, j, j), tile(M, j, j), dp, sm);
+        cluster.sync();
+        // ---- row and column j
+        for (int q = rank; q < nt - 1; q += CS) {
+            SmallAcc acc;
             acc.zero();
-            tile_mma<false, false>(acc, sm.ta, sm.td);
-            double* out = tile(F, i, j);
-            small_epilogue(acc, [&](int r, int c, double2 v) {
-                *reinterpret_cast<double2*>(out + (size_t)r * dp + c) = v;
-            });
-            __syncthreads();
-        }
-        // A_ik -= F_ij F_kj^T for j < k <= i
-        for (int i = j + 1; i < nt; ++i)
-            for (int k = j + 1; k <= i; ++k) {
-                tile_async(sm.ta, tile(F, i, j), dp);
-                tile_async(sm.tb, tile(F, k, j), dp);
-                cp_async_commit();
-                cp_async_wait<0>();
-                __syncthreads();
-                acc.zero();
+            if (q < nt - 1 - j) {
+                const int i = j + 1 + q;
+                fetch(tile(A, i, j), tile(M, j, j));
                 tile_mma<false, false>(acc, sm.ta, sm.tb);
-                double* out = tile(A, i, k);
-                small_epilogue(acc, [&](int r, int c, double2 v) {
-                    double2* o = reinterpret_cast<double2*>(out + (size_t)r * dp + c);
-                    double2 cur = *o;
-                    cur.x -= v.x; cur.y -= v.y;
-                    *o = cur;
-                });
-                __syncthreads();
-            }
-    }
-    // M_ij = -M_ii (sum over j <= k < i of F_ik M_kj), column by column
-    for (int j = 0; j < nt; ++j)
-        for (int i = j + 1; i < nt; ++i) {
-            acc.zero();
-            for (int k = j; k < i; ++k) {
-                tile_async(sm.ta, tile(F, i, k), dp);
-                tile_async(sm.tb, tile(M, k, j), dp);
-                cp_async_commit();
-                cp_async_wait<0>();
-                __syncthreads();
+                store(acc, tile(F, i, j), 1.0, false);
+            } else {
+                const int k = q - (nt - 1 - j);
+                fetch(tile(M, j, j), tile(M, j, k));
                 tile_mma<false, true>(acc, sm.ta, sm.tb);
-                __syncthreads();
+                store(acc, tile(M, j, k), 1.0, false);
             }
-            tile_async(sm.ta, tile(M, i, i), dp);
-            cp_async_commit();
-            small_epilogue(acc, [&](int r, int c, double2 v) {
-                *reinterpret_cast<double2*>(sm.tb + r * PS + c) = v;
-            });
-            cp_async_wait<0>();
-            __syncthreads();
-            acc.zero();
-            tile_mma<false, true>(acc, sm.ta, sm.tb);
-            double* out = tile(M, i, j);
-            small_epilogue(acc, [&](int r, int c, double2 v) {
-                *reinterpret_cast<double2*>(out + (size_t)r * dp + c) = make_double2(-v.x, -v.y);
-            });
-            __syncthreads();
         }
+        if (j + 1 == nt) break;
+        cluster.sync();
+        // ---- what is behind them: tile 0 is the next diagonal tile and rank 0's
+        const int rest = nt - 1 - j, n_a = rest * (rest + 1) / 2, n_all = n_a + rest * (j + 1);
+        for (int q = rank; q < n_all; q += (rank == 0 || CS == 1) ? (CS == 1 ? 1 : n_all) : CS - 1) {
+            SmallAcc acc;
+            acc.zero();
+            if (q < n_a) {
+                int ii = 0, kk = q;
+                while (kk > ii) { kk -= ii + 1; ++ii; }
+                const int i = j + 1 + ii, k = j + 1 + kk;
+                fetch(tile(F, i, j), tile(F, k, j));
+                tile_mma<false, false>(acc, sm.ta, sm.tb);
+                store(acc, tile(A, i, k), -1.0, true);
+            } else {
+                const int i = j + 1 + (q - n_a) / (j + 1), k = (q - n_a) % (j + 1);
+                fetch(tile(F, i, j), tile(M, j, k));
+                tile_mma<false, true>(acc, sm.ta, sm.tb);
+                store(acc, tile(M, i, k), -1.0, k < j);
+            }
+        }
+    }
     if (threadIdx.x == 0 && sm.flag) set_layer_status(layer_status, l, sm.flag);
 }
 
@@ -665,22 +666,25 @@ ziplm_status factor_range(const InvCtx& c, int lo, int hi) {
             k_factor_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
         if (attr != cudaSuccess) return ZIPLM_ERR_CUDA;
         PhaseScope ps(PH_INV_LEAVES, c.st);
-        // One CTA per layer and a long dependent chain: launched at the highest priority, so that
+        // A few CTAs per layer and a long dependent chain: launched at the highest priority, so that
         // it does not queue behind the wide kernels of other layer groups.
         static int prio = [] {
             int least = 0, greatest = 0;
             return cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess ? greatest : 0;
         }();
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(c.L);
+        cfg.gridDim = dim3(c.L * kSmallCluster);
         cfg.blockDim = dim3(kSmallThreads);
         cfg.dynamicSmemBytes = sizeof(SmallSmem);
         cfg.stream = c.st;
-        cudaLaunchAttribute la[1];
+        cudaLaunchAttribute la[2];
         la[0].id = cudaLaunchAttributePriority;
         la[0].val.priority = prio;
+        la[1].id = cudaLaunchAttributeClusterDimension;
+        la[1].val.clusterDim.x = kSmallCluster;
+        la[1].val.clusterDim.y = la[1].val.clusterDim.z = 1;
         cfg.attrs = la;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_factor_small, c.A, c.F, c.M, c.dp, lo, hi - lo,
                                             c.layer_status));
         ZIPLM_CHECK_LAUNCH();
