@@ -1,0 +1,39 @@
+// What the two tensor-core product kernels of the Hessian share (hessian_tc.cu, hessian_pair.cu).
+#pragma once
+
+#include <cuda.h>
+
+#include "common.cuh"
+
+namespace ziplm {
+
+// One product launch: H[layer0 + l] = beta H + alpha X X^T for `layers` layers of a K-major operand.
+struct HessianProduct {
+    CUtensorMap hi, lo;          // 16-bit operand, or the two fp16 parts of fp32 input (split)
+    float* H;
+    int d, layers, num_kb;       // K blocks of 64 tokens
+    float alpha, beta;
+    int layer0;
+    int* err_word;
+    uint32_t fmt16, spin;        // operand format of the instruction; poll limit of the producer
+    const unsigned* amax;        // split: largest magnitudes of the feature rows
+    bool split;
+};
+
+// The pair kernel takes a launch when its tiles of 256 x 256 fill the CTA pairs of the chip.
+bool hessian_pair_fits(int layers, int d);
+size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split);
+ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st);
+
+// Power-of-two scale of a feature row from the bit pattern of its largest magnitude m: the largest
+// scaled entry lies in [2^13, 2^14).  inverse = true gives 1 / scale.  Rows of zeros and
+// non-finite rows are left alone; the exponent is clamped so that the scale is a normal number.
+__device__ __forceinline__ float row_scale(unsigned amax_bits, bool inverse) {
+    const int e = (int)((amax_bits >> 23) & 255u);
+    if (amax_bits == 0u || e == 255) return 1.f;
+    int k = 140 - e;                       // m in [2^(e-127), 2^(e-126))  ->  m 2^k < 2^14
+    k = k > 100 ? 100 : (k < -100 ? -100 : k);
+    return __int_as_float((127 + (inverse ? -k : k)) << 23);
+}
+
+}  // namespace ziplm

@@ -1,0 +1,372 @@
+// Calibration Hessian on CTA pairs: the product kernel for problems of many tiles.
+//
+// Same contraction, operands and numerics as k_syrk_tc (hessian_tc.cu), on tiles of 256 x 256 that a
+// pair of CTAs computes together with tcgen05.mma.cta_group::2 (M = N = 256): each CTA holds 128 rows of
+// both operands in its shared memory and 128 rows of the product in its tensor memory.  The 128 x 128
+// kernel was bound by its operand traffic from L2 (64 KB per K block of split fp32 against 800 clocks of
+// MMAs, about 40 B per clock and SM arrive): a pair moves the same bytes per CTA for twice the products.
+//
+// Tensor memory holds two accumulators of 256 columns, drained in turn after every chunk of K into fp32
+// registers (accumulation in tensor memory truncates, so a chain is kept to at most eight MMAs of the
+// main term).  There is no room for a third accumulator for the cross terms X_1 X_2^T + X_2 X_1^T of
+// split fp32: they go first into the chunk's own accumulator, where they meet nothing but each other
+// (2^-11 of the main term, so what their truncation loses is negligible), and the main term follows on
+// top.  The partial sums are added in two levels; 64 columns of running sums per thread fill the
+// registers, so the second level is a tile of scratch in global memory (in L2) that every FOLD drains
+// are added to with red.add: one writer per address, so the sums are the same on every run.
+//
+// Roles of a CTA: warp 0 loads its own half of the operands by TMA (no multicast; the bytes of both
+// halves are counted on the leader's barrier), one thread of warp 1 of the leader issues the MMAs for
+// both CTAs, warps 2 .. 17 drain (four TMEM lane quarters x four quarters of the columns).  Every wait
+// is bounded; a role that gives up raises the abort flag of both CTAs.
+#include <cuda.h>
+
+#include "common.cuh"
+#include "hessian_common.cuh"
+#include "tc_common.cuh"
+
+namespace ziplm {
+namespace {
+using namespace tc;
+
+constexpr int PT = 256;                       // tile rows / columns of a pair
+constexpr int HALF = 128;                     // rows of an operand per CTA
+constexpr int BK = 64;                        // K block: one 128-byte swizzle row of 16-bit elements
+constexpr int OP_BYTES = HALF * 128;          // one operand half, one part, one K block: 16 KiB
+constexpr int PAIR_EPI = 16;                  // epilogue warps
+constexpr int PAIR_THREADS = 32 * (2 + PAIR_EPI);
+constexpr int FOLD = 32;                      // drains between additions to the second level
+constexpr int NC = 64;                        // columns per epilogue thread
+
+template <bool SPLIT> struct PairCfg;         // SPLIT: two fp16 parts per operand (fp32 inputs)
+template <> struct PairCfg<true>  { static constexpr int STAGES = 3, PARTS = 2, CHUNK = 1; };
+template <> struct PairCfg<false> { static constexpr int STAGES = 6, PARTS = 1, CHUNK = 2; };
+template <bool SPLIT>
+constexpr int kStageBytes = 2 * PairCfg<SPLIT>::PARTS * OP_BYTES;      // A half and B half
+template <bool SPLIT>
+constexpr int kPairSmem = PairCfg<SPLIT>::STAGES * kStageBytes<SPLIT> + 1024;
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Arrive at a barrier of the pair's other CTA (or of this one), by its shared::cluster address.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// Wait whose phase another CTA of the cluster may complete.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                                  uint32_t limit) {
+    const long long t0 = clock64();
+    for (uint32_t it = 0; it < limit; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if ((it & 63u) == 63u && (*abort_flag || clock64() - t0 > kSpinClocks)) return false;
+    }
+    return false;
+}
+// TMA load into this CTA's shared memory, counted on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
+                                                 int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Arrive at the barrier at this offset in both CTAs once the MMAs issued so far have completed.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+        ::"r"(bar), "h"((uint16_t)3) : "memory");
+}
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(PAIR_THREADS, 1) __cluster_dims__(2, 1, 1)
+k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+            float* __restrict__ H, int d, int num_kb, float alpha, float beta, int layer0,
+            int* __restrict__ err_word, uint32_t fmt16, uint32_t empty_spin_limit,
+            const unsigned* __restrict__ amax, float4* __restrict__ level2) {
+    using C = PairCfg<SPLIT>;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bar_full[C::STAGES], bar_empty[C::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_final;
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag;
+
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t tiles = (raw + 1023u) & ~1023u;        // swizzled tiles need 1024-byte alignment
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = blockIdx.x & 1u;                // CTA of the pair; 0 leads
+    const int l = blockIdx.y;                             // layer within the launched chunk
+    int ti = 0, rem = (int)(blockIdx.x >> 1);
+    while (rem > ti) { rem -= ti + 1; ++ti; }
+    const int tj = rem;
+    const int i0 = ti * PT, j0 = tj * PT;
+    const bool diag = (ti == tj);
+    const int num_chunks = (num_kb + C::CHUNK - 1) / C::CHUNK;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int s = 0; s < C::STAGES; ++s) {
+            mbar_init(smem_u32(&bar_full[s]), 1);
+            mbar_init(smem_u32(&bar_empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&bar_acc_full[b]), 1);
+            mbar_init(smem_u32(&bar_acc_empty[b]), 2 * PAIR_EPI);     // every epilogue warp of both CTAs
+        }
+        mbar_init(smem_u32(&bar_final), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_barrier();                                    // both CTAs' barriers are initialised
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = tmem_base_slot;
+    volatile int* abortp = &abort_flag;
+    bool failed = false;
+    int issued = 0;                                       // K blocks whose copies were started (thread 0)
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---------------- TMA producer (each CTA its own half of the operands)
+            const uint32_t bytes = (uint32_t)((diag ? 1 : 2) * C::PARTS * OP_BYTES);
+            const int ya = i0 + (int)rank * HALF, yb = j0 + (int)rank * HALF;
+            for (int kb = 0; kb < num_kb; ++kb) {
+                const int s = kb % C::STAGES;
+                const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
+                if (empty_spin_limit < kSpinLimit
+                        ? !mbar_wait_limit(smem_u32(&bar_empty[s]), ph ^ 1u, abortp, empty_spin_limit)
+                        : !mbar_wait_cluster(smem_u32(&bar_empty[s]), ph ^ 1u, abortp, kSpinLimit)) {
+                    failed = true;
+                    break;
+                }
+                const uint32_t full = cluster_addr(smem_u32(&bar_full[s]), 0);
+                const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
+                if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2 * bytes);
+                const int x = kb * BK;
+                tma_load_3d_pair(base, &map_hi, full, x, ya, l);
+                if (SPLIT) tma_load_3d_pair(base + OP_BYTES, &map_lo, full, x, ya, l);
+                if (!diag) {
+                    tma_load_3d_pair(base + C::PARTS * OP_BYTES, &map_hi, full, x, yb, l);
+                    if (SPLIT) tma_load_3d_pair(base + 3 * OP_BYTES, &map_lo, full, x, yb, l);
+                }
+                issued = kb + 1;
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && rank == 0) {
+            // ---------------- MMA issuer (the leader, for both CTAs)
+            const uint32_t idesc = make_idesc(SPLIT ? 0u : fmt16, PT, PT);
+            int kb = 0;
+            for (int c = 0; c < num_chunks && !failed; ++c) {
+                const int b = c & 1;
+                const uint32_t acc = tmem_base + (uint32_t)b * PT;
+                // both CTAs must have drained this buffer (first use of each buffer passes)
+                if (!mbar_wait_cluster(smem_u32(&bar_acc_empty[b]), (((uint32_t)c >> 1) & 1u) ^ 1u, abortp,
+                                       kSpinLimit)) {
+                    failed = true;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int kb_end = (kb + C::CHUNK < num_kb) ? kb + C::CHUNK : num_kb;
+                uint32_t add = 0u;
+                for (; kb < kb_end; ++kb) {
+                    const int s = kb % C::STAGES;
+                    const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
+                    if (!mbar_wait_cluster(smem_u32(&bar_full[s]), ph, abortp, kSpinLimit)) { failed = true; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
+                    const uint64_t a_hi = make_desc(base), a_lo = make_desc(base + OP_BYTES);
+                    const uint64_t b_hi = diag ? a_hi : make_desc(base + C::PARTS * OP_BYTES);
+                    const uint64_t b_lo = diag ? a_lo : make_desc(base + 3 * OP_BYTES);
+                    if (SPLIT) {
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k) {
+                            umma_pair(acc, a_hi + 2u * k, b_lo + 2u * k, idesc, add);
+                            add = 1u;
+                            umma_pair(acc, a_lo + 2u * k, b_hi + 2u * k, idesc, 1u);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k) {       // 32 bytes per MMA along K
+                        umma_pair(acc, a_hi + 2u * k, b_hi + 2u * k, idesc, add);
+                        add = 1u;
+                    }
+                    umma_commit_pair(smem_u32(&bar_empty[s]));     // stage free once these MMAs have read it
+                }
+                if (!failed) umma_commit_pair(smem_u32(&bar_acc_full[b]));
+            }
+            // whatever was issued has completed before tensor memory is given back
+            umma_commit_pair(smem_u32(&bar_final));
+            mbar_wait_quiet(smem_u32(&bar_final), 0u);
+        }
+    } else {
+        // ---------------- epilogue: lane quarter = warp % 4, quarter of the columns by warp
+        const int q = warp & 3, cq = (warp - 2) >> 2;
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        const uint32_t empty0 = cluster_addr(smem_u32(&bar_acc_empty[0]), 0);
+        const uint32_t empty1 = cluster_addr(smem_u32(&bar_acc_empty[1]), 0);
+        const int et = (int)threadIdx.x - 64;
+        float4* l2 = level2 + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (HALF * PT / 4) + et;
+        float acc[NC];
+#pragma unroll
+        for (int e = 0; e < NC; ++e) acc[e] = 0.f;
+        bool folded = false;
+        for (int c = 0; c < num_chunks; ++c) {
+            const int b = c & 1;
+            if (!mbar_wait_cluster(smem_u32(&bar_acc_full[b]), ((uint32_t)c >> 1) & 1u, abortp, kSpinLimit))
+                failed = true;
+            failed = __any_sync(0xffffffffu, failed);
+            if (failed) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int cc = 0; cc < NC / 16; ++cc) {
+                uint32_t v[16];
+                tmem_ld16(tmem_base + lane_base + (uint32_t)(b * PT + cq * NC + cc * 16), v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) acc[cc * 16 + e] += __uint_as_float(v[e]);
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(b ? empty1 : empty0);
+            if ((c % FOLD) == FOLD - 1 && c + 1 < num_chunks) {
+                // second level, [16 quads][512 threads]
+#pragma unroll
+                for (int e = 0; e < NC / 4; ++e) {
+                    float4* p = l2 + (size_t)e * (32 * PAIR_EPI);
+                    if (folded)
+                        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(acc[4 * e]),
+                                     "f"(acc[4 * e + 1]), "f"(acc[4 * e + 2]), "f"(acc[4 * e + 3]) : "memory");
+                    else
+                        __stcg(p, make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
+                    acc[4 * e] = acc[4 * e + 1] = acc[4 * e + 2] = acc[4 * e + 3] = 0.f;
+                }
+                folded = true;
+            }
+        }
+        if (!failed) {
+            if (folded)
+#pragma unroll
+                for (int e = 0; e < NC / 4; ++e) {
+                    const float4 t = __ldcg(l2 + (size_t)e * (32 * PAIR_EPI));
+                    acc[4 * e] += t.x; acc[4 * e + 1] += t.y; acc[4 * e + 2] += t.z; acc[4 * e + 3] += t.w;
+                }
+            // The operand ring is free (every MMA has completed): the warp's 32 x 64 results pass
+            // through it, so that rows [i][j] leave along j and mirrored rows [j][i] along i.
+            float* buf = reinterpret_cast<float*>(smem_raw + (tiles - raw)) + (size_t)(warp - 2) * 32 * (NC + 1);
+            float* Hl = H + (size_t)(layer0 + l) * d * d;
+            const int r0 = i0 + (int)rank * HALF + q * 32, c0 = j0 + cq * NC;
+            const unsigned* am = SPLIT ? amax + (size_t)l * d : nullptr;
+            // split route: undo the power-of-two scales of the two feature rows (exact)
+            const float inv_row = (SPLIT && r0 + lane < d) ? row_scale(am[r0 + lane], true) : 1.f;
+#pragma unroll
+            for (int e = 0; e < NC; ++e) {
+                float v = alpha * acc[e];
+                if (SPLIT && c0 + e < d) v = (v * inv_row) * row_scale(am[c0 + e], true);
+                buf[lane * (NC + 1) + e] = v;
+            }
+            __syncwarp();
+            for (int rr = 0; rr < 32; ++rr) {
+                const int row = r0 + rr;
+                if (row >= d) break;
+#pragma unroll
+                for (int h = 0; h < NC / 32; ++h) {
+                    const int cc = 32 * h + lane, col = c0 + cc;
+                    if (col > row) continue;                 // (col <= row < d)
+                    float v = buf[rr * (NC + 1) + cc];
+                    float* p = Hl + (size_t)row * d + col;
+                    if (beta != 0.f) {
+                        v += *p;
+                        buf[rr * (NC + 1) + cc] = v;
+                    }
+                    *p = v;
+                }
+            }
+            __syncwarp();
+            const int row = r0 + lane;
+#pragma unroll 4
+            for (int e = 0; e < NC; ++e) {
+                const int col = c0 + e;
+                if (row < d && col < row) Hl[(size_t)col * d + row] = buf[lane * (NC + 1) + e];
+            }
+        }
+    }
+
+    if (failed) {
+        atomicExch(err_word, (int)ZIPLM_ERR_TIMEOUT);
+        for (uint32_t r = 0; r < 2; ++r)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), r)), "r"(1)
+                         : "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && rank == 0 && abort_flag) {
+        // Copies that were started land in the pair's shared memory and are counted here: wait for
+        // them (bounded; the last STAGES K blocks are the latest phases of their barriers) before
+        // either CTA retires.
+        for (int kb = issued > C::STAGES ? issued - C::STAGES : 0; kb < issued; ++kb)
+            mbar_wait_quiet(smem_u32(&bar_full[kb % C::STAGES]), (uint32_t)(kb / C::STAGES) & 1u);
+    }
+    __syncwarp();
+    cluster_barrier();            // the pair's MMAs, copies and remote arrivals are over
+    if (warp == 1) {
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    }
+}
+
+int pair_count(int d) {
+    const int T = (d + PT - 1) / PT;
+    return T * (T + 1) / 2;
+}
+
+template <bool SPLIT>
+ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t st) {
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_pair<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          kPairSmem<SPLIT>));
+    k_syrk_pair<SPLIT><<<dim3(2 * pair_count(p.d), p.layers), PAIR_THREADS, kPairSmem<SPLIT>, st>>>(
+        p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0, p.err_word, p.fmt16, p.spin, p.amax, level2);
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
+}  // namespace
+
+bool hessian_pair_fits(int layers, int d) { return (long long)layers * pair_count(d) >= 74; }
+
+// Scratch of the second summation level, for the layers of one launch; none where FOLD drains are
+// never reached.
+size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split) {
+    const long long kb = (N + BK - 1) / BK, per = split ? PairCfg<true>::CHUNK : PairCfg<false>::CHUNK;
+    if ((kb + per - 1) / per <= FOLD) return 0;
+    return (size_t)layers * 2 * pair_count(d) * HALF * PT * sizeof(float);
+}
+
+ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st) {
+    float4* l2 = static_cast<float4*>(scratch);
+    return p.split ? launch_pair<true>(p, l2, st) : launch_pair<false>(p, l2, st);
+}
+
+}  // namespace ziplm

@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "hessian_common.cuh"
 #include "tc_common.cuh"
 
 namespace ziplm {
@@ -56,17 +57,6 @@ constexpr int CHUNK = 2;
 constexpr int FOLD = 32;
 constexpr int EPI_WARPS = 8;                  // two warps per TMEM lane quarter, 64 columns each
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
-
-// Power-of-two scale of a feature row from the bit pattern of its largest magnitude m: the largest
-// scaled entry lies in [2^13, 2^14).  inverse = true gives 1 / scale.  Rows of zeros and
-// non-finite rows are left alone; the exponent is clamped so that the scale is a normal number.
-__device__ __forceinline__ float row_scale(unsigned amax_bits, bool inverse) {
-    const int e = (int)((amax_bits >> 23) & 255u);
-    if (amax_bits == 0u || e == 255) return 1.f;
-    int k = 140 - e;                       // m in [2^(e-127), 2^(e-126))  ->  m 2^k < 2^14
-    k = k > 100 ? 100 : (k < -100 ? -100 : k);
-    return __int_as_float((127 + (inverse ? -k : k)) << 23);
-}
 
 template <bool TF32>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -520,7 +510,6 @@ bool make_map(CUtensorMap* m, const void* base, ziplm_dtype dt, long long K, int
 
 constexpr size_t kSplitCapBytes = (size_t)8 << 30;   // bound on the hi/lo scratch of one chunk
 
-long long padded_tokens(long long N) { return (N + 3) / 4 * 4; }
 long long padded_tokens_bf16(long long N) { return (N + 7) / 8 * 8; }   // 16-byte row pitch
 
 // Layers per chunk of the K-major bf16 copy of a token-major input.
@@ -539,6 +528,13 @@ int split_chunk_layers(int L, int d, long long N) {
     return (int)(lc < (size_t)L ? lc : (size_t)L);
 }
 
+// Most layers of one product launch.
+int product_layers(int L, int d, long long N, ziplm_dtype dt, bool token_major) {
+    if (dt == ZIPLM_F32) return split_chunk_layers(L, d, N);
+    if (token_major) return transpose_chunk_layers(L, d, N);
+    return L < 65535 ? L : 65535;
+}
+
 }  // namespace
 
 size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, bool token_major) {
@@ -551,8 +547,34 @@ size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, boo
         const int lc = transpose_chunk_layers(L, d, N);
         b += align_up((size_t)lc * d * (size_t)padded_tokens_bf16(N) * 2);
     }
+    const int layers = product_layers(L, d, N, dt, token_major);
+    if (hessian_pair_fits(layers, d)) b += align_up(hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32));
     return b;
 }
+
+namespace {
+
+// One product launch on the kernel that suits its number of tiles.
+ziplm_status run_product(const HessianProduct& p, void* scratch, cudaStream_t st) {
+    if (hessian_pair_fits(p.layers, p.d)) return run_hessian_pair(p, scratch, st);
+    const int T = (p.d + TM - 1) / TM;
+    const dim3 grid(T * (T + 1) / 2, p.layers);
+    if (p.split) {
+        constexpr int smem = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
+        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_syrk_tc<true><<<grid, THREADS, smem, st>>>(p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0,
+                                                     p.err_word, 0u, p.spin, p.amax);
+    } else {
+        constexpr int smem = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
+        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_syrk_tc<false><<<grid, THREADS, smem, st>>>(p.hi, p.hi, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0,
+                                                      p.err_word, p.fmt16, p.spin, nullptr);
+    }
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
+}  // namespace
 
 ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_major, int L, int d,
                             long long N, long long ldx, float alpha, float beta, void* ws,
@@ -565,24 +587,24 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(err_word, 0, sizeof(int), st));
     const int spin_opt = option_value(ZIPLM_OPT_SPIN_LIMIT);
     const uint32_t spin = spin_opt > 0 ? (uint32_t)spin_opt : kSpinLimit;
-    const int T = (d + TM - 1) / TM;
-    const int n_tiles = T * (T + 1) / 2;
-    const size_t smem_tf32 = (size_t)Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
-    const size_t smem_bf16 = (size_t)Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
-    if (f32) {
-        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem_tf32));
-    } else {
-        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem_bf16));
-    }
+    HessianProduct prod = {};
+    prod.H = H; prod.d = d; prod.alpha = alpha; prod.beta = beta; prod.err_word = err_word;
+    prod.num_kb = (int)((N + Cfg<false>::BK - 1) / Cfg<false>::BK);
+    prod.fmt16 = fmt16; prod.spin = spin; prod.split = f32;
+    const int most_layers = product_layers(L, d, N, dt, token_major);
+    void* scratch = nullptr;             // of the pair kernel, behind the operands
+    auto take_scratch = [&] {
+        if (hessian_pair_fits(most_layers, d))
+            scratch = c.take<char>(hessian_pair_scratch_bytes(most_layers, d, N, f32));
+    };
     if (f32) {
         const long long np = padded_tokens_bf16(N);
         const int lc = split_chunk_layers(L, d, N);
         unsigned* amax = c.take<unsigned>((size_t)lc * d);
         __half* hi = c.take<__half>((size_t)lc * d * np);
         __half* lo = c.take<__half>((size_t)lc * d * np);
-        const int num_kb = (int)((N + Cfg<true>::BK - 1) / Cfg<true>::BK);
+        take_scratch();
+        prod.amax = amax;
         for (int l0 = 0; l0 < L; l0 += lc) {
             const int ln = (L - l0 < lc) ? (L - l0) : lc;
             const size_t rows = (size_t)ln * d;
@@ -643,19 +665,18 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                     }
                 }
             }
-            CUtensorMap mh, ml;
-            if (!make_map(&mh, hi, ZIPLM_F16, N, d, ln, np) || !make_map(&ml, lo, ZIPLM_F16, N, d, ln, np))
+            if (!make_map(&prod.hi, hi, ZIPLM_F16, N, d, ln, np) || !make_map(&prod.lo, lo, ZIPLM_F16, N, d, ln, np))
                 return ZIPLM_ERR_CUDA;
-            k_syrk_tc<true><<<dim3(n_tiles, ln), THREADS, smem_tf32, st>>>(mh, ml, H, d, num_kb, alpha, beta,
-                                                                      l0, err_word, 0u, spin, amax);
-            ZIPLM_CHECK_LAUNCH();
+            prod.layer0 = l0; prod.layers = ln;
+            const ziplm_status s = run_product(prod, scratch, st);
+            if (s != ZIPLM_OK) return s;
         }
     } else if (token_major) {
         // K-major bf16 copy of a chunk of layers, then the same product kernel
         const long long np = padded_tokens_bf16(N);
         const int lc = transpose_chunk_layers(L, d, N);
         uint16_t* xt = c.take<uint16_t>((size_t)lc * d * np);
-        const int num_kb = (int)((N + Cfg<false>::BK - 1) / Cfg<false>::BK);
+        take_scratch();
         for (int l0 = 0; l0 < L; l0 += lc) {
             const int ln = (L - l0 < lc) ? (L - l0) : lc;
             const uint16_t* Ac = static_cast<const uint16_t*>(X) + (size_t)l0 * (size_t)N * ldx;
@@ -668,24 +689,22 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                     <<<dim3((unsigned)((np + 31) / 32), (unsigned)((d + 31) / 32), (unsigned)ln), 256, 0, st>>>(
                         Ac, ldx, N, d, np, nullptr, xt, nullptr);
             ZIPLM_CHECK_LAUNCH();
-            CUtensorMap mx;
-            if (!make_map(&mx, xt, dt, N, d, ln, np)) return ZIPLM_ERR_CUDA;
-            k_syrk_tc<false><<<dim3(n_tiles, ln), THREADS, smem_bf16, st>>>(mx, mx, H, d, num_kb, alpha, beta,
-                                                                       l0, err_word, fmt16, spin, nullptr);
-            ZIPLM_CHECK_LAUNCH();
+            if (!make_map(&prod.hi, xt, dt, N, d, ln, np)) return ZIPLM_ERR_CUDA;
+            prod.lo = prod.hi; prod.layer0 = l0; prod.layers = ln;
+            const ziplm_status s = run_product(prod, scratch, st);
+            if (s != ZIPLM_OK) return s;
         }
     } else {
-        const int num_kb = (int)((N + Cfg<false>::BK - 1) / Cfg<false>::BK);
+        take_scratch();
         // tensor-map dimensions are 32-bit boxes over up to 2^32 elements; chunk layers so that the
         // grid stays within limits
         for (int l0 = 0; l0 < L; l0 += 65535) {
             const int ln = (L - l0 < 65535) ? (L - l0) : 65535;
-            CUtensorMap mx;
             const __nv_bfloat16* Xc = static_cast<const __nv_bfloat16*>(X) + (size_t)l0 * d * ldx;
-            if (!make_map(&mx, Xc, dt, N, d, ln, ldx)) return ZIPLM_ERR_CUDA;
-            k_syrk_tc<false><<<dim3(n_tiles, ln), THREADS, smem_bf16, st>>>(mx, mx, H, d, num_kb, alpha, beta,
-                                                                       l0, err_word, fmt16, spin, nullptr);
-            ZIPLM_CHECK_LAUNCH();
+            if (!make_map(&prod.hi, Xc, dt, N, d, ln, ldx)) return ZIPLM_ERR_CUDA;
+            prod.lo = prod.hi; prod.layer0 = l0; prod.layers = ln;
+            const ziplm_status s = run_product(prod, scratch, st);
+            if (s != ZIPLM_OK) return s;
         }
     }
     k_hessian_flag_timeout<<<(L + 127) / 128, 128, 0, st>>>(H, L, d, err_word);

@@ -767,3 +767,41 @@ def test_delayed_path_widths_that_are_no_multiple_of_four(d, r, levels):
     sh = wl.scaled(wl.CONFIGS["c3_bert_base_fc2"][0], d_col=d, d_row=r, d_latent=max(4, d // 4),
                    n_tokens=2 * d + 8, n_layers=2, levels=tuple(levels))
     run_case(sh)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("d,N,L", [(900, 40, 8), (257, 4500, 25), (1030, 2112, 5)])
+def test_hessian_on_cta_pairs_matches_oracle(dtype, d, N, L):
+    """Enough 256 x 256 tiles for the pair kernel: one K block, ragged edges of tiles and of the last
+    K block, more drains than the first summation level takes; then once more on top (beta = 1)."""
+    z = zb()
+    sh = wl.scaled(wl.CONFIGS["c3_bert_base_fc2"][0], d_col=d, d_latent=32, n_tokens=N, n_layers=1, x_dtype=dtype)
+    X1 = wl.make_activations(sh, 0)
+    Ad = torch.stack([X1.t().contiguous() * (1 + l) for l in range(L)]).cuda()      # exact powers are not needed
+    H = z.hessian_accumulate_tokens(Ad)
+    H2 = z.hessian_accumulate_tokens(Ad, H.clone(), beta=1.0)
+    torch.cuda.synchronize()
+    for l in (0, L - 1):
+        Ho = zo.hessian(Ad[l].t().cpu())
+        scale = np.sqrt(np.outer(np.diag(Ho), np.diag(Ho)))
+        assert np.max(np.abs(H[l].cpu().double().numpy() - Ho) / scale) < 2e-6
+        assert np.max(np.abs(H2[l].cpu().double().numpy() - 2 * Ho) / scale) < 4e-6
+        assert torch.equal(H2[l], H2[l].t())
+
+
+def test_a_bounded_wait_of_the_pair_kernel_that_runs_out_is_reported():
+    """As above for the kernel on CTA pairs: both producers give up after one look."""
+    z = zb()
+    Xd = torch.randn(25, 300, 1024, generator=torch.Generator().manual_seed(1)).cuda()
+    z.set_option(z.Option.SPIN_LIMIT, 1)
+    try:
+        H = z.hessian_accumulate(Xd)
+        torch.cuda.synchronize()
+    finally:
+        z.set_option(z.Option.SPIN_LIMIT, 0)
+    assert torch.isnan(H[:, 0, 0]).all()
+    H = z.hessian_accumulate(Xd)
+    torch.cuda.synchronize()
+    Ho = zo.hessian(Xd[24].cpu())
+    scale = np.sqrt(np.outer(np.diag(Ho), np.diag(Ho)))
+    assert np.max(np.abs(H[24].cpu().double().numpy() - Ho) / scale) < 2e-6
