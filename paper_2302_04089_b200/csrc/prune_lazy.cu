@@ -175,21 +175,57 @@ __device__ __forceinline__ Cand warp_best(const Cand& mine, float r, float* warp
 
 __device__ __forceinline__ Cand warp_best(const Cand& mine) { return warp_best(mine, cand_quotient(mine)); }
 
+// What a warp, or a CTA, offers as its next pick.
+struct __align__(16) Offer {
+    Cand c;
+};
+
+// Pick among n <= 32 offers by their fp32 keys (good to 1e-5): when exactly one key lies within 4e-5 of
+// the smallest, that offer is the pick and is read directly; otherwise -- near ties, an invalid entry,
+// nothing left -- all of them go through the exact comparison.  Every lane returns the pick and its index.
+__device__ __forceinline__ Cand pick_offer(const Offer* offers, const float* keys, int n, int lane, int* which) {
+    const float k = lane < n ? keys[lane] : INFINITY;
+    const unsigned bits = __float_as_uint(k);
+    const unsigned kmin = __reduce_min_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
+    const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
+    const unsigned near_min = __ballot_sync(0xffffffffu, k <= rmin + fabsf(rmin) * 4e-5f);
+    if (fabsf(rmin) < INFINITY && __popc(near_min) == 1) {
+        *which = __ffs(near_min) - 1;
+        return offers[*which].c;
+    }
+    Cand g;
+    g.a = 1.0; g.q = 0.0; g.org = 0x7fffffff; g.pos = -1;
+    if (lane < n) g = offers[lane].c;
+    const Cand best = warp_best(g);
+    const unsigned mine = __ballot_sync(0xffffffffu, lane < n && best.pos >= 0 && g.pos == best.pos);
+    *which = mine ? __ffs(mine) - 1 : 0;
+    return best;
+}
+
 // nsteps greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
 // chosen so that a CTA's slice of positions fits its shared memory).  CTA `rank` owns the
 // positions [rank * S, rank * S + S); each of its 256 threads owns four consecutive ones and
 // keeps their float64 diagonal entries of H^-1 and Q in registers for the whole block.  The
-// pending vectors u_s, z_s of the block live in shared memory, sliced the same way, so the
+// pending vectors u_s, z_s of the block live in shared memory, sliced the same way (pitch Sp), so the
 // correction of a pivot column touches no global memory; copies go to global memory only for
-// the update kernels that follow.  Per step there is one cluster barrier: every warp publishes
-// its best candidate, after the barrier warp 0 of every CTA reads all of them through
-// distributed shared memory and reaches the same pick, then fetches the pending vectors'
-// entries at the pivot from the CTA that owns it.
+// the update kernels that follow.
+//
+// A step is a chain of latencies, so its parts are as short as they can be made and nothing waits for a
+// hand-over that it can do without: the fp32 quotients of a thread's four positions are formed without
+// branches (validity is tested on the upper words; the exact float64 comparison only sees positions within
+// 1e-5 of each other), every warp offers its best, and after the barrier every warp makes the pick for
+// itself and requests the pivot rows at once.  On a cluster (MULTI) warp 0 of a CTA picks the CTA's best
+// first and pushes it to all CTAs together with the pending entries at its position, which the winner's
+// column needs; the cluster barrier is then the only one after it.  The step took 4800 to 5200 clocks when
+// the four quotients and their comparisons ran one after the other (1400 of them) and warp 0 fetched the
+// pending entries after the pick and handed over (1450).
+//
 // The scaled pivot columns of W (c_s) do not feed the selection; they are solved for at the end
 // of the block by forward substitution with the 32 x 32 triangle T[m][s] = u_s[p_m].
 // Finally the per-position vectors are compacted (stable) across the cluster.
+template <bool MULTI>
 __global__ void __launch_bounds__(STEP_THREADS, 1)
-k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r, int rp,
+k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int G, int r, int rp,
              const float* __restrict__ A, const float* __restrict__ Q, const float* __restrict__ Wt,
              const double* __restrict__ dA_in, const double* __restrict__ dQ_in,
              const int* __restrict__ idx_in, double* __restrict__ dA_out,
@@ -199,24 +235,25 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
              int* layer_status) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    const int CS = (int)cluster.num_blocks();
-    const int rank = (int)cluster.block_rank();
+    const int CS = MULTI ? (int)cluster.num_blocks() : 1;
+    const int rank = MULTI ? (int)cluster.block_rank() : 0;
     const int l = blockIdx.x / CS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = STEP_THREADS / 32;
 
     extern __shared__ float4 dyn_smem4[];
-    float* sU = reinterpret_cast<float*>(dyn_smem4);       // [BMAX][S]
-    float* sZ = sU + (size_t)BMAX * S;                     // [BMAX][S]
-    __shared__ Cand s_cand[2][CLUSTER_MAX * NW];           // all warps of the cluster, by step parity
-    __shared__ float s_key[2][CLUSTER_MAX * NW];           // ... and their smallest fp32 quotients
+    float* sU = reinterpret_cast<float*>(dyn_smem4);       // [BMAX][Sp]
+    float* sZ = sU + (size_t)BMAX * Sp;                    // [BMAX][Sp]
+    double (*sTd)[BMAX] = reinterpret_cast<double (*)[BMAX]>(dyn_smem4);   // T in float64, after the last step
+    __shared__ Offer s_warp[2][NW];                        // the warps' offers, by step parity, and their keys
+    __shared__ float s_wkey[2][NW];
+    __shared__ Offer s_cta[2][CLUSTER_MAX];                // the CTAs' offers, their keys, and the pending
+    __shared__ float s_ckey[2][CLUSTER_MAX];               // entries (u_s[p], z_s[p]) at their positions
+    __shared__ float2 s_pend[2][CLUSTER_MAX][BMAX];
     __shared__ float sT[BMAX][BMAX];                       // T[m][s] = u_s[p_m]
-    __shared__ double sTd[BMAX][BMAX];                     // ... in float64, for the solve of c_m
-    __shared__ float sUp[BMAX], sZp[BMAX];
     __shared__ int s_pm[BMAX];
     __shared__ double s_rsm[BMAX];
-    __shared__ int s_p, s_count, s_wsum[NW];
-    __shared__ double s_rs, s_half;
+    __shared__ int s_count, s_wsum[NW];
 
     const float* Al = A + (size_t)l * d * d;
     const float* Ql = Q + (size_t)l * d * d;
@@ -246,85 +283,82 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
 
     for (int m = 0; m < nsteps; ++m) {
         const int par = m & 1;
-        // ---- per-warp best of rho = Q[k,k] / H^-1[k,k] (ties: lowest original index).  The four
-        //      owned positions are ordered by an fp32 quotient; only those within 1e-5 of the
-        //      smallest (almost always one) go through the exact float64 comparison.
-        Cand best;
-        best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff; best.pos = -1;
-        float rq[4], rbest = INFINITY;
+        // ---- best of the four owned positions of rho = Q[k,k] / H^-1[k,k] (ties: lowest original index)
+        float rq[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            rq[e] = INFINITY;
-            if (alive[e]) {
-                const bool ok = da[e] > 0.0 && isfinite(da[e]) && isfinite(dq[e]);
-                rq[e] = ok ? __fdividef((float)dq[e], (float)da[e]) : -INFINITY;
-            }
-            rbest = fminf(rbest, rq[e]);
+            const int ha = __double2hiint(da[e]), hq = __double2hiint(dq[e]);
+            const bool ok = (unsigned)(ha - 1) < 0x7fefffffu && (hq & 0x7fffffff) < 0x7ff00000;   // a > 0, finite
+            const float x = __fdividef((float)dq[e], (float)da[e]);
+            rq[e] = alive[e] ? (ok ? x : -INFINITY) : INFINITY;
         }
+        const float rbest = fminf(fminf(rq[0], rq[1]), fminf(rq[2], rq[3]));
+        const float thr = rbest + fabsf(rbest) * 1e-5f;
+        unsigned near_mine = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (!alive[e] || !(rq[e] == rbest || rq[e] <= rbest + fabsf(rbest) * 1e-5f)) continue;
-            Cand c;
-            c.a = da[e]; c.q = dq[e]; c.org = org[e]; c.pos = k0 + e;
-            merge_cand(best, c);
+        for (int e = 0; e < 4; ++e) near_mine |= (alive[e] && (rq[e] == rbest || rq[e] <= thr)) ? 1u << e : 0u;
+        Cand best;
+        best.a = near_mine & 1 ? da[0] : near_mine & 2 ? da[1] : near_mine & 4 ? da[2] : da[3];
+        best.q = near_mine & 1 ? dq[0] : near_mine & 2 ? dq[1] : near_mine & 4 ? dq[2] : dq[3];
+        best.org = near_mine & 1 ? org[0] : near_mine & 2 ? org[1] : near_mine & 4 ? org[2] : org[3];
+        best.pos = near_mine ? k0 + __ffs(near_mine) - 1 : -1;
+        if (near_mine & (near_mine - 1)) {         // several within 1e-5: the exact comparison
+            best.pos = -1;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (!(near_mine >> e & 1)) continue;
+                Cand c;
+                c.a = da[e]; c.q = dq[e]; c.org = org[e]; c.pos = k0 + e;
+                merge_cand(best, c);
+            }
         }
         float wmin;
         best = warp_best(best, best.pos >= 0 ? rbest : INFINITY, &wmin);
-        // push: lane c < CS hands the warp's candidate to CTA c, so that after the barrier every
-        // CTA finds all candidates in its own shared memory -- together with the warp's smallest
-        // fp32 quotient (within 1e-5 of the candidate's own), the key of the coarse ordering below
-        if (lane < CS) {
-            *cluster.map_shared_rank(&s_cand[par][rank * NW + warp], lane) = best;
-            *cluster.map_shared_rank(&s_key[par][rank * NW + warp], lane) = wmin;
-        }
-        cluster.sync();
-        // ---- warp 0 of every CTA: global pick from all warps of all CTAs, then the pending
-        //      vectors' entries at the pivot (from the CTA that owns it)
-        if (warp == 0) {
-            // Coarse ordering by the pushed keys: when exactly one of them lies within 4e-5 of the
-            // smallest (the keys are good to 1e-5), its candidate is the pick and is read directly;
-            // otherwise -- near ties, an invalid entry, nothing left -- all candidates go through
-            // the exact comparison.
-            Cand g;
-            {
-                const float k0v = (lane < CS * NW) ? s_key[par][lane] : INFINITY;
-                const float k1v = (lane + 32 < CS * NW) ? s_key[par][lane + 32] : INFINITY;
-                const float kl = fminf(k0v, k1v);
-                const unsigned bits = __float_as_uint(kl);
-                const unsigned key = bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
-                const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
-                const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
-                const float thr = rmin + fabsf(rmin) * 4e-5f;
-                const unsigned n0 = __ballot_sync(0xffffffffu, k0v <= thr);
-                const unsigned n1 = __ballot_sync(0xffffffffu, k1v <= thr);
-                if (fabsf(rmin) < INFINITY && __popc(n0) + __popc(n1) == 1) {
-                    g = s_cand[par][n0 ? __ffs(n0) - 1 : 32 + __ffs(n1) - 1];
-                } else {
-                    g.a = 1.0; g.q = 0.0; g.org = 0x7fffffff; g.pos = -1;
-                    for (int e = lane; e < CS * NW; e += 32) merge_cand(g, s_cand[par][e]);
-                    g = warp_best(g);
+        if (lane == 0) { s_warp[par][warp].c = best; s_wkey[par][warp] = wmin; }
+        __syncthreads();
+        // ---- the pick: made by every warp for itself
+        Cand g;
+        int which;
+        if (MULTI) {
+            if (warp == 0) {
+                // the CTA's own offer, pushed to every CTA with its pending entries
+                const Cand own = pick_offer(s_warp[par], s_wkey[par], NW, lane, &which);
+                const float key = s_wkey[par][which];
+                const int pl = own.pos >= 0 ? own.pos - rank * S : 0;
+                float2 uz = make_float2(0.f, 0.f);
+                if (lane < m) uz = make_float2(sU[(size_t)lane * Sp + pl], sZ[(size_t)lane * Sp + pl]);
+                for (int c = 0; c < CS; ++c) {
+                    float2* to = cluster.map_shared_rank(&s_pend[par][rank][0], c);
+                    to[lane] = uz;
+                }
+                if (lane < CS) {
+                    cluster.map_shared_rank(&s_cta[par][rank], lane)->c = own;
+                    *cluster.map_shared_rank(&s_ckey[par][rank], lane) = key;
                 }
             }
-            int p = g.pos;
-            if (p < 0) p = 0;
-            double h = g.a;
-            int bad = 0;
-            if (!isfinite(g.q) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
-            else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
-            const double rs = rsqrt(h);
-            const int prow = p / S, pl = p - prow * S;
-            float up = 0.f, zp = 0.f;
-            if (lane < m) {
-                up = *cluster.map_shared_rank(sU + (size_t)lane * S + pl, prow);
-                zp = *cluster.map_shared_rank(sZ + (size_t)lane * S + pl, prow);
-            }
-            sUp[lane] = up;
-            sZp[lane] = zp;
-            sT[m][lane] = up;
+            cluster.sync();
+            g = pick_offer(s_cta[par], s_ckey[par], CS, lane, &which);
+        } else {
+            g = pick_offer(s_warp[par], s_wkey[par], NW, lane, &which);
+        }
+        const int p = g.pos < 0 ? 0 : g.pos;
+        // both triangles of H^-1 and Q are kept, so the pivot column is the contiguous row p
+        float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), q4 = a4;
+        if (owner_thread) {
+            a4 = *reinterpret_cast<const float4*>(Al + (size_t)p * d + k0);
+            q4 = *reinterpret_cast<const float4*>(Ql + (size_t)p * d + k0);
+        }
+        double h = g.a;
+        int bad = 0;
+        if (!isfinite(g.q) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
+        else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
+        const double rs = rsqrt(h), half = 0.5 * g.q * rs * rs;
+        // pending entries at the pivot: pushed by its owner, or in this CTA's own slice
+        const float2* pend = s_pend[par][which];
+        const float *pu = sU + p, *pz = sZ + p;
+        if (warp == NW - 1) {                     // (the last warp: the others may own more positions)
+            sT[m][lane] = lane < m ? (MULTI ? pend[lane].x : pu[(size_t)lane * Sp]) : 0.f;
             if (lane == 0) {
-                s_p = p;
-                s_rs = rs;
-                s_half = 0.5 * g.q * rs * rs;
                 s_pm[m] = p;
                 s_rsm[m] = rs;
                 if (rank == 0) {
@@ -336,25 +370,21 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
                 }
             }
         }
-        __syncthreads();
-        const int p = s_p;
-        const double rs = s_rs, half = s_half;
         // ---- true pivot columns of H^-1 and Q on the owned positions; float64 diagonal downdate
         if (owner_thread) {
-            // both triangles of H^-1 and Q are kept, so the pivot column is the contiguous row p
-            const float4 a4 = *reinterpret_cast<const float4*>(Al + (size_t)p * d + k0);
-            const float4 q4 = *reinterpret_cast<const float4*>(Ql + (size_t)p * d + k0);
-            float a[4] = {a4.x, a4.y, a4.z, a4.w}, q[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (!alive[e] || k0 + e == p) { a[e] = 0.f; q[e] = 0.f; }
             // pending terms at the pivot, summed while the gathered entries are still in flight
             float ca[4] = {0.f, 0.f, 0.f, 0.f}, cq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
             for (int s = 0; s < m; ++s) {
-                const float4 u4 = *reinterpret_cast<const float4*>(sU + (size_t)s * S + kloc);
-                const float4 z4 = *reinterpret_cast<const float4*>(sZ + (size_t)s * S + kloc);
-                const float up = sUp[s], zp = sZp[s];
+                const float4 u4 = *reinterpret_cast<const float4*>(sU + (size_t)s * Sp + kloc);
+                const float4 z4 = *reinterpret_cast<const float4*>(sZ + (size_t)s * Sp + kloc);
+                float up, zp;
+                if (MULTI) {
+                    const float2 uz = pend[s];
+                    up = uz.x; zp = uz.y;
+                } else {
+                    up = pu[(size_t)s * Sp]; zp = pz[(size_t)s * Sp];
+                }
                 const float uu[4] = {u4.x, u4.y, u4.z, u4.w}, zz[4] = {z4.x, z4.y, z4.z, z4.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -363,33 +393,31 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
                     cq[e] = fmaf(uu[e], zp, cq[e]);
                 }
             }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { a[e] -= ca[e]; q[e] -= cq[e]; }
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, q[4] = {q4.x, q4.y, q4.z, q4.w};
             float u32[4], z32[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int k = k0 + e;
-                u32[e] = 0.f; z32[e] = 0.f;
-                if (alive[e] && k != p) {
-                    const double u = (double)a[e] * rs;
-                    const double z = (double)q[e] * rs - half * u;
-                    da[e] -= u * u;
-                    dq[e] -= 2.0 * z * u;
-                    u32[e] = (float)u;
-                    z32[e] = (float)z;
-                }
-                if (k == p) alive[e] = false;
+                // removed positions and the pivot itself: zero, which leaves the diagonals as they are
+                alive[e] = alive[e] && k0 + e != p;
+                const float ae = alive[e] ? a[e] - ca[e] : 0.f, qe = alive[e] ? q[e] - cq[e] : 0.f;
+                const double u = (double)ae * rs;
+                const double z = (double)qe * rs - half * u;
+                da[e] -= u * u;
+                dq[e] -= 2.0 * z * u;
+                u32[e] = alive[e] ? (float)u : 0.f;
+                z32[e] = alive[e] ? (float)z : 0.f;
             }
             const float4 uo = make_float4(u32[0], u32[1], u32[2], u32[3]);
             const float4 zo = make_float4(z32[0], z32[1], z32[2], z32[3]);
-            *reinterpret_cast<float4*>(sU + (size_t)m * S + kloc) = uo;
-            *reinterpret_cast<float4*>(sZ + (size_t)m * S + kloc) = zo;
+            *reinterpret_cast<float4*>(sU + (size_t)m * Sp + kloc) = uo;
+            *reinterpret_cast<float4*>(sZ + (size_t)m * Sp + kloc) = zo;
             *reinterpret_cast<float4*>(Ul + (size_t)m * d + k0) = uo;
             *reinterpret_cast<float4*>(Zl + (size_t)m * d + k0) = zo;
         }
-        // no barrier here: the next step's cluster barrier orders these writes before any read
+        // no barrier here: the next step's barrier orders these writes before any read
     }
-    cluster.sync();
+    if (MULTI) cluster.sync();
+    else __syncthreads();
 
     // ---- c_m = (W[:,p_m] - sum_{s<m} c_s T[m][s]) / sqrt(h_m): forward substitution per row
     //      index i of W, each CTA takes a slice of the d_row indices.  The triangle is widened to
@@ -434,11 +462,10 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
                 idx_out[(size_t)l * d + k] = alive[e] ? org[e] : -1;
             }
         }
-        if (rank == 0 && tid == 0) {
+        if (rank == 0 && warp == NW - 1 && lane == 0) {
             state[l].sumrho += sumrho;
             state[l].n_new = n0;
         }
-        cluster.sync();      // no CTA may retire while another can still read its shared memory
         solve_c();
         return;
     }
@@ -457,9 +484,11 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
         for (int w2 = 0; w2 < NW; ++w2) { const int v = s_wsum[w2]; s_wsum[w2] = t; t += v; }
         s_count = t;
     }
-    cluster.sync();
+    if (MULTI) cluster.sync();
+    else __syncthreads();
     int base = 0;
-    for (int c2 = 0; c2 < rank; ++c2) base += *cluster.map_shared_rank(&s_count, c2);
+    if (MULTI)
+        for (int c2 = 0; c2 < rank; ++c2) base += *cluster.map_shared_rank(&s_count, c2);
     int np = base + s_wsum[warp] + incl - mine;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -471,9 +500,9 @@ k_lazy_steps(int n0, int S, int t0, int nsteps, int compact, int d, int G, int r
             ++np;
         }
     }
-    if (rank == 0 && tid == 0) state[l].sumrho += sumrho;
+    if (rank == 0 && warp == NW - 1 && lane == 0) state[l].sumrho += sumrho;
     if (rank == CS - 1 && tid == 0) state[l].n_new = base + s_count;
-    cluster.sync();      // no CTA may retire while another can still read its shared memory
+    if (MULTI) cluster.sync();      // no CTA may retire while another can still read its shared memory
     solve_c();
 }
 
@@ -977,6 +1006,14 @@ LazyWs carve_lazy(void* ws, int L, int r, int d) {
 
 }  // namespace
 
+// Pitch of the pending vectors in the steps kernel: four more than a multiple of 32, so that the entries at
+// one position (one per pending step) lie in eight different banks instead of one.
+static int steps_pitch(int S) { return round_up_int(S, 32) + 4; }
+static int steps_smem(int S) {
+    const int b = 2 * BMAX * steps_pitch(S) * (int)sizeof(float), t = BMAX * BMAX * (int)sizeof(double);
+    return b > t ? b : t;
+}
+
 bool lazy_path_supported(int d) { return d >= 1 && d <= CLUSTER_MAX * SLICE_MAX; }
 
 size_t lazy_workspace_bytes(int L, int r, int d, int n_levels) {
@@ -1025,8 +1062,10 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     s = init();
     if (s != ZIPLM_OK) return s;
 
-    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_steps, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          2 * BMAX * SLICE_MAX * (int)sizeof(float)));
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_steps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          steps_smem(SLICE_MAX)));
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_steps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          steps_smem(SLICE_MAX)));
     int cur = 0;
     auto snapshot = [&](int n, int slot) -> ziplm_status {
         PhaseScope ps(PH_SNAPSHOT, st);
@@ -1086,7 +1125,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(L * cs);
             cfg.blockDim = dim3(STEP_THREADS);
-            cfg.dynamicSmemBytes = (size_t)2 * BMAX * S * sizeof(float);
+            cfg.dynamicSmemBytes = (size_t)steps_smem(S);
             cfg.stream = st;
             cudaLaunchAttribute attr[2];
             attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1101,7 +1140,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(
-                &cfg, k_lazy_steps, npos, S, t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
+                &cfg, cs > 1 ? k_lazy_steps<true> : k_lazy_steps<false>, npos, S, steps_pitch(S), t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
                 (const float*)w.Q[cur], (const float*)w.Wt[cur], (const double*)w.dA[cur],
                 (const double*)w.dQ[cur], (const int*)w.idx[cur], w.dA[nxt], w.dQ[nxt], w.idx[nxt],
                 w.src, w.U, w.Z, w.C, w.state, order, saliency, layer_status));
