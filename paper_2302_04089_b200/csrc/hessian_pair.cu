@@ -54,25 +54,11 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Arrive at a barrier of the pair's other CTA (or of this one), by its shared::cluster address.
+// Arrive at a barrier of the pair's other CTA (or of this one), by its shared::cluster address.  The
+// barriers here order accesses of the asynchronous proxy and of tensor memory only, so arrivals and waits
+// keep the default scope: cluster scope would fence generic memory at every one of them.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
-}
-// Wait whose phase another CTA of the cluster may complete.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                                  uint32_t limit) {
-    const long long t0 = clock64();
-    for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
-        if ((it & 63u) == 63u && (*abort_flag || clock64() - t0 > kSpinClocks)) return false;
-    }
-    return false;
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // TMA load into this CTA's shared memory, counted on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
@@ -153,16 +139,15 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
             // ---------------- TMA producer (each CTA its own half of the operands)
             const uint32_t bytes = (uint32_t)((diag ? 1 : 2) * C::PARTS * OP_BYTES);
             const int ya = i0 + (int)rank * HALF, yb = j0 + (int)rank * HALF;
+            const uint32_t full0 = cluster_addr(smem_u32(&bar_full[0]), 0);
+            int s = 0;
+            uint32_t ph = 1u;
             for (int kb = 0; kb < num_kb; ++kb) {
-                const int s = kb % C::STAGES;
-                const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
-                if (empty_spin_limit < kSpinLimit
-                        ? !mbar_wait_limit(smem_u32(&bar_empty[s]), ph ^ 1u, abortp, empty_spin_limit)
-                        : !mbar_wait_cluster(smem_u32(&bar_empty[s]), ph ^ 1u, abortp, kSpinLimit)) {
+                if (!mbar_wait_limit(smem_u32(&bar_empty[s]), ph, abortp, empty_spin_limit)) {
                     failed = true;
                     break;
                 }
-                const uint32_t full = cluster_addr(smem_u32(&bar_full[s]), 0);
+                const uint32_t full = full0 + 8u * (uint32_t)s;
                 const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
                 if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2 * bytes);
                 const int x = kb * BK;
@@ -173,48 +158,48 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                     if (SPLIT) tma_load_3d_pair(base + 3 * OP_BYTES, &map_lo, full, x, yb, l);
                 }
                 issued = kb + 1;
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
             }
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
             // ---------------- MMA issuer (the leader, for both CTAs)
             const uint32_t idesc = make_idesc(SPLIT ? 0u : fmt16, PT, PT);
-            int kb = 0;
+            // One thread issues every MMA of the pair, 128 clocks of tensor-core time each, so the code
+            // between two MMAs has to be short: stage and phase are counted, descriptors are one addition.
+            const uint64_t desc0 = make_desc(tiles);
+            const uint32_t b_off = diag ? 0u : (uint32_t)(C::PARTS * OP_BYTES / 16);
+            int s = 0, kb = 0;
+            uint32_t ph = 0u;
             for (int c = 0; c < num_chunks && !failed; ++c) {
                 const int b = c & 1;
                 const uint32_t acc = tmem_base + (uint32_t)b * PT;
                 // both CTAs must have drained this buffer (first use of each buffer passes)
-                if (!mbar_wait_cluster(smem_u32(&bar_acc_empty[b]), (((uint32_t)c >> 1) & 1u) ^ 1u, abortp,
-                                       kSpinLimit)) {
+                if (!mbar_wait(smem_u32(&bar_acc_empty[b]), (((uint32_t)c >> 1) & 1u) ^ 1u, abortp)) {
                     failed = true;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int kb_end = (kb + C::CHUNK < num_kb) ? kb + C::CHUNK : num_kb;
-                uint32_t add = 0u;
-                for (; kb < kb_end; ++kb) {
-                    const int s = kb % C::STAGES;
-                    const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
-                    if (!mbar_wait_cluster(smem_u32(&bar_full[s]), ph, abortp, kSpinLimit)) { failed = true; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
-                    const uint64_t a_hi = make_desc(base), a_lo = make_desc(base + OP_BYTES);
-                    const uint64_t b_hi = diag ? a_hi : make_desc(base + C::PARTS * OP_BYTES);
-                    const uint64_t b_lo = diag ? a_lo : make_desc(base + 3 * OP_BYTES);
-                    if (SPLIT) {
 #pragma unroll
-                        for (int k = 0; k < BK / 16; ++k) {
-                            umma_pair(acc, a_hi + 2u * k, b_lo + 2u * k, idesc, add);
-                            add = 1u;
+                for (int j = 0; j < C::CHUNK; ++j) {
+                    if (j > 0 && kb >= num_kb) break;
+                    if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { failed = true; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t a_hi = desc0 + (uint32_t)(s * (kStageBytes<SPLIT> / 16)), b_hi = a_hi + b_off;
+                    if (SPLIT) {
+                        const uint64_t a_lo = a_hi + OP_BYTES / 16, b_lo = b_hi + OP_BYTES / 16;
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k) {       // 32 bytes per MMA along K
+                            umma_pair(acc, a_hi + 2u * k, b_lo + 2u * k, idesc, k > 0 || j > 0);
                             umma_pair(acc, a_lo + 2u * k, b_hi + 2u * k, idesc, 1u);
                         }
                     }
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {       // 32 bytes per MMA along K
-                        umma_pair(acc, a_hi + 2u * k, b_hi + 2u * k, idesc, add);
-                        add = 1u;
-                    }
+                    for (int k = 0; k < BK / 16; ++k)
+                        umma_pair(acc, a_hi + 2u * k, b_hi + 2u * k, idesc, SPLIT || k > 0 || j > 0);
                     umma_commit_pair(smem_u32(&bar_empty[s]));     // stage free once these MMAs have read it
+                    ++kb;
+                    if (++s == C::STAGES) { s = 0; ph ^= 1u; }
                 }
                 if (!failed) umma_commit_pair(smem_u32(&bar_acc_full[b]));
             }
@@ -236,8 +221,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
         bool folded = false;
         for (int c = 0; c < num_chunks; ++c) {
             const int b = c & 1;
-            if (!mbar_wait_cluster(smem_u32(&bar_acc_full[b]), ((uint32_t)c >> 1) & 1u, abortp, kSpinLimit))
-                failed = true;
+            if (!mbar_wait(smem_u32(&bar_acc_full[b]), ((uint32_t)c >> 1) & 1u, abortp)) failed = true;
             failed = __any_sync(0xffffffffu, failed);
             if (failed) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -113,10 +113,10 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
         if (lane == 0) {
             // ---------------- TMA producer
             const uint32_t bytes = (uint32_t)((diag ? C::TILES / 2 : C::TILES) * TILE_BYTES);
+            int s = 0;
+            uint32_t ph = 1u;
             for (int kb = 0; kb < num_kb; ++kb) {
-                const int s = kb % C::STAGES;
-                const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
-                if (!mbar_wait_limit(smem_u32(&bar_empty[s]), ph ^ 1u, abortp, empty_spin_limit)) {
+                if (!mbar_wait_limit(smem_u32(&bar_empty[s]), ph, abortp, empty_spin_limit)) {
                     failed = true;
                     break;
                 }
@@ -131,6 +131,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                     if (!diag) tma_load_3d(base + 3 * TILE_BYTES, &map_lo, full, x, j0, l);
                 }
                 issued = kb + 1;
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
             }
         }
     } else if (warp == 1) {
@@ -139,7 +140,8 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
             // operand format of the instruction: 1 = BF16, 0 = F16 (A and B alike; the split is fp16)
             const uint32_t idesc = make_idesc(TF32 ? 0u : fmt16, TM, TM);
             const uint32_t tmem_cross = tmem_base + 256u;
-            int kb = 0;
+            int kb = 0, s = 0;
+            uint32_t ph = 0u;
             for (int c = 0; c < num_chunks && !failed; ++c) {
                 const int b = c & 1;
                 const uint32_t tmem_main = tmem_base + (uint32_t)b * 128u;
@@ -152,8 +154,6 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                 const int kb_end = (kb + CHUNK < num_kb) ? kb + CHUNK : num_kb;
                 const int kb_first = kb;
                 for (; kb < kb_end; ++kb) {
-                    const int s = kb % C::STAGES;
-                    const uint32_t ph = (uint32_t)(kb / C::STAGES) & 1u;
                     if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { failed = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t base = tiles + (uint32_t)s * STAGE_BYTES;
@@ -174,6 +174,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                         }
                     }
                     umma_commit(smem_u32(&bar_empty[s]));     // stage free once these MMAs have read it
+                    if (++s == C::STAGES) { s = 0; ph ^= 1u; }
                 }
                 if (!failed) umma_commit(smem_u32(&bar_acc_full[b]));   // chunk (and all before) done
             }
