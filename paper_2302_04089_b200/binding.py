@@ -168,7 +168,7 @@ def hessian_accumulate(X: torch.Tensor, H: Optional[torch.Tensor] = None, alpha:
     ldx = X.stride(1) if N > 0 else max(N, 1)
     dt = _DTYPES[X.dtype]
     if H is None:
-        H = torch.zeros(L, d, d, dtype=torch.float32, device=X.device)
+        H = torch.empty(L, d, d, dtype=torch.float32, device=X.device)      # beta = 0 writes every entry
         beta = 0.0
     _check(H, torch.float32, "H")
     need = hessian_workspace_bytes(L, d, N, dt)
@@ -198,7 +198,7 @@ def hessian_accumulate_tokens(A: torch.Tensor, H: Optional[torch.Tensor] = None,
         raise ValueError("layers of A must be evenly pitched")
     dt = _DTYPES[A.dtype]
     if H is None:
-        H = torch.zeros(L, d, d, dtype=torch.float32, device=A.device)
+        H = torch.empty(L, d, d, dtype=torch.float32, device=A.device)      # beta = 0 writes every entry
         beta = 0.0
     _check(H, torch.float32, "H")
     need = hessian_tokens_workspace_bytes(L, d, N, dt)

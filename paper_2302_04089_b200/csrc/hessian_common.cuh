@@ -20,7 +20,7 @@ struct HessianProduct {
     bool split;
 };
 
-// The pair kernel takes a launch when its tiles of 256 x 256 fill the CTA pairs of the chip.
+// Whether the kernel on CTA pairs takes a launch of that many layers.
 bool hessian_pair_fits(int layers, int d);
 size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split);
 ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st);

@@ -338,7 +338,13 @@ ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t s
 
 }  // namespace
 
-bool hessian_pair_fits(int layers, int d) { return (long long)layers * pair_count(d) >= 74; }
+// A K block of a 256 x 256 tile takes a pair about 4/3 of the time that one of a 128 x 128 tile takes a CTA
+// (12 MMAs of 128 clocks against 12 of 92, where the shared-memory reads of a 128 x 128 MMA bound it), so
+// the pair kernel wins where it needs fewer than three quarters of the waves.
+bool hessian_pair_fits(int layers, int d) {
+    const long long T = (d + HALF - 1) / HALF, tiles = T * (T + 1) / 2 * layers, pairs = (long long)pair_count(d) * layers;
+    return 4 * ((pairs + 73) / 74) < 3 * ((tiles + 147) / 148);
+}
 
 // Scratch of the second summation level, for the layers of one launch; none where FOLD drains are
 // never reached.

@@ -25,6 +25,7 @@
 // the producer for the copies it has started, and the CTA leaves through the normal exit (TMEM
 // freed), so a lost copy can never hang the GPU.  A small kernel after the product launches turns
 // a raised error word into NaN in H[l][0][0] of every layer.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -32,6 +33,8 @@
 #include "common.cuh"
 #include "hessian_common.cuh"
 #include "tc_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ziplm {
 namespace {
@@ -57,11 +60,12 @@ constexpr int CHUNK = 2;
 constexpr int FOLD = 32;
 constexpr int EPI_WARPS = 8;                  // two warps per TMEM lane quarter, 64 columns each
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
+constexpr int OUT_PITCH = TM + 1;             // floats of a row of the finished tile in shared memory
 
 template <bool TF32>
 __global__ void __launch_bounds__(THREADS, 1)
 k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-          float* __restrict__ H, int d, int num_kb, float alpha, float beta, int layer0,
+          float* __restrict__ H, int d, int num_kb_all, int n_split, float alpha, float beta, int layer0,
           int* __restrict__ err_word, uint32_t fmt16, uint32_t empty_spin_limit,
           const unsigned* __restrict__ amax) {
     using C = Cfg<TF32>;
@@ -76,7 +80,11 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     const uint32_t tiles = (raw + 1023u) & ~1023u;       // swizzled tiles need 1024-byte alignment
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int l = blockIdx.y;                             // layer within the launched chunk
-    int ti = 0, rem = blockIdx.x;
+    // a cluster of n_split CTAs shares a tile, each a range of its K blocks
+    const int rank = (int)blockIdx.x % n_split;
+    const int kb_begin = (int)((long long)num_kb_all * rank / n_split);
+    const int num_kb = (int)((long long)num_kb_all * (rank + 1) / n_split) - kb_begin;
+    int ti = 0, rem = (int)blockIdx.x / n_split;
     while (rem > ti) { rem -= ti + 1; ++ti; }
     const int tj = rem;
     const int i0 = ti * TM, j0 = tj * TM;
@@ -106,6 +114,8 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_slot;            // main[0] = +0, main[1] = +128, cross = +256
     volatile int* abortp = &abort_flag;
+    float* out_tile = reinterpret_cast<float*>(smem_raw + (tiles - raw));    // [TM][OUT_PITCH], over the ring
+    float* mirror = n_split > 1 ? out_tile + TM * OUT_PITCH : out_tile;      // finished rows of this CTA
     bool failed = false;
     int issued = 0;                                       // K blocks whose copies were started (thread 0)
 
@@ -123,7 +133,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                 const uint32_t full = smem_u32(&bar_full[s]);
                 const uint32_t base = tiles + (uint32_t)s * STAGE_BYTES;
                 mbar_expect_tx(full, bytes);
-                const int x = kb * C::BK;
+                const int x = (kb_begin + kb) * C::BK;
                 tma_load_3d(base, &map_hi, full, x, i0, l);
                 if (!diag) tma_load_3d(base + TILE_BYTES, &map_hi, full, x, j0, l);
                 if (TF32) {
@@ -224,22 +234,10 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                     for (int e = 0; e < 32; ++e) acc[cc * 32 + e] += __uint_as_float(v[e]);
                 }
             }
-            float* Hl = H + (size_t)(layer0 + l) * d * d;
-            const int row = i0 + q * 32 + lane;
-            // split route: undo the power-of-two scales of the two feature rows (exact)
-            const unsigned* am = TF32 ? amax + (size_t)l * d : nullptr;
-            const float inv_row = (TF32 && row < d) ? row_scale(am[row], true) : 1.f;
+            // The operand ring is free (every MMA has completed): the partial tile goes there.
+            const int row = q * 32 + lane;
 #pragma unroll
-            for (int e = 0; e < NC; ++e) {
-                const int col = j0 + half * NC + e;
-                float val = alpha * (tot[e] + acc[e]);
-                if (TF32 && col < d) val = (val * inv_row) * row_scale(am[col], true);
-                if (row < d && col < d && col <= row) {
-                    if (beta != 0.f) val += Hl[(size_t)row * d + col];
-                    Hl[(size_t)row * d + col] = val;
-                    if (col != row) Hl[(size_t)col * d + row] = val;
-                }
-            }
+            for (int e = 0; e < NC; ++e) out_tile[row * OUT_PITCH + half * NC + e] = tot[e] + acc[e];
         }
     }
 
@@ -249,18 +247,55 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (abort_flag) {
+    if (threadIdx.x == 0 && abort_flag) {
         // Copies that were started land in this CTA's shared memory: wait for them (bounded) before
         // the CTA retires.  The last STAGES K blocks started are the latest phases of their barriers.
-        if (threadIdx.x == 0)
-            for (int kb = issued > C::STAGES ? issued - C::STAGES : 0; kb < issued; ++kb)
-                mbar_wait_quiet(smem_u32(&bar_full[kb % C::STAGES]), (uint32_t)(kb / C::STAGES) & 1u);
-        __syncthreads();
+        for (int kb = issued > C::STAGES ? issued - C::STAGES : 0; kb < issued; ++kb)
+            mbar_wait_quiet(smem_u32(&bar_full[kb % C::STAGES]), (uint32_t)(kb / C::STAGES) & 1u);
     }
+    __syncwarp();
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
                      : "memory");
     }
+    cg::cluster_group cluster = cg::this_cluster();
+    if (n_split > 1) cluster.sync();
+
+    // Every CTA of the cluster finishes its share of the rows: sums over the CTAs in rank order,
+    // rows [i][j] written along j, mirrored rows [j][i] along i.
+    const int n_rows = TM / n_split, first = rank * n_rows;
+    float* Hl = H + (size_t)(layer0 + l) * d * d;
+    const unsigned* am = TF32 ? amax + (size_t)l * d : nullptr;
+    for (int rr = first + warp; rr < first + n_rows; rr += THREADS / 32) {
+        const int row = i0 + rr;
+        if (row >= d) break;
+        // split route: undo the power-of-two scales of the two feature rows (exact)
+        const float inv_row = TF32 ? row_scale(am[row], true) : 1.f;
+#pragma unroll
+        for (int h = 0; h < TM / 32; ++h) {
+            const int cc = 32 * h + lane, col = j0 + cc;
+            float v = 0.f;
+            if (n_split == 1) v = out_tile[rr * OUT_PITCH + cc];
+            else
+                for (int s = 0; s < n_split; ++s) v += cluster.map_shared_rank(out_tile, s)[rr * OUT_PITCH + cc];
+            if (col > row) continue;                         // (col <= row < d)
+            v *= alpha;
+            if (TF32) v = (v * inv_row) * row_scale(am[col], true);
+            float* p = Hl + (size_t)row * d + col;
+            if (beta != 0.f) v += *p;
+            *p = v;
+            mirror[(rr - first) * OUT_PITCH + cc] = v;
+        }
+    }
+    __syncthreads();
+    // lanes along the rows of this share (32, or all of them where there are fewer), then along columns
+    const int lanes = n_rows < 32 ? n_rows : 32, per = 32 / lanes;
+    for (int c = warp * per + lane / lanes; c < TM; c += (THREADS / 32) * per)
+        for (int rr = lane % lanes; rr < n_rows; rr += lanes) {
+            const int row = i0 + first + rr, col = j0 + c;
+            if (row < d && col < row) Hl[(size_t)col * d + row] = mirror[rr * OUT_PITCH + c];
+        }
+    if (n_split > 1) cluster.sync();                         // no CTA retires while others read its tile
 }
 
 // A product kernel that gave up on a wait leaves ZIPLM_ERR_TIMEOUT in the error word; the layers'
@@ -485,6 +520,108 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
     }
 }
 
+// Both pre-passes of token-major fp32 batches in one: a cluster of up to eight CTAs takes 64 features of
+// all N tokens, each CTA a range of tokens that it keeps in shared memory; the features' largest magnitudes
+// meet through distributed shared memory, and the scaled fp16 parts leave K-major.  A is read once instead
+// of twice and nothing has to be zeroed beforehand (a batch of 12 x 2048 x 3072: 0.45 -> TIME_HERE ms; for
+// a small one it is one launch instead of three).  VEC: rows of A start on 16 bytes.
+constexpr int TS_FEATURES = 64, TS_PITCH = TS_FEATURES + 1;
+constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 195 KiB of shared memory
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ A, long long lda, int N, int d,
+                                                      long long np, int tokens, unsigned* __restrict__ amax,
+                                                      __half* __restrict__ hi, __half* __restrict__ lo) {
+    extern __shared__ float ts_tile[];           // [tokens][TS_PITCH]
+    __shared__ unsigned s_max[TS_FEATURES];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int l = blockIdx.z, f0 = blockIdx.y * TS_FEATURES;
+    const int t0 = rank * tokens, t1 = min(N, t0 + tokens);
+    const int tid = threadIdx.x, q = tid & 15, rr = tid >> 4;
+    const float* Al = A + (size_t)l * (size_t)N * (size_t)lda;
+    if (tid < TS_FEATURES) s_max[tid] = 0u;
+    __syncthreads();
+    unsigned m[4] = {0u, 0u, 0u, 0u};
+    const int f = f0 + 4 * q;
+    const bool whole = VEC && f + 3 < d;
+    for (int t = t0 + rr; t < t1; t += 64) {
+        float v[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int tk = t + 16 * k;
+            v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0.f;
+            if (tk >= t1) continue;
+            const float* src = Al + (size_t)tk * (size_t)lda + f;
+            if (whole) {
+                const float4 x = __ldcs(reinterpret_cast<const float4*>(src));
+                v[k][0] = x.x; v[k][1] = x.y; v[k][2] = x.z; v[k][3] = x.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) if (f + e < d) v[k][e] = src[e];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                m[e] = max(m[e], __float_as_uint(v[k][e]) & 0x7fffffffu);
+                if (t + 16 * k < t1) ts_tile[(t + 16 * k - t0) * TS_PITCH + 4 * q + e] = v[k][e];
+            }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) atomicMax(&s_max[4 * q + e], m[e]);
+    if (CS > 1) cluster.sync();
+    else __syncthreads();
+    // pairs of tokens along the lanes, a feature per warp and turn
+    const int lane = tid & 31, warp = tid >> 5;
+    const int p1 = (int)min(np, (long long)(t0 + tokens));       // the last range also writes the padding
+    for (int fl = warp; fl < TS_FEATURES; fl += 8) {
+        if (f0 + fl >= d) break;
+        unsigned mx = lane < CS ? cluster.map_shared_rank(s_max, lane)[fl] : 0u;
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (rank == 0 && lane == 0) amax[(size_t)l * d + f0 + fl] = mx;
+        const float sc = row_scale(mx, false);
+        const size_t row = ((size_t)l * d + f0 + fl) * (size_t)np;
+        for (int t = t0 + 2 * lane; t < p1; t += 64) {
+            const float x0 = t < t1 ? ts_tile[(t - t0) * TS_PITCH + fl] : 0.f;
+            const float x1 = t + 1 < t1 ? ts_tile[(t + 1 - t0) * TS_PITCH + fl] : 0.f;
+            __half2 h, w;
+            split_f16x2(x0 * sc, h.x, w.x);
+            split_f16x2(x1 * sc, h.y, w.y);
+            *reinterpret_cast<__half2*>(hi + row + t) = h;
+            *reinterpret_cast<__half2*>(lo + row + t) = w;
+        }
+    }
+    if (CS > 1) cluster.sync();                  // the magnitudes stay readable until all have them
+}
+
+// Launch of k_tokens_split: ranges of about 256 tokens (a multiple of 8), more per CTA where eight of them
+// do not reach.
+ziplm_status run_tokens_split(const float* A, long long lda, int N, int d, long long np, int layers,
+                              unsigned* amax, __half* hi, __half* lo, cudaStream_t st) {
+    int cs = 1;
+    while (cs < 8 && cs * 256 < N) cs *= 2;
+    const int tokens = round_up_int((int)((np + cs - 1) / cs), 8);
+    const bool vec = (reinterpret_cast<uintptr_t>(A) % 16) == 0 && lda % 4 == 0;
+    auto kernel = vec ? k_tokens_split<true> : k_tokens_split<false>;
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          TS_TOKENS * TS_PITCH * (int)sizeof(float)));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs, (d + TS_FEATURES - 1) / TS_FEATURES, layers);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = (size_t)tokens * TS_PITCH * sizeof(float);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, A, lda, N, d, np, tokens, amax, hi, lo));
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
 bool quad_rows(const void* A, long long lda, size_t esz) {
     return (reinterpret_cast<uintptr_t>(A) % (4 * esz)) == 0 && lda % 4 == 0;
 }
@@ -555,22 +692,34 @@ size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, boo
 
 namespace {
 
-// One product launch on the kernel that suits its number of tiles.
+// One product launch on the kernel that suits its number of tiles.  Where the 128 x 128 tiles leave half of
+// the SMs idle, up to eight CTAs share a tile: the largest power of two with which all fit and each keeps
+// four K blocks (one layer of 256 features, 2048 tokens: three tiles, a chain of 32 K blocks on one CTA).
 ziplm_status run_product(const HessianProduct& p, void* scratch, cudaStream_t st) {
     if (hessian_pair_fits(p.layers, p.d)) return run_hessian_pair(p, scratch, st);
     const int T = (p.d + TM - 1) / TM;
-    const dim3 grid(T * (T + 1) / 2, p.layers);
-    if (p.split) {
-        constexpr int smem = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
-        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        k_syrk_tc<true><<<grid, THREADS, smem, st>>>(p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0,
-                                                     p.err_word, 0u, p.spin, p.amax);
-    } else {
-        constexpr int smem = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
-        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        k_syrk_tc<false><<<grid, THREADS, smem, st>>>(p.hi, p.hi, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0,
-                                                      p.err_word, p.fmt16, p.spin, nullptr);
-    }
+    const long long tiles = (long long)T * (T + 1) / 2 * p.layers;
+    int split = 1;
+    while (split < 8 && tiles * split * 2 <= 148 && p.num_kb / (split * 2) >= 4) split *= 2;
+    constexpr int smem2 = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
+    constexpr int smem1 = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
+    static_assert(2 * TM * OUT_PITCH * (int)sizeof(float) + 1024 <= smem1, "finished tiles fit the operand ring");
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(T * (T + 1) / 2 * split, p.layers);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = p.split ? smem2 : smem1;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = split;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, p.split ? k_syrk_tc<true> : k_syrk_tc<false>, p.hi,
+                                        p.split ? p.lo : p.hi, p.H, p.d, p.num_kb, split, p.alpha, p.beta,
+                                        p.layer0, p.err_word, p.fmt16, p.spin, p.amax));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }
@@ -611,12 +760,20 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
             const size_t rows = (size_t)ln * d;
             if (token_major) {
                 const float* Ac = static_cast<const float*>(X) + (size_t)l0 * (size_t)N * ldx;
-                ZIPLM_CHECK_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned) * rows, st));
+                const bool one_pass = np <= 8ll * TS_TOKENS;
+                if (!one_pass) ZIPLM_CHECK_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned) * rows, st));
                 // slabs of at least 256 tokens, at most 65535 of them (grid.y)
                 const long long slab = N / 65535 + 1 > 256 ? N / 65535 + 1 : 256;
                 // grid.z is limited to 65535 layers per launch
                 for (int z0 = 0; z0 < ln; z0 += 65535) {
                     const int zn = ln - z0 < 65535 ? ln - z0 : 65535;
+                    if (one_pass) {
+                        const ziplm_status s = run_tokens_split(Ac + (size_t)z0 * N * ldx, ldx, (int)N, d, np, zn,
+                                                                amax + (size_t)z0 * d, hi + (size_t)z0 * d * np,
+                                                                lo + (size_t)z0 * d * np, st);
+                        if (s != ZIPLM_OK) return s;
+                        continue;
+                    }
                     k_tokens_absmax<<<dim3((unsigned)((d + 255) / 256), (unsigned)((N + slab - 1) / slab),
                                            (unsigned)zn), 256, 0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, slab,
                                                                         amax + (size_t)z0 * d);

@@ -770,7 +770,7 @@ def test_delayed_path_widths_that_are_no_multiple_of_four(d, r, levels):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
-@pytest.mark.parametrize("d,N,L", [(900, 40, 8), (257, 4500, 25), (1030, 2112, 5)])
+@pytest.mark.parametrize("d,N,L", [(900, 40, 7), (513, 4500, 12), (1030, 2112, 4)])
 def test_hessian_on_cta_pairs_matches_oracle(dtype, d, N, L):
     """Enough 256 x 256 tiles for the pair kernel: one K block, ragged edges of tiles and of the last
     K block, more drains than the first summation level takes; then once more on top (beta = 1)."""
@@ -792,7 +792,7 @@ def test_hessian_on_cta_pairs_matches_oracle(dtype, d, N, L):
 def test_a_bounded_wait_of_the_pair_kernel_that_runs_out_is_reported():
     """As above for the kernel on CTA pairs: both producers give up after one look."""
     z = zb()
-    Xd = torch.randn(25, 300, 1024, generator=torch.Generator().manual_seed(1)).cuda()
+    Xd = torch.randn(12, 513, 1024, generator=torch.Generator().manual_seed(1)).cuda()
     z.set_option(z.Option.SPIN_LIMIT, 1)
     try:
         H = z.hessian_accumulate(Xd)
@@ -802,6 +802,24 @@ def test_a_bounded_wait_of_the_pair_kernel_that_runs_out_is_reported():
     assert torch.isnan(H[:, 0, 0]).all()
     H = z.hessian_accumulate(Xd)
     torch.cuda.synchronize()
-    Ho = zo.hessian(Xd[24].cpu())
+    Ho = zo.hessian(Xd[11].cpu())
     scale = np.sqrt(np.outer(np.diag(Ho), np.diag(Ho)))
-    assert np.max(np.abs(H[24].cpu().double().numpy() - Ho) / scale) < 2e-6
+    assert np.max(np.abs(H[11].cpu().double().numpy() - Ho) / scale) < 2e-6
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d,N,L", [(130, 2050, 1), (65, 520, 2), (257, 6144, 1), (300, 6200, 1), (64, 16500, 1)])
+def test_hessian_small_calls_on_clusters_match_oracle(dtype, d, N, L):
+    """Few tiles: a tile's K blocks shared by a cluster of CTAs (ragged splits, two row shares), and the
+    one-pass preparation of token-major fp32 batches on both sides of its largest batch."""
+    z = zb()
+    X, A = token_major_case(dtype, d, N, d, L=L)
+    H = z.hessian_accumulate_tokens(A.cuda())
+    H2 = z.hessian_accumulate_tokens(A.cuda(), H.clone(), beta=1.0)
+    torch.cuda.synchronize()
+    for l in range(L):
+        Ho = zo.hessian(X[l])
+        scale = np.sqrt(np.outer(np.diag(Ho), np.diag(Ho)))
+        assert np.max(np.abs(H[l].cpu().double().numpy() - Ho) / scale) < 2e-6
+        assert np.max(np.abs(H2[l].cpu().double().numpy() - 2 * Ho) / scale) < 4e-6
+        assert torch.equal(H2[l], H2[l].t())
