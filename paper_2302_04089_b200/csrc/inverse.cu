@@ -724,34 +724,62 @@ size_t inverse_workspace_bytes(int L, int d) {
     return c.off;
 }
 
+namespace {
+
+InvCtx carve_inverse(void* ws, int L, int dp, double** lam) {
+    Carver c(ws);
+    InvCtx ctx = {};
+    ctx.A = c.take<double>((size_t)L * dp * dp);
+    ctx.F = c.take<double>((size_t)L * dp * dp);
+    ctx.M = c.take<double>((size_t)L * dp * dp);
+    *lam = c.take<double>((size_t)L);
+    ctx.dp = dp;
+    ctx.L = L;
+    return ctx;
+}
+
+// Factorisation of ctx.A and M^T M.
+ziplm_status invert(const InvCtx& ctx, int d, double* out64, float* tri32, int pitch32, int rows32,
+                    double* diag64) {
+    const int T = ctx.dp / kTile;
+    const ziplm_status s = factor_range(ctx, 0, T);
+    if (s != ZIPLM_OK) return s;
+    PhaseScope ps(PH_INV_LAUUM, ctx.st);
+    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lauum, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kProductSmemBytes));
+    k_lauum<<<dim3(lower_macro_count(T), ctx.L), GT, kProductSmemBytes, ctx.st>>>(ctx.M, ctx.dp, T, d, out64, tri32,
+                                                                                pitch32, rows32, diag64);
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
+}  // namespace
+
+double* inverse_matrix(void* ws) { return static_cast<double*>(ws); }     // the first piece of the workspace
+
+ziplm_status run_inverse_of(void* ws, int L, int d, double* out64, int* layer_status, cudaStream_t st) {
+    double* lam;
+    InvCtx ctx = carve_inverse(ws, L, round_up_int(d, kTile), &lam);
+    ctx.layer_status = layer_status;
+    ctx.st = st;
+    return invert(ctx, d, out64, nullptr, 0, 0, nullptr);
+}
+
 ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, double* out64,
                                 float* tri32, int pitch32, int rows32, double* diag64, double* lam_out,
                                 int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (ws_bytes < inverse_workspace_bytes(L, d)) return ZIPLM_ERR_WORKSPACE;
     const int dp = round_up_int(d, kTile), T = dp / kTile;
-    Carver c(ws);
-    InvCtx ctx;
-    ctx.A = c.take<double>((size_t)L * dp * dp);
-    ctx.F = c.take<double>((size_t)L * dp * dp);
-    ctx.M = c.take<double>((size_t)L * dp * dp);
-    double* lam = c.take<double>((size_t)L);
-    ctx.dp = dp; ctx.L = L; ctx.layer_status = layer_status; ctx.st = st;
-
+    double* lam;
+    InvCtx ctx = carve_inverse(ws, L, dp, &lam);
+    ctx.layer_status = layer_status;
+    ctx.st = st;
     k_mean_diag<<<L, 256, 0, st>>>(H, d, damp_frac, lam, layer_status);
     ZIPLM_CHECK_LAUNCH();
     k_fill_damped<<<dim3(T, dp / 16, L), 256, 0, st>>>(H, d, dp, lam, ctx.A, layer_status);
     ZIPLM_CHECK_LAUNCH();
-    ziplm_status s = factor_range(ctx, 0, T);
+    const ziplm_status s = invert(ctx, d, out64, tri32, pitch32, rows32, diag64);
     if (s != ZIPLM_OK) return s;
-    {
-        PhaseScope ps(PH_INV_LAUUM, st);
-        const cudaError_t attr = cudaFuncSetAttribute(
-            k_lauum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProductSmemBytes);
-        if (attr != cudaSuccess) return ZIPLM_ERR_CUDA;
-        k_lauum<<<dim3(lower_macro_count(T), L), GT, kProductSmemBytes, st>>>(ctx.M, dp, T, d, out64, tri32,
-                                                                            pitch32, rows32, diag64);
-        ZIPLM_CHECK_LAUNCH();
-    }
     if (lam_out) {
         ZIPLM_CHECK_CUDA(cudaMemcpyAsync(lam_out, lam, sizeof(double) * L, cudaMemcpyDeviceToDevice, st));
     }

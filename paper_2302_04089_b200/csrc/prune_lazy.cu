@@ -32,6 +32,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "pick.cuh"
 
 namespace ziplm {
 
@@ -67,7 +68,7 @@ struct LazyState {
 // the start.
 __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, int r, int d, int ld, int rp,
                                                    float* __restrict__ Wt, double* __restrict__ dQ,
-                                                   int* __restrict__ idx,
+                                                   double* __restrict__ norm2, int* __restrict__ idx,
                                                    LazyState* __restrict__ state) {
     __shared__ float tile[32][33];
     const int l = blockIdx.y;
@@ -102,104 +103,13 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
         const int c = c0 + ty + 8 * m;
         if (tx == 0 && c < ld) {
             dQ[(size_t)l * ld + c] = s;
+            norm2[(size_t)l * ld + c] = s;
             idx[(size_t)l * ld + c] = c < d ? c : -1;
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         state[l].sumrho = 0.0; state[l].dw2 = 0.0; state[l].n_new = ld; state[l].pad = 0;
     }
-}
-
-// Candidate of the argmin of rho = q / a (q = Q[k,k], a = H^-1[k,k]).  Candidates are compared by
-// cross-multiplication (q_x a_y < q_y a_x), which needs no float64 division on the critical path;
-// the quotient is formed once, for the winner.  An entry whose a is not positive or whose values
-// are not finite sorts first, so that it is picked -- and its layer flagged -- at once.
-struct Cand {
-    double a, q;
-    int org, pos;
-};
-
-__device__ __forceinline__ bool cand_valid(const Cand& x) {
-    return x.a > 0.0 && isfinite(x.a) && isfinite(x.q);
-}
-
-__device__ __forceinline__ bool better(const Cand& x, const Cand& y) {   // x strictly before y
-    const bool vx = cand_valid(x), vy = cand_valid(y);
-    if (vx != vy) return !vx;
-    if (!vx) return x.org < y.org;
-    const double lhs = x.q * y.a, rhs = y.q * x.a;
-    return lhs < rhs || (lhs == rhs && x.org < y.org);
-}
-
-__device__ __forceinline__ void merge_cand(Cand& best, const Cand& o) {
-    if (o.pos >= 0 && (best.pos < 0 || better(o, best))) best = o;
-}
-
-__device__ __forceinline__ Cand bcast_cand(const Cand& c, int src_lane) {
-    Cand o;
-    o.a = __shfl_sync(0xffffffffu, c.a, src_lane);
-    o.q = __shfl_sync(0xffffffffu, c.q, src_lane);
-    o.org = __shfl_sync(0xffffffffu, c.org, src_lane);
-    o.pos = __shfl_sync(0xffffffffu, c.pos, src_lane);
-    return o;
-}
-
-// fp32 quotient that orders candidates coarsely: +inf for "none", -inf for an invalid entry.
-__device__ __forceinline__ float cand_quotient(const Cand& c) {
-    if (c.pos < 0) return INFINITY;
-    return cand_valid(c) ? __fdividef((float)c.q, (float)c.a) : -INFINITY;
-}
-
-// Best candidate of a warp (every lane returns it).  The cheap fp32 quotient r orders the lanes;
-// only the lanes within 1e-5 of the fp32 minimum (almost always a single one) go through the exact
-// float64 comparison, so the common case costs one reduction and six 32-bit shuffles instead of
-// five rounds of 64-bit exchanges.
-__device__ __forceinline__ Cand warp_best(const Cand& mine, float r, float* warp_min = nullptr) {
-    // warp minimum in one reduction instruction, on keys that order like the floats they encode
-    const unsigned bits = __float_as_uint(r);
-    const unsigned key = bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
-    const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
-    const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
-    if (warp_min) *warp_min = rmin;
-    const bool near_min = mine.pos >= 0 && (r == rmin || r <= rmin + fabsf(rmin) * 1e-5f);
-    unsigned mask = __ballot_sync(0xffffffffu, near_min);
-    Cand best;
-    best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff; best.pos = -1;
-    while (mask) {
-        const int b = __ffs(mask) - 1;
-        mask &= mask - 1;
-        merge_cand(best, bcast_cand(mine, b));
-    }
-    return best;
-}
-
-__device__ __forceinline__ Cand warp_best(const Cand& mine) { return warp_best(mine, cand_quotient(mine)); }
-
-// What a warp, or a CTA, offers as its next pick.
-struct __align__(16) Offer {
-    Cand c;
-};
-
-// Pick among n <= 32 offers by their fp32 keys (good to 1e-5): when exactly one key lies within 4e-5 of
-// the smallest, that offer is the pick and is read directly; otherwise -- near ties, an invalid entry,
-// nothing left -- all of them go through the exact comparison.  Every lane returns the pick and its index.
-__device__ __forceinline__ Cand pick_offer(const Offer* offers, const float* keys, int n, int lane, int* which) {
-    const float k = lane < n ? keys[lane] : INFINITY;
-    const unsigned bits = __float_as_uint(k);
-    const unsigned kmin = __reduce_min_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
-    const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
-    const unsigned near_min = __ballot_sync(0xffffffffu, k <= rmin + fabsf(rmin) * 4e-5f);
-    if (fabsf(rmin) < INFINITY && __popc(near_min) == 1) {
-        *which = __ffs(near_min) - 1;
-        return offers[*which].c;
-    }
-    Cand g;
-    g.a = 1.0; g.q = 0.0; g.org = 0x7fffffff; g.pos = -1;
-    if (lane < n) g = offers[lane].c;
-    const Cand best = warp_best(g);
-    const unsigned mine = __ballot_sync(0xffffffffu, lane < n && best.pos >= 0 && g.pos == best.pos);
-    *which = mine ? __ffs(mine) - 1 : 0;
-    return best;
 }
 
 // nsteps greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
@@ -738,126 +648,6 @@ __global__ void __launch_bounds__(256, 3) k_lazy_update_w(int n_new, int m, int 
     }
 }
 
-// Exact refresh of the state of the last kRefresh structures.  By then the surviving entries of
-// H^-1 have been reduced by orders of magnitude through thousands of fp32 downdates, and the
-// relative error of the saliencies, below 5e-6 until about 64 structures remain, would grow to
-// 1e-4 over the last steps.  H^-1 restricted to the survivors is the inverse of H_lambda
-// restricted to them (Sec. 3.1, the remark on Eq. 4), and Q is the Gram matrix of the current
-// weight columns, so both are rebuilt here from their definitions in float64: one CTA per layer,
-// n <= 64 compacted positions; CTA (l, 0) does the Cholesky, the inverse of the factor and M^T M
-// in shared memory, CTA (l, 1) the Gram matrix.
-constexpr int kRefresh = 64;
-__device__ void lazy_refresh_gram(int n, int d, int r, int rp, const float* __restrict__ Wl,
-                                  float* __restrict__ Ql, double* __restrict__ dQl, float* sW);
-__global__ void __launch_bounds__(256) k_lazy_refresh(int n, int d_in, int d, int r, int rp,
-                                                      const float* __restrict__ H,
-                                                      const double* __restrict__ lam,
-                                                      const int* __restrict__ idx,
-                                                      const float* __restrict__ Wt, float* __restrict__ A,
-                                                      float* __restrict__ Q, double* __restrict__ dA,
-                                                      double* __restrict__ dQ, int* layer_status) {
-    extern __shared__ double dyn_refresh[];
-    double (*sB)[kRefresh + 1] = reinterpret_cast<double (*)[kRefresh + 1]>(dyn_refresh);
-    double (*sI)[kRefresh + 1] = reinterpret_cast<double (*)[kRefresh + 1]>(dyn_refresh + kRefresh * (kRefresh + 1));
-    __shared__ int sidx[kRefresh];
-    __shared__ int flag;
-    const int l = blockIdx.x, tid = threadIdx.x;
-    if (blockIdx.y == 1) {
-        lazy_refresh_gram(n, d, r, rp, Wt + (size_t)l * d * rp, Q + (size_t)l * d * d,
-                          dQ + (size_t)l * d, reinterpret_cast<float*>(dyn_refresh));
-        return;
-    }
-    const float* Hl = H + (size_t)l * d_in * d_in;       // the caller's H has the width d_in itself as its pitch
-    float* Al = A + (size_t)l * d * d;
-    if (tid == 0) flag = 0;
-    if (tid < n) sidx[tid] = idx[(size_t)l * d + tid];
-    __syncthreads();
-    for (int e = tid; e < n * n; e += 256) {
-        const int i = e / n, j = e % n;
-        sB[i][j] = (double)Hl[(size_t)sidx[i] * d_in + sidx[j]] + (i == j ? lam[l] : 0.0);
-    }
-    __syncthreads();
-    // Cholesky B = C C^T, column by column
-    for (int c = 0; c < n; ++c) {
-        if (tid == 0) {
-            double p = sB[c][c];
-            if (!(p > 0.0) || !isfinite(p)) {
-                if (!flag) flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
-                p = 1.0;
-            }
-            sB[c][c] = sqrt(p);
-        }
-        __syncthreads();
-        for (int i = c + 1 + tid; i < n; i += 256) sB[i][c] /= sB[c][c];
-        __syncthreads();
-        const int m = n - 1 - c;
-        for (int e = tid; e < m * m; e += 256) {
-            const int i = c + 1 + e / m, jj = c + 1 + e % m;
-            if (jj <= i) sB[i][jj] -= sB[i][c] * sB[jj][c];
-        }
-        __syncthreads();
-    }
-    // M = C^-1, one thread per column
-    if (tid < n) {
-        const int j = tid;
-        for (int k = 0; k < j; ++k) sI[k][j] = 0.0;
-        for (int k = j; k < n; ++k) {
-            double v = (k == j) ? 1.0 : 0.0;
-            for (int m = j; m < k; ++m) v -= sB[k][m] * sI[m][j];
-            sI[k][j] = v / sB[k][k];
-        }
-    }
-    __syncthreads();
-    // H^-1 = M^T M: fp32 off-diagonal entries in both triangles, float64 diagonal
-    for (int e = tid; e < n * n; e += 256) {
-        const int i = e / n, j = e % n;
-        double t = 0.0;
-        for (int k = (i > j ? i : j); k < n; ++k) t = fma(sI[k][i], sI[k][j], t);
-        if (i == j) dA[(size_t)l * d + i] = t;
-        else Al[(size_t)i * d + j] = (float)t;
-    }
-    if (tid == 0 && flag) set_layer_status(layer_status, l, flag);
-}
-
-// Second half of the refresh, CTA (l, 1): Q = W^T W on the surviving columns (rows of Wt),
-// float64 sums of the fp32 weights.  Chunks of 32 weights per row go through shared memory; every
-// thread owns a 4 x 4 tile of the n x n result.
-__device__ void lazy_refresh_gram(int n, int d, int r, int rp, const float* __restrict__ Wl,
-                                  float* __restrict__ Ql, double* __restrict__ dQl, float* sW) {
-    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < r; k0 += 32) {
-        for (int e = tid; e < kRefresh * 32; e += 256) {
-            const int row = e >> 5, k = e & 31;
-            sW[row * 33 + k] = (row < n && k0 + k < r) ? Wl[(size_t)row * rp + k0 + k] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < 32; ++k) {
-            double a[4], b[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                a[x] = (double)sW[(ti + 16 * x) * 33 + k];
-                b[x] = (double)sW[(tj + 16 * x) * 33 + k];
-            }
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-#pragma unroll
-                for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-            const int i = ti + 16 * x, j = tj + 16 * y;
-            if (i >= n || j >= n) continue;
-            if (i == j) dQl[i] = acc[x][y];
-            else Ql[(size_t)i * d + j] = (float)acc[x][y];
-        }
-}
-
 __global__ void __launch_bounds__(256) k_lazy_pos_of(int n, int d, const int* __restrict__ idx,
                                                      int* __restrict__ pos_of) {
     const int l = blockIdx.x;
@@ -966,15 +756,15 @@ __global__ void k_lazy_base_finish(int L, const double* __restrict__ acc64,
 
 struct LazyWs {
     float* A[2]; float* Q[2]; float* Wt[2];
-    double* dA[2]; double* dQ[2]; int* idx[2];
+    double* dA[2]; double* dQ[2]; double* norm2; int* idx[2];
     int* src; int* pos_of; float* U; float* Z; float* C;
     float* P; int* sched;              // packed operands and work counter of the tensor-core update
     LazyState* state; double* lam; double* base_acc;
-    void* aux; size_t aux_bytes;       // shared by the inverse and by the Gram-matrix product
+    void* aux; size_t aux_bytes;       // shared by the inverse, the Gram-matrix product and the endgame
     int rp, ld; size_t total;
 };
 
-LazyWs carve_lazy(void* ws, int L, int r, int d) {
+LazyWs carve_lazy(void* ws, int L, int r, int d, int n_levels) {
     LazyWs w;
     w.rp = round_up_int(r, 4);
     w.ld = round_up_int(d, 4);
@@ -985,6 +775,7 @@ LazyWs carve_lazy(void* ws, int L, int r, int d) {
     for (int b = 0; b < 2; ++b) w.Wt[b] = c.take<float>((size_t)L * ld * w.rp);
     for (int b = 0; b < 2; ++b) w.dA[b] = c.take<double>((size_t)L * ld);
     for (int b = 0; b < 2; ++b) w.dQ[b] = c.take<double>((size_t)L * ld);
+    w.norm2 = c.take<double>((size_t)L * ld);
     for (int b = 0; b < 2; ++b) w.idx[b] = c.take<int>((size_t)L * ld);
     w.src = c.take<int>((size_t)L * ld);
     w.pos_of = c.take<int>((size_t)L * ld);
@@ -998,7 +789,9 @@ LazyWs carve_lazy(void* ws, int L, int r, int d) {
     w.base_acc = c.take<double>((size_t)L);
     const size_t inv = inverse_workspace_bytes(L, d);
     const size_t gram = hessian_tc_workspace_bytes(L, ld, w.rp, ZIPLM_F32, false);
+    const size_t tail = endgame_workspace_bytes(L, r, kEndgame, n_levels);
     w.aux_bytes = inv > gram ? inv : gram;
+    if (tail > w.aux_bytes) w.aux_bytes = tail;
     w.aux = c.take<char>(w.aux_bytes);
     w.total = c.off;
     return w;
@@ -1017,8 +810,8 @@ static int steps_smem(int S) {
 bool lazy_path_supported(int d) { return d >= 1 && d <= CLUSTER_MAX * SLICE_MAX; }
 
 size_t lazy_workspace_bytes(int L, int r, int d, int n_levels) {
-    (void)n_levels;
-    return carve_lazy(nullptr, L, r, d).total;
+    if (d <= kEndgame) return endgame_workspace_bytes(L, r, d, n_levels);
+    return carve_lazy(nullptr, L, r, d, n_levels).total;
 }
 
 ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d, float damp_frac,
@@ -1027,7 +820,10 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
                             void* ws, size_t ws_bytes, cudaStream_t st) {
     if (!lazy_path_supported(d)) return ZIPLM_ERR_UNSUPPORTED;
     if (ws_bytes < lazy_workspace_bytes(L, r, d, n_levels)) return ZIPLM_ERR_WORKSPACE;
-    LazyWs w = carve_lazy(ws, L, r, d);
+    if (d <= kEndgame)
+        return run_endgame_whole(W, H, L, r, d, damp_frac, levels, n_levels, W_snap, loss, base_loss, order,
+                                 saliency, layer_status, ws, ws_bytes, st);
+    LazyWs w = carve_lazy(ws, L, r, d, n_levels);
     // The matrices have the pitch ld = d rounded up to 4, so that every row starts on 16 bytes (128-bit
     // loads, TMA); the up to three positions behind d are treated as removed ones.
     const int G = d, rp = w.rp, ld = w.ld;
@@ -1043,7 +839,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         ZIPLM_CHECK_CUDA(cudaMemsetAsync(order, 0xFF, sizeof(int) * (size_t)L * G, st));
         if (saliency)
             ZIPLM_CHECK_CUDA(cudaMemsetAsync(saliency, 0, sizeof(float) * (size_t)L * G, st));
-        k_lazy_init<<<dim3((ld + 31) / 32, L), 256, 0, st>>>(W, r, d, ld, rp, w.Wt[0], w.dQ[0], w.idx[0],
+        k_lazy_init<<<dim3((ld + 31) / 32, L), 256, 0, st>>>(W, r, d, ld, rp, w.Wt[0], w.dQ[0], w.norm2, w.idx[0],
                                                            w.state);
         ZIPLM_CHECK_LAUNCH();
         // Q = W^T W: the symmetric product kernel of the Hessian with X = W^T (K = d_row)
@@ -1101,20 +897,20 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             !lazy_tc_make_matrix_map(&map_w[b], w.Wt[b], L, ld, rp))
             return ZIPLM_ERR_CUDA;
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.sched, 0, sizeof(int) * 2, st));
-    constexpr size_t kRefreshSmem = sizeof(double) * 2 * kRefresh * (kRefresh + 1);
-    ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_refresh, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)kRefreshSmem));
+    // The last kEndgame structures go to the float64 endgame unless only a few of them are to be removed
+    // (its set-up costs as much as two blocks).
+    const bool endgame = n_min <= kEndgame - 2 * BMAX;
     while (n > n_min) {
         int stop = (slot < n_levels) ? levels[slot] : n_min;         // next block boundary
-        if (n > kRefresh && stop < kRefresh) stop = kRefresh;        // ... and the refresh point
+        if (endgame && stop < kEndgame) stop = kEndgame;             // ... and where the endgame begins
         const int nsteps = (n - stop < BMAX) ? (n - stop) : BMAX;
         const int nxt = cur ^ 1;
         // Squeezing removed positions out makes the update kernels gather through a map; leaving
         // them in place keeps their reads and writes dense at the price of dead rows and columns.
         // They are squeezed out once they make up kDeadMax positions or a sixteenth of all.
         const int dead_after = npos - (n - nsteps);
-        const bool refresh = (n > kRefresh && n - nsteps == kRefresh);
-        const int compact = (every_block || refresh || dead_after >= kDeadMax ||
+        const bool last = endgame && n - nsteps == kEndgame;
+        const int compact = (every_block || last || dead_after >= kDeadMax ||
                              dead_after * kDeadFraction >= npos) ? 1 : 0;
         {
             PhaseScope ps(PH_LAZY_STEPS, st);
@@ -1174,16 +970,22 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         npos = n_new;
         n -= nsteps;
         t += nsteps;
-        if (refresh) {
-            PhaseScope ps(PH_LAZY_REFRESH, st);
-            k_lazy_refresh<<<dim3(L, 2), 256, kRefreshSmem, st>>>(npos, d, ld, r, rp, H, w.lam, w.idx[cur],
-                                                                  w.Wt[cur], w.A[cur], w.Q[cur], w.dA[cur],
-                                                                  w.dQ[cur], layer_status);
-            ZIPLM_CHECK_LAUNCH();
-        }
         if (slot < n_levels && levels[slot] == n) {
             s = snapshot(npos, slot++);
             if (s != ZIPLM_OK) return s;
+        }
+        if (last) {
+            EndgameTail tail = {};
+            tail.L = L; tail.r = r; tail.d = d;
+            tail.W = W; tail.H = H;
+            tail.Wt = w.Wt[cur]; tail.wt_rows = ld; tail.rp = rp;
+            tail.idx = w.idx[cur]; tail.idx_pitch = ld;
+            tail.norm2 = w.norm2; tail.norm2_pitch = ld;
+            tail.sumrho = &w.state->sumrho; tail.sumrho_stride = (int)(sizeof(LazyState) / sizeof(double));
+            tail.lam = w.lam;
+            tail.W_snap = W_snap; tail.loss = loss; tail.order = order; tail.saliency = saliency;
+            tail.layer_status = layer_status;
+            return run_endgame_tail(tail, levels, n_levels, slot, w.aux, st);
         }
     }
     return ZIPLM_OK;

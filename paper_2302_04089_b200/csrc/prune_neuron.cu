@@ -487,7 +487,8 @@ static ziplm_status run_prune_lazy_grouped(const float* W, const float* H, int L
                                            float* W_snap, float* loss, float* base_loss, int* order,
                                            float* saliency, int* layer_status, void* ws,
                                            cudaStream_t st) {
-    const int groups = layer_groups(L);
+    // layers that run in registers from the start (a few launches for all of them) are not grouped
+    const int groups = d <= kEndgame ? 1 : layer_groups(L);
     DevicePool* pool = groups > 1 ? device_pool() : nullptr;
     EventSet* ev = pool ? take_events(pool) : nullptr;
     if (groups <= 1 || !ev)
