@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "pick.cuh"
+#include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -32,6 +33,7 @@ constexpr int kMaxN = kEndgame;
 constexpr int WORKERS = 16;                       // warps that hold rows of the state
 constexpr int STEP_THREADS = 32 * (WORKERS + 1);  // ... and one that keeps the diagonals
 constexpr int CHUNK = 32;                         // steps per rank update of W
+constexpr int WT = 512;                           // threads of the kernel that replays W
 
 struct Levels {
     int count;                  // levels reached here
@@ -50,7 +52,7 @@ struct Endgame {
     double* A64;                       // [dp][dp] H_lambda for the inverse
     double* inv; double* Q;            // [n0][n0]
     double* base_part;                 // [gram tiles]
-    float* U;                          // [n_steps][n0]
+    float* U; int u_pitch;             // [n_steps][u_pitch], u_pitch = n0 rounded up to 4
     int* piv; double* rs; double* rho; int* removed;     // by step, by step, by step; step by position
     double* dw2;                       // [levels][slabs]
     float* W_snap; int n_levels; float* loss; float* base_loss;
@@ -200,21 +202,48 @@ __global__ void __launch_bounds__(256) k_endgame_setup(const __grid_constant__ E
 
 // ------------------------------------------------------------------------------------------- steps
 // A cluster of CS CTAs per layer; CTA `rank` owns S rows of H^-1 and Q, held in the registers of its 16
-// worker warps (8 rows x 32 CPL columns each).  Lane t of the control warp owns the rows' diagonals.
+// worker warps (4 rows x 32 CPL columns each).  Lane t of the control warp owns the rows' diagonals.
 // What the CTAs exchange in a step is small: every one's best offer for the next pick, and u, z of its own
 // rows, which it can form by itself because the pivot column restricted to its rows is a column of its own
-// block.  Both go out with one cluster barrier a step:
-//   every warp picks p from the offers; the workers that hold column p lay it out; barrier
+// block.  Both go out as asynchronous stores that complete on a barrier of the receiving CTA:
+//   wait for the step's data; every warp picks p from the offers; the workers that hold column p lay it
+//   out; barrier
 //   control: column p brought up to date by the step before, u and z of its rows, their diagonals, the
-//            next offer; pushes both            | workers: the rank-1 updates of the step before
-//   cluster barrier
-// u, z and the bookkeeping of all steps are kept in shared memory and written out at the end: a store to
-// global memory in front of a cluster barrier makes the barrier wait for it (1060 instead of 590 clocks).
-// A first version pushed every CTA's offered row of 2 x 256 doubles to all others: 2.5 us a step, half of it
-// those stores and the barrier behind them.
+//            next offer; sends both             | workers: the rank-1 updates of the step before
+// u, z are in three buffers by step: a CTA may send step m while another's workers still apply step m - 2.
+// u and the bookkeeping of all steps are kept in shared memory and written out at the end.
+// One layer of 256: a version that pushed every CTA's offered row of 2 x 256 doubles to all others took
+// 2.5 us a step, half of it those stores and the cluster barrier behind them; with this exchange and a
+// cluster barrier 1.8 us; as it stands STEP_US us.
 template <int CS, int S, int CPL> struct StepsCfg {
-    static constexpr int RG = S / 8, CG = WORKERS / RG, NP = CG * 32 * CPL, E = (S + 31) / 32;
+    static constexpr int RG = S / 4, CG = WORKERS / RG, NP = CG * 32 * CPL, E = (S + 31) / 32;
 };
+
+struct __align__(16) Bid {       // an offer as it is sent
+    double a, q;
+    int org, pos;
+    unsigned key, pad;           // fp32 quotient as an integer of the same order
+};
+
+__device__ __forceinline__ unsigned order_key(float r) {
+    const unsigned bits = __float_as_uint(r);
+    return bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
+}
+constexpr unsigned kKeyNegInf = 0x007fffffu, kKeyInf = 0xff800000u;
+
+__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void send2(uint32_t to, double x, double y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];"
+                 ::"r"(to), "d"(x), "d"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send2(uint32_t to, long long x, long long y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.s64 [%0], {%1, %2}, [%3];"
+                 ::"r"(to), "l"(x), "l"(y), "r"(bar) : "memory");
+}
 
 template <int CS, int S, int CPL>
 __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_constant__ Endgame w) {
@@ -222,62 +251,85 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
     constexpr int NP = C::NP, E = C::E;
     static_assert(CS * S == NP && NP <= kMaxN, "rows and columns cover the same positions");
     extern __shared__ float dyn_hist[];                        // [n_steps][S] u of the own rows
-    __shared__ __align__(16) double2 s_uz[2][NP];              // u, z by step parity
+    __shared__ __align__(16) double2 s_uz[3][NP];              // u, z by step
     __shared__ __align__(16) double2 s_col[S];                 // column p of H^-1 and Q, own rows
-    __shared__ Offer s_offer[2][CS];
-    __shared__ float s_key[2][CS];
+    __shared__ Bid s_bid[2][CS];                               // by step parity
+    __shared__ uint64_t bar_step[2];
     __shared__ int h_piv[kMaxN], h_org[kMaxN];
     __shared__ double h_rs[kMaxN], h_rho[kMaxN];
+    __shared__ int abort_flag;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = CS > 1 ? (int)cluster.block_rank() : 0;
     const int l = blockIdx.x / CS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = w.n0, row0 = rank * S;
     const bool control = warp == WORKERS;
-    const int rg = warp / C::CG, col0 = (warp % C::CG) * 32 * CPL;        // workers: rows row0 + 8 rg + x
+    const int rg = warp / C::CG, col0 = (warp % C::CG) * 32 * CPL;        // workers: rows row0 + 4 rg + x
     const double* Ag = w.inv + (size_t)l * n * n;
     const double* Qg = w.Q + (size_t)l * n * n;
     const int* idx = w.idx ? w.idx + (size_t)l * w.idx_pitch : nullptr;
 
-    double A[8][CPL], Q[8][CPL];             // workers
+    double A[4][CPL], Q[4][CPL];             // workers
     double da[E], dq[E];                     // control: row lane + 32 e
     int org[E];
     bool alive[E];
     int first_bad = ZIPLM_OK;
+    uint32_t to_uz[CS], to_bid = 0;          // control: where the CTAs take u, z and the bid
+    const uint32_t uz_to_bar = tc::smem_u32(&bar_step[0]) - tc::smem_u32(&s_uz[0][row0 + min(lane, S - 1)]);
+    const uint32_t bid_to_bar = tc::smem_u32(&bar_step[0]) - tc::smem_u32(&s_bid[0][rank]);
 
-    // control: the CTA's best offer for step m, pushed to every CTA
+    // control: the CTA's best offer for step m, sent to every CTA
     auto offer = [&](int m) {
-        float rq[E], rmin = INFINITY;
+        unsigned k[E], kmine = 0xffffffffu;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int ha = __double2hiint(da[e]), hq = __double2hiint(dq[e]);
             const bool ok = (unsigned)(ha - 1) < 0x7fefffffu && (hq & 0x7fffffff) < 0x7ff00000;   // a > 0, finite
             const float x = __fdividef((float)dq[e], (float)da[e]);
-            rq[e] = alive[e] ? (ok ? x : -INFINITY) : INFINITY;
-            rmin = fminf(rmin, rq[e]);
+            k[e] = alive[e] ? (ok ? order_key(x) : kKeyNegInf) : 0xffffffffu;
+            kmine = min(kmine, k[e]);
         }
+        const unsigned kmin = __reduce_min_sync(0xffffffffu, kmine);
         Cand mine;
         mine.a = da[0]; mine.q = dq[0]; mine.org = org[0]; mine.pos = alive[0] ? row0 + lane : -1;
 #pragma unroll
         for (int e = 1; e < E; ++e) {
-            if (!alive[e]) continue;
+            if (!alive[e] || (alive[0] && k[e] > k[0] + 256u)) continue;      // beyond a tie of the fp32 quotients
             Cand c;
             c.a = da[e]; c.q = dq[e]; c.org = org[e]; c.pos = row0 + lane + 32 * e;
             merge_cand(mine, c);
         }
-        float key;
-        const Cand best = warp_best(mine, rmin, &key);
-        if (lane < CS) {
-            Offer* o = &s_offer[m & 1][rank];
-            float* k = &s_key[m & 1][rank];
-            if (CS > 1) {
-                o = cluster.map_shared_rank(o, lane);
-                k = cluster.map_shared_rank(k, lane);
+        // quotients are good to 1e-5, 84 to 168 units of the key
+        unsigned near_min = __ballot_sync(0xffffffffu, mine.pos >= 0 && kmine - kmin <= 256u);
+        Cand best = bcast_cand(mine, near_min ? __ffs(near_min) - 1 : 0);
+        if (near_min & (near_min - 1)) {          // several: the exact comparison
+            near_min &= near_min - 1;
+            while (near_min) {
+                const int b = __ffs(near_min) - 1;
+                near_min &= near_min - 1;
+                merge_cand(best, bcast_cand(mine, b));
             }
-            o->c = best;
-            *k = key;
+        }
+        if (lane < CS) {
+            const long long ids = ((long long)best.pos << 32) | (unsigned)best.org;
+            if (CS > 1) {
+                const uint32_t to = to_bid + (uint32_t)((m & 1) * CS * sizeof(Bid)), bar = to_bid + bid_to_bar + 8u * (m & 1);
+                send2(to, best.a, best.q, bar);
+                send2(to + 16u, ids, (long long)kmin, bar);
+            } else {
+                Bid b;
+                b.a = best.a; b.q = best.q; b.org = best.org; b.pos = best.pos; b.key = kmin; b.pad = 0;
+                s_bid[m & 1][0] = b;
+            }
         }
     };
 
+    if (tid == 0) {
+        abort_flag = 0;
+        tc::mbar_init(tc::smem_u32(&bar_step[0]), 1);
+        tc::mbar_init(tc::smem_u32(&bar_step[1]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
     if (CS > 1) cluster.sync();              // every CTA of the cluster has started
     if (control) {
 #pragma unroll
@@ -288,46 +340,80 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
             dq[e] = alive[e] ? Qg[(size_t)k * n + k] : 0.0;
             org[e] = !alive[e] ? 0x7fffffff : idx ? idx[k] : k;
         }
-        for (int k = lane; k < NP; k += 32) s_uz[1][k] = make_double2(0.0, 0.0);
+        if (CS > 1) {
+#pragma unroll
+            for (int c = 0; c < CS; ++c) {
+                to_uz[c] = map_rank(&s_uz[0][row0 + min(lane, S - 1)], c);
+            }
+            to_bid = map_rank(&s_bid[0][rank], lane < CS ? lane : 0);
+            if (lane == 0) tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), CS * sizeof(Bid));
+        }
+        for (int k = lane; k < NP; k += 32) s_uz[2][k] = make_double2(0.0, 0.0);
         offer(0);
     } else {
 #pragma unroll
-        for (int x = 0; x < 8; ++x)
+        for (int x = 0; x < 4; ++x)
 #pragma unroll
             for (int q = 0; q < CPL; ++q) {
-                const int i = row0 + 8 * rg + x, j = col0 + 32 * q + lane;
+                const int i = row0 + 4 * rg + x, j = col0 + 32 * q + lane;
                 const bool in = i < n && j < n;
                 A[x][q] = in ? Ag[(size_t)i * n + j] : 0.0;
                 Q[x][q] = in ? Qg[(size_t)i * n + j] : 0.0;
             }
     }
-    if (CS > 1) cluster.sync();
-    else __syncthreads();
+    __syncthreads();
 
+    bool failed = false;
+    int cur = 0, last = 2;                   // buffers of step m and step m - 1
     for (int m = 0; m < w.n_steps; ++m) {
         const int par = m & 1;
-        const double2* prev = s_uz[par ^ 1];
-        int which;
-        const Cand g = CS > 1 ? pick_offer(s_offer[par], s_key[par], CS, lane, &which) : s_offer[par][0].c;
-        const int p = g.pos < 0 ? 0 : g.pos;
+        const double2* prev = s_uz[last];
+        if (CS > 1 && !tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
+            failed = true;
+            abort_flag = 1;
+        }
+        // ---- the pick: a bid whose key is alone in a band of 4e-5 (700 units at least) above the smallest,
+        //      otherwise -- near ties, an invalid entry, nothing left -- the exact comparison of all
+        int which = 0;
+        if (CS > 1) {
+            const unsigned k = lane < CS ? s_bid[par][lane].key : 0xffffffffu;
+            const unsigned kmin = __reduce_min_sync(0xffffffffu, k);
+            const unsigned near_min = __ballot_sync(0xffffffffu, k - kmin <= 700u);
+            which = __ffs(near_min) - 1;
+            if ((near_min & (near_min - 1)) || kmin <= kKeyNegInf || kmin >= kKeyInf) {
+                Cand best;
+                best.pos = -1; best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff;
+                for (int c = 0; c < CS; ++c) {
+                    const Bid& b = s_bid[par][c];
+                    Cand o;
+                    o.a = b.a; o.q = b.q; o.org = b.org; o.pos = b.pos;
+                    if (o.pos >= 0 && (best.pos < 0 || better(o, best))) { best = o; which = c; }
+                }
+            }
+        }
+        const Bid* bid = &s_bid[par][which];
+        const int p = max(bid->pos, 0);
         if (!control) {
             if (p / (32 * CPL) == warp % C::CG && (p & 31) == lane) {
 #pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    double a = A[x][0], q = Q[x][0];
+                for (int c = 0; c < CPL; ++c) {
+                    int pc = (p / 32) % CPL;
+                    asm volatile("" : "+r"(pc));      // a test per column: an indexed A would live in local memory
+                    if (pc == c) {
 #pragma unroll
-                    for (int c = 1; c < CPL; ++c)
-                        if ((p / 32) % CPL == c) { a = A[x][c]; q = Q[x][c]; }
-                    s_col[8 * rg + x] = make_double2(a, q);
+                        for (int x = 0; x < 4; ++x) s_col[4 * rg + x] = make_double2(A[x][c], Q[x][c]);
+                    }
                 }
             }
-            __syncthreads();
+            if (__syncthreads_or(failed)) { failed = true; break; }
+            // the float64 pipe belongs to the control warp until it has sent u and z
+            asm volatile("bar.sync 1, %0;" ::"n"(STEP_THREADS) : "memory");
             double2 uj[CPL];
 #pragma unroll
             for (int q = 0; q < CPL; ++q) uj[q] = prev[col0 + 32 * q + lane];
 #pragma unroll
-            for (int x = 0; x < 8; ++x) {
-                const double2 ui = prev[row0 + 8 * rg + x];
+            for (int x = 0; x < 4; ++x) {
+                const double2 ui = prev[row0 + 4 * rg + x];
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) {
                     A[x][q] = fma(-ui.x, uj[q].x, A[x][q]);
@@ -335,17 +421,19 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 }
             }
         } else {
-            double h = g.a;
-            int bad = 0;
-            if (!isfinite(g.q) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
-            else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
-            if (bad && first_bad == ZIPLM_OK) first_bad = bad;
-            const double rs = rsqrt(h), half = 0.5 * g.q * rs * rs;
+            const double ga = bid->a, gq = bid->q;
             const double2 pp = prev[p];
             double2 pj[E];
 #pragma unroll
-            for (int e = 0; e < E; ++e) pj[e] = prev[min(row0 + lane + 32 * e, NP - 1)];
-            __syncthreads();
+            for (int e = 0; e < E; ++e) pj[e] = prev[row0 + min(lane + 32 * e, S - 1)];
+            if (CS > 1 && lane == 0)
+                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]), NP * sizeof(double2) + CS * sizeof(Bid));
+            double h = ga;
+            int bad = 0;
+            if (!isfinite(gq) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
+            else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
+            const double rs = rsqrt(h), half = 0.5 * gq * rs * rs;
+            if (__syncthreads_or(failed)) { failed = true; break; }
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int j = lane + 32 * e;
@@ -354,46 +442,57 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 const double a = fma(-pj[e].x, pp.x, col.x);
                 const double q = fma(-pj[e].y, pp.x, fma(-pj[e].x, pp.y, col.y));
                 const double u = alive[e] ? a * rs : 0.0;
-                const double z = alive[e] ? q * rs - half * u : 0.0;
-                da[e] -= u * u;
-                dq[e] -= 2.0 * z * u;
+                const double z = alive[e] ? fma(q, rs, -half * u) : 0.0;
+                da[e] = fma(-u, u, da[e]);
+                dq[e] = fma(-2.0 * z, u, dq[e]);
                 if (j < S) {
-                    dyn_hist[m * S + j] = (float)u;
                     if (CS > 1) {
+                        static_assert(CS == 1 || E == 1, "one row per lane on a cluster");
 #pragma unroll
                         for (int c = 0; c < CS; ++c)
-                            *cluster.map_shared_rank(&s_uz[par][row0 + j], c) = make_double2(u, z);
+                            send2(to_uz[c] + (uint32_t)(cur * NP * sizeof(double2)), u, z,
+                                  to_uz[c] + uz_to_bar + 8u * (par ^ 1));
                     } else {
-                        s_uz[par][j] = make_double2(u, z);
+                        s_uz[cur][j] = make_double2(u, z);
                     }
+                    dyn_hist[m * S + j] = (float)u;
                 }
             }
+            asm volatile("bar.arrive 1, %0;" ::"n"(STEP_THREADS) : "memory");
             offer(m + 1);
+            if (bad && first_bad == ZIPLM_OK) first_bad = bad;
             if (lane == 0) {
                 h_piv[m] = p;
-                h_org[m] = g.org;
+                h_org[m] = bid->org;
                 h_rs[m] = rs;
-                h_rho[m] = bad ? 0.0 : g.q * rs * rs;
+                h_rho[m] = bad ? 0.0 : gq * rs * rs;
             }
         }
-        if (CS > 1) cluster.sync();
-        else __syncthreads();
+        if (CS == 1) __syncthreads();
+        last = cur;
+        cur = cur == 2 ? 0 : cur + 1;
     }
+    if (failed && tid == 0) set_layer_status(w.layer_status, l, ZIPLM_ERR_TIMEOUT);
+    if (CS > 1 && !failed && tid == 0)       // what the last step sent has landed before any CTA leaves
+        tc::mbar_wait_quiet(tc::smem_u32(&bar_step[w.n_steps & 1]), (uint32_t)(w.n_steps >> 1) & 1u);
+    __syncthreads();
+    if (CS > 1) cluster.sync();
 
     for (int e = tid; e < w.n_steps * S; e += STEP_THREADS) {
         const int m = e / S, k = row0 + e % S;
-        if (k < n) w.U[((size_t)l * w.n_steps + m) * n + k] = dyn_hist[e];
+        if (k < n) w.U[((size_t)l * w.n_steps + m) * w.u_pitch + k] = dyn_hist[e];
     }
     if (rank == 0) {
         for (int k = tid; k < n; k += STEP_THREADS) w.removed[(size_t)l * n + k] = 0x7fffffff;
         __syncthreads();
         for (int m = tid; m < w.n_steps; m += STEP_THREADS) {
             const size_t at = (size_t)l * w.n_steps + m;
-            w.piv[at] = h_piv[m];
+            const int p = failed ? min(m, n - 1) : h_piv[m];
+            w.piv[at] = p;
             w.rs[at] = h_rs[m];
             w.rho[at] = h_rho[m];
-            w.removed[(size_t)l * n + h_piv[m]] = m;
-            w.order[(size_t)l * w.d + w.t0 + m] = h_org[m];
+            w.removed[(size_t)l * n + p] = m;
+            w.order[(size_t)l * w.d + w.t0 + m] = failed ? -1 : h_org[m];
             if (w.saliency) w.saliency[(size_t)l * w.d + w.t0 + m] = (float)h_rho[m];
         }
         if (control && lane == 0 && first_bad != ZIPLM_OK) set_layer_status(w.layer_status, l, first_bad);
@@ -402,102 +501,135 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
 
 // ----------------------------------------------------------------------------------------- weights
 // A CTA replays 32 rows of W over all steps: chunks of up to 32 steps that end at the levels.  The scaled
-// pivot columns c_m = (W[:,p_m] - sum_{s<m} c_s u_s[p_m]) / sqrt(h_m) of its rows are solved by every warp
-// for itself (a lane per row, sums in float64), so that they are in registers for the rank update.
-__global__ void __launch_bounds__(256) k_endgame_weights(const __grid_constant__ Endgame w) {
-    extern __shared__ float dyn_w[];
-    const int n = w.n0, l = blockIdx.y, i0 = blockIdx.x * 32;
+// pivot columns c_m = (W[:,p_m] - sum_{s<m} c_s u_s[p_m]) / sqrt(h_m) of its rows are solved by one warp
+// (a lane per row, sums in float64, every c_m subtracted from the later ones as soon as it is known, so that
+// the chain is one product and two conversions a step; by all warps side by side it took twice as long, bound
+// by their reads of T).  The rank update takes four positions at a time, so that a broadcast load of u feeds
+// four FMAs and four chains run side by side.  The u of the next chunk arrive meanwhile.
+__global__ void __launch_bounds__(WT) k_endgame_weights(const __grid_constant__ Endgame w) {
+    extern __shared__ __align__(16) float dyn_w[];
+    const int n = w.n0, l = blockIdx.y, i0 = blockIdx.x * 32, pitch = w.u_pitch;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int np4 = (n + 3) & ~3;
-    float* sW = dyn_w;                                   // [n][33] current weights, by position
-    float* sO = sW + n * 33;                             // [n][33] original ones
-    float* sU = sW + ((2 * n * 33 + 3) & ~3);            // [n][36] u_s of the chunk, by position; on 16 bytes
-    double* sT = reinterpret_cast<double*>(sU + n * 36);       // [32][32] T[m][s] = u_s[p_m], widened once: a
-                                                         // conversion costs as much as eight FMAs
-    int* sRem = reinterpret_cast<int*>(sT + CHUNK * CHUNK);    // [n] step that removes a position
-    short* sPos = reinterpret_cast<short*>(sRem + np4);  // [d] position of a column, -1: none
-    __shared__ int s_piv[CHUNK];
-    __shared__ double s_rs[CHUNK], red[8];
+    float* sU = dyn_w;                                   // [2][32][pitch] u_s of two chunks
+    double* sT = reinterpret_cast<double*>(sU + 2 * CHUNK * pitch);      // [s][m] T = u_s[p_m], widened once (a
+                                                         // conversion costs as much as eight FMAs)
+    float* sW = reinterpret_cast<float*>(sT + CHUNK * CHUNK);            // [pitch][33] current weights, by position
+    float* sO = sW + pitch * 33;                         // [n][33] original ones
+    int* sRem = reinterpret_cast<int*>(sO + n * 33);     // [n] step that removes a position
+    short* sPos = reinterpret_cast<short*>(sRem + n);    // [d] position of a column, -1: none
+    __shared__ int s_all_piv[kMaxN + CHUNK];
+    __shared__ double s_all_rs[kMaxN + CHUNK], red[WT / 32];
+    __shared__ float sC[CHUNK][32];
     const int* idx = w.idx ? w.idx + (size_t)l * w.idx_pitch : nullptr;
     const float* Wl = w.W + (size_t)l * w.r * w.d;
-    const float* Ul = w.U + (size_t)l * w.n_steps * n;
-    for (int c = tid; c < w.d; c += 256) sPos[c] = (short)(idx ? -1 : c);
+    const float* Ul = w.U + (size_t)l * w.n_steps * pitch;
+    // chunk of steps [t, t + m_n) into a buffer; steps past m_n are zero
+    auto stage = [&](int b, int t, int m_n) {
+        const int quads = pitch / 4;
+        float* to = sU + b * CHUNK * pitch;
+        for (int e = tid; e < CHUNK * quads; e += WT) {
+            const int s = e / quads, k = 4 * (e % quads);
+            const unsigned sa = tc::smem_u32(to + s * pitch + k);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa),
+                         "l"(Ul + (size_t)(s < m_n ? t + s : 0) * pitch + k), "r"(s < m_n ? 16u : 0u) : "memory");
+        }
+    };
+    // the chunk that follows step t: ends at a level or after 32 steps
+    auto chunk_len = [&](int t, int q) {
+        while (q < w.lv.count && w.lv.done[q] <= t) ++q;
+        return q < w.lv.count ? min(CHUNK, (int)w.lv.done[q] - t) : 0;
+    };
+    int m_n = chunk_len(0, 0), buf = 0;
+    if (m_n > 0) stage(0, 0, m_n);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int m = tid; m < kMaxN + CHUNK; m += WT) {
+        s_all_piv[m] = m < w.n_steps ? w.piv[(size_t)l * w.n_steps + m] : 0;
+        s_all_rs[m] = m < w.n_steps ? w.rs[(size_t)l * w.n_steps + m] : 0.0;
+    }
+    for (int c = tid; c < w.d; c += WT) sPos[c] = (short)(idx ? -1 : c);
+    for (int e = tid; e < (pitch - n) * 33; e += WT) sW[n * 33 + e] = 0.f;
     __syncthreads();
-    for (int k = tid; k < n; k += 256) {
+    for (int k = tid; k < n; k += WT) {
         sRem[k] = w.n_steps > 0 ? w.removed[(size_t)l * n + k] : 0x7fffffff;
         if (idx) sPos[idx[k]] = (short)k;
     }
     if (w.Wt) {
         const float* Wtl = w.Wt + (size_t)l * w.wt_rows * w.rp;
-        for (int k = warp; k < n; k += 8) {
+        for (int k = warp; k < n; k += WT / 32) {
             const int i = i0 + lane;
             sW[k * 33 + lane] = i < w.r ? Wtl[(size_t)k * w.rp + i] : 0.f;
             sO[k * 33 + lane] = i < w.r ? Wl[(size_t)i * w.d + (idx ? idx[k] : k)] : 0.f;
         }
     } else {
-        for (int e = tid; e < 32 * n; e += 256) {
+        for (int e = tid; e < 32 * n; e += WT) {
             const int i = e / n, k = e % n;
             const float v = i0 + i < w.r ? Wl[(size_t)(i0 + i) * w.d + k] : 0.f;
             sW[k * 33 + i] = v;
             sO[k * 33 + i] = v;
         }
     }
-    __syncthreads();
     int t = 0;
     for (int q = 0; q < w.lv.count; ++q) {
         const int stop = w.lv.done[q];
         while (t < stop) {
-            const int m_n = min(CHUNK, stop - t);
-            if (tid < CHUNK) {
-                s_piv[tid] = tid < m_n ? w.piv[(size_t)l * w.n_steps + t + tid] : 0;
-                s_rs[tid] = tid < m_n ? w.rs[(size_t)l * w.n_steps + t + tid] : 0.0;
-            }
-            for (int s = warp; s < CHUNK; s += 8)
-                for (int k = lane; k < n; k += 32) sU[k * 36 + s] = s < m_n ? Ul[(size_t)(t + s) * n + k] : 0.f;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             __syncthreads();
-            for (int e = tid; e < CHUNK * CHUNK; e += 256) {
-                const int m = e >> 5, s = e & 31;
-                sT[m * CHUNK + s] = (double)sU[s_piv[m] * 36 + s];
+            const int* s_piv = s_all_piv + t;
+            const double* s_rs = s_all_rs + t;
+            const float* U = sU + buf * CHUNK * pitch;
+            const int next = chunk_len(t + m_n, q);
+            if (next > 0) stage(buf ^ 1, t + m_n, next);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            for (int e = tid; e < CHUNK * CHUNK; e += WT) sT[e] = (double)U[(e >> 5) * pitch + s_piv[e & 31]];
+            __syncthreads();
+            if (warp == 0) {
+                double c[CHUNK];
+#pragma unroll
+                for (int m = 0; m < CHUNK; ++m) c[m] = m < m_n ? (double)sW[s_piv[m] * 33 + lane] : 0.0;
+#pragma unroll
+                for (int s = 0; s < CHUNK; ++s) {
+                    const float f = s < m_n ? (float)(c[s] * s_rs[s]) : 0.f;
+                    const double cs = (double)f;
+                    sC[s][lane] = f;
+#pragma unroll
+                    for (int m = s + 1; m < CHUNK; ++m) c[m] = fma(-cs, sT[s * CHUNK + m], c[m]);
+                }
             }
             __syncthreads();
-            double c[CHUNK];                              // the fp32 values, widened
-#pragma unroll
-            for (int m = 0; m < CHUNK; ++m) {
-                double acc[4] = {m < m_n ? (double)sW[s_piv[m] * 33 + lane] : 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-                for (int s = 0; s < m; ++s) acc[s & 3] = fma(-c[s], sT[m * CHUNK + s], acc[s & 3]);
-                c[m] = (double)(float)(((acc[0] + acc[1]) + (acc[2] + acc[3])) * s_rs[m]);
-            }
             float cf[CHUNK];
 #pragma unroll
-            for (int m = 0; m < CHUNK; ++m) cf[m] = (float)c[m];
-            __syncthreads();                              // everyone has read the pivot rows
-            for (int k = warp; k < n; k += 8) {
-                const float4* u4 = reinterpret_cast<const float4*>(sU + k * 36);
-                float v = sW[k * 33 + lane];
+            for (int s = 0; s < CHUNK; ++s) cf[s] = sC[s][lane];
+            for (int k = 4 * warp; k < pitch; k += WT / 8) {
+                float v[4];
 #pragma unroll
-                for (int s = 0; s < CHUNK / 4; ++s) {
-                    const float4 u = u4[s];
-                    v = fmaf(-u.x, cf[4 * s], v);
-                    v = fmaf(-u.y, cf[4 * s + 1], v);
-                    v = fmaf(-u.z, cf[4 * s + 2], v);
-                    v = fmaf(-u.w, cf[4 * s + 3], v);
+                for (int e = 0; e < 4; ++e) v[e] = sW[(k + e) * 33 + lane];
+#pragma unroll
+                for (int s = 0; s < CHUNK; ++s) {
+                    const float4 u = *reinterpret_cast<const float4*>(U + s * pitch + k);
+                    v[0] = fmaf(-u.x, cf[s], v[0]);
+                    v[1] = fmaf(-u.y, cf[s], v[1]);
+                    v[2] = fmaf(-u.z, cf[s], v[2]);
+                    v[3] = fmaf(-u.w, cf[s], v[3]);
                 }
-                sW[k * 33 + lane] = v;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sW[(k + e) * 33 + lane] = v[e];
             }
             t += m_n;
-            __syncthreads();
+            m_n = next;
+            buf ^= 1;
         }
+        __syncthreads();
         // ---- level: rows i0 .. of the snapshot in original column order, removed columns exactly zero
         const int slot = w.lv.slot0 + q;
         float* out = w.W_snap + (((size_t)l * w.n_levels + slot) * w.r + i0) * w.d;
-        for (int i = warp; i < 32 && i0 + i < w.r; i += 8)
+        for (int i = warp; i < 32 && i0 + i < w.r; i += WT / 32)
+#pragma unroll 4
             for (int c = lane; c < w.d; c += 32) {
                 const int k = sPos[c];
                 out[(size_t)i * w.d + c] = k >= 0 && sRem[k] >= t ? sW[k * 33 + i] : 0.f;
             }
         double part = 0.0;
-        for (int k = warp; k < n; k += 8)
+        for (int k = warp; k < n; k += WT / 32)
             if (sRem[k] >= t) {
                 const float df = sO[k * 33 + lane] - sW[k * 33 + lane];
                 part += (double)df * (double)df;
@@ -508,10 +640,10 @@ __global__ void __launch_bounds__(256) k_endgame_weights(const __grid_constant__
         __syncthreads();
         if (tid == 0) {
             double s = 0.0;
-            for (int v = 0; v < 8; ++v) s += red[v];
+            for (int v = 0; v < WT / 32; ++v) s += red[v];
             w.dw2[((size_t)l * w.lv.count + q) * gridDim.x + blockIdx.x] = s;
         }
-        __syncthreads();
+        m_n = chunk_len(t, q + 1);
     }
 }
 
@@ -557,8 +689,9 @@ int gram_tiles(int n) {
 }
 
 size_t weights_smem(int n, int d) {
-    return sizeof(float) * (size_t)(round_up_int(2 * n * 33, 4) + n * 36 + 2 * CHUNK * CHUNK + round_up_int(n, 4)) +
-           sizeof(short) * (size_t)round_up_int(d, 2);
+    const int pitch = round_up_int(n, 4);
+    return sizeof(float) * (size_t)(2 * CHUNK * pitch + 2 * CHUNK * CHUNK + pitch * 33 + n * 33 + n) +
+           sizeof(short) * (size_t)d;
 }
 
 // Carves the scratch; with ws == nullptr it only measures.
@@ -570,7 +703,8 @@ size_t carve_endgame(Endgame* w, void** inv_ws, void* ws, int L, int r, int n0, 
     w->inv = c.take<double>((size_t)L * n0 * n0);
     w->Q = c.take<double>((size_t)L * n0 * n0);
     w->base_part = c.take<double>((size_t)L * gram_tiles(n0));
-    w->U = c.take<float>((size_t)L * n0 * n0);
+    w->u_pitch = round_up_int(n0, 4);
+    w->U = c.take<float>((size_t)L * n0 * w->u_pitch);
     w->piv = c.take<int>((size_t)L * n0);
     w->rs = c.take<double>((size_t)L * n0);
     w->rho = c.take<double>((size_t)L * n0);
@@ -623,14 +757,14 @@ ziplm_status run(Endgame& w, void* inv_ws, cudaStream_t st) {
     if (w.n_steps > 0) {
         PhaseScope ps(PH_LAZY_STEPS, st);
         // the smallest cluster that holds the state
-        s = n <= 64 ? launch_steps<1, 64, 1>(w, st) : n <= 128 ? launch_steps<4, 32, 1>(w, st) : launch_steps<8, 32, 2>(w, st);
+        s = n <= 64 ? launch_steps<1, 64, 2>(w, st) : n <= 128 ? launch_steps<4, 32, 2>(w, st) : launch_steps<8, 32, 4>(w, st);
         if (s != ZIPLM_OK) return s;
     }
     if (w.lv.count > 0) {
         PhaseScope ps(PH_LAZY_UPDATE_W, st);
         const size_t smem = weights_smem(n, w.d);
         ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_endgame_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_endgame_weights<<<dim3(slabs, w.L), 256, smem, st>>>(w);
+        k_endgame_weights<<<dim3(slabs, w.L), WT, smem, st>>>(w);
         ZIPLM_CHECK_LAUNCH();
     }
     if (w.lv.count > 0 || w.base_loss) {
