@@ -363,19 +363,17 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
     }
     __syncthreads();
 
+    // The pick of step m: a bid whose key is alone in a band of 4e-5 (700 units at least) above the smallest,
+    // otherwise -- near ties, an invalid entry, nothing left -- the exact comparison of all.
     bool failed = false;
-    int cur = 0, last = 2;                   // buffers of step m and step m - 1
-    for (int m = 0; m < w.n_steps; ++m) {
+    auto pick = [&](int m) -> const Bid* {
         const int par = m & 1;
-        const double2* prev = s_uz[last];
-        if (CS > 1 && !tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
-            failed = true;
-            abort_flag = 1;
-        }
-        // ---- the pick: a bid whose key is alone in a band of 4e-5 (700 units at least) above the smallest,
-        //      otherwise -- near ties, an invalid entry, nothing left -- the exact comparison of all
         int which = 0;
         if (CS > 1) {
+            if (!tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
+                failed = true;
+                abort_flag = 1;
+            }
             const unsigned k = lane < CS ? s_bid[par][lane].key : 0xffffffffu;
             const unsigned kmin = __reduce_min_sync(0xffffffffu, k);
             const unsigned near_min = __ballot_sync(0xffffffffu, k - kmin <= 700u);
@@ -391,9 +389,14 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 }
             }
         }
-        const Bid* bid = &s_bid[par][which];
-        const int p = max(bid->pos, 0);
-        if (!control) {
+        return &s_bid[par][which];
+    };
+    // two loops, so that the workers' state and the control warp's share registers
+    int cur = 0, last = 2;                   // buffers of step m and step m - 1
+    if (!control) {
+        for (int m = 0; m < w.n_steps; ++m) {
+            const double2* prev = s_uz[last];
+            const int p = max(pick(m)->pos, 0);
             if (p / (32 * CPL) == warp % C::CG && (p & 31) == lane) {
 #pragma unroll
                 for (int c = 0; c < CPL; ++c) {
@@ -406,21 +409,30 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 }
             }
             if (__syncthreads_or(failed)) { failed = true; break; }
+            double2 ui[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) ui[x] = prev[row0 + 4 * rg + x];
             // the float64 pipe belongs to the control warp until it has sent u and z
             asm volatile("bar.sync 1, %0;" ::"n"(STEP_THREADS) : "memory");
-            double2 uj[CPL];
 #pragma unroll
-            for (int q = 0; q < CPL; ++q) uj[q] = prev[col0 + 32 * q + lane];
+            for (int q = 0; q < CPL; ++q) {
+                const double2 uj = prev[col0 + 32 * q + lane];
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const double2 ui = prev[row0 + 4 * rg + x];
-#pragma unroll
-                for (int q = 0; q < CPL; ++q) {
-                    A[x][q] = fma(-ui.x, uj[q].x, A[x][q]);
-                    Q[x][q] = fma(-ui.y, uj[q].x, fma(-ui.x, uj[q].y, Q[x][q]));
+                for (int x = 0; x < 4; ++x) {
+                    A[x][q] = fma(-ui[x].x, uj.x, A[x][q]);
+                    Q[x][q] = fma(-ui[x].y, uj.x, fma(-ui[x].x, uj.y, Q[x][q]));
                 }
             }
-        } else {
+            if (CS == 1) __syncthreads();
+            last = cur;
+            cur = cur == 2 ? 0 : cur + 1;
+        }
+    } else {
+        for (int m = 0; m < w.n_steps; ++m) {
+            const int par = m & 1;
+            const double2* prev = s_uz[last];
+            const Bid* bid = pick(m);
+            const int p = max(bid->pos, 0);
             const double ga = bid->a, gq = bid->q;
             const double2 pp = prev[p];
             double2 pj[E];
@@ -434,6 +446,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
             else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
             const double rs = rsqrt(h), half = 0.5 * gq * rs * rs;
             if (__syncthreads_or(failed)) { failed = true; break; }
+            float uh[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int j = lane + 32 * e;
@@ -443,8 +456,6 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 const double q = fma(-pj[e].y, pp.x, fma(-pj[e].x, pp.y, col.y));
                 const double u = alive[e] ? a * rs : 0.0;
                 const double z = alive[e] ? fma(q, rs, -half * u) : 0.0;
-                da[e] = fma(-u, u, da[e]);
-                dq[e] = fma(-2.0 * z, u, dq[e]);
                 if (j < S) {
                     if (CS > 1) {
                         static_assert(CS == 1 || E == 1, "one row per lane on a cluster");
@@ -455,11 +466,16 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                     } else {
                         s_uz[cur][j] = make_double2(u, z);
                     }
-                    dyn_hist[m * S + j] = (float)u;
                 }
+                da[e] = fma(-u, u, da[e]);
+                dq[e] = fma(-2.0 * z, u, dq[e]);
+                uh[e] = (float)u;
             }
             asm volatile("bar.arrive 1, %0;" ::"n"(STEP_THREADS) : "memory");
             offer(m + 1);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (lane + 32 * e < S) dyn_hist[m * S + lane + 32 * e] = uh[e];
             if (bad && first_bad == ZIPLM_OK) first_bad = bad;
             if (lane == 0) {
                 h_piv[m] = p;
@@ -467,10 +483,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 h_rs[m] = rs;
                 h_rho[m] = bad ? 0.0 : gq * rs * rs;
             }
+            if (CS == 1) __syncthreads();
+            last = cur;
+            cur = cur == 2 ? 0 : cur + 1;
         }
-        if (CS == 1) __syncthreads();
-        last = cur;
-        cur = cur == 2 ? 0 : cur + 1;
     }
     if (failed && tid == 0) set_layer_status(w.layer_status, l, ZIPLM_ERR_TIMEOUT);
     if (CS > 1 && !failed && tid == 0)       // what the last step sent has landed before any CTA leaves
