@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import enum
+import functools
 import os
 from typing import Optional, Sequence
 
@@ -121,7 +122,23 @@ def status_string(status: int) -> str:
 
 
 def _stream_ptr(t: torch.Tensor) -> int:
-    return torch.cuda.current_stream(t.device).cuda_stream
+    return torch._C._cuda_getCurrentRawStream(t.device.index)
+
+
+class _Nothing:
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        return False
+
+
+_NOTHING = _Nothing()
+
+
+def _on(device):
+    """The device made current for a call; nothing to do, and nothing paid for, where it is already."""
+    return _NOTHING if torch._C._cuda_getDevice() == device.index else torch.cuda.device(device)
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -138,10 +155,12 @@ def _workspace(nbytes: int, device) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
+@functools.lru_cache(maxsize=256)
 def hessian_workspace_bytes(L: int, d: int, n_tokens: int, x_dtype: int) -> int:
     return int(load_library().ziplm_hessian_workspace_bytes(L, d, n_tokens, x_dtype))
 
 
+@functools.lru_cache(maxsize=256)
 def hessian_tokens_workspace_bytes(L: int, d: int, n_tokens: int, a_dtype: int) -> int:
     return int(load_library().ziplm_hessian_tokens_workspace_bytes(L, d, n_tokens, a_dtype))
 
@@ -174,7 +193,7 @@ def hessian_accumulate(X: torch.Tensor, H: Optional[torch.Tensor] = None, alpha:
     need = hessian_workspace_bytes(L, d, N, dt)
     if workspace is None:
         workspace = _workspace(need, X.device)
-    with torch.cuda.device(X.device):
+    with _on(X.device):
         st = lib.ziplm_hessian_accumulate(H.data_ptr(), X.data_ptr(), dt, L, d, N, ldx, alpha, beta,
                                           workspace.data_ptr(), workspace.numel(), _stream_ptr(X))
     if st != 0:
@@ -204,7 +223,7 @@ def hessian_accumulate_tokens(A: torch.Tensor, H: Optional[torch.Tensor] = None,
     need = hessian_tokens_workspace_bytes(L, d, N, dt)
     if workspace is None:
         workspace = _workspace(need, A.device)
-    with torch.cuda.device(A.device):
+    with _on(A.device):
         st = lib.ziplm_hessian_accumulate_tokens(H.data_ptr(), A.data_ptr(), dt, L, d, N, lda, alpha,
                                                  beta, workspace.data_ptr(), workspace.numel(),
                                                  _stream_ptr(A))
@@ -222,7 +241,7 @@ def damped_inverse(H: torch.Tensor, damp_frac: float, workspace: Optional[torch.
     status = torch.zeros(L, dtype=torch.int32, device=H.device)
     if workspace is None:
         workspace = _workspace(inverse_workspace_bytes(L, d), H.device)
-    with torch.cuda.device(H.device):
+    with _on(H.device):
         st = lib.ziplm_damped_inverse(H.data_ptr(), L, d, damp_frac, Hinv.data_ptr(),
                                       status.data_ptr(), workspace.data_ptr(), workspace.numel(),
                                       _stream_ptr(H))
@@ -247,7 +266,7 @@ def damped_inverse_noalloc(H: torch.Tensor, damp_frac: float, Hinv: torch.Tensor
     L, d, _ = H.shape
     if tuple(Hinv.shape) != (L, d, d) or layer_status.numel() != L:
         raise ValueError("Hinv must be [L, d, d] and layer_status [L]")
-    with torch.cuda.device(H.device):
+    with _on(H.device):
         st = lib.ziplm_damped_inverse_noalloc(H.data_ptr(), L, d, damp_frac, Hinv.data_ptr(),
                                               layer_status.data_ptr(), _stream_ptr(H))
     if st != 0:
@@ -292,7 +311,7 @@ def prune_layers(W: torch.Tensor, H: torch.Tensor, group_size: int, damp_frac: f
             out["workspace"] = None          # let go of it before a new one is allocated
             workspace = _workspace(need, dev)
     lv = (ctypes.c_int * max(n_levels, 1))(*levels)
-    with torch.cuda.device(dev):
+    with _on(dev):
         st = lib.ziplm_prune_layers(W.data_ptr(), H.data_ptr(), L, r, d, group_size, damp_frac, lv,
                                     n_levels, _ptr(out["W_snap"]), _ptr(out["loss"]),
                                     _ptr(out["base_loss"]), _ptr(out["order"]), _ptr(out["saliency"]),
@@ -312,7 +331,7 @@ def kept_structures(order: torch.Tensor, level: int):
     L, G = order.shape
     kept = torch.empty(L, max(level, 0), dtype=torch.int32, device=order.device)
     status = torch.empty(L, dtype=torch.int32, device=order.device)
-    with torch.cuda.device(order.device):
+    with _on(order.device):
         st = lib.ziplm_kept_structures(order.data_ptr(), L, G, level, kept.data_ptr(),
                                        status.data_ptr(), _stream_ptr(order))
     if st != 0:
@@ -336,7 +355,7 @@ def gather_columns(M: torch.Tensor, kept: torch.Tensor, group_size: int) -> torc
     level = kept.shape[1]
     G = width // group_size
     out = torch.empty(L, rows, level * group_size, dtype=torch.float32, device=M.device)
-    with torch.cuda.device(M.device):
+    with _on(M.device):
         st = lib.ziplm_gather_columns(M.data_ptr(), ld, ls, kept.data_ptr(), L, rows, G, group_size,
                                       level, out.data_ptr(), _stream_ptr(M))
     if st != 0:
@@ -354,7 +373,7 @@ def gather_rows(M: torch.Tensor, kept: torch.Tensor, group_size: int) -> torch.T
     level = kept.shape[1]
     G = height // group_size
     out = torch.empty(L, level * group_size, cols, dtype=torch.float32, device=M.device)
-    with torch.cuda.device(M.device):
+    with _on(M.device):
         st = lib.ziplm_gather_rows(M.data_ptr(), ld, ls, kept.data_ptr(), L, cols, G, group_size,
                                    level, out.data_ptr(), _stream_ptr(M))
     if st != 0:
@@ -362,6 +381,7 @@ def gather_rows(M: torch.Tensor, kept: torch.Tensor, group_size: int) -> torch.T
     return out
 
 
+@functools.lru_cache(maxsize=256)
 def select_workspace_bytes(n_candidates: int, n_modules: int, n_buckets: int) -> int:
     return int(load_library().ziplm_select_workspace_bytes(n_candidates, n_modules, n_buckets))
 
@@ -391,7 +411,7 @@ def select_levels(loss: torch.Tensor, base_loss: torch.Tensor, time: torch.Tenso
                status=torch.empty(K, dtype=torch.int32, device=dev))
     if workspace is None:
         workspace = _workspace(select_workspace_bytes(K, n_mod, n_buckets), dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         st = lib.ziplm_select_levels(loss.data_ptr(), base_loss.data_ptr(), time.data_ptr(),
                                      n_options.data_ptr(), n_mod, max_opt, coef.data_ptr(), K,
                                      float(budget), n_buckets, out["selected"].data_ptr(),
@@ -403,6 +423,7 @@ def select_levels(loss: torch.Tensor, base_loss: torch.Tensor, time: torch.Tenso
     return out
 
 
+@functools.lru_cache(maxsize=256)
 def search_workspace_bytes(n_searches: int, n_modules: int, n_buckets: int) -> int:
     return int(load_library().ziplm_search_workspace_bytes(n_searches, n_modules, n_buckets))
 
@@ -434,7 +455,7 @@ def search_levels(loss: torch.Tensor, base_loss: torch.Tensor, time: torch.Tenso
                status=torch.empty(S, dtype=torch.int32, device=dev))
     if workspace is None:
         workspace = _workspace(search_workspace_bytes(S, n_mod, n_buckets), dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         st = lib.ziplm_search_levels(loss.data_ptr(), base_loss.data_ptr(), time.data_ptr(),
                                      n_options.data_ptr(), n_mod, max_opt, objective.data_ptr(),
                                      coef0.data_ptr(), budgets.data_ptr(), S, n_buckets,
