@@ -13,8 +13,8 @@ struct HessianProduct {
     float* H;
     int d, layers, num_kb;       // K blocks of 64 tokens
     float alpha, beta;
-    int layer0;
-    int* err_word;
+    int layer0, L;               // L: all layers of the call
+    unsigned long long* err_word; unsigned long long call;     // the word a wait that runs out sets to `call`
     uint32_t fmt16, spin;        // operand format of the instruction; poll limit of the producer
     const unsigned* amax;        // split: largest magnitudes of the feature rows
     bool split;
@@ -24,6 +24,24 @@ struct HessianProduct {
 bool hessian_pair_fits(int layers, int d);
 size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split);
 ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st);
+
+// A product kernel that gives up on a wait leaves NaN in H[l][0][0] of every layer of the call, so that
+// whichever stage reads H next reports ZIPLM_ERR_NONFINITE.  The thread that gives up records the call's
+// number first and poisons the layers then; the CTA that writes an entry (0, 0) looks for the number
+// afterwards (hessian_check): whichever of the two comes second sees the other.  The number is new for
+// every call, so the word needs no clearing.
+__device__ __forceinline__ void hessian_give_up(float* H, int L, int d, unsigned long long* err_word,
+                                                unsigned long long call) {
+    atomicExch(err_word, call);
+    __threadfence();
+    for (int l = 0; l < L; ++l) *reinterpret_cast<volatile float*>(H + (size_t)l * d * d) = __int_as_float(0x7fc00000);
+}
+__device__ __forceinline__ void hessian_check(float* entry, const unsigned long long* err_word,
+                                              unsigned long long call) {
+    __threadfence();
+    if (*reinterpret_cast<const volatile unsigned long long*>(err_word) == call)
+        *reinterpret_cast<volatile float*>(entry) = __int_as_float(0x7fc00000);
+}
 
 // Power-of-two scale of a feature row from the bit pattern of its largest magnitude m: the largest
 // scaled entry lies in [2^13, 2^14).  inverse = true gives 1 / scale.  Rows of zeros and

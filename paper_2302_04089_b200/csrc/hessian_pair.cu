@@ -87,7 +87,7 @@ template <bool SPLIT>
 __global__ void __launch_bounds__(PAIR_THREADS, 1) __cluster_dims__(2, 1, 1)
 k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
             float* __restrict__ H, int d, int num_kb, float alpha, float beta, int layer0,
-            int* __restrict__ err_word, uint32_t fmt16, uint32_t empty_spin_limit,
+            int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
             const unsigned* __restrict__ amax, float4* __restrict__ level2) {
     using C = PairCfg<SPLIT>;
     extern __shared__ uint8_t smem_raw[];
@@ -129,6 +129,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     __syncthreads();
     cluster_barrier();                                    // both CTAs' barriers are initialised
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    grid_wait();                                          // the operands are there
     const uint32_t tmem_base = tmem_base_slot;
     volatile int* abortp = &abort_flag;
     bool failed = false;
@@ -287,6 +288,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                         buf[rr * (NC + 1) + cc] = v;
                     }
                     *p = v;
+                    if ((row | col) == 0) hessian_check(p, err_word, call);
                 }
             }
             __syncwarp();
@@ -300,7 +302,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     }
 
     if (failed) {
-        atomicExch(err_word, (int)ZIPLM_ERR_TIMEOUT);
+        hessian_give_up(H, L, d, err_word, call);
         for (uint32_t r = 0; r < 2; ++r)
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), r)), "r"(1)
                          : "memory");
@@ -330,8 +332,18 @@ template <bool SPLIT>
 ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t st) {
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_pair<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           kPairSmem<SPLIT>));
-    k_syrk_pair<SPLIT><<<dim3(2 * pair_count(p.d), p.layers), PAIR_THREADS, kPairSmem<SPLIT>, st>>>(
-        p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta, p.layer0, p.err_word, p.fmt16, p.spin, p.amax, level2);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pair_count(p.d), p.layers);
+    cfg.blockDim = dim3(PAIR_THREADS);
+    cfg.dynamicSmemBytes = kPairSmem<SPLIT>;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_syrk_pair<SPLIT>, p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta,
+                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, level2));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }

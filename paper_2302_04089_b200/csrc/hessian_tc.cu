@@ -23,12 +23,14 @@
 // below).  Every mbarrier wait is bounded; if one runs out the kernel raises the error word and
 // every role leaves its loop; the issuer then waits (one more commit) for the MMAs it has issued,
 // the producer for the copies it has started, and the CTA leaves through the normal exit (TMEM
-// freed), so a lost copy can never hang the GPU.  A small kernel after the product launches turns
-// a raised error word into NaN in H[l][0][0] of every layer.
+// freed), so a lost copy can never hang the GPU.  H[l][0][0] of every layer is NaN then
+// (hessian_common.cuh).
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <chrono>
 
 #include "common.cuh"
 #include "hessian_common.cuh"
@@ -66,7 +68,7 @@ template <bool TF32>
 __global__ void __launch_bounds__(THREADS, 1)
 k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
           float* __restrict__ H, int d, int num_kb_all, int n_split, float alpha, float beta, int layer0,
-          int* __restrict__ err_word, uint32_t fmt16, uint32_t empty_spin_limit,
+          int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
           const unsigned* __restrict__ amax) {
     using C = Cfg<TF32>;
     constexpr int STAGE_BYTES = C::TILES * TILE_BYTES;
@@ -112,6 +114,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    grid_wait();                                          // the operands are there
     const uint32_t tmem_base = tmem_base_slot;            // main[0] = +0, main[1] = +128, cross = +256
     volatile int* abortp = &abort_flag;
     float* out_tile = reinterpret_cast<float*>(smem_raw + (tiles - raw));    // [TM][OUT_PITCH], over the ring
@@ -243,7 +246,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
 
     if (failed) {
         abort_flag = 1;
-        atomicExch(err_word, (int)ZIPLM_ERR_TIMEOUT);
+        hessian_give_up(H, L, d, err_word, call);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -284,6 +287,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
             float* p = Hl + (size_t)row * d + col;
             if (beta != 0.f) v += *p;
             *p = v;
+            if ((row | col) == 0) hessian_check(p, err_word, call);
             mirror[(rr - first) * OUT_PITCH + cc] = v;
         }
     }
@@ -296,14 +300,6 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
             if (row < d && col < row) Hl[(size_t)col * d + row] = mirror[rr * OUT_PITCH + c];
         }
     if (n_split > 1) cluster.sync();                         // no CTA retires while others read its tile
-}
-
-// A product kernel that gave up on a wait leaves ZIPLM_ERR_TIMEOUT in the error word; the layers'
-// first entries then become NaN, after every product launch of the call, so that whichever stage
-// reads H next reports ZIPLM_ERR_NONFINITE.
-__global__ void k_hessian_flag_timeout(float* __restrict__ H, int L, int d, const int* __restrict__ err_word) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l < L && *err_word != 0) H[(size_t)l * d * d] = __int_as_float(0x7fc00000);
 }
 
 // Largest magnitude of every feature row of a token-contiguous X (bit pattern of |x|, which
@@ -354,6 +350,7 @@ __global__ void __launch_bounds__(256) k_split_f16(const float* __restrict__ X, 
                                                    long long N, long long np, size_t rows,
                                                    const unsigned* __restrict__ amax,
                                                    __half* __restrict__ hi, __half* __restrict__ lo) {
+    grid_trigger();
     const size_t row = blockIdx.y;
     const long long k = ((long long)blockIdx.x * 256 + threadIdx.x) * 4;
     if (row >= rows || k >= np) return;
@@ -382,6 +379,7 @@ __global__ void __launch_bounds__(256) k_row_absmax_split(const float* __restric
                                                           long long N, long long np,
                                                           unsigned* __restrict__ amax,
                                                           __half* __restrict__ hi, __half* __restrict__ lo) {
+    grid_trigger();
     __shared__ unsigned red[8];
     __shared__ unsigned row_max;
     const size_t row = blockIdx.x;
@@ -436,6 +434,7 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor(const T* __restrict__ 
                                                           long long N, int d, long long np,
                                                           const unsigned* __restrict__ amax,
                                                           O* __restrict__ hi, O* __restrict__ lo) {
+    grid_trigger();
     __shared__ T tile[32][33];
     const int l = blockIdx.z;
     const long long t0 = (long long)blockIdx.x * 32;
@@ -473,6 +472,7 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
                                                              long long N, int d, long long np,
                                                              const unsigned* __restrict__ amax,
                                                              O* __restrict__ hi, O* __restrict__ lo) {
+    grid_trigger();
     __shared__ T tile[64][65];                       // [token][feature]
     union Quad { V v; T e[4]; };
     const int l = blockIdx.z;
@@ -531,6 +531,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ A, long long lda, int N, int d,
                                                       long long np, int tokens, unsigned* __restrict__ amax,
                                                       __half* __restrict__ hi, __half* __restrict__ lo) {
+    grid_trigger();
     extern __shared__ float ts_tile[];           // [tokens][TS_PITCH]
     __shared__ unsigned s_max[TS_FEATURES];
     cg::cluster_group cluster = cg::this_cluster();
@@ -544,10 +545,11 @@ __global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ 
     unsigned m[4] = {0u, 0u, 0u, 0u};
     const int f = f0 + 4 * q;
     const bool whole = VEC && f + 3 < d;
-    for (int t = t0 + rr; t < t1; t += 64) {
-        float v[4][4];
+    constexpr int FLY = 16;                      // 16-byte loads in flight per thread
+    for (int t = t0 + rr; t < t1; t += 16 * FLY) {
+        float v[FLY][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < FLY; ++k) {
             const int tk = t + 16 * k;
             v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0.f;
             if (tk >= t1) continue;
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ 
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < FLY; ++k)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 m[e] = max(m[e], __float_as_uint(v[k][e]) & 0x7fffffffu);
@@ -692,6 +694,13 @@ size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, boo
 
 namespace {
 
+// A number that no call had before and that stale scratch does not hold by accident.
+unsigned long long next_call() {
+    static std::atomic<unsigned long long> calls{
+        (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() * 0x9e3779b97f4a7c15ull};
+    return calls.fetch_add(0x9e3779b97f4a7c15ull) | 1ull;
+}
+
 // One product launch on the kernel that suits its number of tiles.  Where the 128 x 128 tiles leave half of
 // the SMs idle, up to eight CTAs share a tile: the largest power of two with which all fit and each keeps
 // four K blocks (one layer of 256 features, 2048 tokens: three tiles, a chain of 32 K blocks on one CTA).
@@ -711,15 +720,17 @@ ziplm_status run_product(const HessianProduct& p, void* scratch, cudaStream_t st
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = p.split ? smem2 : smem1;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = split;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, p.split ? k_syrk_tc<true> : k_syrk_tc<false>, p.hi,
                                         p.split ? p.lo : p.hi, p.H, p.d, p.num_kb, split, p.alpha, p.beta,
-                                        p.layer0, p.err_word, p.fmt16, p.spin, p.amax));
+                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }
@@ -733,12 +744,12 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
     const bool f32 = (dt == ZIPLM_F32);
     const uint32_t fmt16 = (dt == ZIPLM_F16) ? 0u : 1u;
     Carver c(ws);
-    int* err_word = c.take<int>(1);
-    ZIPLM_CHECK_CUDA(cudaMemsetAsync(err_word, 0, sizeof(int), st));
+    unsigned long long* err_word = c.take<unsigned long long>(1);
     const int spin_opt = option_value(ZIPLM_OPT_SPIN_LIMIT);
     const uint32_t spin = spin_opt > 0 ? (uint32_t)spin_opt : kSpinLimit;
     HessianProduct prod = {};
     prod.H = H; prod.d = d; prod.alpha = alpha; prod.beta = beta; prod.err_word = err_word;
+    prod.L = L; prod.call = next_call();
     prod.num_kb = (int)((N + Cfg<false>::BK - 1) / Cfg<false>::BK);
     prod.fmt16 = fmt16; prod.spin = spin; prod.split = f32;
     const int most_layers = product_layers(L, d, N, dt, token_major);
@@ -865,8 +876,6 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
             if (s != ZIPLM_OK) return s;
         }
     }
-    k_hessian_flag_timeout<<<(L + 127) / 128, 128, 0, st>>>(H, L, d, err_word);
-    ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }
 
