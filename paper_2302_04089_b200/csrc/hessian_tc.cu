@@ -269,23 +269,38 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     const int n_rows = TM / n_split, first = rank * n_rows;
     float* Hl = H + (size_t)(layer0 + l) * d * d;
     const unsigned* am = TF32 ? amax + (size_t)l * d : nullptr;
+    // (All parts of a row are requested together: one after the other they took 15000 clocks for two CTAs,
+    // a third of a 1322-wide call; parts sent by the threads that hold them, a row per lane, took longer.)
     for (int rr = first + warp; rr < first + n_rows; rr += THREADS / 32) {
         const int row = i0 + rr;
         if (row >= d) break;
         // split route: undo the power-of-two scales of the two feature rows (exact)
         const float inv_row = TF32 ? row_scale(am[row], true) : 1.f;
+        float part[8][TM / 32], old[TM / 32], scale[TM / 32];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const float* from = out_tile + rr * OUT_PITCH + lane;
+            if (n_split > 1 && s < n_split) from = cluster.map_shared_rank(from, s);
+#pragma unroll
+            for (int h = 0; h < TM / 32; ++h) part[s][h] = s < n_split ? from[32 * h] : 0.f;
+        }
+#pragma unroll
+        for (int h = 0; h < TM / 32; ++h) {
+            const int col = j0 + 32 * h + lane;
+            old[h] = beta != 0.f && col <= row ? Hl[(size_t)row * d + col] : 0.f;
+            scale[h] = TF32 && col <= row ? row_scale(am[col], true) : 1.f;
+        }
 #pragma unroll
         for (int h = 0; h < TM / 32; ++h) {
             const int cc = 32 * h + lane, col = j0 + cc;
-            float v = 0.f;
-            if (n_split == 1) v = out_tile[rr * OUT_PITCH + cc];
-            else
-                for (int s = 0; s < n_split; ++s) v += cluster.map_shared_rank(out_tile, s)[rr * OUT_PITCH + cc];
+            float v = part[0][h];
+#pragma unroll
+            for (int s = 1; s < 8; ++s) if (s < n_split) v += part[s][h];
             if (col > row) continue;                         // (col <= row < d)
             v *= alpha;
-            if (TF32) v = (v * inv_row) * row_scale(am[col], true);
+            if (TF32) v = (v * inv_row) * scale[h];
+            v += old[h];
             float* p = Hl + (size_t)row * d + col;
-            if (beta != 0.f) v += *p;
             *p = v;
             if ((row | col) == 0) hessian_check(p, err_word, call);
             mirror[(rr - first) * OUT_PITCH + cc] = v;
