@@ -41,62 +41,52 @@ __device__ __forceinline__ Cand bcast_cand(const Cand& c, int src_lane) {
     return o;
 }
 
-// fp32 quotient that orders candidates coarsely: +inf for "none", -inf for an invalid entry.
-__device__ __forceinline__ float cand_quotient(const Cand& c) {
-    if (c.pos < 0) return INFINITY;
-    return cand_valid(c) ? __fdividef((float)c.q, (float)c.a) : -INFINITY;
-}
-
-// Best candidate of a warp (every lane returns it).  The cheap fp32 quotient r orders the lanes;
-// only the lanes within 1e-5 of the fp32 minimum (almost always a single one) go through the exact
-// float64 comparison, so the common case costs one reduction and six 32-bit shuffles instead of
-// five rounds of 64-bit exchanges.
-__device__ __forceinline__ Cand warp_best(const Cand& mine, float r, float* warp_min = nullptr) {
-    // warp minimum in one reduction instruction, on keys that order like the floats they encode
+// An fp32 quotient as an integer of the same order.  Quotients of float64 values rounded to fp32 and divided
+// approximately are good to 1e-5, 84 to 168 units of the key: candidates within kKeyNear of each other have
+// to be compared exactly, and so have offers within kKeyFar (4e-5 at least) of each other, which are the
+// best of their warps or CTAs up to kKeyNear.
+constexpr unsigned kKeyNegInf = 0x007fffffu, kKeyInf = 0xff800000u, kKeyNone = 0xffffffffu;
+constexpr unsigned kKeyNear = 256u, kKeyFar = 700u;
+__device__ __forceinline__ unsigned order_key(float r) {
     const unsigned bits = __float_as_uint(r);
-    const unsigned key = bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
-    const unsigned kmin = __reduce_min_sync(0xffffffffu, key);
-    const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
-    if (warp_min) *warp_min = rmin;
-    const bool near_min = mine.pos >= 0 && (r == rmin || r <= rmin + fabsf(rmin) * 1e-5f);
-    unsigned mask = __ballot_sync(0xffffffffu, near_min);
-    Cand best;
-    best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff; best.pos = -1;
-    while (mask) {
-        const int b = __ffs(mask) - 1;
-        mask &= mask - 1;
-        merge_cand(best, bcast_cand(mine, b));
-    }
-    return best;
+    return bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
 }
-
-__device__ __forceinline__ Cand warp_best(const Cand& mine) { return warp_best(mine, cand_quotient(mine)); }
+__device__ __forceinline__ unsigned cand_key(bool alive, double a, double q) {
+    const int ha = __double2hiint(a), hq = __double2hiint(q);
+    const bool ok = (unsigned)(ha - 1) < 0x7fefffffu && (hq & 0x7fffffff) < 0x7ff00000;   // a > 0, finite
+    const float x = __fdividef((float)q, (float)a);
+    return alive ? (ok ? order_key(x) : kKeyNegInf) : kKeyNone;
+}
 
 // What a warp, or a CTA, offers as its next pick.
-struct __align__(16) Offer {
-    Cand c;
+struct __align__(16) Bid {
+    double a, q;
+    int org, pos;
+    unsigned key, pad;
 };
+__device__ __forceinline__ Cand cand_of(const Bid& b) {
+    Cand c;
+    c.a = b.a; c.q = b.q; c.org = b.org; c.pos = b.pos;
+    return c;
+}
 
-// Pick among n <= 32 offers by their fp32 keys (good to 1e-5): when exactly one key lies within 4e-5 of
-// the smallest, that offer is the pick and is read directly; otherwise -- near ties, an invalid entry,
-// nothing left -- all of them go through the exact comparison.  Every lane returns the pick and its index.
-__device__ __forceinline__ Cand pick_offer(const Offer* offers, const float* keys, int n, int lane, int* which) {
-    const float k = lane < n ? keys[lane] : INFINITY;
-    const unsigned bits = __float_as_uint(k);
-    const unsigned kmin = __reduce_min_sync(0xffffffffu, bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u));
-    const float rmin = __uint_as_float(kmin ^ ((kmin >> 31) ? 0x80000000u : 0xffffffffu));
-    const unsigned near_min = __ballot_sync(0xffffffffu, k <= rmin + fabsf(rmin) * 4e-5f);
-    if (fabsf(rmin) < INFINITY && __popc(near_min) == 1) {
-        *which = __ffs(near_min) - 1;
-        return offers[*which].c;
+// Index of the best of n <= 32 bids: the one whose key is alone within kKeyFar of the smallest, otherwise --
+// near ties, an invalid entry, nothing left -- by the exact comparison.  Every lane returns it.
+__device__ __forceinline__ int best_bid(const Bid* bids, int n, int lane) {
+    const unsigned k = lane < n ? bids[lane].key : kKeyNone;
+    const unsigned kmin = __reduce_min_sync(0xffffffffu, k);
+    const unsigned near_min = __ballot_sync(0xffffffffu, k - kmin <= kKeyFar);
+    int which = __ffs(near_min) - 1;
+    if ((near_min & (near_min - 1)) || kmin <= kKeyNegInf || kmin >= kKeyInf) {
+        Cand best;
+        best.pos = -1; best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff;
+        which = 0;
+        for (int c = 0; c < n; ++c) {
+            const Cand o = cand_of(bids[c]);
+            if (o.pos >= 0 && (best.pos < 0 || better(o, best))) { best = o; which = c; }
+        }
     }
-    Cand g;
-    g.a = 1.0; g.q = 0.0; g.org = 0x7fffffff; g.pos = -1;
-    if (lane < n) g = offers[lane].c;
-    const Cand best = warp_best(g);
-    const unsigned mine = __ballot_sync(0xffffffffu, lane < n && best.pos >= 0 && g.pos == best.pos);
-    *which = mine ? __ffs(mine) - 1 : 0;
-    return best;
+    return which;
 }
 
 }  // namespace ziplm

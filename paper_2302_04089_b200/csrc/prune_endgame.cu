@@ -219,32 +219,6 @@ template <int CS, int S, int CPL> struct StepsCfg {
     static constexpr int RG = S / 4, CG = WORKERS / RG, NP = CG * 32 * CPL, E = (S + 31) / 32;
 };
 
-struct __align__(16) Bid {       // an offer as it is sent
-    double a, q;
-    int org, pos;
-    unsigned key, pad;           // fp32 quotient as an integer of the same order
-};
-
-__device__ __forceinline__ unsigned order_key(float r) {
-    const unsigned bits = __float_as_uint(r);
-    return bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
-}
-constexpr unsigned kKeyNegInf = 0x007fffffu, kKeyInf = 0xff800000u;
-
-__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_u32(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void send2(uint32_t to, double x, double y, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];"
-                 ::"r"(to), "d"(x), "d"(y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void send2(uint32_t to, long long x, long long y, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.s64 [%0], {%1, %2}, [%3];"
-                 ::"r"(to), "l"(x), "l"(y), "r"(bar) : "memory");
-}
-
 template <int CS, int S, int CPL>
 __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_constant__ Endgame w) {
     using C = StepsCfg<CS, S, CPL>;
@@ -279,13 +253,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
 
     // control: the CTA's best offer for step m, sent to every CTA
     auto offer = [&](int m) {
-        unsigned k[E], kmine = 0xffffffffu;
+        unsigned k[E], kmine = kKeyNone;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const int ha = __double2hiint(da[e]), hq = __double2hiint(dq[e]);
-            const bool ok = (unsigned)(ha - 1) < 0x7fefffffu && (hq & 0x7fffffff) < 0x7ff00000;   // a > 0, finite
-            const float x = __fdividef((float)dq[e], (float)da[e]);
-            k[e] = alive[e] ? (ok ? order_key(x) : kKeyNegInf) : 0xffffffffu;
+            k[e] = cand_key(alive[e], da[e], dq[e]);
             kmine = min(kmine, k[e]);
         }
         const unsigned kmin = __reduce_min_sync(0xffffffffu, kmine);
@@ -293,13 +264,12 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
         mine.a = da[0]; mine.q = dq[0]; mine.org = org[0]; mine.pos = alive[0] ? row0 + lane : -1;
 #pragma unroll
         for (int e = 1; e < E; ++e) {
-            if (!alive[e] || (alive[0] && k[e] > k[0] + 256u)) continue;      // beyond a tie of the fp32 quotients
+            if (!alive[e] || (alive[0] && k[e] > k[0] + kKeyNear)) continue;      // beyond a tie of the fp32 quotients
             Cand c;
             c.a = da[e]; c.q = dq[e]; c.org = org[e]; c.pos = row0 + lane + 32 * e;
             merge_cand(mine, c);
         }
-        // quotients are good to 1e-5, 84 to 168 units of the key
-        unsigned near_min = __ballot_sync(0xffffffffu, mine.pos >= 0 && kmine - kmin <= 256u);
+        unsigned near_min = __ballot_sync(0xffffffffu, mine.pos >= 0 && kmine - kmin <= kKeyNear);
         Cand best = bcast_cand(mine, near_min ? __ffs(near_min) - 1 : 0);
         if (near_min & (near_min - 1)) {          // several: the exact comparison
             near_min &= near_min - 1;
@@ -313,8 +283,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
             const long long ids = ((long long)best.pos << 32) | (unsigned)best.org;
             if (CS > 1) {
                 const uint32_t to = to_bid + (uint32_t)((m & 1) * CS * sizeof(Bid)), bar = to_bid + bid_to_bar + 8u * (m & 1);
-                send2(to, best.a, best.q, bar);
-                send2(to + 16u, ids, (long long)kmin, bar);
+                tc::send2(to, best.a, best.q, bar);
+                tc::send2(to + 16u, ids, (long long)kmin, bar);
             } else {
                 Bid b;
                 b.a = best.a; b.q = best.q; b.org = best.org; b.pos = best.pos; b.key = kmin; b.pad = 0;
@@ -343,9 +313,9 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
         if (CS > 1) {
 #pragma unroll
             for (int c = 0; c < CS; ++c) {
-                to_uz[c] = map_rank(&s_uz[0][row0 + min(lane, S - 1)], c);
+                to_uz[c] = tc::map_rank(&s_uz[0][row0 + min(lane, S - 1)], c);
             }
-            to_bid = map_rank(&s_bid[0][rank], lane < CS ? lane : 0);
+            to_bid = tc::map_rank(&s_bid[0][rank], lane < CS ? lane : 0);
             if (lane == 0) tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), CS * sizeof(Bid));
         }
         for (int k = lane; k < NP; k += 32) s_uz[2][k] = make_double2(0.0, 0.0);
@@ -363,8 +333,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
     }
     __syncthreads();
 
-    // The pick of step m: a bid whose key is alone in a band of 4e-5 (700 units at least) above the smallest,
-    // otherwise -- near ties, an invalid entry, nothing left -- the exact comparison of all.
+    // The pick of step m.
     bool failed = false;
     auto pick = [&](int m) -> const Bid* {
         const int par = m & 1;
@@ -374,20 +343,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                 failed = true;
                 abort_flag = 1;
             }
-            const unsigned k = lane < CS ? s_bid[par][lane].key : 0xffffffffu;
-            const unsigned kmin = __reduce_min_sync(0xffffffffu, k);
-            const unsigned near_min = __ballot_sync(0xffffffffu, k - kmin <= 700u);
-            which = __ffs(near_min) - 1;
-            if ((near_min & (near_min - 1)) || kmin <= kKeyNegInf || kmin >= kKeyInf) {
-                Cand best;
-                best.pos = -1; best.a = 1.0; best.q = 0.0; best.org = 0x7fffffff;
-                for (int c = 0; c < CS; ++c) {
-                    const Bid& b = s_bid[par][c];
-                    Cand o;
-                    o.a = b.a; o.q = b.q; o.org = b.org; o.pos = b.pos;
-                    if (o.pos >= 0 && (best.pos < 0 || better(o, best))) { best = o; which = c; }
-                }
-            }
+            which = best_bid(s_bid[par], CS, lane);
         }
         return &s_bid[par][which];
     };
@@ -396,7 +352,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
     if (!control) {
         for (int m = 0; m < w.n_steps; ++m) {
             const double2* prev = s_uz[last];
-            const int p = max(pick(m)->pos, 0);
+            const int p = min(max(pick(m)->pos, 0), NP - 1);
             if (p / (32 * CPL) == warp % C::CG && (p & 31) == lane) {
 #pragma unroll
                 for (int c = 0; c < CPL; ++c) {
@@ -432,7 +388,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
             const int par = m & 1;
             const double2* prev = s_uz[last];
             const Bid* bid = pick(m);
-            const int p = max(bid->pos, 0);
+            const int p = min(max(bid->pos, 0), NP - 1);
             const double ga = bid->a, gq = bid->q;
             const double2 pp = prev[p];
             double2 pj[E];
@@ -461,7 +417,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                         static_assert(CS == 1 || E == 1, "one row per lane on a cluster");
 #pragma unroll
                         for (int c = 0; c < CS; ++c)
-                            send2(to_uz[c] + (uint32_t)(cur * NP * sizeof(double2)), u, z,
+                            tc::send2(to_uz[c] + (uint32_t)(cur * NP * sizeof(double2)), u, z,
                                   to_uz[c] + uz_to_bar + 8u * (par ^ 1));
                     } else {
                         s_uz[cur][j] = make_double2(u, z);

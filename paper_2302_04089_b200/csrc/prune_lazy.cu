@@ -32,24 +32,15 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "lazy_common.cuh"
 #include "pick.cuh"
+#include "tc_common.cuh"
 
 namespace ziplm {
 
-// Tensor-core rank-32 update of H^-1, Q and W^T for blocks that leave every position in place
-// (prune_lazy_tc.cu).
-size_t lazy_tc_pack_floats(int L, int d, int rp);
-bool lazy_tc_make_map(CUtensorMap* m, const float* P, int L, int d, int rp);
-bool lazy_tc_make_matrix_map(CUtensorMap* m, const float* M, int L, int d, int cols);
-ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& map_a,
-                                   const CUtensorMap& map_q, const CUtensorMap& map_w, int L, int n_pos,
-                                   int m, int d, int rp, float* A2, float* Q2, float* W2, const float* U,
-                                   const float* Z, const float* C, float* P, int* counter,
-                                   int* layer_status, unsigned slot_spin_limit, cudaStream_t st);
-
 namespace {
 
-constexpr int BMAX = 32;         // pending steps per block
+constexpr int BMAX = kPackSteps; // pending steps per block
 constexpr int STEP_THREADS = 256; // threads per CTA of the steps kernel, four positions each
 constexpr int SLICE_MAX = 768;   // positions per CTA: 2 * BMAX * SLICE_MAX * 4 B = 192 KiB of smem
 constexpr int CLUSTER_MAX = 8;   // portable cluster size
@@ -59,8 +50,6 @@ constexpr int kDeadFraction = 16; // ... or this fraction of all positions, whic
 struct LazyState {
     double sumrho;
     double dw2;
-    int n_new;
-    int pad;
 };
 
 // Wt = W^T (zero padded to rp), float64 column norms, identity index, state reset.  Positions d .. ld - 1
@@ -108,7 +97,7 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        state[l].sumrho = 0.0; state[l].dw2 = 0.0; state[l].n_new = ld; state[l].pad = 0;
+        state[l].sumrho = 0.0; state[l].dw2 = 0.0;
     }
 }
 
@@ -117,18 +106,19 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
 // positions [rank * S, rank * S + S); each of its 256 threads owns four consecutive ones and
 // keeps their float64 diagonal entries of H^-1 and Q in registers for the whole block.  The
 // pending vectors u_s, z_s of the block live in shared memory, sliced the same way (pitch Sp), so the
-// correction of a pivot column touches no global memory; copies go to global memory only for
-// the update kernels that follow.
+// correction of a pivot column touches no global memory.
 //
 // A step is a chain of latencies, so its parts are as short as they can be made and nothing waits for a
 // hand-over that it can do without: the fp32 quotients of a thread's four positions are formed without
-// branches (validity is tested on the upper words; the exact float64 comparison only sees positions within
-// 1e-5 of each other), every warp offers its best, and after the barrier every warp makes the pick for
-// itself and requests the pivot rows at once.  On a cluster (MULTI) warp 0 of a CTA picks the CTA's best
-// first and pushes it to all CTAs together with the pending entries at its position, which the winner's
-// column needs; the cluster barrier is then the only one after it.  The step took 4800 to 5200 clocks when
-// the four quotients and their comparisons ran one after the other (1400 of them) and warp 0 fetched the
-// pending entries after the pick and handed over (1450).
+// branches and ordered as integers (the exact float64 comparison only sees candidates within 1e-5 of each
+// other), every warp offers its best, and after the barrier every warp makes the pick for itself and
+// requests the pivot rows at once.  On a cluster (MULTI) warp 0 of a CTA picks the CTA's best first and
+// sends it to all CTAs, with the pending entries at its position, which the winner's column needs, by
+// asynchronous stores that complete on a barrier of the receiving CTA.  No step writes to global memory:
+// a cluster barrier, and every fence, would wait for it.  What the update kernels need -- u, z and the
+// step order -- goes out at the end of the block, for a dense block as the packed operands themselves.
+// (Clocks per step at 3072 positions: 5200 with the comparisons one after the other and the pending
+// entries fetched after the pick; 3700 with a cluster barrier and u, z stored step by step; STEP_CLOCKS.)
 //
 // The scaled pivot columns of W (c_s) do not feed the selection; they are solved for at the end
 // of the block by forward substitution with the 32 x 32 triangle T[m][s] = u_s[p_m].
@@ -141,6 +131,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
              const int* __restrict__ idx_in, double* __restrict__ dA_out,
              double* __restrict__ dQ_out, int* __restrict__ idx_out, int* __restrict__ src,
              float* __restrict__ U, float* __restrict__ Z, float* __restrict__ C,
+             __nv_bfloat16* __restrict__ P, int rows_pad, int rows_tot,
              LazyState* __restrict__ state, int* __restrict__ order, float* __restrict__ saliency,
              int* layer_status) {
     namespace cg = cooperative_groups;
@@ -154,23 +145,20 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     extern __shared__ float4 dyn_smem4[];
     float* sU = reinterpret_cast<float*>(dyn_smem4);       // [BMAX][Sp]
     float* sZ = sU + (size_t)BMAX * Sp;                    // [BMAX][Sp]
-    double (*sTd)[BMAX] = reinterpret_cast<double (*)[BMAX]>(dyn_smem4);   // T in float64, after the last step
-    __shared__ Offer s_warp[2][NW];                        // the warps' offers, by step parity, and their keys
-    __shared__ float s_wkey[2][NW];
-    __shared__ Offer s_cta[2][CLUSTER_MAX];                // the CTAs' offers, their keys, and the pending
-    __shared__ float s_ckey[2][CLUSTER_MAX];               // entries (u_s[p], z_s[p]) at their positions
-    __shared__ float2 s_pend[2][CLUSTER_MAX][BMAX];
+    double (*sTd)[BMAX] = reinterpret_cast<double (*)[BMAX]>(dyn_smem4);   // [s][m] T in float64, after the last step
+    __shared__ Bid s_warp[2][NW];                          // the warps' offers, by step parity
+    __shared__ Bid s_cta[2][CLUSTER_MAX];                  // the CTAs' offers, and the pending entries
+    __shared__ __align__(16) float2 s_pend[2][CLUSTER_MAX][BMAX];   // (u_s[p], z_s[p]) at their positions
+    __shared__ uint64_t bar_step[2];
     __shared__ float sT[BMAX][BMAX];                       // T[m][s] = u_s[p_m]
-    __shared__ int s_pm[BMAX];
-    __shared__ double s_rsm[BMAX];
+    __shared__ int s_pm[BMAX], s_org[BMAX];
+    __shared__ double s_rsm[BMAX], s_rho[BMAX];
     __shared__ int s_count, s_wsum[NW];
+    __shared__ int abort_flag;
 
     const float* Al = A + (size_t)l * d * d;
     const float* Ql = Q + (size_t)l * d * d;
     const float* Wl = Wt + (size_t)l * d * rp;
-    float* Ul = U + (size_t)l * BMAX * d;
-    float* Zl = Z + (size_t)l * BMAX * d;
-    float* Cl = C + (size_t)l * BMAX * rp;
 
     const int kloc = 4 * tid;                  // first owned position within the slice
     const int k0 = rank * S + kloc;            // ... and globally
@@ -178,6 +166,16 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     double da[4], dq[4];
     int org[4];
     bool alive[4];
+    if (MULTI) {
+        if (tid == 0) {
+            abort_flag = 0;
+            tc::mbar_init(tc::smem_u32(&bar_step[0]), 1);
+            tc::mbar_init(tc::smem_u32(&bar_step[1]), 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
+        }
+        cluster.sync();
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const int k = k0 + e;
@@ -189,24 +187,22 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         dq[e] = alive[e] ? dQ_in[(size_t)l * d + k] : 0.0;
         org[e] = alive[e] ? o : 0x7fffffff;
     }
-    double sumrho = 0.0;                       // meaningful in thread 0 of rank 0
+    int first_bad = ZIPLM_OK;                  // meaningful in lane 0 of the last warp
+    bool failed = false;
 
     for (int m = 0; m < nsteps; ++m) {
         const int par = m & 1;
         // ---- best of the four owned positions of rho = Q[k,k] / H^-1[k,k] (ties: lowest original index)
-        float rq[4];
+        unsigned key[4], kmine = kKeyNone;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int ha = __double2hiint(da[e]), hq = __double2hiint(dq[e]);
-            const bool ok = (unsigned)(ha - 1) < 0x7fefffffu && (hq & 0x7fffffff) < 0x7ff00000;   // a > 0, finite
-            const float x = __fdividef((float)dq[e], (float)da[e]);
-            rq[e] = alive[e] ? (ok ? x : -INFINITY) : INFINITY;
+            key[e] = cand_key(alive[e], da[e], dq[e]);
+            kmine = min(kmine, key[e]);
         }
-        const float rbest = fminf(fminf(rq[0], rq[1]), fminf(rq[2], rq[3]));
-        const float thr = rbest + fabsf(rbest) * 1e-5f;
         unsigned near_mine = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) near_mine |= (alive[e] && (rq[e] == rbest || rq[e] <= thr)) ? 1u << e : 0u;
+        for (int e = 0; e < 4; ++e) near_mine |= (alive[e] && key[e] - kmine <= kKeyNear) ? 1u << e : 0u;
+        const unsigned kmin = __reduce_min_sync(0xffffffffu, kmine);
         Cand best;
         best.a = near_mine & 1 ? da[0] : near_mine & 2 ? da[1] : near_mine & 4 ? da[2] : da[3];
         best.q = near_mine & 1 ? dq[0] : near_mine & 2 ? dq[1] : near_mine & 4 ? dq[2] : dq[3];
@@ -222,62 +218,75 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                 merge_cand(best, c);
             }
         }
-        float wmin;
-        best = warp_best(best, best.pos >= 0 ? rbest : INFINITY, &wmin);
-        if (lane == 0) { s_warp[par][warp].c = best; s_wkey[par][warp] = wmin; }
+        // ---- the warp's offer, written by the lane that holds it
+        const unsigned near_warp = __ballot_sync(0xffffffffu, best.pos >= 0 && kmine - kmin <= kKeyNear);
+        int holder = near_warp ? __ffs(near_warp) - 1 : 0;
+        if (near_warp & (near_warp - 1)) {
+            Cand b = bcast_cand(best, holder);
+            for (unsigned left = near_warp & (near_warp - 1); left; left &= left - 1)
+                merge_cand(b, bcast_cand(best, __ffs(left) - 1));
+            best = b;                              // (every lane has it)
+        }
+        if (lane == holder) {
+            Bid b;
+            b.a = best.a; b.q = best.q; b.org = best.org; b.pos = best.pos; b.key = kmin; b.pad = 0;
+            s_warp[par][warp] = b;
+        }
         __syncthreads();
         // ---- the pick: made by every warp for itself
-        Cand g;
-        int which;
+        const Bid* bid;
+        const float2* pend = nullptr;              // pending entries at the pivot
         if (MULTI) {
             if (warp == 0) {
-                // the CTA's own offer, pushed to every CTA with its pending entries
-                const Cand own = pick_offer(s_warp[par], s_wkey[par], NW, lane, &which);
-                const float key = s_wkey[par][which];
+                // the CTA's own offer, sent to every CTA with its pending entries
+                const Bid own = s_warp[par][best_bid(s_warp[par], NW, lane)];
                 const int pl = own.pos >= 0 ? own.pos - rank * S : 0;
                 float2 uz = make_float2(0.f, 0.f);
                 if (lane < m) uz = make_float2(sU[(size_t)lane * Sp + pl], sZ[(size_t)lane * Sp + pl]);
-                for (int c = 0; c < CS; ++c) {
-                    float2* to = cluster.map_shared_rank(&s_pend[par][rank][0], c);
-                    to[lane] = uz;
-                }
+                const long long packed = ((long long)__float_as_uint(uz.y) << 32) | __float_as_uint(uz.x);
                 if (lane < CS) {
-                    cluster.map_shared_rank(&s_cta[par][rank], lane)->c = own;
-                    *cluster.map_shared_rank(&s_ckey[par][rank], lane) = key;
+                    const uint32_t to = tc::map_rank(&s_cta[par][rank], lane), bar = tc::map_rank(&bar_step[par], lane);
+                    tc::send2(to, own.a, own.q, bar);
+                    tc::send2(to + 16u, ((long long)own.pos << 32) | (unsigned)own.org, (long long)own.key, bar);
                 }
+                for (int c = 0; c < CS; ++c)
+                    tc::send1(tc::map_rank(&s_pend[par][rank][lane], c), packed, tc::map_rank(&bar_step[par], c));
+                if (lane == 0 && m + 1 < nsteps)
+                    tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]),
+                                       (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
             }
-            cluster.sync();
-            g = pick_offer(s_cta[par], s_ckey[par], CS, lane, &which);
+            if (!tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
+                failed = true;                     // (the waits that follow give up at once)
+                abort_flag = 1;
+            }
+            const int which = best_bid(s_cta[par], CS, lane);
+            bid = &s_cta[par][which];
+            pend = s_pend[par][which];
         } else {
-            g = pick_offer(s_warp[par], s_wkey[par], NW, lane, &which);
+            bid = &s_warp[par][best_bid(s_warp[par], NW, lane)];
         }
-        const int p = g.pos < 0 ? 0 : g.pos;
+        const int p = min(max(bid->pos, 0), n0 - 1);
         // both triangles of H^-1 and Q are kept, so the pivot column is the contiguous row p
         float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), q4 = a4;
         if (owner_thread) {
             a4 = *reinterpret_cast<const float4*>(Al + (size_t)p * d + k0);
             q4 = *reinterpret_cast<const float4*>(Ql + (size_t)p * d + k0);
         }
-        double h = g.a;
+        const double gq = bid->q;
+        double h = bid->a;
         int bad = 0;
-        if (!isfinite(g.q) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
+        if (!isfinite(gq) || !isfinite(h)) { bad = ZIPLM_ERR_NONFINITE; h = 1.0; }
         else if (!(h > 0.0)) { bad = ZIPLM_ERR_NOT_PD; h = 1.0; }
-        const double rs = rsqrt(h), half = 0.5 * g.q * rs * rs;
-        // pending entries at the pivot: pushed by its owner, or in this CTA's own slice
-        const float2* pend = s_pend[par][which];
-        const float *pu = sU + p, *pz = sZ + p;
-        if (warp == NW - 1) {                     // (the last warp: the others may own more positions)
+        const double rs = rsqrt(h), half = 0.5 * gq * rs * rs;
+        const float *pu = sU + p, *pz = sZ + p;    // pending entries of one CTA: in its own slice
+        if (warp == NW - 1) {                      // (the last warp: the others may own more positions)
             sT[m][lane] = lane < m ? (MULTI ? pend[lane].x : pu[(size_t)lane * Sp]) : 0.f;
             if (lane == 0) {
                 s_pm[m] = p;
                 s_rsm[m] = rs;
-                if (rank == 0) {
-                    const double rho = bad ? 0.0 : g.q * rs * rs;
-                    if (bad) set_layer_status(layer_status, l, bad);
-                    sumrho += rho;
-                    order[(size_t)l * G + t0 + m] = g.org;
-                    if (saliency) saliency[(size_t)l * G + t0 + m] = (float)rho;
-                }
+                s_rho[m] = bad ? 0.0 : gq * rs * rs;
+                s_org[m] = bid->org;
+                if (bad && first_bad == ZIPLM_OK) first_bad = bad;
             }
         }
         // ---- true pivot columns of H^-1 and Q on the owned positions; float64 diagonal downdate
@@ -317,42 +326,110 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                 u32[e] = alive[e] ? (float)u : 0.f;
                 z32[e] = alive[e] ? (float)z : 0.f;
             }
-            const float4 uo = make_float4(u32[0], u32[1], u32[2], u32[3]);
-            const float4 zo = make_float4(z32[0], z32[1], z32[2], z32[3]);
-            *reinterpret_cast<float4*>(sU + (size_t)m * Sp + kloc) = uo;
-            *reinterpret_cast<float4*>(sZ + (size_t)m * Sp + kloc) = zo;
-            *reinterpret_cast<float4*>(Ul + (size_t)m * d + k0) = uo;
-            *reinterpret_cast<float4*>(Zl + (size_t)m * d + k0) = zo;
+            *reinterpret_cast<float4*>(sU + (size_t)m * Sp + kloc) = make_float4(u32[0], u32[1], u32[2], u32[3]);
+            *reinterpret_cast<float4*>(sZ + (size_t)m * Sp + kloc) = make_float4(z32[0], z32[1], z32[2], z32[3]);
         }
         // no barrier here: the next step's barrier orders these writes before any read
     }
-    if (MULTI) cluster.sync();
-    else __syncthreads();
+    if (failed) set_layer_status(layer_status, l, ZIPLM_ERR_TIMEOUT);
+    __syncthreads();
+
+    // ---- what the update kernels read: u, z as they are for a compaction block, packed for a dense one
+    const int n_own = max(0, min(S, n0 - rank * S));
+    if (compact) {
+        float* Ul = U + (size_t)l * BMAX * d + rank * S;
+        float* Zl = Z + (size_t)l * BMAX * d + rank * S;
+        for (int s = warp; s < nsteps; s += NW)
+            for (int k = lane; k < n_own; k += 32) {
+                Ul[(size_t)s * d + k] = sU[(size_t)s * Sp + k];
+                Zl[(size_t)s * d + k] = sZ[(size_t)s * Sp + k];
+            }
+    } else {
+        // two positions per warp, two steps per lane; the last CTA zeroes the rows up to the next whole tile
+        const size_t arr = (size_t)rows_tot * 2 * BMAX;
+        __nv_bfloat16* Pl = P + (size_t)l * kPackArrays * arr;
+        const int sp = 2 * (lane & 15);
+        const int end = rank == CS - 1 ? (n0 + kPackTile - 1) / kPackTile * kPackTile - rank * S : n_own;
+        for (int k = 2 * warp + (lane >> 4); k < end; k += 2 * NW) {
+            __nv_bfloat162 u[3], z[3];
+            __nv_bfloat16 pa[3], pb[3];
+            const bool in = k < n_own;
+            split_bf16x3(in && sp < nsteps ? sU[(size_t)sp * Sp + k] : 0.f, pa);
+            split_bf16x3(in && sp + 1 < nsteps ? sU[(size_t)(sp + 1) * Sp + k] : 0.f, pb);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) u[x] = __nv_bfloat162(pa[x], pb[x]);
+            split_bf16x3(in && sp < nsteps ? sZ[(size_t)sp * Sp + k] : 0.f, pa);
+            split_bf16x3(in && sp + 1 < nsteps ? sZ[(size_t)(sp + 1) * Sp + k] : 0.f, pb);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) z[x] = __nv_bfloat162(pa[x], pb[x]);
+            __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(Pl + (size_t)(rank * S + k) * 2 * BMAX + sp);
+            o[0] = u[0];       o[BMAX / 2] = u[1];
+            o += arr / 2;
+            o[0] = u[2];       o[BMAX / 2] = z[2];
+            o += arr / 2;
+            o[0] = z[0];       o[BMAX / 2] = z[1];
+        }
+    }
+    if (rank == 0) {
+        if (tid < nsteps) {
+            order[(size_t)l * G + t0 + tid] = s_org[tid];
+            if (saliency) saliency[(size_t)l * G + t0 + tid] = (float)s_rho[tid];
+        }
+        if (warp == NW - 1 && lane == 0) {
+            double sum = 0.0;
+            for (int m = 0; m < nsteps; ++m) sum += s_rho[m];
+            state[l].sumrho += sum;
+            if (first_bad != ZIPLM_OK) set_layer_status(layer_status, l, first_bad);
+        }
+    }
+    __syncthreads();                           // sU, sZ are done with
 
     // ---- c_m = (W[:,p_m] - sum_{s<m} c_s T[m][s]) / sqrt(h_m): forward substitution per row
-    //      index i of W, each CTA takes a slice of the d_row indices.  The triangle is widened to
-    //      float64 once, so that the inner loop is loads and FMAs only.  The solve reads this
-    //      CTA's own shared memory only and runs last, when the per-position state is dead.
+    //      index i of W, each CTA takes a slice of the d_row indices; every c_m is subtracted from the later
+    //      ones as soon as it is known, so that the chain is one product and two conversions a step.  The
+    //      triangle is widened to float64 once, so that the inner loop is loads and FMAs only.  The solve
+    //      reads this CTA's own shared memory only and runs last, when the per-position state is dead.
     auto solve_c = [&]() {
         for (int e = tid; e < BMAX * BMAX; e += STEP_THREADS)
-            sTd[e / BMAX][e % BMAX] = (double)sT[e / BMAX][e % BMAX];
+            sTd[e / BMAX][e % BMAX] = (double)sT[e % BMAX][e / BMAX];
         __syncthreads();
+        float* Cl = C + (size_t)l * BMAX * rp;
         const int per = (rp + CS - 1) / CS;
         for (int i = rank * per + tid; i < min(rp, (rank + 1) * per); i += STEP_THREADS) {
-            float w[BMAX];
-            double c[BMAX];          // the fp32 values that are stored, widened
+            double c[BMAX];
 #pragma unroll
             for (int m = 0; m < BMAX; ++m)
-                w[m] = (m < nsteps && i < r) ? Wl[(size_t)s_pm[m] * rp + i] : 0.f;
+                c[m] = (m < nsteps && i < r) ? (double)Wl[(size_t)s_pm[m] * rp + i] : 0.0;
+            float cf[BMAX];
 #pragma unroll
-            for (int m = 0; m < BMAX; ++m) {
-                double acc[4] = {(double)w[m], 0.0, 0.0, 0.0};
+            for (int s = 0; s < BMAX; ++s) {
+                cf[s] = s < nsteps ? (float)(c[s] * s_rsm[s]) : 0.f;
+                const double cs = (double)cf[s];
 #pragma unroll
-                for (int s = 0; s < m; ++s) acc[s & 3] = fma(-c[s], sTd[m][s], acc[s & 3]);
-                const float cm =
-                    (m < nsteps) ? (float)(((acc[0] + acc[1]) + (acc[2] + acc[3])) * s_rsm[m]) : 0.f;
-                c[m] = (double)cm;
-                if (m < nsteps) Cl[(size_t)m * rp + i] = cm;
+                for (int m = s + 1; m < BMAX; ++m) c[m] = fma(-cs, sTd[s][m], c[m]);
+            }
+            if (compact) {
+#pragma unroll
+                for (int m = 0; m < BMAX; ++m)
+                    if (m < nsteps) Cl[(size_t)m * rp + i] = cf[m];
+            } else {
+                // a row of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest was zeroed
+                // before the first block)
+                const size_t arr = (size_t)rows_tot * 2 * BMAX;
+                uint4* o = reinterpret_cast<uint4*>(P + (size_t)l * kPackArrays * arr + (size_t)(rows_pad + i) * 2 * BMAX);
+#pragma unroll
+                for (int g = 0; g < BMAX / 8; ++g) {
+                    union { __nv_bfloat16 h[8]; uint4 v; } x[3];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        __nv_bfloat16 part[3];
+                        split_bf16x3(cf[8 * g + e], part);
+                        x[0].h[e] = part[0]; x[1].h[e] = part[1]; x[2].h[e] = part[2];
+                    }
+                    o[g] = x[0].v;
+                    o[BMAX / 8 + g] = x[1].v;
+                    o[arr / 8 + g] = x[2].v;
+                }
             }
         }
     };
@@ -366,17 +443,13 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         for (int e = 0; e < 4; ++e) {
             const int k = k0 + e;
             if (owner_thread && k < n0) {
-                src[(size_t)l * d + k] = k;
                 dA_out[(size_t)l * d + k] = da[e];
                 dQ_out[(size_t)l * d + k] = dq[e];
                 idx_out[(size_t)l * d + k] = alive[e] ? org[e] : -1;
             }
         }
-        if (rank == 0 && warp == NW - 1 && lane == 0) {
-            state[l].sumrho += sumrho;
-            state[l].n_new = n0;
-        }
         solve_c();
+        if (MULTI) cluster.sync();      // no CTA leaves while others may send to it
         return;
     }
     const int f0 = alive[0] ? 1 : 0, f1 = alive[1] ? 1 : 0, f2 = alive[2] ? 1 : 0, f3 = alive[3] ? 1 : 0;
@@ -410,8 +483,6 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
             ++np;
         }
     }
-    if (rank == 0 && warp == NW - 1 && lane == 0) state[l].sumrho += sumrho;
-    if (rank == CS - 1 && tid == 0) state[l].n_new = base + s_count;
     if (MULTI) cluster.sync();      // no CTA may retire while another can still read its shared memory
     solve_c();
 }
@@ -897,6 +968,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             !lazy_tc_make_matrix_map(&map_w[b], w.Wt[b], L, ld, rp))
             return ZIPLM_ERR_CUDA;
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.sched, 0, sizeof(int) * 2, st));
+    ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.P, 0, sizeof(float) * lazy_tc_pack_floats(L, ld, rp), st));
     // The last kEndgame structures go to the float64 endgame unless only a few of them are to be removed
     // (its set-up costs as much as two blocks).
     const bool endgame = n_min <= kEndgame - 2 * BMAX;
@@ -911,7 +983,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         const int dead_after = npos - (n - nsteps);
         const bool last = endgame && n - nsteps == kEndgame;
         const int compact = (every_block || last || dead_after >= kDeadMax ||
-                             dead_after * kDeadFraction >= npos) ? 1 : 0;
+                             dead_after * kDeadFraction >= npos || npos <= 1) ? 1 : 0;
         {
             PhaseScope ps(PH_LAZY_STEPS, st);
             // smallest cluster whose per-CTA slice of positions fits shared memory
@@ -939,25 +1011,25 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
                 &cfg, cs > 1 ? k_lazy_steps<true> : k_lazy_steps<false>, npos, S, steps_pitch(S), t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
                 (const float*)w.Q[cur], (const float*)w.Wt[cur], (const double*)w.dA[cur],
                 (const double*)w.dQ[cur], (const int*)w.idx[cur], w.dA[nxt], w.dQ[nxt], w.idx[nxt],
-                w.src, w.U, w.Z, w.C, w.state, order, saliency, layer_status));
+                w.src, w.U, w.Z, w.C, reinterpret_cast<__nv_bfloat16*>(w.P), lazy_tc_rows_pad(ld),
+                lazy_tc_rows_tot(ld, rp), w.state, order, saliency, layer_status));
             ZIPLM_CHECK_LAUNCH();
         }
         const int n_new = compact ? n - nsteps : npos;      // positions after this block
         // The update of W goes first: measured, the step is 2 ms shorter than with the wide update
         // of H^-1 and Q in front (the next steps kernel then follows the kernel with the longer,
         // finer-grained tail).
-        if (n_new > 0 && (compact || n_new <= 1)) {     // a dense block updates W^T in the tensor-core kernel
+        if (n_new > 0 && compact) {     // a dense block updates W^T in the tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_W, st);
             k_lazy_update_w<<<dim3((n_new + 63) / 64, (rp + 255) / 256, L), 256, 0, st>>>(
                 n_new, nsteps, ld, rp, w.Wt[cur], w.Wt[nxt], w.src, w.U, w.C);
             ZIPLM_CHECK_LAUNCH();
         }
-        if (n_new > 1 && !compact) {
+        if (!compact) {
             // every position stays in place: dense tiles, tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);
-            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, n_new, nsteps, ld, rp,
-                                      w.A[nxt], w.Q[nxt], w.Wt[nxt], w.U, w.Z, w.C, w.P, w.sched,
-                                      layer_status, 0u, st);
+            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, n_new, ld, rp,
+                                      w.A[nxt], w.Q[nxt], w.Wt[nxt], w.sched, layer_status, 0u, st);
             if (s != ZIPLM_OK) return s;
         } else if (n_new > 1) {
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);

@@ -10,7 +10,7 @@
 // in the place of the column operand, one accumulator, no mirrored store)
 // (the pending vectors are zero at removed positions, whose rows and columns are carried along
 // unchanged).  Nothing is gathered: tiles are plain rectangles, read by TMA and written densely.
-// A pre-pass (k_lazy_pack_uz) transposes the pending vectors to K-major ([position][step]), each
+// The steps kernel leaves the pending vectors K-major ([position][step], lazy_common.cuh), each
 // value split into three bfloat16 parts x = x1 + x2 + x3 (every part the nearest bfloat16 of what
 // the earlier ones left, so |x - x1 - x2 - x3| <= 2^-27 |x|).  Products of two bfloat16 values are
 // exact in the fp32 accumulator, and the six partial products x_a y_b with a + b <= 4 are kept
@@ -41,15 +41,16 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "lazy_common.cuh"
 #include "tc_common.cuh"
 
 namespace ziplm {
 namespace {
 using namespace tc;
 
-constexpr int PK = 32;                       // pending steps per block = K of the products
+constexpr int PK = kPackSteps;
 constexpr int RM = 128, CN = 128;            // tile rows, tile columns (new index space)
-constexpr int NARR = 3;                      // packed arrays: [U1|U2], [U3|Z3], [Z1|Z2], 128-byte rows
+constexpr int NARR = kPackArrays;            // packed arrays: [U1|U2], [U3|Z3], [Z1|Z2], 128-byte rows
 constexpr int BOX_ROWS = 64;                 // rows per TMA box
 constexpr int BOX_BYTES = BOX_ROWS * 128;    // 8 KiB
 constexpr int ARR_BYTES = 2 * BOX_BYTES;     // one packed array, 128 positions
@@ -80,80 +81,6 @@ struct AqSched {
 struct __align__(16) TileSlot {
     int l, i0, j0, flags;
 };
-
-// The three bfloat16 parts of x, each the nearest bfloat16 of what the earlier ones left.
-__device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16 (&p)[3]) {
-    p[0] = __float2bfloat16_rn(x);
-    const float r1 = x - __bfloat162float(p[0]);        // exact
-    p[1] = __float2bfloat16_rn(r1);
-    const float r2 = r1 - __bfloat162float(p[1]);       // exact
-    p[2] = __float2bfloat16_rn(r2);
-}
-
-// P[l][a][i][64] (bfloat16), a = 0: [U1 | U2], 1: [U3 | Z3], 2: [Z1 | Z2], each half the 32 steps
-// of one part: pending vectors by position, zero for steps >= m and for rows n_pos .. the next
-// multiple of 128.
-__global__ void __launch_bounds__(256) k_lazy_pack_uz(int n_pos, int m, int d, int rows_pad, int rows_tot,
-                                                      int pos_blocks, int rp,
-                                                      const float* __restrict__ U,
-                                                      const float* __restrict__ Z,
-                                                      const float* __restrict__ C,
-                                                      __nv_bfloat16* __restrict__ P) {
-    __shared__ float tu[PK][33], tz[PK][33];
-    const int l = blockIdx.y;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const size_t arr = (size_t)rows_tot * 2 * PK;
-    __nv_bfloat16* Pl = P + (size_t)l * NARR * arr;
-    if ((int)blockIdx.x >= pos_blocks) {
-        // rows rows_pad + c: the scaled pivot columns C[s][c] of W (the column operand of the
-        // tiles of W^T) in the place of U, zeros in the place of Z
-        const int c0 = ((int)blockIdx.x - pos_blocks) * 32;
-        const float* Cl = C + (size_t)l * PK * rp;
-#pragma unroll
-        for (int s = ty; s < PK; s += 8) {
-            const int c = c0 + tx;
-            tu[s][tx] = (c < rp && s < m) ? Cl[(size_t)s * rp + c] : 0.f;
-        }
-        __syncthreads();
-        const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-#pragma unroll
-        for (int rr = ty; rr < 32; rr += 8) {
-            const int i = rows_pad + c0 + rr;
-            if (i >= rows_tot) continue;
-            __nv_bfloat16 u[3];
-            split_bf16x3(tu[tx][rr], u);
-            const size_t o = (size_t)i * 2 * PK + tx;
-            Pl[o] = u[0];            Pl[o + PK] = u[1];
-            Pl[arr + o] = u[2];      Pl[arr + o + PK] = zero;
-            Pl[2 * arr + o] = zero;  Pl[2 * arr + o + PK] = zero;
-        }
-        return;
-    }
-    const int i0 = blockIdx.x * 32;
-    const int pos = i0 + tx;
-    const int sp = pos < n_pos ? pos : -1;
-    const float* Ul = U + (size_t)l * PK * d;
-    const float* Zl = Z + (size_t)l * PK * d;
-#pragma unroll
-    for (int s = ty; s < PK; s += 8) {
-        const bool ok = sp >= 0 && s < m;
-        tu[s][tx] = ok ? Ul[(size_t)s * d + sp] : 0.f;
-        tz[s][tx] = ok ? Zl[(size_t)s * d + sp] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int rr = ty; rr < 32; rr += 8) {
-        const int i = i0 + rr;
-        if (i >= rows_pad) continue;
-        __nv_bfloat16 u[3], z[3];
-        split_bf16x3(tu[tx][rr], u);
-        split_bf16x3(tz[tx][rr], z);
-        const size_t o = (size_t)i * 2 * PK + tx;
-        Pl[o] = u[0];            Pl[o + PK] = u[1];
-        Pl[arr + o] = u[2];      Pl[arr + o + PK] = z[2];
-        Pl[2 * arr + o] = z[0];  Pl[2 * arr + o + PK] = z[1];
-    }
-}
 
 __global__ void __launch_bounds__(AQ_THREADS, 1)
 k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_a,
@@ -545,13 +472,6 @@ int sm_count() {
 
 }  // namespace
 
-int lazy_tc_rows_pad(int d) { return round_up_int(d, RM); }
-// rows of P: the positions, then the row indices of W (the packed C), both padded to whole tiles
-static int lazy_tc_rows_tot(int d, int rp) { return lazy_tc_rows_pad(d) + round_up_int(rp, CN); }
-
-// size of the packed operands in floats (NARR arrays of 2 * PK bfloat16 per row of P)
-size_t lazy_tc_pack_floats(int L, int d, int rp) { return (size_t)L * NARR * lazy_tc_rows_tot(d, rp) * PK; }
-
 // Tensor map over the packed operands P[L][3][rows_tot][64] (bfloat16): box = 64 rows of one array.
 bool lazy_tc_make_map(CUtensorMap* m, const float* P, int L, int d, int rp) {
     EncodeTiledFn enc = get_encode();
@@ -589,20 +509,15 @@ bool lazy_tc_make_matrix_map(CUtensorMap* m, const float* M, int L, int d, int c
 // limit of the producer's wait for a free descriptor slot.
 ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& map_a,
                                    const CUtensorMap& map_q, const CUtensorMap& map_w, int L, int n_pos,
-                                   int m, int d, int rp, float* A2, float* Q2, float* W2, const float* U,
-                                   const float* Z, const float* C, float* P, int* counter,
+                                   int d, int rp, float* A2, float* Q2, float* W2, int* counter,
                                    int* layer_status, unsigned slot_spin_limit, cudaStream_t st) {
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_update_aq_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           AQ_SMEM));
     const int sms = sm_count();
     if (sms <= 0) return ZIPLM_ERR_CUDA;
-    const int rows_pad = lazy_tc_rows_pad(d), rows_tot = lazy_tc_rows_tot(d, rp);
+    const int rows_pad = lazy_tc_rows_pad(d);
     const int rows_used = round_up_int(n_pos, RM);
     if (rows_used / RM > MAX_STRIPS) return ZIPLM_ERR_UNSUPPORTED;
-    const int pos_blocks = rows_used / 32, c_blocks = (rows_tot - rows_pad) / 32;
-    k_lazy_pack_uz<<<dim3(pos_blocks + c_blocks, L), 256, 0, st>>>(n_pos, m, d, rows_pad, rows_tot, pos_blocks,
-                                                                  rp, U, Z, C, reinterpret_cast<__nv_bfloat16*>(P));
-    ZIPLM_CHECK_LAUNCH();
     // The kernel is bound by memory bandwidth, which two thirds of the SMs saturate (measured: the
     // same time with 96 as with 148 CTAs, 12 % more with 74); the others are left to the kernels
     // of other layer groups and batches that run beside it.

@@ -155,6 +155,26 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// Asynchronous stores to another CTA of the cluster that complete on a barrier of that CTA (addresses of
+// the shared::cluster window).
+__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void send1(uint32_t to, long long x, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.s64 [%0], %1, [%2];"
+                 ::"r"(to), "l"(x), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send2(uint32_t to, double x, double y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];"
+                 ::"r"(to), "d"(x), "d"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send2(uint32_t to, long long x, long long y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.s64 [%0], {%1, %2}, [%3];"
+                 ::"r"(to), "l"(x), "l"(y), "r"(bar) : "memory");
+}
+
 // Programmatic dependent launch: what comes before the wait overlaps the end of the kernel before, whose
 // results (and everything before it) are complete behind it; the trigger lets the next kernel start its
 // own prologue.
