@@ -35,13 +35,15 @@ ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& ma
                                    int d, int rp, float* A2, float* Q2, float* W2, int* counter,
                                    int* layer_status, unsigned slot_spin_limit, cudaStream_t st);
 
-// The three bfloat16 parts of x, each the nearest bfloat16 of what the earlier ones left.
-__device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16 (&p)[3]) {
-    p[0] = __float2bfloat16_rn(x);
-    const float r1 = x - __bfloat162float(p[0]);        // exact
-    p[1] = __float2bfloat16_rn(r1);
-    const float r2 = r1 - __bfloat162float(p[1]);       // exact
-    p[2] = __float2bfloat16_rn(r2);
+// The three bfloat16 parts of two values, each the nearest bfloat16 of what the earlier ones left (the
+// remainders are exact).
+__device__ __forceinline__ void split_bf16x3(float x, float y, __nv_bfloat162 (&p)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[k] = __floats2bfloat162_rn(x, y);
+        x -= __low2float(p[k]);
+        y -= __high2float(p[k]);
+    }
 }
 
 }  // namespace ziplm

@@ -101,6 +101,12 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
     }
 }
 
+// D(8x8) += A(8x4) B(4x8) in float64 on the tensor core.
+__device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
 // nsteps greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
 // chosen so that a CTA's slice of positions fits its shared memory).  CTA `rank` owns the
 // positions [rank * S, rank * S + S); each of its 256 threads owns four consecutive ones and
@@ -112,9 +118,9 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
 // hand-over that it can do without: the fp32 quotients of a thread's four positions are formed without
 // branches and ordered as integers (the exact float64 comparison only sees candidates within 1e-5 of each
 // other), every warp offers its best, and after the barrier every warp makes the pick for itself and
-// requests the pivot rows at once.  On a cluster (MULTI) warp 0 of a CTA picks the CTA's best first and
-// sends it to all CTAs, with the pending entries at its position, which the winner's column needs, by
-// asynchronous stores that complete on a barrier of the receiving CTA.  No step writes to global memory:
+// requests the pivot rows at once.  On a cluster (MULTI) the CTA's best is picked first and warp c sends
+// it to CTA c, with the pending entries at its position, which the winner's column needs, by asynchronous
+// stores that complete on a barrier of the receiving CTA.  No step writes to global memory:
 // a cluster barrier, and every fence, would wait for it.  What the update kernels need -- u, z and the
 // step order -- goes out at the end of the block, for a dense block as the packed operands themselves.
 // (Clocks per step at 3072 positions: 5200 with the comparisons one after the other and the pending
@@ -145,7 +151,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     extern __shared__ float4 dyn_smem4[];
     float* sU = reinterpret_cast<float*>(dyn_smem4);       // [BMAX][Sp]
     float* sZ = sU + (size_t)BMAX * Sp;                    // [BMAX][Sp]
-    double (*sTd)[BMAX] = reinterpret_cast<double (*)[BMAX]>(dyn_smem4);   // [s][m] T in float64, after the last step
+    double (*sTd)[BMAX + 4] = reinterpret_cast<double (*)[BMAX + 4]>(dyn_smem4);   // T in float64, after the last step
     __shared__ Bid s_warp[2][NW];                          // the warps' offers, by step parity
     __shared__ Bid s_cta[2][CLUSTER_MAX];                  // the CTAs' offers, and the pending entries
     __shared__ __align__(16) float2 s_pend[2][CLUSTER_MAX][BMAX];   // (u_s[p], z_s[p]) at their positions
@@ -175,6 +181,13 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
             tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
         }
         cluster.sync();
+    }
+    // where warp c sends to in CTA c
+    uint32_t to_bid = 0, to_pend = 0, to_bar = 0;
+    if (MULTI && warp < CS) {
+        to_bid = tc::map_rank(&s_cta[0][rank], warp);
+        to_pend = tc::map_rank(&s_pend[0][rank][lane], warp);
+        to_bar = tc::map_rank(&bar_step[0], warp);
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -237,24 +250,24 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         const Bid* bid;
         const float2* pend = nullptr;              // pending entries at the pivot
         if (MULTI) {
-            if (warp == 0) {
-                // the CTA's own offer, sent to every CTA with its pending entries
-                const Bid own = s_warp[par][best_bid(s_warp[par], NW, lane)];
+            // the CTA's own offer, sent to every CTA (warp c to CTA c) with its pending entries
+            const Bid own = s_warp[par][best_bid(s_warp[par], NW, lane)];
+            if (warp < CS) {
                 const int pl = own.pos >= 0 ? own.pos - rank * S : 0;
                 float2 uz = make_float2(0.f, 0.f);
                 if (lane < m) uz = make_float2(sU[(size_t)lane * Sp + pl], sZ[(size_t)lane * Sp + pl]);
-                const long long packed = ((long long)__float_as_uint(uz.y) << 32) | __float_as_uint(uz.x);
-                if (lane < CS) {
-                    const uint32_t to = tc::map_rank(&s_cta[par][rank], lane), bar = tc::map_rank(&bar_step[par], lane);
+                const uint32_t bar = to_bar + 8u * par;
+                if (lane == 0) {
+                    const uint32_t to = to_bid + (uint32_t)(par * CLUSTER_MAX * sizeof(Bid));
                     tc::send2(to, own.a, own.q, bar);
                     tc::send2(to + 16u, ((long long)own.pos << 32) | (unsigned)own.org, (long long)own.key, bar);
                 }
-                for (int c = 0; c < CS; ++c)
-                    tc::send1(tc::map_rank(&s_pend[par][rank][lane], c), packed, tc::map_rank(&bar_step[par], c));
-                if (lane == 0 && m + 1 < nsteps)
-                    tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]),
-                                       (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
+                tc::send1(to_pend + (uint32_t)(par * CLUSTER_MAX * BMAX * sizeof(float2)),
+                          ((long long)__float_as_uint(uz.y) << 32) | __float_as_uint(uz.x), bar);
             }
+            if (tid == 0 && m + 1 < nsteps)
+                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]),
+                                   (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
             if (!tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
                 failed = true;                     // (the waits that follow give up at once)
                 abort_flag = 1;
@@ -345,29 +358,32 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                 Zl[(size_t)s * d + k] = sZ[(size_t)s * Sp + k];
             }
     } else {
-        // two positions per warp, two steps per lane; the last CTA zeroes the rows up to the next whole tile
+        // a position per thread, eight steps per 16-byte store; the last CTA zeroes the rows up to the next
+        // whole tile
         const size_t arr = (size_t)rows_tot * 2 * BMAX;
         __nv_bfloat16* Pl = P + (size_t)l * kPackArrays * arr;
-        const int sp = 2 * (lane & 15);
         const int end = rank == CS - 1 ? (n0 + kPackTile - 1) / kPackTile * kPackTile - rank * S : n_own;
-        for (int k = 2 * warp + (lane >> 4); k < end; k += 2 * NW) {
-            __nv_bfloat162 u[3], z[3];
-            __nv_bfloat16 pa[3], pb[3];
+        for (int k = tid; k < end; k += STEP_THREADS) {
             const bool in = k < n_own;
-            split_bf16x3(in && sp < nsteps ? sU[(size_t)sp * Sp + k] : 0.f, pa);
-            split_bf16x3(in && sp + 1 < nsteps ? sU[(size_t)(sp + 1) * Sp + k] : 0.f, pb);
+            uint4* o = reinterpret_cast<uint4*>(Pl + (size_t)(rank * S + k) * 2 * BMAX);
+#pragma unroll 1
+            for (int g = 0; g < BMAX / 8; ++g) {
+                union { __nv_bfloat162 h[4]; uint4 v; } u[3], z[3];
 #pragma unroll
-            for (int x = 0; x < 3; ++x) u[x] = __nv_bfloat162(pa[x], pb[x]);
-            split_bf16x3(in && sp < nsteps ? sZ[(size_t)sp * Sp + k] : 0.f, pa);
-            split_bf16x3(in && sp + 1 < nsteps ? sZ[(size_t)(sp + 1) * Sp + k] : 0.f, pb);
-#pragma unroll
-            for (int x = 0; x < 3; ++x) z[x] = __nv_bfloat162(pa[x], pb[x]);
-            __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(Pl + (size_t)(rank * S + k) * 2 * BMAX + sp);
-            o[0] = u[0];       o[BMAX / 2] = u[1];
-            o += arr / 2;
-            o[0] = u[2];       o[BMAX / 2] = z[2];
-            o += arr / 2;
-            o[0] = z[0];       o[BMAX / 2] = z[1];
+                for (int e = 0; e < 4; ++e) {
+                    const int s0 = 8 * g + 2 * e;
+                    __nv_bfloat162 x[3];
+                    split_bf16x3(in && s0 < nsteps ? sU[(size_t)s0 * Sp + k] : 0.f,
+                                 in && s0 + 1 < nsteps ? sU[(size_t)(s0 + 1) * Sp + k] : 0.f, x);
+                    u[0].h[e] = x[0]; u[1].h[e] = x[1]; u[2].h[e] = x[2];
+                    split_bf16x3(in && s0 < nsteps ? sZ[(size_t)s0 * Sp + k] : 0.f,
+                                 in && s0 + 1 < nsteps ? sZ[(size_t)(s0 + 1) * Sp + k] : 0.f, x);
+                    z[0].h[e] = x[0]; z[1].h[e] = x[1]; z[2].h[e] = x[2];
+                }
+                o[g] = u[0].v;                  o[BMAX / 8 + g] = u[1].v;
+                o[arr / 8 + g] = u[2].v;        o[arr / 8 + BMAX / 8 + g] = z[2].v;
+                o[2 * arr / 8 + g] = z[0].v;    o[2 * arr / 8 + BMAX / 8 + g] = z[1].v;
+            }
         }
     }
     if (rank == 0) {
@@ -384,51 +400,82 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     }
     __syncthreads();                           // sU, sZ are done with
 
-    // ---- c_m = (W[:,p_m] - sum_{s<m} c_s T[m][s]) / sqrt(h_m): forward substitution per row
-    //      index i of W, each CTA takes a slice of the d_row indices; every c_m is subtracted from the later
-    //      ones as soon as it is known, so that the chain is one product and two conversions a step.  The
-    //      triangle is widened to float64 once, so that the inner loop is loads and FMAs only.  The solve
-    //      reads this CTA's own shared memory only and runs last, when the per-position state is dead.
+    // ---- c_m = (W[:,p_m] - sum_{s<m} c_s T[m][s]) / sqrt(h_m), forward substitution for every row index i
+    //      of W (each CTA a slice of them), in 8 x 8 blocks on the float64 tensor-core instruction: the four
+    //      diagonal blocks of the 32 x 32 triangle are inverted first, a lane for a column; then a warp takes
+    //      eight row indices: C_b = D_b^-1 W_b, W_q -= T_qb C_b for q > b.  C_b is rounded to fp32, as it is
+    //      stored and applied, before it is used.  (One thread per row index ran 500 FMAs and as many loads
+    //      of straight-line code from a cold instruction cache: 21000 to 36000 clocks a block, a fifth of it.)
+    //      It reads this CTA's own shared memory only and runs last, when the per-position state is dead.
     auto solve_c = [&]() {
+        double (*sD)[9] = reinterpret_cast<double (*)[9]>(sTd + BMAX);     // [32][8]: D_b^-1, row m, column m % 8
         for (int e = tid; e < BMAX * BMAX; e += STEP_THREADS)
-            sTd[e / BMAX][e % BMAX] = (double)sT[e % BMAX][e / BMAX];
+            sTd[e / BMAX][e % BMAX] = e / BMAX < nsteps ? (double)sT[e / BMAX][e % BMAX] : 0.0;
+        __syncthreads();
+        if (warp == 0) {
+            const int b8 = lane & 24, j = lane & 7;
+            double x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                double acc = i == j ? 1.0 : 0.0;
+#pragma unroll
+                for (int k = 0; k < i; ++k) acc = fma(-sTd[b8 + i][b8 + k], x[k], acc);
+                x[i] = i >= j && b8 + i < nsteps ? acc * s_rsm[b8 + i] : 0.0;
+                sD[b8 + i][j] = x[i];
+            }
+        }
         __syncthreads();
         float* Cl = C + (size_t)l * BMAX * rp;
-        const int per = (rp + CS - 1) / CS;
-        for (int i = rank * per + tid; i < min(rp, (rank + 1) * per); i += STEP_THREADS) {
-            double c[BMAX];
+        const size_t arr = (size_t)rows_tot * 2 * BMAX;
+        __nv_bfloat16* Pc = P + (size_t)l * kPackArrays * arr + (size_t)rows_pad * 2 * BMAX;
+        const int gr = lane >> 2, qd = lane & 3;         // accumulator: row gr, columns 2 qd, 2 qd + 1
+        const int per = ((rp + CS - 1) / CS + 7) / 8 * 8;
+        const int i_end = min(rp, (rank + 1) * per);
+        for (int i0 = rank * per + 8 * warp; i0 < i_end; i0 += 8 * NW) {
+            const int i = i0 + 2 * qd;
+            double acc[4][2];
 #pragma unroll
-            for (int m = 0; m < BMAX; ++m)
-                c[m] = (m < nsteps && i < r) ? (double)Wl[(size_t)s_pm[m] * rp + i] : 0.0;
-            float cf[BMAX];
-#pragma unroll
-            for (int s = 0; s < BMAX; ++s) {
-                cf[s] = s < nsteps ? (float)(c[s] * s_rsm[s]) : 0.f;
-                const double cs = (double)cf[s];
-#pragma unroll
-                for (int m = s + 1; m < BMAX; ++m) c[m] = fma(-cs, sTd[s][m], c[m]);
+            for (int b = 0; b < 4; ++b) {
+                const int m = 8 * b + gr;
+                const float* w = Wl + (size_t)s_pm[m < nsteps ? m : 0] * rp + i;
+                acc[b][0] = m < nsteps && i < r ? (double)w[0] : 0.0;
+                acc[b][1] = m < nsteps && i + 1 < r ? (double)w[1] : 0.0;
             }
-            if (compact) {
 #pragma unroll
-                for (int m = 0; m < BMAX; ++m)
-                    if (m < nsteps) Cl[(size_t)m * rp + i] = cf[m];
-            } else {
-                // a row of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest was zeroed
-                // before the first block)
-                const size_t arr = (size_t)rows_tot * 2 * BMAX;
-                uint4* o = reinterpret_cast<uint4*>(P + (size_t)l * kPackArrays * arr + (size_t)(rows_pad + i) * 2 * BMAX);
+            for (int b = 0; b < 4; ++b) {
+                // the block as the second operand: element (k = 4 kk + qd, n = gr) of it
+                auto operand = [&](double v0, double v1, int kk) {
+                    const int from = (4 * kk + qd) * 4 + (gr >> 1);
+                    const double x = __shfl_sync(0xffffffffu, v0, from), y = __shfl_sync(0xffffffffu, v1, from);
+                    return gr & 1 ? y : x;
+                };
+                double c[2] = {0.0, 0.0};
 #pragma unroll
-                for (int g = 0; g < BMAX / 8; ++g) {
-                    union { __nv_bfloat16 h[8]; uint4 v; } x[3];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        __nv_bfloat16 part[3];
-                        split_bf16x3(cf[8 * g + e], part);
-                        x[0].h[e] = part[0]; x[1].h[e] = part[1]; x[2].h[e] = part[2];
+                for (int kk = 0; kk < 2; ++kk)
+                    dmma884(c, sD[8 * b + gr][4 * kk + qd], operand(acc[b][0], acc[b][1], kk));
+                const float c0 = (float)c[0], c1 = (float)c[1];
+                const int m = 8 * b + gr;
+                if (compact) {
+                    if (m < nsteps) {
+                        if (i < rp) Cl[(size_t)m * rp + i] = c0;
+                        if (i + 1 < rp) Cl[(size_t)m * rp + i + 1] = c1;
                     }
-                    o[g] = x[0].v;
-                    o[BMAX / 8 + g] = x[1].v;
-                    o[arr / 8 + g] = x[2].v;
+                } else {
+                    // rows of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest was zeroed
+                    // before the first block)
+                    __nv_bfloat162 x[3];
+                    split_bf16x3(c0, c1, x);
+                    __nv_bfloat16* o = Pc + (size_t)i * 2 * BMAX + m;
+                    if (i < rp) { o[0] = __low2bfloat16(x[0]); o[BMAX] = __low2bfloat16(x[1]); o[arr] = __low2bfloat16(x[2]); }
+                    o += 2 * BMAX;
+                    if (i + 1 < rp) { o[0] = __high2bfloat16(x[0]); o[BMAX] = __high2bfloat16(x[1]); o[arr] = __high2bfloat16(x[2]); }
+                }
+                if (b == 3) break;
+                const double b0 = operand((double)c0, (double)c1, 0), b1 = operand((double)c0, (double)c1, 1);
+#pragma unroll
+                for (int q = b + 1; q < 4; ++q) {
+                    dmma884(acc[q], -sTd[8 * q + gr][8 * b + qd], b0);
+                    dmma884(acc[q], -sTd[8 * q + gr][8 * b + 4 + qd], b1);
                 }
             }
         }
@@ -874,7 +921,7 @@ LazyWs carve_lazy(void* ws, int L, int r, int d, int n_levels) {
 // one position (one per pending step) lie in eight different banks instead of one.
 static int steps_pitch(int S) { return round_up_int(S, 32) + 4; }
 static int steps_smem(int S) {
-    const int b = 2 * BMAX * steps_pitch(S) * (int)sizeof(float), t = BMAX * BMAX * (int)sizeof(double);
+    const int b = 2 * BMAX * steps_pitch(S) * (int)sizeof(float), t = BMAX * (BMAX + 4 + 9) * (int)sizeof(double);
     return b > t ? b : t;
 }
 
@@ -986,9 +1033,11 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
                              dead_after * kDeadFraction >= npos || npos <= 1) ? 1 : 0;
         {
             PhaseScope ps(PH_LAZY_STEPS, st);
-            // smallest cluster whose per-CTA slice of positions fits shared memory
+            // Up to four CTAs as long as a CTA has more than 256 positions: the pending terms of a step are
+            // bound by shared-memory bandwidth, 48 clocks per pending step and 768 positions, which outweighs
+            // the exchange.  More only where a slice would not fit shared memory: they hold whole SMs.
             int cs = 1;
-            while (cs < CLUSTER_MAX && round_up_int((npos + cs - 1) / cs, 4) > SLICE_MAX) cs *= 2;
+            while (cs < CLUSTER_MAX && (npos + cs - 1) / cs > (cs < 4 ? 256 : SLICE_MAX)) cs *= 2;
             const int S = round_up_int((npos + cs - 1) / cs, 4);
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(L * cs);
