@@ -358,32 +358,25 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                 Zl[(size_t)s * d + k] = sZ[(size_t)s * Sp + k];
             }
     } else {
-        // a position per thread, eight steps per 16-byte store; the last CTA zeroes the rows up to the next
-        // whole tile
+        // two positions per warp, two steps per lane: 64-byte pieces (a position per thread with 16-byte stores
+        // touches 32 lines an instruction and takes 1.7 times as long); the last CTA zeroes the rows up to the
+        // next whole tile
         const size_t arr = (size_t)rows_tot * 2 * BMAX;
         __nv_bfloat16* Pl = P + (size_t)l * kPackArrays * arr;
+        const int sp = 2 * (lane & 15);
         const int end = rank == CS - 1 ? (n0 + kPackTile - 1) / kPackTile * kPackTile - rank * S : n_own;
-        for (int k = tid; k < end; k += STEP_THREADS) {
-            const bool in = k < n_own;
-            uint4* o = reinterpret_cast<uint4*>(Pl + (size_t)(rank * S + k) * 2 * BMAX);
-#pragma unroll 1
-            for (int g = 0; g < BMAX / 8; ++g) {
-                union { __nv_bfloat162 h[4]; uint4 v; } u[3], z[3];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int s0 = 8 * g + 2 * e;
-                    __nv_bfloat162 x[3];
-                    split_bf16x3(in && s0 < nsteps ? sU[(size_t)s0 * Sp + k] : 0.f,
-                                 in && s0 + 1 < nsteps ? sU[(size_t)(s0 + 1) * Sp + k] : 0.f, x);
-                    u[0].h[e] = x[0]; u[1].h[e] = x[1]; u[2].h[e] = x[2];
-                    split_bf16x3(in && s0 < nsteps ? sZ[(size_t)s0 * Sp + k] : 0.f,
-                                 in && s0 + 1 < nsteps ? sZ[(size_t)(s0 + 1) * Sp + k] : 0.f, x);
-                    z[0].h[e] = x[0]; z[1].h[e] = x[1]; z[2].h[e] = x[2];
-                }
-                o[g] = u[0].v;                  o[BMAX / 8 + g] = u[1].v;
-                o[arr / 8 + g] = u[2].v;        o[arr / 8 + BMAX / 8 + g] = z[2].v;
-                o[2 * arr / 8 + g] = z[0].v;    o[2 * arr / 8 + BMAX / 8 + g] = z[1].v;
-            }
+#pragma unroll 2
+        for (int k = 2 * warp + (lane >> 4); k < end; k += 2 * NW) {
+            const bool i0 = k < n_own && sp < nsteps, i1 = k < n_own && sp + 1 < nsteps;
+            __nv_bfloat162 u[3], z[3];
+            split_bf16x3(i0 ? sU[(size_t)sp * Sp + k] : 0.f, i1 ? sU[(size_t)(sp + 1) * Sp + k] : 0.f, u);
+            split_bf16x3(i0 ? sZ[(size_t)sp * Sp + k] : 0.f, i1 ? sZ[(size_t)(sp + 1) * Sp + k] : 0.f, z);
+            __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(Pl + (size_t)(rank * S + k) * 2 * BMAX + sp);
+            o[0] = u[0];       o[BMAX / 2] = u[1];
+            o += arr / 2;
+            o[0] = u[2];       o[BMAX / 2] = z[2];
+            o += arr / 2;
+            o[0] = z[0];       o[BMAX / 2] = z[1];
         }
     }
     if (rank == 0) {
@@ -431,51 +424,61 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         const int gr = lane >> 2, qd = lane & 3;         // accumulator: row gr, columns 2 qd, 2 qd + 1
         const int per = ((rp + CS - 1) / CS + 7) / 8 * 8;
         const int i_end = min(rp, (rank + 1) * per);
-        for (int i0 = rank * per + 8 * warp; i0 < i_end; i0 += 8 * NW) {
-            const int i = i0 + 2 * qd;
-            double acc[4][2];
+        constexpr int NT = 3;                            // tiles of eight row indices side by side
+        for (int i0 = rank * per + 8 * warp; i0 < i_end; i0 += 8 * NW * NT) {
+            double acc[NT][4][2];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int m = 8 * b + gr;
-                const float* w = Wl + (size_t)s_pm[m < nsteps ? m : 0] * rp + i;
-                acc[b][0] = m < nsteps && i < r ? (double)w[0] : 0.0;
-                acc[b][1] = m < nsteps && i + 1 < r ? (double)w[1] : 0.0;
-            }
+            for (int t = 0; t < NT; ++t)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                // the block as the second operand: element (k = 4 kk + qd, n = gr) of it
-                auto operand = [&](double v0, double v1, int kk) {
-                    const int from = (4 * kk + qd) * 4 + (gr >> 1);
-                    const double x = __shfl_sync(0xffffffffu, v0, from), y = __shfl_sync(0xffffffffu, v1, from);
-                    return gr & 1 ? y : x;
-                };
-                double c[2] = {0.0, 0.0};
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
-                    dmma884(c, sD[8 * b + gr][4 * kk + qd], operand(acc[b][0], acc[b][1], kk));
-                const float c0 = (float)c[0], c1 = (float)c[1];
-                const int m = 8 * b + gr;
-                if (compact) {
-                    if (m < nsteps) {
-                        if (i < rp) Cl[(size_t)m * rp + i] = c0;
-                        if (i + 1 < rp) Cl[(size_t)m * rp + i + 1] = c1;
-                    }
-                } else {
-                    // rows of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest was zeroed
-                    // before the first block)
-                    __nv_bfloat162 x[3];
-                    split_bf16x3(c0, c1, x);
-                    __nv_bfloat16* o = Pc + (size_t)i * 2 * BMAX + m;
-                    if (i < rp) { o[0] = __low2bfloat16(x[0]); o[BMAX] = __low2bfloat16(x[1]); o[arr] = __low2bfloat16(x[2]); }
-                    o += 2 * BMAX;
-                    if (i + 1 < rp) { o[0] = __high2bfloat16(x[0]); o[BMAX] = __high2bfloat16(x[1]); o[arr] = __high2bfloat16(x[2]); }
+                for (int b = 0; b < 4; ++b) {
+                    const int i = i0 + 8 * NW * t + 2 * qd, m = 8 * b + gr;
+                    const float* w = Wl + (size_t)s_pm[m < nsteps ? m : 0] * rp + i;
+                    acc[t][b][0] = m < nsteps && i < r && i < i_end ? (double)w[0] : 0.0;
+                    acc[t][b][1] = m < nsteps && i + 1 < r && i < i_end ? (double)w[1] : 0.0;
                 }
-                if (b == 3) break;
-                const double b0 = operand((double)c0, (double)c1, 0), b1 = operand((double)c0, (double)c1, 1);
+            // a block as the second operand: element (k = 4 kk + qd, n = gr) of it
+            auto operand = [&](double v0, double v1, int kk) {
+                const int from = (4 * kk + qd) * 4 + (gr >> 1);
+                const double x = __shfl_sync(0xffffffffu, v0, from), y = __shfl_sync(0xffffffffu, v1, from);
+                return gr & 1 ? y : x;
+            };
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const double d0 = sD[8 * b + gr][qd], d1 = sD[8 * b + gr][4 + qd];
+                double tq[3][2];
 #pragma unroll
                 for (int q = b + 1; q < 4; ++q) {
-                    dmma884(acc[q], -sTd[8 * q + gr][8 * b + qd], b0);
-                    dmma884(acc[q], -sTd[8 * q + gr][8 * b + 4 + qd], b1);
+                    tq[q - 1][0] = -sTd[8 * q + gr][8 * b + qd];
+                    tq[q - 1][1] = -sTd[8 * q + gr][8 * b + 4 + qd];
+                }
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    double c[2] = {0.0, 0.0};
+                    dmma884(c, d0, operand(acc[t][b][0], acc[t][b][1], 0));
+                    dmma884(c, d1, operand(acc[t][b][0], acc[t][b][1], 1));
+                    const float c0 = (float)c[0], c1 = (float)c[1];
+                    const int i = i0 + 8 * NW * t + 2 * qd, m = 8 * b + gr;
+                    if (i < i_end) {                     // (rp and the slices are even)
+                        if (compact) {
+                            if (m < nsteps) *reinterpret_cast<float2*>(Cl + (size_t)m * rp + i) = make_float2(c0, c1);
+                        } else {
+                            // rows of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest
+                            // was zeroed before the first block)
+                            __nv_bfloat162 x[3];
+                            split_bf16x3(c0, c1, x);
+                            __nv_bfloat16* o = Pc + (size_t)i * 2 * BMAX + m;
+                            o[0] = __low2bfloat16(x[0]); o[BMAX] = __low2bfloat16(x[1]); o[arr] = __low2bfloat16(x[2]);
+                            o += 2 * BMAX;
+                            o[0] = __high2bfloat16(x[0]); o[BMAX] = __high2bfloat16(x[1]); o[arr] = __high2bfloat16(x[2]);
+                        }
+                    }
+                    if (b == 3) continue;
+                    const double b0 = operand((double)c0, (double)c1, 0), b1 = operand((double)c0, (double)c1, 1);
+#pragma unroll
+                    for (int q = b + 1; q < 4; ++q) {
+                        dmma884(acc[t][q], tq[q - 1][0], b0);
+                        dmma884(acc[t][q], tq[q - 1][1], b1);
+                    }
                 }
             }
         }
