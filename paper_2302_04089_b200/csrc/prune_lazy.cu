@@ -202,6 +202,8 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     }
     int first_bad = ZIPLM_OK;                  // meaningful in lane 0 of the last warp
     bool failed = false;
+    // row indices of W that this CTA solves for
+    const int w_per = ((rp + CS - 1) / CS + 7) / 8 * 8, w_first = rank * w_per, w_end = min(rp, w_first + w_per);
 
     for (int m = 0; m < nsteps; ++m) {
         const int par = m & 1;
@@ -294,6 +296,9 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         const float *pu = sU + p, *pz = sZ + p;    // pending entries of one CTA: in its own slice
         if (warp == NW - 1) {                      // (the last warp: the others may own more positions)
             sT[m][lane] = lane < m ? (MULTI ? pend[lane].x : pu[(size_t)lane * Sp]) : 0.f;
+            // this CTA's part of the pivot column of W, which the end of the block reads, on its way to L2
+            for (int i = w_first + 32 * lane; i < w_end; i += 1024)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(Wl + (size_t)p * rp + i));
             if (lane == 0) {
                 s_pm[m] = p;
                 s_rsm[m] = rs;
@@ -422,19 +427,18 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         const size_t arr = (size_t)rows_tot * 2 * BMAX;
         __nv_bfloat16* Pc = P + (size_t)l * kPackArrays * arr + (size_t)rows_pad * 2 * BMAX;
         const int gr = lane >> 2, qd = lane & 3;         // accumulator: row gr, columns 2 qd, 2 qd + 1
-        const int per = ((rp + CS - 1) / CS + 7) / 8 * 8;
-        const int i_end = min(rp, (rank + 1) * per);
         constexpr int NT = 3;                            // tiles of eight row indices side by side
-        for (int i0 = rank * per + 8 * warp; i0 < i_end; i0 += 8 * NW * NT) {
+        for (int i0 = w_first + 8 * warp; i0 < w_end; i0 += 8 * NW * NT) {
             double acc[NT][4][2];
 #pragma unroll
             for (int t = 0; t < NT; ++t)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    const int i = i0 + 8 * NW * t + 2 * qd, m = 8 * b + gr;
-                    const float* w = Wl + (size_t)s_pm[m < nsteps ? m : 0] * rp + i;
-                    acc[t][b][0] = m < nsteps && i < r && i < i_end ? (double)w[0] : 0.0;
-                    acc[t][b][1] = m < nsteps && i + 1 < r && i < i_end ? (double)w[1] : 0.0;
+                    // (rows are zero from r to rp; what lies past the slice or the last step is not used)
+                    const int i = min(i0 + 8 * NW * t + 2 * qd, rp - 2), m = 8 * b + gr;
+                    const float2 w = *reinterpret_cast<const float2*>(Wl + (size_t)s_pm[min(m, nsteps - 1)] * rp + i);
+                    acc[t][b][0] = m < nsteps ? (double)w.x : 0.0;
+                    acc[t][b][1] = m < nsteps ? (double)w.y : 0.0;
                 }
             // a block as the second operand: element (k = 4 kk + qd, n = gr) of it
             auto operand = [&](double v0, double v1, int kk) {
@@ -458,7 +462,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                     dmma884(c, d1, operand(acc[t][b][0], acc[t][b][1], 1));
                     const float c0 = (float)c[0], c1 = (float)c[1];
                     const int i = i0 + 8 * NW * t + 2 * qd, m = 8 * b + gr;
-                    if (i < i_end) {                     // (rp and the slices are even)
+                    if (i < w_end) {                     // (rp and the slices are even)
                         if (compact) {
                             if (m < nsteps) *reinterpret_cast<float2*>(Cl + (size_t)m * rp + i) = make_float2(c0, c1);
                         } else {
