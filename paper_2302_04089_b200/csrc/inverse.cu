@@ -16,6 +16,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "inverse_i8.cuh"
 
 // Built-in scratch of ziplm_damped_inverse_noalloc: lives in every GPU that loads this library
 // until the process exits.  In host code this name is only a handle for cudaGetSymbolAddress,
@@ -173,10 +174,11 @@ __device__ __forceinline__ void lower_macro_index(int idx, int T, int& I, int& J
 }
 
 
+// eq (may be null): powers of two that bring the diagonal of the damped matrix to [1, 4).
 // lambda[l] = damp_frac * mean(diag H[l]); flags non-finite diagonals and non-positive means.
 __global__ void __launch_bounds__(256) k_mean_diag(const float* __restrict__ H, int d,
                                                    float damp_frac, double* __restrict__ lam,
-                                                   int* layer_status) {
+                                                   double* __restrict__ eq, int* layer_status) {
     const int l = blockIdx.x;
     const float* Hl = H + (size_t)l * d * d;
     double s = 0.0;
@@ -208,12 +210,23 @@ __global__ void __launch_bounds__(256) k_mean_diag(const float* __restrict__ H, 
             lm = 1.0;
         }
         lam[l] = lm;
+        red[0] = lm;
+    }
+    if (!eq) return;
+    __syncthreads();
+    const double lm = red[0];
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        const int hi = __double2hiint((double)Hl[(size_t)i * d + i] + lm), e = hi >> 20;
+        const int half = (e - 1023) >> 1;
+        eq[(size_t)l * d + i] = e > 0 && e < 2047 ? __hiloint2double((1023 - half) << 20, 0) : 1.0;
     }
 }
 
-// C = H + lambda I on the d x d corner, identity on the padding (dp x dp, float64).
+// C = H + lambda I on the d x d corner, identity on the padding (dp x dp, float64); with eq, rows and columns
+// scaled by it (exactly).
 __global__ void __launch_bounds__(256) k_fill_damped(const float* __restrict__ H, int d, int dp,
                                                      const double* __restrict__ lam,
+                                                     const double* __restrict__ eq,
                                                      double* __restrict__ C, int* layer_status) {
     const int l = blockIdx.z;
     const int row = blockIdx.y * 16 + (threadIdx.x >> 4);
@@ -232,6 +245,7 @@ __global__ void __launch_bounds__(256) k_fill_damped(const float* __restrict__ H
             const float h = Hl[(size_t)row * d + col];
             if (!isfinite(h)) bad = true;
             v = (double)h + (row == col ? lm : 0.0);
+            if (eq) v *= eq[(size_t)l * d + row] * eq[(size_t)l * d + col];
         } else {
             v = (row == col) ? 1.0 : 0.0;
         }
@@ -627,7 +641,14 @@ struct InvCtx {
     int dp, L;
     int* layer_status;
     cudaStream_t st;
+    const double* eq;      // int8 products: equilibration, and two operands in digits (rows and K set per use)
+    I8Operand X, Y;
 };
+
+// Products of blocks of at least eight tiles a side, and M^T M from sixteen tiles on, run on the int8 tensor
+// cores: below, the passes that write the digits and the few 256 x 128 tiles cost what the products save.
+constexpr int kI8Tiles = 8;
+bool uses_i8(int T) { return T >= 2 * kI8Tiles; }
 
 int task_ctas(const GemmTask& t) {
     const int mm = (t.mt + 1) / 2;                           // macro tiles: mm x t.nt
@@ -694,6 +715,39 @@ ziplm_status factor_range(const InvCtx& c, int lo, int hi) {
     const int n1 = mid - lo, n2 = hi - mid;
     ziplm_status s = factor_range(c, lo, mid);
     if (s != ZIPLM_OK) return s;
+    if (c.X.dig && n1 >= kI8Tiles && n2 >= kI8Tiles) {
+        const size_t lay = (size_t)c.dp * c.dp;
+        auto block = [&](double* m, int i, int j) { return m + (size_t)i * kTile * c.dp + (size_t)j * kTile; };
+        auto operand = [&](I8Operand o, int rows, int K) { o.rows = rows * kTile; o.K = K * kTile; return o; };
+        auto product = [&](const I8Operand& x, const I8Operand& y, double* C, double alpha, int beta, int krange,
+                           int lower) {
+            I8Product p = {};
+            p.C = C; p.layer_stride = lay; p.ld = c.dp;
+            p.alpha = alpha; p.beta = beta; p.krange = krange; p.lower = lower;
+            p.layer_status = c.layer_status;
+            return i8_product(x, y, p, c.L, c.st);
+        };
+        {
+            PhaseScope ps(PH_INV_PRODUCTS, c.st);
+            // F21 = A21 M11^T
+            I8Operand x = operand(c.X, n2, n1), y = operand(c.Y, n1, n1);
+            if ((s = i8_digits(x, block(c.A, mid, lo), lay, c.dp, false, false, c.L, c.st)) != ZIPLM_OK) return s;
+            if ((s = i8_digits(y, block(c.M, lo, lo), lay, c.dp, false, true, c.L, c.st)) != ZIPLM_OK) return s;
+            if ((s = product(x, y, block(c.F, mid, lo), 1.0, 0, K_TO_COL, 0)) != ZIPLM_OK) return s;
+            // A22 -= F21 F21^T, scratch (the dead A21 block) = F21 M11
+            if ((s = i8_digits(x, block(c.F, mid, lo), lay, c.dp, false, false, c.L, c.st)) != ZIPLM_OK) return s;
+            if ((s = product(x, x, block(c.A, mid, mid), -1.0, 1, K_ALL, 1)) != ZIPLM_OK) return s;
+            if ((s = i8_digits(y, block(c.M, lo, lo), lay, c.dp, true, true, c.L, c.st)) != ZIPLM_OK) return s;
+            if ((s = product(x, y, block(c.A, mid, lo), 1.0, 0, K_FROM_COL, 0)) != ZIPLM_OK) return s;
+        }
+        if ((s = factor_range(c, mid, hi)) != ZIPLM_OK) return s;
+        PhaseScope ps(PH_INV_PRODUCTS, c.st);
+        // M21 = -M22 scratch
+        I8Operand x = operand(c.X, n2, n2), y = operand(c.Y, n1, n2);
+        if ((s = i8_digits(x, block(c.M, mid, mid), lay, c.dp, false, true, c.L, c.st)) != ZIPLM_OK) return s;
+        if ((s = i8_digits(y, block(c.A, mid, lo), lay, c.dp, true, false, c.L, c.st)) != ZIPLM_OK) return s;
+        return product(x, y, block(c.M, mid, lo), -1.0, 0, K_TO_ROW, 0);
+    }
     GemmTask t;
     // F21 = A21 M11^T   (M11 lower triangular: opB(k,j) = M11[j,k] vanishes for k > j)
     t = GemmTask{c.A, mid, lo, c.M, lo, lo, c.F, mid, lo, n2, n1, n1, 1, 0, 1.0, 0};
@@ -714,28 +768,31 @@ ziplm_status factor_range(const InvCtx& c, int lo, int hi) {
 
 }  // namespace
 
-size_t inverse_workspace_bytes(int L, int d) {
-    const int dp = round_up_int(d, kTile);
-    Carver c(nullptr);
-    c.take<double>((size_t)L * dp * dp);               // A: damped Hessian / Schur complements
-    c.take<double>((size_t)L * dp * dp);               // F: Cholesky factor
-    c.take<double>((size_t)L * dp * dp);               // M: inverse of the factor
-    c.take<double>((size_t)L);                         // lambda
-    return c.off;
-}
-
 namespace {
 
-InvCtx carve_inverse(void* ws, int L, int dp, double** lam) {
+// Carves the workspace; with ws == nullptr it only measures.
+size_t carve_inverse(InvCtx* ctx, double** lam, double** eq, void* ws, int L, int d) {
+    const int dp = round_up_int(d, kTile), T = dp / kTile;
     Carver c(ws);
-    InvCtx ctx = {};
-    ctx.A = c.take<double>((size_t)L * dp * dp);
-    ctx.F = c.take<double>((size_t)L * dp * dp);
-    ctx.M = c.take<double>((size_t)L * dp * dp);
+    ctx->A = c.take<double>((size_t)L * dp * dp);      // damped Hessian / Schur complements
+    ctx->F = c.take<double>((size_t)L * dp * dp);      // off-diagonal blocks of the Cholesky factor
+    ctx->M = c.take<double>((size_t)L * dp * dp);      // inverse of the factor
     *lam = c.take<double>((size_t)L);
-    ctx.dp = dp;
-    ctx.L = L;
-    return ctx;
+    *eq = nullptr;
+    ctx->X = ctx->Y = I8Operand{};
+    if (uses_i8(T)) {
+        const size_t h = (size_t)(T - T / 2) * kTile;  // the widest blocks: both halves of the whole range
+        *eq = c.take<double>((size_t)L * d);
+        for (I8Operand* o : {&ctx->X, &ctx->Y}) {
+            o->dig = c.take<signed char>((size_t)L * 8 * h * h);
+            o->scale = c.take<double>((size_t)L * dp);
+            o->exps = c.take<int>((size_t)L * dp);
+        }
+    }
+    ctx->eq = *eq;
+    ctx->dp = dp;
+    ctx->L = L;
+    return c.off;
 }
 
 // Factorisation of ctx.A and M^T M.
@@ -745,6 +802,20 @@ ziplm_status invert(const InvCtx& ctx, int d, double* out64, float* tri32, int p
     const ziplm_status s = factor_range(ctx, 0, T);
     if (s != ZIPLM_OK) return s;
     PhaseScope ps(PH_INV_LAUUM, ctx.st);
+    if (ctx.X.dig) {
+        // the digits of all of M take the place of the dead A
+        const size_t lay = (size_t)ctx.dp * ctx.dp;
+        I8Operand x = ctx.X;
+        x.dig = reinterpret_cast<signed char*>(ctx.A);
+        x.rows = x.K = ctx.dp;
+        const ziplm_status e = i8_digits(x, ctx.M, lay, ctx.dp, true, true, ctx.L, ctx.st);
+        if (e != ZIPLM_OK) return e;
+        I8Product p = {};
+        p.alpha = 1.0; p.krange = K_FROM_ROW; p.lower = 1;
+        p.d = d; p.eq = ctx.eq; p.out64 = out64; p.tri32 = tri32; p.pitch32 = pitch32; p.rows32 = rows32;
+        p.diag64 = diag64; p.layer_status = ctx.layer_status;
+        return i8_product(x, x, p, ctx.L, ctx.st);
+    }
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lauum, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)kProductSmemBytes));
     k_lauum<<<dim3(lower_macro_count(T), ctx.L), GT, kProductSmemBytes, ctx.st>>>(ctx.M, ctx.dp, T, d, out64, tri32,
@@ -755,13 +826,22 @@ ziplm_status invert(const InvCtx& ctx, int d, double* out64, float* tri32, int p
 
 }  // namespace
 
+size_t inverse_workspace_bytes(int L, int d) {
+    InvCtx ctx = {};
+    double *lam, *eq;
+    return carve_inverse(&ctx, &lam, &eq, nullptr, L, d);
+}
+
 double* inverse_matrix(void* ws) { return static_cast<double*>(ws); }     // the first piece of the workspace
 
 ziplm_status run_inverse_of(void* ws, int L, int d, double* out64, int* layer_status, cudaStream_t st) {
-    double* lam;
-    InvCtx ctx = carve_inverse(ws, L, round_up_int(d, kTile), &lam);
+    InvCtx ctx = {};
+    double *lam, *eq;
+    carve_inverse(&ctx, &lam, &eq, ws, L, d);
     ctx.layer_status = layer_status;
     ctx.st = st;
+    ctx.eq = nullptr;
+    ctx.X.dig = nullptr;               // the caller's matrix is not equilibrated
     return invert(ctx, d, out64, nullptr, 0, 0, nullptr);
 }
 
@@ -769,14 +849,14 @@ ziplm_status run_damped_inverse(const float* H, int L, int d, float damp_frac, d
                                 float* tri32, int pitch32, int rows32, double* diag64, double* lam_out,
                                 int* layer_status, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (ws_bytes < inverse_workspace_bytes(L, d)) return ZIPLM_ERR_WORKSPACE;
-    const int dp = round_up_int(d, kTile), T = dp / kTile;
-    double* lam;
-    InvCtx ctx = carve_inverse(ws, L, dp, &lam);
+    InvCtx ctx = {};
+    double *lam, *eq;
+    carve_inverse(&ctx, &lam, &eq, ws, L, d);
     ctx.layer_status = layer_status;
     ctx.st = st;
-    k_mean_diag<<<L, 256, 0, st>>>(H, d, damp_frac, lam, layer_status);
+    k_mean_diag<<<L, 256, 0, st>>>(H, d, damp_frac, lam, eq, layer_status);
     ZIPLM_CHECK_LAUNCH();
-    k_fill_damped<<<dim3(T, dp / 16, L), 256, 0, st>>>(H, d, dp, lam, ctx.A, layer_status);
+    k_fill_damped<<<dim3(ctx.dp / kTile, ctx.dp / 16, L), 256, 0, st>>>(H, d, ctx.dp, lam, eq, ctx.A, layer_status);
     ZIPLM_CHECK_LAUNCH();
     const ziplm_status s = invert(ctx, d, out64, tri32, pitch32, rows32, diag64);
     if (s != ZIPLM_OK) return s;

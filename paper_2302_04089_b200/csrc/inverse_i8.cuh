@@ -1,0 +1,37 @@
+// Float64 products on the int8 tensor cores (inverse_i8.cu), as the factorisation (inverse.cu) uses them.
+#pragma once
+
+#include "common.cuh"
+
+namespace ziplm {
+
+// An operand in digits: [L][8][rows][K] int8, a power-of-two scale per row (and room for exponents).
+struct I8Operand {
+    signed char* dig;
+    double* scale;       // [L][rows]
+    int* exps;           // [L][rows]
+    int rows, K;         // multiples of 64
+};
+
+// Which part of K a tile needs: all, up to its last row / column, from its first row / column on.
+enum KRange { K_ALL = 0, K_TO_COL, K_TO_ROW, K_FROM_COL, K_FROM_ROW };
+
+// C[row][col] = beta C + alpha sum_k x[row][k] y[col][k]; with C == nullptr the result is H^-1 = M^T M,
+// cropped to d x d and with the equilibration `eq` ([L][d] powers of two, or null) taken back.
+struct I8Product {
+    double* C; size_t layer_stride; int ld;
+    double alpha; int beta;
+    int krange, lower;                       // lower: only tiles that reach the lower triangle
+    int d; const double* eq; double* out64; float* tri32; int pitch32, rows32; double* diag64;
+    int* layer_status;
+    int rows, cols, K;                       // set by i8_product
+    const double* x_scale; const double* y_scale;
+};
+
+// Digits of a block of a float64 matrix (leading dimension ld): operand rows are its rows, or its columns.
+// tri: block of a lower triangular matrix whose tiles above the diagonal are not written.
+ziplm_status i8_digits(const I8Operand& o, const double* src, size_t layer_stride, int ld, bool columns, bool tri,
+                       int L, cudaStream_t st);
+ziplm_status i8_product(const I8Operand& x, const I8Operand& y, I8Product p, int L, cudaStream_t st);
+
+}  // namespace ziplm

@@ -823,3 +823,26 @@ def test_hessian_small_calls_on_clusters_match_oracle(dtype, d, N, L):
         assert np.max(np.abs(H[l].cpu().double().numpy() - Ho) / scale) < 2e-6
         assert np.max(np.abs(H2[l].cpu().double().numpy() - 2 * Ho) / scale) < 4e-6
         assert torch.equal(H2[l], H2[l].t())
+
+
+@pytest.mark.parametrize("d,L,spread", [(1024, 1, 0.0), (1089, 2, 1.0), (1500, 1, 3.0)])
+def test_damped_inverse_on_int8_products_is_as_good_as_float64(d, L, spread):
+    """Widths whose large products run in digits on the int8 tensor cores: smallest, ragged tiles, and
+    features of very different scale.  The error, scaled by the diagonal (which takes the features' scales
+    out), is held to the float64 bound of the other widths."""
+    z = zb()
+    g = torch.Generator().manual_seed(d)
+    X = torch.randn(L, d, 2 * d, generator=g, dtype=torch.float64) * \
+        torch.exp(spread * torch.randn(L, d, 1, generator=g, dtype=torch.float64))
+    H = (2.0 * X @ X.transpose(1, 2)).float()
+    Hinv, status = z.damped_inverse(H.cuda(), 0.01)
+    torch.cuda.synchronize()
+    assert status.tolist() == [0] * L
+    for l in range(L):
+        H_lam = zo.damped(H[l].numpy(), float(np.float32(0.01)))[0]
+        s = np.sqrt(np.diag(H_lam))
+        ref = zo.inverse_spd(H_lam / np.outer(s, s))
+        got = Hinv[l].cpu().numpy() * np.outer(s, s)
+        assert np.array_equal(Hinv[l].cpu().numpy(), Hinv[l].cpu().numpy().T)
+        tol = 50 * np.linalg.cond(H_lam / np.outer(s, s)) * 2.2e-16
+        assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) < tol
