@@ -346,8 +346,7 @@ constexpr int PS = kTile + 4;    // pitch of a 64 x 64 operand tile in shared me
 struct SmallSmem {
     double ta[kTile * PS];       // operand tiles, as stored (row-major)
     double tb[kTile * PS];
-    double row[2][kTile + 1];    // leaf: current row and the diagonal entry behind it (double-buffered)
-    double piv[kTile];           // leaf: pivots
+    double blk[16 * 20];         // leaf: inverse factor of the current 16 x 16 diagonal block
     int flag;                    // first error seen by this CTA
 };
 
@@ -413,93 +412,213 @@ __device__ __forceinline__ void small_epilogue(const SmallAcc& acc, Fn f) {
             f(r0 + 8 * i, c0 + 8 * j, make_double2(acc.d[i][j][0], acc.d[i][j][1]));
 }
 
-// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg (lower, upper part zeroed).  The factor itself is not needed.  Starts and ends with a barrier.
+// One warp: acc(16 x 16) += A(16 x 16) B(16 x 16), operands in shared memory with pitch PS;
+// BT: B(k,n) = b[n][k], else b[k][n].
+template <bool BT>
+__device__ __forceinline__ void warp_mma16(double (&acc)[2][2][2], const double* a, int lda, const double* b, int ldb) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+        double fa[2], fb[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            fa[i] = a[(8 * i + (lane >> 2)) * lda + 4 * kk + (lane & 3)];
+            fb[i] = BT ? b[(8 * i + (lane >> 2)) * ldb + 4 * kk + (lane & 3)]
+                       : b[(4 * kk + (lane & 3)) * ldb + 8 * i + (lane >> 2)];
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) dmma884(acc[i][j], fa[i], fb[j]);
+    }
+}
+
+// One warp: c(16 x 16) = acc, or c -= acc.
+template <bool SUB>
+__device__ __forceinline__ void warp_put16(const double (&acc)[2][2][2], double* c, int ldc) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            double2* o = reinterpret_cast<double2*>(c + (8 * i + (lane >> 2)) * ldc + 8 * j + 2 * (lane & 3));
+            double2 v = make_double2(acc[i][j][0], acc[i][j][1]);
+            if (SUB) { const double2 x = *o; v.x = x.x - v.x; v.y = x.y - v.y; }
+            *o = v;
+        }
+}
+
+// 1 / x = y0 (1 + e + e^2 + ...), e = 1 - x y0, from the hardware's approximation y0 (relative error
+// below 2^-20, so the terms left out are below 2^-60): y0 and e + e^2.
+__device__ __forceinline__ void reciprocal_terms(double x, double& y0, double& s) {
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double e = fma(-x, y0, 1.0);
+    s = fma(e, e, e);
+}
+
+// One warp: the inverse of the Cholesky factor of an 8 x 8 block (full symmetric), in the lanes as the
+// float64 mma's result: lane 4 i + c holds columns 2 c and 2 c + 1 of row i; lower, zero above.
 // Elimination of [A | I] in place: at column k the rows i > k become
 //     r_ij -= (r_ik / r_kk) r_kj   for all j != k,      r_ik = -r_ik / r_kk,
 // which leaves the Schur complement in the columns j > k and row i of L^-1 (A = L D L^T) in the columns
-// j < i; M = D^-1/2 L^-1.  Threads 0 .. 255 hold the tile in registers, cyclically (rows ty + 16 a,
-// columns tx + 16 b).  The Schur complement is kept in both triangles, so row k is also column k, and a
-// step is one barrier: the half-warp that owns row k publishes it, and every thread forms the next pivot
-// and its reciprocal by itself from the published row and diagonal entry, beside its 16 updates, so that
-// the updates do not wait for a reciprocal.  (The earlier leaf, a Cholesky factor column by column and
-// then its inverse from 16 x 16 blocks, took 37 us; a chain of 64 x (barrier, load, two FMAs, store).)
-__device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp, SmallSmem& sm) {
-    const int tid = threadIdx.x;
-    const int tx = tid & 15, ty = (tid >> 4) & 15;
-    __syncthreads();                          // earlier readers of the shared arrays are done
-    if (tid < 256) {
-        double r[4][4];
+// j < i; the result is D^-1/2 L^-1.  Returns the row's pivot.
+// The chain is that of the pivots, p_{k+1} = a_{k+1,k+1} - a_{k+1,k}^2 / p_k: every lane runs it on its
+// own, from the two entries as they were before column k, so that a column costs it a reciprocal and four
+// FMAs and the shuffles of the rows run beside it.
+__device__ __forceinline__ double warp_factor8(double (&r)[2]) {
+    const int lane = threadIdx.x & 31, i = lane >> 2, c = lane & 3;
+    double p = __shfl_sync(0xffffffffu, r[0], 0), piv = p;
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                // the lower triangle is the valid one
-                const int i = ty + 16 * a, j = tx + 16 * b;
-                r[a][b] = Ag[i >= j ? (size_t)i * dp + j : (size_t)j * dp + i];
-            }
-        int flag = 0;
-        auto pivot = [&](double p) {
-            if (!(p > 0.0) || !isfinite(p)) {   // not positive definite (or NaN): flag, keep going
-                if (!flag) flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
-                p = 1.0;
-            }
-            return p;
-        };
-        auto barrier = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-        if (tid == 0) sm.row[1][kTile] = r[0][0];
-        barrier();
-        double p = pivot(sm.row[1][kTile]), rp = __drcp_rn(p);
-#pragma unroll
-        for (int kb = 0; kb < 4; ++kb) {
-#pragma unroll 1
-            for (int kt = 0; kt < 16; ++kt) {
-                const int k = 16 * kb + kt;
-                double* v = sm.row[k & 1];
-                if (ty == kt) {
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) v[tx + 16 * b] = r[kb][b];
-                }
-                if (kt < 15) {
-                    if (tx == kt + 1 && ty == kt + 1) v[kTile] = r[kb][kb];
-                } else if (tid == 0) {
-                    v[kTile] = kb < 3 ? r[kb < 3 ? kb + 1 : 3][kb < 3 ? kb + 1 : 3] : 1.0;
-                }
-                if (tid == 0) sm.piv[k] = p;
-                barrier();
-                double vi[4], vj[4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) { vi[a] = v[ty + 16 * a]; vj[a] = v[tx + 16 * a]; }
-                const double vn = k + 1 < kTile ? v[k + 1] : 0.0;
-                const double p_next = pivot(fma(-(vn * rp), vn, v[kTile]));
-                const double rp_next = __drcp_rn(p_next);
-#pragma unroll
-                for (int a = kb; a < 4; ++a) {                   // the rows behind k
-                    if (a == kb && ty <= kt) continue;
-                    const double f = vi[a] * rp;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const double x = fma(-f, vj[b], r[a][b]);
-                        r[a][b] = (b == kb && tx == kt) ? -f : x;
-                    }
-                }
-                p = p_next;
-                rp = rp_next;
-            }
+    for (int k = 0; k < 8; ++k) {
+        double y0, s;
+        const double rik = __shfl_sync(0xffffffffu, r[k & 1], (lane & 28) + (k >> 1));
+        reciprocal_terms(p, y0, s);
+        double next = 1.0;
+        if (k < 7) {
+            const int n = k + 1;
+            const double off = __shfl_sync(0xffffffffu, r[k & 1], 4 * n + (k >> 1));
+            const double dia = __shfl_sync(0xffffffffu, r[n & 1], 4 * n + (n >> 1));
+            const double t = off * y0;
+            next = fma(-fma(t, s, t), off, dia);
         }
-        if (tid == 0 && flag && !sm.flag) sm.flag = flag;
-        barrier();
+        const double t = i > k ? rik * y0 : 0.0;
+        const double f = fma(t, s, t);
+        const double rk0 = __shfl_sync(0xffffffffu, r[0], 4 * k + c);
+        const double rk1 = __shfl_sync(0xffffffffu, r[1], 4 * k + c);
+        r[0] = fma(-f, rk0, r[0]);
+        r[1] = fma(-f, rk1, r[1]);
+        if (c == (k >> 1) && i > k) r[k & 1] = -f;
+        p = next;
+        if (i == k + 1) piv = next;
+    }
+    const double sc = rsqrt(piv);
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int i = ty + 16 * a;
-            const double sc = rsqrt(sm.piv[i]);
+    for (int e = 0; e < 2; ++e) r[e] = 2 * c + e < i ? r[e] * sc : 2 * c + e == i ? sc : 0.0;
+    return piv;
+}
+
+// One warp: d += x y^T of 8 x 8 blocks held as above.  The k order of the two mma steps is free, so
+// columns 2 c go into the first and columns 2 c + 1 into the second, and no operand changes lanes.
+__device__ __forceinline__ void warp_mma8(double (&d)[2], const double (&x)[2], const double (&y)[2]) {
+    dmma884(d, x[0], y[0]);
+    dmma884(d, x[1], y[1]);
+}
+
+// One warp: the inverse of the Cholesky factor of the 16 x 16 block at a (its lower triangle; the diagonal
+// 8 x 8 blocks in full; pitch lda) -> out (lower, pitch PB; zero above).  Two 8 x 8 eliminations and seven
+// 8 x 8 products in registers: the shuffles of a column are 5 instead of the 11 of a 16 x 16 elimination,
+// whose columns took 308 clocks.
+constexpr int PB = 20;
+__device__ __forceinline__ int warp_factor16(const double* a, int lda, double* out) {
+    const int lane = threadIdx.x & 31, i = lane >> 2, c = lane & 3;
+    auto load = [&](double (&r)[2], int bi, int bj) {
+        const double2 v = *reinterpret_cast<const double2*>(a + (8 * bi + i) * lda + 8 * bj + 2 * c);
+        r[0] = v.x;
+        r[1] = v.y;
+    };
+    auto store = [&](const double (&r)[2], int bi, int bj) {
+        *reinterpret_cast<double2*>(out + (8 * bi + i) * PB + 8 * bj + 2 * c) = make_double2(r[0], r[1]);
+    };
+    double m1[2], a21[2], m2[2];
+    load(m1, 0, 0);
+    load(a21, 1, 0);
+    load(m2, 1, 1);
+    const double p1 = warp_factor8(m1);
+    double l21[2] = {0.0, 0.0}, t[2] = {0.0, 0.0};
+    warp_mma8(l21, a21, m1);                                 // L21 = A21 M11^T
+    warp_mma8(t, l21, l21);                                  // A22 - L21 L21^T
+    m2[0] -= t[0];
+    m2[1] -= t[1];
+    double m1t[2], x[2] = {0.0, 0.0}, m21[2] = {0.0, 0.0};
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int j = tx + 16 * b;
-                const double x = j < i ? r[a][b] * sc : j == i ? sc : 0.0;
-                Mg[(size_t)i * dp + j] = x;
-            }
+    for (int e = 0; e < 2; ++e) {                            // M11^T
+        const double u = __shfl_sync(0xffffffffu, m1[0], 4 * (2 * c + e) + (i >> 1));
+        const double v = __shfl_sync(0xffffffffu, m1[1], 4 * (2 * c + e) + (i >> 1));
+        m1t[e] = i & 1 ? v : u;
+    }
+    warp_mma8(x, m1t, l21);                                  // (L21 M11)^T
+    const double p2 = warp_factor8(m2);
+    warp_mma8(m21, m2, x);                                   // M21 = -M22 (L21 M11)
+    m21[0] = -m21[0];
+    m21[1] = -m21[1];
+    const double zero[2] = {0.0, 0.0};
+    store(m1, 0, 0);
+    store(zero, 0, 1);
+    store(m21, 1, 0);
+    store(m2, 1, 1);
+    const unsigned bad1 = __ballot_sync(0xffffffffu, !(p1 > 0.0) || !isfinite(p1));
+    const unsigned bad2 = __ballot_sync(0xffffffffu, !(p2 > 0.0) || !isfinite(p2));
+    if (!(bad1 | bad2)) return 0;                            // the first bad pivot: not positive definite, or NaN
+    const double bad = __shfl_sync(0xffffffffu, bad1 ? p1 : p2, __ffs(bad1 ? bad1 : bad2) - 1);
+    return isfinite(bad) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
+}
+
+// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg (lower, upper part zeroed).
+// The factor itself is not needed.  Starts and ends with a barrier.
+// The same elimination by 16 x 16 blocks: one warp turns the diagonal block into M_bb, then
+// L_ib = A_ib M_bb^T and X_bj = M_bb X_bj, then A_ik -= L_ib L_kb^T and X_ij -= L_ib X_bj, a warp and 16
+// float64 mma instructions per block.  Warp 0 updates the next diagonal block and goes on with it while
+// the others do the rest: two barriers a block.  15000 clocks, of which 4 x 2200 are the chain of the
+// pivots; column by column on all threads it was 36000, 560 a column (a barrier, ten shared-memory reads
+// and the CTA's instructions on every column's chain).  12 x 1024 inverse 0.87 -> 0.78 ms.
+__device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp, SmallSmem& sm) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __syncthreads();                          // earlier readers of the shared arrays are done
+#pragma unroll
+    for (int e = tid; e < kTile * kTile; e += kSmallThreads) {
+        const int i = e >> 6, j = e & 63;     // the lower triangle is the valid one
+        if (j <= i) {
+            const double v = Ag[(size_t)i * dp + j];
+            sm.ta[i * PS + j] = v;
+            sm.ta[j * PS + i] = v;
+        }
+        sm.tb[i * PS + j] = 0.0;
+    }
+    __syncthreads();
+    auto A = [&](int i, int j) { return sm.ta + 16 * i * PS + 16 * j; };
+    auto X = [&](int i, int j) { return sm.tb + 16 * i * PS + 16 * j; };
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b) {
+        if (warp == 0) {                      // warp 0 updated A_bb itself and goes on without a barrier
+            __syncwarp();
+            const int flag = warp_factor16(A(b, b), PS, sm.blk);
+            if (lane == 0 && flag && !sm.flag) sm.flag = flag;
+        }
+        __syncthreads();
+        const int n = 3 - b;
+        double acc[2][2][2] = {};
+        if (warp < n) {                                       // L_ib, in A's place
+            double* a = A(b + 1 + warp, b);
+            warp_mma16<true>(acc, a, PS, sm.blk, PB);
+            __syncwarp();
+            warp_put16<false>(acc, a, PS);
+        } else if (warp < n + b) {
+            double* x = X(b, warp - n);
+            warp_mma16<false>(acc, sm.blk, PB, x, PS);
+            __syncwarp();
+            warp_put16<false>(acc, x, PS);
+        } else if (warp == 3) {
+            for (int e = lane; e < 256; e += 32) X(b, b)[(e >> 4) * PS + (e & 15)] = sm.blk[(e >> 4) * PB + (e & 15)];
+        }
+        __syncthreads();
+        const int n_a = n * (n + 1) / 2;
+        if (warp < n_a) {
+            int ii = 0, kk = warp;
+            while (kk > ii) { kk -= ii + 1; ++ii; }
+            const int i = b + 1 + ii, k = b + 1 + kk;
+            double c[2][2][2] = {};
+            warp_mma16<true>(c, A(i, b), PS, A(k, b), PS);
+            warp_put16<true>(c, A(i, k), PS);
+        } else if (warp < n_a + n * (b + 1)) {
+            const int q = warp - n_a, i = b + 1 + q / (b + 1), j = q % (b + 1);
+            double c[2][2][2] = {};
+            warp_mma16<false>(c, A(i, b), PS, X(b, j), PS);
+            warp_put16<true>(c, X(i, j), PS);
         }
     }
+#pragma unroll
+    for (int e = tid; e < kTile * kTile; e += kSmallThreads)
+        Mg[(size_t)(e >> 6) * dp + (e & 63)] = sm.tb[(e >> 6) * PS + (e & 63)];
     __syncthreads();
 }
 

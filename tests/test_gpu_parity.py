@@ -846,3 +846,24 @@ def test_damped_inverse_on_int8_products_is_as_good_as_float64(d, L, spread):
         assert np.array_equal(Hinv[l].cpu().numpy(), Hinv[l].cpu().numpy().T)
         tol = 50 * np.linalg.cond(H_lam / np.outer(s, s)) * 2.2e-16
         assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) < tol
+
+
+@pytest.mark.parametrize("d", [1, 7, 8, 9, 17, 40, 64, 65])
+def test_factorisation_leaf_at_the_edges_of_its_blocks(d):
+    """The 8- and 16-column blocks of a 64 x 64 tile: an exact-width inverse, and a matrix that stops
+    being positive definite in each block is reported, one with a NaN as not finite."""
+    z = zb()
+    g = torch.Generator().manual_seed(d)
+    X = torch.randn(d, 3 * d + 4, generator=g, dtype=torch.float64)
+    H = (X @ X.T).float()
+    bad = [k for k in (0, 7, 8, 15, 16, 63, 64) if k < d]
+    batch = H.repeat(2 + len(bad), 1, 1)
+    for q, k in enumerate(bad):
+        batch[1 + q, k, k] = -1.0 - batch[1 + q, k, k]
+    batch[-1, d - 1, d - 1] = float("nan")
+    Hinv, status = z.damped_inverse(batch.cuda(), 0.01)
+    torch.cuda.synchronize()
+    got = status.tolist()
+    assert got[0] == 0 and all(v == got[1] != 0 for v in got[1:-1]) and got[-1] not in (0, got[1])
+    ref = zo.inverse_spd(zo.damped(H.numpy(), float(np.float32(0.01)))[0])
+    assert np.max(np.abs(Hinv[0].cpu().numpy() - ref)) / np.max(np.abs(ref)) < 1e-9
