@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "factor16.cuh"
 
 namespace ziplm {
 namespace {
@@ -36,7 +37,8 @@ template <int G8>
 struct HeadShape {
     static constexpr int g = 8 * G8, CF = G8 / 2, UN = (2 * G8 + 7) / 8, P_KM = g + 4;
     static constexpr int kOperand = KCH * P_KM > g * P_MK ? KCH * P_KM : g * P_MK;     // doubles
-    static constexpr size_t kSmem = sizeof(double) * 4 * kOperand;                     // two stages
+    static constexpr int kScore = g * P_KM + (g + 16) * PB;                            // a head's block, panel
+    static constexpr size_t kSmem = sizeof(double) * (4 * kOperand > kScore ? 4 * kOperand : kScore);   // two stages
 };
 
 template <int G8>
@@ -64,11 +66,6 @@ struct HeadAcc {
         }
     }
 };
-
-__device__ __forceinline__ void h_dmma(double (&d)[2], double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
 
 __device__ __forceinline__ void h_cp16(double* dst, const double* src, bool ok) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
@@ -134,7 +131,7 @@ __device__ __forceinline__ void h_product(HeadAcc<G8>& acc, const double* X, siz
                 if (rf >= G8) continue;
                 const double a = h_frag<G8, XKM>(sx, 8 * rf, kk, lane);
 #pragma unroll
-                for (int j = 0; j < S::CF; ++j) h_dmma(acc.d[u][j], a, b[j]);
+                for (int j = 0; j < S::CF; ++j) dmma884(acc.d[u][j], a, b[j]);
             }
         }
         __syncthreads();
@@ -179,78 +176,99 @@ __device__ __forceinline__ double h_sum(double v, double* red) {
     return t;
 }
 
-// rho of head s of layer l and -(H^-1)[S,S]^-1, from the diagonal blocks of H^-1 and Q: symmetric
-// sweeps a_ij -= a_ik a_kj / a_kk over all k, the block in registers, cyclically over the 16 x 16
-// threads.  A column is one barrier: the half-warp that owns row k publishes it, and every thread forms
-// the next pivot and its reciprocal by itself from the published row and diagonal entry, beside its
-// updates, so that neither waits for the other.  The pivots are those of the Cholesky factorisation.
+// rho of head s of layer l and -(H^-1)[S,S]^-1, from the diagonal blocks of H^-1 and Q.  With M the inverse
+// of the Cholesky factor of B = (H^-1)[S,S]: B^-1 = M^T M.
+// M by elimination of [B | I] in 16 x 16 blocks, in place in shared memory (block (i, j), j < b, of the
+// lower triangle holds X_ij, the others what is left of B): one warp turns the diagonal block into M_bb,
+// then L_ib = B_ib M_bb^T (kept aside) and X_bj = M_bb X_bj, then B_ik -= L_ib L_kb^T, X_ij -= L_ib X_bj
+// and X_ib = -L_ib M_bb, a warp and 16 mma instructions per block; warp 0 updates the next diagonal block
+// and goes on with it while the others do the rest.  The chain is the pivots'.  Heads of 64: 20000 clocks
+// (symmetric sweeps in registers, one barrier per column, took 45000).
 template <int G8>
-__device__ void h_score(const Heads& w, int l, int s, double* red, double (*v)[HeadShape<G8>::g + 1]) {
+__device__ void h_score(const Heads& w, int l, int s, double* red, double* smem) {
     using S = HeadShape<G8>;
-    constexpr int NB = S::g / 16;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    constexpr int NB = S::g / 16, PG = S::P_KM;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double* m = smem;                                     // [g][PG]
+    double* pan = smem + S::g * PG;                       // [g][PB]: L_ib
+    double* blk = pan + S::g * PB;                        // [16][PB]: M_bb
     const size_t at = (size_t)l * w.d * w.d + (size_t)s * S::g * w.d + (size_t)s * S::g;
-    double a[NB][NB];
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) a[i][j] = w.A[at + (size_t)(ty + 16 * i) * w.d + tx + 16 * j];
-    int flag = 0;
-    auto reciprocal = [&](double p) {
-        if (!(p > 0.0) || !isfinite(p)) {          // not positive definite (or NaN): flag, keep going
-            if (!flag) flag = isfinite(p) ? ZIPLM_ERR_NOT_PD : ZIPLM_ERR_NONFINITE;
-            p = 1.0;
-        }
-        return __drcp_rn(p);
-    };
-    if (tid == 0) v[1][S::g] = a[0][0];
+    for (int e = tid; e < S::g * S::g / 2; e += HT) {
+        const int i = e / (S::g / 2), j = 2 * (e % (S::g / 2));
+        *reinterpret_cast<double2*>(m + i * PG + j) =
+            j >> 4 <= i >> 4 ? *reinterpret_cast<const double2*>(w.A + at + (size_t)i * w.d + j) : make_double2(0.0, 0.0);
+    }
     __syncthreads();
-    double rp = reciprocal(v[1][S::g]);
-#pragma unroll
-    for (int kb = 0; kb < NB; ++kb) {
+    auto X = [&](int i, int j) { return m + 16 * i * PG + 16 * j; };
+    int flag = 0;
 #pragma unroll 1
-        for (int kt = 0; kt < 16; ++kt) {
-            const int k = 16 * kb + kt;
-            double* vk = v[k & 1];
-            if (ty == kt) {
-#pragma unroll
-                for (int j = 0; j < NB; ++j) vk[tx + 16 * j] = a[kb][j];
+    for (int b = 0; b < NB; ++b) {
+        if (warp == 0) {
+            __syncwarp();
+            const int f = warp_factor16(X(b, b), PG, blk);
+            if (!flag) flag = f;
+        }
+        __syncthreads();
+        const int n = NB - 1 - b;
+        for (int q = warp; q < NB; q += HT / 32) {
+            double c[2][2][2] = {};
+            if (q < n) {
+                warp_mma16<true>(c, X(b + 1 + q, b), PG, blk, PB);
+                warp_put16<false>(c, pan + 16 * (b + 1 + q) * PB, PB);
+            } else if (q < n + b) {
+                double* x = X(b, q - n);
+                warp_mma16<false>(c, blk, PB, x, PG);
+                __syncwarp();
+                warp_put16<false>(c, x, PG);
+            } else {
+                for (int e = lane; e < 256; e += 32) X(b, b)[(e >> 4) * PG + (e & 15)] = blk[(e >> 4) * PB + (e & 15)];
             }
-            // the diagonal entry behind the pivot
-            if (kt < 15) {
-                if (tx == kt + 1 && ty == kt + 1) vk[S::g] = a[kb][kb];
-            } else if (tid == 0) {
-                vk[S::g] = kb + 1 < NB ? a[kb + 1 < NB ? kb + 1 : kb][kb + 1 < NB ? kb + 1 : kb] : 1.0;
-            }
-            __syncthreads();
-            double vi[NB], vj[NB];
+        }
+        __syncthreads();
+        const int n_a = n * (n + 1) / 2, n_all = n_a + n * (b + 1);
+        for (int q = warp; q < n_all; q += warp == 0 ? n_all : HT / 32 - 1) {
+            double c[2][2][2] = {};
+            if (q < n_a) {
+                int ii, kk;
+                pair_index(q, ii, kk);
+                const int i = b + 1 + ii, k = b + 1 + kk;
+                warp_mma16<true>(c, pan + 16 * i * PB, PB, pan + 16 * k * PB, PB);
+                warp_put16<true>(c, X(i, k), PG);
+            } else {
+                const int i = b + 1 + (q - n_a) / (b + 1), j = (q - n_a) % (b + 1);
+                warp_mma16<false>(c, pan + 16 * i * PB, PB, X(b, j), PG);
+                if (j == b) {
 #pragma unroll
-            for (int i = 0; i < NB; ++i) { vi[i] = vk[ty + 16 * i]; vj[i] = vk[tx + 16 * i]; }
-            const double vn = k + 1 < S::g ? vk[k + 1] : 0.0;
-            const double rp_next = reciprocal(fma(-(vn * rp), vn, vk[S::g]));
-#pragma unroll
-            for (int i = 0; i < NB; ++i) {
-                const double f = vi[i] * rp;
-                const bool row = i == kb && ty == kt;
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const bool col = j == kb && tx == kt;
-                    const double upd = fma(-f, vj[j], a[i][j]);
-                    a[i][j] = row ? (col ? -rp : vj[j] * rp) : (col ? f : upd);
+                    for (int e = 0; e < 8; ++e) c[e >> 2][(e >> 1) & 1][e & 1] = -c[e >> 2][(e >> 1) & 1][e & 1];
+                    warp_put16<false>(c, X(i, j), PG);
+                } else {
+                    warp_put16<true>(c, X(i, j), PG);
                 }
             }
-            rp = rp_next;
+        }
+    }
+    // B^-1 = M^T M: both operands are M stored by k, whose rows above a column's are zero
+    HeadAcc<G8> acc;
+    acc.zero();
+#pragma unroll
+    for (int u = 0; u < S::UN; ++u) {
+        const int rf = (warp + 8 * u) >> 1;
+        if (rf >= G8) continue;
+#pragma unroll 2
+        for (int kk = 2 * max(rf, (warp & 1) * S::CF); kk < S::g / 4; ++kk) {
+            const double a = m[(kk * 4 + (lane & 3)) * PG + 8 * rf + (lane >> 2)];
+#pragma unroll
+            for (int j = 0; j < S::CF; ++j)
+                dmma884(acc.d[u][j], a, m[(kk * 4 + (lane & 3)) * PG + 8 * ((warp & 1) * S::CF + j) + (lane >> 2)]);
         }
     }
     double part = 0.0;
     double* B = w.Bneg + ((size_t)l * w.G + s) * S::g * S::g;
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            B[(ty + 16 * i) * S::g + tx + 16 * j] = a[i][j];
-            part = fma(-a[i][j], w.Q[at + (size_t)(ty + 16 * i) * w.d + tx + 16 * j], part);
-        }
+    acc.visit([&](int i, int j, double2 x) {
+        const double2 q = *reinterpret_cast<const double2*>(w.Q + at + (size_t)i * w.d + j);
+        *reinterpret_cast<double2*>(B + i * S::g + j) = make_double2(-x.x, -x.y);
+        part = fma(x.x, q.x, fma(x.y, q.y, part));
+    });
     const double rho = h_sum(part, red);
     if (tid == 0) {
         w.rho[(size_t)l * w.G + s] = rho;
@@ -292,8 +310,9 @@ __global__ void __launch_bounds__(HT) k_heads_gram(Heads w) {
 
 template <int G8>
 __global__ void __launch_bounds__(HT) k_heads_score(Heads w) {
-    __shared__ double red[HT / 32], v[2][HeadShape<G8>::g + 1];
-    h_score<G8>(w, blockIdx.y, blockIdx.x, red, v);
+    extern __shared__ __align__(16) double smem[];
+    __shared__ double red[HT / 32];
+    h_score<G8>(w, blockIdx.y, blockIdx.x, red, smem);
 }
 
 // Selection (argmin of rho over the live heads, ties to the lowest index; every CTA makes it for
@@ -371,7 +390,7 @@ template <int G8>
 __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, int rescore) {
     using S = HeadShape<G8>;
     extern __shared__ __align__(16) double smem[];
-    __shared__ double red[HT / 32], v[2][S::g + 1];
+    __shared__ double red[HT / 32];
     const int l = blockIdx.y, x = blockIdx.x, n_pairs = w.G * (w.G + 1) / 2;
     if (slot >= 0 && x == 0 && l == 0 && threadIdx.x == 0) w.steps_of[slot] = t + 1;
     const int* alive = w.alive + ((size_t)l * 2 + ((t + 1) & 1)) * w.G;
@@ -400,7 +419,7 @@ __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, i
         subtract(w.Q);
         if (i == j && rescore) {
             __syncthreads();
-            h_score<G8>(w, l, i, red, v);
+            h_score<G8>(w, l, i, red, smem);
         }
         return;
     }
@@ -529,7 +548,8 @@ ziplm_status run_heads(HeadsWs& ws, float damp_frac, const int* levels, float* l
     }
     if (n_steps > 0) {
         PhaseScope ps(PH_BLOCK_SCORE, st);
-        k_heads_score<G8><<<dim3(G, L), HT, 0, st>>>(w);
+        ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_score<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_heads_score<G8><<<dim3(G, L), HT, smem, st>>>(w);
         ZIPLM_CHECK_LAUNCH();
     }
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_solve<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
