@@ -96,6 +96,27 @@ __device__ __forceinline__ double h_frag(const double* s, int m0, int kk, int la
               : s[(m0 + (lane >> 2)) * P_MK + kk * 4 + (lane & 3)];
 }
 
+// acc += one chunk's product of `steps` mma steps.
+template <int G8, bool XKM, bool YKM>
+__device__ __forceinline__ void h_chunk_mma(HeadAcc<G8>& acc, const double* sx, const double* sy, int steps, int warp,
+                                            int lane) {
+    using S = HeadShape<G8>;
+#pragma unroll 2
+    for (int kk = 0; kk < steps; ++kk) {
+        double b[S::CF];
+#pragma unroll
+        for (int j = 0; j < S::CF; ++j) b[j] = h_frag<G8, YKM>(sy, 8 * ((warp & 1) * S::CF + j), kk, lane);
+#pragma unroll
+        for (int u = 0; u < S::UN; ++u) {
+            const int rf = (warp + 8 * u) >> 1;
+            if (rf >= G8) continue;
+            const double a = h_frag<G8, XKM>(sx, 8 * rf, kk, lane);
+#pragma unroll
+            for (int j = 0; j < S::CF; ++j) dmma884(acc.d[u][j], a, b[j]);
+        }
+    }
+}
+
 // acc(g x g) += X (g x K) Y (K x g).  XKM: X(m,k) = X[k * ldx + m], else X[m * ldx + k] with rows from
 // x_rows on zero; YKM: Y(k,n) = Y[k * ldy + n], else Y[n * ldy + k].  K is a multiple of 16 unless both
 // are stored by k.  Starts with every thread past its use of smem and ends with a barrier.
@@ -120,21 +141,66 @@ __device__ __forceinline__ void h_product(HeadAcc<G8>& acc, const double* X, siz
         const double* sx = smem + (c & 1) * 2 * S::kOperand;
         const double* sy = sx + S::kOperand;
         const int steps = (min(KCH, K - c * KCH) + 3) / 4;        // (a row past K is zero)
-#pragma unroll 2
-        for (int kk = 0; kk < steps; ++kk) {
-            double b[S::CF];
-#pragma unroll
-            for (int j = 0; j < S::CF; ++j) b[j] = h_frag<G8, YKM>(sy, 8 * ((warp & 1) * S::CF + j), kk, lane);
-#pragma unroll
-            for (int u = 0; u < S::UN; ++u) {
-                const int rf = (warp + 8 * u) >> 1;
-                if (rf >= G8) continue;
-                const double a = h_frag<G8, XKM>(sx, 8 * rf, kk, lane);
-#pragma unroll
-                for (int j = 0; j < S::CF; ++j) dmma884(acc.d[u][j], a, b[j]);
-            }
-        }
+        h_chunk_mma<G8, XKM, YKM>(acc, sx, sy, steps, warp, lane);
         __syncthreads();
+    }
+}
+
+// As h_product (both operands stored by k, K = g) for `n` products in a row: operands(i, X, Y) gives those
+// of the i-th, done(i) runs when it is complete.  The copies of the next product run beside `done`.
+template <int G8, typename Ops, typename Done>
+__device__ __forceinline__ void h_products(HeadAcc<G8>& acc, int n, size_t ld, double* smem, Ops operands, Done done) {
+    using S = HeadShape<G8>;
+    constexpr int NC = (S::g + KCH - 1) / KCH;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto start = [&](int c) {
+        const double *X, *Y;
+        operands(c / NC, X, Y);
+        double* s = smem + (c & 1) * 2 * S::kOperand;
+        h_chunk<G8, true>(s, X, ld, (c % NC) * KCH, S::g, S::g);
+        h_chunk<G8, true>(s + S::kOperand, Y, ld, (c % NC) * KCH, S::g, S::g);
+    };
+    start(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int c = 0; c < n * NC; ++c) {
+        if (c + 1 < n * NC) start(c + 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const double* sx = smem + (c & 1) * 2 * S::kOperand;
+        h_chunk_mma<G8, true, true>(acc, sx, sx + S::kOperand, min(KCH, S::g - (c % NC) * KCH) / 4, warp, lane);
+        __syncthreads();
+        if (c % NC == NC - 1) done(c / NC);
+    }
+}
+
+// use(row, col, product, load(row, col)) for every pair of the thread's.  The loads of CF pairs (after(),
+// or with kAhead of all, before the product) are in flight together: a load behind a store it may alias
+// waits for it, and one such pair after the other took 10000 clocks.
+template <int G8, bool kAhead, typename P, typename Ld, typename Use>
+__device__ __forceinline__ void h_combine(HeadAcc<G8>& acc, P product, Ld load, Use use) {
+    using S = HeadShape<G8>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    decltype(load(0, 0)) v[kAhead ? S::UN : 1][S::CF];
+    auto fetch = [&](int u) {
+#pragma unroll
+        for (int j = 0; j < S::CF; ++j)
+            v[kAhead ? u : 0][j] = load(8 * ((warp + 8 * u) >> 1) + (lane >> 2), 8 * ((warp & 1) * S::CF + j) + 2 * (lane & 3));
+    };
+    if (kAhead) {
+#pragma unroll
+        for (int u = 0; u < S::UN; ++u)
+            if ((warp + 8 * u) >> 1 < G8) fetch(u);
+    }
+    product();
+#pragma unroll
+    for (int u = 0; u < S::UN; ++u) {
+        if ((warp + 8 * u) >> 1 >= G8) continue;
+        if (!kAhead) fetch(u);
+#pragma unroll
+        for (int j = 0; j < S::CF; ++j)
+            use(8 * ((warp + 8 * u) >> 1) + (lane >> 2), 8 * ((warp & 1) * S::CF + j) + 2 * (lane & 3),
+                make_double2(acc.d[u][j][0], acc.d[u][j][1]), v[kAhead ? u : 0][j]);
     }
 }
 
@@ -361,23 +427,28 @@ __global__ void __launch_bounds__(HT) k_heads_solve(Heads w, int t) {
                                     : (size_t)s * S::g * w.d + (size_t)j * S::g);
     const double* Bn = w.Bneg + ((size_t)l * w.G + s) * S::g * S::g;
     HeadAcc<G8> acc;
+    constexpr bool kAhead = G8 <= 8;     // one CTA per SM here, so registers are to be had
+    auto block = [&](const double* M) {
+        return [=](int k, int n) {
+            const double* o = M + (below ? blk + (size_t)n * w.d + k : blk + (size_t)k * w.d + n);
+            return below ? make_double2(o[0], o[w.d]) : *reinterpret_cast<const double2*>(o);
+        };
+    };
     acc.zero();
     // B^-1 is symmetric: stored by k as well as by m
-    if (below) h_product<G8, true, false>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
-    else h_product<G8, true, true>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
-    acc.visit([&](int k, int n, double2 x) {
+    h_combine<G8, kAhead>(acc, [&] {
+        if (below) h_product<G8, true, false>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
+        else h_product<G8, true, true>(acc, Bn, S::g, S::g, w.A + blk, w.d, S::g, smem);
+    }, block(w.A), [&](int k, int n, double2 x, double2 p) {
         *reinterpret_cast<double2*>(w.T + out + (size_t)k * w.d + n) = make_double2(-x.x, -x.y);
-        const size_t o = below ? blk + (size_t)n * w.d + k : blk + (size_t)k * w.d + n;
-        *reinterpret_cast<double2*>(w.P + out + (size_t)k * w.d + n) =
-            below ? make_double2(w.A[o], w.A[o + w.d]) : *reinterpret_cast<const double2*>(w.A + o);
+        *reinterpret_cast<double2*>(w.P + out + (size_t)k * w.d + n) = p;
     });
     __syncthreads();                // T is read back below, by the whole CTA
     const size_t ss = lay + (size_t)s * S::g * w.d + (size_t)s * S::g;
     acc.zero();
-    h_product<G8, true, true>(acc, w.Q + ss, w.d, S::g, w.T + out, w.d, S::g, smem);
-    acc.visit([&](int k, int n, double2 x) {
-        const size_t o = below ? blk + (size_t)n * w.d + k : blk + (size_t)k * w.d + n;
-        const double2 q = below ? make_double2(w.Q[o], w.Q[o + w.d]) : *reinterpret_cast<const double2*>(w.Q + o);
+    h_combine<G8, kAhead>(acc, [&] {
+        h_product<G8, true, true>(acc, w.Q + ss, w.d, S::g, w.T + out, w.d, S::g, smem);
+    }, block(w.Q), [&](int k, int n, double2 x, double2 q) {
         *reinterpret_cast<double2*>(w.V + out + (size_t)k * w.d + n) =
             make_double2(fma(-0.5, x.x, q.x), fma(-0.5, x.y, q.y));
     });
@@ -401,22 +472,22 @@ __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, i
         if (x >= w.G) { pair_index(x - w.G, i, j); ++i; }
         if (!alive[i] || !alive[j]) return;
         const size_t at = (size_t)l * w.d * w.d + (size_t)i * S::g * w.d + (size_t)j * S::g;
-        auto subtract = [&](double* M) {
-            acc.visit([&](int row, int col, double2 d) {
-                double2* o = reinterpret_cast<double2*>(M + at + (size_t)row * w.d + col);
-                double2 cur = *o;
-                cur.x -= d.x; cur.y -= d.y;
-                *o = cur;
+        const double *Pi = w.P + ops + i * S::g, *Ti = w.T + ops + i * S::g, *Tj = w.T + ops + j * S::g;
+        const double *Vi = w.V + ops + i * S::g, *Vj = w.V + ops + j * S::g;
+        acc.zero();
+        h_products<G8>(acc, 3, w.d, smem, [&](int q, const double*& X, const double*& Y) {
+            X = q == 0 ? Pi : q == 1 ? Vi : Ti;
+            Y = q == 2 ? Vj : Tj;
+        }, [&](int q) {
+            if (q == 1) return;
+            double* M = (q == 0 ? w.A : w.Q) + at;
+            h_combine<G8, false>(acc, [] {}, [=](int row, int col) {
+                return *reinterpret_cast<const double2*>(M + (size_t)row * w.d + col);
+            }, [=](int row, int col, double2 d, double2 cur) {
+                *reinterpret_cast<double2*>(M + (size_t)row * w.d + col) = make_double2(cur.x - d.x, cur.y - d.y);
             });
-        };
-        const double *Ti = w.T + ops + i * S::g, *Tj = w.T + ops + j * S::g;
-        acc.zero();
-        h_product<G8, true, true>(acc, w.P + ops + i * S::g, w.d, S::g, Tj, w.d, S::g, smem);
-        subtract(w.A);
-        acc.zero();
-        h_product<G8, true, true>(acc, w.V + ops + i * S::g, w.d, S::g, Tj, w.d, S::g, smem);
-        h_product<G8, true, true>(acc, Ti, w.d, S::g, w.V + ops + j * S::g, w.d, S::g, smem);
-        subtract(w.Q);
+            acc.zero();
+        });
         if (i == j && rescore) {
             __syncthreads();
             h_score<G8>(w, l, i, red, smem);
@@ -443,17 +514,19 @@ __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, i
         acc.zero();
         h_product<G8, false, true>(acc, Wl + (size_t)w.chosen[l] * S::g, w.d, rows, w.T + ops + j * S::g, w.d, S::g,
                                    smem);
-        acc.visit([&](int row, int col, double2 d) {
+        struct Cur { double2 w; float2 w0; };
+        h_combine<G8, false>(acc, [] {}, [&](int row, int col) {
+            const size_t o = (size_t)min(row, rows - 1) * w.d + col;
+            return Cur{*reinterpret_cast<const double2*>(Wl + (size_t)j * S::g + o),
+                       snap ? *reinterpret_cast<const float2*>(W0 + o) : make_float2(0.f, 0.f)};
+        }, [&](int row, int col, double2 d, Cur cur) {
             if (row >= rows) return;
             const size_t o = (size_t)row * w.d + col;
-            double2* p = reinterpret_cast<double2*>(Wl + (size_t)j * S::g + o);
-            double2 cur = *p;
-            cur.x -= d.x; cur.y -= d.y;
-            *p = cur;
+            cur.w.x -= d.x; cur.w.y -= d.y;
+            *reinterpret_cast<double2*>(Wl + (size_t)j * S::g + o) = cur.w;
             if (snap) {
-                const float f0 = (float)cur.x, f1 = (float)cur.y, e0 = W0[o] - f0, e1 = W0[o + 1] - f1;
-                snap[o] = f0;
-                snap[o + 1] = f1;
+                const float f0 = (float)cur.w.x, f1 = (float)cur.w.y, e0 = cur.w0.x - f0, e1 = cur.w0.y - f1;
+                *reinterpret_cast<float2*>(snap + o) = make_float2(f0, f1);
                 part += (double)e0 * e0 + (double)e1 * e1;
             }
         });
