@@ -100,18 +100,21 @@ __global__ void __launch_bounds__(256) k_digits_rows(const double* __restrict__ 
 }
 
 // Operand rows = matrix columns: largest exponents first (exps zeroed beforehand), then the digits through a
-// 64 x 64 tile.  tri: column j is zero above the tile of its diagonal entry.
-__global__ void __launch_bounds__(256) k_column_exponents(const double* __restrict__ src, size_t layer_stride,
-                                                          int ld, int cols, int K, int tri, int* __restrict__ exps) {
+// 64 x 64 tile.  tri: column j is zero above the tile of its diagonal entry.  Entries from k_valid and
+// column_valid on (the padding of the operand) are zero and not read.
+template <typename T>
+__global__ void __launch_bounds__(256) k_column_exponents(const T* __restrict__ src, size_t layer_stride, int ld,
+                                                          int cols, int k_valid, int column_valid, int tri,
+                                                          int* __restrict__ exps) {
     __shared__ int red[256];
     const int l = blockIdx.z, tid = threadIdx.x, c = tid & 63, k0 = blockIdx.y * 256;
     const int j = blockIdx.x * 64 + c;
-    const double* s = src + l * layer_stride + j;
-    const int first = tri ? blockIdx.x * 64 : 0, end = min(K, k0 + 256);
+    const T* s = src + l * layer_stride + j;
+    const int first = tri ? blockIdx.x * 64 : 0, end = j < column_valid ? min(k_valid, k0 + 256) : 0;
     int e = 0;
 #pragma unroll 8
     for (int k = k0 + (tid >> 6); k < end; k += 4)
-        if (k >= first) e = max(e, (__double2hiint(s[(size_t)k * ld]) >> 20) & 2047);
+        if (k >= first) e = max(e, (__double2hiint((double)s[(size_t)k * ld]) >> 20) & 2047);
     red[tid] = e;
     __syncthreads();
     if (tid < 64) {
@@ -119,16 +122,21 @@ __global__ void __launch_bounds__(256) k_column_exponents(const double* __restri
         atomicMax(exps + (size_t)l * cols + j, e);
     }
 }
-__global__ void __launch_bounds__(256) k_digits_columns(const double* __restrict__ src, size_t layer_stride, int ld,
-                                                        int cols, int K, int tri, const int* __restrict__ exps,
-                                                        signed char* __restrict__ dig, double* __restrict__ scale) {
+template <typename T>
+__global__ void __launch_bounds__(256) k_digits_columns(const T* __restrict__ src, size_t layer_stride, int ld,
+                                                        int cols, int K, int k_valid, int column_valid, int tri,
+                                                        const int* __restrict__ exps, signed char* __restrict__ dig,
+                                                        double* __restrict__ scale) {
     __shared__ double tile[64][65];              // [k][column]
     const int l = blockIdx.z, tid = threadIdx.x, j0 = blockIdx.x * 64, k0 = blockIdx.y * 64;
     const bool zero = tri && k0 < j0;
-    const double* s = src + l * layer_stride + (size_t)k0 * ld + j0;
+    const T* s = src + l * layer_stride + (size_t)k0 * ld + j0;
     if (!zero)
 #pragma unroll
-        for (int e = 0; e < 16; ++e) tile[(tid >> 6) + 4 * e][tid & 63] = s[(size_t)((tid >> 6) + 4 * e) * ld + (tid & 63)];
+        for (int e = 0; e < 16; ++e) {
+            const int k = (tid >> 6) + 4 * e, c = tid & 63;
+            tile[k][c] = k0 + k < k_valid && j0 + c < column_valid ? (double)s[(size_t)k * ld + c] : 0.0;
+        }
     __syncthreads();
     const int kq = 4 * (tid & 15);
 #pragma unroll
@@ -395,6 +403,19 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
 }
 
+template <typename T>
+ziplm_status column_digits(const I8Operand& o, const T* src, size_t layer_stride, int ld, int k_valid, int column_valid,
+                           bool tri, int L, cudaStream_t st) {
+    ZIPLM_CHECK_CUDA(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)L * o.rows, st));
+    k_column_exponents<T><<<dim3(o.rows / 64, (k_valid + 255) / 256, L), 256, 0, st>>>(
+        src, layer_stride, ld, o.rows, k_valid, column_valid, tri, o.exps);
+    ZIPLM_CHECK_LAUNCH();
+    k_digits_columns<T><<<dim3(o.rows / 64, o.K / 64, L), 256, 0, st>>>(
+        src, layer_stride, ld, o.rows, o.K, k_valid, column_valid, tri, o.exps, o.dig, o.scale);
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
 bool make_digit_map(CUtensorMap* m, const signed char* dig, int L, int rows, int K, int box_rows) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
@@ -416,14 +437,33 @@ ziplm_status i8_digits(const I8Operand& o, const double* src, size_t layer_strid
         ZIPLM_CHECK_LAUNCH();
         return ZIPLM_OK;
     }
-    ZIPLM_CHECK_CUDA(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)L * o.rows, st));
-    k_column_exponents<<<dim3(o.rows / 64, (o.K + 255) / 256, L), 256, 0, st>>>(src, layer_stride, ld, o.rows, o.K, tri,
-                                                                              o.exps);
-    ZIPLM_CHECK_LAUNCH();
-    k_digits_columns<<<dim3(o.rows / 64, o.K / 64, L), 256, 0, st>>>(src, layer_stride, ld, o.rows, o.K, tri, o.exps,
-                                                                     o.dig, o.scale);
-    ZIPLM_CHECK_LAUNCH();
-    return ZIPLM_OK;
+    return column_digits(o, src, layer_stride, ld, o.K, o.rows, tri, L, st);
+}
+
+ziplm_status i8_digits_of_columns(const I8Operand& o, const float* src, size_t layer_stride, int ld, int k_valid,
+                                  int column_valid, int L, cudaStream_t st) {
+    return column_digits(o, src, layer_stride, ld, k_valid, column_valid, false, L, st);
+}
+
+size_t carve_i8_operand(I8Operand* o, void* ws, int L, int rows, int K) {
+    Carver c(ws);
+    I8Operand x = {};
+    x.rows = round_up_int(rows, 64);
+    x.K = round_up_int(K, 64);
+    x.dig = c.take<signed char>((size_t)L * SL * x.rows * x.K);
+    x.scale = c.take<double>((size_t)L * x.rows);
+    x.exps = c.take<int>((size_t)L * x.rows);
+    if (o) *o = x;
+    return c.off;
+}
+
+bool i8_symmetric_pays(int L, int rows, int K, double float64_clocks) {
+    if (K > 16384) return false;
+    const int nI = (rows + PM - 1) / PM, nJ = (rows + PN - 1) / PN;
+    double tiles = 0;
+    for (int I = 0; I < nI; ++I) tiles += 2 * I + 2 < nJ ? 2 * I + 2 : nJ;
+    const double waves = ceil(L * tiles / 74);           // two of the 148 SMs to a tile
+    return 20000.0 + waves * ((K + KB - 1) / KB * 7000.0 + 30000.0) < float64_clocks;
 }
 
 ziplm_status i8_product(const I8Operand& x, const I8Operand& y, I8Product p, int L, cudaStream_t st) {

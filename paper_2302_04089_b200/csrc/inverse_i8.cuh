@@ -32,6 +32,16 @@ struct I8Product {
 // tri: block of a lower triangular matrix whose tiles above the diagonal are not written.
 ziplm_status i8_digits(const I8Operand& o, const double* src, size_t layer_stride, int ld, bool columns, bool tri,
                        int L, cudaStream_t st);
+// Digits of the columns of a float32 matrix, zero from row k_valid and column column_valid on.
+ziplm_status i8_digits_of_columns(const I8Operand& o, const float* src, size_t layer_stride, int ld, int k_valid,
+                                  int column_valid, int L, cudaStream_t st);
+// An operand of at least rows x K in a workspace; returns its bytes.
+size_t carve_i8_operand(I8Operand* o, void* ws, int L, int rows, int K);
+
+// Whether x^T x of L layers (rows x rows from K) is quicker here than in float64_clocks: a wave of tile
+// pairs takes 7000 clocks per 64 of K and some 30000 for the rest, the digits three launches.
+bool i8_symmetric_pays(int L, int rows, int K, double float64_clocks);
+
 ziplm_status i8_product(const I8Operand& x, const I8Operand& y, I8Product p, int L, cudaStream_t st);
 
 }  // namespace ziplm

@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "factor16.cuh"
+#include "inverse_i8.cuh"
 
 namespace ziplm {
 namespace {
@@ -350,12 +351,11 @@ __global__ void __launch_bounds__(HT) k_heads_init(Heads w) {
         w.alive[(size_t)(i / w.G) * 2 * w.G + i % w.G] = 1;
 }
 
-// Block (i, j), i >= j, of Q = W^T W, and its share of <Q, H> = 2 ||W X||^2.
+// Block (i, j), i >= j, of Q = W^T W.
 template <int G8>
 __global__ void __launch_bounds__(HT) k_heads_gram(Heads w) {
     using S = HeadShape<G8>;
     extern __shared__ __align__(16) double smem[];
-    __shared__ double red[HT / 32];
     const int l = blockIdx.y;
     int i, j;
     pair_index(blockIdx.x, i, j);
@@ -364,14 +364,22 @@ __global__ void __launch_bounds__(HT) k_heads_gram(Heads w) {
     acc.zero();
     h_product<G8, true, true>(acc, Wl + i * S::g, w.d, S::g, Wl + j * S::g, w.d, w.r, smem);
     const size_t at = (size_t)l * w.d * w.d + (size_t)i * S::g * w.d + (size_t)j * S::g;
-    double part = 0.0;
     acc.visit([&](int row, int col, double2 x) {
-        const size_t o = at + (size_t)row * w.d + col;
-        *reinterpret_cast<double2*>(w.Q + o) = x;
-        part += x.x * (double)w.H[o] + x.y * (double)w.H[o + 1];
+        *reinterpret_cast<double2*>(w.Q + at + (size_t)row * w.d + col) = x;
     });
+}
+
+// <Q, H> = 2 ||W X||^2 from the lower triangles.
+__global__ void __launch_bounds__(HT) k_heads_base(Heads w) {
+    __shared__ double red[HT / 32];
+    const int l = blockIdx.y;
+    double part = 0.0;
+    for (int i = blockIdx.x; i < w.d; i += gridDim.x) {
+        const size_t row = ((size_t)l * w.d + i) * w.d;
+        for (int j = threadIdx.x; j <= i; j += HT) part += (j < i ? 2.0 : 1.0) * w.Q[row + j] * (double)w.H[row + j];
+    }
     const double t = h_sum(part, red);
-    if (threadIdx.x == 0) atomicAdd(w.dw2 + (size_t)l * (w.n_levels + 1) + w.n_levels, i == j ? t : 2.0 * t);
+    if (threadIdx.x == 0) atomicAdd(w.dw2 + (size_t)l * (w.n_levels + 1) + w.n_levels, t);
 }
 
 template <int G8>
@@ -556,6 +564,13 @@ struct HeadsWs {
     double* lam; void* inv_ws; size_t inv_bytes, zero_bytes; void* zero; size_t total;
 };
 
+// Q = W^T W in digits on the int8 tensor cores when that is quicker (12 x 768 x 768: 262 -> 195 us); the
+// float64 kernel runs at 0.65 of its instruction's rate, and a CTA's chain is 4500 clocks per 64^3.
+bool gram_on_i8(int L, int r, int d, int g) {
+    const double G = d / g, ctas = L * G * (G + 1) / 2, cta = (double)r * g * g / 64 * 1.1 + 4000;
+    return i8_symmetric_pays(L, d, r, cta > ctas * cta / (148 * 0.65) ? cta : ctas * cta / (148 * 0.65));
+}
+
 HeadsWs carve_heads(void* ws, int L, int r, int d, int g, int n_levels) {
     HeadsWs w = {};
     const int G = d / g;
@@ -579,6 +594,7 @@ HeadsWs carve_heads(void* ws, int L, int r, int d, int g, int n_levels) {
     w.zero_bytes = c.off - z0;
     w.lam = c.take<double>((size_t)L);
     w.inv_bytes = inverse_workspace_bytes(L, d);
+    if (gram_on_i8(L, r, d, g)) w.inv_bytes = max(w.inv_bytes, carve_i8_operand(nullptr, nullptr, L, d, r));
     w.inv_ws = c.take<char>(w.inv_bytes);
     w.total = c.off;
     return w;
@@ -607,9 +623,26 @@ ziplm_status run_heads(HeadsWs& ws, float damp_frac, const int* levels, float* l
         k_heads_init<<<592, HT, 0, st>>>(w);
         ZIPLM_CHECK_LAUNCH();
         if (n_steps > 0 || base_loss) {
-            ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_gram<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            k_heads_gram<G8><<<dim3(G * (G + 1) / 2, L), HT, smem, st>>>(w);
-            ZIPLM_CHECK_LAUNCH();
+            if (gram_on_i8(L, w.r, w.d, g)) {
+                I8Operand x;
+                carve_i8_operand(&x, ws.inv_ws, L, w.d, w.r);        // the inverse is done with it
+                s = i8_digits_of_columns(x, w.W, (size_t)w.r * w.d, w.d, w.r, w.d, L, st);
+                if (s != ZIPLM_OK) return s;
+                I8Product p = {};
+                p.alpha = 1.0; p.krange = K_ALL; p.lower = 1;
+                p.d = w.d; p.out64 = w.Q; p.layer_status = w.layer_status;
+                s = i8_product(x, x, p, L, st);
+                if (s != ZIPLM_OK) return s;
+            } else {
+                ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_heads_gram<G8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      smem));
+                k_heads_gram<G8><<<dim3(G * (G + 1) / 2, L), HT, smem, st>>>(w);
+                ZIPLM_CHECK_LAUNCH();
+            }
+            if (base_loss) {
+                k_heads_base<<<dim3(min(64, w.d), L), HT, 0, st>>>(w);
+                ZIPLM_CHECK_LAUNCH();
+            }
         }
         if (n_levels > 0 && levels[0] == G) {              // the unpruned level: loss 0
             const size_t n = (size_t)w.r * w.d;

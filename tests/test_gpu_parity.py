@@ -867,3 +867,20 @@ def test_factorisation_leaf_at_the_edges_of_its_blocks(d):
     assert got[0] == 0 and all(v == got[1] != 0 for v in got[1:-1]) and got[-1] not in (0, got[1])
     ref = zo.inverse_spd(zo.damped(H.numpy(), float(np.float32(0.01)))[0])
     assert np.max(np.abs(Hinv[0].cpu().numpy() - ref)) / np.max(np.abs(ref)) < 1e-9
+
+
+@pytest.mark.parametrize("L,r,d,g", [(12, 700, 768, 64), (24, 200, 1120, 80)])
+def test_heads_gram_matrix_on_int8_products(L, r, d, g):
+    """Enough layers for the Gram matrix W^T W to be formed in digits; ragged rows, padded columns and
+    features of different scale."""
+    z = zb()
+    gen = torch.Generator().manual_seed(r)
+    W = torch.randn(L, r, d, generator=gen)
+    X = torch.randn(L, d, 2 * d, generator=gen) * torch.exp(torch.randn(L, d, 1, generator=gen))
+    H = 2.0 * X @ X.transpose(1, 2)
+    levels = [d // g, d // g - 3]
+    out = z.prune_layers(W.cuda(), H.cuda(), g, 0.01, levels)
+    torch.cuda.synchronize()
+    assert out["layer_status"].tolist() == [0] * L
+    for l in (0, L - 1):
+        compare_layer(W[l].numpy(), H[l].numpy(), g, 0.01, levels, out, l)
