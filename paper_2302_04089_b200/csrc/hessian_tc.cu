@@ -540,20 +540,25 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
 // meet through distributed shared memory, and the scaled fp16 parts leave K-major.  A is read once instead
 // of twice and nothing has to be zeroed beforehand (eight batches of 12 x 2048 x 3072, products included:
 // 9.5 -> 9.2 ms; for a small batch it is one launch instead of three).  VEC: rows of A start on 16 bytes.
-constexpr int TS_FEATURES = 64, TS_PITCH = TS_FEATURES + 1;
-constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 195 KiB of shared memory
+// In shared memory a feature's tokens lie in a row, in quads whose place is permuted by the feature, so that
+// a warp's stores of 8 x 4 features by 4 tokens and its loads of a row's quads meet no bank conflict.
+constexpr int TS_FEATURES = 32, TS_THREADS = 4 * TS_FEATURES;
+constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 192 KiB of shared memory
+__device__ __forceinline__ int ts_at(int f, int t, int pitch) { return f * pitch + (t ^ (f & 28)); }
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ A, long long lda, int N, int d,
+__global__ void __launch_bounds__(TS_THREADS) k_tokens_split(const float* __restrict__ A, long long lda, int N, int d,
                                                       long long np, int tokens, unsigned* __restrict__ amax,
                                                       __half* __restrict__ hi, __half* __restrict__ lo) {
     grid_trigger();
-    extern __shared__ float ts_tile[];           // [tokens][TS_PITCH]
+    extern __shared__ __align__(16) float ts_tile[];     // [TS_FEATURES][pitch]
     __shared__ unsigned s_max[TS_FEATURES];
+    __shared__ float s_scale[TS_FEATURES];
     cg::cluster_group cluster = cg::this_cluster();
     const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int l = blockIdx.z, f0 = blockIdx.y * TS_FEATURES;
-    const int t0 = rank * tokens, t1 = min(N, t0 + tokens);
-    const int tid = threadIdx.x, q = tid & 15, rr = tid >> 4;
+    const int t0 = rank * tokens, t1 = min(N, t0 + tokens), pitch = (tokens + 31) & ~31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int q = lane & 7, rr = (lane >> 3) + 4 * warp;
     const float* Al = A + (size_t)l * (size_t)N * (size_t)lda;
     if (tid < TS_FEATURES) s_max[tid] = 0u;
     __syncthreads();
@@ -582,31 +587,44 @@ __global__ void __launch_bounds__(256) k_tokens_split(const float* __restrict__ 
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 m[e] = max(m[e], __float_as_uint(v[k][e]) & 0x7fffffffu);
-                if (t + 16 * k < t1) ts_tile[(t + 16 * k - t0) * TS_PITCH + 4 * q + e] = v[k][e];
+                if (t + 16 * k < t1) ts_tile[ts_at(4 * q + e, t + 16 * k - t0, pitch)] = v[k][e];
             }
     }
 #pragma unroll
-    for (int e = 0; e < 4; ++e) atomicMax(&s_max[4 * q + e], m[e]);
+    for (int e = 0; e < 4; ++e) {                // the four tokens of a warp's features first
+        m[e] = max(m[e], __shfl_xor_sync(0xffffffffu, m[e], 8));
+        m[e] = max(m[e], __shfl_xor_sync(0xffffffffu, m[e], 16));
+        if (lane < 8) atomicMax(&s_max[4 * q + e], m[e]);
+    }
     if (CS > 1) cluster.sync();
     else __syncthreads();
-    // pairs of tokens along the lanes, a feature per warp and turn
-    const int lane = tid & 31, warp = tid >> 5;
+    {
+        const int fl = tid >> 2;
+        unsigned mx = 0u;
+        for (int r = tid & 3; r < CS; r += 4) mx = max(mx, cluster.map_shared_rank(s_max, r)[fl]);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        if ((tid & 3) == 0) {
+            s_scale[fl] = row_scale(mx, false);
+            if (rank == 0 && f0 + fl < d) amax[(size_t)l * d + f0 + fl] = mx;
+        }
+    }
+    __syncthreads();
+    // four tokens per lane, a feature per warp and turn
     const int p1 = (int)min(np, (long long)(t0 + tokens));       // the last range also writes the padding
-    for (int fl = warp; fl < TS_FEATURES; fl += 8) {
+    for (int fl = warp; fl < TS_FEATURES; fl += TS_THREADS / 32) {
         if (f0 + fl >= d) break;
-        unsigned mx = lane < CS ? cluster.map_shared_rank(s_max, lane)[fl] : 0u;
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (rank == 0 && lane == 0) amax[(size_t)l * d + f0 + fl] = mx;
-        const float sc = row_scale(mx, false);
+        const float sc = s_scale[fl];
         const size_t row = ((size_t)l * d + f0 + fl) * (size_t)np;
-        for (int t = t0 + 2 * lane; t < p1; t += 64) {
-            const float x0 = t < t1 ? ts_tile[(t - t0) * TS_PITCH + fl] : 0.f;
-            const float x1 = t + 1 < t1 ? ts_tile[(t + 1 - t0) * TS_PITCH + fl] : 0.f;
-            __half2 h, w;
-            split_f16x2(x0 * sc, h.x, w.x);
-            split_f16x2(x1 * sc, h.y, w.y);
-            *reinterpret_cast<__half2*>(hi + row + t) = h;
-            *reinterpret_cast<__half2*>(lo + row + t) = w;
+#pragma unroll 2
+        for (int t = t0 + 4 * lane; t < p1; t += 128) {
+            const float4 x4 = *reinterpret_cast<const float4*>(ts_tile + ts_at(fl, t - t0, pitch));
+            const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+            union { uint2 v; __half e[4]; } h, w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) split_f16x2((t + e < t1 ? x[e] : 0.f) * sc, h.e[e], w.e[e]);
+            *reinterpret_cast<uint2*>(hi + row + t) = h.v;
+            *reinterpret_cast<uint2*>(lo + row + t) = w.v;
         }
     }
     if (CS > 1) cluster.sync();                  // the magnitudes stay readable until all have them
@@ -622,11 +640,11 @@ ziplm_status run_tokens_split(const float* A, long long lda, int N, int d, long 
     const bool vec = (reinterpret_cast<uintptr_t>(A) % 16) == 0 && lda % 4 == 0;
     auto kernel = vec ? k_tokens_split<true> : k_tokens_split<false>;
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          TS_TOKENS * TS_PITCH * (int)sizeof(float)));
+                                          TS_TOKENS * TS_FEATURES * (int)sizeof(float)));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, (d + TS_FEATURES - 1) / TS_FEATURES, layers);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = (size_t)tokens * TS_PITCH * sizeof(float);
+    cfg.blockDim = dim3(TS_THREADS);
+    cfg.dynamicSmemBytes = (size_t)round_up_int(tokens, 32) * TS_FEATURES * sizeof(float);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
