@@ -358,6 +358,18 @@ __device__ __forceinline__ void split_f16x2(float y, __half& p1, __half& p2) {
     p1 = __float2half_rn(y);
     p2 = __float2half_rn(y - __half2float(p1));
 }
+// Of four values at once, by packed conversions.
+__device__ __forceinline__ void split_f16x2(const float (&y)[4], uint2& p1, uint2& p2) {
+    union { uint2 v; __half2 e[2]; } a, b;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        a.e[e] = __floats2half2_rn(y[2 * e], y[2 * e + 1]);
+        const float2 f = __half22float2(a.e[e]);
+        b.e[e] = __floats2half2_rn(y[2 * e] - f.x, y[2 * e + 1] - f.y);
+    }
+    p1 = a.v;
+    p2 = b.v;
+}
 
 // X_1, X_2 of a token-contiguous fp32 X, four tokens per thread; np (a multiple of 8) is the row
 // pitch of the parts, zero past N.
@@ -378,11 +390,9 @@ __global__ void __launch_bounds__(256) k_split_f16(const float* __restrict__ X, 
         for (int e = 0; e < 4; ++e) if (k + e < N) v[e] = src[e];
     }
     const float sc = row_scale(amax[row], false);
-    union { uint2 u; __half h[4]; } a, b;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) split_f16x2(v[e] * sc, a.h[e], b.h[e]);
-    *reinterpret_cast<uint2*>(hi + row * (size_t)np + k) = a.u;
-    *reinterpret_cast<uint2*>(lo + row * (size_t)np + k) = b.u;
+    const float y[4] = {v[0] * sc, v[1] * sc, v[2] * sc, v[3] * sc};
+    split_f16x2(y, *reinterpret_cast<uint2*>(hi + row * (size_t)np + k),
+                *reinterpret_cast<uint2*>(lo + row * (size_t)np + k));
 }
 
 // Both pre-passes in one for rows of at most 256 * 4 * VEC tokens: a CTA keeps its feature row in
@@ -429,11 +439,9 @@ __global__ void __launch_bounds__(256) k_row_absmax_split(const float* __restric
     for (int j = 0; j < VEC; ++j) {
         const long long k = ((long long)j * 256 + threadIdx.x) * 4;
         if (k >= np) continue;
-        union { uint2 u; __half h[4]; } a, b;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) split_f16x2(v[j][e] * sc, a.h[e], b.h[e]);
-        *reinterpret_cast<uint2*>(hi + row * (size_t)np + k) = a.u;
-        *reinterpret_cast<uint2*>(lo + row * (size_t)np + k) = b.u;
+        const float y[4] = {v[j][0] * sc, v[j][1] * sc, v[j][2] * sc, v[j][3] * sc};
+        split_f16x2(y, *reinterpret_cast<uint2*>(hi + row * (size_t)np + k),
+                    *reinterpret_cast<uint2*>(lo + row * (size_t)np + k));
     }
 }
 
@@ -538,8 +546,9 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
 // Both pre-passes of token-major fp32 batches in one: a cluster of up to eight CTAs takes 64 features of
 // all N tokens, each CTA a range of tokens that it keeps in shared memory; the features' largest magnitudes
 // meet through distributed shared memory, and the scaled fp16 parts leave K-major.  A is read once instead
-// of twice and nothing has to be zeroed beforehand (eight batches of 12 x 2048 x 3072, products included:
-// 9.5 -> 9.2 ms; for a small batch it is one launch instead of three).  VEC: rows of A start on 16 bytes.
+// of twice and nothing has to be zeroed beforehand (for a small batch it is one launch instead of three).
+// VEC: rows of A start on 16 bytes.  12 x 2048 x 3072: 168 -> 124 us (4.9 TB/s) by the bank-conflict-free
+// rows below, packed conversions (37 instructions an entry before) and no fence behind the stores.
 // In shared memory a feature's tokens lie in a row, in quads whose place is permuted by the feature, so that
 // a warp's stores of 8 x 4 features by 4 tokens and its loads of a row's quads meet no bank conflict.
 constexpr int TS_FEATURES = 32, TS_THREADS = 4 * TS_FEATURES;
@@ -565,30 +574,43 @@ __global__ void __launch_bounds__(TS_THREADS) k_tokens_split(const float* __rest
     unsigned m[4] = {0u, 0u, 0u, 0u};
     const int f = f0 + 4 * q;
     const bool whole = VEC && f + 3 < d;
+    // places of the tokens rr + 16 k: the permutation takes rr's low bits and exchanges k's parity
+    const int swz = (4 * q) & 28;
+    float* place = ts_tile + 4 * q * pitch + (rr ^ (swz & 15));
+    const int odd = swz & 16;
     constexpr int FLY = 16;                      // 16-byte loads in flight per thread
     for (int t = t0 + rr; t < t1; t += 16 * FLY) {
-        float v[FLY][4];
+        float4 v[FLY];
+        const float* src = Al + (size_t)t * (size_t)lda + f;
+        const size_t step = 16 * (size_t)lda;
+        const int n = (t1 - t + 15) >> 4;        // tokens of this thread in the turn, at most FLY
 #pragma unroll
-        for (int k = 0; k < FLY; ++k) {
-            const int tk = t + 16 * k;
-            v[k][0] = v[k][1] = v[k][2] = v[k][3] = 0.f;
-            if (tk >= t1) continue;
-            const float* src = Al + (size_t)tk * (size_t)lda + f;
+        for (int k = 0; k < FLY; ++k, src += step) {
+            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k >= n) continue;
             if (whole) {
-                const float4 x = __ldcs(reinterpret_cast<const float4*>(src));
-                v[k][0] = x.x; v[k][1] = x.y; v[k][2] = x.z; v[k][3] = x.w;
+                v[k] = __ldcs(reinterpret_cast<const float4*>(src));
             } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) if (f + e < d) v[k][e] = src[e];
+                if (f < d) v[k].x = src[0];
+                if (f + 1 < d) v[k].y = src[1];
+                if (f + 2 < d) v[k].z = src[2];
+                if (f + 3 < d) v[k].w = src[3];
             }
         }
+        float* to = place + (t - t0 - rr);
 #pragma unroll
-        for (int k = 0; k < FLY; ++k)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                m[e] = max(m[e], __float_as_uint(v[k][e]) & 0x7fffffffu);
-                if (t + 16 * k < t1) ts_tile[ts_at(4 * q + e, t + 16 * k - t0, pitch)] = v[k][e];
-            }
+        for (int k = 0; k < FLY; ++k) {
+            if (k >= n) break;
+            float* o = to + 16 * (k & ~1) + (k & 1 ? 16 - odd : odd);
+            m[0] = max(m[0], __float_as_uint(v[k].x) & 0x7fffffffu);
+            m[1] = max(m[1], __float_as_uint(v[k].y) & 0x7fffffffu);
+            m[2] = max(m[2], __float_as_uint(v[k].z) & 0x7fffffffu);
+            m[3] = max(m[3], __float_as_uint(v[k].w) & 0x7fffffffu);
+            o[0] = v[k].x;
+            o[pitch] = v[k].y;
+            o[2 * pitch] = v[k].z;
+            o[3 * pitch] = v[k].w;
+        }
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {                // the four tokens of a warp's features first
@@ -609,6 +631,10 @@ __global__ void __launch_bounds__(TS_THREADS) k_tokens_split(const float* __rest
             if (rank == 0 && f0 + fl < d) amax[(size_t)l * d + f0 + fl] = mx;
         }
     }
+    // The magnitudes stay readable until all have them.  (Nothing else to order: a releasing arrival behind
+    // the stores below would wait for them.)
+    __syncwarp();
+    if (CS > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     __syncthreads();
     // four tokens per lane, a feature per warp and turn
     const int p1 = (int)min(np, (long long)(t0 + tokens));       // the last range also writes the padding
@@ -620,14 +646,17 @@ __global__ void __launch_bounds__(TS_THREADS) k_tokens_split(const float* __rest
         for (int t = t0 + 4 * lane; t < p1; t += 128) {
             const float4 x4 = *reinterpret_cast<const float4*>(ts_tile + ts_at(fl, t - t0, pitch));
             const float x[4] = {x4.x, x4.y, x4.z, x4.w};
-            union { uint2 v; __half e[4]; } h, w;
+            float y[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) split_f16x2((t + e < t1 ? x[e] : 0.f) * sc, h.e[e], w.e[e]);
-            *reinterpret_cast<uint2*>(hi + row + t) = h.v;
-            *reinterpret_cast<uint2*>(lo + row + t) = w.v;
+            for (int e = 0; e < 4; ++e) y[e] = (t + e < t1 ? x[e] : 0.f) * sc;
+            uint2 h, w;
+            split_f16x2(y, h, w);
+            *reinterpret_cast<uint2*>(hi + row + t) = h;
+            *reinterpret_cast<uint2*>(lo + row + t) = w;
         }
     }
-    if (CS > 1) cluster.sync();                  // the magnitudes stay readable until all have them
+    __syncwarp();
+    if (CS > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
 // Launch of k_tokens_split: ranges of about 256 tokens (a multiple of 8), more per CTA where eight of them
