@@ -486,38 +486,34 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor(const T* __restrict__ 
     }
 }
 
-// The same move for inputs whose rows allow 4-element vector accesses (A aligned to 4 elements,
-// lda % 4 == 0): a 64 x 64 tile, four elements per access on both sides, so a row of the output
-// leaves in 256-byte (fp32) pieces.  np is a multiple of 4, so a quad that starts below np ends
-// below it.
-template <typename T, typename V, typename O, bool SPLIT>
-__global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict__ A, long long lda,
-                                                             long long N, int d, long long np,
-                                                             const unsigned* __restrict__ amax,
-                                                             O* __restrict__ hi, O* __restrict__ lo) {
+// The same move of split fp32 for inputs whose rows allow 16-byte accesses (A aligned, lda % 4 == 0): a
+// 64 x 64 tile, four elements per access on both sides.  np is a multiple of 8, so a quad that starts below
+// np ends below it.
+__global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const float* __restrict__ A, long long lda, long long N,
+                                                             int d, long long np, const unsigned* __restrict__ amax,
+                                                             __half* __restrict__ hi, __half* __restrict__ lo) {
     grid_trigger();
-    __shared__ T tile[64][65];                       // [token][feature]
-    union Quad { V v; T e[4]; };
+    __shared__ float tile[64][65];                       // [token][feature]
     const int l = blockIdx.z;
     const long long t0 = (long long)blockIdx.x * 64;
     const int f0 = blockIdx.y * 64;
     const int q = threadIdx.x & 15, rr = threadIdx.x >> 4;
-    const T* Al = A + (size_t)l * (size_t)N * (size_t)lda;
+    const float* Al = A + (size_t)l * (size_t)N * (size_t)lda;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int tl = rr + 16 * k;
         const long long t = t0 + tl;
         const int f = f0 + 4 * q;
-        Quad u;
+        float u[4];
         if (t < N && f + 3 < d) {
-            u.v = *reinterpret_cast<const V*>(Al + (size_t)t * (size_t)lda + f);
+            const float4 x = *reinterpret_cast<const float4*>(Al + (size_t)t * (size_t)lda + f);
+            u[0] = x.x; u[1] = x.y; u[2] = x.z; u[3] = x.w;
         } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                u.e[e] = (t < N && f + e < d) ? Al[(size_t)t * (size_t)lda + f + e] : T(0);
+            for (int e = 0; e < 4; ++e) u[e] = (t < N && f + e < d) ? Al[(size_t)t * (size_t)lda + f + e] : 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) tile[tl][4 * q + e] = u.e[e];
+        for (int e = 0; e < 4; ++e) tile[tl][4 * q + e] = u[e];
     }
     __syncthreads();
 #pragma unroll
@@ -526,20 +522,55 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const T* __restrict
         const int f = f0 + fl;
         const long long t = t0 + 4 * q;
         if (f >= d || t >= np) continue;
-        Quad u;
+        const float sc = row_scale(amax[(size_t)l * d + f], false);
+        float y[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) u.e[e] = tile[4 * q + e][fl];
+        for (int e = 0; e < 4; ++e) y[e] = tile[4 * q + e][fl] * sc;
         const size_t o = ((size_t)l * d + f) * (size_t)np + (size_t)t;
-        if constexpr (SPLIT) {
-            union { uint2 v; __half e[4]; } h, w;
-            const float sc = row_scale(amax[(size_t)l * d + f], false);
+        split_f16x2(y, *reinterpret_cast<uint2*>(hi + o), *reinterpret_cast<uint2*>(lo + o));
+    }
+}
+
+// The same move of 16-bit elements whose rows start on 4 bytes (lda even), pairs of features at a time: 128
+// tokens x 64 features, 16 loads in flight per thread (a warp reads 128 bytes of a row), and eight tokens of
+// two features per thread put together from eight words, so that 256 bytes of a feature leave together.  The
+// words of a token lie permuted by the group of eight tokens: no bank conflicts on either side.
+// 4099 x 1322: 10.7 -> 6.7 us (32 x 32 elements one by one before).
+__global__ void __launch_bounds__(256) k_tokens16_to_kmajor(const uint16_t* __restrict__ A, long long lda, long long N,
+                                                            int d, long long np, uint16_t* __restrict__ out) {
+    grid_trigger();
+    __shared__ uint32_t tile[128 * 32];
+    const int l = blockIdx.z, f0 = blockIdx.y * 64, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long t0 = (long long)blockIdx.x * 128;
+    {
+        const int f = f0 + 2 * lane;
+        const uint16_t* src = A + ((size_t)l * (size_t)N + (size_t)t0 + warp) * (size_t)lda + f;
+        uint32_t v[16];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) split_f16x2(u.e[e] * sc, h.e[e], w.e[e]);
-            *reinterpret_cast<uint2*>(hi + o) = h.v;
-            *reinterpret_cast<uint2*>(lo + o) = w.v;
-        } else {
-            *reinterpret_cast<V*>(hi + o) = u.v;
+        for (int k = 0; k < 16; ++k, src += 8 * (size_t)lda) {
+            v[k] = 0u;
+            if (t0 + warp + 8 * k < N && f < d)
+                v[k] = f + 1 < d ? *reinterpret_cast<const uint32_t*>(src) : (uint32_t)*src;
         }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) tile[(warp + 8 * k) * 32 + (lane ^ k)] = v[k];
+    }
+    __syncthreads();
+    const int tg = threadIdx.x & 15;
+    const long long t = t0 + 8 * tg;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int w = warp + 8 * h + 16 * (lane >> 4), f = f0 + 2 * w;
+        uint32_t x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = tile[(8 * tg + k) * 32 + (w ^ tg)];
+        if (t >= np || f >= d) continue;
+        uint16_t* o = out + ((size_t)l * d + f) * (size_t)np + (size_t)t;
+        *reinterpret_cast<uint4*>(o) = make_uint4(__byte_perm(x[0], x[1], 0x5410), __byte_perm(x[2], x[3], 0x5410),
+                                                  __byte_perm(x[4], x[5], 0x5410), __byte_perm(x[6], x[7], 0x5410));
+        if (f + 1 < d)
+            *reinterpret_cast<uint4*>(o + np) = make_uint4(__byte_perm(x[0], x[1], 0x7632), __byte_perm(x[2], x[3], 0x7632),
+                                                           __byte_perm(x[4], x[5], 0x7632), __byte_perm(x[6], x[7], 0x7632));
     }
 }
 
@@ -686,8 +717,8 @@ ziplm_status run_tokens_split(const float* A, long long lda, int N, int d, long 
     return ZIPLM_OK;
 }
 
-bool quad_rows(const void* A, long long lda, size_t esz) {
-    return (reinterpret_cast<uintptr_t>(A) % (4 * esz)) == 0 && lda % 4 == 0;
+bool quad_rows(const void* A, long long lda) {
+    return (reinterpret_cast<uintptr_t>(A) % 16) == 0 && lda % 4 == 0;
 }
 
 // 3-D map over [layers, rows, K] with box {128 bytes of K, 128 rows, 1 layer}, 128-byte swizzle,
@@ -851,8 +882,8 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                                            (unsigned)zn), 256, 0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, slab,
                                                                         amax + (size_t)z0 * d);
                     ZIPLM_CHECK_LAUNCH();
-                    if (quad_rows(X, ldx, 4))
-                        k_tokens_to_kmajor_v4<float, float4, __half, true>
+                    if (quad_rows(X, ldx))
+                        k_tokens_to_kmajor_v4
                             <<<dim3((unsigned)((np + 63) / 64), (unsigned)((d + 63) / 64), (unsigned)zn), 256,
                                0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, np, amax + (size_t)z0 * d,
                                         hi + (size_t)z0 * d * np, lo + (size_t)z0 * d * np);
@@ -911,10 +942,9 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
         for (int l0 = 0; l0 < L; l0 += lc) {
             const int ln = (L - l0 < lc) ? (L - l0) : lc;
             const uint16_t* Ac = static_cast<const uint16_t*>(X) + (size_t)l0 * (size_t)N * ldx;
-            if (quad_rows(X, ldx, 2))
-                k_tokens_to_kmajor_v4<uint16_t, uint2, uint16_t, false>
-                    <<<dim3((unsigned)((np + 63) / 64), (unsigned)((d + 63) / 64), (unsigned)ln), 256, 0, st>>>(
-                        Ac, ldx, N, d, np, nullptr, xt, nullptr);
+            if (ldx % 2 == 0 && reinterpret_cast<uintptr_t>(X) % 4 == 0)
+                k_tokens16_to_kmajor<<<dim3((unsigned)((np + 127) / 128), (unsigned)((d + 63) / 64), (unsigned)ln), 256, 0,
+                                       st>>>(Ac, ldx, N, d, np, xt);
             else
                 k_tokens_to_kmajor<uint16_t, uint16_t, false>
                     <<<dim3((unsigned)((np + 31) / 32), (unsigned)((d + 31) / 32), (unsigned)ln), 256, 0, st>>>(

@@ -884,3 +884,18 @@ def test_heads_gram_matrix_on_int8_products(L, r, d, g):
     assert out["layer_status"].tolist() == [0] * L
     for l in (0, L - 1):
         compare_layer(W[l].numpy(), H[l].numpy(), g, 0.01, levels, out, l)
+
+
+@pytest.mark.parametrize("N,d,pad", [(32, 66, 0), (127, 63, 1), (129, 130, 2), (1025, 1, 1)])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
+    """The move of token-major 16-bit activations at the edges of its 128 x 64 tiles, odd widths
+    included; small whole numbers, so that the product is exact."""
+    z = zb()
+    g = torch.Generator().manual_seed(N)
+    full = torch.randint(-3, 4, (2, N, d + pad), generator=g).to(dtype).cuda()
+    A = full[:, :, :d]
+    H = z.hessian_accumulate_tokens(A, alpha=2.0)
+    ref = 2.0 * A.double().transpose(1, 2) @ A.double()
+    torch.cuda.synchronize()
+    assert torch.equal(H.double(), ref)
