@@ -168,7 +168,8 @@ class ClockSampler:
 # CUDA leg
 # ------------------------------------------------------------------------------------------
 LAZY_BLOCK = 32   # steps per block of the delayed-update neuron path (BMAX in prune_lazy.cu)
-LAZY_REFRESH = 64 # survivors at which that path rebuilds its state exactly (kRefresh there)
+LAZY_ENDGAME = 256  # survivors that go to the float64 endgame (kEndgame there) ...
+LAZY_ENDGAME_MIN = LAZY_ENDGAME - 2 * LAZY_BLOCK    # ... when at most this many are to remain
 LAZY_DEAD_MAX, LAZY_DEAD_FRACTION = 128, 16   # its rule for squeezing removed positions out (kDeadMax, kDeadFraction)
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch: constants from earlier
@@ -181,9 +182,6 @@ NCU_TRAFFIC = {
     # k_lazy_update_aq, a compaction block near full size (12 layers, n_new = 2944)
     "k_lazy_update_aq": dict(bytes=3 * (162.0e6 + 217.3e6), launch="n_new = 2944, m = 32, 12 layers",
                              algorithmic=12 * 24.0 * 2944 * 2943 / 2),
-    # k_dgemm_tiles, top-level product F21 = A21 M11^T
-    "k_dgemm_tiles": dict(bytes=3 * (116.6e6 + 49.0e6), launch="F21 = A21 M11^T, 12 x 24 macro tiles",
-                          algorithmic=None),
     # k_neuron_update, first step at full size (12 layers, n = 3071)
     "k_neuron_update": dict(bytes=343.1e6 + 281.9e6, launch="n = 3071, 12 layers",
                             algorithmic=12 * (8.0 * 768 * 3071 + 4.0 * 3071 * 3071)),
@@ -198,19 +196,21 @@ def lazy_update_work(L, G, levels, r=0):
     4 B x (1 read + 2 writes)) and spends 3 fp32 FMA per pair and pending step.  In the dense
     blocks the same kernel also updates W^T: 8 B x r x n (read + write of the live weights), counted
     separately.  Rows and columns of removed positions that a dense block still carries are
-    overhead, not counted here.  Block boundaries, and which blocks are dense, as in the library.
+    overhead, not counted here, and neither is the endgame.  Block boundaries, and which blocks are
+    dense, as in the library.
     Returns (bytes, fma, launches, bytes of W^T in the dense blocks)."""
     n, npos, slot, nbytes, fma, launches, wbytes = G, G, 0, 0.0, 0.0, 0, 0.0
     levels = [v for v in levels if v < G]
     n_min = levels[-1] if levels else G
-    while n > n_min:
+    endgame = n_min <= LAZY_ENDGAME_MIN
+    while n > (LAZY_ENDGAME if endgame else n_min):
         stop = levels[slot] if slot < len(levels) else n_min
-        if n > LAZY_REFRESH and stop < LAZY_REFRESH:
-            stop = LAZY_REFRESH          # the exact rebuild of the state ends a block
+        if endgame:
+            stop = max(stop, LAZY_ENDGAME)
         m = min(LAZY_BLOCK, n - stop)
         dead_after = npos - (n - m)
-        refresh = n > LAZY_REFRESH and n - m == LAZY_REFRESH
-        compact = refresh or dead_after >= LAZY_DEAD_MAX or dead_after * LAZY_DEAD_FRACTION >= npos
+        last = endgame and n - m == LAZY_ENDGAME
+        compact = last or dead_after >= LAZY_DEAD_MAX or dead_after * LAZY_DEAD_FRACTION >= npos
         n -= m
         npos = n if compact else npos
         if n > 1:
@@ -664,7 +664,7 @@ def run_ours(args, shape):
         prod_ms, prod_n = phases.get("inverse_products", (0.0, 0))
         prod_flop = L * (2.0 / 3.0) * float(d) ** 3
         prod_tflops = prod_flop / (prod_ms * 1e-3) / 1e12 if prod_ms > 0 else 0.0
-        fp64_peak = 37.0      # TFLOP/s, measured with a register-only loop of the float64 mma instruction
+        i8_peak = 4500.0      # TOP/s, nominal dense int8 rate of tcgen05.mma kind::i8
         aq_ms, aq_n = phases.get("lazy_update_aq", (0.0, 0))
         aq_only_bytes, aq_fma, _, aq_w_bytes = lazy_update_work(L, G, levels, r)
         aq_bytes = aq_only_bytes + aq_w_bytes
@@ -705,17 +705,14 @@ def run_ours(args, shape):
                           "step k; single_batch_ms is one such step on its own"),
             gpu_launches=int(launches),
             clocks=clocks,
-            roofline_inverse_products=dict(kernel="k_dgemm_tiles + k_dgemm_pair", bound="alu", achieved=prod_tflops, peak=fp64_peak,
-                          unit="TFLOP/s", frac=prod_tflops / fp64_peak,
-                          traffic=NCU_TRAFFIC["k_dgemm_tiles"]["bytes"] if full_workload else None,
-                          traffic_note=NCU_TRAFFIC["k_dgemm_tiles"],
+            roofline_inverse_products=dict(kernel="k_i8_product", bound="tensor", achieved=36 * prod_tflops, peak=i8_peak,
+                          unit="TOP/s", frac=36 * prod_tflops / i8_peak, traffic=None,
                           launches=prod_n, avg_launch_us=1e3 * prod_ms / max(prod_n, 1),
-                          algorithmic_flop_per_step=prod_flop,
-                          peak_source="measured: register-only loop of mma.sync.m8n8k4.f64, 37.0 TFLOP/s "
-                                      "(plain FMA loop 36.5; nominal 148 SMs x 64 lanes x 2 x 1.965 GHz "
-                                      "= 37.2)",
-                          note="float64 tile products of the Cholesky factor and its inverse "
-                               "(2/3 d^3 flop per layer)"),
+                          algorithmic_flop_per_step=prod_flop, float64_tflops=prod_tflops,
+                          peak_source="nominal dense int8 rate",
+                          note="float64 products of the Cholesky factor and its inverse (2/3 d^3 flop per "
+                               "layer), each as 36 int8 products of digits; the digits' kernels and the blocks "
+                               "below 512 rows, on the float64 instruction (37 TFLOP/s measured), are in the time"),
             roofline=dict(kernel="k_lazy_update_aq_tc (dense blocks) + k_lazy_update_aq (compaction blocks)",
                           bound="hbm", achieved=aq_gbs, peak=peak,
                           unit="GB/s", frac=aq_gbs / peak,

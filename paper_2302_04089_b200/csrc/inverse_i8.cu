@@ -14,7 +14,10 @@
 // of tensor memory), first the digits 4 .. 7 (10 products), then all (26).  A K block is 64 digits (64-byte
 // swizzle): eight slices of both operands fill half of the shared-memory ring, 96 KB for 3328 clocks of
 // MMAs, so the operand traffic stays at 30 bytes per clock and SM.
-// INVERSE_I8_FIGURES
+// Inverse of 12 x 3072: 14.7 -> 9.7 ms, of 24 x 4096: 57 -> 33.6 ms (float64 instruction before).  The tensor
+// pipe bounds it: an MMA of M = 256, N = 128, K = 32 takes 96 clocks in place of 64 (6900 clocks a K block).
+// Tiles of 256 x 256 (163 clocks an MMA in place of 128, a quarter of the drains four times as often through
+// scratch) were slower, 128-byte swizzled rows of two digits the same.
 #include <cuda.h>
 
 #include "common.cuh"

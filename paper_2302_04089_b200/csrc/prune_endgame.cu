@@ -16,7 +16,8 @@
 //                     forward substitution, rank-32 updates, and the snapshot of every level on the way;
 //   k_endgame_loss    losses.
 //
-// One layer of 64 x 256 (192 steps, three levels): 0.715 -> MEASURED ms.
+// One layer of 64 x 256 (192 steps, three levels): 1.08 -> 0.36 ms a whole call, of which the steps 0.205 and the
+// factorisation 0.07 (0.72 ms for the loop alone with pending updates, a launch every 32 steps).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(256) k_endgame_setup(const __grid_constant__ E
 // u and the bookkeeping of all steps are kept in shared memory and written out at the end.
 // One layer of 256: a version that pushed every CTA's offered row of 2 x 256 doubles to all others took
 // 2.5 us a step, half of it those stores and the cluster barrier behind them; with this exchange and a
-// cluster barrier 1.8 us; as it stands STEP_US us.
+// cluster barrier 1.8 us; as it stands 1.05 us.
 template <int CS, int S, int CPL> struct StepsCfg {
     static constexpr int RG = S / 4, CG = WORKERS / RG, NP = CG * 32 * CPL, E = (S + 31) / 32;
 };

@@ -124,7 +124,8 @@ __device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
 // a cluster barrier, and every fence, would wait for it.  What the update kernels need -- u, z and the
 // step order -- goes out at the end of the block, for a dense block as the packed operands themselves.
 // (Clocks per step at 3072 positions: 5200 with the comparisons one after the other and the pending
-// entries fetched after the pick; 3700 with a cluster barrier and u, z stored step by step; STEP_CLOCKS.)
+// entries fetched after the pick; 3700 with a cluster barrier and u, z stored step by step; 2800 to
+// 3300 now.)
 //
 // The scaled pivot columns of W (c_s) do not feed the selection; they are solved for at the end
 // of the block by forward substitution with the 32 x 32 triangle T[m][s] = u_s[p_m].
