@@ -21,7 +21,9 @@ struct HessianProduct {
 };
 
 // Whether the kernel on CTA pairs takes a launch of that many layers.
-bool hessian_pair_fits(int layers, int d);
+bool hessian_pair_fits(int layers, int d, long long N);
+// CTAs that share a 128 x 128 tile of the other one.
+int hessian_tile_split(long long tiles, long long num_kb);
 size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split);
 ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st);
 

@@ -78,17 +78,92 @@ __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t 
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
-// Arrive at the barrier at this offset in both CTAs once the MMAs issued so far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+// Arrive at the barrier at this offset in the pair's two CTAs (a mask of cluster ranks) once the MMAs issued
+// so far have completed.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t both) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        ::"r"(bar), "h"((uint16_t)3) : "memory");
+        ::"r"(bar), "h"(both) : "memory");
+}
+
+// The end of a tile that n_parts pairs have shared.  Every thread of the cluster's CTAs comes here once the
+// parts' sums are in shared memory, [16 quads][512 threads].  Part p finishes the quads [16 p / n, 16 (p + 1) / n)
+// of every epilogue thread's 64 columns: sums over the parts in order, rows along the columns, mirrored rows
+// along the rows.
+template <bool SPLIT>
+__device__ __forceinline__ void finish_parts(uint8_t* ring, int n_parts, int part, int rank, int i0, int j0, int d,
+                                             float alpha, float beta, float* Hl, const unsigned* am,
+                                             const unsigned long long* err_word, unsigned long long call, bool give_up) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, et = (int)threadIdx.x - 64;
+    const int g0 = 16 * part / n_parts, n = 16 * (part + 1) / n_parts - g0;      // at most eight quads
+    float4 sum[8];
+    if (warp >= 2) {
+        const uint32_t mine = smem_u32(ring) + 16u * (uint32_t)(g0 * (32 * PAIR_EPI) + et);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = 0; p < n_parts; ++p) {
+            const uint32_t from = cluster_addr(mine, 2u * (uint32_t)p + (uint32_t)rank);
+            float4 x[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e < n)
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(x[e].x), "=f"(x[e].y), "=f"(x[e].z), "=f"(x[e].w)
+                                 : "r"(from + 16u * (uint32_t)(e * 32 * PAIR_EPI)) : "memory");
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e < n) { sum[e].x += x[e].x; sum[e].y += x[e].y; sum[e].z += x[e].z; sum[e].w += x[e].w; }
+        }
+    }
+    __syncwarp();
+    cluster_barrier();                                    // all have read: the sums' place is free
+    if (warp < 2 || give_up) return;
+    const int q = warp & 3, cols = 4 * n;
+    const int r0 = i0 + rank * HALF + q * 32, c0 = j0 + ((warp - 2) >> 2) * NC + 4 * g0;
+    float* buf = reinterpret_cast<float*>(ring) + (warp - 2) * (32 * 33);
+    const float mul = (SPLIT && r0 + lane < d) ? row_scale(am[r0 + lane], true) : 1.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        if (e < n) {
+            float* b = buf + lane * 33 + 4 * e;
+            b[0] = (alpha * sum[e].x) * mul;
+            b[1] = (alpha * sum[e].y) * mul;
+            b[2] = (alpha * sum[e].z) * mul;
+            b[3] = (alpha * sum[e].w) * mul;
+        }
+    __syncwarp();
+    const int col = c0 + lane;
+    const float sc = SPLIT && lane < cols && col < d ? row_scale(am[col], true) : 1.f;
+#pragma unroll 1
+    for (int g = 0; g < 32; g += 16) {
+        float old[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int row = r0 + g + k;
+            old[k] = beta != 0.f && lane < cols && row < d && col <= row ? Hl[(size_t)row * d + col] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int row = r0 + g + k;
+            if (lane >= cols || row >= d || col > row) continue;
+            const float v = buf[(g + k) * 33 + lane] * sc + old[k];
+            buf[(g + k) * 33 + lane] = v;
+            float* p = Hl + (size_t)row * d + col;
+            *p = v;
+            if ((row | col) == 0) hessian_check(p, err_word, call);
+        }
+    }
+    __syncwarp();
+    const int row = r0 + lane;
+#pragma unroll 4
+    for (int e = 0; e < cols; ++e)
+        if (row < d && c0 + e < row) Hl[(size_t)(c0 + e) * d + row] = buf[lane * 33 + e];
 }
 
 template <bool SPLIT>
-__global__ void __launch_bounds__(PAIR_THREADS, 1) __cluster_dims__(2, 1, 1)
+__global__ void __launch_bounds__(PAIR_THREADS, 1)
 k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-            float* __restrict__ H, int d, int num_kb, float alpha, float beta, int layer0,
+            float* __restrict__ H, int d, int num_kb_all, int n_parts, float alpha, float beta, int layer0,
             int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
             const unsigned* __restrict__ amax, float4* __restrict__ level2) {
     using C = PairCfg<SPLIT>;
@@ -100,9 +175,15 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;        // swizzled tiles need 1024-byte alignment
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a cluster of n_parts pairs shares a tile, each a range of its K blocks
     const uint32_t rank = blockIdx.x & 1u;                // CTA of the pair; 0 leads
+    const int part = (int)(blockIdx.x >> 1) % n_parts;
+    const uint32_t lead = 2u * (uint32_t)part;            // cluster rank of the pair's leader
+    const uint16_t both = (uint16_t)(3u << lead);
+    const int kb_begin = (int)((long long)num_kb_all * part / n_parts);
+    const int num_kb = (int)((long long)num_kb_all * (part + 1) / n_parts) - kb_begin;
     const int l = blockIdx.y;                             // layer within the launched chunk
-    int ti = 0, rem = (int)(blockIdx.x >> 1);
+    int ti = 0, rem = (int)(blockIdx.x >> 1) / n_parts;
     while (rem > ti) { rem -= ti + 1; ++ti; }
     const int tj = rem;
     const int i0 = ti * PT, j0 = tj * PT;
@@ -142,7 +223,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
             // ---------------- TMA producer (each CTA its own half of the operands)
             const uint32_t bytes = (uint32_t)((diag ? 1 : 2) * C::PARTS * OP_BYTES);
             const int ya = i0 + (int)rank * HALF, yb = j0 + (int)rank * HALF;
-            const uint32_t full0 = cluster_addr(smem_u32(&bar_full[0]), 0);
+            const uint32_t full0 = cluster_addr(smem_u32(&bar_full[0]), lead);
             int s = 0;
             uint32_t ph = 1u;
             for (int kb = 0; kb < num_kb; ++kb) {
@@ -153,7 +234,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                 const uint32_t full = full0 + 8u * (uint32_t)s;
                 const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
                 if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2 * bytes);
-                const int x = kb * BK;
+                const int x = (kb_begin + kb) * BK;
                 tma_load_3d_pair(base, &map_hi, full, x, ya, l);
                 if (SPLIT) tma_load_3d_pair(base + OP_BYTES, &map_lo, full, x, ya, l);
                 if (!diag) {
@@ -200,22 +281,22 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
                         umma_pair(acc, a_hi + 2u * k, b_hi + 2u * k, idesc, SPLIT || k > 0 || j > 0);
-                    umma_commit_pair(smem_u32(&bar_empty[s]));     // stage free once these MMAs have read it
+                    umma_commit_pair(smem_u32(&bar_empty[s]), both);     // stage free once these MMAs have read it
                     ++kb;
                     if (++s == C::STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (!failed) umma_commit_pair(smem_u32(&bar_acc_full[b]));
+                if (!failed) umma_commit_pair(smem_u32(&bar_acc_full[b]), both);
             }
             // whatever was issued has completed before tensor memory is given back
-            umma_commit_pair(smem_u32(&bar_final));
+            umma_commit_pair(smem_u32(&bar_final), both);
             mbar_wait_quiet(smem_u32(&bar_final), 0u);
         }
     } else {
         // ---------------- epilogue: lane quarter = warp % 4, quarter of the columns by warp
         const int q = warp & 3, cq = (warp - 2) >> 2;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        const uint32_t empty0 = cluster_addr(smem_u32(&bar_acc_empty[0]), 0);
-        const uint32_t empty1 = cluster_addr(smem_u32(&bar_acc_empty[1]), 0);
+        const uint32_t empty0 = cluster_addr(smem_u32(&bar_acc_empty[0]), lead);
+        const uint32_t empty1 = cluster_addr(smem_u32(&bar_acc_empty[1]), lead);
         const int et = (int)threadIdx.x - 64;
         float4* l2 = level2 + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (HALF * PT / 4) + et;
         float acc[NC];
@@ -261,90 +342,98 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                     const float4 t = __ldcg(l2 + (size_t)e * (32 * PAIR_EPI));
                     acc[4 * e] += t.x; acc[4 * e + 1] += t.y; acc[4 * e + 2] += t.z; acc[4 * e + 3] += t.w;
                 }
-            // The operand ring is free (every MMA has completed): the warp's 32 x 64 results pass
-            // through it, so that rows [i][j] leave along j and mirrored rows [j][i] along i.  The old values
-            // of several rows are requested together: a load behind every row's store made a call with
-            // beta = 1 take 1056 us where beta = 0 took 667 (12 x 3072 x 2048 fp32).
-            float* buf = reinterpret_cast<float*>(smem_raw + (tiles - raw)) + (size_t)(warp - 2) * 32 * OUT_PITCH;
-            float* Hl = H + (size_t)(layer0 + l) * d * d;
-            const int r0 = i0 + (int)rank * HALF + q * 32, c0 = j0 + cq * NC;
-            const unsigned* am = SPLIT ? amax + (size_t)l * d : nullptr;
-            // split route: undo the power-of-two scales of the two feature rows (exact)
-            const float mul = (SPLIT && r0 + lane < d) ? row_scale(am[r0 + lane], true) : 1.f;
+            if (n_parts > 1) {
+                // The operand ring is free (every MMA has completed): the part's sums wait there for finish_parts.
+                float4* mine = reinterpret_cast<float4*>(smem_raw + (tiles - raw)) + et;
 #pragma unroll
-            for (int e = 0; e < NC; e += 4)
-                *reinterpret_cast<float4*>(buf + lane * OUT_PITCH + e) =
-                    make_float4((alpha * acc[e]) * mul, (alpha * acc[e + 1]) * mul, (alpha * acc[e + 2]) * mul,
-                                (alpha * acc[e + 3]) * mul);
-            __syncwarp();
-            if (!diag && d % 4 == 0 && r0 + 32 <= d) {
-                // whole rows below the diagonal: 16 lanes take one, 16 bytes each
-                const int cc = 4 * (lane & 15);
-                float sc[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) sc[e] = SPLIT ? row_scale(am[c0 + cc + e], true) : 1.f;
-                float4* out = reinterpret_cast<float4*>(Hl + (size_t)(r0 + (lane >> 4)) * d + c0 + cc);
-                float4* in = reinterpret_cast<float4*>(buf + (lane >> 4) * OUT_PITCH + cc);
-#pragma unroll
-                for (int g = 0; g < 16; g += FLY) {
-                    float4 old[FLY];
-                    if (beta != 0.f)
-#pragma unroll
-                        for (int k = 0; k < FLY; ++k) old[k] = out[(size_t)(g + k) * (2 * (d / 4))];
-#pragma unroll
-                    for (int k = 0; k < FLY; ++k) {
-                        float4 v = in[(g + k) * (2 * OUT_PITCH / 4)];
-                        v.x *= sc[0]; v.y *= sc[1]; v.z *= sc[2]; v.w *= sc[3];
-                        if (beta != 0.f) { v.x += old[k].x; v.y += old[k].y; v.z += old[k].z; v.w += old[k].w; }
-                        out[(size_t)(g + k) * (2 * (d / 4))] = v;
-                        in[(g + k) * (2 * OUT_PITCH / 4)] = v;
-                    }
-                }
-                __syncwarp();
-                float* mir = Hl + (size_t)c0 * d + r0 + lane;
-#pragma unroll
-                for (int e = 0; e < NC; e += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(buf + lane * OUT_PITCH + e);
-                    mir[(size_t)e * d] = v.x;
-                    mir[(size_t)(e + 1) * d] = v.y;
-                    mir[(size_t)(e + 2) * d] = v.z;
-                    mir[(size_t)(e + 3) * d] = v.w;
-                }
+                for (int e = 0; e < NC / 4; ++e)
+                    mine[e * (32 * PAIR_EPI)] = make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]);
             } else {
-                float sc[NC / 32];
+                // The operand ring is free (every MMA has completed): the warp's 32 x 64 results pass
+                // through it, so that rows [i][j] leave along j and mirrored rows [j][i] along i.  The old values
+                // of several rows are requested together: a load behind every row's store made a call with
+                // beta = 1 take 1056 us where beta = 0 took 667 (12 x 3072 x 2048 fp32).
+                float* buf = reinterpret_cast<float*>(smem_raw + (tiles - raw)) + (size_t)(warp - 2) * 32 * OUT_PITCH;
+                float* Hl = H + (size_t)(layer0 + l) * d * d;
+                const int r0 = i0 + (int)rank * HALF + q * 32, c0 = j0 + cq * NC;
+                const unsigned* am = SPLIT ? amax + (size_t)l * d : nullptr;
+                // split route: undo the power-of-two scales of the two feature rows (exact)
+                const float mul = (SPLIT && r0 + lane < d) ? row_scale(am[r0 + lane], true) : 1.f;
 #pragma unroll
-                for (int h = 0; h < NC / 32; ++h)
-                    sc[h] = SPLIT && c0 + 32 * h + lane < d ? row_scale(am[c0 + 32 * h + lane], true) : 1.f;
-#pragma unroll 1
-                for (int g = 0; g < 32; g += FLY) {
-                    float old[FLY][NC / 32];
-#pragma unroll
-                    for (int k = 0; k < FLY; ++k)
-#pragma unroll
-                        for (int h = 0; h < NC / 32; ++h) {
-                            const int row = r0 + g + k, col = c0 + 32 * h + lane;
-                            old[k][h] = beta != 0.f && row < d && col <= row ? Hl[(size_t)row * d + col] : 0.f;
-                        }
-#pragma unroll
-                    for (int k = 0; k < FLY; ++k)
-#pragma unroll
-                        for (int h = 0; h < NC / 32; ++h) {
-                            const int row = r0 + g + k, col = c0 + 32 * h + lane;
-                            if (row >= d || col > row) continue;
-                            float* b = buf + (g + k) * OUT_PITCH + 32 * h + lane;
-                            const float v = *b * sc[h] + old[k][h];
-                            *b = v;
-                            float* p = Hl + (size_t)row * d + col;
-                            *p = v;
-                            if ((row | col) == 0) hessian_check(p, err_word, call);
-                        }
-                }
+                for (int e = 0; e < NC; e += 4)
+                    *reinterpret_cast<float4*>(buf + lane * OUT_PITCH + e) =
+                        make_float4((alpha * acc[e]) * mul, (alpha * acc[e + 1]) * mul, (alpha * acc[e + 2]) * mul,
+                                    (alpha * acc[e + 3]) * mul);
                 __syncwarp();
-                const int row = r0 + lane;
+                if (!diag && d % 4 == 0 && r0 + 32 <= d) {
+                    // whole rows below the diagonal: 16 lanes take one, 16 bytes each
+                    const int cc = 4 * (lane & 15);
+                    float sc[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sc[e] = SPLIT ? row_scale(am[c0 + cc + e], true) : 1.f;
+                    float4* out = reinterpret_cast<float4*>(Hl + (size_t)(r0 + (lane >> 4)) * d + c0 + cc);
+                    float4* in = reinterpret_cast<float4*>(buf + (lane >> 4) * OUT_PITCH + cc);
+#pragma unroll
+                    for (int g = 0; g < 16; g += FLY) {
+                        float4 old[FLY];
+                        if (beta != 0.f)
+#pragma unroll
+                            for (int k = 0; k < FLY; ++k) old[k] = out[(size_t)(g + k) * (2 * (d / 4))];
+#pragma unroll
+                        for (int k = 0; k < FLY; ++k) {
+                            float4 v = in[(g + k) * (2 * OUT_PITCH / 4)];
+                            v.x *= sc[0]; v.y *= sc[1]; v.z *= sc[2]; v.w *= sc[3];
+                            if (beta != 0.f) { v.x += old[k].x; v.y += old[k].y; v.z += old[k].z; v.w += old[k].w; }
+                            out[(size_t)(g + k) * (2 * (d / 4))] = v;
+                            in[(g + k) * (2 * OUT_PITCH / 4)] = v;
+                        }
+                    }
+                    __syncwarp();
+                    float* mir = Hl + (size_t)c0 * d + r0 + lane;
+#pragma unroll
+                    for (int e = 0; e < NC; e += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(buf + lane * OUT_PITCH + e);
+                        mir[(size_t)e * d] = v.x;
+                        mir[(size_t)(e + 1) * d] = v.y;
+                        mir[(size_t)(e + 2) * d] = v.z;
+                        mir[(size_t)(e + 3) * d] = v.w;
+                    }
+                } else {
+                    float sc[NC / 32];
+#pragma unroll
+                    for (int h = 0; h < NC / 32; ++h)
+                        sc[h] = SPLIT && c0 + 32 * h + lane < d ? row_scale(am[c0 + 32 * h + lane], true) : 1.f;
+#pragma unroll 1
+                    for (int g = 0; g < 32; g += FLY) {
+                        float old[FLY][NC / 32];
+#pragma unroll
+                        for (int k = 0; k < FLY; ++k)
+#pragma unroll
+                            for (int h = 0; h < NC / 32; ++h) {
+                                const int row = r0 + g + k, col = c0 + 32 * h + lane;
+                                old[k][h] = beta != 0.f && row < d && col <= row ? Hl[(size_t)row * d + col] : 0.f;
+                            }
+#pragma unroll
+                        for (int k = 0; k < FLY; ++k)
+#pragma unroll
+                            for (int h = 0; h < NC / 32; ++h) {
+                                const int row = r0 + g + k, col = c0 + 32 * h + lane;
+                                if (row >= d || col > row) continue;
+                                float* b = buf + (g + k) * OUT_PITCH + 32 * h + lane;
+                                const float v = *b * sc[h] + old[k][h];
+                                *b = v;
+                                float* p = Hl + (size_t)row * d + col;
+                                *p = v;
+                                if ((row | col) == 0) hessian_check(p, err_word, call);
+                            }
+                    }
+                    __syncwarp();
+                    const int row = r0 + lane;
 #pragma unroll 4
-                for (int e = 0; e < NC; ++e) {
-                    const int col = c0 + e;
-                    if (row < d && col < row) Hl[(size_t)col * d + row] = buf[lane * OUT_PITCH + e];
+                    for (int e = 0; e < NC; ++e) {
+                        const int col = c0 + e;
+                        if (row < d && col < row) Hl[(size_t)col * d + row] = buf[lane * OUT_PITCH + e];
+                    }
                 }
             }
         }
@@ -353,7 +442,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     if (failed) {
         hessian_give_up(H, L, d, err_word, call);
         for (uint32_t r = 0; r < 2; ++r)
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), r)), "r"(1)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), lead + r)), "r"(1)
                          : "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -367,6 +456,10 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     }
     __syncwarp();
     cluster_barrier();            // the pair's MMAs, copies and remote arrivals are over
+    if (n_parts > 1)
+        finish_parts<SPLIT>(smem_raw + (tiles - raw), n_parts, part, (int)rank, i0, j0, d, alpha, beta,
+                            H + (size_t)(layer0 + l) * d * d, SPLIT ? amax + (size_t)l * d : nullptr, err_word, call,
+                            abort_flag != 0);
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
     }
@@ -377,22 +470,38 @@ int pair_count(int d) {
     return T * (T + 1) / 2;
 }
 
+// Pairs that share a tile where the tiles leave SMs idle: as many as fit at once (the occupancy calculator
+// gives room for MOST_CLUSTERS clusters of that many pairs; one tile more makes a second wave) with four K
+// blocks each.  8 x 512 features, 2048 bf16 tokens: 39.8 -> 29.7 us a call, 2 x 1100 of 500 fp32 37.7 -> 27.6,
+// 1 x 1322 of 4099 64.5 -> 58.3.
+int parts_of(long long pairs, long long kb) {
+    constexpr int MOST_CLUSTERS[5] = {0, 74, 33, 22, 15};
+    int parts = 1;
+    for (int p = 2; p <= 4; ++p)
+        if (pairs <= MOST_CLUSTERS[p] && kb / p >= 4) parts = p;
+    return parts;
+}
+
 template <bool SPLIT>
 ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t st) {
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_pair<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           kPairSmem<SPLIT>));
+    const int parts = parts_of((long long)pair_count(p.d) * p.layers, p.num_kb);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pair_count(p.d), p.layers);
+    cfg.gridDim = dim3(2 * parts * pair_count(p.d), p.layers);
     cfg.blockDim = dim3(PAIR_THREADS);
     cfg.dynamicSmemBytes = kPairSmem<SPLIT>;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2 * parts;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_syrk_pair<SPLIT>, p.hi, p.lo, p.H, p.d, p.num_kb, p.alpha, p.beta,
-                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, level2));
+    cfg.numAttrs = 2;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_syrk_pair<SPLIT>, p.hi, p.lo, p.H, p.d, p.num_kb, parts, p.alpha,
+                                        p.beta, p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, level2));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }
@@ -401,18 +510,22 @@ ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t s
 
 // A K block of a 256 x 256 tile takes a pair about 4/3 of the time that one of a 128 x 128 tile takes a CTA
 // (12 MMAs of 128 clocks against 12 of 92, where the shared-memory reads of a 128 x 128 MMA bound it), so
-// the pair kernel wins where it needs fewer than three quarters of the waves.
-bool hessian_pair_fits(int layers, int d) {
-    const long long T = (d + HALF - 1) / HALF, tiles = T * (T + 1) / 2 * layers, pairs = (long long)pair_count(d) * layers;
-    return 4 * ((pairs + 73) / 74) < 3 * ((tiles + 147) / 148);
+// the pair kernel wins where a chain of its K blocks over all waves is shorter than three quarters of the other's.
+bool hessian_pair_fits(int layers, int d, long long N) {
+    const long long kb = (N + BK - 1) / BK, T = (d + HALF - 1) / HALF, tiles = T * (T + 1) / 2 * layers;
+    const long long pairs = (long long)pair_count(d) * layers, parts = parts_of(pairs, kb);
+    const long long split = hessian_tile_split(tiles, kb);
+    const long long chain = (pairs * parts + 73) / 74 * ((kb + parts - 1) / parts);
+    return 4 * chain < 3 * ((tiles * split + 147) / 148 * ((kb + split - 1) / split));
 }
 
 // Scratch of the second summation level, for the layers of one launch; none where FOLD drains are
 // never reached.
 size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split) {
     const long long kb = (N + BK - 1) / BK, per = split ? PairCfg<true>::CHUNK : PairCfg<false>::CHUNK;
-    if ((kb + per - 1) / per <= FOLD) return 0;
-    return (size_t)layers * 2 * pair_count(d) * HALF * PT * sizeof(float);
+    const long long pairs = (long long)pair_count(d) * layers, parts = parts_of(pairs, kb);
+    if (((kb + parts - 1) / parts + per - 1) / per <= FOLD) return 0;
+    return (size_t)2 * pairs * parts * HALF * PT * sizeof(float);
 }
 
 ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st) {

@@ -770,6 +770,15 @@ int product_layers(int L, int d, long long N, ziplm_dtype dt, bool token_major) 
 
 }  // namespace
 
+// Where the 128 x 128 tiles leave half of the SMs idle, up to eight CTAs share a tile: the largest power of
+// two with which all fit and each keeps four K blocks (one layer of 256 features, 2048 tokens: three tiles,
+// a chain of 32 K blocks on one CTA).
+int hessian_tile_split(long long tiles, long long num_kb) {
+    int split = 1;
+    while (split < 8 && tiles * split * 2 <= 148 && num_kb / (split * 2) >= 4) split *= 2;
+    return split;
+}
+
 size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, bool token_major) {
     size_t b = kAlign;   // error word
     if (dt == ZIPLM_F32) {
@@ -781,7 +790,7 @@ size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, boo
         b += align_up((size_t)lc * d * (size_t)padded_tokens_bf16(N) * 2);
     }
     const int layers = product_layers(L, d, N, dt, token_major);
-    if (hessian_pair_fits(layers, d)) b += align_up(hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32));
+    if (hessian_pair_fits(layers, d, N)) b += align_up(hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32));
     return b;
 }
 
@@ -794,15 +803,12 @@ unsigned long long next_call() {
     return calls.fetch_add(0x9e3779b97f4a7c15ull) | 1ull;
 }
 
-// One product launch on the kernel that suits its number of tiles.  Where the 128 x 128 tiles leave half of
-// the SMs idle, up to eight CTAs share a tile: the largest power of two with which all fit and each keeps
-// four K blocks (one layer of 256 features, 2048 tokens: three tiles, a chain of 32 K blocks on one CTA).
+// One product launch on the kernel that suits its number of tiles.
 ziplm_status run_product(const HessianProduct& p, void* scratch, cudaStream_t st) {
-    if (hessian_pair_fits(p.layers, p.d)) return run_hessian_pair(p, scratch, st);
+    if (hessian_pair_fits(p.layers, p.d, (long long)p.num_kb * 64)) return run_hessian_pair(p, scratch, st);
     const int T = (p.d + TM - 1) / TM;
     const long long tiles = (long long)T * (T + 1) / 2 * p.layers;
-    int split = 1;
-    while (split < 8 && tiles * split * 2 <= 148 && p.num_kb / (split * 2) >= 4) split *= 2;
+    const int split = hessian_tile_split(tiles, p.num_kb);
     constexpr int smem2 = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
     constexpr int smem1 = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
     static_assert(2 * TM * OUT_PITCH * (int)sizeof(float) + 1024 <= smem1, "finished tiles fit the operand ring");
@@ -848,7 +854,7 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
     const int most_layers = product_layers(L, d, N, dt, token_major);
     void* scratch = nullptr;             // of the pair kernel, behind the operands
     auto take_scratch = [&] {
-        if (hessian_pair_fits(most_layers, d))
+        if (hessian_pair_fits(most_layers, d, N))
             scratch = c.take<char>(hessian_pair_scratch_bytes(most_layers, d, N, f32));
     };
     if (f32) {

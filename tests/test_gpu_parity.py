@@ -899,3 +899,18 @@ def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
     ref = 2.0 * A.double().transpose(1, 2) @ A.double()
     torch.cuda.synchronize()
     assert torch.equal(H.double(), ref)
+
+
+@pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030)])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
+def test_hessian_tiles_shared_by_pairs_of_ctas(L, d, N, dtype):
+    """Two, three and four pairs to a 256 x 256 tile, ragged K and widths, added to what is there; small
+    whole numbers, so that every sum is exact."""
+    z = zb()
+    g = torch.Generator().manual_seed(d)
+    A = torch.randint(-3, 4, (L, N, d), generator=g).to(dtype).cuda()
+    ref = A.double().transpose(1, 2) @ A.double()
+    H = z.hessian_accumulate_tokens(A, alpha=2.0)
+    assert torch.equal(H.double(), 2.0 * ref)
+    H = z.hessian_accumulate_tokens(A, H, alpha=1.0, beta=1.0)
+    assert torch.equal(H.double(), 3.0 * ref)
