@@ -308,14 +308,15 @@ __device__ __forceinline__ void dgemm_task(const GemmTask& t, int dp, int bx, in
     double* out = t.C + lay + (size_t)((t.c_r + 2 * I) * kTile + 32 * (warp >> 1)) * dp +
                   (size_t)(t.c_c + J) * kTile + 32 * (warp & 1);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
+        double2* o = reinterpret_cast<double2*>(out + (size_t)(8 * i + (lane >> 2)) * dp + 2 * (lane & 3));
+        double2 cur[4];                        // four old values in flight, not each behind the store before it
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            double2* o = reinterpret_cast<double2*>(out + (size_t)(8 * i + (lane >> 2)) * dp + 8 * j + 2 * (lane & 3));
-            double2 v = make_double2(t.alpha * acc.d[i][j][0], t.alpha * acc.d[i][j][1]);
-            if (t.beta) { const double2 c = *o; v.x += c.x; v.y += c.y; }
-            *o = v;
-        }
+        for (int j = 0; j < 4; ++j) cur[j] = t.beta ? o[4 * j] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            o[4 * j] = make_double2(fma(t.alpha, acc.d[i][j][0], cur[j].x), fma(t.alpha, acc.d[i][j][1], cur[j].y));
+    }
 }
 
 template <bool TA, bool TB>
@@ -406,8 +407,8 @@ __device__ __forceinline__ void small_epilogue(const SmallAcc& acc, Fn f) {
             f(r0 + 8 * i, c0 + 8 * j, make_double2(acc.d[i][j][0], acc.d[i][j][1]));
 }
 
-// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag -> Mg (lower, upper part zeroed).
-// The factor itself is not needed.  Starts and ends with a barrier.
+// Leaf: the inverse M of the Cholesky factor of the 64 x 64 tile at Ag (null: it is in sm.ta) -> Mg (lower, upper
+// part zeroed), and left in sm.tb.  The factor itself is not needed.  Starts and ends with a barrier.
 // The same elimination by 16 x 16 blocks: one warp turns the diagonal block into M_bb, then
 // L_ib = A_ib M_bb^T and X_bj = M_bb X_bj, then A_ik -= L_ib L_kb^T and X_ij -= L_ib X_bj, a warp and 16
 // float64 mma instructions per block.  Warp 0 updates the next diagonal block and goes on with it while
@@ -420,7 +421,7 @@ __device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp
 #pragma unroll
     for (int e = tid; e < kTile * kTile; e += kSmallThreads) {
         const int i = e >> 6, j = e & 63;     // the lower triangle is the valid one
-        if (j <= i) {
+        if (Ag && j <= i) {
             const double v = Ag[(size_t)i * dp + j];
             sm.ta[i * PS + j] = v;
             sm.ta[j * PS + i] = v;
@@ -479,20 +480,24 @@ __device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp
 // layer: right-looking elimination of [A | I] by tiles.  Stage j: rank 0 turns the diagonal tile into
 // M_jj; then F_ij = A_ij M_jj^T below it and M_jk = M_jj X_jk left of it; then A_ik -= F_ij F_kj^T and
 // X_ik -= F_ij M_jk (X_ik, kept in M's tile, is what M_ik is before its own row's stage).  The tiles of a
-// phase are independent and dealt out to the ranks; rank 0 updates the next diagonal tile first and goes
-// on to its leaf without waiting for the others, so the chain is leaf, one product, leaf, ...: two cluster
-// barriers a stage.  Every product is a 64 x 64 x 64 tile product of a whole CTA on the float64 tensor
+// phase are independent and dealt out to the ranks; rank 0 updates the next diagonal tile first, out of its own
+// F and without a detour through memory, and goes on to its leaf without waiting for the others, so the chain is
+// leaf, two products, leaf, ...: one cluster barrier a stage, and the arrival at another.  Every product is a 64 x 64 x 64 tile product of a whole CTA on the float64 tensor
 // core, its operands fetched from global memory (the L2) into shared memory; on one CTA alone the 32
 // products of four tiles took 150 us of 184.
 constexpr int kSmallCluster = 4;
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __global__ void __launch_bounds__(kSmallThreads, 1) k_factor_small(double* A, double* F, double* M, int dp, int lo,
                                                         int nt, int* layer_status) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
-    const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int l = blockIdx.x / CS;
+    const int rank = (int)cluster.block_rank();
+    const int l = blockIdx.x / kSmallCluster;
     const size_t lay = (size_t)l * dp * dp;
     auto tile = [&](double* base, int i, int j) {
         return base + lay + (size_t)(lo + i) * kTile * dp + (size_t)(lo + j) * kTile;
@@ -507,53 +512,101 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_factor_small(double* A, do
         cp_async_wait<0>();
         __syncthreads();
     };
-    // out = sign * product (+ out)
-    auto store = [&](const SmallAcc& acc, double* out, double sign, bool add) {
+    // what is at `out`: requested before the product that is to be taken from it
+    struct Old { double2 v[4]; };
+    auto load = [&](const double* out) {
+        Old old;
+        int e = 0;
+        small_epilogue(SmallAcc(), [&](int r, int c, double2) {
+            old.v[e++] = *reinterpret_cast<const double2*>(out + (size_t)r * dp + c);
+        });
+        return old;
+    };
+    auto store = [&](const SmallAcc& acc, double* out) {
         small_epilogue(acc, [&](int r, int c, double2 v) {
-            double2* o = reinterpret_cast<double2*>(out + (size_t)r * dp + c);
-            double2 x = make_double2(sign * v.x, sign * v.y);
-            if (add) { const double2 cur = *o; x.x += cur.x; x.y += cur.y; }
-            *o = x;
+            *reinterpret_cast<double2*>(out + (size_t)r * dp + c) = v;
         });
     };
+    auto subtract = [&](const SmallAcc& acc, double* out, const Old& old) {
+        int e = 0;
+        small_epilogue(acc, [&](int r, int c, double2 v) {
+            const double2 cur = old.v[e++];
+            *reinterpret_cast<double2*>(out + (size_t)r * dp + c) = make_double2(cur.x - v.x, cur.y - v.y);
+        });
+    };
+    static_assert(kSmallMax <= kSmallCluster, "a rank has one tile of a row and column");
     for (int j = 0; j < nt; ++j) {
-        if (rank == 0) leaf_factor(tile(A, j, j), tile(M, j, j), dp, sm);
+        SmallAcc acc;
+        if (rank == 0) {
+            leaf_factor(j == 0 ? tile(A, j, j) : nullptr, tile(M, j, j), dp, sm);
+            if (j > 0) cluster_wait();
+        }
         cluster.sync();
-        // ---- row and column j
-        for (int q = rank; q < nt - 1; q += CS) {
-            SmallAcc acc;
+        if (rank == 0 && j + 1 < nt) {
+            // F_{j+1,j} from the M_jj in shared memory, then the next diagonal tile from that F, into the
+            // place where the leaf wants it
+            const Old old = load(tile(A, j + 1, j + 1));
+            tile_async(sm.ta, tile(A, j + 1, j), dp);
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncthreads();
             acc.zero();
-            if (q < nt - 1 - j) {
-                const int i = j + 1 + q;
+            tile_mma<false, false>(acc, sm.ta, sm.tb);
+            store(acc, tile(F, j + 1, j));
+            cluster_arrive();                              // the others need F; rank 0 waits after its leaf
+            __syncthreads();
+            small_epilogue(acc, [&](int r, int c, double2 v) {
+                *reinterpret_cast<double2*>(sm.ta + r * PS + c) = v;
+            });
+            __syncthreads();
+            acc.zero();
+            tile_mma<false, false>(acc, sm.ta, sm.ta);
+            __syncthreads();
+            int e = 0;
+            small_epilogue(acc, [&](int r, int c, double2 v) {
+                const double2 cur = old.v[e++];
+                if (c <= r) sm.ta[r * PS + c] = sm.ta[c * PS + r] = cur.x - v.x;
+                if (c + 1 <= r) sm.ta[r * PS + c + 1] = sm.ta[(c + 1) * PS + r] = cur.y - v.y;
+            });
+            continue;
+        }
+        // ---- row and column j
+        if (rank < nt - 1) {
+            acc.zero();
+            if (rank < nt - 1 - j) {
+                const int i = j + 1 + rank;
                 fetch(tile(A, i, j), tile(M, j, j));
                 tile_mma<false, false>(acc, sm.ta, sm.tb);
-                store(acc, tile(F, i, j), 1.0, false);
+                store(acc, tile(F, i, j));
             } else {
-                const int k = q - (nt - 1 - j);
+                const int k = rank - (nt - 1 - j);
                 fetch(tile(M, j, j), tile(M, j, k));
                 tile_mma<false, true>(acc, sm.ta, sm.tb);
-                store(acc, tile(M, j, k), 1.0, false);
+                store(acc, tile(M, j, k));
             }
         }
         if (j + 1 == nt) break;
-        cluster.sync();
+        cluster_arrive();
+        cluster_wait();
         // ---- what is behind them: tile 0 is the next diagonal tile and rank 0's
         const int rest = nt - 1 - j, n_a = rest * (rest + 1) / 2, n_all = n_a + rest * (j + 1);
-        for (int q = rank; q < n_all; q += (rank == 0 || CS == 1) ? (CS == 1 ? 1 : n_all) : CS - 1) {
-            SmallAcc acc;
+        for (int q = rank; q < n_all; q += kSmallCluster - 1) {
             acc.zero();
             if (q < n_a) {
                 int ii = 0, kk = q;
                 while (kk > ii) { kk -= ii + 1; ++ii; }
                 const int i = j + 1 + ii, k = j + 1 + kk;
+                const Old old = load(tile(A, i, k));
                 fetch(tile(F, i, j), tile(F, k, j));
                 tile_mma<false, false>(acc, sm.ta, sm.tb);
-                store(acc, tile(A, i, k), -1.0, true);
+                subtract(acc, tile(A, i, k), old);
             } else {
                 const int i = j + 1 + (q - n_a) / (j + 1), k = (q - n_a) % (j + 1);
+                Old old = {};
+                if (k < j) old = load(tile(M, i, k));
                 fetch(tile(F, i, j), tile(M, j, k));
                 tile_mma<false, true>(acc, sm.ta, sm.tb);
-                store(acc, tile(M, i, k), -1.0, k < j);
+                subtract(acc, tile(M, i, k), old);
             }
         }
     }
