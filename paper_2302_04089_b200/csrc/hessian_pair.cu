@@ -470,15 +470,23 @@ int pair_count(int d) {
     return T * (T + 1) / 2;
 }
 
-// Pairs that share a tile where the tiles leave SMs idle: as many as fit at once (the occupancy calculator
-// gives room for MOST_CLUSTERS clusters of that many pairs; one tile more makes a second wave) with four K
-// blocks each.  8 x 512 features, 2048 bf16 tokens: 39.8 -> 29.7 us a call, 2 x 1100 of 500 fp32 37.7 -> 27.6,
-// 1 x 1322 of 4099 64.5 -> 58.3.
+// Pairs that share a tile: the number with the shortest chain of K blocks over all waves, where the tiles leave
+// SMs idle or a second wave nearly empty (most_clusters: the occupancy calculator's room for clusters of that
+// many pairs); the ends of a tile weigh 14 to 28 K blocks.  Four K blocks each at least.  8 x 512 features,
+// 2048 bf16 tokens: 39.8 -> 29.7 us a call, 2 x 1100 of 500 fp32 37.7 -> 27.6, 1 x 1322 of 4099 64.5 -> 58.3,
+// 1 x 3072 of 8192 (78 tiles) 347 -> 304.
+int most_clusters(int parts) {
+    constexpr int n[5] = {0, 74, 33, 22, 15};
+    return n[parts];
+}
 int parts_of(long long pairs, long long kb) {
-    constexpr int MOST_CLUSTERS[5] = {0, 74, 33, 22, 15};
     int parts = 1;
-    for (int p = 2; p <= 4; ++p)
-        if (pairs <= MOST_CLUSTERS[p] && kb / p >= 4) parts = p;
+    long long best = 0;
+    for (int p = 1; p <= 4; ++p) {
+        if (p > 1 && kb / p < 4) break;
+        const long long cost = (pairs + most_clusters(p) - 1) / most_clusters(p) * ((kb + p - 1) / p + 20);
+        if (p == 1 || cost < best) { best = cost; parts = p; }
+    }
     return parts;
 }
 
@@ -515,7 +523,7 @@ bool hessian_pair_fits(int layers, int d, long long N) {
     const long long kb = (N + BK - 1) / BK, T = (d + HALF - 1) / HALF, tiles = T * (T + 1) / 2 * layers;
     const long long pairs = (long long)pair_count(d) * layers, parts = parts_of(pairs, kb);
     const long long split = hessian_tile_split(tiles, kb);
-    const long long chain = (pairs * parts + 73) / 74 * ((kb + parts - 1) / parts);
+    const long long chain = (pairs + most_clusters(parts) - 1) / most_clusters(parts) * ((kb + parts - 1) / parts);
     return 4 * chain < 3 * ((tiles * split + 147) / 148 * ((kb + split - 1) / split));
 }
 

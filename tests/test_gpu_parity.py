@@ -901,7 +901,7 @@ def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
     assert torch.equal(H.double(), ref)
 
 
-@pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030)])
+@pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030), (1, 2817, 4100)])
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
 def test_hessian_tiles_shared_by_pairs_of_ctas(L, d, N, dtype):
     """Two, three and four pairs to a 256 x 256 tile, ragged K and widths, added to what is there; small
