@@ -24,8 +24,9 @@ struct HessianProduct {
 bool hessian_pair_fits(int layers, int d, long long N);
 // CTAs that share a 128 x 128 tile of the other one.
 int hessian_tile_split(long long tiles, long long num_kb);
+// Scratch that such a launch uses.
 size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split);
-ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st);
+ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, size_t scratch_bytes, cudaStream_t st);
 
 // A product kernel that gives up on a wait leaves NaN in H[l][0][0] of every layer of the call, so that
 // whichever stage reads H next reports ZIPLM_ERR_NONFINITE.  The thread that gives up records the call's

@@ -536,7 +536,9 @@ size_t hessian_pair_scratch_bytes(int layers, int d, long long N, bool split) {
     return (size_t)2 * pairs * parts * HALF * PT * sizeof(float);
 }
 
-ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, cudaStream_t st) {
+ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, size_t scratch_bytes, cudaStream_t st) {
+    if (hessian_pair_scratch_bytes(p.layers, p.d, (long long)p.num_kb * BK, p.split) > scratch_bytes)
+        return ZIPLM_ERR_WORKSPACE;
     float4* l2 = static_cast<float4*>(scratch);
     return p.split ? launch_pair<true>(p, l2, st) : launch_pair<false>(p, l2, st);
 }

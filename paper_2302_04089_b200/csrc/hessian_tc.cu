@@ -814,6 +814,20 @@ int product_layers(int L, int d, long long N, ziplm_dtype dt, bool token_major) 
     return L < 65535 ? L : 65535;
 }
 
+// Scratch of the pair kernel over all product launches of a call.  Kernel and pairs per tile are chosen for the
+// layers of a launch, so the last, smaller one may use more than the others (48 x 1600 features of 131072 fp32
+// tokens: 10 layers 73 MB, the last 8, with two pairs a tile, 117) or be the only one to use any.
+size_t product_scratch_bytes(int L, int d, long long N, ziplm_dtype dt, bool token_major) {
+    const int full = product_layers(L, d, N, dt, token_major), last = L % full;
+    size_t b = 0;
+    for (int layers : {full, last})
+        if (layers > 0 && hessian_pair_fits(layers, d, N)) {
+            const size_t need = hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32);
+            if (need > b) b = need;
+        }
+    return b;
+}
+
 }  // namespace
 
 // Where the 128 x 128 tiles leave half of the SMs idle, up to eight CTAs share a tile: the largest power of
@@ -835,9 +849,7 @@ size_t hessian_tc_workspace_bytes(int L, int d, long long N, ziplm_dtype dt, boo
         const int lc = transpose_chunk_layers(L, d, N);
         b += align_up((size_t)lc * d * (size_t)padded_tokens_bf16(N) * 2);
     }
-    const int layers = product_layers(L, d, N, dt, token_major);
-    if (hessian_pair_fits(layers, d, N)) b += align_up(hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32));
-    return b;
+    return b + align_up(product_scratch_bytes(L, d, N, dt, token_major));
 }
 
 namespace {
@@ -850,8 +862,9 @@ unsigned long long next_call() {
 }
 
 // One product launch on the kernel that suits its number of tiles.
-ziplm_status run_product(const HessianProduct& p, void* scratch, cudaStream_t st) {
-    if (hessian_pair_fits(p.layers, p.d, (long long)p.num_kb * 64)) return run_hessian_pair(p, scratch, st);
+ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_bytes, cudaStream_t st) {
+    if (hessian_pair_fits(p.layers, p.d, (long long)p.num_kb * 64))
+        return run_hessian_pair(p, scratch, scratch_bytes, st);
     const int T = (p.d + TM - 1) / TM;
     const long long tiles = (long long)T * (T + 1) / 2 * p.layers;
     const int split = hessian_tile_split(tiles, p.num_kb);
@@ -897,12 +910,9 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
     prod.L = L; prod.call = next_call();
     prod.num_kb = (int)((N + Cfg<false>::BK - 1) / Cfg<false>::BK);
     prod.fmt16 = fmt16; prod.spin = spin; prod.split = f32;
-    const int most_layers = product_layers(L, d, N, dt, token_major);
+    const size_t scratch_bytes = product_scratch_bytes(L, d, N, dt, token_major);
     void* scratch = nullptr;             // of the pair kernel, behind the operands
-    auto take_scratch = [&] {
-        if (hessian_pair_fits(most_layers, d, N))
-            scratch = c.take<char>(hessian_pair_scratch_bytes(most_layers, d, N, f32));
-    };
+    auto take_scratch = [&] { scratch = c.take<char>(scratch_bytes); };
     if (f32) {
         const long long np = padded_tokens_bf16(N);
         const int lc = split_chunk_layers(L, d, N);
@@ -982,7 +992,7 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
             if (!make_map(&prod.hi, hi, ZIPLM_F16, N, d, ln, np) || !make_map(&prod.lo, lo, ZIPLM_F16, N, d, ln, np))
                 return ZIPLM_ERR_CUDA;
             prod.layer0 = l0; prod.layers = ln;
-            const ziplm_status s = run_product(prod, scratch, st);
+            const ziplm_status s = run_product(prod, scratch, scratch_bytes, st);
             if (s != ZIPLM_OK) return s;
         }
     } else if (token_major) {
@@ -1004,7 +1014,7 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
             ZIPLM_CHECK_LAUNCH();
             if (!make_map(&prod.hi, xt, dt, N, d, ln, np)) return ZIPLM_ERR_CUDA;
             prod.lo = prod.hi; prod.layer0 = l0; prod.layers = ln;
-            const ziplm_status s = run_product(prod, scratch, st);
+            const ziplm_status s = run_product(prod, scratch, scratch_bytes, st);
             if (s != ZIPLM_OK) return s;
         }
     } else {
@@ -1016,7 +1026,7 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
             const __nv_bfloat16* Xc = static_cast<const __nv_bfloat16*>(X) + (size_t)l0 * d * ldx;
             if (!make_map(&prod.hi, Xc, dt, N, d, ln, ldx)) return ZIPLM_ERR_CUDA;
             prod.lo = prod.hi; prod.layer0 = l0; prod.layers = ln;
-            const ziplm_status s = run_product(prod, scratch, st);
+            const ziplm_status s = run_product(prod, scratch, scratch_bytes, st);
             if (s != ZIPLM_OK) return s;
         }
     }

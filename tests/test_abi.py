@@ -55,6 +55,32 @@ def test_status_strings_and_workspace_queries(lib):
     assert lib.ziplm_select_workspace_bytes(0, 24, 10000) == 0
 
 
+@pytest.mark.parametrize("L,d,N,dtype,tokens", [
+    (48, 1600, 131072, 0, False), (36, 768, 131072, 0, True), (36, 1600, 131072, 0, False), (48, 3072, 131072, 0, True),
+    (48, 1600, 262144, 1, True), (443, 300, 16384, 0, False), (880, 300, 16384, 2, True), (12, 3072, 2048, 0, True),
+])
+def test_hessian_workspace_covers_the_last_chunk_of_layers(lib, L, d, N, dtype, tokens):
+    """Operands of more than 8 GiB are prepared in chunks of layers.  The product of the last, smaller chunk may use
+    more scratch than a full one's: a call of all layers asks for at least what a call of its layers alone does."""
+    query = lib.ziplm_hessian_tokens_workspace_bytes if tokens else lib.ziplm_hessian_workspace_bytes
+    query.restype = ctypes.c_size_t
+    query.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_int]
+
+    def up(n):
+        return (n + 255) // 256 * 256
+
+    part = d * ((N + 7) // 8 * 8) * 2                            # a 16-bit operand of one layer
+    per_layer = (2 if dtype == 0 else 1) * part
+
+    def operands(layers):                                        # error word, magnitudes and the 16-bit operands
+        return 256 + (up(4 * layers * d) + 2 * up(layers * part) if dtype == 0 else up(layers * part))
+
+    chunk = min(L, (8 << 30) // per_layer)
+    scratch = query(L, d, N, dtype) - operands(chunk)
+    for layers in {chunk, L % chunk} - {0}:
+        assert scratch >= query(layers, d, N, dtype) - operands(layers)
+
+
 def test_options_round_trip_and_reject_bad_values(lib):
     lib.ziplm_set_option.restype = ctypes.c_int
     lib.ziplm_get_option.restype = ctypes.c_int

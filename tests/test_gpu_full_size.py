@@ -279,3 +279,31 @@ def test_paper_database_grid_from_streamed_token_major_batches():
         scale = np.sqrt(np.outer(np.diag(Ho), np.diag(Ho)))
         err = np.max(np.abs(H[l].cpu().double().numpy() - Ho) / scale)
         assert err < HESSIAN_TOL, err
+
+
+@pytest.mark.parametrize("L,d,N,dtype,tokens", [
+    (18, 1600, 131072, torch.float32, False),       # 10 layers, then 8 with two pairs of CTAs a tile
+    (225, 300, 32768, torch.float32, True),         # 218 layers on the 128 x 128 kernel, then 7 on the pair kernel
+    (443, 300, 32768, torch.float16, True),         # the same with 16-bit operands: 436, then 7
+])
+def test_hessian_of_more_operands_than_a_chunk_holds(L, d, N, dtype, tokens):
+    """Chunks of layers whose last, smaller one uses more scratch than the full ones: every layer against float64,
+    and nothing written behind the workspace that the library asked for."""
+    import paper_2302_04089_b200 as z
+    gen = torch.Generator("cuda").manual_seed(L)
+    X = torch.empty((L, N, d) if tokens else (L, d, N), dtype=dtype, device="cuda")
+    for l in range(L):
+        X[l] = torch.randn(X.shape[1:], generator=gen, device="cuda").to(dtype)
+    code = 0 if dtype == torch.float32 else 2
+    need = (z.hessian_tokens_workspace_bytes if tokens else z.hessian_workspace_bytes)(L, d, N, code)
+    ws = torch.empty(need + (1 << 20), dtype=torch.uint8, device="cuda")
+    ws[need:] = 0xA5
+    H = torch.full((L, d, d), float("nan"), device="cuda")
+    (z.hessian_accumulate_tokens if tokens else z.hessian_accumulate)(X, H, workspace=ws)
+    assert bool((ws[need:] == 0xA5).all())
+    for l in range(L):
+        x = X[l].double()
+        ref = 2.0 * (x.t() @ x if tokens else x @ x.t())
+        s = ref.diagonal().sqrt()
+        assert float(((H[l] - ref) / (s[:, None] * s[None, :])).abs().max()) < 2e-6
+        assert torch.equal(H[l], H[l].t())
