@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1)
 k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
             float* __restrict__ H, int d, int num_kb_all, int n_parts, float alpha, float beta, int layer0,
             int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
-            const unsigned* __restrict__ amax, float4* __restrict__ level2) {
+            const unsigned* __restrict__ amax, float4* __restrict__ level2, int quads) {
     using C = PairCfg<SPLIT>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[C::STAGES], bar_empty[C::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_final;
@@ -365,8 +365,8 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                         make_float4((alpha * acc[e]) * mul, (alpha * acc[e + 1]) * mul, (alpha * acc[e + 2]) * mul,
                                     (alpha * acc[e + 3]) * mul);
                 __syncwarp();
-                if (!diag && d % 4 == 0 && r0 + 32 <= d) {
-                    // whole rows below the diagonal: 16 lanes take one, 16 bytes each
+                if (!diag && quads && r0 + 32 <= d) {
+                    // whole rows below the diagonal that start on 16 bytes: 16 lanes take one, 16 bytes each
                     const int cc = 4 * (lane & 15);
                     float sc[4];
 #pragma unroll
@@ -495,6 +495,7 @@ ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t s
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_pair<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           kPairSmem<SPLIT>));
     const int parts = parts_of((long long)pair_count(p.d) * p.layers, p.num_kb);
+    const int quads = p.d % 4 == 0 && reinterpret_cast<uintptr_t>(p.H) % 16 == 0;     // rows of H start on 16 bytes
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * parts * pair_count(p.d), p.layers);
     cfg.blockDim = dim3(PAIR_THREADS);
@@ -509,7 +510,8 @@ ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t s
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_syrk_pair<SPLIT>, p.hi, p.lo, p.H, p.d, p.num_kb, parts, p.alpha,
-                                        p.beta, p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, level2));
+                                        p.beta, p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, level2,
+                                        quads));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }

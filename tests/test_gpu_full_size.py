@@ -289,7 +289,7 @@ def test_paper_database_grid_from_streamed_token_major_batches():
 def test_hessian_of_more_operands_than_a_chunk_holds(L, d, N, dtype, tokens):
     """Chunks of layers whose last, smaller one uses more scratch than the full ones: every layer against float64,
     and nothing written behind the workspace that the library asked for."""
-    import paper_2302_04089_b200 as z
+    z = zb()
     gen = torch.Generator("cuda").manual_seed(L)
     X = torch.empty((L, N, d) if tokens else (L, d, N), dtype=dtype, device="cuda")
     for l in range(L):

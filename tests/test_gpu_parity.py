@@ -914,3 +914,19 @@ def test_hessian_tiles_shared_by_pairs_of_ctas(L, d, N, dtype):
     assert torch.equal(H.double(), 2.0 * ref)
     H = z.hessian_accumulate_tokens(A, H, alpha=1.0, beta=1.0)
     assert torch.equal(H.double(), 3.0 * ref)
+
+
+@pytest.mark.parametrize("L,d,N,dtype", [(12, 516, 1100, torch.float32), (4, 1028, 2112, torch.bfloat16),
+                                         (1, 1324, 1100, torch.float16), (1, 256, 2048, torch.float32)])
+def test_hessian_into_a_matrix_that_starts_at_any_element(L, d, N, dtype):
+    """H needs the alignment of its elements only, on every product kernel: same bits as an aligned one."""
+    z = zb()
+    A = torch.randn(L, N, d, generator=torch.Generator().manual_seed(d)).to(dtype).cuda()
+    H = z.hessian_accumulate_tokens(A)
+    H2 = z.hessian_accumulate_tokens(A, H.clone(), beta=1.0)
+    for offset in (1, 2, 3):
+        room = torch.full((L * d * d + 8,), float("nan"), device="cuda")
+        Hu = room[offset:offset + L * d * d].view(L, d, d)
+        assert torch.equal(z.hessian_accumulate_tokens(A, Hu), H)
+        assert torch.equal(z.hessian_accumulate_tokens(A, Hu, beta=1.0), H2)
+        assert bool(room[:offset].isnan().all()) and bool(room[offset + L * d * d:].isnan().all())
