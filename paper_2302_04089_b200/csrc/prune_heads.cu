@@ -219,6 +219,7 @@ struct Heads {
     int* chosen;                            // [1]
     int* steps_of;                          // [n_levels], shared by the layers: removals of a level
     float* W_snap; int n_levels;
+    int pairs;                              // W and W_snap start on 8 bytes
     int* order; float* saliency; int* layer_status;
 };
 
@@ -526,7 +527,8 @@ __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, i
         h_combine<G8, false>(acc, [] {}, [&](int row, int col) {
             const size_t o = (size_t)min(row, rows - 1) * w.d + col;
             return Cur{*reinterpret_cast<const double2*>(Wl + (size_t)j * S::g + o),
-                       snap ? *reinterpret_cast<const float2*>(W0 + o) : make_float2(0.f, 0.f)};
+                       !snap ? make_float2(0.f, 0.f)
+                             : w.pairs ? *reinterpret_cast<const float2*>(W0 + o) : make_float2(W0[o], W0[o + 1])};
         }, [&](int row, int col, double2 d, Cur cur) {
             if (row >= rows) return;
             const size_t o = (size_t)row * w.d + col;
@@ -534,7 +536,8 @@ __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, i
             *reinterpret_cast<double2*>(Wl + (size_t)j * S::g + o) = cur.w;
             if (snap) {
                 const float f0 = (float)cur.w.x, f1 = (float)cur.w.y, e0 = cur.w0.x - f0, e1 = cur.w0.y - f1;
-                *reinterpret_cast<float2*>(snap + o) = make_float2(f0, f1);
+                if (w.pairs) *reinterpret_cast<float2*>(snap + o) = make_float2(f0, f1);
+                else { snap[o] = f0; snap[o + 1] = f1; }
                 part += (double)e0 * e0 + (double)e1 * e1;
             }
         });
@@ -696,6 +699,7 @@ ziplm_status run_prune_heads(const float* W, const float* H, int L, int r, int d
     HeadsWs w = carve_heads(ws, L, r, d, g, n_levels);
     if (ws_bytes < w.total) return ZIPLM_ERR_WORKSPACE;
     w.h.W = W; w.h.H = H; w.h.W_snap = W_snap; w.h.order = order; w.h.saliency = saliency;
+    w.h.pairs = (reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(W_snap)) % 8 == 0;    // g is even
     w.h.layer_status = layer_status;
     switch (g / 8) {
         case 4: return run_heads<4>(w, damp_frac, levels, loss, base_loss, st);

@@ -930,3 +930,25 @@ def test_hessian_into_a_matrix_that_starts_at_any_element(L, d, N, dtype):
         assert torch.equal(z.hessian_accumulate_tokens(A, Hu), H)
         assert torch.equal(z.hessian_accumulate_tokens(A, Hu, beta=1.0), H2)
         assert bool(room[:offset].isnan().all()) and bool(room[offset + L * d * d:].isnan().all())
+
+
+@pytest.mark.parametrize("L,r,d,g,levels", [(2, 70, 256, 64, [4, 3, 1]), (1, 33, 320, 80, [3, 0]), (2, 70, 256, 1, [200, 60]),
+                                            (1, 40, 640, 1, [500, 300, 10]), (1, 20, 60, 5, [7, 2])])
+def test_weights_and_snapshots_that_start_at_any_element(L, r, d, g, levels):
+    """W and W_snap need the alignment of their elements only, on every path: same bits as aligned ones."""
+    z = zb()
+    gen = torch.Generator().manual_seed(d + g)
+    W = torch.randn(L, r, d, generator=gen).cuda()
+    H = z.hessian_accumulate_tokens(torch.randn(L, 4 * d, d, generator=gen).cuda())
+    ref = z.prune_layers(W, H, g, 0.01, levels)
+    n = W.numel()
+    for at_w, at_snap in ((1, 0), (0, 1), (3, 3)):
+        Wu = torch.zeros(n + 4, device="cuda")[at_w:at_w + n].view(L, r, d)
+        Wu.copy_(W)
+        room = torch.full((n * len(levels) + 8,), float("nan"), device="cuda")
+        out = {k: torch.empty_like(v) for k, v in ref.items()}
+        out["W_snap"] = room[at_snap:at_snap + n * len(levels)].view(L, len(levels), r, d)
+        z.prune_layers(Wu, H, g, 0.01, levels, out=out)
+        for k in ("W_snap", "loss", "order", "saliency", "layer_status"):
+            assert torch.equal(out[k], ref[k]), k
+        assert bool(room[:at_snap].isnan().all()) and bool(room[at_snap + n * len(levels):].isnan().all())
