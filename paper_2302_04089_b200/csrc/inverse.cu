@@ -672,8 +672,10 @@ struct InvCtx {
 
 // Products of blocks of at least eight tiles a side, and M^T M from sixteen tiles on, run on the int8 tensor
 // cores: below, the passes that write the digits and the few 256 x 128 tiles cost what the products save.
+// M^T M sums over the whole width, which the exactness of the int32 sums limits; wider matrices stay on the
+// float64 instruction.
 constexpr int kI8Tiles = 8;
-bool uses_i8(int T) { return T >= 2 * kI8Tiles; }
+bool uses_i8(int T) { return T >= 2 * kI8Tiles && T * kTile <= kI8MostK; }
 
 int task_ctas(const GemmTask& t) {
     const int mm = (t.mt + 1) / 2;                           // macro tiles: mm x t.nt

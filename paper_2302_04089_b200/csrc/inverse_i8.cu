@@ -4,9 +4,9 @@
 // Oishi and Rump ("Error-free transformations of matrix multiplication", 2012) an operand row is written as
 // a fixed-point number, x = 2^(E - 62) q with |q| < 2^62 and E the exponent of the row's largest entry, and
 // q as eight signed digits of radix 256.  Products of digit matrices are exact in int32 (8 * 2^14 * K stays
-// below 2^31 up to K = 16384); of the 64 pairs the 36 whose weight is at least 256^7 are formed, those of
-// one weight into the same accumulator, and the accumulators are joined exactly in int64 and then rounded
-// once.  Digits and dropped pairs leave an error below 2^-60 of the largest entries per term, less than the
+// below 2^31 up to kI8MostK, the leading digits being 64 at most); of the 64 pairs the 36 whose weight is at least
+// 256^7 are formed, those of one weight into the same accumulator, and the accumulators are joined exactly in
+// int64 and then rounded once.  Digits and dropped pairs leave an error below 2^-60 of the largest entries per term, less than the
 // 2^-53 of every partial sum that a float64 chain makes; the matrices are equilibrated by powers of two
 // beforehand (k_fill_damped), so that a row's entries and the columns they meet are of one scale.
 //
@@ -466,7 +466,7 @@ size_t carve_i8_operand(I8Operand* o, void* ws, int L, int rows, int K) {
 }
 
 bool i8_symmetric_pays(int L, int rows, int K, double float64_clocks) {
-    if (K > 16384) return false;
+    if (K > kI8MostK) return false;
     const int nI = (rows + PM - 1) / PM, nJ = (rows + PN - 1) / PN;
     double tiles = 0;
     for (int I = 0; I < nI; ++I) tiles += 2 * I + 2 < nJ ? 2 * I + 2 : nJ;
@@ -476,6 +476,7 @@ bool i8_symmetric_pays(int L, int rows, int K, double float64_clocks) {
 
 ziplm_status i8_product(const I8Operand& x, const I8Operand& y, I8Product p, int L, cudaStream_t st) {
     CUtensorMap mx, my;
+    if (x.K > kI8MostK) return ZIPLM_ERR_UNSUPPORTED;      // (no caller asks for it)
     p.rows = x.rows; p.cols = y.rows; p.K = x.K;
     p.x_scale = x.scale; p.y_scale = y.scale;
     if (!make_digit_map(&mx, x.dig, L, x.rows, x.K, 128) || !make_digit_map(&my, y.dig, L, y.rows, y.K, 64))

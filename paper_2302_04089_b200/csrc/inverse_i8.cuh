@@ -5,6 +5,8 @@
 
 namespace ziplm {
 
+constexpr int kI8MostK = 16384;      // the int32 sums of digit products are exact up to this K
+
 // An operand in digits: [L][8][rows][K] int8, a power-of-two scale per row (and room for exponents).
 struct I8Operand {
     signed char* dig;

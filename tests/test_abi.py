@@ -81,6 +81,17 @@ def test_hessian_workspace_covers_the_last_chunk_of_layers(lib, L, d, N, dtype, 
         assert scratch >= query(layers, d, N, dtype) - operands(layers)
 
 
+@pytest.mark.parametrize("d,digits", [(960, False), (961, True), (16384, True), (16385, False), (40000, False)])
+def test_int8_products_of_the_inverse_only_where_their_sums_are_exact(lib, d, digits):
+    """Sums of eight digit products over K stay below 2^31 up to K = 16384, and M^T M sums over the padded width: the
+    workspace holds digits of an operand from 1024 (padded) up to there, and only the three float64 matrices beyond."""
+    lib.ziplm_inverse_workspace_bytes.restype = ctypes.c_size_t
+    dp = (d + 63) // 64 * 64
+    rest = lib.ziplm_inverse_workspace_bytes(1, d) - 3 * 8 * dp * dp
+    assert (rest >= 2 * 8 * (dp // 2) ** 2) == digits
+    assert digits or rest <= 256
+
+
 def test_options_round_trip_and_reject_bad_values(lib):
     lib.ziplm_set_option.restype = ctypes.c_int
     lib.ziplm_get_option.restype = ctypes.c_int
