@@ -32,7 +32,7 @@ ziplm_status run_hessian_pair(const HessianProduct& p, void* scratch, size_t scr
 // whichever stage reads H next reports ZIPLM_ERR_NONFINITE.  The thread that gives up records the call's
 // number first and poisons the layers then; the CTA that writes an entry (0, 0) looks for the number
 // afterwards (hessian_check): whichever of the two comes second sees the other.  The number is new for
-// every call, so the word needs no clearing.
+// every call, so the word needs no clearing, except in a captured call, whose replays share it.
 __device__ __forceinline__ void hessian_give_up(float* H, int L, int d, unsigned long long* err_word,
                                                 unsigned long long call) {
     atomicExch(err_word, call);

@@ -903,6 +903,11 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
     const uint32_t fmt16 = (dt == ZIPLM_F16) ? 0u : 1u;
     Carver c(ws);
     unsigned long long* err_word = c.take<unsigned long long>(1);
+    // A captured call is replayed under one number: there the word is cleared first, so that a replay whose wait
+    // ran out does not mark the ones behind it.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    ZIPLM_CHECK_CUDA(cudaStreamIsCapturing(st, &capture));
+    if (capture != cudaStreamCaptureStatusNone) ZIPLM_CHECK_CUDA(cudaMemsetAsync(err_word, 0, sizeof(*err_word), st));
     const int spin_opt = option_value(ZIPLM_OPT_SPIN_LIMIT);
     const uint32_t spin = spin_opt > 0 ? (uint32_t)spin_opt : kSpinLimit;
     HessianProduct prod = {};

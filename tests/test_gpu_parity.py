@@ -952,3 +952,36 @@ def test_weights_and_snapshots_that_start_at_any_element(L, r, d, g, levels):
         for k in ("W_snap", "loss", "order", "saliency", "layer_status"):
             assert torch.equal(out[k], ref[k]), k
         assert bool(room[:at_snap].isnan().all()) and bool(room[at_snap + n * len(levels):].isnan().all())
+
+
+@pytest.mark.parametrize("L,d,N,dtype,tokens", [(1, 256, 2048, torch.float32, True), (2, 64, 16384, torch.bfloat16, False),
+                                                (12, 513, 1024, torch.bfloat16, False), (12, 513, 1024, torch.float32, False)])
+def test_replays_of_a_captured_hessian_call_after_one_whose_wait_ran_out(L, d, N, dtype, tokens):
+    """A wait that runs out leaves the call's number in the workspace, and all replays of a captured call have one
+    number: a replay must not find what an earlier one left.  The number is known from the call before (one odd
+    constant further, then made odd), so the test can put it there."""
+    z = zb()
+    X = torch.randn(L, N, d, generator=torch.Generator().manual_seed(d)).to(dtype).cuda()
+    call, query = (z.hessian_accumulate_tokens, z.hessian_tokens_workspace_bytes) if tokens else \
+        (z.hessian_accumulate, z.hessian_workspace_bytes)
+    X = X if tokens else X.transpose(1, 2).contiguous()
+    ws = torch.zeros(query(L, d, N, {torch.float32: 0, torch.bfloat16: 1}[dtype]), dtype=torch.uint8, device="cuda")
+    H = torch.empty(L, d, d, device="cuda")
+    ref = call(X, workspace=ws).clone()
+    z.set_option(z.Option.SPIN_LIMIT, 1)
+    try:
+        call(X, H, workspace=ws)
+    finally:
+        z.set_option(z.Option.SPIN_LIMIT, 0)
+    assert torch.isnan(H[:, 0, 0]).all()
+    left = int(ws[:8].view(torch.int64).item())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(X, H, workspace=ws)
+    for before in (left, left - 1):
+        number = ((before + 0x9e3779b97f4a7c15) | 1) & (2 ** 64 - 1)
+        ws[:8].view(torch.int64).fill_(number - 2 ** 64 if number >= 2 ** 63 else number)
+        H.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(H, ref)
