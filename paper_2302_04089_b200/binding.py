@@ -121,8 +121,15 @@ def status_string(status: int) -> str:
         return f"status {int(status)}"
 
 
+# The direct calls behind torch.cuda's, a few microseconds cheaper; private, so not taken for granted.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
+
+
 def _stream_ptr(t: torch.Tensor) -> int:
-    return torch._C._cuda_getCurrentRawStream(t.device.index)
+    if _raw_stream is None:
+        return torch.cuda.current_stream(t.device).cuda_stream
+    return _raw_stream(t.device.index)
 
 
 class _Nothing:
@@ -138,7 +145,7 @@ _NOTHING = _Nothing()
 
 def _on(device):
     """The device made current for a call; nothing to do, and nothing paid for, where it is already."""
-    return _NOTHING if torch._C._cuda_getDevice() == device.index else torch.cuda.device(device)
+    return _NOTHING if _raw_device() == device.index else torch.cuda.device(device)
 
 
 def _ptr(t: Optional[torch.Tensor]):

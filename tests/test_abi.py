@@ -128,6 +128,25 @@ def test_binding_mirrors_the_abi_names():
         assert hasattr(z, name[len("ziplm_"):]), name
 
 
+def test_binding_does_without_private_torch_calls(monkeypatch):
+    """The current stream and device come from torch's public interface where the private calls are missing."""
+    import importlib.util
+    import types
+    import torch
+    import paper_2302_04089_b200.binding as b
+    with monkeypatch.context() as m:
+        for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+            m.delattr(torch._C, name, raising=False)
+        m.setattr(torch.cuda, "current_stream", lambda device: types.SimpleNamespace(cuda_stream=77))
+        m.setattr(torch.cuda, "current_device", lambda: 3)
+        spec = importlib.util.spec_from_file_location("binding_without_private_calls", b.__file__)
+        bare = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(bare)
+        assert bare._stream_ptr(types.SimpleNamespace(device=torch.device("cuda", 3))) == 77
+        assert bare._on(torch.device("cuda", 3)) is bare._NOTHING
+        assert bare._on(torch.device("cuda", 1)) is not bare._NOTHING
+
+
 def test_compute_entry_points_fail_loudly_without_a_device(lib):
     import torch
     if torch.cuda.is_available():
