@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
     __shared__ uint64_t bar_step[2];
     __shared__ int h_piv[kMaxN], h_org[kMaxN];
     __shared__ double h_rs[kMaxN], h_rho[kMaxN];
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, s_stopped;                      // step of a give-up
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = CS > 1 ? (int)cluster.block_rank() : 0;
     const int l = blockIdx.x / CS;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
                     }
                 }
             }
-            if (__syncthreads_or(failed)) { failed = true; break; }
+            if (__syncthreads_or(failed)) { failed = true; s_stopped = m; break; }
             double2 ui[4];
 #pragma unroll
             for (int x = 0; x < 4; ++x) ui[x] = prev[row0 + 4 * rg + x];
@@ -450,6 +450,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) k_endgame_steps(const __grid_
         tc::mbar_wait_quiet(tc::smem_u32(&bar_step[w.n_steps & 1]), (uint32_t)(w.n_steps >> 1) & 1u);
     __syncthreads();
     if (CS > 1) cluster.sync();
+    // After a give-up: what the others had sent by then, for this step and the next, lands or runs out once more.
+    if (CS > 1 && failed && tid == 0)
+        for (int m = s_stopped; m < s_stopped + 2; ++m)
+            if (!tc::mbar_wait_quiet(tc::smem_u32(&bar_step[m & 1]), (uint32_t)(m >> 1) & 1u)) break;
 
     for (int e = tid; e < w.n_steps * S; e += STEP_THREADS) {
         const int m = e / S, k = row0 + e % S;

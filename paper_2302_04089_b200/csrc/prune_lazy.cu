@@ -107,6 +107,17 @@ __device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
                  : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
+// Every CTA of a cluster sends its offers of all steps, also past a give-up.  Once all have been sent (behind the
+// last cluster barrier) those from step `first` on, which the CTA has not waited for, land before it leaves, or run
+// out once more: barriers of even and odd steps, armed up to step first + 1.
+__device__ __forceinline__ void land_offers(uint64_t (&bar_step)[2], int first, int nsteps, uint32_t step_bytes) {
+    for (int m = first; m < nsteps; ++m) {
+        const uint32_t bar = tc::smem_u32(&bar_step[m & 1]);
+        if (!tc::mbar_wait_quiet(bar, (uint32_t)(m >> 1) & 1u)) return;
+        if (m + 2 < nsteps) tc::mbar_expect_tx(bar, step_bytes);
+    }
+}
+
 // nsteps greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
 // chosen so that a CTA's slice of positions fits its shared memory).  CTA `rank` owns the
 // positions [rank * S, rank * S + S); each of its 256 threads owns four consecutive ones and
@@ -173,13 +184,15 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     double da[4], dq[4];
     int org[4];
     bool alive[4];
+    // what a step brings to a CTA
+    [[maybe_unused]] const uint32_t step_bytes = (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2)));
     if (MULTI) {
         if (tid == 0) {
             abort_flag = 0;
             tc::mbar_init(tc::smem_u32(&bar_step[0]), 1);
             tc::mbar_init(tc::smem_u32(&bar_step[1]), 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
+            tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), step_bytes);
         }
         cluster.sync();
     }
@@ -202,7 +215,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         org[e] = alive[e] ? o : 0x7fffffff;
     }
     int first_bad = ZIPLM_OK;                  // meaningful in lane 0 of the last warp
-    bool failed = false;
+    int gave_up = nsteps;                      // the first step whose offers did not come in time
     // row indices of W that this CTA solves for
     const int w_per = ((rp + CS - 1) / CS + 7) / 8 * 8, w_first = rank * w_per, w_end = min(rp, w_first + w_per);
 
@@ -268,11 +281,11 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
                 tc::send1(to_pend + (uint32_t)(par * CLUSTER_MAX * BMAX * sizeof(float2)),
                           ((long long)__float_as_uint(uz.y) << 32) | __float_as_uint(uz.x), bar);
             }
-            if (tid == 0 && m + 1 < nsteps)
-                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]),
-                                   (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2))));
+            // (past a give-up the barrier may still be in an older phase)
+            if (tid == 0 && m + 1 < nsteps && gave_up == nsteps)
+                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]), step_bytes);
             if (!tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
-                failed = true;                     // (the waits that follow give up at once)
+                gave_up = min(gave_up, m);         // (the waits that follow give up at once)
                 abort_flag = 1;
             }
             const int which = best_bid(s_cta[par], CS, lane);
@@ -350,7 +363,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         }
         // no barrier here: the next step's barrier orders these writes before any read
     }
-    if (failed) set_layer_status(layer_status, l, ZIPLM_ERR_TIMEOUT);
+    if (gave_up < nsteps) set_layer_status(layer_status, l, ZIPLM_ERR_TIMEOUT);
     __syncthreads();
 
     // ---- what the update kernels read: u, z as they are for a compaction block, packed for a dense one
@@ -505,6 +518,7 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         }
         solve_c();
         if (MULTI) cluster.sync();      // no CTA leaves while others may send to it
+        if (MULTI && tid == 0) land_offers(bar_step, gave_up, nsteps, step_bytes);
         return;
     }
     const int f0 = alive[0] ? 1 : 0, f1 = alive[1] ? 1 : 0, f2 = alive[2] ? 1 : 0, f3 = alive[3] ? 1 : 0;
@@ -538,7 +552,16 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
             ++np;
         }
     }
+    // After a give-up the CTAs may have removed more than one position a step between them: what is left without
+    // an owner becomes column 0 at position 0, so that the kernels behind this one stay in bounds.  (Otherwise
+    // this lies past the live positions.)
+    if (MULTI && rank == CS - 1)
+        for (int k = base + s_count + tid; k < n0; k += STEP_THREADS) {
+            const size_t o = (size_t)l * d + k;
+            src[o] = 0; idx_out[o] = 0; dA_out[o] = 1.0; dQ_out[o] = 0.0;
+        }
     if (MULTI) cluster.sync();      // no CTA may retire while another can still read its shared memory
+    if (MULTI && tid == 0) land_offers(bar_step, gave_up, nsteps, step_bytes);
     solve_c();
 }
 
