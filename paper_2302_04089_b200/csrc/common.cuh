@@ -68,6 +68,13 @@ __device__ inline void set_layer_status(int* layer_status, int l, int code) {
     atomicCAS(layer_status + l, (int)ZIPLM_OK, code);
 }
 
+// D(8x8) += A(8x4) B(4x8) in float64 on the tensor core.  Lane T holds A[T/4][T%4], B[T%4][T/4]
+// and D[T/4][2(T%4)], D[T/4][2(T%4)+1].
+__device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
 // ---- stages implemented in the other translation units (host-side planners) -----------------
 
 // Workspace of the float64 damped inverse for L layers of width d.

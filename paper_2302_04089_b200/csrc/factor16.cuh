@@ -8,13 +8,6 @@
 
 namespace ziplm {
 
-// D(8x8) += A(8x4) B(4x8) in float64 on the tensor core.  Lane T holds A[T/4][T%4], B[T%4][T/4]
-// and D[T/4][2(T%4)], D[T/4][2(T%4)+1].
-__device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
 // One warp: acc(16 x 16) += A(16 x 16) B(16 x 16), operands in shared memory;
 // BT: B(k,n) = b[n][k], else b[k][n].
 template <bool BT>

@@ -48,42 +48,12 @@ constexpr int kStageBytes = 2 * PairCfg<SPLIT>::PARTS * OP_BYTES;      // A half
 template <bool SPLIT>
 constexpr int kPairSmem = PairCfg<SPLIT>::STAGES * kStageBytes<SPLIT> + 1024;
 
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Arrive at a barrier of the pair's other CTA (or of this one), by its shared::cluster address.  The
-// barriers here order accesses of the asynchronous proxy and of tensor memory only, so arrivals and waits
-// keep the default scope: cluster scope would fence generic memory at every one of them.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
-}
-// TMA load into this CTA's shared memory, counted on a barrier of either CTA of the pair.
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
-                                                 int y, int z) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(x), "r"(y), "r"(z)
-        : "memory");
-}
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Arrive at the barrier at this offset in the pair's two CTAs (a mask of cluster ranks) once the MMAs issued
-// so far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t both) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        ::"r"(bar), "h"(both) : "memory");
 }
 
 // The end of a tile that n_parts pairs have shared.  Every thread of the cluster's CTAs comes here once the
@@ -441,9 +411,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
 
     if (failed) {
         hessian_give_up(H, L, d, err_word, call);
-        for (uint32_t r = 0; r < 2; ++r)
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), lead + r)), "r"(1)
-                         : "memory");
+        for (uint32_t r = 0; r < 2; ++r) cluster_store(cluster_addr(smem_u32(&abort_flag), lead + r), 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

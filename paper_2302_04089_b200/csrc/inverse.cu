@@ -16,6 +16,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "damping.cuh"
 #include "factor16.cuh"
 #include "inverse_i8.cuh"
 
@@ -167,7 +168,6 @@ __device__ __forceinline__ void lower_macro_index(int idx, int T, int& I, int& J
     J = idx;
 }
 
-
 // eq (may be null): powers of two that bring the diagonal of the damped matrix to [1, 4).
 // lambda[l] = damp_frac * mean(diag H[l]); flags non-finite diagonals and non-positive means.
 __global__ void __launch_bounds__(256) k_mean_diag(const float* __restrict__ H, int d,
@@ -175,40 +175,9 @@ __global__ void __launch_bounds__(256) k_mean_diag(const float* __restrict__ H, 
                                                    double* __restrict__ eq, int* layer_status) {
     const int l = blockIdx.x;
     const float* Hl = H + (size_t)l * d * d;
-    double s = 0.0;
-    bool bad = false;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const float v = Hl[(size_t)i * d + i];
-        if (!isfinite(v)) bad = true;
-        s += (double)v;
-    }
-    __shared__ double red[256];
-    __shared__ int sbad;
-    if (threadIdx.x == 0) sbad = 0;
-    __syncthreads();
-    if (bad) sbad = 1;
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double mean = red[0] / (double)d;
-        double lm = (double)damp_frac * mean;
-        if (sbad || !isfinite(mean)) {
-            set_layer_status(layer_status, l, ZIPLM_ERR_NONFINITE);
-            lm = 1.0;
-        } else if (damp_frac > 0.f && !(mean > 0.0)) {
-            set_layer_status(layer_status, l, ZIPLM_ERR_NOT_PD);
-            lm = 1.0;
-        }
-        lam[l] = lm;
-        red[0] = lm;
-    }
+    const double lm = mean_diag_lambda(Hl, d, damp_frac, layer_status, l, true);
+    if (threadIdx.x == 0) lam[l] = lm;
     if (!eq) return;
-    __syncthreads();
-    const double lm = red[0];
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
         const int hi = __double2hiint((double)Hl[(size_t)i * d + i] + lm), e = hi >> 20;
         const int half = (e - 1023) >> 1;

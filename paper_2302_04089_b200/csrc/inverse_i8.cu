@@ -6,9 +6,9 @@
 // q as eight signed digits of radix 256.  Products of digit matrices are exact in int32 (8 * 2^14 * K stays
 // below 2^31 up to kI8MostK, the leading digits being 64 at most); of the 64 pairs the 36 whose weight is at least
 // 256^7 are formed, those of one weight into the same accumulator, and the accumulators are joined exactly in
-// int64 and then rounded once.  Digits and dropped pairs leave an error below 2^-60 of the largest entries per term, less than the
-// 2^-53 of every partial sum that a float64 chain makes; the matrices are equilibrated by powers of two
-// beforehand (k_fill_damped), so that a row's entries and the columns they meet are of one scale.
+// int64 and then rounded once.  Digits and dropped pairs leave an error below 2^-60 of the largest entries per
+// term, less than the 2^-53 of every partial sum that a float64 chain makes; the matrices are equilibrated by
+// powers of two beforehand (k_fill_damped), so that a row's entries and the columns they meet are of one scale.
 //
 // A pair of CTAs computes a tile of 256 x 128: the eight accumulators take two passes of four (512 columns
 // of tensor memory), first the digits 4 .. 7 (10 products), then all (26).  A K block is 64 digits (64-byte
@@ -159,34 +159,11 @@ __global__ void __launch_bounds__(256) k_digits_columns(const T* __restrict__ sr
 }
 
 // ---------------------------------------------------------------------------------------- products
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
-                                             int w) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
-}
 __device__ __forceinline__ void umma_i8_pair(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void commit_pair(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
 // K-major tile with 64-byte rows and the 64-byte swizzle: eight-row groups of 512 bytes.
 __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
@@ -270,8 +247,8 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 const int first = pass ? 0 : 4;
                 if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * (uint32_t)((SL - first) * (A_BYTES + B_BYTES)));
                 for (int q = first; q < SL; ++q) {
-                    load_4d_pair(base + q * A_BYTES, &map_x, full, kx, ya, q, l);
-                    load_4d_pair(base + SL * A_BYTES + q * B_BYTES, &map_y, full, kx, yb, q, l);
+                    tma_load_4d_pair(base + q * A_BYTES, &map_x, full, kx, ya, q, l);
+                    tma_load_4d_pair(base + SL * A_BYTES + q * B_BYTES, &map_y, full, kx, yb, q, l);
                 }
                 issued = it + 1;
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
@@ -282,6 +259,7 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             // ---------------- MMA issuer: int8 x int8 -> int32, M = 256, N = 128, K = 32
             constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(PN >> 3) << 17) |
                                        ((uint32_t)(PM >> 4) << 24);
+            constexpr uint16_t both = 3;
             const uint64_t a0 = desc64(ring), b0 = desc64(ring + SL * A_BYTES);
             int s = 0;
             uint32_t ph = 0u;
@@ -304,12 +282,12 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                             umma_i8_pair(acc, da + 2u, db + 2u, idesc, 1u);
                         }
                     }
-                    commit_pair(smem_u32(&bar_empty[s]));
+                    umma_commit_pair(smem_u32(&bar_empty[s]), both);
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (!failed) commit_pair(smem_u32(&bar_acc_full));
+                if (!failed) umma_commit_pair(smem_u32(&bar_acc_full), both);
             }
-            commit_pair(smem_u32(&bar_final));
+            umma_commit_pair(smem_u32(&bar_final), both);
             mbar_wait_quiet(smem_u32(&bar_final), 0u);
         }
     } else {
@@ -338,7 +316,7 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0 && pass == 0) arrive_cluster(acc_empty);
+            if (lane == 0 && pass == 0) mbar_arrive_cluster(acc_empty);
         }
         if (!failed) {
             // The ring is free (every MMA has completed): 32 x 32 results pass through it, rows leave whole.
@@ -395,8 +373,7 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
 
     if (failed) {
         set_layer_status(p.layer_status, l, ZIPLM_ERR_TIMEOUT);
-        for (uint32_t r = 0; r < 2; ++r)
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(&abort_flag), r)), "r"(1) : "memory");
+        for (uint32_t r = 0; r < 2; ++r) cluster_store(cluster_addr(smem_u32(&abort_flag), r), 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -22,6 +22,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "damping.cuh"
 #include "pick.cuh"
 #include "tc_common.cuh"
 
@@ -62,44 +63,6 @@ struct Endgame {
 };
 
 // ------------------------------------------------------------------------------------------ set-up
-// lambda of a layer as the damped inverse defines it; every thread returns it.
-__device__ double mean_diag_lambda(const float* Hl, int d, float damp_frac, int* layer_status, int l, bool report) {
-    __shared__ double red[256];
-    __shared__ int sbad;
-    const int tid = threadIdx.x;
-    double s = 0.0;
-    bool bad = false;
-    for (int i = tid; i < d; i += 256) {
-        const float v = Hl[(size_t)i * d + i];
-        if (!isfinite(v)) bad = true;
-        s += (double)v;
-    }
-    if (tid == 0) sbad = 0;
-    __syncthreads();
-    if (bad) sbad = 1;
-    red[tid] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (tid < o) red[tid] += red[tid + o];
-        __syncthreads();
-    }
-    const double mean = red[0] / (double)d;
-    double lm = (double)damp_frac * mean;
-    int code = ZIPLM_OK;
-    if (sbad || !isfinite(mean)) code = ZIPLM_ERR_NONFINITE;
-    else if (damp_frac > 0.f && !(mean > 0.0)) code = ZIPLM_ERR_NOT_PD;
-    if (code != ZIPLM_OK) {
-        lm = 1.0;
-        if (report && tid == 0) set_layer_status(layer_status, l, code);
-    }
-    return lm;
-}
-
-__device__ __forceinline__ void dmma(double (&d)[2], double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
 // CTAs 0 .. n_gram - 1: a 32 x 32 tile (on or below the diagonal) of Q = W^T W over the live columns, and
 // its share of <Q, H> when the run starts here; the rest: 16 rows of H_lambda, identity on the padding.
 __global__ void __launch_bounds__(256) k_endgame_setup(const __grid_constant__ Endgame w, int n_gram, int dp) {
@@ -144,7 +107,7 @@ __global__ void __launch_bounds__(256) k_endgame_setup(const __grid_constant__ E
                 const double a = sa[(8 * (warp >> 1) + (lane >> 2)) * P + 4 * kk + (lane & 3)];
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
-                    dmma(acc[j], a, sb[(16 * (warp & 1) + 8 * j + (lane >> 2)) * P + 4 * kk + (lane & 3)]);
+                    dmma884(acc[j], a, sb[(16 * (warp & 1) + 8 * j + (lane >> 2)) * P + 4 * kk + (lane & 3)]);
             }
         }
         double* Ql = w.Q + (size_t)l * n * n;

@@ -101,12 +101,6 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
     }
 }
 
-// D(8x8) += A(8x4) B(4x8) in float64 on the tensor core.
-__device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                 : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
 // Every CTA of a cluster sends its offers of all steps, also past a give-up.  Once all have been sent (behind the
 // last cluster barrier) those from step `first` on, which the CTA has not waited for, land before it leaves, or run
 // out once more: barriers of even and odd steps, armed up to step first + 1.

@@ -155,13 +155,55 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-// Asynchronous stores to another CTA of the cluster that complete on a barrier of that CTA (addresses of
-// the shared::cluster window).
-__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+// Addresses of the shared::cluster window: the same place in another CTA of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
     uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+    return cluster_addr(smem_u32(p), (uint32_t)rank);
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t to, int x) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(x) : "memory");
+}
+
+// CTA pairs (cta_group::2).  Arrive at a barrier of the pair's other CTA (or of this one), by its shared::cluster
+// address.  The barriers here order accesses of the asynchronous proxy and of tensor memory only, so arrivals and
+// waits keep the default scope: cluster scope would fence generic memory at every one of them.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// TMA load into this CTA's shared memory, counted on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
+                                                 int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int x,
+                                                 int y, int z, int w) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(x), "r"(y), "r"(z), "r"(w)
+        : "memory");
+}
+// Arrive at the barrier at this offset in the pair's two CTAs (a mask of cluster ranks) once the MMAs issued
+// so far have completed.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t both) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+        ::"r"(bar), "h"(both) : "memory");
+}
+
+// Asynchronous stores to another CTA of the cluster that complete on a barrier of that CTA (addresses of
+// the shared::cluster window).
 __device__ __forceinline__ void send1(uint32_t to, long long x, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.s64 [%0], %1, [%2];"
                  ::"r"(to), "l"(x), "r"(bar) : "memory");
