@@ -76,7 +76,7 @@ struct TileEnd {
     float* Hl; const unsigned* am;
     const unsigned long long* err_word; unsigned long long call;
 
-    template <int S, int R, bool TF32>
+    template <int S, int R, bool SPLIT>
     __device__ __forceinline__ void finish() const {
         constexpr int NH = TM / 32, N_ROWS = TM / S, WARPS = THREADS / 32;
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS;
@@ -85,7 +85,7 @@ struct TileEnd {
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
             const int col = j0 + 32 * h + lane;
-            scale[h] = TF32 && col < d ? row_scale(am[col], true) : 1.f;
+            scale[h] = SPLIT && col < d ? row_scale(am[col], true) : 1.f;
         }
 #pragma unroll 1
         for (int at = warp * R; at < N_ROWS && i0 + first + at < d; at += WARPS * R) {
@@ -102,7 +102,7 @@ struct TileEnd {
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const int row = i0 + first + at + k;
-                mul[k] = TF32 && row < d ? row_scale(am[row], true) : 1.f;
+                mul[k] = SPLIT && row < d ? row_scale(am[row], true) : 1.f;
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
                     const int col = j0 + 32 * h + lane;
@@ -121,7 +121,7 @@ struct TileEnd {
                     for (int p = 1; p < S; ++p) v += part[p][k][h];
                     if (row >= d || col > row) continue;             // (col <= row < d)
                     v *= alpha;
-                    if (TF32) v = (v * mul[k]) * scale[h];
+                    if (SPLIT) v = (v * mul[k]) * scale[h];
                     v += old[k][h];
                     out[32 * h] = v;
                     if ((row | col) == 0) hessian_check(out, err_word, call);
@@ -152,15 +152,15 @@ struct TileEnd {
     }
 };
 
-template <bool TF32>
+template <bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
           float* __restrict__ H, int d, int num_kb_all, int n_split, float alpha, float beta, int layer0,
           int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
           const unsigned* __restrict__ amax) {
-    using C = Cfg<TF32>;
+    using C = Cfg<SPLIT>;
     constexpr int STAGE_BYTES = C::TILES * TILE_BYTES;
-    constexpr uint32_t TMEM_COLS = TF32 ? 512u : 256u;   // main x2 (+ cross terms), power of two
+    constexpr uint32_t TMEM_COLS = SPLIT ? 512u : 256u;   // main x2 (+ cross terms), power of two
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[C::STAGES], bar_empty[C::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_final;
     __shared__ uint32_t tmem_base_slot;
@@ -227,7 +227,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                 const int x = (kb_begin + kb) * C::BK;
                 tma_load_3d(base, &map_hi, full, x, i0, l);
                 if (!diag) tma_load_3d(base + TILE_BYTES, &map_hi, full, x, j0, l);
-                if (TF32) {
+                if (SPLIT) {
                     tma_load_3d(base + 2 * TILE_BYTES, &map_lo, full, x, i0, l);
                     if (!diag) tma_load_3d(base + 3 * TILE_BYTES, &map_lo, full, x, j0, l);
                 }
@@ -239,7 +239,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
         if (lane == 0) {
             // ---------------- MMA issuer
             // operand format of the instruction: 1 = BF16, 0 = F16 (A and B alike; the split is fp16)
-            const uint32_t idesc = make_idesc(TF32 ? 0u : fmt16, TM, TM);
+            const uint32_t idesc = make_idesc(SPLIT ? 0u : fmt16, TM, TM);
             const uint32_t tmem_cross = tmem_base + 256u;
             int kb = 0, s = 0;
             uint32_t ph = 0u;
@@ -266,7 +266,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                     for (int k = 0; k < C::BK / C::UK; ++k) {
                         const uint64_t adv = (uint64_t)(k * 32 / 16);   // 32 bytes per MMA along K
                         const uint32_t acc_main = ((kb - kb_first) | k) ? 1u : 0u;
-                        if (TF32) {
+                        if (SPLIT) {
                             umma_bf16(tmem_main, a_hi + adv, b_hi + adv, idesc, acc_main);
                             umma_bf16(tmem_cross, a_hi + adv, b_lo + adv, idesc, (kb | k) ? 1u : 0u);
                             umma_bf16(tmem_cross, a_lo + adv, b_hi + adv, idesc, 1u);
@@ -315,7 +315,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
             }
         }
         if (!failed) {
-            if (TF32) {
+            if (SPLIT) {
                 // the last chunk's commit also covers every cross-term MMA
 #pragma unroll
                 for (int cc = 0; cc < NC / 32; ++cc) {
@@ -354,12 +354,12 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
 
     // Every CTA of the cluster finishes its share of the rows.
     float* Hl = H + (size_t)(layer0 + l) * d * d;
-    const unsigned* am = TF32 ? amax + (size_t)l * d : nullptr;
+    const unsigned* am = SPLIT ? amax + (size_t)l * d : nullptr;
     const TileEnd end{out_tile, mirror, rank, i0, j0, d, alpha, beta, Hl, am, err_word, call};
-    if (n_split == 1) end.finish<1, 4, TF32>();
-    else if (n_split == 2) end.finish<2, 4, TF32>();
-    else if (n_split == 4) end.finish<4, 4, TF32>();
-    else end.finish<8, 2, TF32>();
+    if (n_split == 1) end.finish<1, 4, SPLIT>();
+    else if (n_split == 2) end.finish<2, 4, SPLIT>();
+    else if (n_split == 4) end.finish<4, 4, SPLIT>();
+    else end.finish<8, 2, SPLIT>();
     if (n_split > 1) cluster.sync();                         // no CTA retires while others read its tile
 }
 
@@ -767,20 +767,18 @@ bool quad_rows(const void* A, long long lda) {
     return (reinterpret_cast<uintptr_t>(A) % 16) == 0 && lda % 4 == 0;
 }
 
-// 3-D map over [layers, rows, K] with box {128 bytes of K, 128 rows, 1 layer}, 128-byte swizzle,
+// 3-D map over a 16-bit [layers, rows, K] with box {128 bytes of K, 128 rows, 1 layer}, 128-byte swizzle,
 // zero fill outside the tensor (ragged d and ragged token counts contribute zeros).
 bool make_map(CUtensorMap* m, const void* base, ziplm_dtype dt, long long K, int rows, int layers,
               long long pitch_elems) {
-    const bool f32 = (dt == ZIPLM_F32);
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
-    const size_t esz = f32 ? 4 : 2;
+    const size_t esz = 2;
     cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)layers};
     cuuint64_t strides[2] = {(cuuint64_t)pitch_elems * esz, (cuuint64_t)pitch_elems * esz * rows};
     cuuint32_t box[3] = {(cuuint32_t)(ROW_BYTES / esz), (cuuint32_t)TM, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = enc(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                            : dt == ZIPLM_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
+    CUresult r = enc(m, dt == ZIPLM_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
                      const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -81,13 +81,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-}
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
@@ -135,8 +128,8 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t smem_addr) {
            (2ull << 61);
 }
 
-// Instruction descriptor: fp32 accumulate, A and B K-major, M x N output tile; operand format
-// 2 = TF32 (kind::tf32); 1 = BF16 or 0 = F16 (kind::f16, A and B of the same type).
+// Instruction descriptor of kind::f16: fp32 accumulate, A and B K-major and of the same type (operand format
+// 1 = BF16, 0 = F16), M x N output tile.
 __host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt, int M, int N) {
     return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
