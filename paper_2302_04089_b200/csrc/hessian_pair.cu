@@ -139,8 +139,9 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     using C = PairCfg<SPLIT>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[C::STAGES], bar_empty[C::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_final;
+    __shared__ uint64_t bar_report;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, reported;
 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;        // swizzled tiles need 1024-byte alignment
@@ -171,6 +172,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
             mbar_init(smem_u32(&bar_acc_empty[b]), 2 * PAIR_EPI);     // every epilogue warp of both CTAs
         }
         mbar_init(smem_u32(&bar_final), 1);
+        mbar_init(smem_u32(&bar_report), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -187,11 +189,11 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     volatile int* abortp = &abort_flag;
     bool failed = false;
     int issued = 0;                                       // K blocks whose copies were started (thread 0)
+    auto bytes = [&](int) { return (uint32_t)((diag ? 1 : 2) * C::PARTS * OP_BYTES); };     // of a K block, per CTA
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- TMA producer (each CTA its own half of the operands)
-            const uint32_t bytes = (uint32_t)((diag ? 1 : 2) * C::PARTS * OP_BYTES);
             const int ya = i0 + (int)rank * HALF, yb = j0 + (int)rank * HALF;
             const uint32_t full0 = cluster_addr(smem_u32(&bar_full[0]), lead);
             int s = 0;
@@ -203,7 +205,7 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                 }
                 const uint32_t full = full0 + 8u * (uint32_t)s;
                 const uint32_t base = tiles + (uint32_t)s * kStageBytes<SPLIT>;
-                if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2 * bytes);
+                if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2 * bytes(kb));
                 const int x = (kb_begin + kb) * BK;
                 tma_load_3d_pair(base, &map_hi, full, x, ya, l);
                 if (SPLIT) tma_load_3d_pair(base + OP_BYTES, &map_lo, full, x, ya, l);
@@ -214,6 +216,8 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
                 issued = kb + 1;
                 if (++s == C::STAGES) { s = 0; ph ^= 1u; }
             }
+            if (rank == 1)
+                pair_report(cluster_addr(smem_u32(&reported), lead), cluster_addr(smem_u32(&bar_report), lead), issued);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
@@ -415,13 +419,8 @@ k_syrk_pair(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ 
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (threadIdx.x == 0 && rank == 0 && abort_flag) {
-        // Copies that were started land in the pair's shared memory and are counted here: wait for
-        // them (bounded; the last STAGES K blocks are the latest phases of their barriers) before
-        // either CTA retires.
-        for (int kb = issued > C::STAGES ? issued - C::STAGES : 0; kb < issued; ++kb)
-            mbar_wait_quiet(smem_u32(&bar_full[kb % C::STAGES]), (uint32_t)(kb / C::STAGES) & 1u);
-    }
+    if (threadIdx.x == 0 && rank == 0 && abort_flag)
+        pair_land<C::STAGES>(bar_full, issued, smem_u32(&bar_report), &reported, bytes);
     __syncwarp();
     cluster_barrier();            // the pair's MMAs, copies and remote arrivals are over
     if (n_parts > 1)

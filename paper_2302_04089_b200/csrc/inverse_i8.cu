@@ -179,9 +179,9 @@ __global__ void __launch_bounds__(I8_THREADS, 1) __cluster_dims__(2, 1, 1)
 k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
              const __grid_constant__ I8Product p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full, bar_acc_empty, bar_final;
+    __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full, bar_acc_empty, bar_final, bar_report;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, reported;
     const uint32_t raw = smem_u32(smem_raw), ring = (raw + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = blockIdx.x & 1u;
@@ -217,6 +217,7 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
         mbar_init(smem_u32(&bar_acc_full), 1);
         mbar_init(smem_u32(&bar_acc_empty), 2 * EPI);
         mbar_init(smem_u32(&bar_final), 1);
+        mbar_init(smem_u32(&bar_report), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -231,7 +232,9 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
     const uint32_t tmem_base = tmem_base_slot;
     volatile int* abortp = &abort_flag;
     bool failed = false;
-    int issued = 0;
+    int issued = 0;                              // K blocks whose copies were started (thread 0)
+    auto first_digit = [&](int it) { return it >= n_kb ? 0 : 4; };
+    auto bytes = [&](int it) { return (uint32_t)((SL - first_digit(it)) * (A_BYTES + B_BYTES)); };   // per CTA
 
     if (warp == 0) {
         if (lane == 0) {
@@ -244,15 +247,16 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                 const int pass = it >= n_kb, kx = (kb0 + it - (pass ? n_kb : 0)) * KB;
                 if (!mbar_wait(smem_u32(&bar_empty[s]), ph, abortp)) { failed = true; break; }
                 const uint32_t full = full0 + 8u * (uint32_t)s, base = ring + (uint32_t)s * STAGE;
-                const int first = pass ? 0 : 4;
-                if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * (uint32_t)((SL - first) * (A_BYTES + B_BYTES)));
-                for (int q = first; q < SL; ++q) {
+                if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * bytes(it));
+                for (int q = first_digit(it); q < SL; ++q) {
                     tma_load_4d_pair(base + q * A_BYTES, &map_x, full, kx, ya, q, l);
                     tma_load_4d_pair(base + SL * A_BYTES + q * B_BYTES, &map_y, full, kx, yb, q, l);
                 }
                 issued = it + 1;
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
+            if (rank == 1)
+                pair_report(cluster_addr(smem_u32(&reported), 0), cluster_addr(smem_u32(&bar_report), 0), issued);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
@@ -377,11 +381,8 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (threadIdx.x == 0 && rank == 0 && abort_flag) {
-        // copies that were started are counted here: wait for them (bounded) before either CTA retires
-        for (int it = issued > STAGES ? issued - STAGES : 0; it < issued; ++it)
-            mbar_wait_quiet(smem_u32(&bar_full[it % STAGES]), (uint32_t)(it / STAGES) & 1u);
-    }
+    if (threadIdx.x == 0 && rank == 0 && abort_flag)
+        pair_land<STAGES>(bar_full, issued, smem_u32(&bar_report), &reported, bytes);
     __syncwarp();
     cluster_barrier();
     if (warp == 1)

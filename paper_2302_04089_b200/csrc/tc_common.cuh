@@ -194,6 +194,29 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t both) {
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
         ::"r"(bar), "h"(both) : "memory");
 }
+// Both CTAs' copies into the operand ring of a pair are counted on the leader's barriers, so only the leader can
+// wait for them.  When a role has given up, the other CTA's producer may have started more K blocks than the
+// leader's, which has not armed their barriers: it tells how many (pair_report, at its end), and the leader waits
+// for the copies under way, with a limit, before either CTA retires.  bytes(kb): of one CTA's half of K block kb.
+__device__ __forceinline__ void pair_report(uint32_t leader_count, uint32_t leader_bar, int issued) {
+    cluster_store(leader_count, issued);
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(leader_bar) : "memory");
+}
+template <int STAGES, typename Bytes>
+__device__ __forceinline__ void pair_land(uint64_t (&bar_full)[STAGES], int issued, uint32_t bar_report,
+                                          const volatile int* reported, Bytes bytes) {
+    int all = issued;
+    if (mbar_wait_quiet(bar_report, 0u)) {
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+        all = max(all, *reported);
+    }
+    // the last STAGES blocks are the latest phases of their barriers
+    for (int kb = max(all - STAGES, 0); kb < all; ++kb) {
+        const uint32_t bar = smem_u32(&bar_full[kb % STAGES]);
+        if (kb >= issued) mbar_expect_tx(bar, bytes(kb));
+        mbar_wait_quiet(bar, (uint32_t)(kb / STAGES) & 1u);
+    }
+}
 
 // Asynchronous stores to another CTA of the cluster that complete on a barrier of that CTA (addresses of
 // the shared::cluster window).
