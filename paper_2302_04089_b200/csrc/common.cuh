@@ -12,6 +12,10 @@ namespace ziplm {
 
 constexpr int kTile = 64;          // tile edge of the float64 factorisation kernels
 constexpr size_t kAlign = 256;     // alignment of every carve-out of a workspace
+// SMs of the part this library is built for, for the rules that choose kernels and splits.  Another count makes them
+// choose worse, not wrongly.  A constant, because workspace sizes follow from some of the rules: they must not depend
+// on the device that is current, or on whether there is one, when the size is asked for.
+constexpr int kSMs = 148;
 
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 inline int round_up_int(int x, int a) { return (x + a - 1) / a * a; }

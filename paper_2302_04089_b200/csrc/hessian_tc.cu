@@ -833,7 +833,7 @@ size_t product_scratch_bytes(int L, int d, long long N, ziplm_dtype dt, bool tok
 // a chain of 32 K blocks on one CTA).
 int hessian_tile_split(long long tiles, long long num_kb) {
     int split = 1;
-    while (split < 8 && tiles * split * 2 <= 148 && num_kb / (split * 2) >= 4) split *= 2;
+    while (split < 8 && tiles * split * 2 <= kSMs && num_kb / (split * 2) >= 4) split *= 2;
     return split;
 }
 

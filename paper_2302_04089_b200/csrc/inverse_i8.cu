@@ -448,7 +448,7 @@ bool i8_symmetric_pays(int L, int rows, int K, double float64_clocks) {
     const int nI = (rows + PM - 1) / PM, nJ = (rows + PN - 1) / PN;
     double tiles = 0;
     for (int I = 0; I < nI; ++I) tiles += 2 * I + 2 < nJ ? 2 * I + 2 : nJ;
-    const double waves = ceil(L * tiles / 74);           // two of the 148 SMs to a tile
+    const double waves = ceil(L * tiles / (kSMs / 2));     // two SMs to a tile
     return 20000.0 + waves * ((K + KB - 1) / KB * 7000.0 + 30000.0) < float64_clocks;
 }
 

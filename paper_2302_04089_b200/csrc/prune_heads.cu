@@ -571,7 +571,7 @@ struct HeadsWs {
 // float64 kernel runs at 0.65 of its instruction's rate, and a CTA's chain is 4500 clocks per 64^3.
 bool gram_on_i8(int L, int r, int d, int g) {
     const double G = d / g, ctas = L * G * (G + 1) / 2, cta = (double)r * g * g / 64 * 1.1 + 4000;
-    return i8_symmetric_pays(L, d, r, cta > ctas * cta / (148 * 0.65) ? cta : ctas * cta / (148 * 0.65));
+    return i8_symmetric_pays(L, d, r, cta > ctas * cta / (kSMs * 0.65) ? cta : ctas * cta / (kSMs * 0.65));
 }
 
 HeadsWs carve_heads(void* ws, int L, int r, int d, int g, int n_levels) {
@@ -623,7 +623,7 @@ ziplm_status run_heads(HeadsWs& ws, float damp_frac, const int* levels, float* l
         ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.order, 0xFF, sizeof(int) * (size_t)L * G, st));
         if (w.saliency) ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.saliency, 0, sizeof(float) * (size_t)L * G, st));
         ZIPLM_CHECK_CUDA(cudaMemsetAsync(ws.zero, 0, ws.zero_bytes, st));
-        k_heads_init<<<592, HT, 0, st>>>(w);
+        k_heads_init<<<4 * kSMs, HT, 0, st>>>(w);
         ZIPLM_CHECK_LAUNCH();
         if (n_steps > 0 || base_loss) {
             if (gram_on_i8(L, w.r, w.d, g)) {

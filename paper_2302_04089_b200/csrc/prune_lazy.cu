@@ -1045,7 +1045,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         if (g != ZIPLM_OK) return g;
         if (base_loss) {
             ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.base_acc, 0, sizeof(double) * L, st));
-            k_lazy_base_loss<<<dim3(148, L), 256, 0, st>>>(d, ld, w.Q[0], H, w.base_acc);
+            k_lazy_base_loss<<<dim3(kSMs, L), 256, 0, st>>>(d, ld, w.Q[0], H, w.base_acc);
             ZIPLM_CHECK_LAUNCH();
             k_lazy_base_finish<<<(L + 63) / 64, 64, 0, st>>>(L, w.base_acc, base_loss);
             ZIPLM_CHECK_LAUNCH();

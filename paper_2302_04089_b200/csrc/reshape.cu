@@ -158,8 +158,8 @@ ziplm_status run_gather_columns(const float* M, long long ld, long long layer_st
         // stores of two or four columns where they stay aligned and leave enough threads
         const long long threads = (long long)n_out * ((rows + COL_ROWS - 1) / COL_ROWS) * ln;
         const bool al = reinterpret_cast<uintptr_t>(out) % 16 == 0;
-        const int vec = al && n_out % 4 == 0 && threads >= 4ll * 148 * 1024 ? 4
-                        : al && n_out % 2 == 0 && threads >= 2ll * 148 * 1024 ? 2 : 1;
+        const int vec = al && n_out % 4 == 0 && threads >= 4ll * kSMs * 1024 ? 4
+                        : al && n_out % 2 == 0 && threads >= 2ll * kSMs * 1024 ? 2 : 1;
         auto kernel = vec == 4 ? k_gather_columns<4> : vec == 2 ? k_gather_columns<2> : k_gather_columns<1>;
         const dim3 grid((unsigned)((n_out + 256 * vec - 1) / (256 * vec)), (unsigned)((rows + COL_ROWS - 1) / COL_ROWS),
                         (unsigned)ln);
