@@ -735,8 +735,7 @@ def run_ours(args, shape):
                                               "count (24 B) includes the second, mirrored store that "
                                               "lets the steps kernel read a pivot column as a row"),
                           note="rank-32 update of H^-1 and Q, the operation with the largest summed "
-                               "time in the timed path (the phase also holds the small kernel that "
-                               "packs the pending vectors for the tensor cores).  About three blocks "
+                               "time in the timed path.  About three blocks "
                                "in four at full width leave removed positions in place and run dense "
                                "128 x 128 tiles on tcgen05 (bf16 x 3 split of the rank-32 operands, TMA "
                                "loads, direct and mirrored stores), W^T included as extra tiles of the "
@@ -755,11 +754,12 @@ def run_ours(args, shape):
                               ms=phases.get("lazy_steps", (0.0, 0))[0],
                               us_per_greedy_step=1e3 * phases.get("lazy_steps", (0.0, 0))[0] / max(n_removed, 1),
                               note="32 sequential greedy steps per launch on a cluster of 4, 2 or 1 CTAs "
-                                   "per layer; a chain of long-latency instructions (cluster barrier, "
-                                   "shuffles, shared-memory loads, float64 conversions), second to the "
-                                   "rank-32 update in summed time and without a throughput roofline"),
+                                   "per layer, the last 256 structures in one launch of the float64 "
+                                   "endgame (in the time); a chain of long-latency instructions (offers "
+                                   "exchanged between CTAs, shuffles, shared-memory loads, float64 "
+                                   "conversions) without a throughput roofline"),
             roofline_hessian=dict(
-                kernel="k_row_absmax_split + k_syrk_tc<split>", bound="tensor",
+                kernel="k_row_absmax_split + k_syrk_pair<split>", bound="tensor",
                 achieved=3.0 * hs_useful / (hs_ms * 1e-3) / 1e12 if hs_ms > 0 else 0.0, peak=f16_peak,
                 unit="TFLOP/s", frac=(3.0 * hs_useful / (hs_ms * 1e-3) / 1e12 / f16_peak) if hs_ms > 0 else 0.0,
                 useful_tflops=hs_useful / (hs_ms * 1e-3) / 1e12 if hs_ms > 0 else 0.0,
@@ -771,9 +771,9 @@ def run_ours(args, shape):
                 note="fp32 activations: every feature row is scaled by a power of two and split "
                      "into two fp16 parts, every product is three fp16 MMAs (x1*x1, x1*x2, x2*x1), "
                      "so the tensor-pipe work is 3 x the useful d^2 N flop per layer; the time is "
-                     "that of the whole call, the row-maximum and split pre-pass included; the "
-                     "kernel is bound by its L2 -> shared-memory operand traffic (64 KB per K "
-                     "block of 64 tokens against 816 clocks of MMAs)"),
+                     "that of the whole call, the row-maximum and split pre-pass included; a pair of "
+                     "CTAs computes 256 x 256 tiles, 64 KB of operands per CTA and K block of 64 "
+                     "tokens for 1536 clocks of MMAs, and the ends of the tiles overlap no MMA"),
             roofline_streaming_update=dict(
                 kernel="k_neuron_update", bound="hbm", achieved=achieved, peak=peak, unit="GB/s",
                 frac=achieved / peak,

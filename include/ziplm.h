@@ -68,7 +68,8 @@ const char* ziplm_status_string(ziplm_status s);
  * three exact partial products per product, about 21 significant bits), bf16 and fp16 inputs are multiplied exactly
  * (an fp16 or bf16 product has at most 22 significant bits).
  *
- *   H          dev, [L, d, d] fp32, in/out; full symmetric matrix on return
+ *   H          dev, [L, d, d] fp32, in/out; full symmetric matrix on return.  Aligned to its
+ *              element size, as every buffer here that does not say otherwise.
  *   X          dev, [L, d, ldx] of x_dtype, token index contiguous; only the first n_tokens
  *              entries of each row are read; not modified.  The base address must be 16-byte
  *              aligned and ldx * sizeof(element) a multiple of 16.
@@ -82,7 +83,8 @@ const char* ziplm_status_string(ziplm_status s);
  * Every wait inside the tensor-core kernel is bounded.  Should one run out (it cannot on a healthy
  * device), the call has no status output of its own: H[l][0][0] of every layer is NaN on return,
  * so that ziplm_damped_inverse or ziplm_prune_layers on that H reports ZIPLM_ERR_NONFINITE for
- * every layer.  The same holds for ziplm_hessian_accumulate_tokens.
+ * every layer.  Replays of a captured call report their own waits only.  The same holds for
+ * ziplm_hessian_accumulate_tokens.
  */
 size_t ziplm_hessian_workspace_bytes(int L, int d, long long n_tokens, ziplm_dtype x_dtype);
 
@@ -338,8 +340,8 @@ ziplm_status ziplm_select_levels(const float* loss, const float* base_loss, cons
  *                    fastest configuration), ZIPLM_ERR_NONFINITE
  *   workspace        dev scratch >= ziplm_search_workspace_bytes(...), 256-byte aligned
  *
- * One thread block runs one whole search, so the call is efficient when many targets are searched
- * together.  Errors: as ziplm_select_levels; ZIPLM_ERR_UNSUPPORTED also for n_modules > 512.
+ * A search runs on a cluster of up to 16 thread blocks, each evaluating another step from the current
+ * best vector, and on fewer where many targets are searched together.  Errors: as ziplm_select_levels; ZIPLM_ERR_UNSUPPORTED also for n_modules > 512.
  */
 size_t ziplm_search_workspace_bytes(int n_searches, int n_modules, int n_buckets);
 
@@ -360,8 +362,8 @@ ziplm_status ziplm_search_levels(const float* loss, const float* base_loss, cons
  *                          option defaults to 0.  ZIPLM_ERR_INVALID_ARG for an unknown option or a
  *                          value outside its range.  Results never depend on an option beyond
  *                          rounding (every variant passes the same parity tests).
- *     ZIPLM_OPT_NEURON_PATH       0: delayed rank-32 updates where the shape allows them
- *                                 (d_col % 4 == 0, d_col <= 6144); 1: per-step streaming update.
+ *     ZIPLM_OPT_NEURON_PATH       0: delayed rank-32 updates (d_col <= 6144; wider layers take the
+ *                                 other path); 1: per-step streaming update.
  *     ZIPLM_OPT_LAYER_GROUPS      0: default (6); 1..8: number of layer groups that
  *                                 ziplm_prune_layers runs on internal streams (1 = none).
  *     ZIPLM_OPT_FORCE_BLOCK_PATH  1: group_size 1 takes the general block path (float64 state).

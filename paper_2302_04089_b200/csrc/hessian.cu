@@ -6,8 +6,8 @@
 // This file holds the route choice and the CUDA-core route: fp32 FMA on 64 x 64 tiles with a
 // two-level fp32 sum (the running tile sum is folded into a second accumulator every 512 tokens,
 // which keeps the rounding error of a 1e4 .. 1e5 term sum near the fp32 unit roundoff).  The
-// tensor-core route (hessian_tc.cu) is the default; the CUDA-core route serves token counts
-// below one K block and can be forced with ziplm_set_option(ZIPLM_OPT_HESSIAN_ROUTE, 1) for comparison.
+// tensor-core route (hessian_tc.cu) is the default; the CUDA-core route serves fewer than 32
+// tokens (half a K block) and can be forced with ziplm_set_option(ZIPLM_OPT_HESSIAN_ROUTE, 1) for comparison.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 

@@ -439,9 +439,9 @@ int pair_count(int d) {
 
 // Pairs that share a tile: the number with the shortest chain of K blocks over all waves, where the tiles leave
 // SMs idle or a second wave nearly empty (most_clusters: the occupancy calculator's room for clusters of that
-// many pairs on the kSMs of a B200, whose GPCs differ in size); the ends of a tile weigh 14 to 28 K blocks.  Four K blocks each at least.  8 x 512 features,
-// 2048 bf16 tokens: 39.8 -> 29.7 us a call, 2 x 1100 of 500 fp32 37.7 -> 27.6, 1 x 1322 of 4099 64.5 -> 58.3,
-// 1 x 3072 of 8192 (78 tiles) 347 -> 304.
+// many pairs on the kSMs of a B200, whose GPCs differ in size); the ends of a tile weigh 14 to 28 K blocks.
+// Four K blocks each at least.  8 x 512 features, 2048 bf16 tokens: 39.8 -> 29.7 us a call, 2 x 1100 of 500
+// fp32 37.7 -> 27.6, 1 x 1322 of 4099 64.5 -> 58.3, 1 x 3072 of 8192 (78 tiles) 347 -> 304.
 int most_clusters(int parts) {
     constexpr int n[5] = {0, kSMs / 2, 33, 22, 15};
     return n[parts];

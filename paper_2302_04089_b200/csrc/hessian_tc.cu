@@ -18,9 +18,10 @@
 //            accuracy, which matters because the kernel is bound by the L2 -> shared-memory
 //            operand traffic.
 //
-// One CTA per tile: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, warps 2..9 =
-// epilogue (two per TMEM lane quarter; they drain the accumulator every few K blocks, see
-// below).  Every mbarrier wait is bounded; if one runs out the kernel raises the error word and
+// One CTA per tile, or a cluster of up to eight where the tiles are few, each CTA a range of the
+// tile's K blocks (problems of many tiles go to hessian_pair.cu).  Warp 0 = TMA producer, warp 1 =
+// TMEM owner + MMA issuer, warps 2..9 = epilogue (two per TMEM lane quarter; they drain the
+// accumulator every few K blocks, see below).  Every mbarrier wait is bounded; if one runs out the kernel raises the error word and
 // every role leaves its loop; the issuer then waits (one more commit) for the MMAs it has issued,
 // the producer for the copies it has started, and the CTA leaves through the normal exit (TMEM
 // freed), so a lost copy can never hang the GPU.  H[l][0][0] of every layer is NaN then
@@ -620,7 +621,7 @@ __global__ void __launch_bounds__(256) k_tokens16_to_kmajor(const uint16_t* __re
     }
 }
 
-// Both pre-passes of token-major fp32 batches in one: a cluster of up to eight CTAs takes 64 features of
+// Both pre-passes of token-major fp32 batches in one: a cluster of up to eight CTAs takes 32 features of
 // all N tokens, each CTA a range of tokens that it keeps in shared memory; the features' largest magnitudes
 // meet through distributed shared memory, and the scaled fp16 parts leave K-major.  A is read once instead
 // of twice and nothing has to be zeroed beforehand (for a small batch it is one launch instead of three).
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(256) k_tokens16_to_kmajor(const uint16_t* __re
 // In shared memory a feature's tokens lie in a row, in quads whose place is permuted by the feature, so that
 // a warp's stores of 8 x 4 features by 4 tokens and its loads of a row's quads meet no bank conflict.
 constexpr int TS_FEATURES = 32, TS_THREADS = 4 * TS_FEATURES;
-constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 192 KiB of shared memory
+constexpr int TS_TOKENS = 768;                   // most tokens per CTA: 96 KiB of shared memory
 __device__ __forceinline__ int ts_at(int f, int t, int pitch) { return f * pitch + (t ^ (f & 28)); }
 template <bool VEC>
 __global__ void __launch_bounds__(TS_THREADS) k_tokens_split(const float* __restrict__ A, long long lda, int N, int d,

@@ -6,10 +6,12 @@
 //     factor [lo, mid);   F21 = A21 M11^T;   A22 -= F21 F21^T;   factor [mid, hi);
 //     M21 = -M22 (F21 M11)
 // so that nearly all of the work sits in large, wide products (thousands of independent tiles
-// per launch) and only the 64 x 64 leaves are sequential.  Everything is float64: the greedy
-// loop that follows needs the diagonal of H^-1 to roughly 1e-7 relative, which an fp32
-// factorisation of a matrix with condition number 1e3 .. 1e5 does not give.  The matrix is
-// padded to a multiple of 64 with an identity block, whose inverse is again the identity.
+// per launch) and only the 64 x 64 leaves are sequential.  Everything has float64 accuracy: the
+// greedy loop that follows needs the diagonal of H^-1 to roughly 1e-7 relative, which an fp32
+// factorisation of a matrix with condition number 1e3 .. 1e5 does not give.  Products of blocks of
+// at least eight tiles a side run in digits on the int8 tensor cores (inverse_i8.cu), the others and
+// the ranges of up to four tiles on the float64 instruction.  The matrix is padded to a multiple of
+// 64 with an identity block, whose inverse is again the identity.
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -451,9 +453,9 @@ __device__ __forceinline__ void leaf_factor(const double* Ag, double* Mg, int dp
 // X_ik -= F_ij M_jk (X_ik, kept in M's tile, is what M_ik is before its own row's stage).  The tiles of a
 // phase are independent and dealt out to the ranks; rank 0 updates the next diagonal tile first, out of its own
 // F and without a detour through memory, and goes on to its leaf without waiting for the others, so the chain is
-// leaf, two products, leaf, ...: one cluster barrier a stage, and the arrival at another.  Every product is a 64 x 64 x 64 tile product of a whole CTA on the float64 tensor
-// core, its operands fetched from global memory (the L2) into shared memory; on one CTA alone the 32
-// products of four tiles took 150 us of 184.
+// leaf, two products, leaf, ...: one cluster barrier a stage, and the arrival at another.  Every product is a
+// 64 x 64 x 64 tile product of a whole CTA on the float64 tensor core, its operands fetched from global memory (the
+// L2) into shared memory; on one CTA alone the 32 products of four tiles took 150 us of 184.
 constexpr int kSmallCluster = 4;
 __device__ __forceinline__ void cluster_arrive() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -1,8 +1,8 @@
 // The last steps of a greedy run over neurons (up to kEndgame = 256 live structures), and whole runs of
 // layers that are no wider.
 //
-// The delayed-update path (prune_lazy.cu) pays three dependent launches for every 32 steps and a chain of
-// about 3700 clocks a step, whatever the size: a layer of 64 x 256 took 0.7 ms, nearly all of it latency.
+// The delayed-update path (prune_lazy.cu) pays two or three dependent launches for every 32 steps and a chain
+// of 2800 to 3300 clocks a step, whatever the size: a layer of 64 x 256 took 0.7 ms, nearly all of it latency.
 // With 256 structures or fewer the state fits the registers of a cluster of eight CTAs, in float64:
 //
 //   k_endgame_setup   H_lambda restricted to the live structures (by the remark after Eq. 4 its inverse is

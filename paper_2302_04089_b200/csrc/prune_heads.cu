@@ -14,10 +14,10 @@
 // factorisation with three barriers per column, a forward substitution and a Gram product over all
 // rows of W for every head and step (232 us a step for 12 layers of 12 heads of 64), then another
 // 250 us for the update on the float64 FMA pipe.  Here every product is a g x g x g tile product on
-// the float64 tensor-core instruction, the inverse of a head's block is one pass of symmetric sweeps
-// in registers (one barrier per column), and a step is two launches: `solve` (which also selects) and
-// `update` (whose diagonal tiles go on to score their head for the next step, and whose tiles of W
-// write the snapshot).
+// the float64 tensor-core instruction, the inverse of a head's block goes by 16 x 16 blocks (two
+// barriers per block), and a step is two launches: `solve` (which also selects) and `update` (whose
+// diagonal tiles go on to score their head for the next step, and whose tiles of W write the
+// snapshot).
 #include <math.h>
 
 #include "common.cuh"

@@ -19,15 +19,15 @@
 //     again the leading n x n corner in original column order.
 //
 // Launches per block, for all L layers at once: one "steps" kernel (one thread-block cluster per
-// layer runs the B greedy steps back to back with one cluster barrier per step -- layers are
-// independent, so no grid-wide synchronisation is needed) and two update kernels.  Block boundaries are placed on
-// the requested levels, where W is up to date and can be snapshotted.
+// layer runs the B greedy steps back to back; its CTAs exchange their offers by asynchronous stores,
+// and layers are independent, so a step has neither a cluster barrier nor a grid-wide one) and one
+// update kernel, or two where the block squeezes removed positions out.  Block boundaries are placed
+// on the requested levels, where W is up to date and can be snapshotted.
 //
 // Layout per layer: A, Q fp32 [d, d], off-diagonal entries in both triangles (two buffers each, ping-pong),
 // Wt = W^T fp32 [d, rp] (two buffers), float64 diagonals, pending U, Z [B, d] and C [B, rp].
 #include <cooperative_groups.h>
 #include <math.h>
-
 
 #include <cuda.h>
 

@@ -16,10 +16,11 @@
 // exact in the fp32 accumulator, and the six partial products x_a y_b with a + b <= 4 are kept
 // (the others are below 2^-26 of the product), so a product is as good as an fp32 one.
 //
-// The update kernel runs one CTA per SM.  Work is cut into tiles of 128 x 128 entries on or
-// below the diagonal; runs of consecutive tiles of one row strip ("segments") are handed out
-// through an atomic counter, so a CTA that starts late (another kernel holds its SM) simply finds
-// less left to do.  Inside a CTA three kinds of warps work as a pipeline, linked by mbarriers only:
+// The update kernel runs one CTA on each of two thirds of the SMs.  Work is cut into tiles of
+// 128 x 128 entries on or below the diagonal; runs of consecutive tiles of one row strip
+// ("segments") are handed out through an atomic counter, so a CTA that starts late (another kernel
+// holds its SM) simply finds less left to do.  Inside a CTA three kinds of warps work as a pipeline,
+// linked by mbarriers only:
 //   warp 0      fetches segments, publishes one descriptor per tile (layer, tile origin) and
 //               loads the tile's packed operands by TMA (the 128 rows once per segment, the 128
 //               columns per tile);

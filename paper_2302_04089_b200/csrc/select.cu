@@ -7,7 +7,7 @@
 // coefficient vector (1000 mutation steps), so the kernel solves K candidates per launch.
 //
 // Time is discretised into n_buckets units of budget / n_buckets, every option rounded UP, so a
-// selection that fits in units also fits in real time.  One CTA per candidate runs the dynamic
+// selection that fits in units also fits in real time.  A CTA runs a candidate's dynamic
 // programme over modules with the two value rows f[0 .. n_buckets] in shared memory (float64):
 //     f_{m+1}[b] = min over options s with u[m][s] <= b of  f_m[b - u[m][s]] + c[m] p[m][s]
 // (ties: lowest s), stores the argmin per (module, b) in global scratch and walks it back from
