@@ -21,11 +21,11 @@
 // One CTA per tile, or a cluster of up to eight where the tiles are few, each CTA a range of the
 // tile's K blocks (problems of many tiles go to hessian_pair.cu).  Warp 0 = TMA producer, warp 1 =
 // TMEM owner + MMA issuer, warps 2..9 = epilogue (two per TMEM lane quarter; they drain the
-// accumulator every few K blocks, see below).  Every mbarrier wait is bounded; if one runs out the kernel raises the error word and
-// every role leaves its loop; the issuer then waits (one more commit) for the MMAs it has issued,
-// the producer for the copies it has started, and the CTA leaves through the normal exit (TMEM
-// freed), so a lost copy can never hang the GPU.  H[l][0][0] of every layer is NaN then
-// (hessian_common.cuh).
+// accumulator every few K blocks, see below).  Every mbarrier wait is bounded; if one runs out the
+// kernel raises the error word and every role leaves its loop; the issuer then waits (one more commit)
+// for the MMAs it has issued, the producer for the copies it has started, and the CTA leaves through
+// the normal exit (TMEM freed), so a lost copy can never hang the GPU.  H[l][0][0] of every layer is
+// NaN then (hessian_common.cuh).
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>

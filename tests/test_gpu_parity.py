@@ -901,11 +901,13 @@ def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
     assert torch.equal(H.double(), ref)
 
 
-@pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030), (1, 2817, 4100)])
+@pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030), (1, 2817, 4100),
+                                   (1, 3072, 4100), (1, 1700, 8300), (15, 256, 8300)])
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
 def test_hessian_tiles_shared_by_pairs_of_ctas(L, d, N, dtype):
-    """Two, three and four pairs to a 256 x 256 tile, ragged K and widths, added to what is there; small
-    whole numbers, so that every sum is exact."""
+    """Two, three and four pairs to a 256 x 256 tile (and, at 2100 and 2817, one and the 128 x 128 tiles, beside
+    them), ragged K and widths, parts long enough for the second summation level, added to what is there;
+    small whole numbers, so that every sum is exact."""
     z = zb()
     g = torch.Generator().manual_seed(d)
     A = torch.randint(-3, 4, (L, N, d), generator=g).to(dtype).cuda()
