@@ -177,10 +177,10 @@ LAZY_DEAD_MAX, LAZY_DEAD_FRACTION = 128, 16   # its rule for squeezing removed p
 # proportion to the layers), not measurements of this run.  Only valid for the bench workload.
 NCU_TRAFFIC = {
     # k_lazy_update_aq_tc, first block at full size (12 layers, 3072 positions of which 3040 live)
-    "k_lazy_update_aq_tc": dict(bytes=3 * (209.6e6 + 291.3e6), launch="n_pos = 3072, m = 32, 12 layers",
+    "k_lazy_update_aq_tc": dict(bytes=3 * (210.1e6 + 291.3e6), launch="n_pos = 3072, m = 32, 12 layers",
                                 algorithmic=12 * (24.0 * 3040 * 3039 / 2 + 8.0 * 768 * 3040)),
     # k_lazy_update_aq, a compaction block near full size (12 layers, n_new = 2944)
-    "k_lazy_update_aq": dict(bytes=3 * (162.0e6 + 217.3e6), launch="n_new = 2944, m = 32, 12 layers",
+    "k_lazy_update_aq": dict(bytes=3 * (162.8e6 + 217.4e6), launch="n_new = 2944, m = 32, 12 layers",
                              algorithmic=12 * 24.0 * 2944 * 2943 / 2),
     # k_neuron_update, first step at full size (12 layers, n = 3071)
     "k_neuron_update": dict(bytes=343.1e6 + 281.9e6, launch="n = 3071, 12 layers",
