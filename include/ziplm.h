@@ -341,7 +341,8 @@ ziplm_status ziplm_select_levels(const float* loss, const float* base_loss, cons
  *   workspace        dev scratch >= ziplm_search_workspace_bytes(...), 256-byte aligned
  *
  * A search runs on a cluster of up to 16 thread blocks, each evaluating another step from the current
- * best vector, and on fewer where many targets are searched together.  Errors: as ziplm_select_levels; ZIPLM_ERR_UNSUPPORTED also for n_modules > 512.
+ * best vector, and on fewer where many targets are searched together.  Errors: as
+ * ziplm_select_levels; ZIPLM_ERR_UNSUPPORTED also for n_modules > 512.
  */
 size_t ziplm_search_workspace_bytes(int n_searches, int n_modules, int n_buckets);
 
