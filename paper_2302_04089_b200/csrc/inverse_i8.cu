@@ -245,7 +245,7 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
             uint32_t ph = 1u;
             for (int it = 0; it < 2 * n_kb; ++it) {
                 const int pass = it >= n_kb, kx = (kb0 + it - (pass ? n_kb : 0)) * KB;
-                if (!mbar_wait(smem_u32(&bar_empty[s]), ph, abortp)) { failed = true; break; }
+                if (!mbar_wait_limit(smem_u32(&bar_empty[s]), ph, abortp, p.spin)) { failed = true; break; }
                 const uint32_t full = full0 + 8u * (uint32_t)s, base = ring + (uint32_t)s * STAGE;
                 if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * bytes(it));
                 for (int q = first_digit(it); q < SL; ++q) {
@@ -457,6 +457,8 @@ ziplm_status i8_product(const I8Operand& x, const I8Operand& y, I8Product p, int
     if (x.K > kI8MostK) return ZIPLM_ERR_UNSUPPORTED;      // (no caller asks for it)
     p.rows = x.rows; p.cols = y.rows; p.K = x.K;
     p.x_scale = x.scale; p.y_scale = y.scale;
+    const int spin = option_value(ZIPLM_OPT_SPIN_LIMIT);
+    p.spin = spin > 0 ? (unsigned)spin : kSpinLimit;
     if (!make_digit_map(&mx, x.dig, L, x.rows, x.K, 128) || !make_digit_map(&my, y.dig, L, y.rows, y.K, 64))
         return ZIPLM_ERR_CUDA;
     const int nI = (p.rows + PM - 1) / PM, nJ = (p.cols + PN - 1) / PN;

@@ -26,7 +26,8 @@ struct I8Product {
     int krange, lower;                       // lower: only tiles that reach the lower triangle
     int d; const double* eq; double* out64; float* tri32; int pitch32, rows32; double* diag64;
     int* layer_status;
-    int rows, cols, K;                       // set by i8_product
+    int rows, cols, K;                       // set by i8_product, as is the
+    unsigned spin;                           // poll limit of the producers' waits
     const double* x_scale; const double* y_scale;
 };
 

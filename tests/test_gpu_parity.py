@@ -987,3 +987,21 @@ def test_replays_of_a_captured_hessian_call_after_one_whose_wait_ran_out(L, d, N
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(H, ref)
+
+
+def test_a_bounded_wait_of_the_int8_products_that_runs_out_is_reported():
+    """As for the Hessian's kernels: both producers of a pair give up after one look, the layers report the time-out,
+    and the same call is right again afterwards."""
+    z = zb()
+    H = z.hessian_accumulate_tokens(torch.randn(2, 3000, 1500, generator=torch.Generator().manual_seed(5)).cuda())
+    ref, status = z.damped_inverse(H, 0.01)
+    assert status.tolist() == [0, 0]
+    z.set_option(z.Option.SPIN_LIMIT, 1)
+    try:
+        _, status = z.damped_inverse(H, 0.01)
+        torch.cuda.synchronize()
+    finally:
+        z.set_option(z.Option.SPIN_LIMIT, 0)
+    assert status.tolist() == [int(z.Status.ERR_TIMEOUT)] * 2
+    again, status = z.damped_inverse(H, 0.01)
+    assert status.tolist() == [0, 0] and torch.equal(again, ref)
