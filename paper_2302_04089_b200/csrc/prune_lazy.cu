@@ -14,9 +14,13 @@
 //     pivot column of the true matrix is the stale column minus the pending terms evaluated at
 //     p -- O(n * pending) work instead of a pass over n^2 entries.
 //   * At the end of a block the pending terms are applied to H^-1, Q and W as rank-B updates
-//     (one read + write of each matrix per B steps instead of per step), and the removed
-//     positions are squeezed out by a stable, out-of-place compaction, so the live problem is
-//     again the leading n x n corner in original column order.
+//     (one read + write of each matrix per B steps instead of per step).  Removed positions stay in
+//     place for a few blocks (idx = -1), then a block squeezes them out by a stable, out-of-place
+//     compaction, so the live problem is again the leading n x n corner in original column order.
+//
+// B is 64 where the pending vectors of a slice fit shared memory on up to eight CTAs (up to 3072 positions),
+// less above (48 up to 4096), and 32 in a block that squeezes: the update moves the same bytes for twice the
+// steps (12 x 3072: 27.3 -> 24.4 ms with all other work, 24 x 4096: 107 -> 99, 12 x 1814: 12.1 -> 11.1).
 //
 // Launches per block, for all L layers at once: one "steps" kernel (one thread-block cluster per
 // layer runs the B greedy steps back to back; its CTAs exchange their offers by asynchronous stores,
@@ -40,12 +44,18 @@ namespace ziplm {
 
 namespace {
 
-constexpr int BMAX = kPackSteps; // pending steps per block
+constexpr int GS = kPackSteps;   // steps per group of packed operands, and at most in a compaction block
+constexpr int BMAX = kPackGroups * GS;   // pending steps per dense block, at most
 constexpr int STEP_THREADS = 256; // threads per CTA of the steps kernel, four positions each
-constexpr int SLICE_MAX = 768;   // positions per CTA: 2 * BMAX * SLICE_MAX * 4 B = 192 KiB of smem
+constexpr int SLICE_MAX = 768;   // positions per CTA
+constexpr int SLICE_WIDE = 384;  // ... up to which BMAX steps are pending
+constexpr int STEPS_SMEM = 2 * BMAX * (SLICE_WIDE + 4) * 4;    // bytes of pending vectors per CTA
 constexpr int CLUSTER_MAX = 8;   // portable cluster size
-constexpr int kDeadMax = 128;    // removed positions tolerated in the arrays before they are squeezed out
-constexpr int kDeadFraction = 16; // ... or this fraction of all positions, whichever comes first
+// Removed positions tolerated in the arrays before they are squeezed out, or this fraction of all positions,
+// whichever comes first.  12 x 3072 / 24 x 4096 / 12 x 1814: 24.6 / 98 / 11.4 ms with 256 and a twelfth, 24.4 / 99 /
+// 11.1 with 320 and an eighth or 384 and an eighth, 24.4 / 100 / 11.1 with 512 and a sixth.
+constexpr int kDeadMax = 320;
+constexpr int kDeadFraction = 8;
 
 struct LazyState {
     double sumrho;
@@ -104,15 +114,16 @@ __global__ void __launch_bounds__(256) k_lazy_init(const float* __restrict__ W, 
 // Every CTA of a cluster sends its offers of all steps, also past a give-up.  Once all have been sent (behind the
 // last cluster barrier) those from step `first` on, which the CTA has not waited for, land before it leaves, or run
 // out once more: barriers of even and odd steps, armed up to step first + 1.
-__device__ __forceinline__ void land_offers(uint64_t (&bar_step)[2], int first, int nsteps, uint32_t step_bytes) {
+template <typename Bytes>
+__device__ __forceinline__ void land_offers(uint64_t (&bar_step)[2], int first, int nsteps, const Bytes& step_bytes) {
     for (int m = first; m < nsteps; ++m) {
         const uint32_t bar = tc::smem_u32(&bar_step[m & 1]);
         if (!tc::mbar_wait_quiet(bar, (uint32_t)(m >> 1) & 1u)) return;
-        if (m + 2 < nsteps) tc::mbar_expect_tx(bar, step_bytes);
+        if (m + 2 < nsteps) tc::mbar_expect_tx(bar, step_bytes(m + 2));
     }
 }
 
-// nsteps greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
+// nsteps (at most cap) greedy steps of one layer, run by a thread-block cluster of CS CTAs (CS = 1, 2, 4 or 8,
 // chosen so that a CTA's slice of positions fits its shared memory).  CTA `rank` owns the
 // positions [rank * S, rank * S + S); each of its 256 threads owns four consecutive ones and
 // keeps their float64 diagonal entries of H^-1 and Q in registers for the whole block.  The
@@ -130,14 +141,14 @@ __device__ __forceinline__ void land_offers(uint64_t (&bar_step)[2], int first, 
 // step order -- goes out at the end of the block, for a dense block as the packed operands themselves.
 // (Clocks per step at 3072 positions: 5200 with the comparisons one after the other and the pending
 // entries fetched after the pick; 3700 with a cluster barrier and u, z stored step by step; 2800 to
-// 3300 now.)
+// 3300 now, on twice the CTAs and for 64 steps with as many clocks for the pending terms.)
 //
 // The scaled pivot columns of W (c_s) do not feed the selection; they are solved for at the end
-// of the block by forward substitution with the 32 x 32 triangle T[m][s] = u_s[p_m].
+// of the block by forward substitution with the triangle T[m][s] = u_s[p_m].
 // Finally the per-position vectors are compacted (stable) across the cluster.
 template <bool MULTI>
 __global__ void __launch_bounds__(STEP_THREADS, 1)
-k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int G, int r, int rp,
+k_lazy_steps(int n0, int S, int Sp, int cap, int t0, int nsteps, int compact, int d, int G, int r, int rp,
              const float* __restrict__ A, const float* __restrict__ Q, const float* __restrict__ Wt,
              const double* __restrict__ dA_in, const double* __restrict__ dQ_in,
              const int* __restrict__ idx_in, double* __restrict__ dA_out,
@@ -155,8 +166,8 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     constexpr int NW = STEP_THREADS / 32;
 
     extern __shared__ float4 dyn_smem4[];
-    float* sU = reinterpret_cast<float*>(dyn_smem4);       // [BMAX][Sp]
-    float* sZ = sU + (size_t)BMAX * Sp;                    // [BMAX][Sp]
+    float* sU = reinterpret_cast<float*>(dyn_smem4);       // [cap][Sp]
+    float* sZ = sU + (size_t)cap * Sp;                     // [cap][Sp]
     double (*sTd)[BMAX + 4] = reinterpret_cast<double (*)[BMAX + 4]>(dyn_smem4);   // T in float64, after the last step
     __shared__ Bid s_warp[2][NW];                          // the warps' offers, by step parity
     __shared__ Bid s_cta[2][CLUSTER_MAX];                  // the CTAs' offers, and the pending entries
@@ -178,15 +189,15 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     double da[4], dq[4];
     int org[4];
     bool alive[4];
-    // what a step brings to a CTA
-    [[maybe_unused]] const uint32_t step_bytes = (uint32_t)(CS * (sizeof(Bid) + BMAX * sizeof(float2)));
+    // what step m brings to a CTA: offers and the pending entries, in groups of 32
+    auto step_bytes = [&](int m) { return (uint32_t)(CS * (sizeof(Bid) + (m > GS ? BMAX : GS) * sizeof(float2))); };
     if (MULTI) {
         if (tid == 0) {
             abort_flag = 0;
             tc::mbar_init(tc::smem_u32(&bar_step[0]), 1);
             tc::mbar_init(tc::smem_u32(&bar_step[1]), 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), step_bytes);
+            tc::mbar_expect_tx(tc::smem_u32(&bar_step[0]), step_bytes(0));
         }
         cluster.sync();
     }
@@ -264,20 +275,27 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
             const Bid own = s_warp[par][best_bid(s_warp[par], NW, lane)];
             if (warp < CS) {
                 const int pl = own.pos >= 0 ? own.pos - rank * S : 0;
-                float2 uz = make_float2(0.f, 0.f);
-                if (lane < m) uz = make_float2(sU[(size_t)lane * Sp + pl], sZ[(size_t)lane * Sp + pl]);
+                float2 uz[BMAX / GS];
+#pragma unroll
+                for (int g = 0; g < BMAX / GS; ++g) {
+                    const int s = g * GS + lane;
+                    uz[g] = s < m ? make_float2(sU[(size_t)s * Sp + pl], sZ[(size_t)s * Sp + pl]) : make_float2(0.f, 0.f);
+                }
                 const uint32_t bar = to_bar + 8u * par;
                 if (lane == 0) {
                     const uint32_t to = to_bid + (uint32_t)(par * CLUSTER_MAX * sizeof(Bid));
                     tc::send2(to, own.a, own.q, bar);
                     tc::send2(to + 16u, ((long long)own.pos << 32) | (unsigned)own.org, (long long)own.key, bar);
                 }
-                tc::send1(to_pend + (uint32_t)(par * CLUSTER_MAX * BMAX * sizeof(float2)),
-                          ((long long)__float_as_uint(uz.y) << 32) | __float_as_uint(uz.x), bar);
+#pragma unroll
+                for (int g = 0; g < BMAX / GS; ++g)
+                    if (g == 0 || m > g * GS)
+                        tc::send1(to_pend + (uint32_t)((par * CLUSTER_MAX * BMAX + g * GS) * sizeof(float2)),
+                                  ((long long)__float_as_uint(uz[g].y) << 32) | __float_as_uint(uz[g].x), bar);
             }
             // (past a give-up the barrier may still be in an older phase)
             if (tid == 0 && m + 1 < nsteps && gave_up == nsteps)
-                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]), step_bytes);
+                tc::mbar_expect_tx(tc::smem_u32(&bar_step[par ^ 1]), step_bytes(m + 1));
             if (!tc::mbar_wait(tc::smem_u32(&bar_step[par]), (uint32_t)(m >> 1) & 1u, &abort_flag)) {
                 gave_up = min(gave_up, m);         // (the waits that follow give up at once)
                 abort_flag = 1;
@@ -303,7 +321,8 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         const double rs = rsqrt(h), half = 0.5 * gq * rs * rs;
         const float *pu = sU + p, *pz = sZ + p;    // pending entries of one CTA: in its own slice
         if (warp == NW - 1) {                      // (the last warp: the others may own more positions)
-            sT[m][lane] = lane < m ? (MULTI ? pend[lane].x : pu[(size_t)lane * Sp]) : 0.f;
+#pragma unroll
+            for (int s = lane; s < BMAX; s += 32) sT[m][s] = s < m ? (MULTI ? pend[s].x : pu[(size_t)s * Sp]) : 0.f;
             // this CTA's part of the pivot column of W, which the end of the block reads, on its way to L2
             for (int i = w_first + 32 * lane; i < w_end; i += 1024)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(Wl + (size_t)p * rp + i));
@@ -363,8 +382,8 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     // ---- what the update kernels read: u, z as they are for a compaction block, packed for a dense one
     const int n_own = max(0, min(S, n0 - rank * S));
     if (compact) {
-        float* Ul = U + (size_t)l * BMAX * d + rank * S;
-        float* Zl = Z + (size_t)l * BMAX * d + rank * S;
+        float* Ul = U + (size_t)l * GS * d + rank * S;
+        float* Zl = Z + (size_t)l * GS * d + rank * S;
         for (int s = warp; s < nsteps; s += NW)
             for (int k = lane; k < n_own; k += 32) {
                 Ul[(size_t)s * d + k] = sU[(size_t)s * Sp + k];
@@ -374,22 +393,24 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
         // two positions per warp, two steps per lane: 64-byte pieces (a position per thread with 16-byte stores
         // touches 32 lines an instruction and takes 1.7 times as long); the last CTA zeroes the rows up to the
         // next whole tile
-        const size_t arr = (size_t)rows_tot * 2 * BMAX;
-        __nv_bfloat16* Pl = P + (size_t)l * kPackArrays * arr;
-        const int sp = 2 * (lane & 15);
+        const size_t arr = (size_t)rows_tot * 2 * GS;
         const int end = rank == CS - 1 ? (n0 + kPackTile - 1) / kPackTile * kPackTile - rank * S : n_own;
+        for (int g = 0; g * GS < nsteps; ++g) {
+            __nv_bfloat16* Pl = P + ((size_t)l * kPackGroups + g) * kPackArrays * arr;
+            const int sl = 2 * (lane & 15), sp = g * GS + sl;
 #pragma unroll 2
-        for (int k = 2 * warp + (lane >> 4); k < end; k += 2 * NW) {
-            const bool i0 = k < n_own && sp < nsteps, i1 = k < n_own && sp + 1 < nsteps;
-            __nv_bfloat162 u[3], z[3];
-            split_bf16x3(i0 ? sU[(size_t)sp * Sp + k] : 0.f, i1 ? sU[(size_t)(sp + 1) * Sp + k] : 0.f, u);
-            split_bf16x3(i0 ? sZ[(size_t)sp * Sp + k] : 0.f, i1 ? sZ[(size_t)(sp + 1) * Sp + k] : 0.f, z);
-            __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(Pl + (size_t)(rank * S + k) * 2 * BMAX + sp);
-            o[0] = u[0];       o[BMAX / 2] = u[1];
-            o += arr / 2;
-            o[0] = u[2];       o[BMAX / 2] = z[2];
-            o += arr / 2;
-            o[0] = z[0];       o[BMAX / 2] = z[1];
+            for (int k = 2 * warp + (lane >> 4); k < end; k += 2 * NW) {
+                const bool i0 = k < n_own && sp < nsteps, i1 = k < n_own && sp + 1 < nsteps;
+                __nv_bfloat162 u[3], z[3];
+                split_bf16x3(i0 ? sU[(size_t)sp * Sp + k] : 0.f, i1 ? sU[(size_t)(sp + 1) * Sp + k] : 0.f, u);
+                split_bf16x3(i0 ? sZ[(size_t)sp * Sp + k] : 0.f, i1 ? sZ[(size_t)(sp + 1) * Sp + k] : 0.f, z);
+                __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(Pl + (size_t)(rank * S + k) * 2 * GS + sl);
+                o[0] = u[0];       o[GS / 2] = u[1];
+                o += arr / 2;
+                o[0] = u[2];       o[GS / 2] = z[2];
+                o += arr / 2;
+                o[0] = z[0];       o[GS / 2] = z[1];
+            }
         }
     }
     if (rank == 0) {
@@ -407,19 +428,21 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
     __syncthreads();                           // sU, sZ are done with
 
     // ---- c_m = (W[:,p_m] - sum_{s<m} c_s T[m][s]) / sqrt(h_m), forward substitution for every row index i
-    //      of W (each CTA a slice of them), in 8 x 8 blocks on the float64 tensor-core instruction: the four
-    //      diagonal blocks of the 32 x 32 triangle are inverted first, a lane for a column; then a warp takes
-    //      eight row indices: C_b = D_b^-1 W_b, W_q -= T_qb C_b for q > b.  C_b is rounded to fp32, as it is
-    //      stored and applied, before it is used.  (One thread per row index ran 500 FMAs and as many loads
-    //      of straight-line code from a cold instruction cache: 21000 to 36000 clocks a block, a fifth of it.)
+    //      of W (each CTA a slice of them), in 8 x 8 blocks on the float64 tensor-core instruction: the
+    //      diagonal blocks of the triangle are inverted first, a lane for a column; then a warp takes
+    //      eight row indices and 32 steps at a time: C_b = D_b^-1 W_b, W_q -= T_qb C_b for q > b, the second 32
+    //      steps behind the first.  C_b is rounded to fp32, as it is stored and applied, before it is used.
+    //      (One thread per row index ran 500 FMAs and as many loads of straight-line code from a cold
+    //      instruction cache: 21000 to 36000 clocks a block of 32 steps, a fifth of it.)
     //      It reads this CTA's own shared memory only and runs last, when the per-position state is dead.
     auto solve_c = [&]() {
-        double (*sD)[9] = reinterpret_cast<double (*)[9]>(sTd + BMAX);     // [32][8]: D_b^-1, row m, column m % 8
-        for (int e = tid; e < BMAX * BMAX; e += STEP_THREADS)
+        double (*sD)[9] = reinterpret_cast<double (*)[9]>(sTd + BMAX);     // [BMAX][8]: D_b^-1, row m, column m % 8
+        const int groups = (nsteps + GS - 1) / GS;
+        for (int e = tid; e < groups * GS * BMAX; e += STEP_THREADS)
             sTd[e / BMAX][e % BMAX] = e / BMAX < nsteps ? (double)sT[e / BMAX][e % BMAX] : 0.0;
         __syncthreads();
-        if (warp == 0) {
-            const int b8 = lane & 24, j = lane & 7;
+        if (warp < groups) {
+            const int b8 = warp * GS + (lane & 24), j = lane & 7;
             double x[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -431,65 +454,86 @@ k_lazy_steps(int n0, int S, int Sp, int t0, int nsteps, int compact, int d, int 
             }
         }
         __syncthreads();
-        float* Cl = C + (size_t)l * BMAX * rp;
-        const size_t arr = (size_t)rows_tot * 2 * BMAX;
-        __nv_bfloat16* Pc = P + (size_t)l * kPackArrays * arr + (size_t)rows_pad * 2 * BMAX;
+        float* Cl = C + (size_t)l * GS * rp;
+        const size_t arr = (size_t)rows_tot * 2 * GS;
         const int gr = lane >> 2, qd = lane & 3;         // accumulator: row gr, columns 2 qd, 2 qd + 1
         constexpr int NT = 3;                            // tiles of eight row indices side by side
+        // a block as the second operand: element (k = 4 kk + qd, n = gr) of it
+        auto operand = [&](double v0, double v1, int kk) {
+            const int from = (4 * kk + qd) * 4 + (gr >> 1);
+            const double x = __shfl_sync(0xffffffffu, v0, from), y = __shfl_sync(0xffffffffu, v1, from);
+            return gr & 1 ? y : x;
+        };
         for (int i0 = w_first + 8 * warp; i0 < w_end; i0 += 8 * NW * NT) {
-            double acc[NT][4][2];
+            float done[NT][4][2] = {};                   // C of the first group
+#pragma unroll 1
+            for (int g = 0; g < groups; ++g) {
+                const int m0 = g * GS;
+                __nv_bfloat16* Pc = P + ((size_t)l * kPackGroups + g) * kPackArrays * arr + (size_t)rows_pad * 2 * GS;
+                double acc[NT][4][2];
 #pragma unroll
-            for (int t = 0; t < NT; ++t)
+                for (int t = 0; t < NT; ++t)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        // (rows are zero from r to rp; what lies past the slice or the last step is not used)
+                        const int i = min(i0 + 8 * NW * t + 2 * qd, rp - 2), m = m0 + 8 * b + gr;
+                        const float2 w = *reinterpret_cast<const float2*>(Wl + (size_t)s_pm[min(m, nsteps - 1)] * rp + i);
+                        acc[t][b][0] = m < nsteps ? (double)w.x : 0.0;
+                        acc[t][b][1] = m < nsteps ? (double)w.y : 0.0;
+                    }
+                if (g)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk) {
+                            double tq[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) tq[q] = -sTd[m0 + 8 * q + gr][8 * b + 4 * kk + qd];
+#pragma unroll
+                            for (int t = 0; t < NT; ++t) {
+                                const double x = operand((double)done[t][b][0], (double)done[t][b][1], kk);
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) dmma884(acc[t][q], tq[q], x);
+                            }
+                        }
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    // (rows are zero from r to rp; what lies past the slice or the last step is not used)
-                    const int i = min(i0 + 8 * NW * t + 2 * qd, rp - 2), m = 8 * b + gr;
-                    const float2 w = *reinterpret_cast<const float2*>(Wl + (size_t)s_pm[min(m, nsteps - 1)] * rp + i);
-                    acc[t][b][0] = m < nsteps ? (double)w.x : 0.0;
-                    acc[t][b][1] = m < nsteps ? (double)w.y : 0.0;
-                }
-            // a block as the second operand: element (k = 4 kk + qd, n = gr) of it
-            auto operand = [&](double v0, double v1, int kk) {
-                const int from = (4 * kk + qd) * 4 + (gr >> 1);
-                const double x = __shfl_sync(0xffffffffu, v0, from), y = __shfl_sync(0xffffffffu, v1, from);
-                return gr & 1 ? y : x;
-            };
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const double d0 = sD[8 * b + gr][qd], d1 = sD[8 * b + gr][4 + qd];
-                double tq[3][2];
-#pragma unroll
-                for (int q = b + 1; q < 4; ++q) {
-                    tq[q - 1][0] = -sTd[8 * q + gr][8 * b + qd];
-                    tq[q - 1][1] = -sTd[8 * q + gr][8 * b + 4 + qd];
-                }
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    double c[2] = {0.0, 0.0};
-                    dmma884(c, d0, operand(acc[t][b][0], acc[t][b][1], 0));
-                    dmma884(c, d1, operand(acc[t][b][0], acc[t][b][1], 1));
-                    const float c0 = (float)c[0], c1 = (float)c[1];
-                    const int i = i0 + 8 * NW * t + 2 * qd, m = 8 * b + gr;
-                    if (i < w_end) {                     // (rp and the slices are even)
-                        if (compact) {
-                            if (m < nsteps) *reinterpret_cast<float2*>(Cl + (size_t)m * rp + i) = make_float2(c0, c1);
-                        } else {
-                            // rows of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest
-                            // was zeroed before the first block)
-                            __nv_bfloat162 x[3];
-                            split_bf16x3(c0, c1, x);
-                            __nv_bfloat16* o = Pc + (size_t)i * 2 * BMAX + m;
-                            o[0] = __low2bfloat16(x[0]); o[BMAX] = __low2bfloat16(x[1]); o[arr] = __low2bfloat16(x[2]);
-                            o += 2 * BMAX;
-                            o[0] = __high2bfloat16(x[0]); o[BMAX] = __high2bfloat16(x[1]); o[arr] = __high2bfloat16(x[2]);
-                        }
-                    }
-                    if (b == 3) continue;
-                    const double b0 = operand((double)c0, (double)c1, 0), b1 = operand((double)c0, (double)c1, 1);
+                    const double d0 = sD[m0 + 8 * b + gr][qd], d1 = sD[m0 + 8 * b + gr][4 + qd];
+                    double tq[3][2];
 #pragma unroll
                     for (int q = b + 1; q < 4; ++q) {
-                        dmma884(acc[t][q], tq[q - 1][0], b0);
-                        dmma884(acc[t][q], tq[q - 1][1], b1);
+                        tq[q - 1][0] = -sTd[m0 + 8 * q + gr][m0 + 8 * b + qd];
+                        tq[q - 1][1] = -sTd[m0 + 8 * q + gr][m0 + 8 * b + 4 + qd];
+                    }
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) {
+                        double c[2] = {0.0, 0.0};
+                        dmma884(c, d0, operand(acc[t][b][0], acc[t][b][1], 0));
+                        dmma884(c, d1, operand(acc[t][b][0], acc[t][b][1], 1));
+                        const float c0 = (float)c[0], c1 = (float)c[1];
+                        done[t][b][0] = c0; done[t][b][1] = c1;
+                        const int i = i0 + 8 * NW * t + 2 * qd, sl = 8 * b + gr;
+                        if (i < w_end) {                     // (rp and the slices are even)
+                            if (compact) {
+                                if (sl < nsteps) *reinterpret_cast<float2*>(Cl + (size_t)sl * rp + i) = make_float2(c0, c1);
+                            } else {
+                                // rows of the packed operands behind the positions: [C1 | C2], [C3 | 0] (the rest
+                                // was zeroed before the first block)
+                                __nv_bfloat162 x[3];
+                                split_bf16x3(c0, c1, x);
+                                __nv_bfloat16* o = Pc + (size_t)i * 2 * GS + sl;
+                                o[0] = __low2bfloat16(x[0]); o[GS] = __low2bfloat16(x[1]); o[arr] = __low2bfloat16(x[2]);
+                                o += 2 * GS;
+                                o[0] = __high2bfloat16(x[0]); o[GS] = __high2bfloat16(x[1]); o[arr] = __high2bfloat16(x[2]);
+                            }
+                        }
+                        if (b == 3) continue;
+                        const double b0 = operand((double)c0, (double)c1, 0), b1 = operand((double)c0, (double)c1, 1);
+#pragma unroll
+                        for (int q = b + 1; q < 4; ++q) {
+                            dmma884(acc[t][q], tq[q - 1][0], b0);
+                            dmma884(acc[t][q], tq[q - 1][1], b1);
+                        }
                     }
                 }
             }
@@ -585,7 +629,7 @@ __global__ void __launch_bounds__(128, 5) k_lazy_update_aq(int n_new, int m, int
                                                         const int* __restrict__ src,
                                                         const float* __restrict__ U,
                                                         const float* __restrict__ Z) {
-    __shared__ __align__(16) float stage[4][BMAX][64];   // pending slabs of the tile's rows and columns
+    __shared__ __align__(16) float stage[4][GS][64];   // pending slabs of the tile's rows and columns
     float (*sUr)[64] = stage[0];
     float (*sZr)[64] = stage[1];
     float (*sUc)[64] = stage[2];
@@ -608,8 +652,8 @@ __global__ void __launch_bounds__(128, 5) k_lazy_update_aq(int n_new, int m, int
     // The pending slabs of the tile's rows and columns go straight to shared memory with
     // asynchronous 4-byte copies (zero-filled past the last live row), so that all of them and the
     // gathered old entries below are in flight together.
-    const float* Ul = U + (size_t)l * BMAX * d;
-    const float* Zl = Z + (size_t)l * BMAX * d;
+    const float* Ul = U + (size_t)l * GS * d;
+    const float* Zl = Z + (size_t)l * GS * d;
     {
         const int c = tid & 63;
         const int idx = (tid < 64) ? srow[c] : scol[c];
@@ -735,16 +779,16 @@ __global__ void __launch_bounds__(256, 3) k_lazy_update_w(int n_new, int m, int 
                                                        const int* __restrict__ src,
                                                        const float* __restrict__ U,
                                                        const float* __restrict__ C) {
-    __shared__ float4 sC[BMAX][64];       // C[s][col0 .. col0+255]
-    __shared__ __align__(16) float sUr[BMAX][64];       // U[s][src[row]]
+    __shared__ float4 sC[GS][64];       // C[s][col0 .. col0+255]
+    __shared__ __align__(16) float sUr[GS][64];       // U[s][src[row]]
     __shared__ int srow[64];
     const int l = blockIdx.z;
     const int i0 = blockIdx.x * 64, c0 = blockIdx.y * 256;
     const int tid = threadIdx.x, tx = tid & 63, ty = tid >> 6;      // ty: rows 16 ty .. 16 ty + 15
     if (tid < 64) srow[tid] = (i0 + tid < n_new) ? src[(size_t)l * d + i0 + tid] : -1;
     __syncthreads();
-    const float* Ul = U + (size_t)l * BMAX * d;
-    const float* Cl = C + (size_t)l * BMAX * rp;
+    const float* Ul = U + (size_t)l * GS * d;
+    const float* Cl = C + (size_t)l * GS * rp;
     // asynchronous copies (zero-filled where there is nothing to read), in flight together with
     // the gathered rows below
     for (int e = tid; e < m * 64; e += 256) {
@@ -976,9 +1020,9 @@ LazyWs carve_lazy(void* ws, int L, int r, int d, int n_levels) {
     for (int b = 0; b < 2; ++b) w.idx[b] = c.take<int>((size_t)L * ld);
     w.src = c.take<int>((size_t)L * ld);
     w.pos_of = c.take<int>((size_t)L * ld);
-    w.U = c.take<float>((size_t)L * BMAX * ld);
-    w.Z = c.take<float>((size_t)L * BMAX * ld);
-    w.C = c.take<float>((size_t)L * BMAX * w.rp);
+    w.U = c.take<float>((size_t)L * GS * ld);
+    w.Z = c.take<float>((size_t)L * GS * ld);
+    w.C = c.take<float>((size_t)L * GS * w.rp);
     w.P = c.take<float>(lazy_tc_pack_floats(L, ld, w.rp));
     w.sched = c.take<int>(2);
     w.state = c.take<LazyState>((size_t)L);
@@ -999,8 +1043,13 @@ LazyWs carve_lazy(void* ws, int L, int r, int d, int n_levels) {
 // Pitch of the pending vectors in the steps kernel: four more than a multiple of 32, so that the entries at
 // one position (one per pending step) lie in eight different banks instead of one.
 static int steps_pitch(int S) { return round_up_int(S, 32) + 4; }
-static int steps_smem(int S) {
-    const int b = 2 * BMAX * steps_pitch(S) * (int)sizeof(float), t = BMAX * (BMAX + 4 + 9) * (int)sizeof(double);
+// Steps that may be pending on slices of S positions, whole groups of 16 (the K of an MMA of the update).
+static int steps_cap(int S) {
+    const int fit = STEPS_SMEM / (2 * steps_pitch(S) * (int)sizeof(float));
+    return fit >= BMAX ? BMAX : fit / 16 * 16;
+}
+static int steps_smem(int S, int cap) {
+    const int b = 2 * cap * steps_pitch(S) * (int)sizeof(float), t = BMAX * (BMAX + 4 + 9) * (int)sizeof(double);
     return b > t ? b : t;
 }
 
@@ -1056,9 +1105,9 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     if (s != ZIPLM_OK) return s;
 
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_steps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          steps_smem(SLICE_MAX)));
+                                          STEPS_SMEM));
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_steps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          steps_smem(SLICE_MAX)));
+                                          STEPS_SMEM));
     int cur = 0;
     auto snapshot = [&](int n, int slot) -> ziplm_status {
         PhaseScope ps(PH_SNAPSHOT, st);
@@ -1099,31 +1148,38 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     ZIPLM_CHECK_CUDA(cudaMemsetAsync(w.P, 0, sizeof(float) * lazy_tc_pack_floats(L, ld, rp), st));
     // The last kEndgame structures go to the float64 endgame unless only a few of them are to be removed
     // (its set-up costs as much as two blocks).
-    const bool endgame = n_min <= kEndgame - 2 * BMAX;
+    const bool endgame = n_min <= kEndgame - 2 * GS;
     while (n > n_min) {
         int stop = (slot < n_levels) ? levels[slot] : n_min;         // next block boundary
         if (endgame && stop < kEndgame) stop = kEndgame;             // ... and where the endgame begins
-        const int nsteps = (n - stop < BMAX) ? (n - stop) : BMAX;
         const int nxt = cur ^ 1;
+        // Up to four CTAs a layer as long as a CTA has more than 256 positions: the pending terms of a step are
+        // bound by shared-memory bandwidth, 24 clocks per pending step and 384 positions, which outweighs
+        // the exchange.  Eight where a slice of BMAX pending steps would not fit shared memory: four with
+        // 32 pending steps up to 3072 positions took 27.5 ms where eight take 25.0 (12 x 3072, all work).
+        int cs = 1;
+        while (cs < CLUSTER_MAX && (npos + cs - 1) / cs > (cs < 4 ? 256 : SLICE_WIDE)) cs *= 2;
+        const int S = round_up_int((npos + cs - 1) / cs, 4), cap = steps_cap(S);
         // Squeezing removed positions out makes the update kernels gather through a map; leaving
         // them in place keeps their reads and writes dense at the price of dead rows and columns.
-        // They are squeezed out once they make up kDeadMax positions or a sixteenth of all.
+        // They are squeezed out, by a block of at most 32 steps, once they make up kDeadMax positions or an
+        // eighth of all.
+        int nsteps = (n - stop < GS) ? (n - stop) : GS;
         const int dead_after = npos - (n - nsteps);
         const bool last = endgame && n - nsteps == kEndgame;
         const int compact = (every_block || last || dead_after >= kDeadMax ||
                              dead_after * kDeadFraction >= npos || npos <= 1) ? 1 : 0;
+        if (!compact) {
+            nsteps = (n - stop < cap) ? (n - stop) : cap;
+            // (the block that reaches the endgame squeezes)
+            if (endgame && n - nsteps == kEndgame) nsteps -= GS;
+        }
         {
             PhaseScope ps(PH_LAZY_STEPS, st);
-            // Up to four CTAs as long as a CTA has more than 256 positions: the pending terms of a step are
-            // bound by shared-memory bandwidth, 48 clocks per pending step and 768 positions, which outweighs
-            // the exchange.  More only where a slice would not fit shared memory: they hold whole SMs.
-            int cs = 1;
-            while (cs < CLUSTER_MAX && (npos + cs - 1) / cs > (cs < 4 ? 256 : SLICE_MAX)) cs *= 2;
-            const int S = round_up_int((npos + cs - 1) / cs, 4);
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(L * cs);
             cfg.blockDim = dim3(STEP_THREADS);
-            cfg.dynamicSmemBytes = (size_t)steps_smem(S);
+            cfg.dynamicSmemBytes = (size_t)steps_smem(S, cap);
             cfg.stream = st;
             cudaLaunchAttribute attr[2];
             attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1138,7 +1194,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(
-                &cfg, cs > 1 ? k_lazy_steps<true> : k_lazy_steps<false>, npos, S, steps_pitch(S), t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
+                &cfg, cs > 1 ? k_lazy_steps<true> : k_lazy_steps<false>, npos, S, steps_pitch(S), cap, t, nsteps, compact, ld, G, r, rp, (const float*)w.A[cur],
                 (const float*)w.Q[cur], (const float*)w.Wt[cur], (const double*)w.dA[cur],
                 (const double*)w.dQ[cur], (const int*)w.idx[cur], w.dA[nxt], w.dQ[nxt], w.idx[nxt],
                 w.src, w.U, w.Z, w.C, reinterpret_cast<__nv_bfloat16*>(w.P), lazy_tc_rows_pad(ld),
@@ -1158,7 +1214,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         if (!compact) {
             // every position stays in place: dense tiles, tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);
-            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, n_new, ld, rp,
+            s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, (nsteps + GS - 1) / GS, n_new, ld, rp,
                                       w.A[nxt], w.Q[nxt], w.Wt[nxt], w.sched, layer_status, 0u, st);
             if (s != ZIPLM_OK) return s;
         } else if (n_new > 1) {

@@ -1,4 +1,4 @@
-// Rank-32 update of H^-1, of the Gram matrix Q = W^T W and of W^T itself (delayed Eq. 4 / Eq. 3)
+// Rank-32 or rank-64 update of H^-1, of the Gram matrix Q = W^T W and of W^T itself (delayed Eq. 4 / Eq. 3)
 // for the blocks that leave the removed positions in place, on the 5th-generation tensor cores,
 // as one persistent kernel:
 //
@@ -15,6 +15,13 @@
 // the earlier ones left, so |x - x1 - x2 - x3| <= 2^-27 |x|).  Products of two bfloat16 values are
 // exact in the fp32 accumulator, and the six partial products x_a y_b with a + b <= 4 are kept
 // (the others are below 2^-26 of the product), so a product is as good as an fp32 one.
+//
+// Two groups of 32 steps: the operands of a group at a time fill their shared memory, each group has an
+// accumulator of its own and the two are joined in fp32 (one chain of both would truncate more).  12 x 3072 with two
+// groups 545 us on two thirds of the SMs, where one group takes 365: the L2 moves the operands besides the matrices (7
+// TB/s in all), and the MMAs, at 128 bytes a clock, share the shared memory with the epilogue.  Rows of both groups kept
+// in shared memory beside a ring of narrower slices: the same; old entries read into registers from the other side of
+// the diagonal, with operands of both groups in shared memory: 740 us (loads queue behind the stores).
 //
 // The update kernel runs one CTA on each of two thirds of the SMs.  Work is cut into tiles of
 // 128 x 128 entries on or below the diagonal; runs of consecutive tiles of one row strip
@@ -57,7 +64,7 @@ constexpr int BOX_BYTES = BOX_ROWS * 128;    // 8 KiB
 constexpr int ARR_BYTES = 2 * BOX_BYTES;     // one packed array, 128 positions
 constexpr int ROWS_BYTES = NARR * ARR_BYTES; // 48 KiB
 constexpr int COLS_BYTES = NARR * ARR_BYTES; // 48 KiB
-constexpr int ACC_STAGES = 2;
+constexpr int ACC_STAGES = 2;                // accumulator regions: the groups of the tiles in turn
 constexpr int N_EPI = 16;                    // epilogue warps: 4 lane quarters x 2 matrices x 2 column halves
 constexpr int SUBS = 4;                      // slices of 16 columns per warp and tile
 constexpr int RING = 3;                      // slices per epilogue warp
@@ -74,6 +81,7 @@ enum { TILE_STOP = 1, TILE_NEW_ROWS = 2, TILE_W = 4 };
 // of segments (over all layers) of the k longest strips.
 struct AqSched {
     int n_strips, seg, n_segments, L;
+    int groups;               // groups of 32 pending steps
     int n_wt;                 // tiles of 128 columns of W^T that follow the tiles of a row strip
     int rows_pad;             // first row of the packed C in P
     int prefix[MAX_STRIPS + 1];
@@ -134,7 +142,7 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
     if (warp == 0) {
         // ---------------- scheduler and TMA producer ----------------
         int t = 0;                       // tiles published so far by this CTA
-        int issued = 0;                  // tiles whose operand copies were issued
+        int issued = 0;                  // groups whose operand copies were issued
         int s = 0;
         if (lane == 0) s = atomicAdd(counter, 1);
         s = __shfl_sync(0xffffffffu, s, 0);
@@ -167,27 +175,33 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_tile_full[slot]));
-                // the operand tiles are free once the MMAs of the previous tile have completed
-                if (t > 0)
-                    failed = !__all_sync(0xffffffffu,
-                                         mbar_wait(smem_u32(&bar_acc_full[(t - 1) & 1]),
-                                                   (uint32_t)(((t - 1) >> 1) & 1), abortp));
-                if (failed) break;
-                if (lane == 0) {
-                    const uint32_t full = smem_u32(&bar_ops_full);
-                    mbar_expect_tx(full, (uint32_t)((J == Jb ? ROWS_BYTES : 0) + COLS_BYTES));
+                for (int k2 = 0; k2 < sch.groups; ++k2) {
+                    // The operand tiles are free once the MMAs of the previous group have completed.  The rows stay
+                    // for the next tile of the segment: the order of two groups alternates from tile to tile.
+                    if (issued > 0)
+                        failed = !__all_sync(0xffffffffu,
+                                             mbar_wait(smem_u32(&bar_acc_full[(issued - 1) & 1]),
+                                                       (uint32_t)(((issued - 1) >> 1) & 1), abortp));
+                    if (failed) break;
+                    if (lane == 0) {
+                        const uint32_t full = smem_u32(&bar_ops_full);
+                        const int g = sch.groups > 1 ? k2 ^ (t & 1) : 0;
+                        const bool rows = J == Jb || k2 > 0;
+                        mbar_expect_tx(full, (uint32_t)((rows ? ROWS_BYTES : 0) + COLS_BYTES));
 #pragma unroll
-                    for (int a = 0; a < NARR; ++a)
+                        for (int a = 0; a < NARR; ++a)
 #pragma unroll
-                        for (int b = 0; b < 2; ++b) {
-                            if (J == Jb)
-                                tma_load_4d(rows_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
-                                            i0 + b * BOX_ROWS, a, l);
-                            tma_load_4d(cols_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
-                                        j0 + b * BOX_ROWS, a, l);
-                        }
+                            for (int b = 0; b < 2; ++b) {
+                                if (rows)
+                                    tma_load_4d(rows_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
+                                                i0 + b * BOX_ROWS, g * NARR + a, l);
+                                tma_load_4d(cols_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
+                                            j0 + b * BOX_ROWS, g * NARR + a, l);
+                            }
+                    }
+                    ++issued;
                 }
-                issued = t + 1;
+                if (failed) break;
             }
             s = __shfl_sync(0xffffffffu, s_next, 0);
         }
@@ -221,38 +235,42 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 c[p] = make_desc(cols_smem + (part_off[p] & ~127u)) + (uint64_t)((part_off[p] & 127u) >> 4);
             }
             enum { U1 = 0, U2 = 1, U3 = 2, Z1 = 3, Z2 = 4, Z3 = 5 };
+            int unit = 0;                // groups of 32 steps so far
             for (int t = 0;; ++t) {
                 const int slot = t & (DESC_RING - 1);
                 if (!mbar_wait(smem_u32(&bar_tile_full[slot]), (uint32_t)((t >> 2) & 1), abortp)) { failed = true; break; }
                 const int flags = *reinterpret_cast<volatile int*>(&slots[slot].flags);
                 mbar_arrive(smem_u32(&bar_tile_empty[slot]));
                 if (flags & TILE_STOP) break;
-                const int st = t & 1;
-                if (!mbar_wait(smem_u32(&bar_ops_full), (uint32_t)(t & 1), abortp)) { failed = true; break; }
-                if (t >= ACC_STAGES &&
-                    !mbar_wait(smem_u32(&bar_acc_empty[st]), (uint32_t)(((t >> 1) - 1) & 1), abortp)) {
-                    failed = true;
-                    break;
+                for (int g = 0; g < sch.groups; ++g, ++unit) {
+                    const int st = unit & 1;
+                    if (!mbar_wait(smem_u32(&bar_ops_full), (uint32_t)(unit & 1), abortp)) { failed = true; break; }
+                    if (unit >= ACC_STAGES &&
+                        !mbar_wait(smem_u32(&bar_acc_empty[st]), (uint32_t)(((unit >> 1) - 1) & 1), abortp)) {
+                        failed = true;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t t_a = tmem_base + (uint32_t)(st * 2 * CN), t_q = t_a + (uint32_t)CN;
+                    // one partial product x_a y_b over the 32 steps: two MMAs of K = 16 (32 bytes each)
+                    auto prod = [&](uint32_t acc, int pr, int pc2, bool first) {
+                        umma_bf16(acc, r[pr], c[pc2], idesc, first ? 0u : 1u);
+                        umma_bf16(acc, r[pr] + 2u, c[pc2] + 2u, idesc, 1u);
+                    };
+                    // H^-1: U U^T; smallest terms first
+                    prod(t_a, U1, U3, true);  prod(t_a, U3, U1, false); prod(t_a, U2, U2, false);
+                    prod(t_a, U1, U2, false); prod(t_a, U2, U1, false); prod(t_a, U1, U1, false);
+                    // Q: Z U^T + U Z^T (a tile of W^T has no second matrix: its column operand is C
+                    // in the place of U, and the products above are the whole update U^T C)
+                    if (!(flags & TILE_W)) {
+                        prod(t_q, Z1, U3, true);  prod(t_q, Z3, U1, false); prod(t_q, Z2, U2, false);
+                        prod(t_q, U1, Z3, false); prod(t_q, U3, Z1, false); prod(t_q, U2, Z2, false);
+                        prod(t_q, Z1, U2, false); prod(t_q, Z2, U1, false); prod(t_q, U1, Z2, false);
+                        prod(t_q, U2, Z1, false); prod(t_q, Z1, U1, false); prod(t_q, U1, Z1, false);
+                    }
+                    umma_commit(smem_u32(&bar_acc_full[st]));
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t t_a = tmem_base + (uint32_t)(st * 2 * CN), t_q = t_a + (uint32_t)CN;
-                // one partial product x_a y_b over the 32 steps: two MMAs of K = 16 (32 bytes each)
-                auto prod = [&](uint32_t acc, int pr, int pc2, bool first) {
-                    umma_bf16(acc, r[pr], c[pc2], idesc, first ? 0u : 1u);
-                    umma_bf16(acc, r[pr] + 2u, c[pc2] + 2u, idesc, 1u);
-                };
-                // H^-1: U U^T; smallest terms first
-                prod(t_a, U1, U3, true);  prod(t_a, U3, U1, false); prod(t_a, U2, U2, false);
-                prod(t_a, U1, U2, false); prod(t_a, U2, U1, false); prod(t_a, U1, U1, false);
-                // Q: Z U^T + U Z^T (a tile of W^T has no second matrix: its column operand is C
-                // in the place of U, and the products above are the whole update U^T C)
-                if (!(flags & TILE_W)) {
-                    prod(t_q, Z1, U3, true);  prod(t_q, Z3, U1, false); prod(t_q, Z2, U2, false);
-                    prod(t_q, U1, Z3, false); prod(t_q, U3, Z1, false); prod(t_q, U2, Z2, false);
-                    prod(t_q, Z1, U2, false); prod(t_q, Z2, U1, false); prod(t_q, U1, Z2, false);
-                    prod(t_q, U2, Z1, false); prod(t_q, Z1, U1, false); prod(t_q, U1, Z1, false);
-                }
-                umma_commit(smem_u32(&bar_acc_full[st]));
+                if (failed) break;
             }
             if (failed) abort_flag = 1;
             // whatever was issued has completed before tensor memory is given back
@@ -324,30 +342,52 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
         int cl = nl, ci0 = ni0, cj0 = nj0, cflags = pflags;   // tile being worked on
         copy_next();
         copy_next();
+        int unit = 0;
         for (int t = 0; !(cflags & TILE_STOP) && !failed; ++t) {
-            const int stage = t & 1;
+            for (int g = 0; g < sch.groups && !failed; ++g)
+                if (!mbar_wait(smem_u32(&bar_acc_full[(unit + g) & 1]), (uint32_t)(((unit + g) >> 1) & 1), abortp))
+                    failed = true;
+            failed = __any_sync(0xffffffffu, failed);
+            if (failed) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            float upd[32];
 #pragma unroll 1
             for (int sub = 0; sub < SUBS; ++sub) {
+                if (!(sub & 1)) {
+                    // ---- the update of two slices, summed over the groups (each in an accumulator of its own and
+                    //      joined in fp32 here: a longer chain in tensor memory would truncate more)
+                    // (a tile of W^T has one accumulator, which both matrices' warps read)
+                    const uint32_t from = lane_taddr - ((cflags & TILE_W) ? (uint32_t)(mat * CN) : 0u) + (uint32_t)(16 * sub);
+#pragma unroll
+                    for (int cc = 0; cc < 2; ++cc) {
+                        uint32_t v[16];
+                        tmem_ld16(from + (uint32_t)((unit & 1) * 2 * CN + 16 * cc), v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) upd[16 * cc + e] = __uint_as_float(v[e]);
+                        if (sch.groups > 1) {
+                            tmem_ld16(from + (uint32_t)(((unit + 1) & 1) * 2 * CN + 16 * cc), v);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) upd[16 * cc + e] += __uint_as_float(v[e]);
+                        }
+                    }
+                    if (sub == SUBS - 2) {               // all of the tile's entries are in registers
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0)
+                            for (int g = 0; g < sch.groups; ++g) mbar_arrive(smem_u32(&bar_acc_empty[(unit + g) & 1]));
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) upd[e] = upd[16 + e];
+                }
                 const int c = SUBS * t + sub;
                 // ---- start the copy of the slice two ahead, then wait for slice c
                 if (!copy_next()) { failed = true; break; }
                 if (!mbar_wait(bar0 + 8u * (uint32_t)(c % RING), (uint32_t)((c / RING) & 1), abortp)) failed = true;
-                if (sub == 0 && !failed &&
-                    !mbar_wait(smem_u32(&bar_acc_full[stage]), (uint32_t)((t >> 1) & 1), abortp))
-                    failed = true;
                 failed = __any_sync(0xffffffffu, failed);
                 if (failed) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                uint32_t v[16];
-                // (a tile of W^T has one accumulator, which both matrices' warps read)
-                tmem_ld16(lane_taddr - ((cflags & TILE_W) ? (uint32_t)(mat * CN) : 0u) +
-                              (uint32_t)(stage * 2 * CN + 16 * sub), v);
-                tmem_ld_wait();
-                if (sub == SUBS - 1) {
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[stage]));
-                }
                 float* buf = ring + (size_t)(c % RING) * SLICE_FLOATS;
                 if (cflags & TILE_W) {
                     // ---- tile of W^T: rows = positions, columns = row indices of W; no mirror.
@@ -359,8 +399,8 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                         for (int g = 0; g < 4; ++g) {
                             const int pg = g ^ ((lane >> 1) & 3);
                             const float4 o = b4[pg];
-                            b4[pg] = make_float4(o.x - __uint_as_float(v[4 * g]), o.y - __uint_as_float(v[4 * g + 1]),
-                                                 o.z - __uint_as_float(v[4 * g + 2]), o.w - __uint_as_float(v[4 * g + 3]));
+                            b4[pg] = make_float4(o.x - upd[4 * g], o.y - upd[4 * g + 1],
+                                                 o.z - upd[4 * g + 2], o.w - upd[4 * g + 3]);
                         }
                         __syncwarp();
                         float* Wo = W2 + (size_t)cl * d * rp;
@@ -385,10 +425,10 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 for (int g = 0; g < 4; ++g) {
                     const int pg = g ^ ((lane >> 1) & 3);
                     const float4 o = b4[pg];
-                    rr[4 * g] = o.x - __uint_as_float(v[4 * g]);
-                    rr[4 * g + 1] = o.y - __uint_as_float(v[4 * g + 1]);
-                    rr[4 * g + 2] = o.z - __uint_as_float(v[4 * g + 2]);
-                    rr[4 * g + 3] = o.w - __uint_as_float(v[4 * g + 3]);
+                    rr[4 * g] = o.x - upd[4 * g];
+                    rr[4 * g + 1] = o.y - upd[4 * g + 1];
+                    rr[4 * g + 2] = o.z - upd[4 * g + 2];
+                    rr[4 * g + 3] = o.w - upd[4 * g + 3];
                     b4[pg] = make_float4(rr[4 * g], rr[4 * g + 1], rr[4 * g + 2], rr[4 * g + 3]);
                 }
                 float* Mo = Mout + (size_t)cl * dd;
@@ -430,6 +470,7 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 // before the cursor can replace it (it opens tile t + 2 during slice 1 of tile t + 1)
                 if (sub == SUBS - 1) { cl = nl; ci0 = ni0; cj0 = nj0; cflags = pflags; }
             }
+            unit += sch.groups;
         }
         // every copy this warp started has landed before the CTA leaves (the last RING slices
         // started are the latest phases of their barriers)
@@ -473,14 +514,14 @@ int sm_count() {
 
 }  // namespace
 
-// Tensor map over the packed operands P[L][3][rows_tot][64] (bfloat16): box = 64 rows of one array.
+// Tensor map over the packed operands P[L][2][3][rows_tot][64] (bfloat16): box = 64 rows of one array.
 bool lazy_tc_make_map(CUtensorMap* m, const float* P, int L, int d, int rp) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
     const int rows_pad = lazy_tc_rows_tot(d, rp);
-    cuuint64_t dims[4] = {(cuuint64_t)2 * PK, (cuuint64_t)rows_pad, NARR, (cuuint64_t)L};
+    cuuint64_t dims[4] = {(cuuint64_t)2 * PK, (cuuint64_t)rows_pad, kPackGroups * NARR, (cuuint64_t)L};
     cuuint64_t strides[3] = {(cuuint64_t)128, (cuuint64_t)rows_pad * 128,
-                             (cuuint64_t)NARR * rows_pad * 128};
+                             (cuuint64_t)kPackGroups * NARR * rows_pad * 128};
     cuuint32_t box[4] = {(cuuint32_t)2 * PK, (cuuint32_t)BOX_ROWS, 1, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<float*>(P), dims, strides, box, estr,
@@ -509,7 +550,7 @@ bool lazy_tc_make_matrix_map(CUtensorMap* m, const float* M, int L, int d, int c
 // launch; every launch leaves them zero again.  slot_spin_limit = 0 selects the default poll
 // limit of the producer's wait for a free descriptor slot.
 ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& map_a,
-                                   const CUtensorMap& map_q, const CUtensorMap& map_w, int L, int n_pos,
+                                   const CUtensorMap& map_q, const CUtensorMap& map_w, int L, int groups, int n_pos,
                                    int d, int rp, float* A2, float* Q2, float* W2, int* counter,
                                    int* layer_status, unsigned slot_spin_limit, cudaStream_t st) {
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_lazy_update_aq_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -523,9 +564,11 @@ ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& ma
     // same time with 96 as with 148 CTAs, 12 % more with 74); the others are left to the kernels
     // of other layer groups and batches that run beside it.
     const int ctas = (2 * sms + 2) / 3;
+
     AqSched sch;
     sch.n_strips = rows_used / RM;
     sch.L = L;
+    sch.groups = groups;
     sch.n_wt = (rp + CN - 1) / CN;
     sch.rows_pad = rows_pad;
     const long long tiles = (long long)L * sch.n_strips * ((sch.n_strips + 1) / 2 + sch.n_wt);   // about
