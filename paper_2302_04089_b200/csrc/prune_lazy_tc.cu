@@ -18,30 +18,31 @@
 //
 // Two groups of 32 steps: the operands of a group at a time fill their shared memory, each group has an
 // accumulator of its own and the two are joined in fp32 (one chain of both would truncate more).  12 x 3072 with two
-// groups 545 us on two thirds of the SMs, where one group takes 365: the L2 moves the operands besides the matrices (7
-// TB/s in all), and the MMAs, at 128 bytes a clock, share the shared memory with the epilogue.  Rows of both groups kept
-// in shared memory beside a ring of narrower slices: the same; old entries read into registers from the other side of
-// the diagonal, with operands of both groups in shared memory: 740 us (loads queue behind the stores).
+// groups 487 us on two thirds of the SMs, where one group took 365: the MMAs of a tile's groups follow one another, each
+// behind its operands (545 us with slices of 16 columns, 515 with 32, whole lines of 128 bytes; the rest is operands
+// requested array by array and descriptors a tile ahead).  Rows of both groups kept in shared memory beside a ring of
+// narrower slices: 547 us; old entries read into registers from the other side of the diagonal, with operands of both
+// groups in shared memory: 740 us (loads queue behind the stores).
 //
 // The update kernel runs one CTA on each of two thirds of the SMs.  Work is cut into tiles of
 // 128 x 128 entries on or below the diagonal; runs of consecutive tiles of one row strip
 // ("segments") are handed out through an atomic counter, so a CTA that starts late (another kernel
 // holds its SM) simply finds less left to do.  Inside a CTA three kinds of warps work as a pipeline,
 // linked by mbarriers only:
-//   warp 0      fetches segments, publishes one descriptor per tile (layer, tile origin) and
-//               loads the tile's packed operands by TMA (the 128 rows once per segment, the 128
-//               columns per tile);
+//   warp 0      one thread fetches segments, publishes one descriptor per tile (layer, tile origin), a tile
+//               ahead, and loads the tile's packed operands by TMA (rows that are there already stay).  One thread
+//               throughout: as a whole warp whose lane 0 issued the copies, the other lanes ran ahead of it into the
+//               next tile, and lane 0 met their values;
 //   warp 1      one thread issues the 36 tcgen05.mma (kind::f16, bfloat16, M = N = 128, K = 16)
-//               of a tile (12 for a tile of W^T), the smallest partial products first, so that the truncating
+//               of a tile and group (12 for a tile of W^T), the smallest partial products first, so that the truncating
 //               accumulation meets them while the accumulator is small, into one of two
-//               accumulator stages in tensor memory;
+//               accumulator regions in tensor memory;
 //   warps 2-17  each owns 32 rows x 64 columns of one matrix (H^-1 or Q) in every tile, worked
-//               on as four slices of 16 columns: one lane brings the old entries of a slice in
-//               by TMA (64-byte swizzle) into a ring of three slices of the warp's own (two in
-//               flight while one is worked on), the warp reads the accumulator with tcgen05.ld
-//               (one row per lane), subtracts, stores the mirrored entries [j][i] straight from
-//               registers (lanes run along i: 128-byte pieces) and the entries [i][j] after a
-//               pass through its slice (lanes run along j, 128-bit stores).
+//               on as two slices of 32 columns: one lane brings the old entries of a slice in
+//               by TMA (128-byte swizzle) into a ring of two slices of the warp's own, a tile ahead, the warp
+//               reads the accumulators with tcgen05.ld (one row per lane), subtracts, stores the mirrored
+//               entries [j][i] straight from registers (lanes run along i: 128-byte pieces) and the entries
+//               [i][j] after a pass through its slice (eight lanes along a row: 128-byte pieces).
 // No CTA-wide barrier exists between set-up and exit.  Every mbarrier wait is bounded; a wait that
 // runs out raises an abort flag that all roles poll, the issuer still commits and waits for the
 // MMAs it has issued, every lane that started copies waits for them, and the CTA leaves through
@@ -66,16 +67,16 @@ constexpr int ROWS_BYTES = NARR * ARR_BYTES; // 48 KiB
 constexpr int COLS_BYTES = NARR * ARR_BYTES; // 48 KiB
 constexpr int ACC_STAGES = 2;                // accumulator regions: the groups of the tiles in turn
 constexpr int N_EPI = 16;                    // epilogue warps: 4 lane quarters x 2 matrices x 2 column halves
-constexpr int SUBS = 4;                      // slices of 16 columns per warp and tile
-constexpr int RING = 3;                      // slices per epilogue warp
-constexpr int SLICE_FLOATS = 32 * 16;        // 32 rows x 16 columns
-constexpr int RING_BYTES = N_EPI * RING * SLICE_FLOATS * 4;   // 96 KiB
+constexpr int SUBS = 2;                      // slices of 32 columns per warp and tile
+constexpr int RING = 2;                      // slices per epilogue warp
+constexpr int SLICE_FLOATS = 32 * 32;        // 32 rows x 32 columns
+constexpr int RING_BYTES = N_EPI * RING * SLICE_FLOATS * 4;   // 128 KiB
 constexpr int AQ_SMEM = ROWS_BYTES + COLS_BYTES + RING_BYTES + 1024;
 constexpr int AQ_THREADS = 32 * (2 + N_EPI);
 constexpr uint32_t AQ_TMEM_COLS = 512;       // two stages of (H^-1: 128 columns, Q: 128 columns)
 constexpr int DESC_RING = 4;
 constexpr int MAX_STRIPS = 48;               // d <= 6144
-enum { TILE_STOP = 1, TILE_NEW_ROWS = 2, TILE_W = 4 };
+enum { TILE_STOP = 1, TILE_W = 2 };
 
 // Work list of one launch: the row strips from the longest to the shortest; prefix[k] = number
 // of segments (over all layers) of the k longest strips.
@@ -99,7 +100,7 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                     int* __restrict__ counter, int* __restrict__ layer_status, uint32_t slot_spin_limit) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_tile_full[DESC_RING], bar_tile_empty[DESC_RING];
-    __shared__ uint64_t bar_ops_full, bar_acc_full[ACC_STAGES], bar_acc_empty[ACC_STAGES], bar_final;
+    __shared__ uint64_t bar_ops_full[NARR], bar_ops_free[NARR], bar_acc_full[ACC_STAGES], bar_acc_empty[ACC_STAGES], bar_final;
     __shared__ uint64_t bar_slice[N_EPI][RING];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
@@ -118,7 +119,10 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
             mbar_init(smem_u32(&bar_tile_full[i]), 1);
             mbar_init(smem_u32(&bar_tile_empty[i]), 1 + N_EPI);
         }
-        mbar_init(smem_u32(&bar_ops_full), 1);
+        for (int a = 0; a < NARR; ++a) {
+            mbar_init(smem_u32(&bar_ops_full[a]), 1);
+            mbar_init(smem_u32(&bar_ops_free[a]), 1);
+        }
         for (int i = 0; i < ACC_STAGES; ++i) {
             mbar_init(smem_u32(&bar_acc_full[i]), 1);
             mbar_init(smem_u32(&bar_acc_empty[i]), N_EPI);
@@ -140,87 +144,83 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
     bool failed = false;
 
     if (warp == 0) {
-        // ---------------- scheduler and TMA producer ----------------
-        int t = 0;                       // tiles published so far by this CTA
-        int issued = 0;                  // groups whose operand copies were issued
-        int s = 0;
-        if (lane == 0) s = atomicAdd(counter, 1);
-        s = __shfl_sync(0xffffffffu, s, 0);
-        while (s < sch.n_segments && !failed) {
-            int s_next = 0;
-            if (lane == 0) s_next = atomicAdd(counter, 1);      // in flight while this segment is set up
-            int k = 0;
-            while (k + 1 < sch.n_strips && sch.prefix[k + 1] <= s) ++k;
-            const int I = sch.n_strips - 1 - k;
-            const int within = s - sch.prefix[k];
-            const int segs_strip = (sch.prefix[k + 1] - sch.prefix[k]) / sch.L;
-            const int l = within / segs_strip, sidx = within - l * segs_strip;
-            const int nJ = I + 1 + sch.n_wt;      // tiles J = 0 .. I (the last one holds the diagonal), then W^T
-            const int Jb = sidx * sch.seg, Je = min(Jb + sch.seg, nJ);
-            const int i0 = I * RM;
-            for (int J = Jb; J < Je; ++J, ++t) {
-                const int slot = t & (DESC_RING - 1);
-                if (t >= DESC_RING)
-                    failed = !__all_sync(0xffffffffu,
-                                         mbar_wait_limit(smem_u32(&bar_tile_empty[slot]),
-                                                         (uint32_t)(((t >> 2) - 1) & 1), abortp, slot_spin_limit));
-                if (failed) break;
-                // a tile of W^T takes its column operand from the rows of P that hold C
-                const bool wtile = J > I;
-                const int j0 = wtile ? sch.rows_pad + (J - I - 1) * CN : J * CN;
-                if (lane == 0) {
-                    TileSlot& ts = slots[slot];
-                    ts.l = l; ts.i0 = i0; ts.j0 = j0;
-                    ts.flags = ((J == Jb) ? TILE_NEW_ROWS : 0) | (wtile ? TILE_W : 0);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bar_tile_full[slot]));
+        // ---------------- scheduler and TMA producer (one thread) ----------------
+        if (lane == 0) {
+            int published = 0;               // descriptors so far
+            int issued = 0;                  // groups whose copies were issued
+            int copies[NARR] = {0, 0, 0};    // ... by packed array, the one under way counted
+            auto publish = [&](int l, int i0, int j0, int flags) {
+                const int slot = published & (DESC_RING - 1);
+                if (published >= DESC_RING &&
+                    !mbar_wait_limit(smem_u32(&bar_tile_empty[slot]), (uint32_t)(((published >> 2) - 1) & 1), abortp,
+                                     slot_spin_limit))
+                    return false;
+                TileSlot& ts = slots[slot];
+                ts.l = l; ts.i0 = i0; ts.j0 = j0; ts.flags = flags;
+                mbar_arrive(smem_u32(&bar_tile_full[slot]));
+                ++published;
+                return true;
+            };
+            // The operands of a tile, group after group, an array as soon as the MMAs of the group before are done
+            // with it.  Rows that are there already stay; the order of two groups alternates from tile to tile.
+            int rows_l = -1, rows_i0 = -1, rows_g = -1;      // the rows in shared memory
+            auto load = [&](int t, int l, int i0, int j0) {
                 for (int k2 = 0; k2 < sch.groups; ++k2) {
-                    // The operand tiles are free once the MMAs of the previous group have completed.  The rows stay
-                    // for the next tile of the segment: the order of two groups alternates from tile to tile.
-                    if (issued > 0)
-                        failed = !__all_sync(0xffffffffu,
-                                             mbar_wait(smem_u32(&bar_acc_full[(issued - 1) & 1]),
-                                                       (uint32_t)(((issued - 1) >> 1) & 1), abortp));
-                    if (failed) break;
-                    if (lane == 0) {
-                        const uint32_t full = smem_u32(&bar_ops_full);
-                        const int g = sch.groups > 1 ? k2 ^ (t & 1) : 0;
-                        const bool rows = J == Jb || k2 > 0;
-                        mbar_expect_tx(full, (uint32_t)((rows ? ROWS_BYTES : 0) + COLS_BYTES));
-#pragma unroll
-                        for (int a = 0; a < NARR; ++a)
-#pragma unroll
-                            for (int b = 0; b < 2; ++b) {
-                                if (rows)
-                                    tma_load_4d(rows_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
-                                                i0 + b * BOX_ROWS, g * NARR + a, l);
-                                tma_load_4d(cols_smem + a * ARR_BYTES + b * BOX_BYTES, &map, full, 0,
-                                            j0 + b * BOX_ROWS, g * NARR + a, l);
-                            }
+                    const int g = sch.groups > 1 ? k2 ^ (t & 1) : 0;
+                    const bool rows = l != rows_l || i0 != rows_i0 || g != rows_g;
+                    rows_l = l; rows_i0 = i0; rows_g = g;
+                    for (int k = 0; k < NARR; ++k) {
+                        const int a = k + 1 < NARR ? k + 1 : 0;         // 1, 2, 0: the order in which they are done with
+                        if (issued > 0 && !mbar_wait(smem_u32(&bar_ops_free[a]), (uint32_t)((issued - 1) & 1), abortp))
+                            return false;
+                        const uint32_t full = smem_u32(&bar_ops_full[a]);
+                        const uint32_t to_rows = rows_smem + (uint32_t)(a * ARR_BYTES), to_cols = cols_smem + (uint32_t)(a * ARR_BYTES);
+                        mbar_expect_tx(full, (uint32_t)((rows ? 2 : 1) * ARR_BYTES));
+                        ++copies[a];
+                        for (int b = 0; b < 2; ++b) {
+                            if (rows) tma_load_4d(to_rows + b * BOX_BYTES, &map, full, 0, i0 + b * BOX_ROWS, g * NARR + a, l);
+                            tma_load_4d(to_cols + b * BOX_BYTES, &map, full, 0, j0 + b * BOX_ROWS, g * NARR + a, l);
+                        }
                     }
                     ++issued;
                 }
-                if (failed) break;
+                return true;
+            };
+            // descriptors run a tile ahead of the operands, so that nobody waits for one
+            int t = 0, pl = 0, pi0 = 0, pj0 = 0;           // tile t: published, its operands are next
+            bool pending = false;
+            int s = atomicAdd(counter, 1);
+            while (s < sch.n_segments && !failed) {
+                const int s_next = atomicAdd(counter, 1);   // in flight while this segment is set up
+                int k = 0;
+                while (k + 1 < sch.n_strips && sch.prefix[k + 1] <= s) ++k;
+                const int I = sch.n_strips - 1 - k;
+                const int within = s - sch.prefix[k];
+                const int segs_strip = (sch.prefix[k + 1] - sch.prefix[k]) / sch.L;
+                const int l = within / segs_strip, sidx = within - l * segs_strip;
+                const int nJ = I + 1 + sch.n_wt;      // tiles J = 0 .. I (the last one holds the diagonal), then W^T
+                const int Jb = sidx * sch.seg, Je = min(Jb + sch.seg, nJ);
+                const int i0 = I * RM;
+                for (int J = Jb; J < Je; ++J) {
+                    // a tile of W^T takes its column operand from the rows of P that hold C
+                    const bool wtile = J > I;
+                    const int j0 = wtile ? sch.rows_pad + (J - I - 1) * CN : J * CN;
+                    if (!publish(l, i0, j0, wtile ? TILE_W : 0) || (pending && !load(t, pl, pi0, pj0))) { failed = true; break; }
+                    t += pending;
+                    pl = l; pi0 = i0; pj0 = j0;
+                    pending = true;
+                }
+                s = s_next;
             }
-            s = __shfl_sync(0xffffffffu, s_next, 0);
-        }
-        if (!failed) {                   // stop descriptor
-            const int slot = t & (DESC_RING - 1);
-            if (t >= DESC_RING)
-                failed = !__all_sync(0xffffffffu,
-                                     mbar_wait_limit(smem_u32(&bar_tile_empty[slot]),
-                                                     (uint32_t)(((t >> 2) - 1) & 1), abortp, slot_spin_limit));
-            if (!failed && lane == 0) {
-                slots[slot].flags = TILE_STOP;
-                mbar_arrive(smem_u32(&bar_tile_full[slot]));
+            if (!failed) failed = !publish(0, 0, 0, TILE_STOP) || (pending && !load(t, pl, pi0, pj0));
+            if (failed) {
+                abort_flag = 1;
+                // copies already issued land in this CTA's shared memory: give them a bounded chance
+                for (int a = 0; a < NARR; ++a)
+                    if (copies[a] > 0) mbar_wait_quiet(smem_u32(&bar_ops_full[a]), (uint32_t)((copies[a] - 1) & 1));
             }
         }
-        if (failed) {
-            abort_flag = 1;
-            // copies already issued land in this CTA's shared memory: give them a bounded chance
-            if (lane == 0 && issued > 0) mbar_wait_quiet(smem_u32(&bar_ops_full), (uint32_t)((issued - 1) & 1));
-        }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer (one thread) ----------------
         if (lane == 0) {
@@ -244,7 +244,9 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 if (flags & TILE_STOP) break;
                 for (int g = 0; g < sch.groups; ++g, ++unit) {
                     const int st = unit & 1;
-                    if (!mbar_wait(smem_u32(&bar_ops_full), (uint32_t)(unit & 1), abortp)) { failed = true; break; }
+                    for (int a = 0; a < NARR && !failed; ++a)
+                        if (!mbar_wait(smem_u32(&bar_ops_full[a]), (uint32_t)(unit & 1), abortp)) failed = true;
+                    if (failed) break;
                     if (unit >= ACC_STAGES &&
                         !mbar_wait(smem_u32(&bar_acc_empty[st]), (uint32_t)(((unit >> 1) - 1) & 1), abortp)) {
                         failed = true;
@@ -257,17 +259,25 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                         umma_bf16(acc, r[pr], c[pc2], idesc, first ? 0u : 1u);
                         umma_bf16(acc, r[pr] + 2u, c[pc2] + 2u, idesc, 1u);
                     };
-                    // H^-1: U U^T; smallest terms first
-                    prod(t_a, U1, U3, true);  prod(t_a, U3, U1, false); prod(t_a, U2, U2, false);
-                    prod(t_a, U1, U2, false); prod(t_a, U2, U1, false); prod(t_a, U1, U1, false);
-                    // Q: Z U^T + U Z^T (a tile of W^T has no second matrix: its column operand is C
-                    // in the place of U, and the products above are the whole update U^T C)
-                    if (!(flags & TILE_W)) {
-                        prod(t_q, Z1, U3, true);  prod(t_q, Z3, U1, false); prod(t_q, Z2, U2, false);
-                        prod(t_q, U1, Z3, false); prod(t_q, U3, Z1, false); prod(t_q, U2, Z2, false);
+                    // H^-1: U U^T, Q: Z U^T + U Z^T (a tile of W^T has no second matrix: its column operand is C
+                    // in the place of U, and the products of the first are the whole update U^T C); smallest terms
+                    // first, and arranged so that the arrays with the third parts and with Z are done with early
+                    const bool w = flags & TILE_W;
+                    prod(t_a, U1, U3, true);  prod(t_a, U3, U1, false);
+                    if (!w) {
+                        prod(t_q, Z1, U3, true);  prod(t_q, Z3, U1, false);
+                        prod(t_q, U1, Z3, false); prod(t_q, U3, Z1, false);
+                    }
+                    umma_commit(smem_u32(&bar_ops_free[1]));
+                    if (!w) {
+                        prod(t_q, Z2, U2, false); prod(t_q, U2, Z2, false);
                         prod(t_q, Z1, U2, false); prod(t_q, Z2, U1, false); prod(t_q, U1, Z2, false);
                         prod(t_q, U2, Z1, false); prod(t_q, Z1, U1, false); prod(t_q, U1, Z1, false);
                     }
+                    umma_commit(smem_u32(&bar_ops_free[2]));
+                    prod(t_a, U2, U2, false);
+                    prod(t_a, U1, U2, false); prod(t_a, U2, U1, false); prod(t_a, U1, U1, false);
+                    umma_commit(smem_u32(&bar_ops_free[0]));
                     umma_commit(smem_u32(&bar_acc_full[st]));
                 }
                 if (failed) break;
@@ -289,8 +299,8 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
         const uint32_t bar0 = smem_u32(&bar_slice[ew][0]);
         const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(mat * CN + 64 * h);
         const size_t dd = (size_t)d * d;
-        // A slice is [32 rows][16 columns] as TMA writes it with the 64-byte swizzle: 64-byte rows,
-        // the 16-byte unit index of row r XORed with (r >> 1) & 3: a lane per row and four lanes
+        // A slice is [32 rows][32 columns] as TMA writes it with the 128-byte swizzle: 128-byte rows,
+        // the 16-byte unit index of row r XORed with r & 7: a lane per row and eight lanes
         // per row both reach it without bank conflicts.
 
         // Copy cursor: tile pt (descriptor in its ring slot), next slice psub.  One call starts
@@ -320,13 +330,13 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                     const uint32_t bar = bar0 + 8u * (uint32_t)(c % RING);
                     mbar_expect_tx(bar, (uint32_t)(SLICE_FLOATS * 4));
                     // a tile of W^T: both matrices' warps bring the same slices in (the second
-                    // copy is served by L2) and work on two of the four each
+                    // copy is served by L2) and work on one of the two each
                     if (pflags & TILE_W)
                         tma_load_3d(ring_u32 + (uint32_t)((c % RING) * SLICE_FLOATS * 4), &map_w, bar,
-                                    nj0 - sch.rows_pad + 64 * h + 16 * psub, ni0 + 32 * q, nl);
+                                    nj0 - sch.rows_pad + 64 * h + 32 * psub, ni0 + 32 * q, nl);
                     else
                         tma_load_3d(ring_u32 + (uint32_t)((c % RING) * SLICE_FLOATS * 4), min_map, bar,
-                                    nj0 + 64 * h + 16 * psub, ni0 + 32 * q, nl);
+                                    nj0 + 64 * h + 32 * psub, ni0 + 32 * q, nl);
                 }
                 issued = c + 1;
                 if (++psub == SUBS) {
@@ -350,125 +360,106 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
             failed = __any_sync(0xffffffffu, failed);
             if (failed) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float upd[32];
 #pragma unroll 1
             for (int sub = 0; sub < SUBS; ++sub) {
-                if (!(sub & 1)) {
-                    // ---- the update of two slices, summed over the groups (each in an accumulator of its own and
-                    //      joined in fp32 here: a longer chain in tensor memory would truncate more)
-                    // (a tile of W^T has one accumulator, which both matrices' warps read)
-                    const uint32_t from = lane_taddr - ((cflags & TILE_W) ? (uint32_t)(mat * CN) : 0u) + (uint32_t)(16 * sub);
+                const int c = SUBS * t + sub;
+                // ---- the update of the slice, summed over the groups (each in an accumulator of its own and
+                //      joined in fp32 here: a longer chain in tensor memory would truncate more)
+                // (a tile of W^T has one accumulator, which both matrices' warps read)
+                const uint32_t from = lane_taddr - ((cflags & TILE_W) ? (uint32_t)(mat * CN) : 0u) + (uint32_t)(32 * sub);
+                float upd[32];
 #pragma unroll
-                    for (int cc = 0; cc < 2; ++cc) {
-                        uint32_t v[16];
-                        tmem_ld16(from + (uint32_t)((unit & 1) * 2 * CN + 16 * cc), v);
+                for (int cc = 0; cc < 2; ++cc) {
+                    uint32_t v[16];
+                    tmem_ld16(from + (uint32_t)((unit & 1) * 2 * CN + 16 * cc), v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) upd[16 * cc + e] = __uint_as_float(v[e]);
+                    if (sch.groups > 1) {
+                        tmem_ld16(from + (uint32_t)(((unit + 1) & 1) * 2 * CN + 16 * cc), v);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) upd[16 * cc + e] = __uint_as_float(v[e]);
-                        if (sch.groups > 1) {
-                            tmem_ld16(from + (uint32_t)(((unit + 1) & 1) * 2 * CN + 16 * cc), v);
-                            tmem_ld_wait();
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) upd[16 * cc + e] += __uint_as_float(v[e]);
-                        }
+                        for (int e = 0; e < 16; ++e) upd[16 * cc + e] += __uint_as_float(v[e]);
                     }
-                    if (sub == SUBS - 2) {               // all of the tile's entries are in registers
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0)
-                            for (int g = 0; g < sch.groups; ++g) mbar_arrive(smem_u32(&bar_acc_empty[(unit + g) & 1]));
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) upd[e] = upd[16 + e];
                 }
-                const int c = SUBS * t + sub;
-                // ---- start the copy of the slice two ahead, then wait for slice c
-                if (!copy_next()) { failed = true; break; }
+                if (sub == SUBS - 1) {                   // all of the tile's entries are in registers
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        for (int g = 0; g < sch.groups; ++g) mbar_arrive(smem_u32(&bar_acc_empty[(unit + g) & 1]));
+                }
                 if (!mbar_wait(bar0 + 8u * (uint32_t)(c % RING), (uint32_t)((c / RING) & 1), abortp)) failed = true;
                 failed = __any_sync(0xffffffffu, failed);
                 if (failed) break;
                 float* buf = ring + (size_t)(c % RING) * SLICE_FLOATS;
+                float4* b4 = reinterpret_cast<float4*>(buf);
+                const int ib = ci0 + 32 * q;             // first row of the slice
+                const int jc = cj0 + 64 * h + 32 * sub;  // first column of the slice
+                // ---- new entries: old - update, one matrix row per lane
+                //      (tile of W^T: the two warps that share a quarter of the rows and a half of the columns
+                //      take one of its two slices each)
+                if (!(cflags & TILE_W) || sub == mat) {
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) {
+                        float4& o = b4[lane * 8 + (g ^ (lane & 7))];
+                        upd[4 * g] = o.x - upd[4 * g];
+                        upd[4 * g + 1] = o.y - upd[4 * g + 1];
+                        upd[4 * g + 2] = o.z - upd[4 * g + 2];
+                        upd[4 * g + 3] = o.w - upd[4 * g + 3];
+                        o = make_float4(upd[4 * g], upd[4 * g + 1], upd[4 * g + 2], upd[4 * g + 3]);
+                    }
+                }
                 if (cflags & TILE_W) {
-                    // ---- tile of W^T: rows = positions, columns = row indices of W; no mirror.
-                    //      The two warps that share a quarter of the rows and a half of the columns
-                    //      take two of its four slices each.
-                    if ((sub >> 1) == mat) {
-                        float4* b4 = reinterpret_cast<float4*>(buf) + lane * 4;
-#pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const int pg = g ^ ((lane >> 1) & 3);
-                            const float4 o = b4[pg];
-                            b4[pg] = make_float4(o.x - upd[4 * g], o.y - upd[4 * g + 1],
-                                                 o.z - upd[4 * g + 2], o.w - upd[4 * g + 3]);
-                        }
-                        __syncwarp();
+                    // ---- tile of W^T: rows = positions, columns = row indices of W; no mirror
+                    __syncwarp();
+                    if (sub == mat) {
                         float* Wo = W2 + (size_t)cl * d * rp;
-                        const int jc = cj0 - sch.rows_pad + 64 * h + 16 * sub, ib = ci0 + 32 * q;
 #pragma unroll
-                        for (int it = 0; it < 4; ++it) {
-                            const int row = 8 * it + (lane >> 2), u = lane & 3;
-                            const float4 x = reinterpret_cast<const float4*>(buf)[row * 4 + (u ^ ((row >> 1) & 3))];
-                            const int gi = ib + row, gj = jc + 4 * u;
+                        for (int it = 0; it < 8; ++it) {
+                            const int row = 4 * it + (lane >> 3), u = lane & 7;
+                            const float4 x = b4[row * 8 + (u ^ (row & 7))];
+                            const int gi = ib + row, gj = jc - sch.rows_pad + 4 * u;
                             if (gi < n_pos && gj < rp) *reinterpret_cast<float4*>(Wo + (size_t)gi * rp + gj) = x;
                         }
                     }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (sub == SUBS - 1) { cl = nl; ci0 = ni0; cj0 = nj0; cflags = pflags; }
-                    continue;
-                }
-                // ---- new entries: old - update, one matrix row per lane
-                float4* b4 = reinterpret_cast<float4*>(buf) + lane * 4;
-                float rr[16];
+                } else {
+                    float* Mo = Mout + (size_t)cl * dd;
+                    // ---- mirror [j][i]: lanes run along i
+                    {
+                        const int i = ib + lane;
+                        const int jlim = (i < n_pos) ? i - jc : 0;     // entries e < jlim lie below the diagonal
+                        float* mp = Mo + (size_t)jc * d + i;
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const int pg = g ^ ((lane >> 1) & 3);
-                    const float4 o = b4[pg];
-                    rr[4 * g] = o.x - upd[4 * g];
-                    rr[4 * g + 1] = o.y - upd[4 * g + 1];
-                    rr[4 * g + 2] = o.z - upd[4 * g + 2];
-                    rr[4 * g + 3] = o.w - upd[4 * g + 3];
-                    b4[pg] = make_float4(rr[4 * g], rr[4 * g + 1], rr[4 * g + 2], rr[4 * g + 3]);
-                }
-                float* Mo = Mout + (size_t)cl * dd;
-                const int jc = cj0 + 64 * h + 16 * sub;  // first column of the slice
-                const int ib = ci0 + 32 * q;             // first row of the slice
-                // ---- mirror [j][i]: lanes run along i
-                {
-                    const int i = ib + lane;
-                    const int jlim = (i < n_pos) ? i - jc : 0;     // entries e < jlim lie below the diagonal
-                    float* mp = Mo + (size_t)jc * d + i;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        if (e < jlim) *mp = rr[e];
-                        mp += d;
+                        for (int e = 0; e < 32; ++e) {
+                            if (e < jlim) *mp = upd[e];
+                            mp += d;
+                        }
                     }
-                }
-                __syncwarp();
-                // ---- [i][j]: eight rows per instruction, four lanes along a row
+                    __syncwarp();
+                    // ---- [i][j]: four rows per instruction, eight lanes along a row
 #pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    const int row = 8 * it + (lane >> 2), u = lane & 3;
-                    const float4 x = reinterpret_cast<const float4*>(buf)[row * 4 + (u ^ ((row >> 1) & 3))];
-                    const int gi = ib + row, gj = jc + 4 * u;
-                    if (gi < n_pos) {
-                        float* p = Mo + (size_t)gi * d + gj;
-                        if (gj + 3 < gi) {
-                            *reinterpret_cast<float4*>(p) = x;
-                        } else {
-                            if (gj < gi) p[0] = x.x;
-                            if (gj + 1 < gi) p[1] = x.y;
-                            if (gj + 2 < gi) p[2] = x.z;
+                    for (int it = 0; it < 8; ++it) {
+                        const int row = 4 * it + (lane >> 3), u = lane & 7;
+                        const float4 x = b4[row * 8 + (u ^ (row & 7))];
+                        const int gi = ib + row, gj = jc + 4 * u;
+                        if (gi < n_pos) {
+                            float* p = Mo + (size_t)gi * d + gj;
+                            if (gj + 3 < gi) {
+                                *reinterpret_cast<float4*>(p) = x;
+                            } else {
+                                if (gj < gi) p[0] = x.x;
+                                if (gj + 1 < gi) p[1] = x.y;
+                                if (gj + 2 < gi) p[2] = x.z;
+                            }
                         }
                     }
                 }
-                // the slice may be refilled by a copy: fence this lane's accesses, then the warp
+                // the slice is refilled: fence this lane's accesses, then the warp; the copy of the slice two ahead
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                // the copy cursor has moved on to the next tile by now: take its origin over
-                // before the cursor can replace it (it opens tile t + 2 during slice 1 of tile t + 1)
+                // (the cursor is in the next tile; with the last slice's copy it moves on to the one behind)
                 if (sub == SUBS - 1) { cl = nl; ci0 = ni0; cj0 = nj0; cflags = pflags; }
+                if (!copy_next()) { failed = true; break; }
             }
             unit += sch.groups;
         }
@@ -530,17 +521,17 @@ bool lazy_tc_make_map(CUtensorMap* m, const float* P, int L, int d, int rp) {
 }
 
 // Tensor map over one of the fp32 matrices M[L][d][cols] (cols a multiple of 4; d for H^-1 and Q,
-// the padded row count of W for W^T): box = 32 rows x 16 columns, 64-byte swizzle; what lies
+// the padded row count of W for W^T): box = 32 rows x 32 columns, 128-byte swizzle; what lies
 // outside the matrix reads as zero.
 bool lazy_tc_make_matrix_map(CUtensorMap* m, const float* M, int L, int d, int cols) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
     cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)d, (cuuint64_t)L};
     cuuint64_t strides[2] = {(cuuint64_t)cols * 4, (cuuint64_t)d * cols * 4};
-    cuuint32_t box[3] = {16, 32, 1};
+    cuuint32_t box[3] = {32, 32, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(M), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
