@@ -7,12 +7,35 @@
 //   k_gather_rows       out[l][k*g + c][:] = M[l][kept[l][k]*g + c][:]
 //
 // All three only move data: results are bit-exact.
+//
+// A level is three launches of 5 to 25 us, so they are programmatic dependent launches: a kernel lets the next one
+// start once all of its own CTAs run, and the next one's CTAs take the SMs that the last ones leave and wait there for
+// its end (griddepcontrol.wait, by every thread before it reads or writes anything; loads are coherent ones, which
+// nothing moves in front of it).  Eleven levels of 12 x 768 x 3072, 33 launches: 634 -> 561 us.
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace ziplm {
 namespace {
 
 constexpr int KEEP_THREADS = 1024;
+
+template <typename... P, typename... A>
+ziplm_status launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
 
 // One CTA per layer.  The removed structures are marked in a bitmap in shared memory; every thread then
 // owns whole words of it, counts their survivors, a scan over the threads (within the warps by shuffles,
@@ -28,13 +51,15 @@ __global__ void __launch_bounds__(KEEP_THREADS) k_kept_structures(const int* __r
     const int words = (G + 31) / 32;
     const int l = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int* ord = order + (size_t)l * G;
+    tc::grid_trigger();
+    tc::grid_wait();
     if (tid == 0) fail = 0;
     for (int w = tid; w < words; w += KEEP_THREADS)
         bits[w] = (w + 1) * 32 <= G ? 0u : ~0u << (G & 31);   // what lies past G counts as removed
     __syncthreads();
     const int n_removed = G - level;
     for (int t = tid; t < n_removed; t += KEEP_THREADS) {
-        const int s = ord[t];
+        const int s = __ldca(ord + t);
         if (s < 0 || s >= G) {
             fail = 1;
         } else {
@@ -79,11 +104,13 @@ __global__ void __launch_bounds__(256) k_gather_columns(const float* __restrict_
     const int l = blockIdx.z;
     const int n_out = level * g;
     const int j = (blockIdx.x * 256 + threadIdx.x) * VEC;
+    tc::grid_trigger();
+    tc::grid_wait();
     if (j >= n_out) return;
     int src[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) {
-        const int s = kept[(size_t)l * level + (j + e) / g];
+        const int s = __ldca(kept + (size_t)l * level + (j + e) / g);
         src[e] = (unsigned)s < (unsigned)G ? s * g + (j + e) % g : -1;      // an index outside [0, G) gives zeros
     }
     const int i0 = blockIdx.y * COL_ROWS;
@@ -97,7 +124,7 @@ __global__ void __launch_bounds__(256) k_gather_columns(const float* __restrict_
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int e = 0; e < VEC; ++e)
-                v[i][e] = h + i < n && src[e] >= 0 ? __ldg(Ml + (size_t)(h + i) * (size_t)ld + src[e]) : 0.f;
+                v[i][e] = h + i < n && src[e] >= 0 ? __ldca(Ml + (size_t)(h + i) * (size_t)ld + src[e]) : 0.f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (h + i >= n) break;
@@ -118,8 +145,10 @@ __global__ void __launch_bounds__(256) k_gather_rows(const float* __restrict__ M
     constexpr int N = sizeof(V) / sizeof(float);
     const int l = blockIdx.y, lane = threadIdx.x & 31;
     const int k = blockIdx.x * 8 + (threadIdx.x >> 5);         // output row
+    tc::grid_trigger();
+    tc::grid_wait();
     if (k >= level * g) return;
-    const int s = kept[(size_t)l * level + k / g];
+    const int s = __ldca(kept + (size_t)l * level + k / g);
     const bool ok = (unsigned)s < (unsigned)G;                 // an index outside [0, G) gives zeros
     const V* row = reinterpret_cast<const V*>(M + (size_t)l * (size_t)layer_stride +
                                               (size_t)(ok ? s * g + k % g : 0) * (size_t)ld);
@@ -128,7 +157,7 @@ __global__ void __launch_bounds__(256) k_gather_rows(const float* __restrict__ M
     for (int c0 = lane; c0 < n; c0 += 256) {
         V v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = ok && c0 + 32 * e < n ? __ldg(row + c0 + 32 * e) : V();
+        for (int e = 0; e < 8; ++e) v[e] = ok && c0 + 32 * e < n ? __ldca(row + c0 + 32 * e) : V();
 #pragma unroll
         for (int e = 0; e < 8; ++e)
             if (c0 + 32 * e < n) __stcs(dst + c0 + 32 * e, v[e]);
@@ -144,9 +173,7 @@ ziplm_status run_kept_structures(const int* order, int L, int G, int level, int*
     if (smem > 48 * 1024)
         ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_kept_structures, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
-    k_kept_structures<<<L, KEEP_THREADS, smem, st>>>(order, G, level, kept, bad);
-    ZIPLM_CHECK_LAUNCH();
-    return ZIPLM_OK;
+    return launch_dependent(k_kept_structures, dim3(L), KEEP_THREADS, smem, st, order, G, level, kept, bad);
 }
 
 ziplm_status run_gather_columns(const float* M, long long ld, long long layer_stride, const int* kept,
@@ -164,10 +191,10 @@ ziplm_status run_gather_columns(const float* M, long long ld, long long layer_st
         const dim3 grid((unsigned)((n_out + 256 * vec - 1) / (256 * vec)), (unsigned)((rows + COL_ROWS - 1) / COL_ROWS),
                         (unsigned)ln);
         if (grid.y > 65535) return ZIPLM_ERR_UNSUPPORTED;
-        kernel<<<grid, 256, 0, st>>>(M + (size_t)l0 * (size_t)layer_stride, ld, layer_stride,
-                                               kept + (size_t)l0 * level, rows, G, g, level,
-                                               out + (size_t)l0 * rows * n_out);
-        ZIPLM_CHECK_LAUNCH();
+        const ziplm_status s = launch_dependent(kernel, grid, 256, 0, st, M + (size_t)l0 * (size_t)layer_stride, ld,
+                                                layer_stride, kept + (size_t)l0 * level, rows, G, g, level,
+                                                out + (size_t)l0 * rows * n_out);
+        if (s != ZIPLM_OK) return s;
     }
     return ZIPLM_OK;
 }
@@ -180,10 +207,11 @@ ziplm_status run_gather_rows(const float* M, long long ld, long long layer_strid
         const bool quads = cols % 4 == 0 && ld % 4 == 0 && layer_stride % 4 == 0 &&
                            (reinterpret_cast<uintptr_t>(M) | reinterpret_cast<uintptr_t>(out)) % 16 == 0;
         auto kernel = quads ? k_gather_rows<float4> : k_gather_rows<float>;
-        kernel<<<dim3((unsigned)((level * g + 7) / 8), (unsigned)ln), 256, 0, st>>>(
-            M + (size_t)l0 * (size_t)layer_stride, ld, layer_stride, kept + (size_t)l0 * level, cols, G, g,
-            level, out + (size_t)l0 * level * g * (size_t)cols);
-        ZIPLM_CHECK_LAUNCH();
+        const ziplm_status s = launch_dependent(kernel, dim3((unsigned)((level * g + 7) / 8), (unsigned)ln), 256, 0, st,
+                                                M + (size_t)l0 * (size_t)layer_stride, ld, layer_stride,
+                                                kept + (size_t)l0 * level, cols, G, g, level,
+                                                out + (size_t)l0 * level * g * (size_t)cols);
+        if (s != ZIPLM_OK) return s;
     }
     return ZIPLM_OK;
 }

@@ -1015,3 +1015,40 @@ def test_blocks_of_one_and_two_groups_of_steps(d, r, levels):
     sh = wl.scaled(wl.CONFIGS["c3_bert_base_fc2"][0], d_col=d, d_row=r, d_latent=d // 4,
                    n_tokens=d + 500, n_layers=1, levels=tuple(levels))
     run_case(sh)
+
+
+def test_reshaping_launches_wait_for_what_they_read_also_in_a_graph():
+    """The three launches of a level overlap the end of the one in front: they must see what it and a torch kernel
+    before them wrote, call after call into the same buffers and in replays of a captured graph."""
+    z = zb()
+    L, r, d, level = 3, 700, 1024, 600
+    gen = torch.Generator("cuda").manual_seed(3)
+    orders = torch.rand(5, L, d, generator=gen, device="cuda").argsort(dim=2).to(torch.int32)
+    weights = torch.randn(5, L, r, d, generator=gen, device="cuda")
+    order, M = orders[0].clone(), weights[0].clone()
+
+    def level_of_it():
+        order.copy_(src_order)
+        M.copy_(src_M)
+        kept, _ = z.kept_structures(order, level)
+        cols = z.gather_columns(M, kept, 1)
+        return kept, cols, z.gather_rows(M.transpose(1, 2).contiguous(), kept, 1)
+
+    src_order, src_M = orders[0].clone(), weights[0].clone()
+    level_of_it()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        captured = level_of_it()
+    for i in range(5):
+        src_order.copy_(orders[i])
+        src_M.copy_(weights[i])
+        graph.replay()
+        eager = level_of_it()
+        torch.cuda.synchronize()
+        for l in range(L):
+            keep = torch.sort(orders[i, l, d - level:]).values
+            for kept, cols, rows in (captured, eager):
+                assert torch.equal(kept[l], keep)
+                assert torch.equal(cols[l], weights[i, l][:, keep.long()])
+                assert torch.equal(rows[l], weights[i, l][:, keep.long()].t())
