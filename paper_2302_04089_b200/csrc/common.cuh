@@ -67,6 +67,25 @@ struct PhaseScope {
         if (e__ != cudaSuccess) return ZIPLM_ERR_CUDA;         \
     } while (0)
 
+// Programmatic dependent launch: the kernel's CTAs may start when all CTAs of the kernel before have issued
+// griddepcontrol.launch_dependents or ended; it waits for that kernel itself (griddepcontrol.wait).
+template <typename... P, typename... A>
+inline ziplm_status launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+    ZIPLM_CHECK_LAUNCH();
+    return ZIPLM_OK;
+}
+
 // A layer's status only ever moves from OK to the first error seen.
 __device__ inline void set_layer_status(int* layer_status, int l, int code) {
     atomicCAS(layer_status + l, (int)ZIPLM_OK, code);

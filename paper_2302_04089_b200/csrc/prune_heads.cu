@@ -15,7 +15,7 @@
 // rows of W for every head and step (232 us a step for 12 layers of 12 heads of 64), then another
 // 250 us for the update on the float64 FMA pipe.  Here every product is a g x g x g tile product on
 // the float64 tensor-core instruction, the inverse of a head's block goes by 16 x 16 blocks (two
-// barriers per block), and a step is two launches: `solve` (which also selects) and `update` (whose
+// barriers per block), and a step is two launches (programmatic dependent ones): `solve` (which also selects) and `update` (whose
 // diagonal tiles go on to score their head for the next step, and whose tiles of W write the
 // snapshot).
 #include <math.h>
@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "factor16.cuh"
 #include "inverse_i8.cuh"
+#include "tc_common.cuh"
 
 namespace ziplm {
 namespace {
@@ -102,7 +103,7 @@ template <int G8, bool XKM, bool YKM>
 __device__ __forceinline__ void h_chunk_mma(HeadAcc<G8>& acc, const double* sx, const double* sy, int steps, int warp,
                                             int lane) {
     using S = HeadShape<G8>;
-#pragma unroll 2
+#pragma unroll 4
     for (int kk = 0; kk < steps; ++kk) {
         double b[S::CF];
 #pragma unroll
@@ -399,6 +400,8 @@ __global__ void __launch_bounds__(HT) k_heads_solve(Heads w, int t) {
     __shared__ int s_pick;
     const int l = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
     const int* alive = w.alive + ((size_t)l * 2 + (t & 1)) * w.G;
+    tc::grid_trigger();
+    tc::grid_wait();
     if (tid < 32) {
         double best = INFINITY;
         int at = 0x7fffffff;
@@ -463,15 +466,18 @@ __global__ void __launch_bounds__(HT) k_heads_solve(Heads w, int t) {
     });
 }
 
-// CTAs 0 .. G - 1: diagonal blocks of H^-1 and Q, then the head's next score (the longest CTAs first);
-// the next G (G - 1) / 2: blocks below the diagonal; the rest: blocks of g rows of W and, when `slot` is a
-// level, of the snapshot.
+// CTAs 0 .. G - 1 of every layer: diagonal blocks of H^-1 and Q, then the head's next score; the next G (G - 1) / 2:
+// blocks below the diagonal; the rest: blocks of g rows of W and, when `slot` is a level, of the snapshot.  The
+// longest CTAs come first, those of all layers before the next kind (layer after layer the last layer's scores, a chain
+// of 20000 clocks, began when the rest was nearly done: twelve updates of 12 x 768 x 768 took 910 us, now 749).
 template <int G8>
 __global__ void __launch_bounds__(HT) k_heads_update(Heads w, int t, int slot, int rescore) {
     using S = HeadShape<G8>;
     extern __shared__ __align__(16) double smem[];
     __shared__ double red[HT / 32];
-    const int l = blockIdx.y, x = blockIdx.x, n_pairs = w.G * (w.G + 1) / 2;
+    const int l = blockIdx.x % w.L, x = blockIdx.x / w.L, n_pairs = w.G * (w.G + 1) / 2;
+    tc::grid_trigger();
+    tc::grid_wait();
     if (slot >= 0 && x == 0 && l == 0 && threadIdx.x == 0) w.steps_of[slot] = t + 1;
     const int* alive = w.alive + ((size_t)l * 2 + ((t + 1) & 1)) * w.G;
     const size_t ops = (size_t)l * S::g * w.d;
@@ -667,14 +673,14 @@ ziplm_status run_heads(HeadsWs& ws, float damp_frac, const int* levels, float* l
     for (int t = 0; t < n_steps; ++t) {
         {
             PhaseScope ps(PH_BLOCK_SCORE, st);
-            k_heads_solve<G8><<<dim3(G, L), HT, smem, st>>>(w, t);
-            ZIPLM_CHECK_LAUNCH();
+            if ((s = launch_dependent(k_heads_solve<G8>, dim3(G, L), HT, smem, st, w, t)) != ZIPLM_OK) return s;
         }
         const bool level = levels[slot] == G - t - 1;
         if (G - t > 1 || level) {
             PhaseScope ps(PH_BLOCK_UPDATE, st);
-            k_heads_update<G8><<<dim3(ctas, L), HT, smem, st>>>(w, t, level ? slot : -1, t + 1 < n_steps);
-            ZIPLM_CHECK_LAUNCH();
+            s = launch_dependent(k_heads_update<G8>, dim3((unsigned)ctas * (unsigned)L), HT, smem, st, w, t,
+                                 level ? slot : -1, t + 1 < n_steps ? 1 : 0);
+            if (s != ZIPLM_OK) return s;
         }
         if (level) ++slot;
     }

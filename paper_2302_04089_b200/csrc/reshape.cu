@@ -20,23 +20,6 @@ namespace {
 
 constexpr int KEEP_THREADS = 1024;
 
-template <typename... P, typename... A>
-ziplm_status launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
-    ZIPLM_CHECK_LAUNCH();
-    return ZIPLM_OK;
-}
-
 // One CTA per layer.  The removed structures are marked in a bitmap in shared memory; every thread then
 // owns whole words of it, counts their survivors, a scan over the threads (within the warps by shuffles,
 // then over the warps' totals) gives its first output slot, and the words are written in order.
