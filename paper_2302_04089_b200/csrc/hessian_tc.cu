@@ -64,65 +64,101 @@ constexpr int FOLD = 32;
 constexpr int EPI_WARPS = 8;                  // two warps per TMEM lane quarter, 64 columns each
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int OUT_PITCH = TM + 1;             // floats of a row of the finished tile in shared memory
+constexpr int PART_PITCH = TM + 4;            // ... of a part of it, whose rows are read 16 bytes a lane
 
 // The end of a tile that S CTAs of a cluster have shared, their parts in out_tile of each: a CTA finishes 128 / S
 // rows.  Sums over the parts in rank order, rows [i][j] written along j, mirrored rows [j][i] along i.
 // A warp takes R rows at a time, the parts and the old values of all of them requested together, and eight
 // mirrored pieces at a time: one after the other the two took 22000 clocks of a tile's 32000 (13 x 1145 features,
 // 324 bf16 tokens: 70 -> 54 us a call).
+// Parts are read 16 bytes a lane, four columns, and the scales wait in shared memory: 1 x 256 x 2048 fp32 on clusters of
+// eight 12.8 us, against 15.5 with 4 bytes a lane and the scales from global memory behind the last barrier.
 struct TileEnd {
     float* out_tile; float* mirror;
-    int rank, i0, j0, d;
+    int rank, i0, j0, d, quads;
     float alpha, beta;
-    float* Hl; const unsigned* am;
+    float* Hl; const float* scales;           // inverse scales of the tile's rows and columns [2][TM]
     const unsigned long long* err_word; unsigned long long call;
 
+    // rows of `mirror`: this CTA's share
     template <int S, int R, bool SPLIT>
-    __device__ __forceinline__ void finish() const {
-        constexpr int NH = TM / 32, N_ROWS = TM / S, WARPS = THREADS / 32;
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS;
+    __device__ __forceinline__ void rows_of_parts() const {
+        constexpr int N_ROWS = TM / S, WARPS = THREADS / 32;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS, cc = 4 * lane, col = j0 + cc;
+        const float4 scale = SPLIT ? *reinterpret_cast<const float4*>(scales + TM + cc) : make_float4(1.f, 1.f, 1.f, 1.f);
+#pragma unroll 1
+        for (int at = warp * R; at < N_ROWS && i0 + first + at < d; at += WARPS * R) {
+            float4 part[S][R], old[R];
+#pragma unroll
+            for (int p = 0; p < S; ++p) {
+                const float* from = cg::this_cluster().map_shared_rank(out_tile + (first + at) * PART_PITCH + cc, p);
+#pragma unroll
+                for (int k = 0; k < R; ++k) part[p][k] = *reinterpret_cast<const float4*>(from + k * PART_PITCH);
+            }
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int row = i0 + first + at + k, n = beta != 0.f && row < d ? row - col + 1 : 0;
+                const float* o = Hl + (size_t)row * d + col;
+                if (quads && n > 3) old[k] = *reinterpret_cast<const float4*>(o);
+                else old[k] = make_float4(n > 0 ? o[0] : 0.f, n > 1 ? o[1] : 0.f, n > 2 ? o[2] : 0.f, n > 3 ? o[3] : 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int row = i0 + first + at + k, n = row < d ? row - col + 1 : 0;       // entries up to the diagonal
+                float v[4] = {part[0][k].x, part[0][k].y, part[0][k].z, part[0][k].w};
+#pragma unroll
+                for (int p = 1; p < S; ++p) { v[0] += part[p][k].x; v[1] += part[p][k].y; v[2] += part[p][k].z; v[3] += part[p][k].w; }
+                const float o[4] = {old[k].x, old[k].y, old[k].z, old[k].w}, sc[4] = {scale.x, scale.y, scale.z, scale.w};
+                const float mul = SPLIT ? scales[first + at + k] : 1.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    v[e] *= alpha;
+                    if (SPLIT) v[e] = (v[e] * mul) * sc[e];
+                    v[e] += o[e];
+                    mirror[(at + k) * OUT_PITCH + cc + e] = v[e];
+                }
+                float* out = Hl + (size_t)row * d + col;
+                if (quads && n > 3) {
+                    *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (e < n) out[e] = v[e];
+                }
+                if ((row | col) == 0) hessian_check(out, err_word, call);
+            }
+        }
+    }
+
+    template <int R, bool SPLIT>
+    __device__ __forceinline__ void rows_of_tile() const {
+        constexpr int NH = TM / 32, WARPS = THREADS / 32;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         // split route: undo the power-of-two scales of the two feature rows (exact)
         float scale[NH];
 #pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            const int col = j0 + 32 * h + lane;
-            scale[h] = SPLIT && col < d ? row_scale(am[col], true) : 1.f;
-        }
+        for (int h = 0; h < NH; ++h) scale[h] = SPLIT ? scales[TM + 32 * h + lane] : 1.f;
 #pragma unroll 1
-        for (int at = warp * R; at < N_ROWS && i0 + first + at < d; at += WARPS * R) {
-            float part[S][R][NH], old[R][NH], mul[R];
+        for (int at = warp * R; at < TM && i0 + at < d; at += WARPS * R) {
+            float part[R][NH], old[R][NH];
 #pragma unroll
-            for (int p = 0; p < S; ++p) {
-                const float* from = out_tile + (first + at) * OUT_PITCH + lane;
-                if (S > 1) from = cg::this_cluster().map_shared_rank(from, p);
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-#pragma unroll
-                    for (int h = 0; h < NH; ++h) part[p][k][h] = from[k * OUT_PITCH + 32 * h];
-            }
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const int row = i0 + first + at + k;
-                mul[k] = SPLIT && row < d ? row_scale(am[row], true) : 1.f;
+            for (int k = 0; k < R; ++k)
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
-                    const int col = j0 + 32 * h + lane;
+                    const int row = i0 + at + k, col = j0 + 32 * h + lane;
+                    part[k][h] = out_tile[(at + k) * OUT_PITCH + 32 * h + lane];
                     old[k][h] = beta != 0.f && row < d && col <= row ? Hl[(size_t)row * d + col] : 0.f;
                 }
-            }
 #pragma unroll
             for (int k = 0; k < R; ++k) {
-                const int row = i0 + first + at + k;
+                const int row = i0 + at + k;
                 float* out = Hl + (size_t)row * d + j0 + lane;
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
                     const int cc = 32 * h + lane, col = j0 + cc;
-                    float v = part[0][k][h];
-#pragma unroll
-                    for (int p = 1; p < S; ++p) v += part[p][k][h];
                     if (row >= d || col > row) continue;             // (col <= row < d)
-                    v *= alpha;
-                    if (SPLIT) v = (v * mul[k]) * scale[h];
+                    float v = part[k][h] * alpha;
+                    if (SPLIT) v = (v * scales[at + k]) * scale[h];
                     v += old[k][h];
                     out[32 * h] = v;
                     if ((row | col) == 0) hessian_check(out, err_word, call);
@@ -130,6 +166,14 @@ struct TileEnd {
                 }
             }
         }
+    }
+
+    template <int S, int R, bool SPLIT>
+    __device__ __forceinline__ void finish() const {
+        constexpr int N_ROWS = TM / S, WARPS = THREADS / 32;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS;
+        if constexpr (S > 1) rows_of_parts<S, R, SPLIT>();
+        else rows_of_tile<R, SPLIT>();
         __syncthreads();
         // lanes along the rows of this share (32, or all of them where there are fewer), then along columns
         constexpr int LANES = N_ROWS < 32 ? N_ROWS : 32, PER = 32 / LANES, SEG = N_ROWS / LANES, FLY = 8;
@@ -158,7 +202,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
           float* __restrict__ H, int d, int num_kb_all, int n_split, float alpha, float beta, int layer0,
           int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
-          const unsigned* __restrict__ amax) {
+          const unsigned* __restrict__ amax, int quads) {
     using C = Cfg<SPLIT>;
     constexpr int STAGE_BYTES = C::TILES * TILE_BYTES;
     constexpr uint32_t TMEM_COLS = SPLIT ? 512u : 256u;   // main x2 (+ cross terms), power of two
@@ -166,6 +210,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     __shared__ uint64_t bar_full[C::STAGES], bar_empty[C::STAGES], bar_acc_full[2], bar_acc_empty[2], bar_final;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
+    __shared__ __align__(16) float scales[2 * TM];
 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;       // swizzled tiles need 1024-byte alignment
@@ -207,7 +252,11 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
     const uint32_t tmem_base = tmem_base_slot;            // main[0] = +0, main[1] = +128, cross = +256
     volatile int* abortp = &abort_flag;
     float* out_tile = reinterpret_cast<float*>(smem_raw + (tiles - raw));    // [TM][OUT_PITCH], over the ring
-    float* mirror = n_split > 1 ? out_tile + TM * OUT_PITCH : out_tile;      // finished rows of this CTA
+    float* mirror = n_split > 1 ? out_tile + TM * PART_PITCH : out_tile;     // finished rows of this CTA
+    if (SPLIT && threadIdx.x >= THREADS - 2 * TM) {       // the epilogue's threads; read behind the barrier at the end
+        const int e = (int)threadIdx.x - (THREADS - 2 * TM), row = (e < TM ? i0 : j0 - TM) + e;
+        scales[e] = row < d ? row_scale(__ldcg(amax + (size_t)l * d + row), true) : 1.f;
+    }
     bool failed = false;
     int issued = 0;                                       // K blocks whose copies were started (thread 0)
 
@@ -328,8 +377,15 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
             }
             // The operand ring is free (every MMA has completed): the partial tile goes there.
             const int row = q * 32 + lane;
+            if (n_split > 1) {
 #pragma unroll
-            for (int e = 0; e < NC; ++e) out_tile[row * OUT_PITCH + half * NC + e] = tot[e] + acc[e];
+                for (int e = 0; e < NC; e += 4)
+                    *reinterpret_cast<float4*>(out_tile + row * PART_PITCH + half * NC + e) =
+                        make_float4(tot[e] + acc[e], tot[e + 1] + acc[e + 1], tot[e + 2] + acc[e + 2], tot[e + 3] + acc[e + 3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < NC; ++e) out_tile[row * OUT_PITCH + half * NC + e] = tot[e] + acc[e];
+            }
         }
     }
 
@@ -355,8 +411,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
 
     // Every CTA of the cluster finishes its share of the rows.
     float* Hl = H + (size_t)(layer0 + l) * d * d;
-    const unsigned* am = SPLIT ? amax + (size_t)l * d : nullptr;
-    const TileEnd end{out_tile, mirror, rank, i0, j0, d, alpha, beta, Hl, am, err_word, call};
+    const TileEnd end{out_tile, mirror, rank, i0, j0, d, quads, alpha, beta, Hl, scales, err_word, call};
     if (n_split == 1) end.finish<1, 4, SPLIT>();
     else if (n_split == 2) end.finish<2, 4, SPLIT>();
     else if (n_split == 4) end.finish<4, 4, SPLIT>();
@@ -867,9 +922,10 @@ ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_
     const int T = (p.d + TM - 1) / TM;
     const long long tiles = (long long)T * (T + 1) / 2 * p.layers;
     const int split = hessian_tile_split(tiles, p.num_kb);
+    const int quads = p.d % 4 == 0 && reinterpret_cast<uintptr_t>(p.H) % 16 == 0;     // rows of H start on 16 bytes
     constexpr int smem2 = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
     constexpr int smem1 = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
-    static_assert(2 * TM * OUT_PITCH * (int)sizeof(float) + 1024 <= smem1, "finished tiles fit the operand ring");
+    static_assert(TM * (PART_PITCH + OUT_PITCH) * (int)sizeof(float) + 1024 <= smem1, "finished tiles fit the operand ring");
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2));
     ZIPLM_CHECK_CUDA(cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1));
     cudaLaunchConfig_t cfg = {};
@@ -887,7 +943,7 @@ ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_
     cfg.numAttrs = 2;
     ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, p.split ? k_syrk_tc<true> : k_syrk_tc<false>, p.hi,
                                         p.split ? p.lo : p.hi, p.H, p.d, p.num_kb, split, p.alpha, p.beta,
-                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax));
+                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, quads));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }

@@ -934,6 +934,27 @@ def test_hessian_into_a_matrix_that_starts_at_any_element(L, d, N, dtype):
         assert bool(room[:offset].isnan().all()) and bool(room[offset + L * d * d:].isnan().all())
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("L,d,N", [(2, 400, 1000), (3, 400, 600), (2, 398, 1000), (1, 132, 2048)])
+def test_hessian_tiles_shared_by_two_four_and_eight(L, d, N, dtype):
+    """Ends of shared tiles with four columns a lane (width and start of H allow it) and one by one: the same bits, and
+    within the bound of the other widths (fp32 sums of products that fp32 accumulators hold: 2e-6 of the diagonal)."""
+    z = zb()
+    A = torch.randn(L, N, d, generator=torch.Generator().manual_seed(d)).to(dtype).cuda()
+    H = z.hessian_accumulate_tokens(A)
+    H2 = z.hessian_accumulate_tokens(A, H.clone(), beta=1.0)
+    ref = 2.0 * A.double().transpose(1, 2) @ A.double()
+    dia = ref.diagonal(dim1=1, dim2=2)
+    scale = (dia[:, :, None] * dia[:, None, :]).sqrt()
+    assert float(((H.double() - ref) / scale).abs().max()) < 2e-6
+    assert float(((H2.double() - 2 * ref) / scale).abs().max()) < 4e-6
+    room = torch.full((L * d * d + 8,), float("nan"), device="cuda")
+    Hu = room[1:1 + L * d * d].view(L, d, d)
+    assert torch.equal(z.hessian_accumulate_tokens(A, Hu), H)
+    assert torch.equal(z.hessian_accumulate_tokens(A, Hu, beta=1.0), H2)
+    assert bool(room[:1].isnan().all()) and bool(room[1 + L * d * d:].isnan().all())
+
+
 @pytest.mark.parametrize("L,r,d,g,levels", [(2, 70, 256, 64, [4, 3, 1]), (1, 33, 320, 80, [3, 0]), (2, 70, 256, 1, [200, 60]),
                                             (1, 40, 640, 1, [500, 300, 10]), (1, 20, 60, 5, [7, 2])])
 def test_weights_and_snapshots_that_start_at_any_element(L, r, d, g, levels):
