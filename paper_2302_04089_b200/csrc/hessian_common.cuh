@@ -20,8 +20,8 @@ struct HessianProduct {
     bool split;
 };
 
-// Whether the kernel on CTA pairs takes a launch of that many layers.
-bool hessian_pair_fits(int layers, int d, long long N);
+// Whether the kernel on CTA pairs takes a launch of that many layers (split: fp32 input in two parts).
+bool hessian_pair_fits(int layers, int d, long long N, bool split);
 // CTAs that share a 128 x 128 tile of the other one.
 int hessian_tile_split(long long tiles, long long num_kb);
 // Scratch that such a launch uses.

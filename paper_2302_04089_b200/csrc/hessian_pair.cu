@@ -486,14 +486,20 @@ ziplm_status launch_pair(const HessianProduct& p, float4* level2, cudaStream_t s
 }  // namespace
 
 // A K block of a 256 x 256 tile takes a pair about 4/3 of the time that one of a 128 x 128 tile takes a CTA
-// (12 MMAs of 128 clocks against 12 of 92, where the shared-memory reads of a 128 x 128 MMA bound it), so
-// the pair kernel wins where a chain of its K blocks over all waves is shorter than three quarters of the other's.
-bool hessian_pair_fits(int layers, int d, long long N) {
+// (12 MMAs of 128 clocks against 12 of 92, where the shared-memory reads of a 128 x 128 MMA bound it).  The end of a
+// tile of 16-bit input weighs as much as eight of its K blocks, six where a pair has a tile to itself.  The lines lie where
+// the device times of the two kernels' calls cross (us, pairs and CTAs): 1 x 1000 x 4000 27.0 and 34.7, 1 x 1322 x 4099
+// 28.7 and 29.3, 1 x 1700 x 2000 25.5 and 29.4, 1 x 1884 x 15943 123 and 138, 13 x 237 x 4318 45.9 and 47.3;
+// 2 x 1000 x 2000 25.3 and 22.6, 2 x 1400 x 2000 34.5 and 30.8, 2 x 502 x 19169 61.1 and 54.8, 5 x 314 x 750 20.6 and
+// 16.4.  Of fp32 the K blocks alone count: pairs sum it the more exactly (6 x 287 x 843: 1.4e-8 of the diagonal in the
+// mean square against 2.7e-8, 28.2 us against 22.6; 1 x 1000 x 4000: 7e-9 against 15e-9, 41.1 us against 47.3).
+bool hessian_pair_fits(int layers, int d, long long N, bool split) {
     const long long kb = (N + BK - 1) / BK, T = (d + HALF - 1) / HALF, tiles = T * (T + 1) / 2 * layers;
     const long long pairs = (long long)pair_count(d) * layers, parts = parts_of(pairs, kb);
-    const long long split = hessian_tile_split(tiles, kb);
-    const long long chain = (pairs + most_clusters(parts) - 1) / most_clusters(parts) * ((kb + parts - 1) / parts);
-    return 4 * chain < 3 * ((tiles * split + kSMs - 1) / kSMs * ((kb + split - 1) / split));
+    const long long share = hessian_tile_split(tiles, kb);
+    const long long end = split ? 0 : parts > 1 ? 8 : 6, other_end = split ? 0 : 8;
+    const long long cost = (pairs + most_clusters(parts) - 1) / most_clusters(parts) * ((kb + parts - 1) / parts + end);
+    return 4 * cost < 3 * ((tiles * share + kSMs - 1) / kSMs * ((kb + share - 1) / share + other_end));
 }
 
 // Scratch of the second summation level, for the layers of one launch; none where FOLD drains are

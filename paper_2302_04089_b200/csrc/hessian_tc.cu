@@ -875,7 +875,7 @@ size_t product_scratch_bytes(int L, int d, long long N, ziplm_dtype dt, bool tok
     const int full = product_layers(L, d, N, dt, token_major), last = L % full;
     size_t b = 0;
     for (int layers : {full, last})
-        if (layers > 0 && hessian_pair_fits(layers, d, N)) {
+        if (layers > 0 && hessian_pair_fits(layers, d, N, dt == ZIPLM_F32)) {
             const size_t need = hessian_pair_scratch_bytes(layers, d, N, dt == ZIPLM_F32);
             if (need > b) b = need;
         }
@@ -886,10 +886,13 @@ size_t product_scratch_bytes(int L, int d, long long N, ziplm_dtype dt, bool tok
 
 // Where the 128 x 128 tiles leave half of the SMs idle, up to eight CTAs share a tile: the largest power of
 // two with which all fit and each keeps four K blocks (one layer of 256 features, 2048 tokens: three tiles,
-// a chain of 32 K blocks on one CTA).
+// a chain of 32 K blocks on one CTA).  `most`: the occupancy calculator's room for clusters of 2, 4 and 8 CTAs on the
+// kSMs of a B200, whose GPCs differ in size: what does not fit would wait for a second round (18 tiles of
+// 3 x 333 x 2276 bf16 on clusters of eight 26.5 us, of four 20.3; 12 x 198 x 2221 on four 29.4, on two 24.2).
 int hessian_tile_split(long long tiles, long long num_kb) {
+    constexpr int most[9] = {0, kSMs, kSMs / 2, 0, 33, 0, 0, 0, 15};
     int split = 1;
-    while (split < 8 && tiles * split * 2 <= kSMs && num_kb / (split * 2) >= 4) split *= 2;
+    while (split < 8 && tiles <= most[split * 2] && num_kb / (split * 2) >= 4) split *= 2;
     return split;
 }
 
@@ -917,7 +920,7 @@ unsigned long long next_call() {
 
 // One product launch on the kernel that suits its number of tiles.
 ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_bytes, cudaStream_t st) {
-    if (hessian_pair_fits(p.layers, p.d, (long long)p.num_kb * 64))
+    if (hessian_pair_fits(p.layers, p.d, (long long)p.num_kb * 64, p.split))
         return run_hessian_pair(p, scratch, scratch_bytes, st);
     const int T = (p.d + TM - 1) / TM;
     const long long tiles = (long long)T * (T + 1) / 2 * p.layers;

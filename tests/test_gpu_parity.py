@@ -955,6 +955,22 @@ def test_hessian_tiles_shared_by_two_four_and_eight(L, d, N, dtype):
     assert bool(room[:1].isnan().all()) and bool(room[1 + L * d * d:].isnan().all())
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("L,d,N", [(1, 1001, 3999), (13, 237, 4318), (7, 482, 4859), (6, 287, 843), (18, 96, 9001), (3, 333, 2276),
+                                   (1, 1700, 2000), (12, 198, 2221)])
+def test_hessian_on_both_sides_of_the_line_between_its_kernels(L, d, N, dtype):
+    """Calls next to where pairs of CTAs take over from clusters, and clusters of eight from four from two: the bound of
+    the other widths (fp32 sums of products that fp32 accumulators hold: 2e-6 of the diagonal)."""
+    z = zb()
+    A = torch.randn(L, N, d, generator=torch.Generator().manual_seed(N)).to(dtype).cuda()
+    H = z.hessian_accumulate_tokens(A)
+    for l in range(L):
+        ref = 2.0 * A[l].double().T @ A[l].double()
+        scale = (ref.diagonal()[:, None] * ref.diagonal()[None, :]).sqrt()
+        assert float(((H[l].double() - ref) / scale).abs().max()) < 2e-6
+        assert torch.equal(H[l], H[l].T)
+
+
 @pytest.mark.parametrize("L,r,d,g,levels", [(2, 70, 256, 64, [4, 3, 1]), (1, 33, 320, 80, [3, 0]), (2, 70, 256, 1, [200, 60]),
                                             (1, 40, 640, 1, [500, 300, 10]), (1, 20, 60, 5, [7, 2])])
 def test_weights_and_snapshots_that_start_at_any_element(L, r, d, g, levels):
