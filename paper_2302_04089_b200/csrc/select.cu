@@ -199,15 +199,21 @@ __device__ __forceinline__ void dp_row(int f0, int f1, int cost, int no, int lo,
         for (int r = 0; r < R; ++r) {
             if (r > 0 && r * 32 >= no) break;
             unsigned left = __ballot_sync(0xffffffffu, low[r] <= bound);
-            while (left) {
-                const int s = r * 32 + __ffs(left) - 1;
-                left &= left - 1;
-                const double2 t = table[s];
-                const int i = b0 + lane - __double2loint(t.y);
-                const double v0 = sel_smem[f0 + max(min(i, hi_prev), -1)] + t.x;
-                const double v1 = sel_smem[f0 + max(min(i + 32, hi_prev), -1)] + t.x;
-                if (v0 < best0) { best0 = v0; arg0 = s; }
-                if (v1 < best1) { best1 = v1; arg1 = s; }
+            if (left) {       // the next option's pair is requested while this one is tested (1024 candidates: 751 -> 741 us)
+                int s = r * 32 + __ffs(left) - 1;
+                double2 t = table[s];
+                for (;;) {
+                    left &= left - 1;
+                    const int q = left ? r * 32 + __ffs(left) - 1 : s;
+                    const double2 x = table[q];
+                    const int i = b0 + lane - __double2loint(t.y);
+                    const double v0 = sel_smem[f0 + max(min(i, hi_prev), -1)] + t.x;
+                    const double v1 = sel_smem[f0 + max(min(i + 32, hi_prev), -1)] + t.x;
+                    if (v0 < best0) { best0 = v0; arg0 = s; }
+                    if (v1 < best1) { best1 = v1; arg1 = s; }
+                    if (!left) break;
+                    s = q; t = x;
+                }
             }
         }
         const int b = b0 + lane;
