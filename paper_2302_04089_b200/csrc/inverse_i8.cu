@@ -14,10 +14,11 @@
 // of tensor memory), first the digits 4 .. 7 (10 products), then all (26).  A K block is 64 digits (64-byte
 // swizzle): eight slices of both operands fill half of the shared-memory ring, 96 KB for 3328 clocks of
 // MMAs, so the operand traffic stays at 30 bytes per clock and SM.
-// Inverse of 12 x 3072: 14.7 -> 9.7 ms, of 24 x 4096: 57 -> 33.6 ms (float64 instruction before).  The tensor
-// pipe bounds it: an MMA of M = 256, N = 128, K = 32 takes 96 clocks in place of 64 (6900 clocks a K block).
-// Tiles of 256 x 256 (163 clocks an MMA in place of 128, a quarter of the drains four times as often through
-// scratch) were slower, 128-byte swizzled rows of two digits the same.
+// Inverse of 12 x 3072: 14.7 -> 8.8 ms, of 24 x 4096: 57 -> 31 ms (float64 instruction before).  The tensor
+// pipe bounds it: an MMA of M = 256, N = 128, K = 32 takes some 92 clocks in place of 64.  Neither an operand kept in
+// the collector for up to four MMAs nor a ring of 16 single slices (12 of them in flight) changes that; tiles of
+// 256 x 256 (163 clocks an MMA in place of 128, a quarter of the drains four times as often through scratch) were
+// slower, 128-byte swizzled rows of two digits the same.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -179,6 +180,22 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
                  : "r"(taddr) : "memory");
 }
 
+// The MMAs of a K block in one pass: products of weight 256^t, t = qa + qb from T0 to T0 + 3, each weight with an
+// accumulator of its own.  Unrolled, so that the one issuing thread adds constants only (with its descriptors' arithmetic
+// between the MMAs M^T M of 12 x 3072 took 2.19 ms, now 2.08).
+template <int T0>
+__device__ __forceinline__ void issue_block(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, bool add) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int qa = T0 + c - 7; qa <= 7; ++qa)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                umma_i8_pair(tmem + (uint32_t)(c * PN), a + (uint32_t)(qa * (A_BYTES / 16) + 2 * h),
+                             b + (uint32_t)((T0 + c - qa) * (B_BYTES / 16) + 2 * h), idesc,
+                             add || h || qa > T0 + c - 7 ? 1u : 0u);
+}
+
 __global__ void __launch_bounds__(I8_THREADS, 1) __cluster_dims__(2, 1, 1)
 k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
              const __grid_constant__ I8Product p) {
@@ -279,17 +296,8 @@ k_i8_product(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ 
                     if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { failed = true; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t a = a0 + (uint32_t)(s * (STAGE / 16)), b = b0 + (uint32_t)(s * (STAGE / 16));
-                    // weight 256^t, t = qa + qb: pass 0 t = 11 .. 14, pass 1 t = 7 .. 10; accumulator t - first
-                    const int t0 = pass ? 7 : 11;
-                    for (int c = 0; c < 4; ++c) {
-                        const int t = t0 + c, lo = t - 7;
-                        const uint32_t acc = tmem_base + (uint32_t)(c * PN);
-                        for (int qa = lo; qa <= 7; ++qa) {
-                            const uint64_t da = a + (uint32_t)(qa * (A_BYTES / 16)), db = b + (uint32_t)((t - qa) * (B_BYTES / 16));
-                            umma_i8_pair(acc, da, db, idesc, (kb | (qa - lo)) ? 1u : 0u);
-                            umma_i8_pair(acc, da + 2u, db + 2u, idesc, 1u);
-                        }
-                    }
+                    if (pass) issue_block<7>(tmem_base, a, b, idesc, kb > 0);
+                    else issue_block<11>(tmem_base, a, b, idesc, kb > 0);
                     umma_commit_pair(smem_u32(&bar_empty[s]), both);
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
