@@ -439,28 +439,39 @@ __global__ void __launch_bounds__(256) k_row_absmax(const float* __restrict__ X,
     }
 }
 
-// The same for token-major input A [layers, N, lda] (one token per row): every thread walks one
-// feature over a slab of tokens, the slabs meet through atomicMax (amax zeroed beforehand).
+// The same for token-major input A [layers, N, lda] (one token per row): a CTA takes 32 features of a slab of tokens, a
+// warp 32 tokens of them in a turn with all reads in flight; the slabs meet through atomicMax (amax zeroed beforehand).
+// Bound by memory: 6 x 7265 x 317 24.0 -> 16.5 us, 1 x 7232 x 2376 23.9 -> 19.9 (a thread to a feature and
+// one read after the other before).
+constexpr int AM_TOKENS = 32;                    // of a warp in a turn
 __global__ void __launch_bounds__(256) k_tokens_absmax(const float* __restrict__ A, long long lda,
                                                        long long N, int d, long long slab,
                                                        unsigned* __restrict__ amax) {
-    const int l = blockIdx.z;
-    const int f = blockIdx.x * 256 + threadIdx.x;
-    if (f >= d) return;
-    const long long t0 = (long long)blockIdx.y * slab, t1 = min(N, t0 + slab);
-    const float* Al = A + (size_t)l * (size_t)N * (size_t)lda + f;
+    __shared__ unsigned red[8][32];
+    const int l = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int f = blockIdx.x * 32 + lane;
+    const long long t1 = min(N, (long long)(blockIdx.y + 1) * slab);
     unsigned m = 0u;
-    for (long long t = t0; t < t1; ++t) m = max(m, __float_as_uint(Al[(size_t)t * (size_t)lda]) & 0x7fffffffu);
+    for (long long t = (long long)blockIdx.y * slab + warp * AM_TOKENS; t < t1; t += 8 * AM_TOKENS) {
+        const float* src = A + ((size_t)l * (size_t)N + (size_t)t) * (size_t)lda + min(f, d - 1);
+        const int last = (int)min((long long)AM_TOKENS, t1 - t) - 1;         // (read again past the end: no branches)
+        unsigned v[AM_TOKENS];
+#pragma unroll
+        for (int k = 0; k < AM_TOKENS; ++k)
+            v[k] = __float_as_uint(src[(size_t)min(k, last) * (size_t)lda]) & 0x7fffffffu;
+#pragma unroll
+        for (int k = 0; k < AM_TOKENS; ++k) m = max(m, v[k]);
+    }
+    red[warp][lane] = m;
+    __syncthreads();
+    if (warp || f >= d) return;
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
     atomicMax(amax + (size_t)l * d + f, m);
 }
 
-// The two fp16 parts of a scaled fp32 value y: y_1 = fp16(y), y_2 = fp16(y - y_1) (the difference
-// is exact in fp32).
-__device__ __forceinline__ void split_f16x2(float y, __half& p1, __half& p2) {
-    p1 = __float2half_rn(y);
-    p2 = __float2half_rn(y - __half2float(p1));
-}
-// Of four values at once, by packed conversions.
+// The two fp16 parts of four scaled fp32 values: y_1 = fp16(y), y_2 = fp16(y - y_1) (the difference is exact in fp32),
+// by packed conversions.
 __device__ __forceinline__ void split_f16x2(const float (&y)[4], uint2& p1, uint2& p2) {
     union { uint2 v; __half2 e[2]; } a, b;
 #pragma unroll
@@ -547,51 +558,15 @@ __global__ void __launch_bounds__(256) k_row_absmax_split(const float* __restric
     }
 }
 
-// Token-major input (one calibration token per row, as a forward pass emits activations):
-// A is [layers, N, lda] with the feature index contiguous.  A 32 x 32 tile goes through shared
-// memory, so the reads run along features and the writes along tokens, both coalesced; the output
-// is the K-major [layers * d, np] matrix the product kernel loads.  SPLIT writes the scaled fp16
-// parts X_1 / X_2 of an fp32 input directly (same values as k_split_f16; O = __half, amax holds
-// the features' largest magnitudes); otherwise the elements are moved as raw bits (T = O =
-// uint16_t for bf16 and fp16).
-template <typename T, typename O, bool SPLIT>
-__global__ void __launch_bounds__(256) k_tokens_to_kmajor(const T* __restrict__ A, long long lda,
-                                                          long long N, int d, long long np,
-                                                          const unsigned* __restrict__ amax,
-                                                          O* __restrict__ hi, O* __restrict__ lo) {
-    grid_trigger();
-    __shared__ T tile[32][33];
-    const int l = blockIdx.z;
-    const long long t0 = (long long)blockIdx.x * 32;
-    const int f0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const T* Al = A + (size_t)l * (size_t)N * (size_t)lda;
-#pragma unroll
-    for (int r = ty; r < 32; r += 8) {
-        const long long t = t0 + r;
-        const int f = f0 + tx;
-        tile[r][tx] = (t < N && f < d) ? Al[(size_t)t * (size_t)lda + f] : T(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = ty; r < 32; r += 8) {
-        const int f = f0 + r;
-        const long long t = t0 + tx;
-        if (f >= d || t >= np) continue;
-        const size_t o = ((size_t)l * d + f) * (size_t)np + (size_t)t;
-        const T v = tile[tx][r];
-        if constexpr (SPLIT) {
-            split_f16x2(v * row_scale(amax[(size_t)l * d + f], false), hi[o], lo[o]);
-        } else {
-            hi[o] = v;
-        }
-    }
-}
-
-// The same move of split fp32 for inputs whose rows allow 16-byte accesses (A aligned, lda % 4 == 0): a
-// 64 x 64 tile, four elements per access on both sides.  np is a multiple of 8, so a quad that starts below
-// np ends below it.
-__global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const float* __restrict__ A, long long lda, long long N,
+// Token-major fp32 input (one calibration token per row, as a forward pass emits activations): A is [layers, N, lda]
+// with the feature index contiguous.  A 64 x 64 tile goes through shared memory, so the reads run along features and
+// the writes along tokens, both coalesced; the scaled fp16 parts X_1 / X_2 leave in the K-major [layers * d, np]
+// matrices that the product kernel loads (same values as k_split_f16; amax holds the features' largest magnitudes).
+// QUADS: rows of A start on 16 bytes (A aligned, lda % 4 == 0); otherwise a warp reads 32 neighbouring features,
+// sixteen tokens a thread in flight.  np is a multiple of 8, so a quad that starts below np ends below it.
+// Bound by memory: 6 x 7265 x 320 20 us, x 317 35.3 -> 19.3 (32 x 32 tiles, entries one by one before).
+template <bool QUADS>
+__global__ void __launch_bounds__(256) k_tokens_to_kmajor(const float* __restrict__ A, long long lda, long long N,
                                                              int d, long long np, const unsigned* __restrict__ amax,
                                                              __half* __restrict__ hi, __half* __restrict__ lo) {
     grid_trigger();
@@ -601,21 +576,32 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const float* __rest
     const int f0 = blockIdx.y * 64;
     const int q = threadIdx.x & 15, rr = threadIdx.x >> 4;
     const float* Al = A + (size_t)l * (size_t)N * (size_t)lda;
+    if (QUADS) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int tl = rr + 16 * k;
-        const long long t = t0 + tl;
-        const int f = f0 + 4 * q;
-        float u[4];
-        if (t < N && f + 3 < d) {
-            const float4 x = *reinterpret_cast<const float4*>(Al + (size_t)t * (size_t)lda + f);
-            u[0] = x.x; u[1] = x.y; u[2] = x.z; u[3] = x.w;
-        } else {
+        for (int k = 0; k < 4; ++k) {
+            const int tl = rr + 16 * k;
+            const long long t = t0 + tl;
+            const int f = f0 + 4 * q;
+            float u[4];
+            if (t < N && f + 3 < d) {
+                const float4 x = *reinterpret_cast<const float4*>(Al + (size_t)t * (size_t)lda + f);
+                u[0] = x.x; u[1] = x.y; u[2] = x.z; u[3] = x.w;
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) u[e] = (t < N && f + e < d) ? Al[(size_t)t * (size_t)lda + f + e] : 0.f;
+                for (int e = 0; e < 4; ++e) u[e] = (t < N && f + e < d) ? Al[(size_t)t * (size_t)lda + f + e] : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) tile[tl][4 * q + e] = u[e];
         }
+    } else {
+        const int fl = threadIdx.x & 63, r0 = threadIdx.x >> 6;
+        const float* src = Al + ((size_t)t0 + r0) * (size_t)lda + f0 + fl;
+        float u[16];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) tile[tl][4 * q + e] = u[e];
+        for (int k = 0; k < 16; ++k, src += 4 * (size_t)lda)
+            u[k] = t0 + r0 + 4 * k < N && f0 + fl < d ? *src : 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) tile[r0 + 4 * k][fl] = u[k];
     }
     __syncthreads();
 #pragma unroll
@@ -633,39 +619,63 @@ __global__ void __launch_bounds__(256) k_tokens_to_kmajor_v4(const float* __rest
     }
 }
 
-// The same move of 16-bit elements whose rows start on 4 bytes (lda even), pairs of features at a time: 128
-// tokens x 64 features, 16 loads in flight per thread (a warp reads 128 bytes of a row), and eight tokens of
+// The same move of 16-bit elements (raw bits of bf16 or fp16), pairs of features at a time: 128 tokens x 64
+// features, 16 loads in flight per thread (a warp reads 128 bytes of a row; PAIRS: rows start on 4 bytes, lda
+// even, otherwise a pair is two loads), and eight tokens of
 // two features per thread put together from eight words, so that 256 bytes of a feature leave together.  The
 // words of a token lie permuted by the group of eight tokens: no bank conflicts on either side.
-// 4099 x 1322: 10.7 -> 6.7 us (32 x 32 elements one by one before).
+// 4099 x 1322: 10.7 -> 6.7 us, 19 x 2186 x 1203 79.6 -> 46 (32 x 32 elements one by one before).
+// TOKENS of a tile: 128, or 32 without PAIRS where tiles of 128 leave SMs idle and the chain of a thread's loads is what
+// counts (a call 1 x 700 x 513 18.2 -> 16.6 us, 2 x 2402 x 89 16.0 -> 14.6; with PAIRS 1 x 600 x 1322 16.7 -> 17.9).
+template <bool PAIRS, int TOKENS>
 __global__ void __launch_bounds__(256) k_tokens16_to_kmajor(const uint16_t* __restrict__ A, long long lda, long long N,
                                                             int d, long long np, uint16_t* __restrict__ out) {
     grid_trigger();
-    __shared__ uint32_t tile[128 * 32];
+    constexpr int GROUPS = TOKENS / 8;                   // of eight tokens; a thread reads a token of each
+    constexpr int SHIFT = TOKENS == 128 ? 0 : 3;         // place of word w in group k: w ^ (k << SHIFT)
+    static_assert(TOKENS == 128 || TOKENS == 32, "the places below are worked out for these");
+    __shared__ uint32_t tile[TOKENS * 32];
     const int l = blockIdx.z, f0 = blockIdx.y * 64, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long t0 = (long long)blockIdx.x * 128;
+    const long long t0 = (long long)blockIdx.x * TOKENS;
     {
         const int f = f0 + 2 * lane;
-        const uint16_t* src = A + ((size_t)l * (size_t)N + (size_t)t0 + warp) * (size_t)lda + f;
-        uint32_t v[16];
+        const long long left = N - 1 - t0;               // tokens behind the tile's first, which is below N
+        const uint16_t* src = A + ((size_t)l * (size_t)N + (size_t)t0) * (size_t)lda;
+        uint32_t v[GROUPS];
+        if (PAIRS) {
+            src += warp * (size_t)lda + f;
 #pragma unroll
-        for (int k = 0; k < 16; ++k, src += 8 * (size_t)lda) {
-            v[k] = 0u;
-            if (t0 + warp + 8 * k < N && f < d)
-                v[k] = f + 1 < d ? *reinterpret_cast<const uint32_t*>(src) : (uint32_t)*src;
+            for (int k = 0; k < GROUPS; ++k, src += 8 * (size_t)lda) {
+                v[k] = 0u;
+                if (warp + 8 * k <= left && f < d)
+                    v[k] = f + 1 < d ? *reinterpret_cast<const uint32_t*>(src) : (uint32_t)*src;
+            }
+        } else {                                         // (read again past the ends: no branches around the loads)
+            const int c0 = min(f, d - 1), c1 = min(f + 1, d - 1);
+            uint16_t x0[GROUPS], x1[GROUPS];
+#pragma unroll
+            for (int k = 0; k < GROUPS; ++k) {
+                const uint16_t* row = src + (size_t)min((long long)(warp + 8 * k), left) * (size_t)lda;
+                x0[k] = row[c0];
+                x1[k] = row[c1];
+            }
+#pragma unroll
+            for (int k = 0; k < GROUPS; ++k)
+                v[k] = warp + 8 * k > left || f >= d ? 0u : x0[k] | (f + 1 < d ? (uint32_t)x1[k] << 16 : 0u);
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) tile[(warp + 8 * k) * 32 + (lane ^ k)] = v[k];
+        for (int k = 0; k < GROUPS; ++k) tile[(warp + 8 * k) * 32 + (lane ^ (k << SHIFT))] = v[k];
     }
     __syncthreads();
-    const int tg = threadIdx.x & 15;
+    const int tg = threadIdx.x & (GROUPS - 1);
     const long long t = t0 + 8 * tg;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int w = warp + 8 * h + 16 * (lane >> 4), f = f0 + 2 * w;
+    for (int h = 0; h < (TOKENS == 128 ? 2 : 1); ++h) {
+        const int w = TOKENS == 128 ? warp + 8 * h + 16 * (lane >> 4) : threadIdx.x / GROUPS, f = f0 + 2 * w;
+        if (w >= 32) break;
         uint32_t x[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = tile[(8 * tg + k) * 32 + (w ^ tg)];
+        for (int k = 0; k < 8; ++k) x[k] = tile[(8 * tg + k) * 32 + (w ^ (tg << SHIFT))];
         if (t >= np || f >= d) continue;
         uint16_t* o = out + ((size_t)l * d + f) * (size_t)np + (size_t)t;
         *reinterpret_cast<uint4*>(o) = make_uint4(__byte_perm(x[0], x[1], 0x5410), __byte_perm(x[2], x[3], 0x5410),
@@ -1003,20 +1013,14 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                         if (s != ZIPLM_OK) return s;
                         continue;
                     }
-                    k_tokens_absmax<<<dim3((unsigned)((d + 255) / 256), (unsigned)((N + slab - 1) / slab),
+                    k_tokens_absmax<<<dim3((unsigned)((d + 31) / 32), (unsigned)((N + slab - 1) / slab),
                                            (unsigned)zn), 256, 0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, slab,
                                                                         amax + (size_t)z0 * d);
                     ZIPLM_CHECK_LAUNCH();
-                    if (quad_rows(X, ldx))
-                        k_tokens_to_kmajor_v4
-                            <<<dim3((unsigned)((np + 63) / 64), (unsigned)((d + 63) / 64), (unsigned)zn), 256,
-                               0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, np, amax + (size_t)z0 * d,
-                                        hi + (size_t)z0 * d * np, lo + (size_t)z0 * d * np);
-                    else
-                        k_tokens_to_kmajor<float, __half, true>
-                            <<<dim3((unsigned)((np + 31) / 32), (unsigned)((d + 31) / 32), (unsigned)zn), 256,
-                               0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, np, amax + (size_t)z0 * d,
-                                        hi + (size_t)z0 * d * np, lo + (size_t)z0 * d * np);
+                    auto move = quad_rows(X, ldx) ? k_tokens_to_kmajor<true> : k_tokens_to_kmajor<false>;
+                    move<<<dim3((unsigned)((np + 63) / 64), (unsigned)((d + 63) / 64), (unsigned)zn), 256, 0, st>>>(
+                        Ac + (size_t)z0 * N * ldx, ldx, N, d, np, amax + (size_t)z0 * d, hi + (size_t)z0 * d * np,
+                        lo + (size_t)z0 * d * np);
                     ZIPLM_CHECK_LAUNCH();
                 }
             } else {
@@ -1067,13 +1071,13 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
         for (int l0 = 0; l0 < L; l0 += lc) {
             const int ln = (L - l0 < lc) ? (L - l0) : lc;
             const uint16_t* Ac = static_cast<const uint16_t*>(X) + (size_t)l0 * (size_t)N * ldx;
-            if (ldx % 2 == 0 && reinterpret_cast<uintptr_t>(X) % 4 == 0)
-                k_tokens16_to_kmajor<<<dim3((unsigned)((np + 127) / 128), (unsigned)((d + 63) / 64), (unsigned)ln), 256, 0,
-                                       st>>>(Ac, ldx, N, d, np, xt);
-            else
-                k_tokens_to_kmajor<uint16_t, uint16_t, false>
-                    <<<dim3((unsigned)((np + 31) / 32), (unsigned)((d + 31) / 32), (unsigned)ln), 256, 0, st>>>(
-                        Ac, ldx, N, d, np, nullptr, xt, nullptr);
+            const bool pairs = ldx % 2 == 0 && reinterpret_cast<uintptr_t>(X) % 4 == 0;
+            const bool small = !pairs && (np + 127) / 128 * ((d + 63) / 64) * ln < kSMs;
+            auto move = pairs ? k_tokens16_to_kmajor<true, 128>
+                              : small ? k_tokens16_to_kmajor<false, 32> : k_tokens16_to_kmajor<false, 128>;
+            const int tokens = small ? 32 : 128;
+            move<<<dim3((unsigned)((np + tokens - 1) / tokens), (unsigned)((d + 63) / 64), (unsigned)ln), 256, 0, st>>>(
+                Ac, ldx, N, d, np, xt);
             ZIPLM_CHECK_LAUNCH();
             if (!make_map(&prod.hi, xt, dt, N, d, ln, np)) return ZIPLM_ERR_CUDA;
             prod.lo = prod.hi; prod.layer0 = l0; prod.layers = ln;

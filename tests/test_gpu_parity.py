@@ -901,6 +901,27 @@ def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
     assert torch.equal(H.double(), ref)
 
 
+@pytest.mark.parametrize("N,d,pad,dtype", [(32, 65, 0, torch.bfloat16), (127, 63, 0, torch.float16), (129, 129, 2, torch.bfloat16),
+                                           (1025, 1, 0, torch.float16), (200, 64, 1, torch.float16),
+                                           (6145, 31, 0, torch.float32), (6401, 64, 0, torch.float32),
+                                           (6463, 65, 2, torch.float32), (7265, 130, 2, torch.float32)])
+def test_tokens_in_rows_of_any_pitch(N, d, pad, dtype):
+    """The moves of token-major activations whose rows start on their elements only, and of fp32 batches too long for
+    one pass, at the edges of their tiles and slabs; small whole numbers (times a power of two per feature in
+    fp32, so that a wrong largest magnitude overflows the fp16 parts), so that the product is exact."""
+    z = zb()
+    g = torch.Generator().manual_seed(N)
+    full = torch.randint(-3, 4, (2, N, d + pad), generator=g).to(dtype)
+    if dtype == torch.float32:
+        full[:, -1, :] = 7.0                     # the largest stands in the last token
+        full *= 2.0 ** (torch.arange(d + pad) % 30)
+    A = full.cuda()[:, :, :d]
+    H = z.hessian_accumulate_tokens(A, alpha=2.0)
+    ref = 2.0 * A.double().transpose(1, 2) @ A.double()
+    torch.cuda.synchronize()
+    assert torch.equal(H.double(), ref)
+
+
 @pytest.mark.parametrize("L,d,N", [(1, 1322, 1100), (1, 2100, 1024), (1, 1700, 700), (15, 256, 1030), (1, 2817, 4100),
                                    (1, 3072, 4100), (1, 1700, 8300), (15, 256, 8300)])
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
