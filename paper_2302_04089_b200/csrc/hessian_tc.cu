@@ -439,34 +439,30 @@ __global__ void __launch_bounds__(256) k_row_absmax(const float* __restrict__ X,
     }
 }
 
-// The same for token-major input A [layers, N, lda] (one token per row): a CTA takes 32 features of a slab of tokens, a
-// warp 32 tokens of them in a turn with all reads in flight; the slabs meet through atomicMax (amax zeroed beforehand).
-// Bound by memory: 6 x 7265 x 317 24.0 -> 16.5 us, 1 x 7232 x 2376 23.9 -> 19.9 (a thread to a feature and
-// one read after the other before).
-constexpr int AM_TOKENS = 32;                    // of a warp in a turn
+// The same for token-major input A [layers, N, lda] (one token per row): every thread walks one feature over a slab of
+// tokens with AM_FLY reads in flight, the slabs meet through atomicMax (amax zeroed beforehand).  Slabs are as short
+// as it takes to fill the SMs, and no longer than 256 tokens: 6 x 7265 x 317 23.2 -> 14.0 us, 1 x 9000 x 65 19.1 -> 4.8
+// (slabs of 256 always, four reads in flight); 12 x 16384 x 768 as before, 95 us (6.4 TB/s): without branches and with
+// indexes held at the edge 119, a warp to 32 features with 32 tokens in flight 140.
+constexpr int AM_FLY = 16, AM_SLAB = 256;
 __global__ void __launch_bounds__(256) k_tokens_absmax(const float* __restrict__ A, long long lda,
                                                        long long N, int d, long long slab,
                                                        unsigned* __restrict__ amax) {
-    __shared__ unsigned red[8][32];
-    const int l = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int f = blockIdx.x * 32 + lane;
-    const long long t1 = min(N, (long long)(blockIdx.y + 1) * slab);
+    const int l = blockIdx.z;
+    const int f = blockIdx.x * 256 + threadIdx.x;
+    if (f >= d) return;
+    const long long t0 = (long long)blockIdx.y * slab, t1 = min(N, t0 + slab);
     unsigned m = 0u;
-    for (long long t = (long long)blockIdx.y * slab + warp * AM_TOKENS; t < t1; t += 8 * AM_TOKENS) {
-        const float* src = A + ((size_t)l * (size_t)N + (size_t)t) * (size_t)lda + min(f, d - 1);
-        const int last = (int)min((long long)AM_TOKENS, t1 - t) - 1;         // (read again past the end: no branches)
-        unsigned v[AM_TOKENS];
+    const float* src = A + ((size_t)l * (size_t)N + (size_t)t0) * (size_t)lda + f;
+    long long t = t0;
+    for (; t + AM_FLY <= t1; t += AM_FLY) {
+        unsigned v[AM_FLY];
 #pragma unroll
-        for (int k = 0; k < AM_TOKENS; ++k)
-            v[k] = __float_as_uint(src[(size_t)min(k, last) * (size_t)lda]) & 0x7fffffffu;
+        for (int k = 0; k < AM_FLY; ++k, src += lda) v[k] = __float_as_uint(*src) & 0x7fffffffu;
 #pragma unroll
-        for (int k = 0; k < AM_TOKENS; ++k) m = max(m, v[k]);
+        for (int k = 0; k < AM_FLY; ++k) m = max(m, v[k]);
     }
-    red[warp][lane] = m;
-    __syncthreads();
-    if (warp || f >= d) return;
-#pragma unroll
-    for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
+    for (; t < t1; ++t, src += lda) m = max(m, __float_as_uint(*src) & 0x7fffffffu);
     atomicMax(amax + (size_t)l * d + f, m);
 }
 
@@ -1001,8 +997,11 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                 const float* Ac = static_cast<const float*>(X) + (size_t)l0 * (size_t)N * ldx;
                 const bool one_pass = np <= 8ll * TS_TOKENS;
                 if (!one_pass) ZIPLM_CHECK_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned) * rows, st));
-                // slabs of at least 256 tokens, at most 65535 of them (grid.y)
-                const long long slab = N / 65535 + 1 > 256 ? N / 65535 + 1 : 256;
+                // slabs of AM_SLAB tokens, shorter ones where those would leave SMs idle, at most 65535 of them (grid.y)
+                const long long columns = (long long)((d + 255) / 256) * ln;
+                long long slab = (N * columns / (8 * kSMs) + AM_FLY) / AM_FLY * AM_FLY;
+                if (slab > AM_SLAB) slab = AM_SLAB;
+                if (slab < N / 65535 + 1) slab = N / 65535 + 1;
                 // grid.z is limited to 65535 layers per launch
                 for (int z0 = 0; z0 < ln; z0 += 65535) {
                     const int zn = ln - z0 < 65535 ? ln - z0 : 65535;
@@ -1013,7 +1012,7 @@ ziplm_status run_hessian_tc(float* H, const void* X, ziplm_dtype dt, bool token_
                         if (s != ZIPLM_OK) return s;
                         continue;
                     }
-                    k_tokens_absmax<<<dim3((unsigned)((d + 31) / 32), (unsigned)((N + slab - 1) / slab),
+                    k_tokens_absmax<<<dim3((unsigned)((d + 255) / 256), (unsigned)((N + slab - 1) / slab),
                                            (unsigned)zn), 256, 0, st>>>(Ac + (size_t)z0 * N * ldx, ldx, N, d, slab,
                                                                         amax + (size_t)z0 * d);
                     ZIPLM_CHECK_LAUNCH();
