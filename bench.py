@@ -167,29 +167,39 @@ class ClockSampler:
 # ------------------------------------------------------------------------------------------
 # CUDA leg
 # ------------------------------------------------------------------------------------------
-LAZY_BLOCK = 32   # steps per block of the delayed-update neuron path (BMAX in prune_lazy.cu)
+LAZY_BLOCK = 32   # steps per group of a block of the delayed-update neuron path (GS in prune_lazy.cu)
 LAZY_ENDGAME = 256  # survivors that go to the float64 endgame (kEndgame there) ...
 LAZY_ENDGAME_MIN = LAZY_ENDGAME - 2 * LAZY_BLOCK    # ... when at most this many are to remain
-LAZY_DEAD_MAX, LAZY_DEAD_FRACTION = 128, 16   # its rule for squeezing removed positions out (kDeadMax, kDeadFraction)
+LAZY_DEAD_MAX, LAZY_DEAD_FRACTION = 320, 8   # its rule for squeezing removed positions out (kDeadMax, kDeadFraction)
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch: constants from earlier
 # ncu captures of these kernels (taken on 4 of the 12 layers and scaled by 3: traffic grows in
 # proportion to the layers), not measurements of this run.  Only valid for the bench workload.
 NCU_TRAFFIC = {
-    # k_lazy_update_aq_tc, first block at full size (12 layers, 3072 positions of which 3040 live)
-    "k_lazy_update_aq_tc": dict(bytes=3 * (210.1e6 + 291.3e6), launch="n_pos = 3072, m = 32, 12 layers",
-                                algorithmic=12 * (24.0 * 3040 * 3039 / 2 + 8.0 * 768 * 3040)),
-    # k_lazy_update_aq, a compaction block near full size (12 layers, n_new = 2944)
-    "k_lazy_update_aq": dict(bytes=3 * (162.8e6 + 217.4e6), launch="n_new = 2944, m = 32, 12 layers",
-                             algorithmic=12 * 24.0 * 2944 * 2943 / 2),
+    # k_lazy_update_aq_tc, first block at full size (12 layers, 3072 positions of which 3008 live)
+    "k_lazy_update_aq_tc": dict(bytes=3 * (223.8e6 + 291.0e6), launch="n_pos = 3072, m = 64, 12 layers",
+                                algorithmic=12 * (24.0 * 3008 * 3007 / 2 + 8.0 * 768 * 3008)),
+    # k_lazy_update_aq, the first compaction block (12 layers, n_new = 2720)
+    "k_lazy_update_aq": dict(bytes=3 * (149.7e6 + 176.7e6), launch="n_new = 2720, m = 32, 12 layers",
+                             algorithmic=12 * 24.0 * 2720 * 2719 / 2),
     # k_neuron_update, first step at full size (12 layers, n = 3071)
     "k_neuron_update": dict(bytes=343.1e6 + 281.9e6, launch="n = 3071, 12 layers",
                             algorithmic=12 * (8.0 * 768 * 3071 + 4.0 * 3071 * 3071)),
 }
 
 
+def lazy_steps_cap(npos):
+    """Most steps that a block in place leaves pending: 64, whole groups of 16 that fit a CTA's shared memory
+    where its slice of the positions is wider than 384."""
+    cs = 1
+    while cs < 8 and -(-npos // cs) > (256 if cs < 4 else 384):
+        cs *= 2
+    fit = 64 * (384 + 4) // (-(-npos // cs // 32) * 32 + 4)
+    return 64 if fit >= 64 else fit // 16 * 16
+
+
 def lazy_update_work(L, G, levels, r=0):
-    """Algorithmic work of the rank-32 update of H^-1 and Q (k_lazy_update_aq_tc in blocks that
+    """Algorithmic work of the rank-32 or rank-64 update of H^-1 and Q (k_lazy_update_aq_tc in blocks that
     leave removed positions in place, k_lazy_update_aq in blocks that squeeze them out) over one
     greedy run: a launch that leaves n live structures reads the off-diagonal entries of H^-1 and
     Q once per symmetric pair and writes them at [i][j] and [j][i] (2 matrices x n(n-1)/2 pairs x
@@ -199,7 +209,8 @@ def lazy_update_work(L, G, levels, r=0):
     overhead, not counted here, and neither is the endgame.  Block boundaries, and which blocks are
     dense, as in the library.
     Returns (bytes, fma, launches, bytes of W^T in the dense blocks)."""
-    n, npos, slot, nbytes, fma, launches, wbytes = G, G, 0, 0.0, 0.0, 0, 0.0
+    npos = (G + 3) // 4 * 4              # the pitch of the matrices
+    n, slot, nbytes, fma, launches, wbytes = G, 0, 0.0, 0.0, 0, 0.0
     levels = [v for v in levels if v < G]
     n_min = levels[-1] if levels else G
     endgame = n_min <= LAZY_ENDGAME_MIN
@@ -210,7 +221,11 @@ def lazy_update_work(L, G, levels, r=0):
         m = min(LAZY_BLOCK, n - stop)
         dead_after = npos - (n - m)
         last = endgame and n - m == LAZY_ENDGAME
-        compact = last or dead_after >= LAZY_DEAD_MAX or dead_after * LAZY_DEAD_FRACTION >= npos
+        compact = last or dead_after >= LAZY_DEAD_MAX or dead_after * LAZY_DEAD_FRACTION >= npos or npos <= 1
+        if not compact:
+            m = min(lazy_steps_cap(npos), n - stop)
+            if endgame and n - m == LAZY_ENDGAME:
+                m -= LAZY_BLOCK
         n -= m
         npos = n if compact else npos
         if n > 1:
@@ -734,10 +749,10 @@ def run_ours(args, shape):
                                               "symmetric matrices (16 B per pair); the kernel's own "
                                               "count (24 B) includes the second, mirrored store that "
                                               "lets the steps kernel read a pivot column as a row"),
-                          note="rank-32 update of H^-1 and Q, the operation with the largest summed "
+                          note="rank-32 or rank-64 update of H^-1 and Q, the operation with the largest summed "
                                "time in the timed path.  About three blocks "
-                               "in four at full width leave removed positions in place and run dense "
-                               "128 x 128 tiles on tcgen05 (bf16 x 3 split of the rank-32 operands, TMA "
+                               "in four leave removed positions in place and run dense "
+                               "128 x 128 tiles on tcgen05 (bf16 x 3 split of the packed operands, TMA "
                                "loads, direct and mirrored stores), W^T included as extra tiles of the "
                                "same kernel; the others squeeze removed positions "
                                "out with 4-byte gathers on the CUDA cores.  A stand-alone kernel "
@@ -753,7 +768,7 @@ def run_ours(args, shape):
                               launches=phases.get("lazy_steps", (0.0, 0))[1],
                               ms=phases.get("lazy_steps", (0.0, 0))[0],
                               us_per_greedy_step=1e3 * phases.get("lazy_steps", (0.0, 0))[0] / max(n_removed, 1),
-                              note="32 sequential greedy steps per launch on a cluster of 4, 2 or 1 CTAs "
+                              note="up to 64 sequential greedy steps per launch on a cluster of 8, 4, 2 or 1 CTAs "
                                    "per layer, the last 256 structures in one launch of the float64 "
                                    "endgame (in the time); a chain of long-latency instructions (offers "
                                    "exchanged between CTAs, shuffles, shared-memory loads, float64 "
