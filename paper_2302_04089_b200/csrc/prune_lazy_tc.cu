@@ -213,12 +213,11 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
                 s = s_next;
             }
             if (!failed) failed = !publish(0, 0, 0, TILE_STOP) || (pending && !load(t, pl, pi0, pj0));
-            if (failed) {
-                abort_flag = 1;
-                // copies already issued land in this CTA's shared memory: give them a bounded chance
-                for (int a = 0; a < NARR; ++a)
-                    if (copies[a] > 0) mbar_wait_quiet(smem_u32(&bar_ops_full[a]), (uint32_t)((copies[a] - 1) & 1));
-            }
+            if (failed) abort_flag = 1;
+            // The copies land in this CTA's shared memory before it leaves, also where another role gives up and
+            // the issuer no longer waits for them.
+            for (int a = 0; a < NARR; ++a)
+                if (copies[a] > 0) mbar_wait_quiet(smem_u32(&bar_ops_full[a]), (uint32_t)((copies[a] - 1) & 1));
         }
         __syncwarp();
     } else if (warp == 1) {
