@@ -372,9 +372,11 @@ ziplm_status ziplm_search_levels(const float* loss, const float* base_loss, cons
  *                                 before the query and leave it until the call.
  *     ZIPLM_OPT_HESSIAN_ROUTE     0: tensor cores from 32 tokens on; 1: CUDA-core kernel always.
  *     ZIPLM_OPT_SPIN_LIMIT        0: default; n > 0: poll limit of the wait for a free pipeline stage
- *                                 in the Hessian's kernels and the inverse's int8 products (tests
- *                                 make a bounded wait run out with it; see ziplm_hessian_accumulate
- *                                 for how that is reported; the inverse reports ZIPLM_ERR_TIMEOUT).
+ *                                 in the Hessian's kernels and the inverse's int8 products, and of
+ *                                 the waits for tile descriptors in the neuron path's dense update
+ *                                 (tests make a bounded wait run out with it; see
+ *                                 ziplm_hessian_accumulate for how that is reported; the inverse and
+ *                                 the neuron path report ZIPLM_ERR_TIMEOUT).
  *     ZIPLM_OPT_COMPACT_EVERY_BLOCK  0: the delayed-update neuron path leaves removed positions in
  *                                 place for a few blocks (dense tensor-core update of H^-1 and Q)
  *                                 and squeezes them out when 128 of them, or a sixteenth of all

@@ -482,7 +482,8 @@ class Option:
     LAYER_GROUPS = 1         # 1..8 layer groups on internal streams (0: default)
     FORCE_BLOCK_PATH = 2     # 1: group_size 1 through the general block path
     HESSIAN_ROUTE = 3        # 1: CUDA-core Hessian kernel always
-    SPIN_LIMIT = 4           # poll limit of the Hessian's and the int8 products' waits for a free pipeline stage
+    SPIN_LIMIT = 4           # poll limit of bounded waits: the Hessian's and the int8 products' for a free pipeline
+                             # stage, the dense neuron update's for tile descriptors
     COMPACT_EVERY_BLOCK = 5  # 1: squeeze removed positions out after every block of the neuron path
 
 

@@ -1137,6 +1137,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
     // last block that squeezed the removed positions out)
     int npos = ld;
     const bool every_block = option_value(ZIPLM_OPT_COMPACT_EVERY_BLOCK) == 1;
+    const unsigned spin = (unsigned)option_value(ZIPLM_OPT_SPIN_LIMIT);
     CUtensorMap map_p, map_a[2], map_q[2], map_w[2];
     if (!lazy_tc_make_map(&map_p, w.P, L, ld, rp)) return ZIPLM_ERR_CUDA;
     for (int b = 0; b < 2; ++b)
@@ -1215,7 +1216,7 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
             // every position stays in place: dense tiles, tensor-core kernel
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);
             s = run_lazy_update_aq_tc(map_p, map_a[cur], map_q[cur], map_w[cur], L, (nsteps + GS - 1) / GS, n_new, ld, rp,
-                                      w.A[nxt], w.Q[nxt], w.Wt[nxt], w.sched, layer_status, 0u, st);
+                                      w.A[nxt], w.Q[nxt], w.Wt[nxt], w.sched, layer_status, spin, st);
             if (s != ZIPLM_OK) return s;
         } else if (n_new > 1) {
             PhaseScope ps(PH_LAZY_UPDATE_AQ, st);

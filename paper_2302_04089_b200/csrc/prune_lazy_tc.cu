@@ -311,8 +311,9 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
         int issued = 0;                                      // slices whose copies were started
         auto open_tile = [&]() -> bool {
             const int slot = pt & (DESC_RING - 1);
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_tile_full[slot]),
-                                                              (uint32_t)((pt >> 2) & 1), abortp));
+            // (the limit is for what the pipeline leaves behind, not for the kernel's first descriptor)
+            const bool ok = __all_sync(0xffffffffu, mbar_wait_limit(smem_u32(&bar_tile_full[slot]), (uint32_t)((pt >> 2) & 1),
+                                                                    abortp, pt > 0 ? slot_spin_limit : kSpinLimit));
             if (!ok) { pflags = TILE_STOP; return false; }
             const TileSlot& ts = slots[slot];
             nl = ts.l; ni0 = ts.i0; nj0 = ts.j0;
@@ -349,8 +350,7 @@ k_lazy_update_aq_tc(const __grid_constant__ CUtensorMap map, const __grid_consta
 
         failed = !open_tile();
         int cl = nl, ci0 = ni0, cj0 = nj0, cflags = pflags;   // tile being worked on
-        copy_next();
-        copy_next();
+        failed = failed || !copy_next() || !copy_next();
         int unit = 0;
         for (int t = 0; !(cflags & TILE_STOP) && !failed; ++t) {
             for (int g = 0; g < sch.groups && !failed; ++g)
@@ -538,7 +538,7 @@ bool lazy_tc_make_matrix_map(CUtensorMap* m, const float* M, int L, int d, int c
 // map_q cover the matrices as they stand (n_pos positions), A2 / Q2 receive the result.
 // `counter` points at two ints (work counter, CTAs that have left) that are zero before the first
 // launch; every launch leaves them zero again.  slot_spin_limit = 0 selects the default poll
-// limit of the producer's wait for a free descriptor slot.
+// limit of the waits for descriptors: the producer's for a free slot, the epilogue's for the next one.
 ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& map_a,
                                    const CUtensorMap& map_q, const CUtensorMap& map_w, int L, int groups, int n_pos,
                                    int d, int rp, float* A2, float* Q2, float* W2, int* counter,

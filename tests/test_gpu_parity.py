@@ -1065,6 +1065,34 @@ def test_a_bounded_wait_of_the_int8_products_that_runs_out_is_reported():
     assert status.tolist() == [0, 0] and torch.equal(again, ref)
 
 
+def test_a_bounded_wait_of_the_dense_neuron_update_that_runs_out_is_reported():
+    """The update's epilogue warps give up after one look for their second descriptor, which the producer publishes
+    behind an atomic's round trip with all CTAs at the same counter: the layers report the time-out, and the same call
+    is right again afterwards.  What shares the option stays within it here (one K block, no int8 products)."""
+    z = zb()
+    gen = torch.Generator().manual_seed(11)
+    H = z.hessian_accumulate_tokens(torch.randn(12, 1300, 600, generator=gen).cuda())
+    W = torch.randn(12, 64, 600, generator=gen).cuda()
+    z.set_option(z.Option.LAYER_GROUPS, 1)
+    try:
+        ref = z.prune_layers(W, H, 1, 0.01, [400])
+        assert ref["layer_status"].tolist() == [0] * 12
+        z.set_option(z.Option.SPIN_LIMIT, 1)
+        _, status = z.damped_inverse(H, 0.01)
+        gram = z.hessian_accumulate(W.transpose(1, 2).contiguous())
+        out = z.prune_layers(W, H, 1, 0.01, [400])
+        torch.cuda.synchronize()
+        z.set_option(z.Option.SPIN_LIMIT, 0)
+        again = z.prune_layers(W, H, 1, 0.01, [400])
+    finally:
+        z.set_option(z.Option.SPIN_LIMIT, 0)
+        z.set_option(z.Option.LAYER_GROUPS, 0)
+    assert status.tolist() == [0] * 12 and not bool(gram.isnan().any())
+    assert out["layer_status"].tolist() == [int(z.Status.ERR_TIMEOUT)] * 12
+    for k in ("W_snap", "loss", "order", "saliency", "layer_status"):
+        assert torch.equal(again[k], ref[k]), k
+
+
 @pytest.mark.parametrize("d,r,levels", [(700, 40, [667, 603, 540, 492, 428, 391, 330, 265, 255, 0]),
                                         (1560, 20, [1527, 1463, 1400, 1336, 1295]), (3100, 12, [3067, 3019, 2970])])
 def test_blocks_of_one_and_two_groups_of_steps(d, r, levels):
