@@ -72,10 +72,14 @@ constexpr int PART_PITCH = TM + 4;            // ... of a part of it, whose rows
 // mirrored pieces at a time: one after the other the two took 22000 clocks of a tile's 32000 (13 x 1145 features,
 // 324 bf16 tokens: 70 -> 54 us a call).
 // Parts are read 16 bytes a lane, four columns, and the scales wait in shared memory: 1 x 256 x 2048 fp32 on clusters of
-// eight 12.8 us, against 15.5 with 4 bytes a lane and the scales from global memory behind the last barrier.
+// eight 12.8 us, against 15.5 with 4 bytes a lane and the scales from global memory behind the last barrier.  H is read
+// and written with lanes along the columns, 128 bytes an instruction, also where its rows start on 16 bytes: four columns
+// a lane took 18.5 us in place of 16.6 (1 x 1322 x 600 fp16, rows at any element, written in four passes of half-empty
+// sectors), 18.5 and 16.7 (4 x 576 x 693), 16.4 and 14.8 (8 x 80 x 2178 bf16); 20.8 and 22.2 the other way (2 x 408 x 1267
+// fp32).
 struct TileEnd {
     float* out_tile; float* mirror;
-    int rank, i0, j0, d, quads;
+    int rank, i0, j0, d;
     float alpha, beta;
     float* Hl; const float* scales;           // inverse scales of the tile's rows and columns [2][TM]
     const unsigned long long* err_word; unsigned long long call;
@@ -83,49 +87,55 @@ struct TileEnd {
     // rows of `mirror`: this CTA's share
     template <int S, int R, bool SPLIT>
     __device__ __forceinline__ void rows_of_parts() const {
-        constexpr int N_ROWS = TM / S, WARPS = THREADS / 32;
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS, cc = 4 * lane, col = j0 + cc;
+        constexpr int N_ROWS = TM / S, WARPS = THREADS / 32, NH = TM / 32;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = rank * N_ROWS, cc = 4 * lane;
         const float4 scale = SPLIT ? *reinterpret_cast<const float4*>(scales + TM + cc) : make_float4(1.f, 1.f, 1.f, 1.f);
 #pragma unroll 1
         for (int at = warp * R; at < N_ROWS && i0 + first + at < d; at += WARPS * R) {
-            float4 part[S][R], old[R];
+            float4 part[S][R];
+            float old[R][NH];
+            float* own = out_tile + (first + at) * PART_PITCH;
 #pragma unroll
             for (int p = 0; p < S; ++p) {
-                const float* from = cg::this_cluster().map_shared_rank(out_tile + (first + at) * PART_PITCH + cc, p);
+                const float* from = cg::this_cluster().map_shared_rank(own + cc, p);
 #pragma unroll
                 for (int k = 0; k < R; ++k) part[p][k] = *reinterpret_cast<const float4*>(from + k * PART_PITCH);
             }
 #pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const int row = i0 + first + at + k, n = beta != 0.f && row < d ? row - col + 1 : 0;
-                const float* o = Hl + (size_t)row * d + col;
-                if (quads && n > 3) old[k] = *reinterpret_cast<const float4*>(o);
-                else old[k] = make_float4(n > 0 ? o[0] : 0.f, n > 1 ? o[1] : 0.f, n > 2 ? o[2] : 0.f, n > 3 ? o[3] : 0.f);
-            }
+            for (int k = 0; k < R; ++k)
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    const int row = i0 + first + at + k, col = j0 + 32 * h + lane;
+                    old[k][h] = beta != 0.f && row < d && col <= row ? Hl[(size_t)row * d + col] : 0.f;
+                }
+            // the scaled sums go back to the place of this CTA's own part, which nobody else reads
 #pragma unroll
             for (int k = 0; k < R; ++k) {
-                const int row = i0 + first + at + k, n = row < d ? row - col + 1 : 0;       // entries up to the diagonal
                 float v[4] = {part[0][k].x, part[0][k].y, part[0][k].z, part[0][k].w};
 #pragma unroll
                 for (int p = 1; p < S; ++p) { v[0] += part[p][k].x; v[1] += part[p][k].y; v[2] += part[p][k].z; v[3] += part[p][k].w; }
-                const float o[4] = {old[k].x, old[k].y, old[k].z, old[k].w}, sc[4] = {scale.x, scale.y, scale.z, scale.w};
-                const float mul = SPLIT ? scales[first + at + k] : 1.f;
+                const float sc[4] = {scale.x, scale.y, scale.z, scale.w}, mul = SPLIT ? scales[first + at + k] : 1.f;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     v[e] *= alpha;
                     if (SPLIT) v[e] = (v[e] * mul) * sc[e];
-                    v[e] += o[e];
-                    mirror[(at + k) * OUT_PITCH + cc + e] = v[e];
                 }
-                float* out = Hl + (size_t)row * d + col;
-                if (quads && n > 3) {
-                    *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
-                } else {
+                *reinterpret_cast<float4*>(own + k * PART_PITCH + cc) = make_float4(v[0], v[1], v[2], v[3]);
+            }
+            __syncwarp();
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if (e < n) out[e] = v[e];
+            for (int k = 0; k < R; ++k) {
+                const int row = i0 + first + at + k;
+                float* out = Hl + (size_t)row * d + j0 + lane;
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    const int c = 32 * h + lane, col = j0 + c;
+                    if (row >= d || col > row) continue;             // (col <= row < d)
+                    const float v = own[k * PART_PITCH + c] + old[k][h];
+                    out[32 * h] = v;
+                    if ((row | col) == 0) hessian_check(out, err_word, call);
+                    mirror[(at + k) * OUT_PITCH + c] = v;
                 }
-                if ((row | col) == 0) hessian_check(out, err_word, call);
             }
         }
     }
@@ -202,7 +212,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
           float* __restrict__ H, int d, int num_kb_all, int n_split, float alpha, float beta, int layer0,
           int L, unsigned long long* err_word, unsigned long long call, uint32_t fmt16, uint32_t empty_spin_limit,
-          const unsigned* __restrict__ amax, int quads) {
+          const unsigned* __restrict__ amax) {
     using C = Cfg<SPLIT>;
     constexpr int STAGE_BYTES = C::TILES * TILE_BYTES;
     constexpr uint32_t TMEM_COLS = SPLIT ? 512u : 256u;   // main x2 (+ cross terms), power of two
@@ -366,13 +376,14 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
         }
         if (!failed) {
             if (SPLIT) {
-                // the last chunk's commit also covers every cross-term MMA
+                // the last chunk's commit also covers every cross-term MMA (16 columns at a time: 32 spill)
 #pragma unroll
-                for (int cc = 0; cc < NC / 32; ++cc) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + lane_base + (uint32_t)(256 + half * NC + cc * 32), v);
+                for (int cc = 0; cc < NC / 16; ++cc) {
+                    uint32_t v[16];
+                    tmem_ld16(tmem_base + lane_base + (uint32_t)(256 + half * NC + cc * 16), v);
+                    tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) acc[cc * 32 + e] += __uint_as_float(v[e]);
+                    for (int e = 0; e < 16; ++e) acc[cc * 16 + e] += __uint_as_float(v[e]);
                 }
             }
             // The operand ring is free (every MMA has completed): the partial tile goes there.
@@ -411,7 +422,7 @@ k_syrk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
 
     // Every CTA of the cluster finishes its share of the rows.
     float* Hl = H + (size_t)(layer0 + l) * d * d;
-    const TileEnd end{out_tile, mirror, rank, i0, j0, d, quads, alpha, beta, Hl, scales, err_word, call};
+    const TileEnd end{out_tile, mirror, rank, i0, j0, d, alpha, beta, Hl, scales, err_word, call};
     if (n_split == 1) end.finish<1, 4, SPLIT>();
     else if (n_split == 2) end.finish<2, 4, SPLIT>();
     else if (n_split == 4) end.finish<4, 4, SPLIT>();
@@ -931,7 +942,6 @@ ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_
     const int T = (p.d + TM - 1) / TM;
     const long long tiles = (long long)T * (T + 1) / 2 * p.layers;
     const int split = hessian_tile_split(tiles, p.num_kb);
-    const int quads = p.d % 4 == 0 && reinterpret_cast<uintptr_t>(p.H) % 16 == 0;     // rows of H start on 16 bytes
     constexpr int smem2 = Cfg<true>::STAGES * Cfg<true>::TILES * TILE_BYTES + 1024;
     constexpr int smem1 = Cfg<false>::STAGES * Cfg<false>::TILES * TILE_BYTES + 1024;
     static_assert(TM * (PART_PITCH + OUT_PITCH) * (int)sizeof(float) + 1024 <= smem1, "finished tiles fit the operand ring");
@@ -952,7 +962,7 @@ ziplm_status run_product(const HessianProduct& p, void* scratch, size_t scratch_
     cfg.numAttrs = 2;
     ZIPLM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, p.split ? k_syrk_tc<true> : k_syrk_tc<false>, p.hi,
                                         p.split ? p.lo : p.hi, p.H, p.d, p.num_kb, split, p.alpha, p.beta,
-                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax, quads));
+                                        p.layer0, p.L, p.err_word, p.call, p.fmt16, p.spin, p.amax));
     ZIPLM_CHECK_LAUNCH();
     return ZIPLM_OK;
 }

@@ -958,7 +958,7 @@ def test_hessian_into_a_matrix_that_starts_at_any_element(L, d, N, dtype):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("L,d,N", [(2, 400, 1000), (3, 400, 600), (2, 398, 1000), (1, 132, 2048)])
 def test_hessian_tiles_shared_by_two_four_and_eight(L, d, N, dtype):
-    """Ends of shared tiles with four columns a lane (width and start of H allow it) and one by one: the same bits, and
+    """Ends of shared tiles, at widths that are multiples of four and not, H on 16 bytes and at any element: the same bits, and
     within the bound of the other widths (fp32 sums of products that fp32 accumulators hold: 2e-6 of the diagonal)."""
     z = zb()
     A = torch.randn(L, N, d, generator=torch.Generator().manual_seed(d)).to(dtype).cuda()
