@@ -908,12 +908,16 @@ def test_16_bit_tokens_in_rows_of_even_pitch(N, d, pad, dtype):
 def test_tokens_in_rows_of_any_pitch(N, d, pad, dtype):
     """The moves of token-major activations whose rows start on their elements only, and of fp32 batches too long for
     one pass, at the edges of their tiles and slabs; small whole numbers (times a power of two per feature in
-    fp32, so that a wrong largest magnitude overflows the fp16 parts), so that the product is exact."""
+    fp32), so that the product is exact.  Each fp32 feature has one value far above the others, beside a multiple of
+    16 tokens, where the reads in flight and the slabs end, or in the last token: without it the feature would be
+    scaled until that value overflows its fp16 part."""
     z = zb()
     g = torch.Generator().manual_seed(N)
     full = torch.randint(-3, 4, (2, N, d + pad), generator=g).to(dtype)
     if dtype == torch.float32:
-        full[:, -1, :] = 7.0                     # the largest stands in the last token
+        f = torch.arange(d + pad)
+        for l in range(2):                       # 64 in place of at most 3: 2^18 if it is missed
+            full[l, torch.where(f % 5 == 4, N - 1, (16 * (f + 1) - 1 + l) % N), f] = 64.0
         full *= 2.0 ** (torch.arange(d + pad) % 30)
     A = full.cuda()[:, :, :d]
     H = z.hessian_accumulate_tokens(A, alpha=2.0)
