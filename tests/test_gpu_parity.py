@@ -982,10 +982,14 @@ def test_hessian_tiles_shared_by_two_four_and_eight(L, d, N, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("L,d,N", [(1, 1001, 3999), (13, 237, 4318), (7, 482, 4859), (6, 287, 843), (18, 96, 9001), (3, 333, 2276),
-                                   (1, 1700, 2000), (12, 198, 2221)])
+                                   (1, 1700, 2000), (12, 198, 2221),
+                                   (1, 1001, 700), (1, 1001, 730), (1, 1001, 1152), (1, 1001, 1216), (1, 1000, 4000), (2, 1000, 2000),
+                                   (15, 127, 2050), (16, 127, 2050), (33, 100, 1030), (34, 100, 1030), (74, 65, 600), (75, 65, 600)])
 def test_hessian_on_both_sides_of_the_line_between_its_kernels(L, d, N, dtype):
-    """Calls next to where pairs of CTAs take over from clusters, and clusters of eight from four from two: the bound of
-    the other widths (fp32 sums of products that fp32 accumulators hold: 2e-6 of the diagonal)."""
+    """Calls next to where pairs of CTAs take over from clusters (1 x 1001: fp32 between 11 and 12 K blocks, 16 bits between
+    18 and 19; 1 x 1000 x 4000 on pairs, 2 x 1000 x 2000 in 16 bits on clusters), and clusters of eight (up to 15 tiles) from
+    four (33) from two (74) from single CTAs: the bound of the other widths (fp32 sums of products that fp32
+    accumulators hold: 2e-6 of the diagonal)."""
     z = zb()
     A = torch.randn(L, N, d, generator=torch.Generator().manual_seed(N)).to(dtype).cuda()
     H = z.hessian_accumulate_tokens(A)
