@@ -1102,10 +1102,12 @@ def test_a_bounded_wait_of_the_dense_neuron_update_that_runs_out_is_reported():
 
 
 @pytest.mark.parametrize("d,r,levels", [(700, 40, [667, 603, 540, 492, 428, 391, 330, 265, 255, 0]),
-                                        (1560, 20, [1527, 1463, 1400, 1336, 1295]), (3100, 12, [3067, 3019, 2970])])
+                                        (1560, 20, [1527, 1463, 1400, 1336, 1295]), (3100, 12, [3067, 3019, 2970]),
+                                        (4500, 8, [4467, 4420])])
 def test_blocks_of_one_and_two_groups_of_steps(d, r, levels):
-    """Blocks of 33, 37, 48, 63 and 64 pending steps (two groups of packed operands, the second one full and
-    ragged) and of up to 32, on clusters of four and eight CTAs, up to and above the width where 64 fit."""
+    """Blocks of 33, 48, 61, 63 and 64 pending steps (two groups of packed operands, the second one full and
+    ragged) and of up to 32, on clusters of two, four and eight CTAs, up to and above the widths where 64 (3072
+    positions) and 48 (4096) fit."""
     sh = wl.scaled(wl.CONFIGS["c3_bert_base_fc2"][0], d_col=d, d_row=r, d_latent=d // 4,
                    n_tokens=d + 500, n_layers=1, levels=tuple(levels))
     run_case(sh)
