@@ -363,8 +363,8 @@ ziplm_status ziplm_search_levels(const float* loss, const float* base_loss, cons
  *                          option defaults to 0.  ZIPLM_ERR_INVALID_ARG for an unknown option or a
  *                          value outside its range.  Results never depend on an option beyond
  *                          rounding (every variant passes the same parity tests).
- *     ZIPLM_OPT_NEURON_PATH       0: delayed rank-32 updates (d_col <= 6144; wider layers take the
- *                                 other path); 1: per-step streaming update.
+ *     ZIPLM_OPT_NEURON_PATH       0: delayed updates of up to 64 steps (d_col <= 6144; wider layers take
+ *                                 the other path); 1: per-step streaming update.
  *     ZIPLM_OPT_LAYER_GROUPS      0: default (6); 1..8: number of layer groups that
  *                                 ziplm_prune_layers runs on internal streams (1 = none).
  *     ZIPLM_OPT_FORCE_BLOCK_PATH  1: group_size 1 takes the general block path (float64 state).
@@ -379,9 +379,9 @@ ziplm_status ziplm_search_levels(const float* loss, const float* base_loss, cons
  *                                 the neuron path report ZIPLM_ERR_TIMEOUT).
  *     ZIPLM_OPT_COMPACT_EVERY_BLOCK  0: the delayed-update neuron path leaves removed positions in
  *                                 place for a few blocks (dense tensor-core update of H^-1 and Q)
- *                                 and squeezes them out when 128 of them, or a sixteenth of all
+ *                                 and squeezes them out when 320 of them, or an eighth of all
  *                                 positions, have gathered; 1: squeezes them out after every
- *                                 block (gathering CUDA-core update only).
+ *                                 block (gathering CUDA-core update only, up to 32 steps a block).
  * ziplm_get_option         current value of an option.
  * ziplm_launch_count       kernels launched by this library since it was loaded.
  * ziplm_profile_begin      from now on every phase of every call is bracketed by a pair of CUDA

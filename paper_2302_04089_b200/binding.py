@@ -478,7 +478,7 @@ def search_levels(loss: torch.Tensor, base_loss: torch.Tensor, time: torch.Tenso
 
 class Option:
     """Diagnostic options of ziplm_set_option (all default to 0)."""
-    NEURON_PATH = 0          # 1: per-step streaming update instead of delayed rank-32 updates
+    NEURON_PATH = 0          # 1: per-step streaming update instead of delayed updates of up to 64 steps
     LAYER_GROUPS = 1         # 1..8 layer groups on internal streams (0: default)
     FORCE_BLOCK_PATH = 2     # 1: group_size 1 through the general block path
     HESSIAN_ROUTE = 3        # 1: CUDA-core Hessian kernel always

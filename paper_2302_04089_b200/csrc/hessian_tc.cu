@@ -904,8 +904,10 @@ size_t product_scratch_bytes(int L, int d, long long N, ziplm_dtype dt, bool tok
 // Where the 128 x 128 tiles leave half of the SMs idle, up to eight CTAs share a tile: the largest power of
 // two with which all fit and each keeps four K blocks (one layer of 256 features, 2048 tokens: three tiles,
 // a chain of 32 K blocks on one CTA).  `most`: the occupancy calculator's room for clusters of 2, 4 and 8 CTAs on the
-// kSMs of a B200, whose GPCs differ in size: what does not fit would wait for a second round (18 tiles of
-// 3 x 333 x 2276 bf16 on clusters of eight 26.5 us, of four 20.3; 12 x 198 x 2221 on four 29.4, on two 24.2).
+// kSMs of a B200, whose GPCs differ in size: what does not fit would wait for a second round (calls with 18
+// tiles on clusters of eight and of four: 3 x 333 x 2276 bf16 25.3 and 20.0 us, 18 x 93 x 2000 25.9 and 19.5; with 34
+// and 36 on four and on two: 34 x 100 x 1030 fp16 26.0 and 20.4, 6 x 353 x 1142 26.7 and 20.6, 36 x 100 x 1200 fp32
+// 39.3 and 33.0).
 int hessian_tile_split(long long tiles, long long num_kb) {
     constexpr int most[9] = {0, kSMs, kSMs / 2, 0, 33, 0, 0, 0, 15};
     int split = 1;

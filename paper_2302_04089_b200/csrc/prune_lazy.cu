@@ -1156,8 +1156,12 @@ ziplm_status run_prune_lazy(const float* W, const float* H, int L, int r, int d,
         const int nxt = cur ^ 1;
         // Up to four CTAs a layer as long as a CTA has more than 256 positions: the pending terms of a step are
         // bound by shared-memory bandwidth, 24 clocks per pending step and 384 positions, which outweighs
-        // the exchange.  Eight where a slice of BMAX pending steps would not fit shared memory: four with
-        // 32 pending steps up to 3072 positions took 27.5 ms where eight take 25.0 (12 x 3072, all work).
+        // the exchange.  Eight where a slice of BMAX pending steps would not fit shared memory (from 1537
+        // positions on), whatever the number of layers: four with as many steps as then fit take longer in
+        // all, 28.7 ms where eight take 26.3 (12 x 3072), 48.7 and 43.8 (24 x 3072), 102 and 97 (24 x 4096), or as
+        // long (24 x 1814 and 24 x 2048, to 1 %), although 15 clusters of eight fit the part at a time: with all 24
+        // layers in one group 53.3 and 48.9 (3072), 18.15 and 18.14 (1814), 19.97 and 20.32 (2048).  The steps
+        // of 4 x 4096 by themselves: 9.5 ms on four CTAs up to 3072, 9.2 on eight, 8.8 with never more than 32 pending.
         int cs = 1;
         while (cs < CLUSTER_MAX && (npos + cs - 1) / cs > (cs < 4 ? 256 : SLICE_WIDE)) cs *= 2;
         const int S = round_up_int((npos + cs - 1) / cs, 4), cap = steps_cap(S);

@@ -550,11 +550,12 @@ ziplm_status run_lazy_update_aq_tc(const CUtensorMap& map, const CUtensorMap& ma
     const int rows_pad = lazy_tc_rows_pad(d);
     const int rows_used = round_up_int(n_pos, RM);
     if (rows_used / RM > MAX_STRIPS) return ZIPLM_ERR_UNSUPPORTED;
-    // The kernel is bound by memory bandwidth, which two thirds of the SMs saturate (measured: the
-    // same time with 96 as with 148 CTAs, 12 % more with 74); the others are left to the kernels
-    // of other layer groups and batches that run beside it.
+    // Two thirds of the SMs; the others are left to the kernels of other layer groups and batches that run beside it.
+    // With two groups of steps the kernel is not bound by memory (0.47 of the copy rate on 99 CTAs) and all SMs make
+    // it shorter: a call whose layers are one group takes 27.5 ms on 99 CTAs and 25.7 on 148 (12 x 768 x 3072), 18.1 and
+    // 17.2 (24 x 768 x 1814), 108 and 102 (24 x 1024 x 4096).  With six groups beside one another both are the same to
+    // about 1.5 %: 26.3 and 26.4, 16.4 and 16.6, 43.8 and 43.8 (24 x 768 x 3072), 96.7 and 95.7; one layer 11.4 and 11.1.
     const int ctas = (2 * sms + 2) / 3;
-
     AqSched sch;
     sch.n_strips = rows_used / RM;
     sch.L = L;
