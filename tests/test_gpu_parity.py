@@ -302,8 +302,8 @@ def test_full_width_every_step_one_layer_of_3072():
 
 
 def test_cluster_of_eight_every_step_down_to_3072():
-    """Width 4096 (the BERT-large fc2 layers): the steps kernel runs on clusters of 8 CTAs while
-    more than 3072 positions are live, with 64 candidates per pick.  The first 1024 picks, their
+    """Width 4096 (the BERT-large fc2 layers): the steps kernel runs on clusters of 8 CTAs with 48
+    pending steps while there are more than 3072 positions, with 64 candidates per pick.  The first 1024 picks, their
     saliencies and the two levels are compared one by one (few weight rows, so that the oracle's
     replay stays within two minutes)."""
     sh = wl.scaled(wl.CONFIGS["c4_bert_large"][1], d_col=4096, d_row=64, d_latent=1024,
